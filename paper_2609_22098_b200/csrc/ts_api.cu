@@ -52,6 +52,9 @@ static bool select_paths(ts_ctx* ctx) {
   ctx->tmapW_ptr = nullptr;
   if (ctx->use_mma && !choose_tile_mma(c, ctx->num_sms, ctx->max_smem, !(tm & TS_TEST_NO_TMA), &ctx->tile)) ctx->use_mma = 0;
   if (!ctx->use_mma && !choose_tile(c, ctx->num_sms, ctx->max_smem, &ctx->tile)) return false;
+  ctx->use_tree = (c.dt_U == TS_DTYPE_BF16 && c.r % 8 == 0 && ctx->cc_major == 10 && !(tm & TS_TEST_FORCE_FMA) &&
+                   tree_plan(c, ctx->num_sms, ctx->max_smem, &ctx->tree)) ? 1 : 0;
+  ctx->tmapT_ptr = nullptr;
   ctx->few_ok = (few_supported(ctx) && !(tm & TS_TEST_NO_FEW)) ? 1 : 0;
   ctx->wait_limit = (tm & TS_TEST_SHORT_WAITS) ? 4096u : WAIT_LIMIT;
   return true;
@@ -116,6 +119,7 @@ extern "C" int32_t ts_create(const ts_config* cfg, ts_ctx** out) {
   ctx->calib.lo = cfg->calib_lo; ctx->calib.hi = cfg->calib_hi;
   ctx->calib.table = ctx->d_table;
   e = score_setup(ctx);
+  if (e == cudaSuccess && ctx->use_tree) e = tree_setup(ctx);
   if (e == cudaSuccess) e = verify_setup(ctx);
   if (e == cudaSuccess) e = expand_setup(ctx);
   if (e != cudaSuccess) { cudaFree(ctx->d_table); delete (Prof*)ctx->prof; delete ctx; return set_cuda_error("ts_create", e); }

@@ -55,6 +55,17 @@ struct TileCfg {
   int w_ring;   // 0: the W tile is resident; > 0: that many 64-token slabs of W stream through a ring (large ranks)
 };
 
+// Shared-memory and vocabulary plan of the one-launch expansion (ts_tree.cu).
+struct TreePlan {
+  int TV, ntiles;        // tokens per CTA (a multiple of 64), CTAs with tokens
+  int Vs;                // row stride of W and the base logits as the scan reads them (V rounded up to 8)
+  int BN, nU, nW;        // tokens per block, stages of the base-logit and W rings
+  int npiece;            // pieces of a base-logit row whose best tokens become seed candidates
+  int w_over;            // owners work in the W ring too
+  uint32_t oU, oL, oW, oX;   // shared-memory offsets (bytes)
+  size_t smem;
+};
+
 }  // namespace ts
 
 struct ts_ctx {
@@ -65,6 +76,8 @@ struct ts_ctx {
   int cc_major;
   int max_smem;
   ts::TileCfg tile;
+  ts::TreePlan tree;
+  int use_tree;     // 1: expansion and scoring run on the one-launch tensor-core kernel
   int vt_TV, vt_n;  // vocabulary ranges of the verification walk, one per CTA
   int use_mma;      // 1: scoring runs on the tensor-core kernel, 0: on the fp32 FMA kernel
   int few_ok;       // 1: levels with <= FEW_MAX parents run on the few-parents kernel instead
@@ -74,6 +87,8 @@ struct ts_ctx {
   // driver's encoder is not available, the kernel stages W with plain loads
   alignas(64) unsigned char tmapW[128];
   const void* tmapW_ptr;
+  alignas(64) unsigned char tmapT[128];   // the one-launch kernel's tensor map of W (boxes of 64 tokens x r rows)
+  const void* tmapT_ptr;
   alignas(64) unsigned char tmapU[128];   // tensor map of the base logits last expanded with ([request][depth][token] boxes)
   const void* tmapU_ptr; int tmapU_B;
   int tma_state;   // 0 not tried yet, 1 encoder found, -1 unavailable
@@ -117,8 +132,11 @@ struct WsLayout {
   size_t vf_child;                       // int[2][B][N+1]: first child and child count of every node
   size_t vf_lists;                       // int[2][B] reduction list, int[2][B] rescan list, int[8] counters
   size_t vf_edge;                        // double[3][B][N]: per edge p(x), q(x) and the accept uniform
+  size_t tree;                           // the one-launch expansion's region (ts_tree.cu lays it out)
   size_t total;
 };
+
+size_t tree_ws_bytes(const ts_ctx* ctx, int B);
 
 __host__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -195,6 +213,7 @@ __host__ inline WsLayout make_layout(const ts_ctx* ctx, int B) {
   L.vf_child = take(2 * b * (N + 1) * 4);
   L.vf_lists = take((4 * b + 8) * 4);
   L.vf_edge = take(3 * b * N * 8);
+  L.tree = ctx->use_tree ? take(tree_ws_bytes(ctx, B)) : 0;
   L.total = off;
   return L;
 }

@@ -172,6 +172,11 @@ extern "C" int32_t ts_expand_tree(ts_ctx* ctx, const void* U, const void* A, con
   char* ws = (char*)ws_v;
   cudaStream_t st = (cudaStream_t)stream;
 
+  if (ctx->use_tree) {
+    const TreeOut o{n_nodes, tok, parent, depth, sib_rank, logS, q0, logqT, logkey, pop_rank, node_hash, node_lseT, mask, n_scored, status};
+    const cudaError_t et = tree_expand(ctx, ws + L.tree, o, U, A, W, B, anchor_tok, theta, T, seed, st);
+    return et == cudaSuccess ? TS_OK : set_cuda_error("ts_expand_tree", et);
+  }
   ExpandArgs a{};
   a.B = B; a.D = c.D; a.K = c.K; a.N = c.Nmax; a.V = c.V; a.T = T; a.anchor = anchor_tok; a.theta = theta;
   a.calib = ctx->calib;

@@ -3,6 +3,8 @@
 
 #include <vector>
 
+#include <cuda.h>
+
 #include "ts_common.cuh"
 
 namespace ts {
@@ -109,6 +111,22 @@ bool few_supported(const ts_ctx* ctx);
 cudaError_t launch_score_few(const ts_ctx* ctx, const ScoreArgs& a, int p_bound, cudaStream_t st);
 // encodes (or finds cached in the context) the tensor map of W for 64-token boxes; false: not available
 bool w_tensor_map(ts_ctx* ctx, const void* W);
+
+// the one-launch expansion and scoring (ts_tree.cu)
+struct TreeOut {
+  int *n_nodes, *tok, *parent, *depth, *sib_rank; float *logS, *q0, *logqT, *logkey; int* pop_rank;
+  uint64_t* node_hash; float* node_lseT; uint64_t* mask; int *n_scored, *status;
+};
+bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out);
+cudaError_t tree_setup(ts_ctx* ctx);
+size_t tree_score_bytes(const ts_ctx* ctx, int P);
+cudaError_t tree_score(ts_ctx* ctx, char* scratch, const void* U, const void* A, const void* W, int P, const int* p_req, const int* p_depth, const int* p_token,
+                       const uint64_t* p_hash, float T, uint64_t seed, float* lse0, float* lseT, int* top_tok, float* top_logit, int* draw_tok,
+                       float* draw_logit, int rows, cudaStream_t st);
+cudaError_t tree_expand(ts_ctx* ctx, char* ws, const TreeOut& o, const void* U, const void* A, const void* W, int B, const int* anchor, const float* theta,
+                        float T, uint64_t seed, cudaStream_t st);
+// tensor map of a bf16 matrix [r][stride] for boxes of 64 tokens x r rows (rounded up to 16); false: not available
+bool tree_tensor_map(ts_ctx* ctx, const void* W, int stride, CUtensorMap* out);
 
 enum KernelId { K_INIT, K_SCORE, K_MERGE, K_LEVEL, K_FINAL, K_ZROWS, K_GREEDY, K_WALK, K_CHECK, K_SCORE_FEW, K_ALLOC_SELECT, K_ALLOC_CUT, K_CALIB_ACC, K_CALIB_FIT, K_ATTN_INPUTS, K_SEED, K_PERSIST, K_COUNT };
 

@@ -35,11 +35,22 @@ extern "C" int32_t ts_score_parents_static(ts_ctx* ctx, const void* U, const voi
   if (!(T >= 0.f)) return set_error(TS_ERR_INVALID, "ts_score_parents_static: T must be >= 0");
   if (P == 0) return TS_OK;
 
+  int dev = -1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return set_cuda_error("ts_score_parents_static(device)", e);
+  const size_t tree_need = ctx->use_tree ? tree_score_bytes(ctx, P) : 0;   // 0: this context scores on the fp32 kernels here
+  if (tree_need > (size_t)TS_STATIC_SCRATCH_BYTES) {
+    char msg[256];
+    snprintf(msg, sizeof(msg),
+             "ts_score_parents_static: %d parents need %zu bytes of scratch, the built-in array holds %u; use ts_score_parents with a workspace instead",
+             P, tree_need, (unsigned)TS_STATIC_SCRATCH_BYTES);
+    return set_error(TS_ERR_WORKSPACE, msg);
+  }
   // records of P parents over all vocabulary tiles, plus the scoring kernel's error word
   int cap = 0;
   const size_t rec_bytes = align_up(score_scratch_bytes(ctx, P, &cap), 256);
   const size_t need = rec_bytes + 256;
-  if (need > (size_t)TS_STATIC_SCRATCH_BYTES) {
+  if (tree_need == 0 && need > (size_t)TS_STATIC_SCRATCH_BYTES) {
     int cap1 = 0;
     const size_t unit = score_scratch_bytes(ctx, 1, &cap1);  // bytes for the smallest slot block
     char msg[256];
@@ -50,9 +61,6 @@ extern "C" int32_t ts_score_parents_static(ts_ctx* ctx, const void* U, const voi
     return set_error(TS_ERR_WORKSPACE, msg);
   }
 
-  int dev = -1;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return set_cuda_error("ts_score_parents_static(device)", e);
   if (dev != ctx->device || dev < 0 || dev >= kMaxDevices)
     return set_error(TS_ERR_INVALID, "ts_score_parents_static: the context's device must be the current device");
   void* scratch = nullptr;
@@ -65,6 +73,11 @@ extern "C" int32_t ts_score_parents_static(ts_ctx* ctx, const void* U, const voi
       g_scratch_addr[dev] = p;
     }
     scratch = g_scratch_addr[dev];
+  }
+  if (tree_need) {
+    e = tree_score(const_cast<ts_ctx*>(ctx), (char*)scratch, U, A, W, P, parent_req, parent_depth, parent_token, parent_hash, T, seed, lse0, lseT, top_tok,
+                   top_logit, draw_tok, draw_logit, 0, (cudaStream_t)stream);
+    return e == cudaSuccess ? TS_OK : set_cuda_error("ts_score_parents_static", e);
   }
   // The records need no clearing: the scoring kernel writes every record of (piece, parent < P) before
   // the merge kernel, next on the same stream, reads exactly those.  The error word and the pruning

@@ -254,6 +254,11 @@ extern "C" int32_t ts_score_parents(ts_ctx* ctx, const void* U, const void* A, c
   if (!(T >= 0.f)) return set_error(TS_ERR_INVALID, "ts_score_parents: T must be >= 0");
   if (ws_bytes < L.total) return set_error(TS_ERR_WORKSPACE, "ts_score_parents: workspace too small");
   if (P == 0) return TS_OK;
+  if (ctx->use_tree) {
+    const cudaError_t et = tree_score(ctx, (char*)ws + L.tree, U, A, W, P, parent_req, parent_depth, parent_token, parent_hash, T, seed, lse0, lseT, top_tok,
+                                      top_logit, draw_tok, draw_logit, ctx->cfg.max_batch * ctx->cfg.D, (cudaStream_t)stream);
+    return et == cudaSuccess ? TS_OK : set_cuda_error("ts_score_parents", et);
+  }
   cudaError_t e = cudaMemsetAsync((char*)ws + L.err, 0, 16, (cudaStream_t)stream);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(thr_base(ctx, (float*)((char*)ws + L.rec), L.rec_cap), 0, thr_bytes(ctx, L.rec_cap), (cudaStream_t)stream);

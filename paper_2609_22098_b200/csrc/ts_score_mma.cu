@@ -988,6 +988,29 @@ bool w_tensor_map(ts_ctx* ctx, const void* W) {
   return true;
 }
 
+bool tree_tensor_map(ts_ctx* ctx, const void* W, int stride, CUtensorMap* out) {
+  if (ctx->test_mode & TS_TEST_NO_TMA) return false;
+  if (ctx->tmapT_ptr == W) { memcpy(out, ctx->tmapT, sizeof(*out)); return true; }
+  if (!g_encode) {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || !fn || q != cudaDriverEntryPointSuccess) {
+      (void)cudaGetLastError();
+      return false;
+    }
+    g_encode = (EncodeTiledFn)fn;
+  }
+  const cuuint64_t gdim[2] = {(cuuint64_t)stride, (cuuint64_t)ctx->cfg.r};
+  const cuuint64_t gstride[1] = {(cuuint64_t)stride * 2};
+  const cuuint32_t box[2] = {64u, (cuuint32_t)((ctx->cfg.r + 15) / 16 * 16)};
+  const cuuint32_t estr[2] = {1u, 1u};
+  if (g_encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(W), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return false;
+  memcpy(ctx->tmapT, out, sizeof(*out));
+  ctx->tmapT_ptr = W;
+  return true;
+}
+
 // Tensor map of the base logits U = [B][D][V] bf16 for boxes of 64 tokens x 1 depth x UMMA_REQ requests (requests past
 // B arrive as zeros), in the 128-byte swizzle of a B-operand slab whose K rows are the requests.
 static bool u_tensor_map(ts_ctx* ctx, const void* U, int B) {

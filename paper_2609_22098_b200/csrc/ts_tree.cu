@@ -1,0 +1,1499 @@
+// The whole expansion of a batch in one cooperative launch (bf16 inputs on the 5th-generation tensor cores).
+//
+// One CTA per SM holds one vocabulary range for the whole launch.  A level of the trees is two phases, each
+// closed by a bounded grid barrier:
+//   scan   every CTA scores all of the level's parents on its range: the low-rank bias [128 parents x r].[r x BN
+//          tokens] is a tcgen05 tile per block of BN tokens, W streams through a ring of bulk-tensor loads (and runs
+//          ahead across levels: it does not depend on them), the parents' base-logit rows come by cp.async into
+//          a ring beside it, and 16 warps read the accumulators (one tensor-memory lane = one parent), add the base
+//          logits, and keep (max reference, sums) and the few tokens that can be among a parent's K best.
+//   owner  the CTA that owns a request merges the request's parents (one warp each), runs the level step and makes
+//          the next level's parent list with its seed bounds; the CTAs without a request meanwhile sweep the base
+//          logits of the level after (best token of every 1024: where the next seed bounds come from).
+// Before this, a level was three dependent launches (scan with its own set-up, merge of fixed-size records, level
+// step on global-memory state): about 70 us per level at 32 requests, V = 151,936, r = 64, of which the arithmetic
+// needs less than ten.  See the phase comments for what each part costs now.
+//
+// Bounds.  Per parent K slots in global memory, slot j = best value published by the pieces (range, split, replica)
+// whose number is j mod K; pieces hold disjoint tokens, so the minimum over the slots is a lower bound of the K-th
+// best value and a token strictly below it is skipped.  The scan starts from the parent's seed bounds: the K-th
+// best exact value among the tokens with the largest base logits, less a rounding margin.
+#include <math.h>
+#include <string.h>
+
+#include "ts_tree.cuh"
+
+namespace ts {
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// arrives on `bar` when this thread's earlier cp.async have landed (the barrier counts every thread that says so)
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// Shared-memory state of a CTA.
+struct TxSm {
+  unsigned char *As, *Us, *Ws;
+  uint4* q;                    // [TX_QCAP] queued candidates: token, logit, row | split << 8 | kind << 12 | c16 << 16, tag
+  float* lists;                // [128][5K]: topv, topi, keyv, keyi, keyl of every row, sorted (value desc, token asc)
+  int* ln;                     // [2][128] entries in use
+  volatile float* lthr;        // [2][128] K-th best of the row's own list (-inf until it is full)
+  volatile float* best;        // [2][TX_SPLIT][128] best value published by the piece (row, split)
+  float* part;                 // [3][TX_SPLIT][128] reference, sum, tempered sum of every (split, row)
+  float* ghi;                  // [512] noise bounds
+  volatile float* thr;         // [2][128] launch-wide bounds of the rows' parents
+  ParentEntry* ent;            // [128] the group's parents by tile row
+  uint64_t *a_full, *t_full, *t_empty, *u_full, *w_full, *w_free;
+  uint32_t* tmem;
+  volatile int *abort, *done;
+  volatile unsigned* q_head; unsigned* q_tail;
+};
+
+constexpr size_t tx_select_bytes(int K) {
+  return (size_t)TX_QCAP * 16 + (size_t)TX_ROWS * 5 * K * 4 + 2 * TX_ROWS * 4 + 2 * TX_ROWS * 4 + 2 * TX_SPLIT * TX_ROWS * 4 + 3 * TX_SPLIT * TX_ROWS * 4;
+}
+constexpr size_t TX_FIXED_BYTES = 512 * 4 + 2 * TX_ROWS * 4 + TX_ROWS * sizeof(ParentEntry) + (1 + 5 * TX_STAGE_MAX) * 8 + 64;
+
+__device__ __forceinline__ TxSm tx_carve(unsigned char* sm, const TreeArgs& a) {
+  TxSm s;
+  s.As = sm; s.Us = sm + a.oU; s.Ws = sm + a.oW;
+  s.q = reinterpret_cast<uint4*>(sm + a.oL);
+  s.lists = reinterpret_cast<float*>(s.q + TX_QCAP);
+  s.ln = reinterpret_cast<int*>(s.lists + (size_t)TX_ROWS * 5 * a.K);
+  s.lthr = reinterpret_cast<float*>(s.ln + 2 * TX_ROWS);
+  s.best = s.lthr + 2 * TX_ROWS;
+  s.part = const_cast<float*>(s.best) + 2 * TX_SPLIT * TX_ROWS;
+  s.ent = reinterpret_cast<ParentEntry*>(sm + a.oX);
+  s.ghi = reinterpret_cast<float*>(s.ent + TX_ROWS);
+  s.thr = s.ghi + 512;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(const_cast<float*>(s.thr) + 2 * TX_ROWS);
+  s.a_full = bars; s.t_full = bars + 1; s.t_empty = s.t_full + TX_STAGE_MAX; s.u_full = s.t_empty + TX_STAGE_MAX;
+  s.w_full = s.u_full + TX_STAGE_MAX; s.w_free = s.w_full + TX_STAGE_MAX;
+  s.tmem = reinterpret_cast<uint32_t*>(s.w_free + TX_STAGE_MAX);
+  s.abort = reinterpret_cast<volatile int*>(s.tmem + 1);
+  s.done = reinterpret_cast<volatile int*>(s.tmem + 2);
+  s.q_head = reinterpret_cast<volatile unsigned*>(s.tmem + 3);
+  s.q_tail = s.tmem + 4;
+  return s;
+}
+
+// insertion into one sorted list of at most K entries (value desc, token asc); returns the K-th value (-inf: not full)
+__device__ __forceinline__ float tx_insert(float* v, int* t, float* aux, int& n, int K, float val, int tok, float lg) {
+  int pos = n < K ? n : K - 1;
+  if (n == K && !(val > v[pos] || (val == v[pos] && (unsigned)tok < (unsigned)t[pos]))) return v[pos];
+  while (pos > 0 && (val > v[pos - 1] || (val == v[pos - 1] && (unsigned)tok < (unsigned)t[pos - 1]))) {
+    v[pos] = v[pos - 1]; t[pos] = t[pos - 1];
+    if (aux) aux[pos] = aux[pos - 1];
+    --pos;
+  }
+  v[pos] = val; t[pos] = tok;
+  if (aux) aux[pos] = lg;
+  n = n < K ? n + 1 : K;
+  return n == K ? v[K - 1] : -INFINITY;
+}
+
+// The sampling key of one token, exactly (both generator streams).
+__device__ __forceinline__ float exact_key(uint64_t seed, int req, uint64_t hash, int tok, float lg, float invT) {
+  const uint4 cw = stream_words(seed, req, hash, STREAM_GUMBEL_COARSE, (uint32_t)tok >> 3);
+  const uint4 fw = stream_words(seed, req, hash, STREAM_GUMBEL_FINE, (uint32_t)tok >> 3);
+  const uint32_t c16 = (word_of(cw, (tok & 7) >> 1) >> (16 * (tok & 1))) & 0xFFFFu;
+  const uint32_t f16 = (word_of(fw, (tok & 7) >> 1) >> (16 * (tok & 1))) & 0xFFFFu;
+  return lg * invT + gumbel_from_bits((c16 << 16) | f16);
+}
+
+// Coarse words of the sampling uniforms, with everything that is fixed per parent worked out once: of the generator's
+// counter only the index changes from call to call, and it reaches the other lane pair one round later, so one of the
+// two products of the first round and one of the second are constants of the parent.
+struct CoarseGen {
+  uint32_t x0, x1, y2, y3;   // round 1's c0 ^ , c1 ; round 2's constants
+  uint32_t k0, k1, c3;
+  __device__ __forceinline__ void init(uint64_t seed, int req, uint64_t hash) {
+    k0 = (uint32_t)seed; k1 = (uint32_t)(seed >> 32);
+    c3 = (((uint32_t)req & 0xFFFFFFu) | ((uint32_t)STREAM_GUMBEL_COARSE << 24)) ^ k1;
+    const uint32_t c1 = (uint32_t)hash, c2 = (uint32_t)(hash >> 32);
+    const uint32_t n0 = __umulhi(0xCD9E8D57u, c2) ^ c1 ^ k0;   // round 1, word 0
+    x1 = 0xCD9E8D57u * c2;                                      // round 1, word 1
+    y2 = __umulhi(0xD2511F53u, n0) ^ (k1 + 0xBB67AE85u);        // round 2, word 2 = y2 ^ (word 3 of round 1)
+    y3 = 0xD2511F53u * n0;                                      // round 2, word 3
+    x0 = x1 ^ (k0 + 0x9E3779B9u);                               // round 2, word 0 = hi(M1 * word 2 of round 1) ^ x0
+  }
+  __device__ __forceinline__ uint4 words(uint32_t index) const {
+    // round 1: words 2 and 3
+    const uint32_t a2 = __umulhi(0xD2511F53u, index) ^ c3, a3 = 0xD2511F53u * index;
+    // round 2
+    uint32_t c0 = __umulhi(0xCD9E8D57u, a2) ^ x0, c1 = 0xCD9E8D57u * a2, c2 = y2 ^ a3, cc3 = y3;
+    uint32_t q0 = k0 + 2u * 0x9E3779B9u, q1 = k1 + 2u * 0xBB67AE85u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t hi0 = __umulhi(0xD2511F53u, c0), lo0 = 0xD2511F53u * c0;
+      const uint32_t hi1 = __umulhi(0xCD9E8D57u, c2), lo1 = 0xCD9E8D57u * c2;
+      c0 = hi1 ^ c1 ^ q0; c1 = lo1; c2 = hi0 ^ cc3 ^ q1; cc3 = lo0;
+      q0 += 0x9E3779B9u; q1 += 0xBB67AE85u;
+    }
+    return make_uint4(c0, c1, c2, cc3);
+  }
+};
+
+// One candidate, handled by one lane of the selecting warp: exact key, insertion, publication.
+__device__ __forceinline__ void tx_select(const TreeArgs& a, const TxSm& sm, const uint4 e, float invT, int tile, int R, int g) {
+  const int K = a.K, tok = (int)e.x;
+  const float lg = __uint_as_float(e.y);
+  const int row = (int)(e.z & 0xFFu), s = (int)((e.z >> 8) & 0xFu);
+  const uint32_t kind = (e.z >> 12) & 0xFu, c16 = e.z >> 16;
+  const int per = TX_ROWS / R;
+  const int prow = R > 1 ? row % per : row, rho = R > 1 ? row / per : 0;
+  const int p = R > 1 ? prow : g * TX_ROWS + row;
+  const int pid = ((tile * TX_SPLIT + s) * R + rho) % K;
+  float* L = sm.lists + (size_t)row * 5 * K;
+  if (kind & 1u) {
+    if (lg >= sm.thr[prow] && lg >= sm.lthr[row]) {
+      sm.lthr[row] = tx_insert(L, reinterpret_cast<int*>(L) + K, nullptr, sm.ln[row], K, lg, tok, 0.f);
+      volatile float* b = sm.best + s * TX_ROWS + row;
+      if (lg > *b) { *b = lg; atomicMax(a.slots + ((size_t)p * K + pid) * SLOT_STRIDE, enc_f(lg)); }
+    }
+  }
+  if (kind & 2u) {
+    const float thr = fmaxf(sm.thr[TX_ROWS + prow], sm.lthr[TX_ROWS + row]);
+    const float bnd = lg * invT + sm.ghi[noise_bound_index(c16)];
+    if (bnd >= thr) {   // the bounds have often risen since the candidate was queued
+      const ParentEntry& pe = sm.ent[row];
+      const uint4 fw = stream_words(a.seed, pe.req, pe.hash, STREAM_GUMBEL_FINE, (uint32_t)tok >> 3);
+      const uint32_t f16 = (word_of(fw, (tok & 7) >> 1) >> (16 * (tok & 1))) & 0xFFFFu;
+      const float key = lg * invT + gumbel_from_bits((c16 << 16) | f16);
+      if (key >= thr) {
+        sm.lthr[TX_ROWS + row] = tx_insert(L + 2 * K, reinterpret_cast<int*>(L) + 3 * K, L + 4 * K, sm.ln[TX_ROWS + row], K, key, tok, lg);
+        volatile float* b = sm.best + (TX_SPLIT + s) * TX_ROWS + row;
+        if (key > *b) { *b = key; atomicMax(a.slots + (((size_t)a.cap + p) * K + pid) * SLOT_STRIDE, enc_f(key)); }
+      }
+    }
+  }
+}
+
+// Where a role stands in the stream of blocks: every role passes every block of every group in the same order.
+struct BlockPos {
+  int slot, use;
+  __device__ __forceinline__ void next(int n) { if (++slot == n) { slot = 0; ++use; } }
+};
+
+__device__ __forceinline__ bool tx_wait(uint64_t* bar, uint32_t parity, const TxSm& sm, const TreeArgs& a) {
+  for (uint32_t i = 0; i < a.wait_limit; ++i) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if (*sm.abort) return false;
+    if (i > 64) __nanosleep(64);
+  }
+  *sm.abort = 1;
+  atomicExch(a.err, 1);
+  return false;
+}
+
+// ---- scanning warps: one group of up to 128 parents over this CTA's range ---------------------------------
+// Cost: two generator calls (76 multiply-xor steps), 16 ex2 and about 100 other instructions per 16 tokens and
+// parent; a warp owns every (4R)-th chunk of 16 tokens, so with few parents (R = 2, 4 replicas of the rows) the
+// copies share the range.
+__device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int t0, const int tlen,
+                                        const uint32_t tmem_base, BlockPos& pos) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int q = warp & 3, s = warp >> 2, row = q * 32 + lane;
+  const int per = TX_ROWS / R, K = a.K;
+  (void)K;
+  {
+    const int cpr = (a.r + 63) / 64 * 8;          // 16-byte chunks per A row
+    const __nv_bfloat16* Ag = reinterpret_cast<const __nv_bfloat16*>(a.A);
+    for (int idx = tid; idx < TX_ROWS * cpr; idx += TX_SCAN_WARPS * 32) {
+      const int rr = idx / cpr, ck = idx % cpr;
+      const ParentEntry& pe = sm.ent[rr];
+      const bool in = pe.row >= 0 && ck * 8 < a.r;
+      cp_async16(sm.As + (size_t)(ck >> 3) * (TX_ROWS * 128) + rr * 128 + (((ck & 7) ^ (rr & 7)) << 4), in ? Ag + (size_t)pe.token * a.r + ck * 8 : Ag, in);
+    }
+    cp_async_wait_all();
+    fence_async_smem();
+    mbar_arrive(sm.a_full);
+  }
+  const ParentEntry& me = sm.ent[row];
+  const bool active = me.row >= 0;
+  const int prow = R > 1 ? row % per : row, rho = R > 1 ? row / per : 0;   // rho is uniform within a warp
+  const float T = a.T, invT = T > 0.f ? 1.f / T : 1.f;
+  const bool keys = T > 0.f, two = keys && T != 1.f;
+  const float slack = 8.f * fminf(1.f, T > 0.f ? T : 1.f);   // how far a logit may exceed the sums' reference
+  CoarseGen gen; gen.init(a.seed, me.req, me.hash);
+  float m = me.mref, s0 = 0.f, sT = 0.f;
+  const uint32_t ztag = (uint32_t)row | ((uint32_t)s << 8);
+  const int CB = a.BN / 16, nblk = (tlen + a.BN - 1) / a.BN, stride = R * TX_SPLIT, own = rho * TX_SPLIT + s;
+  const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16);
+  bool alive = true;
+  for (int nb = 0; nb < nblk; ++nb, pos.next(a.nU)) {
+    const int slot = pos.slot;
+    const bool got = tx_wait(sm.t_full + slot, pos.use & 1, sm, a) && tx_wait(sm.u_full + slot, pos.use & 1, sm, a);
+    if (!__all_sync(0xFFFFFFFFu, got)) { alive = false; break; }
+    tc_fence_after();
+    const int nch = min(CB, (tlen - nb * a.BN + 15) / 16);
+    const unsigned char* urow = sm.Us + (size_t)slot * (TX_ROWS * 2) * a.BN + (size_t)prow * 2 * a.BN;
+    for (int c = (own - nb * CB) & (stride - 1); c < nch; c += stride) {
+      uint32_t ra[16];
+      __syncwarp();   // (the tensor-memory load is a warp-wide instruction)
+      tmem_ld16_issue(trow + (uint32_t)(slot * a.BN + c * 16), ra);
+      const uint4 u0 = *reinterpret_cast<const uint4*>(urow + (((2 * c) ^ (prow & 7)) << 4));
+      const uint4 u1 = *reinterpret_cast<const uint4*>(urow + (((2 * c + 1) ^ (prow & 7)) << 4));
+      const int v0 = t0 + nb * a.BN + c * 16, valid = min(16, a.V - v0);
+      // high halves of the sixteen uniforms: issued first, their long dependent chains overlap the rest
+      uint4 cw0 = make_uint4(0, 0, 0, 0), cw1 = cw0;
+      if (keys) { cw0 = gen.words((uint32_t)v0 >> 3); cw1 = gen.words(((uint32_t)v0 >> 3) + 1u); }
+      tmem_ld_wait();
+      if (!active) continue;
+      float acc[16];
+      unpack_bf16x8(u0, acc); unpack_bf16x8(u1, acc + 8);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) acc[i] += __uint_as_float(ra[i]);
+      if (valid < 16) {   // warp-uniform: the vocabulary's last chunk
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc[i] = (i < valid) ? acc[i] : -INFINITY;
+      }
+      const float thrL = sm.thr[prow], thrK = sm.thr[TX_ROWS + prow];
+      float gmax[4], cm = -INFINITY;
+#pragma unroll
+      for (int sg = 0; sg < 4; ++sg) {
+        gmax[sg] = fmaxf(fmaxf(acc[4 * sg], acc[4 * sg + 1]), fmaxf(acc[4 * sg + 2], acc[4 * sg + 3]));
+        cm = fmaxf(cm, gmax[sg]);
+      }
+      if (cm > m + slack) {   // rare: the reference is an exact logit of one of the parent's best tokens
+        const float d = m == -INFINITY ? 0.f : m - cm;
+        s0 *= __expf(d); sT *= __expf(d * invT);
+        m = cm;
+      }
+      {
+        // exp(l - m) as ex2(l log2(e) - m log2(e)); while nothing finite has been seen every l is -inf and adds 0
+        constexpr float LOG2E = 1.4426950408889634f;
+        const float off0 = m == -INFINITY ? 0.f : -m * LOG2E, scT = LOG2E * invT, offT = off0 * invT;
+        float a0 = 0.f, a1 = 0.f, aT = 0.f, aU = 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; i += 2) {
+          a0 += ex2_approx(fmaf(acc[i], LOG2E, off0));
+          a1 += ex2_approx(fmaf(acc[i + 1], LOG2E, off0));
+          if (two) { aT += ex2_approx(fmaf(acc[i], scT, offT)); aU += ex2_approx(fmaf(acc[i + 1], scT, offT)); }
+        }
+        a0 += a1;
+        s0 += a0;
+        sT += two ? aT + aU : a0;
+      }
+      uint32_t mkK = 0, mkL = 0;
+      if (cm >= thrL) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) mkL |= (uint32_t)(acc[i] >= thrL && acc[i] > -INFINITY) << i;
+      }
+      if (keys) {
+        // the whole chunk first: its best logit plus the noise bound of the largest leading bits bounds every key
+        // in it; then four tokens at a time, then singly
+        const uint32_t m8 = __vmaxu2(__vmaxu2(__vmaxu2(cw0.x, cw0.y), __vmaxu2(cw0.z, cw0.w)),
+                                     __vmaxu2(__vmaxu2(cw1.x, cw1.y), __vmaxu2(cw1.z, cw1.w)));
+        const uint32_t c16all = max(m8 & 0xFFFFu, m8 >> 16);
+        if (cm * invT + sm.ghi[noise_bound_index(c16all)] >= thrK && cm > -INFINITY) {
+#pragma unroll
+          for (int sg = 0; sg < 4; ++sg) {
+            const uint4& cw = sg < 2 ? cw0 : cw1;
+            const uint32_t wa = (sg & 1) ? cw.z : cw.x, wb = (sg & 1) ? cw.w : cw.y;
+            const uint32_t m2 = __vmaxu2(wa, wb);
+            const uint32_t c16m = max(m2 & 0xFFFFu, m2 >> 16);
+            if (gmax[sg] * invT + sm.ghi[noise_bound_index(c16m)] >= thrK && gmax[sg] > -INFINITY) {
+#pragma unroll
+              for (int i = 4 * sg; i < 4 * sg + 4; ++i) {
+                const uint32_t word = word_of(i < 8 ? cw0 : cw1, (i & 7) >> 1);
+                const uint32_t c16 = (word >> (16 * (i & 1))) & 0xFFFFu;
+                mkK |= (uint32_t)(acc[i] * invT + sm.ghi[noise_bound_index(c16)] >= thrK && acc[i] > -INFINITY) << i;
+              }
+            }
+          }
+        }
+      }
+      uint32_t mk = mkK | mkL;
+#pragma unroll 1
+      while (mk) {   // rare: hand the token to the selecting warp
+        const int i = __ffs(mk) - 1;
+        mk &= mk - 1;
+        const uint32_t kind = ((mkL >> i) & 1u) | ((mkK >> i) & 1u) << 1;
+        const uint32_t c16 = (pick8(cw0, cw1, i >> 1) >> (16 * (i & 1))) & 0xFFFFu;
+        const unsigned idx = atomicAdd(sm.q_tail, 1u);
+        uint32_t spin = 0;
+        while ((int)(idx - *sm.q_head) >= TX_QCAP) {   // queue full: the selecting warp is behind
+          if (*sm.abort) break;
+          if (++spin > a.wait_limit) { *sm.abort = 1; atomicExch(a.err, 1); break; }
+          __nanosleep(64);
+        }
+        uint4* e = sm.q + (idx & (TX_QCAP - 1));
+        e->x = (uint32_t)(v0 + i); e->y = __float_as_uint(pick16(acc, i));
+        e->z = ztag | (kind << 12) | (c16 << 16);
+        __threadfence_block();
+        *reinterpret_cast<volatile uint32_t*>(&e->w) = idx + 1u;   // tag: the entry is complete
+      }
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(sm.t_empty + slot);
+  }
+  sm.part[(0 * TX_SPLIT + s) * TX_ROWS + row] = m; sm.part[(1 * TX_SPLIT + s) * TX_ROWS + row] = s0; sm.part[(2 * TX_SPLIT + s) * TX_ROWS + row] = sT;
+  __threadfence_block();
+  __syncwarp();
+  if (lane == 0) atomicAdd((int*)sm.done, alive ? 1 : (1 << 20));   // one tick per warp per group (a large one releases the others after a failed wait)
+}
+
+// ---- the copying warp: base-logit rows of every block into the ring (and W, where no tensor map could be made) ----
+__device__ __forceinline__ void tx_copy(const TreeArgs& a, const TxSm& sm, const int nrow, const int t0, const int tlen, BlockPos& pos, BlockPos& wpos) {
+  const int lane = threadIdx.x & 31;
+  const int CB8 = a.BN / 8, nblk = (tlen + a.BN - 1) / a.BN;
+  const int sh = a.BN == 128 ? 4 : 3;             // log2 of the 16-byte chunks per row and block
+  const int ck = lane & (CB8 - 1), r0 = lane >> sh, rstep = 32 >> sh;
+  const __nv_bfloat16* Ug = reinterpret_cast<const __nv_bfloat16*>(a.Uscan);
+  for (int nb = 0; nb < nblk; ++nb, pos.next(a.nU)) {
+    if (pos.use >= 1 && !tx_wait(sm.t_empty + pos.slot, (pos.use - 1) & 1, sm, a)) return;
+    const int v = t0 + nb * a.BN + ck * 8;
+    const bool in = v < a.Vs;
+    unsigned char* dst = sm.Us + (size_t)pos.slot * (TX_ROWS * 2) * a.BN;
+    for (int rr = r0; rr < nrow; rr += rstep)
+      cp_async16(dst + (size_t)rr * 2 * a.BN + ((ck ^ (rr & 7)) << 4), in ? Ug + (size_t)sm.ent[rr].row * a.Vs + v : Ug, in);
+    cp_async_arrive(sm.u_full + pos.slot);
+    if (!a.use_tma) {
+      const int rw = (a.r + 15) / 16 * 16;
+      const __nv_bfloat16* Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wscan);
+      if (wpos.use >= 1 && !tx_wait(sm.w_free + wpos.slot, (wpos.use - 1) & 1, sm, a)) return;
+      unsigned char* wd = sm.Ws + (size_t)wpos.slot * rw * 2 * a.BN;
+      for (int k = r0; k < rw; k += rstep) {
+        const bool win = in && k < a.r;
+        cp_async16(wd + (size_t)(ck >> 3) * rw * 128 + k * 128 + (((ck & 7) ^ (k & 7)) << 4), win ? Wg + (size_t)k * a.Vs + v : Wg, win);
+      }
+      cp_async_wait_all();
+      fence_async_smem();
+      mbar_arrive(sm.w_full + wpos.slot);
+      wpos.next(a.nW);
+    }
+  }
+}
+
+// ---- the issuing lane: W blocks through their ring, one tile of MMAs per block ----------------------------------
+struct WStream { uint32_t requested, issued; };   // blocks of W asked for / handed to the tensor cores, whole launch
+
+__device__ __forceinline__ void tx_request_w(const TreeArgs& a, const TxSm& sm, const CUtensorMap* tm, const int t0, const int tlen, WStream& w, const uint32_t limit) {
+  const int nblk = (tlen + a.BN - 1) / a.BN, rw = (a.r + 15) / 16 * 16;
+  while (w.requested - w.issued < (uint32_t)a.nW && w.requested < limit) {
+    const uint32_t slot = w.requested % (uint32_t)a.nW, use = w.requested / (uint32_t)a.nW;
+    if (use >= 1 && !mbar_test_wait(sm.w_free + slot, (use - 1) & 1)) break;
+    const int nb = (int)(w.requested % (uint32_t)nblk);
+    const int ns = min(a.BN / 64, (tlen - nb * a.BN + 63) / 64);
+    mbar_expect_tx(sm.w_full + slot, (uint32_t)ns * rw * 128u);
+    for (int h = 0; h < ns; ++h)
+      tma_load_box(sm.Ws + ((size_t)slot * (a.BN / 64) + h) * rw * 128, tm, t0 + nb * a.BN + h * 64, 0, sm.w_full + slot);
+    ++w.requested;
+  }
+}
+
+__device__ __forceinline__ void tx_issue(const TreeArgs& a, const TxSm& sm, const CUtensorMap* tm, const int t0, const int tlen, const uint32_t tmem_base,
+                                         BlockPos& pos, WStream& w, const int group_no, const int groups_left, const bool run_ahead) {
+  const int nblk = (tlen + a.BN - 1) / a.BN, ksteps = (a.r + 15) / 16;
+  const uint32_t slab = (uint32_t)ksteps * 2048u;
+  // requests stop at the end of the level where owners will work in the ring, and run on into the next scan elsewhere:
+  // W does not depend on which parents that will score
+  const uint32_t limit = w.issued + (uint32_t)(nblk * groups_left + (run_ahead ? a.nW : 0));
+  if (a.use_tma) tx_request_w(a, sm, tm, t0, tlen, w, limit);
+  if (!tx_wait(sm.a_full, group_no & 1, sm, a)) return;
+  tc_fence_after();
+  const uint64_t adesc0 = smem_desc(smem_u32(sm.As), 16u, 1024u);
+  for (int nb = 0; nb < nblk; ++nb, pos.next(a.nU)) {
+    const uint32_t ws = w.issued % (uint32_t)a.nW, wu = w.issued / (uint32_t)a.nW;
+    if (a.use_tma) tx_request_w(a, sm, tm, t0, tlen, w, limit);
+    if (!tx_wait(sm.w_full + ws, wu & 1, sm, a)) return;
+    if (pos.use >= 1 && !tx_wait(sm.t_empty + pos.slot, (pos.use - 1) & 1, sm, a)) return;
+    tc_fence_after();
+    const int n = min(a.BN, (tlen - nb * a.BN + 63) / 64 * 64);   // whole 64-token slabs
+    const uint32_t idesc = instr_desc(n), d = tmem_base + (uint32_t)(pos.slot * a.BN);
+    const uint64_t bdesc0 = smem_desc(smem_u32(sm.Ws) + ws * (uint32_t)(a.BN / 64) * slab, slab, 1024u);
+    for (int ks = 0; ks < ksteps; ++ks)
+      mma_bf16(d, adesc0 + (uint64_t)((ks >> 2) * (TX_ROWS * 128 / 16) + (ks & 3) * 2), bdesc0 + (uint64_t)(ks * 128), idesc, ks > 0 ? 1u : 0u);
+    mma_commit(sm.t_full + pos.slot);
+    mma_commit(sm.w_free + ws);
+    ++w.issued;
+  }
+  if (a.use_tma) {
+    for (uint32_t i = 0; i < a.wait_limit && w.requested - w.issued < (uint32_t)a.nW && w.requested < limit; ++i) { tx_request_w(a, sm, tm, t0, tlen, w, limit); if (*sm.abort) break; }
+  }
+}
+
+// ---- the refreshing warp -----------------------------------------------------------------------------------------
+// Condenses the slots of the parents this CTA is responsible for (parent p belongs to range p mod ntiles) into two
+// words per parent and copies the condensed words of its rows into shared memory, until the scan is over.
+__device__ __forceinline__ void tx_refresh(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int tile, const int done_target) {
+  const int lane = threadIdx.x & 31, per = TX_ROWS / R, K = a.K;
+  const int p_lo = R > 1 ? 0 : g * TX_ROWS, p_hi = min(P, p_lo + per), nt = a.ntiles;
+  const int p_own = p_lo + ((tile - p_lo % nt + nt) % nt);
+  const int which = lane >> 4, j = lane & 15;
+  for (uint32_t spin = 0; spin < a.wait_limit; ++spin) {
+    if (*sm.done >= done_target || *sm.abort) break;
+    unsigned v = 0xFFFFFFFFu;
+    if (p_own < p_hi && j < K) v = __ldcg(a.slots + (((size_t)which * a.cap + p_own) * K + j) * SLOT_STRIDE);
+    unsigned rL[4], rK[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int rr = lane + 32 * k, p = p_lo + rr;
+      const bool in = rr < per && p < P;
+      rL[k] = in ? __ldcg(a.thr + p) : 0u;
+      rK[k] = in ? __ldcg(a.thr + (size_t)a.cap + p) : 0u;
+    }
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) v = min(v, __shfl_xor_sync(0xFFFFFFFFu, v, off));
+    if (p_own < p_hi && j == 0) __stcg(a.thr + (size_t)which * a.cap + p_own, v);
+    for (int p = p_own + nt; p < p_hi; p += nt) {
+      unsigned w = 0xFFFFFFFFu;
+      if (j < K) w = __ldcg(a.slots + (((size_t)which * a.cap + p) * K + j) * SLOT_STRIDE);
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) w = min(w, __shfl_xor_sync(0xFFFFFFFFu, w, off));
+      if (j == 0) __stcg(a.thr + (size_t)which * a.cap + p, w);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int rr = lane + 32 * k, p = p_lo + rr;
+      if (rr < per && p < P) {   // never below the seed bounds
+        sm.thr[rr] = fmaxf(dec_f(rL[k]), sm.ent[rr].thrL);
+        sm.thr[TX_ROWS + rr] = fmaxf(dec_f(rK[k]), sm.ent[rr].thrK);
+      }
+    }
+    __nanosleep(spin < 16u ? 100 : 500);
+  }
+  __syncwarp();
+}
+
+// ---- the selecting warp: drains the queue until the scan is over ----------------------------------------------------
+__device__ __forceinline__ void tx_drain(const TreeArgs& a, const TxSm& sm, const int R, const int g, const int tile, const int done_target) {
+  const int lane = threadIdx.x & 31;
+  const float invT = a.T > 0.f ? 1.f / a.T : 1.f;
+  unsigned head = *sm.q_head;
+  for (uint32_t spin = 0; spin < a.wait_limit; ++spin) {
+    if (*sm.abort) break;
+    const bool finished = *sm.done >= done_target;   // read before the tail: pushes precede the tick
+    const unsigned tail = *reinterpret_cast<volatile unsigned*>(sm.q_tail);
+    const int avail = (int)(tail - head);
+    if (avail <= 0) {
+      if (finished) break;
+      __nanosleep(100);
+      continue;
+    }
+    spin = 0;
+    const int n = min(avail, 32);
+    uint4 e = make_uint4(0u, 0u, 0u, 0u);
+    bool have = false;
+    if (lane < n) {
+      uint4* slot = sm.q + ((head + lane) & (TX_QCAP - 1));
+      uint32_t w = 0;
+      for (uint32_t t = 0; t < a.wait_limit; ++t) {   // the producer writes right after claiming: a few cycles
+        w = *reinterpret_cast<volatile uint32_t*>(&slot->w);
+        if (w == head + lane + 1u || *sm.abort) break;
+      }
+      have = (w == head + lane + 1u);
+      __threadfence_block();
+      if (have) { e.x = slot->x; e.y = slot->y; e.z = slot->z; }
+    }
+    __threadfence_block();
+    __syncwarp();
+    head += (unsigned)n;
+    if (lane == 0) *sm.q_head = head;   // the slots may be reused
+    // candidates of one row are inserted one after the other (lanes of a row take turns)
+    const unsigned peers = __match_any_sync(0xFFFFFFFFu, have ? (int)(e.z & 0xFFu) : -1 - lane);
+    const int turn = __popc(peers & ((1u << lane) - 1u));
+    const int turns = __reduce_max_sync(0xFFFFFFFFu, have ? turn + 1 : 0);
+    for (int t = 0; t < turns; ++t) {
+      if (have && turn == t) tx_select(a, sm, e, invT, tile, R, g);
+      __syncwarp();
+    }
+  }
+}
+
+// ---- end of a group: the range's sums and surviving candidates of every parent -------------------------------------
+__device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int tile) {
+  const int tid = threadIdx.x, per = TX_ROWS / R, K = a.K;
+  if (tid >= TX_ROWS) return;
+  const int row = tid, prow = R > 1 ? row % per : row, p = R > 1 ? prow : g * TX_ROWS + row;
+  if (p >= P) return;
+  const float T = a.T, invT = T > 0.f ? 1.f / T : 1.f;
+  if (row < per) {
+    // the pieces' sums in a fixed order: the same bits on every run
+    float m = -INFINITY, s0 = 0.f, sT = 0.f;
+    for (int rho = 0; rho < R; ++rho)
+#pragma unroll
+      for (int s = 0; s < TX_SPLIT; ++s) {
+        const int rr = rho * per + row;
+        const float hm = sm.part[(0 * TX_SPLIT + s) * TX_ROWS + rr], h0 = sm.part[(1 * TX_SPLIT + s) * TX_ROWS + rr], hT = sm.part[(2 * TX_SPLIT + s) * TX_ROWS + rr];
+        if (hm == -INFINITY) { s0 += h0; continue; }   // (nothing finite: h0 is 0, or NaN if the piece met one)
+        if (hm > m) { const float d = m == -INFINITY ? 0.f : m - hm; s0 *= __expf(d); sT *= __expf(d * invT); m = hm; }
+        const float d = hm - m;
+        s0 += h0 * __expf(d); sT += hT * __expf(d * invT);
+      }
+    a.sums[(size_t)p * a.ntiles + tile] = make_float4(m, s0, sT, 0.f);
+  }
+  const size_t base = (size_t)p * a.ntiles * (R * K);
+  const float gL = sm.thr[prow], gK = sm.thr[TX_ROWS + prow];
+  const float* L = sm.lists + (size_t)row * 5 * K;
+  const int* Li = reinterpret_cast<const int*>(L);
+  int n = sm.ln[row], k = 0;
+  while (k < n && L[k] >= gL) ++k;
+  if (k) {
+    const int at = atomicAdd(a.cand_cnt + p, k);
+    for (int j = 0; j < k; ++j) a.cand_top[base + at + j] = make_uint2(__float_as_uint(L[j]), (unsigned)Li[K + j]);
+  }
+  n = sm.ln[TX_ROWS + row]; k = 0;
+  while (k < n && L[2 * K + k] >= gK) ++k;
+  if (k) {
+    const int at = atomicAdd(a.cand_cnt + a.cap + p, k);
+    for (int j = 0; j < k; ++j) {
+      a.cand_key[base + at + j] = make_uint2(__float_as_uint(L[2 * K + j]), (unsigned)Li[3 * K + j]);
+      a.cand_lg[base + at + j] = L[4 * K + j];
+    }
+  }
+}
+
+// ---- merge of one parent, by one warp --------------------------------------------------------------------------------
+// The K best of n (value, token) pairs (value desc, token asc): lane j < K gets the j-th in (tok, val, lg).  Batches of
+// up to 224 entries in registers beside the winners so far; a round is two warp-wide maxima (the value's order-
+// preserving image, then the inverted token among its ties) and one removal.
+__device__ __forceinline__ void warp_topk(const uint2* cand, const float* lgs, int n, int K, int lane, int& tok, float& val, float& lg) {
+  uint32_t wv = 0u, wt = 0u; float wl = 0.f;   // winner `lane` so far: 0 = none
+  for (int base = 0; base < n; base += 7 * 32) {
+    uint32_t ev[8], et[8]; float el[8];
+    ev[0] = wv; et[0] = wt; el[0] = wl;
+#pragma unroll
+    for (int u = 1; u < 8; ++u) {
+      const int i = base + (u - 1) * 32 + lane;
+      ev[u] = 0u; et[u] = 0u; el[u] = 0.f;
+      if (i < n) {
+        const uint2 c = __ldcg(cand + i);
+        ev[u] = enc_f(__uint_as_float(c.x)); et[u] = ~c.y;
+        el[u] = lgs ? __ldcg(lgs + i) : __uint_as_float(c.x);
+      }
+    }
+    wv = 0u; wt = 0u; wl = 0.f;
+    for (int j = 0; j < K; ++j) {
+      uint32_t bv = ev[0], bt = et[0]; float bl = el[0];
+#pragma unroll
+      for (int u = 1; u < 8; ++u)
+        if (ev[u] > bv || (ev[u] == bv && et[u] > bt)) { bv = ev[u]; bt = et[u]; bl = el[u]; }
+      const uint32_t mv = __reduce_max_sync(0xFFFFFFFFu, bv);
+      if (mv == 0u) break;   // warp-uniform
+      const uint32_t mt = __reduce_max_sync(0xFFFFFFFFu, bv == mv ? bt : 0u);
+      const bool mine = bv == mv && bt == mt;
+      const unsigned who = __ballot_sync(0xFFFFFFFFu, mine);
+      const float l = __shfl_sync(0xFFFFFFFFu, bl, __ffs(who) - 1);
+      if (mine) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) if (ev[u] == mv && et[u] == mt) { ev[u] = 0u; et[u] = 0u; }
+      }
+      if (lane == j) { wv = mv; wt = mt; wl = l; }
+    }
+  }
+  tok = wv ? (int)~wt : -1; val = wv ? dec_f(wv) : 0.f; lg = wv ? wl : 0.f;
+}
+
+// Log-normalisers of a parent from its ranges' sums; every lane gets them.
+__device__ __forceinline__ void warp_lse(const TreeArgs& a, int p, int lane, float& lse0, float& lseT) {
+  const float T = a.T, invT = T > 0.f ? 1.f / T : 1.f;
+  const float4* h = a.sums + (size_t)p * a.ntiles;
+  float m = -INFINITY, s0 = 0.f, sT = 0.f;
+  for (int t0 = 0; t0 < a.ntiles; t0 += 5 * 32) {
+    float4 x[5];
+#pragma unroll
+    for (int u = 0; u < 5; ++u) { const int t = t0 + u * 32 + lane; x[u] = t < a.ntiles ? __ldcg(h + t) : make_float4(-INFINITY, 0.f, 0.f, 0.f); }
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+      if (x[u].x == -INFINITY) { s0 += x[u].y; continue; }
+      if (x[u].x > m) { const float d = m == -INFINITY ? 0.f : m - x[u].x; s0 *= __expf(d); sT *= __expf(d * invT); m = x[u].x; }
+      const float d = x[u].x - m;
+      s0 += x[u].y * __expf(d); sT += x[u].z * __expf(d * invT);
+    }
+  }
+  float gm = m;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xFFFFFFFFu, gm, off));
+  if (m > -INFINITY) { s0 *= __expf(m - gm); sT *= __expf((m - gm) * invT); }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) { s0 += __shfl_xor_sync(0xFFFFFFFFu, s0, off); sT += __shfl_xor_sync(0xFFFFFFFFu, sT, off); }
+  lse0 = gm + logf(s0);
+  lseT = T > 0.f ? gm * invT + logf(sT) : lse0;
+}
+
+// ---- seed bounds ------------------------------------------------------------------------------------------------------
+// Best base logit (and its token) of one piece of one row, by one warp; a ragged vocabulary's rows are copied to
+// their padded places on the way.
+__device__ __forceinline__ void scout_piece(const TreeArgs& a, int row, int piece, int piece_len, uint2* out, int lane) {
+  const int lo = piece * piece_len, hi = min(a.V, lo + piece_len);
+  const __nv_bfloat16* src = reinterpret_cast<const __nv_bfloat16*>(a.U) + (size_t)row * a.V;
+  float bv = -INFINITY; int bi = 0x7FFFFFFF;
+  uint4 x[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int v = lo + (u * 32 + lane) * 8;
+    x[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);   // -inf
+    if (v < hi) {
+      if (!a.ragged) x[u] = __ldg(reinterpret_cast<const uint4*>(src + v));
+      else {
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t e0 = v + 2 * i < a.V ? __ldg(reinterpret_cast<const unsigned short*>(src) + v + 2 * i) : 0xFF80u;
+          const uint32_t e1 = v + 2 * i + 1 < a.V ? __ldg(reinterpret_cast<const unsigned short*>(src) + v + 2 * i + 1) : 0xFF80u;
+          w[i] = e0 | (e1 << 16);
+        }
+        x[u] = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(const_cast<__nv_bfloat16*>(reinterpret_cast<const __nv_bfloat16*>(a.Uscan)) + (size_t)row * a.Vs + v) = x[u];
+      }
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    float f[8];
+    unpack_bf16x8(x[u], f);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) if (f[i] > bv) { bv = f[i]; bi = lo + (u * 32 + lane) * 8 + i; }
+  }
+  const unsigned e = bi == 0x7FFFFFFF ? 0u : enc_f(bv);
+  const unsigned mv = __reduce_max_sync(0xFFFFFFFFu, e);
+  const unsigned mt = __reduce_min_sync(0xFFFFFFFFu, (e == mv && e != 0u) ? (unsigned)bi : 0x7FFFFFFFu);
+  if (lane == 0) *out = make_uint2(mv, mt);   // (0: nothing above -inf in the piece)
+}
+
+// The seed tokens of one row: the best of its pieces, picked by one warp (lane j: the j-th).
+__device__ __forceinline__ void pick_seeds(const TreeArgs& a, const uint2* ut, int NS, int* stok, float* sval, int lane) {
+  uint32_t ev[8], et[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) { ev[u] = 0u; et[u] = 0u; }
+  for (int i0 = 0; i0 < a.npiece; i0 += 256) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u * 32 + lane;
+      if (i < a.npiece) {
+        const uint2 e = __ldcg(ut + i);
+        if (e.x > ev[u]) { ev[u] = e.x; et[u] = e.y; }   // (beyond 256 pieces the best of every 256th: any tokens give valid bounds)
+      }
+    }
+  }
+  int tok = -1; float val = -INFINITY;
+  for (int j = 0; j < NS; ++j) {
+    uint32_t bv = ev[0], bt = et[0];
+#pragma unroll
+    for (int u = 1; u < 8; ++u) if (ev[u] > bv) { bv = ev[u]; bt = et[u]; }
+    const uint32_t mv = __reduce_max_sync(0xFFFFFFFFu, bv);
+    if (mv == 0u) break;
+    const int src = __ffs(__ballot_sync(0xFFFFFFFFu, bv == mv)) - 1;
+    const uint32_t t = __shfl_sync(0xFFFFFFFFu, bt, src);
+    if (lane == src) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) if (ev[u] == mv && et[u] == t) ev[u] = 0u;
+    }
+    if (lane == j) { tok = (int)t; val = dec_f(mv); }
+  }
+  if (lane < NS) { stok[lane] = tok; sval[lane] = val; }
+}
+
+// Shared-memory pieces of an owner (offsets of OwnerLayout).
+struct OwnerSm {
+  PoolView pv; float *lse0, *lseT; int* pslot; int *ttok, *dtok; float *tlog, *dlog; double *ckey, *clogS;
+  unsigned char *valid, *best; int *hist, *newl, *tcnt, *toff, *npl; uint32_t* Wc; int* stok; float* sval; float* res;
+};
+__device__ __forceinline__ OwnerSm owner_carve(unsigned char* sm, const TreeArgs& a) {
+  const int N = a.N, K = a.K;
+  const OwnerLayout o = owner_layout(N, K, a.r);
+  OwnerSm s;
+  s.pv = pool_view(sm + o.pool, N);
+  s.lse0 = reinterpret_cast<float*>(sm + o.lse); s.lseT = s.lse0 + N; s.pslot = reinterpret_cast<int*>(s.lseT + N);
+  s.ttok = reinterpret_cast<int*>(sm + o.toks); s.dtok = s.ttok + N * K; s.tlog = reinterpret_cast<float*>(s.dtok + N * K); s.dlog = s.tlog + N * K;
+  s.ckey = reinterpret_cast<double*>(sm + o.cand); s.clogS = s.ckey + N * K; s.res = reinterpret_cast<float*>(sm + o.cand);
+  s.valid = sm + o.flags; s.best = s.valid + N * K;
+  s.hist = reinterpret_cast<int*>(sm + o.lists); s.newl = s.hist + 256; s.tcnt = s.newl + 256; s.toff = s.tcnt + 256; s.npl = s.toff + 256;
+  s.Wc = reinterpret_cast<uint32_t*>(sm + o.seeds);
+  s.stok = reinterpret_cast<int*>(s.Wc + (size_t)seed_count(K) * (a.r + 1)); s.sval = reinterpret_cast<float*>(s.stok + 32);
+  return s;
+}
+
+// The seed tokens' columns of W on their way into shared memory (words of two tokens; rows of r + 1 words: the threads
+// that later read one k of different tokens hit different banks).  All threads; cp_async_wait_all and a barrier follow.
+__device__ __forceinline__ void fetch_seed_columns(const TreeArgs& a, const OwnerSm& s, int NS) {
+  const __nv_bfloat16* Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wscan);
+  for (int e = threadIdx.x; e < NS * a.r; e += TX_THREADS) {
+    const int j = e % NS, k = e / NS, tok = s.stok[j];
+    cp_async4(s.Wc + (size_t)j * (a.r + 1) + k, tok >= 0 ? Wg + (size_t)k * a.Vs + (tok & ~1) : Wg, tok >= 0);
+  }
+}
+
+// Seed bounds and list entries of `cnt` parents of one row (all threads; the columns have landed).  Parent i: token
+// s.ttok[i], hash hs[i], pool slot s.npl[i]; its place in the level's list is li0 + i.
+__device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s, const int cnt, const int li0, const int req, const int row, const int NS,
+                                             const int* ptok, const uint64_t* phash, ParentEntry* ent, int* ent_slot) {
+  const int tid = threadIdx.x, r = a.r, K = a.K;
+  const float invT = a.T > 0.f ? 1.f / a.T : 1.f;
+  const __nv_bfloat16* Ag = reinterpret_cast<const __nv_bfloat16*>(a.A);
+  // the parents' pruning state and candidate counts start clean
+  for (int e = tid; e < cnt * 2 * K; e += TX_THREADS) {
+    const int i = e / (2 * K), w = (e / K) & 1, j = e % K;
+    a.slots[(((size_t)w * a.cap + li0 + i) * K + j) * SLOT_STRIDE] = 0u;
+  }
+  for (int e = tid; e < cnt * 2; e += TX_THREADS) {
+    a.thr[(size_t)(e & 1) * a.cap + li0 + (e >> 1)] = 0u;
+    a.cand_cnt[(size_t)(e & 1) * a.cap + li0 + (e >> 1)] = 0;
+  }
+  // every (parent, seed token) pair exactly: eight lanes a pair, 16 bytes of the head row a lane and step
+  const int sub = tid & 7;
+  for (int e0 = 0; e0 < cnt * NS; e0 += TX_THREADS / 8) {
+    const int e = e0 + (tid >> 3);
+    const bool have = e < cnt * NS;
+    const int i = have ? e / NS : 0, j = have ? e % NS : 0, tok = s.stok[j];
+    float dot = 0.f;
+    if (have && tok >= 0) {
+      const uint32_t* wc = s.Wc + (size_t)j * (r + 1);
+      const int hi = tok & 1;
+      for (int k = sub * 8; k < r; k += 64) {
+        float av[8];
+        unpack_bf16x8(__ldg(reinterpret_cast<const uint4*>(Ag + (size_t)ptok[i] * r + k)), av);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) { const uint32_t w = wc[k + u]; dot = fmaf(av[u], __uint_as_float(hi ? (w & 0xFFFF0000u) : (w << 16)), dot); }
+      }
+    }
+    dot += __shfl_xor_sync(0xFFFFFFFFu, dot, 1); dot += __shfl_xor_sync(0xFFFFFFFFu, dot, 2); dot += __shfl_xor_sync(0xFFFFFFFFu, dot, 4);
+    if (have && sub == 0) {
+      float lg = -INFINITY, key = -INFINITY;
+      if (tok >= 0) {
+        lg = s.sval[j] + dot;
+        key = a.T > 0.f ? exact_key(a.seed, req, phash[i], tok, lg, invT) : lg;
+      }
+      s.res[2 * e] = lg; s.res[2 * e + 1] = key;
+    }
+  }
+  float* bL = reinterpret_cast<float*>(s.tcnt); float* bK = reinterpret_cast<float*>(s.toff); float* bM = reinterpret_cast<float*>(s.hist);
+  for (int i = tid; i < cnt; i += TX_THREADS) { bL[i] = -INFINITY; bK[i] = -INFINITY; bM[i] = -INFINITY; }
+  __syncthreads();
+  for (int e = tid; e < 2 * cnt * NS; e += TX_THREADS) {
+    // one thread per value: the one with exactly K - 1 values before it (ties broken by place) is the K-th best
+    const int j = e % NS, which = (e / NS) & 1, i = e / (2 * NS);
+    const float* val = s.res + (size_t)i * NS * 2 + which;
+    const float mine = val[2 * j];
+    int before = 0;
+    for (int t = 0; t < NS; ++t) before += (val[2 * t] > mine || (val[2 * t] == mine && t < j)) ? 1 : 0;
+    const bool fin = mine == mine && fabsf(mine) < INFINITY;
+    if (before == K - 1 && fin && !a.no_seed) {
+      // rounding of an r-term fp32 sum in another order, of the division by T and of the fast logarithms
+      const float margin = (2e-4f + 4e-5f * fabsf(mine)) * (which == 0 ? 1.f : fmaxf(invT, 1.f)) + (which == 0 ? 0.f : 2e-4f);
+      (which ? bK : bL)[i] = mine - margin;
+    }
+    if (before == 0 && which == 0 && fin) bM[i] = mine;
+  }
+  __syncthreads();
+  for (int i = tid; i < cnt; i += TX_THREADS) {
+    ParentEntry pe;
+    pe.row = row; pe.token = ptok[i]; pe.hash = phash[i]; pe.thrL = bL[i]; pe.thrK = a.T > 0.f ? bK[i] : -INFINITY; pe.mref = bM[i]; pe.req = req;
+    const uint4* src = reinterpret_cast<const uint4*>(&pe);
+    uint4* dst = reinterpret_cast<uint4*>(ent + li0 + i);
+    dst[0] = src[0]; dst[1] = src[1];
+    if (ent_slot) ent_slot[li0 + i] = s.npl[i];
+  }
+}
+
+__device__ __forceinline__ void tx_caps(const TreeArgs& a, int b, int& K_eff, int& N_eff, double& log_theta) {
+  const float th = a.theta[b];
+  K_eff = a.K < a.V ? a.K : a.V; N_eff = a.N;
+  if (th >= 1.f) { K_eff = 1; N_eff = a.D < a.N ? a.D : a.N; log_theta = -INFINITY; }   // chain member of the price ladder
+  else log_theta = th > 0.f ? log((double)th) : -INFINITY;
+}
+
+// The start of a request: an empty pool and the root as the only parent of level 0 (its seed bounds come from the
+// sweep of the depth-0 row that every CTA has just finished).
+__device__ __noinline__ void tx_root(const TreeArgs& a, unsigned char* sm, const int b) {
+  const OwnerSm s = owner_carve(sm, a);
+  const int tid = threadIdx.x, NS = seed_count(a.K);
+  __shared__ int tok0; __shared__ uint64_t hash0;
+  PoolView g = pool_view(a.pool + (size_t)b * a.pool_stride, a.N);
+  for (int i = tid; i < a.N; i += TX_THREADS) g.meta[i] = 0;
+  if (tid == 0) {
+    const int t = a.anchor[b];
+    const bool ok = t >= 0 && t < a.V && a.theta[b] == a.theta[b];
+    a.status[b] = ok ? TS_OK : TS_ERR_INVALID;
+    tok0 = ok ? t : 0; hash0 = 0ull; s.npl[0] = -1;
+    a.req_npar[b] = 1; a.req_base[b] = b; a.req_nscored[b] = 0;
+    a.root_lseT[b] = nanf("");
+  }
+  if ((tid >> 5) == 1) pick_seeds(a, a.utop + (size_t)b * a.npiece, NS, s.stok, s.sval, tid & 31);
+  __syncthreads();
+  fetch_seed_columns(a, s, NS);
+  cp_async_wait_all();
+  __syncthreads();
+  make_parents(a, s, 1, b, b, b * a.D, NS, &tok0, &hash0, a.ent[0], a.ent_slot[0]);
+  __syncthreads();
+}
+
+// A given parent of ts_score_parents: list place i.
+__device__ __noinline__ void tx_given(const TreeArgs& a, unsigned char* sm, const int i) {
+  const OwnerSm s = owner_carve(sm, a);
+  const int tid = threadIdx.x, NS = seed_count(a.K);
+  __shared__ int tok0; __shared__ uint64_t hash0;
+  const int req = a.p_req[i], dep = a.p_depth[i];
+  if (tid == 0) { tok0 = a.p_token[i]; hash0 = a.p_hash[i]; }
+  if ((tid >> 5) == 1) pick_seeds(a, a.utop + (size_t)i * a.npiece, NS, s.stok, s.sval, tid & 31);
+  __syncthreads();
+  fetch_seed_columns(a, s, NS);
+  cp_async_wait_all();
+  __syncthreads();
+  make_parents(a, s, 1, i, req, req * a.D + dep, NS, &tok0, &hash0, a.ent[0], nullptr);
+  __syncthreads();
+}
+
+// One level of one request: merge of its parents, slots and cut of Algorithm 1, the next level's parents.
+// d = depth of the parents just scanned.
+__device__ __noinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, const int b, const int d) {
+  const OwnerSm s = owner_carve(sm, a);
+  __shared__ int sh[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int N = a.N, K = a.K, cur = d & 1, nxt = cur ^ 1, NS = seed_count(K);
+  const int npar = __ldcg(a.req_npar + cur * a.B + b), base = __ldcg(a.req_base + b);
+  if (npar == 0 || __ldcg(a.status + b) != TS_OK) {   // uniform: nothing below has run yet
+    if (tid == 0) a.req_npar[nxt * a.B + b] = 0;
+    return;
+  }
+  int K_eff, N_eff; double log_theta;
+  tx_caps(a, b, K_eff, N_eff, log_theta);
+  const bool more = d + 1 < a.D;
+  unsigned char* gpool = a.pool + (size_t)b * a.pool_stride;
+  {
+    uint4* dst = reinterpret_cast<uint4*>(s.pv.key); const uint4* src = reinterpret_cast<const uint4*>(gpool);
+    for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) dst[i] = __ldcg(src + i);
+  }
+  for (int i = tid; i < npar; i += TX_THREADS) s.pslot[i] = __ldcg(a.ent_slot[cur] + base + i);
+  if (tid < 8) sh[tid] = 0;
+  // ---- merge: one warp per parent (the last warp picks the next level's seed tokens meanwhile) ----
+  if (warp == TX_WARPS - 1) {
+    if (more) pick_seeds(a, a.utop + ((size_t)nxt * a.B + b) * a.npiece, NS, s.stok, s.sval, lane);
+  } else {
+    for (int i = warp; i < npar; i += TX_WARPS - 1) {
+      const int p = base + i;
+      const int P = __ldcg(a.lvl_count + d), R = mma_replicas(P);
+      const int nt = __ldcg(a.cand_cnt + p), nk = __ldcg(a.cand_cnt + a.cap + p);
+      const size_t cb = (size_t)p * a.ntiles * (R * K);
+      float l0, lT, val, lg; int tok;
+      warp_lse(a, p, lane, l0, lT);
+      warp_topk(a.cand_top + cb, nullptr, nt, K, lane, tok, val, lg);
+      const int ttok = tok; const float tlog = val;
+      int dtok = ttok; float dlog = tlog;
+      if (a.T > 0.f) { warp_topk(a.cand_key + cb, a.cand_lg + cb, nk, K, lane, tok, val, lg); dtok = tok; dlog = lg; }
+      if (lane < K) { s.ttok[i * K + lane] = ttok; s.tlog[i * K + lane] = tlog; s.dtok[i * K + lane] = dtok; s.dlog[i * K + lane] = dlog; }
+      if (lane == 0) { s.lse0[i] = l0; s.lseT[i] = lT; }
+      // the best token of q0 not among the first j draws, for every j: places of the draws in the top list, or-ed up
+      unsigned used = 0u;
+      for (int t = 0; t < K; ++t) { const int tt = __shfl_sync(0xFFFFFFFFu, ttok, t); if (lane < K && tt == dtok && tt >= 0) used |= 1u << t; }
+      if (!(a.T > 0.f)) used = lane < K ? 1u << lane : 0u;
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) { const unsigned u = __shfl_up_sync(0xFFFFFFFFu, used, o); if (lane >= o) used |= u; }
+      const unsigned before = __shfl_up_sync(0xFFFFFFFFu, used, 1);
+      if (lane < K) { const unsigned freeb = ~(lane ? before : 0u) & ((1u << K_eff) - 1u); s.best[i * K + lane] = freeb ? (unsigned char)(__ffs(freeb) - 1) : 255u; }
+    }
+  }
+  __syncthreads();
+  if (more) fetch_seed_columns(a, s, NS);   // lands while the slots are formed
+  // ---- slots of every scored parent, one thread per (parent, sibling rank) ----
+  for (int t = tid; t < npar * K; t += TX_THREADS) {
+    const int i = t / K, j = t % K;
+    const double lse0 = s.lse0[i], lseT = s.lseT[i];
+    const int slot = s.pslot[i];
+    const bool bad = !(lse0 == lse0) || isinf(lse0);
+    if (j == 0) {
+      if (slot < 0) a.root_lseT[b] = (float)lseT; else s.pv.lseT[slot] = (float)lseT;
+      if (bad) a.status[b] = TS_ERR_NUMERIC;
+    }
+    int ok = 0;
+    if (j < K_eff && !bad) {
+      const int bi = s.best[t], x = s.dtok[t];
+      if (bi < K_eff && s.ttok[i * K + bi] >= 0 && x >= 0) {
+        const double logS_v = slot < 0 ? 0.0 : s.pv.logS[slot];
+        // the calibrator's input: the untempered conditional, or (ablation) the tempered one
+        const bool tempered = a.calib_qT && a.T > 0.f;
+        const double lsc = tempered ? 1.0 / (double)a.T : 1.0, lsn = tempered ? lseT : lse0;
+        const double key = logS_v + log_phat(a.calib, d, (double)s.tlog[i * K + bi] * lsc, lsn);
+        if (!(key < log_theta)) {
+          ok = 1;
+          s.ckey[t] = key;
+          s.clogS[t] = logS_v + log_phat(a.calib, d, (double)s.dlog[t] * lsc, lsn);
+        }
+      }
+    }
+    s.valid[t] = (unsigned char)ok;
+  }
+  __syncthreads();
+  // a sibling slot exists only if the one before it was admitted (keys are non-increasing in j)
+  {
+    int nv = 0, np = 0;
+    for (int i = tid; i < npar; i += TX_THREADS) {
+      bool open = true;
+      for (int j = 0; j < K; ++j) { if (!s.valid[i * K + j]) open = false; if (open) ++nv; else s.valid[i * K + j] = 0; }
+    }
+    for (int i = tid; i < N; i += TX_THREADS) np += s.pv.meta[i] >> 16;
+    nv = __reduce_add_sync(0xFFFFFFFFu, nv); np = __reduce_add_sync(0xFFFFFFFFu, np);
+    if (lane == 0) { if (np) atomicAdd(&sh[0], np); if (nv) atomicAdd(&sh[1], nv); }
+  }
+  __syncthreads();
+  const int ncand = npar * K, shift = 60 - 4 * d;
+  auto skey = [](double k) -> uint64_t {
+    if (k == 0.0) k = 0.0;   // -0 and +0 compare equal: one pattern
+    const uint64_t u = (uint64_t)__double_as_longlong(k);
+    return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
+  };
+  // entry e: a pool slot (e < N) or a candidate
+  const int M = N + ncand;
+  auto live = [&](int e) -> bool { return e < N ? (s.pv.meta[e] >> 16) != 0 : s.valid[e - N] != 0; };
+  auto key_of = [&](int e) -> double { return e < N ? s.pv.key[e] : s.ckey[e - N]; };
+  auto depth_of = [&](int e) -> int { return e < N ? (s.pv.meta[e] >> 8) & 255 : d + 1; };
+  auto path_of = [&](int e) -> uint64_t {
+    if (e < N) return s.pv.path[e];
+    const int c = e - N, slot = s.pslot[c / K];
+    return (slot < 0 ? 0ull : s.pv.path[slot]) | ((uint64_t)(c % K) << shift);
+  };
+  if (sh[0] + sh[1] > N_eff) {
+    // The N_eff-th largest key by radix selection over the keys' order-preserving bit patterns (eight bits a pass);
+    // entries above it stay, entries below it go, and those that tie with it are ranked among themselves by
+    // (depth, path) for the places that are left.
+    uint64_t prefix = 0;
+    int need = N_eff;
+    for (int sh8 = 56; sh8 >= 0; sh8 -= 8) {
+      if (tid < 256) s.hist[tid] = 0;
+      __syncthreads();
+      for (int e = tid; e < M; e += TX_THREADS) {
+        if (!live(e)) continue;
+        const uint64_t k = skey(key_of(e));
+        if (sh8 == 56 || (k >> (sh8 + 8)) == (prefix >> (sh8 + 8))) atomicAdd(&s.hist[(int)((k >> sh8) & 255u)], 1);
+      }
+      __syncthreads();
+      if (warp == 0) {
+        // lane l owns bins 255 - 8l .. 248 - 8l (descending); the bin where the running count reaches `need`
+        int mine = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) mine += s.hist[255 - 8 * lane - j];
+        int incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o); if (lane >= o) incl += v; }
+        const unsigned reach = __ballot_sync(0xFFFFFFFFu, incl >= need);
+        if (lane == __ffs(reach) - 1) {   // reach != 0: at least `need` entries match the prefix
+          int cum = incl - mine, bin = 255 - 8 * lane;
+          for (int j = 0; j < 8; ++j) {
+            const int h = s.hist[255 - 8 * lane - j];
+            if (cum + h >= need) { bin = 255 - 8 * lane - j; break; }
+            cum += h;
+          }
+          sh[2] = bin; sh[3] = need - cum;
+        }
+      }
+      __syncthreads();
+      prefix |= (uint64_t)sh[2] << sh8;
+      need = sh[3];
+    }
+    if (tid == 0) sh[4] = 0;
+    __syncthreads();
+    for (int e = tid; e < M; e += TX_THREADS)
+      if (live(e) && skey(key_of(e)) == prefix) { const int at = atomicAdd(&sh[4], 1); if (at < 256) s.newl[at] = e; }
+    __syncthreads();
+    const int ntie = sh[4];
+    unsigned drop = 0u;   // bit per trip: M <= 17 * 256 entries, at most 7 trips
+    for (int e = tid, it = 0; e < M; e += TX_THREADS, ++it) {
+      if (!live(e)) continue;
+      const double ke = key_of(e);
+      const uint64_t k = skey(ke);
+      bool out = k < prefix;
+      if (k == prefix && ntie > need) {
+        int rank = 0;
+        const int de = depth_of(e); const uint64_t pe = path_of(e);
+        const int nn = ntie <= 256 ? ntie : M;
+        for (int t = 0; t < nn; ++t) {
+          const int f = ntie <= 256 ? s.newl[t] : t;
+          if (f == e || (ntie > 256 && !(live(f) && skey(key_of(f)) == prefix))) continue;
+          if (before(key_of(f), depth_of(f), path_of(f), ke, de, pe)) ++rank;
+        }
+        out = rank >= need;
+      }
+      drop |= (out ? 1u : 0u) << it;
+    }
+    __syncthreads();
+    for (int e = tid, it = 0; e < M; e += TX_THREADS, ++it)
+      if ((drop >> it) & 1u) { if (e < N) s.pv.meta[e] &= 0xFFFF; else s.valid[e - N] = 0; }
+    __syncthreads();
+  }
+  // ---- placement: the t-th surviving candidate (in candidate order) takes the t-th free slot (in slot order) ----
+  {
+    const bool fr = tid < N && (s.pv.meta[tid] >> 16) == 0;
+    const unsigned bal = __ballot_sync(0xFFFFFFFFu, fr);
+    if (lane == 0 && warp < 8) s.npl[warp] = __popc(bal);
+    const int ntrip = (ncand + TX_THREADS - 1) / TX_THREADS;   // <= 7
+    unsigned vm = 0;
+    for (int it = 0; it < ntrip; ++it) {
+      const int c = it * TX_THREADS + tid;
+      const bool v = c < ncand && s.valid[c];
+      const unsigned vb = __ballot_sync(0xFFFFFFFFu, v);
+      vm |= (v ? 1u : 0u) << it;
+      if (lane == 0) s.tcnt[it * TX_WARPS + warp] = __popc(vb);
+    }
+    __syncthreads();
+    int off = 0, nfree = 0;
+    for (int w = 0; w < 8; ++w) { if (w < warp) off += s.npl[w]; nfree += s.npl[w]; }
+    if (fr) s.hist[off + __popc(bal & ((1u << lane) - 1u))] = tid;
+    const int ne = ntrip * TX_WARPS;
+    if (warp == 0) {   // exclusive prefix over (trip, warp)
+      int run = 0;
+      for (int e0 = 0; e0 < ne; e0 += 32) {
+        const int e = e0 + lane, c = e < ne ? s.tcnt[e] : 0;
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o); if (lane >= o) incl += v; }
+        if (e < ne) s.toff[e] = run + incl - c;
+        run += __shfl_sync(0xFFFFFFFFu, incl, 31);
+      }
+      if (lane == 0) sh[5] = min(run, nfree);
+      if (lane == 0 && run > nfree) a.status[b] = TS_ERR_OVERFLOW;
+    }
+    __syncthreads();
+    for (int it = 0; it < ntrip; ++it) {
+      const bool v = (vm >> it) & 1u;
+      const unsigned vb = __ballot_sync(0xFFFFFFFFu, v);
+      if (!v) continue;
+      const int c = it * TX_THREADS + tid, t = s.toff[it * TX_WARPS + warp] + __popc(vb & ((1u << lane) - 1u));
+      if (t >= nfree) continue;
+      const int sl = s.hist[t], i = c / K, j = c % K, slot = s.pslot[i], x = s.dtok[c];
+      const double lx = s.dlog[c], lse0 = s.lse0[i], lseT = s.lseT[i];
+      s.pv.meta[sl] = (1 << 16) | ((d + 1) << 8) | j; s.pv.parent[sl] = slot; s.pv.tok[sl] = x;
+      s.pv.key[sl] = s.ckey[c]; s.pv.logS[sl] = s.clogS[c];
+      s.pv.q0[sl] = (float)exp(lx - lse0);
+      s.pv.logqT[sl] = a.T > 0.f ? (float)(lx / (double)a.T - lseT) : (float)(lx - lse0);
+      s.pv.lseT[sl] = nanf("");
+      s.pv.hash[sl] = path_hash(slot < 0 ? 0ull : s.pv.hash[slot], x);
+      s.pv.path[sl] = (slot < 0 ? 0ull : s.pv.path[slot]) | ((uint64_t)j << shift);
+      s.newl[t] = sl;
+    }
+  }
+  __syncthreads();
+  const int nnew = sh[5];
+  // ---- next level's parents: new nodes that can still have admissible children ----
+  {
+    const bool par = more && tid < nnew && !(s.pv.logS[s.newl[tid]] < log_theta);
+    const unsigned bal = __ballot_sync(0xFFFFFFFFu, par);
+    if (lane == 0 && warp < 8) s.tcnt[warp] = __popc(bal);
+    __syncthreads();
+    int off = 0, cnt = 0;
+    for (int w = 0; w < 8; ++w) { if (w < warp) off += s.tcnt[w]; cnt += s.tcnt[w]; }
+    if (tid == 0) {
+      const int nb = cnt > 0 ? atomicAdd(a.lvl_count + d + 1, cnt) : 0;
+      sh[6] = nb; a.req_base[b] = nb; a.req_npar[nxt * a.B + b] = cnt; a.req_nscored[b] += npar;
+    }
+    int* ptok = s.ttok; uint64_t* phash = reinterpret_cast<uint64_t*>(s.tlog);   // (merged results are done with; tlog is 8-byte aligned: N * K * 8 bytes in)
+    uint64_t ph = 0; int pt = 0, sl = 0;
+    if (par) { sl = s.newl[tid]; ph = s.pv.hash[sl]; pt = s.pv.tok[sl]; }
+    __syncthreads();
+    if (par) { const int i = off + __popc(bal & ((1u << lane) - 1u)); s.npl[i] = sl; ptok[i] = pt; phash[i] = ph; }
+    if (more) cp_async_wait_all();
+    __syncthreads();
+    if (cnt > 0) make_parents(a, s, cnt, sh[6], b, b * a.D + d + 1, NS, ptok, phash, a.ent[nxt], a.ent_slot[nxt]);
+  }
+  {
+    uint4* dst = reinterpret_cast<uint4*>(gpool); const uint4* src = reinterpret_cast<const uint4*>(s.pv.key);
+    for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) dst[i] = src[i];
+  }
+  __syncthreads();
+}
+
+// Canonical (BFS) renumbering, outputs and ancestor bitmasks of one request, out of shared memory.
+__device__ __noinline__ void tx_finalize(const TreeArgs& a, unsigned char* sm, const int b, const bool timed_out) {
+  const OwnerSm s = owner_carve(sm, a);
+  const int tid = threadIdx.x, N = a.N;
+  const size_t pb = (size_t)b * N;
+  int* canon = s.ttok; int* cpar = s.dtok;
+  __shared__ int n_sh;
+  {
+    uint4* dst = reinterpret_cast<uint4*>(s.pv.key); const uint4* src = reinterpret_cast<const uint4*>(a.pool + (size_t)b * a.pool_stride);
+    for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) dst[i] = __ldcg(src + i);
+  }
+  if (tid == 0) n_sh = 0;
+  __syncthreads();
+  // a node's places by counting; G neighbouring lanes share a node's comparisons
+  const int G = N <= 80 ? 8 : (N <= 160 ? 4 : 2);
+  for (int q0 = 0; q0 < N; q0 += TX_THREADS / G) {
+    const int x = q0 + tid / G, sub = tid % G;
+    const bool have = x < N && (s.pv.meta[x] >> 16) != 0;
+    int cr = 0, pr = 0;
+    if (have) {
+      const int dx = (s.pv.meta[x] >> 8) & 255; const uint64_t px = s.pv.path[x]; const double kx = s.pv.key[x];
+      for (int t = sub; t < N; t += G) {
+        const int mt = s.pv.meta[t];
+        if (t == x || !(mt >> 16)) continue;
+        const int dt = (mt >> 8) & 255; const uint64_t pt = s.pv.path[t];
+        if (dt < dx || (dt == dx && pt < px)) ++cr;
+        if (before(s.pv.key[t], dt, pt, kx, dx, px)) ++pr;
+      }
+    }
+    for (int o = 1; o < G; o <<= 1) { cr += __shfl_xor_sync(0xFFFFFFFFu, cr, o); pr += __shfl_xor_sync(0xFFFFFFFFu, pr, o); }
+    if (x < N && sub == 0) canon[x] = have ? cr : -1;
+    if (have && sub == 0) {
+      atomicAdd(&n_sh, 1);
+      const size_t o = pb + cr;
+      a.tok[o] = s.pv.tok[x]; a.depth[o] = (s.pv.meta[x] >> 8) & 255; a.sib_rank[o] = s.pv.meta[x] & 255;
+      a.logS[o] = (float)s.pv.logS[x]; a.q0[o] = s.pv.q0[x]; a.logqT[o] = s.pv.logqT[x];
+      if (a.logkey) a.logkey[o] = (float)s.pv.key[x];
+      if (a.pop_rank) a.pop_rank[o] = pr;
+      a.node_hash[(size_t)b * (N + 1) + cr + 1] = s.pv.hash[x];
+      if (a.node_lseT) a.node_lseT[(size_t)b * (N + 1) + cr + 1] = s.pv.lseT[x];
+    }
+  }
+  __syncthreads();
+  for (int x = tid; x < N; x += TX_THREADS) {
+    const int c = canon[x];
+    if (c < 0) continue;
+    const int px = s.pv.parent[x], cp = px < 0 ? -1 : canon[px];
+    cpar[c] = cp;
+    a.parent[pb + c] = cp;
+  }
+  if (tid == 0) {
+    if (timed_out && a.status[b] == TS_OK) a.status[b] = TS_ERR_TIMEOUT;
+    a.n_nodes[b] = n_sh;
+    a.node_hash[(size_t)b * (N + 1)] = 0ull;
+    if (a.node_lseT) a.node_lseT[(size_t)b * (N + 1)] = a.root_lseT[b];
+    if (a.n_scored) a.n_scored[b] = a.req_nscored[b];
+  }
+  __syncthreads();
+  // a node's mask row: its own bit and its ancestors', up the (short) chain of parents
+  const int n = n_sh;
+  for (int e = tid; e < n * a.words; e += TX_THREADS) {
+    const int i = e / a.words, w = e % a.words;
+    uint64_t m = 0ull;
+    for (int x = i; x >= 0; x = cpar[x]) if ((x >> 6) == w) m |= 1ull << (x & 63);
+    a.mask[pb * a.words + e] = m;
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_constant__ TreeArgs a, const __grid_constant__ CUtensorMap tmW) {
+  extern __shared__ unsigned char raw[];
+  unsigned char* base_sm = raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u);
+  const TxSm sm = tx_carve(base_sm, a);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = (int)blockIdx.x, ncta = (int)gridDim.x;
+  const int t0 = cta * a.TV, tlen = min(a.TV, a.V - t0);     // this CTA's vocabulary range (empty for the last CTAs of some vocabularies)
+  // ---- set-up: nothing here reads what an earlier kernel wrote -----------------------------------------------------
+  if (warp == TX_MMA) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(sm.tmem)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 0) {
+    mbar_init(sm.a_full, TX_SCAN_WARPS * 32 + (a.lost_arrival ? 1 : 0));
+    for (int i = 0; i < TX_STAGE_MAX; ++i) {
+      mbar_init(sm.t_full + i, 1); mbar_init(sm.t_empty + i, TX_SCAN_WARPS); mbar_init(sm.u_full + i, 32);
+      mbar_init(sm.w_full + i, a.use_tma ? 1 : 32); mbar_init(sm.w_free + i, 1);
+    }
+    *sm.abort = 0; *sm.done = 0; *sm.q_head = 0u; *sm.q_tail = 0u;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  fill_gumbel_bounds(sm.ghi, tid, TX_THREADS);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *sm.tmem;
+  pdl_wait();                 // inputs, workspace and the words the kernel before cleared
+  pdl_launch_dependents();
+
+  unsigned gen = 0;
+  const unsigned nexpect = (unsigned)ncta + (a.lost_arrival ? 1u : 0u);
+  bool dead = false;
+  WStream ws{0u, 0u};
+  BlockPos pos{0, 0}, wpos{0, 0};
+  int groups = 0;
+  const int nreq = a.score_P > 0 ? a.score_P : a.B;
+  const int piece_len = (((a.V + a.npiece - 1) / a.npiece) + 7) & ~7;
+
+  // ---- the first rows' best base logits per piece (and, for a ragged vocabulary, W with padded rows) ----------------
+  if (a.ragged) {
+    const unsigned short* src = reinterpret_cast<const unsigned short*>(a.W);
+    const int cpr = a.Vs / 8;
+    for (int e = cta * TX_THREADS + tid; e < a.r * cpr; e += ncta * TX_THREADS) {
+      const int k = e / cpr, v = (e % cpr) * 8;
+      uint32_t w[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t e0 = v + 2 * i < a.V ? __ldg(src + (size_t)k * a.V + v + 2 * i) : 0u, e1 = v + 2 * i + 1 < a.V ? __ldg(src + (size_t)k * a.V + v + 2 * i + 1) : 0u;
+        w[i] = e0 | (e1 << 16);
+      }
+      *reinterpret_cast<uint4*>(const_cast<unsigned short*>(reinterpret_cast<const unsigned short*>(a.Wscan)) + (size_t)k * a.Vs + v) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    asm volatile("fence.proxy.async;" ::: "memory");   // the bulk-tensor loads of W read these through the other proxy
+  }
+  for (int i = cta * TX_WARPS + warp; i < nreq * a.npiece; i += ncta * TX_WARPS) {
+    const int x = i / a.npiece;
+    const int row = a.score_P > 0 ? a.p_req[x] * a.D + a.p_depth[x] : x * a.D;
+    scout_piece(a, row, i % a.npiece, piece_len, a.utop + i, lane);
+  }
+  __threadfence();
+  if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) dead = true;
+  if (a.ragged) asm volatile("fence.proxy.async;" ::: "memory");
+
+  if (!dead) {
+    if (a.score_P > 0) { for (int i = cta; i < a.score_P; i += ncta) tx_given(a, base_sm, i); }
+    else {
+      for (int b = cta; b < a.B; b += ncta) tx_root(a, base_sm, b);
+      // sweep of the depth-1 rows, by the CTAs that own no request where there are enough of them
+      const int h0 = ncta - a.B >= ncta / 4 ? a.B : 0;
+      if (a.D > 1 && cta >= h0)
+        for (int i = (cta - h0) * TX_WARPS + warp; i < a.B * a.npiece; i += (ncta - h0) * TX_WARPS)
+          scout_piece(a, (i / a.npiece) * a.D + 1, i % a.npiece, piece_len, a.utop + (size_t)a.B * a.npiece + i, lane);
+    }
+    fence_async_smem();   // (owners work in memory that the scan's bulk loads may write)
+    __threadfence();
+    if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) dead = true;
+  } else if (a.score_P == 0) {
+    for (int b = cta; b < a.B; b += ncta) {   // nothing of these requests exists yet: an empty tree
+      PoolView g = pool_view(a.pool + (size_t)b * a.pool_stride, a.N);
+      for (int i = tid; i < a.N; i += TX_THREADS) g.meta[i] = 0;
+      if (tid == 0) { a.status[b] = TS_OK; a.req_nscored[b] = 0; a.root_lseT[b] = nanf(""); }
+    }
+    __syncthreads();
+  }
+
+  for (int d = 0; !dead && d < (a.score_P > 0 ? 1 : a.D); ++d) {
+    const int P = a.score_P > 0 ? a.score_P : (d == 0 ? a.B : __ldcg(a.lvl_count + d));
+    if (d == 0 && a.score_P == 0 && cta == 0 && tid == 0) a.lvl_count[0] = a.B;   // (read by the owners, after the scan's barrier)
+    if (P <= 0) break;
+    // ---- scan ---------------------------------------------------------------------------------------------------------
+    if (tlen > 0) {
+      const int R = mma_replicas(P), per = TX_ROWS / R, ngroups = R > 1 ? 1 : (P + TX_ROWS - 1) / TX_ROWS;
+      for (int g = 0; g < ngroups; ++g, ++groups) {
+        if (tid < TX_ROWS) {
+          const int p = R > 1 ? tid % per : g * TX_ROWS + tid;
+          uint4 e0 = make_uint4(0xFFFFFFFFu, 0u, 0u, 0u), e1 = make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0u);   // row -1: unused
+          if (p < P) { const uint4* src = reinterpret_cast<const uint4*>(a.ent[d & 1] + p); e0 = __ldcg(src); e1 = __ldcg(src + 1); }
+          uint4* dst = reinterpret_cast<uint4*>(sm.ent + tid);
+          dst[0] = e0; dst[1] = e1;
+          sm.thr[tid] = __uint_as_float(e1.x); sm.thr[TX_ROWS + tid] = __uint_as_float(e1.y);
+          sm.ln[tid] = 0; sm.ln[TX_ROWS + tid] = 0; sm.lthr[tid] = -INFINITY; sm.lthr[TX_ROWS + tid] = -INFINITY;
+        }
+        for (int i = tid; i < 2 * TX_SPLIT * TX_ROWS; i += TX_THREADS) sm.best[i] = -INFINITY;
+        if (g == 0) for (int i = tid; i < TX_QCAP; i += TX_THREADS) sm.q[i].w = 0u;   // (owners work in this memory: the queue's tags start clean)
+        __syncthreads();
+        const int done_target = (groups + 1) * TX_SCAN_WARPS;
+        if (warp < TX_SCAN_WARPS) tx_scan(a, sm, R, P, g, t0, tlen, tmem_base, pos);
+        else if (warp == TX_MMA) {
+          if (lane == 0) tx_issue(a, sm, &tmW, t0, tlen, tmem_base, pos, ws, groups, ngroups - g, !a.w_over && a.score_P == 0);
+          __syncwarp();
+        } else if (warp == TX_REFRESH) tx_refresh(a, sm, R, P, g, cta, done_target);
+        else if (warp == TX_SELECT) tx_drain(a, sm, R, g, cta, done_target);
+        else tx_copy(a, sm, R > 1 ? P : min(TX_ROWS, P - g * TX_ROWS), t0, tlen, pos, wpos);
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        if (*sm.abort) { dead = true; break; }
+        tx_publish(a, sm, R, P, g, cta);
+        __syncthreads();
+      }
+    }
+    __threadfence();
+    if (dead) { if (tid == 0) atomicExch(a.barrier + 1, 1u); break; }
+    if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
+    if (a.score_P > 0) {
+      // given parents: merged by all CTAs, results to the caller
+      const int R = mma_replicas(P), K = a.K;
+      for (int p = cta + ncta * warp; p < P; p += ncta * TX_WARPS) {
+        const int nt = __ldcg(a.cand_cnt + p), nk = __ldcg(a.cand_cnt + a.cap + p);
+        const size_t cb = (size_t)p * a.ntiles * (R * K);
+        float l0, lT, val, lg; int tok;
+        warp_lse(a, p, lane, l0, lT);
+        if (lane == 0) { a.o_lse0[p] = l0; a.o_lseT[p] = lT; }
+        warp_topk(a.cand_top + cb, nullptr, nt, K, lane, tok, val, lg);
+        if (lane < K) { a.o_top_tok[(size_t)p * K + lane] = tok; a.o_top_logit[(size_t)p * K + lane] = val; }
+        if (a.T > 0.f) { warp_topk(a.cand_key + cb, a.cand_lg + cb, nk, K, lane, tok, val, lg); val = lg; }
+        if (lane < K) { a.o_draw_tok[(size_t)p * K + lane] = tok; a.o_draw_logit[(size_t)p * K + lane] = val; }
+      }
+      break;
+    }
+    // ---- owners ---------------------------------------------------------------------------------------------------------
+    for (int b = cta; b < a.B; b += ncta) tx_owner(a, base_sm, b, d);
+    const int h0 = ncta - a.B >= ncta / 4 ? a.B : 0;
+    if (d + 2 < a.D && cta >= h0)
+      for (int i = (cta - h0) * TX_WARPS + warp; i < a.B * a.npiece; i += (ncta - h0) * TX_WARPS) {
+        const int b = i / a.npiece;
+        if (__ldcg(a.req_npar + (d & 1) * a.B + b) > 0)
+          scout_piece(a, b * a.D + d + 2, i % a.npiece, piece_len, a.utop + (size_t)(d & 1) * a.B * a.npiece + i, lane);
+      }
+    if (d + 1 >= a.D) break;
+    fence_async_smem();   // owners work in memory that the next scan's bulk loads may write
+    __threadfence();
+    if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
+  }
+  // ---- no copy may still be writing this CTA's shared memory when the last phase works in it or the CTA ends -----------
+  cp_async_wait_all();
+  if (a.use_tma && warp == TX_MMA && lane == 0)
+    for (; ws.issued < ws.requested; ++ws.issued) {
+      const uint32_t slot = ws.issued % (uint32_t)a.nW, use = ws.issued / (uint32_t)a.nW;
+      bool landed = false;
+      for (uint32_t i = 0; i < WAIT_LIMIT && !landed; ++i) { landed = mbar_test_wait(sm.w_full + slot, use & 1); if (!landed) __nanosleep(100); }
+    }
+  if (dead && tid == 0) { atomicExch(a.barrier + 1, 1u); atomicExch(a.err, 1); }
+  __syncthreads();
+  if (a.score_P == 0) {
+    const bool late = dead || *reinterpret_cast<volatile int*>(a.err) != 0;
+    for (int b = cta; b < a.B; b += ncta) tx_finalize(a, base_sm, b, late);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == TX_MMA) {
+    __syncwarp();
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+  }
+}
+
+__global__ void tree_init_kernel(unsigned* words, int n) {
+  pdl_wait();                // the launch before may still be using them
+  pdl_launch_dependents();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) words[i] = 0u;
+}
+
+// ------------------------------------------------------------------------------------------------------------------------
+// Host side
+// ------------------------------------------------------------------------------------------------------------------------
+
+// Shared-memory plan: A tile, ring of base-logit blocks, selection state, ring of W blocks.  Blocks of 128 tokens where two
+// stages of each ring fit (one MMA instruction a K step fills 128 columns: issuing costs per instruction), else 64;
+// what is left goes to deeper rings.
+bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
+  const size_t rp = (size_t)(c.r + 63) / 64 * 64, rw = (size_t)(c.r + 15) / 16 * 16;
+  const size_t avail = (size_t)max_smem - 1024 - 512;   // alignment, static shared memory
+  auto up = [](size_t x) { return (x + 1023) & ~(size_t)1023; };
+  TreePlan p{};
+  p.TV = ((c.V + num_sms - 1) / num_sms + 63) / 64 * 64;
+  p.ntiles = (c.V + p.TV - 1) / p.TV;
+  p.Vs = (c.V + 7) & ~7;
+  int piece = ((c.V + 127) / 128 + 7) & ~7;
+  piece = piece < 64 ? 64 : (piece > TX_PIECE ? TX_PIECE : piece);
+  p.npiece = (c.V + piece - 1) / piece;
+  for (int BN = 128; BN >= 64; BN /= 2) {
+    const size_t u = (size_t)TX_ROWS * 2 * BN, w = rw * 2 * BN, sel = up(tx_select_bytes(c.K)), fix = up(TX_FIXED_BYTES), A = rp * 256;
+    int nU = 2, nW = 2;
+    auto total = [&](int nu, int nw) { return A + (size_t)nu * u + sel + fix + (size_t)nw * w; };
+    if (total(nU, nW) > avail) continue;
+    for (;;) {   // the base-logit ring first: its loads start late
+      if (nU < 3 && total(nU + 1, nW) <= avail) { ++nU; continue; }
+      if (nW < TX_STAGE_MAX && total(nU, nW + 1) <= avail) { ++nW; continue; }
+      if (nU < TX_STAGE_MAX && total(nU + 1, nW) <= avail) { ++nU; continue; }
+      break;
+    }
+    p.BN = BN; p.nU = nU; p.nW = nW;
+    p.oU = (uint32_t)A; p.oL = (uint32_t)(A + (size_t)nU * u); p.oW = (uint32_t)(p.oL + sel); p.oX = (uint32_t)(p.oW + (size_t)nW * w);
+    // owners work in [A, U ring, selection state], and in the W ring too when that is not enough (the ring then does not run ahead)
+    const size_t own = owner_layout(c.Nmax, c.K, c.r).total;
+    if (own > p.oX) return false;
+    p.w_over = own > p.oW ? 1 : 0;
+    p.smem = total(nU, nW) + 1024;
+    *out = p;
+    return true;
+  }
+  return false;
+}
+
+// Workspace of one call over `nreq` requests (or given parents) whose lists hold up to `cap` parents.
+struct TreeWs { size_t head, ent[2], slot[2], sums, cnt, top, key, lg, thr, utop, pool, state, upad, wpad, total; int cap; };
+static TreeWs tree_ws(const ts_ctx* ctx, int nreq, int cap, bool expand, int rows) {
+  const ts_config& c = ctx->cfg; const TreePlan& p = ctx->tree;
+  TreeWs w{}; size_t at = 0;
+  auto take = [&](size_t bytes) { const size_t o = at; at = align_up(at + bytes, 256); return o; };
+  w.cap = cap = (cap + 7) / 8 * 8;
+  const size_t C = (size_t)cap, nt = (size_t)p.ntiles, cands = (C > TX_ROWS ? C : (size_t)TX_ROWS) * nt * c.K;   // (replicated rows: R * P <= 128)
+  w.head = take(256);
+  w.ent[0] = take(C * sizeof(ParentEntry));
+  if (expand) { w.ent[1] = take(C * sizeof(ParentEntry)); w.slot[0] = take(C * 4); w.slot[1] = take(C * 4); }
+  w.sums = take(C * nt * 16); w.cnt = take(2 * C * 4);
+  w.top = take(cands * 8); w.key = take(cands * 8); w.lg = take(cands * 4);
+  w.thr = take(2 * C * 4 + 2 * C * c.K * SLOT_STRIDE * 4);
+  w.utop = take((size_t)nreq * (expand ? 2 : 1) * p.npiece * 8);
+  if (expand) { w.pool = take((size_t)nreq * pool_bytes(c.Nmax)); w.state = take((size_t)nreq * 5 * 4); }
+  if (c.V % 8) { w.upad = take((size_t)rows * p.Vs * 2); w.wpad = take((size_t)c.r * p.Vs * 2); }
+  w.total = at;
+  return w;
+}
+
+// the region of the caller's workspace: sized for expansion, and for given parents up to the same list length
+size_t tree_ws_bytes(const ts_ctx* ctx, int B) {
+  const int cap = B * ctx->cfg.Nmax > B ? B * ctx->cfg.Nmax : B;
+  const size_t e = tree_ws(ctx, B, cap, true, B * ctx->cfg.D).total, g = tree_ws(ctx, cap, cap, false, B * ctx->cfg.D).total;
+  return e > g ? e : g;
+}
+
+// scratch of a scoring call over P given parents; 0: not possible without the caller's workspace (padded copies)
+size_t tree_score_bytes(const ts_ctx* ctx, int P) { return ctx->cfg.V % 8 ? 0 : tree_ws(ctx, P, P, false, 0).total; }
+
+static void fill_args(ts_ctx* ctx, TreeArgs& a, char* base, const TreeWs& w, bool expand, const void* U, const void* A, const void* W, float T, uint64_t seed) {
+  const ts_config& c = ctx->cfg; const TreePlan& p = ctx->tree;
+  a.U = U; a.A = A; a.W = W; a.V = c.V; a.D = c.D; a.r = c.r; a.K = c.K; a.N = c.Nmax; a.T = T; a.seed = seed;
+  a.ragged = c.V % 8 ? 1 : 0;
+  a.Vs = p.Vs; a.Uscan = a.ragged ? base + w.upad : U; a.Wscan = a.ragged ? base + w.wpad : W;
+  a.TV = p.TV; a.ntiles = p.ntiles; a.BN = p.BN; a.nW = p.nW; a.nU = p.nU; a.npiece = p.npiece; a.w_over = p.w_over;
+  a.oU = p.oU; a.oL = p.oL; a.oW = p.oW; a.oX = p.oX;
+  a.no_seed = (ctx->test_mode & TS_TEST_NO_SEED) ? 1 : 0;
+  int* head = (int*)(base + w.head);
+  a.barrier = (unsigned*)head; a.err = head + 4; a.lvl_count = head + 8;
+  for (int i = 0; i < (expand ? 2 : 1); ++i) { a.ent[i] = (ParentEntry*)(base + w.ent[i]); a.ent_slot[i] = expand ? (int*)(base + w.slot[i]) : nullptr; }
+  a.sums = (float4*)(base + w.sums); a.cand_cnt = (int*)(base + w.cnt);
+  a.cand_top = (uint2*)(base + w.top); a.cand_key = (uint2*)(base + w.key); a.cand_lg = (float*)(base + w.lg);
+  a.cap = w.cap; a.thr = (unsigned*)(base + w.thr); a.slots = a.thr + 2 * (size_t)w.cap;
+  a.utop = (uint2*)(base + w.utop);
+  a.wait_limit = ctx->wait_limit; a.lost_arrival = (ctx->test_mode & TS_TEST_LOST_ARRIVAL) ? 1 : 0;
+}
+
+static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream_t st) {
+  CUtensorMap tm;
+  memset(&tm, 0, sizeof(tm));
+  a.use_tma = tree_tensor_map(ctx, a.Wscan, a.Vs, &tm) ? 1 : 0;
+  cudaError_t e;
+  { ProfScope ps(ctx, K_INIT, st); e = launch_kernel(tree_init_kernel, 1, 64, 0, st, true, a.barrier, 8 + DMAX + 2); }
+  if (e != cudaSuccess) return e;
+  ProfScope ps(ctx, prof_id, st);
+  void* kargs[] = {(void*)&a, (void*)&tm};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctx->num_sms); cfg.blockDim = dim3(TX_THREADS); cfg.dynamicSmemBytes = ctx->tree.smem; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;   // grid barriers: every CTA resident
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = ctx->persist_pdl >= 0 ? 2 : 1;
+  e = cudaLaunchKernelExC(&cfg, (const void*)tree_kernel, kargs);
+  if (e != cudaSuccess && cfg.numAttrs == 2) {   // not accepted together: remember, and launch cooperative only
+    (void)cudaGetLastError();
+    ctx->persist_pdl = -1;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelExC(&cfg, (const void*)tree_kernel, kargs);
+  }
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t tree_setup(ts_ctx* ctx) { return cudaFuncSetAttribute(tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->tree.smem); }
+
+cudaError_t tree_score(ts_ctx* ctx, char* scratch, const void* U, const void* A, const void* W, int P, const int* p_req, const int* p_depth, const int* p_token,
+                       const uint64_t* p_hash, float T, uint64_t seed, float* lse0, float* lseT, int* top_tok, float* top_logit, int* draw_tok,
+                       float* draw_logit, int rows, cudaStream_t st) {
+  TreeArgs a{};
+  fill_args(ctx, a, scratch, tree_ws(ctx, P, P, false, rows), false, U, A, W, T, seed);
+  a.score_P = P; a.B = 1;
+  a.p_req = p_req; a.p_depth = p_depth; a.p_token = p_token; a.p_hash = p_hash;
+  a.o_lse0 = lse0; a.o_lseT = lseT; a.o_top_tok = top_tok; a.o_top_logit = top_logit; a.o_draw_tok = draw_tok; a.o_draw_logit = draw_logit;
+  return launch_tree(ctx, a, K_SCORE, st);
+}
+
+cudaError_t tree_expand(ts_ctx* ctx, char* ws, const TreeOut& o, const void* U, const void* A, const void* W, int B, const int* anchor, const float* theta,
+                        float T, uint64_t seed, cudaStream_t st) {
+  const ts_config& c = ctx->cfg;
+  TreeArgs a{};
+  const TreeWs w = tree_ws(ctx, B, B * c.Nmax > B ? B * c.Nmax : B, true, B * c.D);
+  fill_args(ctx, a, ws, w, true, U, A, W, T, seed);
+  a.B = B; a.anchor = anchor; a.theta = theta; a.calib = ctx->calib; a.calib_qT = (ctx->ablation & TS_ABLATE_CALIB_QT) ? 1 : 0;
+  a.pool = (unsigned char*)ws + w.pool; a.pool_stride = pool_bytes(c.Nmax);
+  int* state = (int*)(ws + w.state);
+  a.req_npar = state; a.req_base = state + 2 * (size_t)B; a.req_nscored = state + 3 * (size_t)B; a.root_lseT = (float*)(state + 4 * (size_t)B);
+  a.n_nodes = o.n_nodes; a.tok = o.tok; a.parent = o.parent; a.depth = o.depth; a.sib_rank = o.sib_rank; a.logS = o.logS; a.q0 = o.q0; a.logqT = o.logqT;
+  a.logkey = o.logkey; a.pop_rank = o.pop_rank; a.node_hash = o.node_hash; a.node_lseT = o.node_lseT; a.mask = o.mask; a.n_scored = o.n_scored; a.status = o.status;
+  a.words = (c.Nmax + 63) / 64;
+  return launch_tree(ctx, a, K_PERSIST, st);
+}
+
+}  // namespace ts
