@@ -37,6 +37,13 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// one lane of a converged warp (the instruction tells the compiler that the branch is uniform)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // Shared-memory state of a CTA.
 struct TxSm {
   unsigned char *As, *Us, *Ws;
@@ -181,15 +188,22 @@ struct BlockPos {
   __device__ __forceinline__ void next(int n) { if (++slot == n) { slot = 0; ++use; } }
 };
 
-__device__ __forceinline__ bool tx_wait(uint64_t* bar, uint32_t parity, const TxSm& sm, const TreeArgs& a) {
-  for (uint32_t i = 0; i < a.wait_limit; ++i) {
+__device__ __noinline__ bool tx_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort, int* err, uint32_t limit) {
+  for (uint32_t i = 0; i < limit; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
-    if (*sm.abort) return false;
+    if (*abort) return false;
     if (i > 64) __nanosleep(64);
   }
-  *sm.abort = 1;
-  atomicExch(a.err, 1);
+  *abort = 1;
+  atomicExch(err, 1);
   return false;
+}
+__device__ __forceinline__ bool tx_wait(uint64_t* bar, uint32_t parity, const TxSm& sm, const TreeArgs& a) {
+  return mbar_try_wait(bar, parity) || tx_wait_slow(bar, parity, sm.abort, a.err, a.wait_limit);
+}
+// the same by a whole warp, one answer for all its lanes
+__device__ __forceinline__ bool tx_wait_warp(uint64_t* bar, uint32_t parity, const TxSm& sm, const TreeArgs& a) {
+  return __all_sync(0xFFFFFFFFu, tx_wait(bar, parity, sm, a));
 }
 
 // ---- scanning warps: one group of up to 128 parents over this CTA's range ---------------------------------
@@ -229,8 +243,7 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
   bool alive = true;
   for (int nb = 0; nb < nblk; ++nb, pos.next(a.nU)) {
     const int slot = pos.slot;
-    const bool got = tx_wait(sm.t_full + slot, pos.use & 1, sm, a) && tx_wait(sm.u_full + slot, pos.use & 1, sm, a);
-    if (!__all_sync(0xFFFFFFFFu, got)) { alive = false; break; }
+    if (!tx_wait_warp(sm.t_full + slot, pos.use & 1, sm, a) || !tx_wait_warp(sm.u_full + slot, pos.use & 1, sm, a)) { alive = false; break; }
     tc_fence_after();
     const int nch = min(CB, (tlen - nb * a.BN + 15) / 16);
     const unsigned char* urow = sm.Us + (size_t)slot * (TX_ROWS * 2) * a.BN + (size_t)prow * 2 * a.BN;
@@ -349,17 +362,27 @@ __device__ __forceinline__ void tx_copy(const TreeArgs& a, const TxSm& sm, const
   const int ck = lane & (CB8 - 1), r0 = lane >> sh, rstep = 32 >> sh;
   const __nv_bfloat16* Ug = reinterpret_cast<const __nv_bfloat16*>(a.Uscan);
   for (int nb = 0; nb < nblk; ++nb, pos.next(a.nU)) {
-    if (pos.use >= 1 && !tx_wait(sm.t_empty + pos.slot, (pos.use - 1) & 1, sm, a)) return;
+    if (pos.use >= 1 && !tx_wait_warp(sm.t_empty + pos.slot, (pos.use - 1) & 1, sm, a)) return;
     const int v = t0 + nb * a.BN + ck * 8;
     const bool in = v < a.Vs;
+    const __nv_bfloat16* src = in ? Ug + v : Ug;
     unsigned char* dst = sm.Us + (size_t)pos.slot * (TX_ROWS * 2) * a.BN;
-    for (int rr = r0; rr < nrow; rr += rstep)
-      cp_async16(dst + (size_t)rr * 2 * a.BN + ((ck ^ (rr & 7)) << 4), in ? Ug + (size_t)sm.ent[rr].row * a.Vs + v : Ug, in);
+    // (the row indices of eight copies are read together: one at a time the loop is a chain of shared-memory reads)
+    for (int rr = r0; rr < nrow; rr += 8 * rstep) {
+      int row[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) row[u] = sm.ent[min(rr + u * rstep, nrow - 1)].row;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int x = rr + u * rstep;
+        if (x < nrow) cp_async16(dst + x * 2 * a.BN + ((ck ^ (x & 7)) << 4), src + (size_t)row[u] * a.Vs, in);
+      }
+    }
     cp_async_arrive(sm.u_full + pos.slot);
     if (!a.use_tma) {
       const int rw = (a.r + 15) / 16 * 16;
       const __nv_bfloat16* Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wscan);
-      if (wpos.use >= 1 && !tx_wait(sm.w_free + wpos.slot, (wpos.use - 1) & 1, sm, a)) return;
+      if (wpos.use >= 1 && !tx_wait_warp(sm.w_free + wpos.slot, (wpos.use - 1) & 1, sm, a)) return;
       unsigned char* wd = sm.Ws + (size_t)wpos.slot * rw * 2 * a.BN;
       for (int k = r0; k < rw; k += rstep) {
         const bool win = in && k < a.r;
@@ -373,63 +396,66 @@ __device__ __forceinline__ void tx_copy(const TreeArgs& a, const TxSm& sm, const
   }
 }
 
-// ---- the issuing lane: W blocks through their ring, one tile of MMAs per block ----------------------------------
-struct WStream { uint32_t requested, issued; };   // blocks of W asked for / handed to the tensor cores, whole launch
-
-__device__ __forceinline__ void tx_request_w(const TreeArgs& a, const TxSm& sm, const CUtensorMap* tm, const int t0, const int tlen, WStream& w, const uint32_t limit) {
+// ---- W blocks into their ring (by the refreshing warp) ----------------------------------------------------------------
+// `upto`: blocks of the whole launch that may be requested while this group runs.  Requests run on into the next scan (W
+// does not depend on which parents that will score) except where the owners work in the ring.  Not the issuing warp's
+// business: a request costs its thread most of a microsecond of instruction latency, which held up the MMAs.
+struct WLoad { BlockPos pos; int nb; uint32_t requested; };
+template <bool BLOCKING>
+__device__ __forceinline__ void tx_load(const TreeArgs& a, const TxSm& sm, const CUtensorMap* tm, const int t0, const int tlen, WLoad& w, const uint32_t upto) {
   const int nblk = (tlen + a.BN - 1) / a.BN, rw = (a.r + 15) / 16 * 16;
-  while (w.requested - w.issued < (uint32_t)a.nW && w.requested < limit) {
-    const uint32_t slot = w.requested % (uint32_t)a.nW, use = w.requested / (uint32_t)a.nW;
-    if (use >= 1 && !mbar_test_wait(sm.w_free + slot, (use - 1) & 1)) break;
-    const int nb = (int)(w.requested % (uint32_t)nblk);
-    const int ns = min(a.BN / 64, (tlen - nb * a.BN + 63) / 64);
-    mbar_expect_tx(sm.w_full + slot, (uint32_t)ns * rw * 128u);
-    for (int h = 0; h < ns; ++h)
-      tma_load_box(sm.Ws + ((size_t)slot * (a.BN / 64) + h) * rw * 128, tm, t0 + nb * a.BN + h * 64, 0, sm.w_full + slot);
-    ++w.requested;
+  const uint32_t slab = (uint32_t)rw * 128u;
+  for (; w.requested < upto; ++w.requested, w.pos.next(a.nW)) {
+    if (w.pos.use >= 1) {
+      if (BLOCKING) { if (!tx_wait_warp(sm.w_free + w.pos.slot, (w.pos.use - 1) & 1, sm, a)) return; }
+      else if (!__all_sync(0xFFFFFFFFu, mbar_test_wait(sm.w_free + w.pos.slot, (w.pos.use - 1) & 1))) return;
+    }
+    if (elect_one()) {
+      const int ns = min(a.BN / 64, (tlen - w.nb * a.BN + 63) / 64);
+      mbar_expect_tx(sm.w_full + w.pos.slot, (uint32_t)ns * slab);
+      unsigned char* dst = sm.Ws + (size_t)(w.pos.slot * (a.BN / 64)) * slab;
+      for (int h = 0; h < ns; ++h) tma_load_box(dst + (size_t)h * slab, tm, t0 + w.nb * a.BN + h * 64, 0, sm.w_full + w.pos.slot);
+    }
+    __syncwarp();
+    if (++w.nb == nblk) w.nb = 0;
   }
 }
 
-__device__ __forceinline__ void tx_issue(const TreeArgs& a, const TxSm& sm, const CUtensorMap* tm, const int t0, const int tlen, const uint32_t tmem_base,
-                                         BlockPos& pos, WStream& w, const int group_no, const int groups_left, const bool run_ahead) {
+// ---- the issuing warp: one tile of MMAs per block -----------------------------------------------------------------------
+__device__ __forceinline__ void tx_issue(const TreeArgs& a, const TxSm& sm, const int tlen, const uint32_t tmem_base, BlockPos& pos, BlockPos& wpos, const int group_no) {
   const int nblk = (tlen + a.BN - 1) / a.BN, ksteps = (a.r + 15) / 16;
   const uint32_t slab = (uint32_t)ksteps * 2048u;
-  // requests stop at the end of the level where owners will work in the ring, and run on into the next scan elsewhere:
-  // W does not depend on which parents that will score
-  const uint32_t limit = w.issued + (uint32_t)(nblk * groups_left + (run_ahead ? a.nW : 0));
-  if (a.use_tma) tx_request_w(a, sm, tm, t0, tlen, w, limit);
-  if (!tx_wait(sm.a_full, group_no & 1, sm, a)) return;
-  tc_fence_after();
-  const uint64_t adesc0 = smem_desc(smem_u32(sm.As), 16u, 1024u);
-  for (int nb = 0; nb < nblk; ++nb, pos.next(a.nU)) {
-    const uint32_t ws = w.issued % (uint32_t)a.nW, wu = w.issued / (uint32_t)a.nW;
-    if (a.use_tma) tx_request_w(a, sm, tm, t0, tlen, w, limit);
-    if (!tx_wait(sm.w_full + ws, wu & 1, sm, a)) return;
-    if (pos.use >= 1 && !tx_wait(sm.t_empty + pos.slot, (pos.use - 1) & 1, sm, a)) return;
+  const uint64_t adesc0 = smem_desc(smem_u32(sm.As), 16u, 1024u), bdesc0 = smem_desc(smem_u32(sm.Ws), slab, 1024u);
+  if (!tx_wait_warp(sm.a_full, group_no & 1, sm, a)) return;
+  for (int nb = 0; nb < nblk; ++nb, pos.next(a.nU), wpos.next(a.nW)) {
+    if (!tx_wait_warp(sm.w_full + wpos.slot, wpos.use & 1, sm, a)) return;
+    if (pos.use >= 1 && !tx_wait_warp(sm.t_empty + pos.slot, (pos.use - 1) & 1, sm, a)) return;
     tc_fence_after();
-    const int n = min(a.BN, (tlen - nb * a.BN + 63) / 64 * 64);   // whole 64-token slabs
-    const uint32_t idesc = instr_desc(n), d = tmem_base + (uint32_t)(pos.slot * a.BN);
-    const uint64_t bdesc0 = smem_desc(smem_u32(sm.Ws) + ws * (uint32_t)(a.BN / 64) * slab, slab, 1024u);
-    for (int ks = 0; ks < ksteps; ++ks)
-      mma_bf16(d, adesc0 + (uint64_t)((ks >> 2) * (TX_ROWS * 128 / 16) + (ks & 3) * 2), bdesc0 + (uint64_t)(ks * 128), idesc, ks > 0 ? 1u : 0u);
-    mma_commit(sm.t_full + pos.slot);
-    mma_commit(sm.w_free + ws);
-    ++w.issued;
-  }
-  if (a.use_tma) {
-    for (uint32_t i = 0; i < a.wait_limit && w.requested - w.issued < (uint32_t)a.nW && w.requested < limit; ++i) { tx_request_w(a, sm, tm, t0, tlen, w, limit); if (*sm.abort) break; }
+    if (elect_one()) {
+      const int n = min(a.BN, (tlen - nb * a.BN + 63) / 64 * 64);   // whole 64-token slabs
+      const uint32_t idesc = instr_desc(n), d = tmem_base + (uint32_t)(pos.slot * a.BN);
+      const uint64_t bd = bdesc0 + (uint64_t)((uint32_t)(wpos.slot * (a.BN / 64)) * (slab >> 4));
+#pragma unroll 4
+      for (int ks = 0; ks < ksteps; ++ks)
+        mma_bf16(d, adesc0 + (uint64_t)((ks >> 2) * (TX_ROWS * 128 / 16) + (ks & 3) * 2), bd + (uint64_t)(ks * 128), idesc, ks > 0 ? 1u : 0u);
+      mma_commit(sm.t_full + pos.slot);
+      mma_commit(sm.w_free + wpos.slot);
+    }
+    __syncwarp();
   }
 }
 
 // ---- the refreshing warp -----------------------------------------------------------------------------------------
 // Condenses the slots of the parents this CTA is responsible for (parent p belongs to range p mod ntiles) into two
 // words per parent and copies the condensed words of its rows into shared memory, until the scan is over.
-__device__ __forceinline__ void tx_refresh(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int tile, const int done_target) {
+__device__ __forceinline__ void tx_refresh(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int tile, const int done_target,
+                                           const CUtensorMap* tm, const int t0, const int tlen, WLoad& w, const uint32_t upto) {
   const int lane = threadIdx.x & 31, per = TX_ROWS / R, K = a.K;
   const int p_lo = R > 1 ? 0 : g * TX_ROWS, p_hi = min(P, p_lo + per), nt = a.ntiles;
   const int p_own = p_lo + ((tile - p_lo % nt + nt) % nt);
   const int which = lane >> 4, j = lane & 15;
   for (uint32_t spin = 0; spin < a.wait_limit; ++spin) {
+    if (a.use_tma) tx_load<false>(a, sm, tm, t0, tlen, w, upto);
     if (*sm.done >= done_target || *sm.abort) break;
     unsigned v = 0xFFFFFFFFu;
     if (p_own < p_hi && j < K) v = __ldcg(a.slots + (((size_t)which * a.cap + p_own) * K + j) * SLOT_STRIDE);
@@ -459,9 +485,10 @@ __device__ __forceinline__ void tx_refresh(const TreeArgs& a, const TxSm& sm, co
         sm.thr[TX_ROWS + rr] = fmaxf(dec_f(rK[k]), sm.ent[rr].thrK);
       }
     }
-    __nanosleep(spin < 16u ? 100 : 500);
+    __nanosleep(spin < 16u ? 32 : 200);
   }
   __syncwarp();
+  if (a.use_tma && !*sm.abort) tx_load<true>(a, sm, tm, t0, tlen, w, upto);
 }
 
 // ---- the selecting warp: drains the queue until the scan is over ----------------------------------------------------
@@ -556,27 +583,34 @@ __device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, co
 // The K best of n (value, token) pairs (value desc, token asc): lane j < K gets the j-th in (tok, val, lg).  Batches of
 // up to 224 entries in registers beside the winners so far; a round is two warp-wide maxima (the value's order-
 // preserving image, then the inverted token among its ties) and one removal.
-__device__ __forceinline__ void warp_topk(const uint2* cand, const float* lgs, int n, int K, int lane, int& tok, float& val, float& lg) {
+__device__ __noinline__ float3 warp_topk(const uint2* cand, const float* lgs, const int* count, int K, int lane) {
   uint32_t wv = 0u, wt = 0u; float wl = 0.f;   // winner `lane` so far: 0 = none
+  // the first 64 entries are requested together with the count (there is always room for 128 of them)
+  const int n = __ldcg(count);
+  const uint2 pre0 = __ldcg(cand + lane), pre1 = __ldcg(cand + 32 + lane);
+  const float pl0 = lgs ? __ldcg(lgs + lane) : 0.f, pl1 = lgs ? __ldcg(lgs + 32 + lane) : 0.f;
+#pragma unroll 1
   for (int base = 0; base < n; base += 7 * 32) {
     uint32_t ev[8], et[8]; float el[8];
     ev[0] = wv; et[0] = wt; el[0] = wl;
+    const int used = min(7, (n - base + 31) / 32);   // (warp-uniform) slots of 32 entries in this batch
 #pragma unroll
     for (int u = 1; u < 8; ++u) {
       const int i = base + (u - 1) * 32 + lane;
       ev[u] = 0u; et[u] = 0u; el[u] = 0.f;
-      if (i < n) {
-        const uint2 c = __ldcg(cand + i);
+      if (u <= used && i < n) {
+        const uint2 c = (u == 1 && base == 0) ? pre0 : ((u == 2 && base == 0) ? pre1 : __ldcg(cand + i));
         ev[u] = enc_f(__uint_as_float(c.x)); et[u] = ~c.y;
-        el[u] = lgs ? __ldcg(lgs + i) : __uint_as_float(c.x);
+        el[u] = !lgs ? __uint_as_float(c.x) : ((u == 1 && base == 0) ? pl0 : ((u == 2 && base == 0) ? pl1 : __ldcg(lgs + i)));
       }
     }
     wv = 0u; wt = 0u; wl = 0.f;
+#pragma unroll 1
     for (int j = 0; j < K; ++j) {
       uint32_t bv = ev[0], bt = et[0]; float bl = el[0];
 #pragma unroll
       for (int u = 1; u < 8; ++u)
-        if (ev[u] > bv || (ev[u] == bv && et[u] > bt)) { bv = ev[u]; bt = et[u]; bl = el[u]; }
+        if (u <= used && (ev[u] > bv || (ev[u] == bv && et[u] > bt))) { bv = ev[u]; bt = et[u]; bl = el[u]; }
       const uint32_t mv = __reduce_max_sync(0xFFFFFFFFu, bv);
       if (mv == 0u) break;   // warp-uniform
       const uint32_t mt = __reduce_max_sync(0xFFFFFFFFu, bv == mv ? bt : 0u);
@@ -590,18 +624,18 @@ __device__ __forceinline__ void warp_topk(const uint2* cand, const float* lgs, i
       if (lane == j) { wv = mv; wt = mt; wl = l; }
     }
   }
-  tok = wv ? (int)~wt : -1; val = wv ? dec_f(wv) : 0.f; lg = wv ? wl : 0.f;
+  return make_float3(__int_as_float(wv ? (int)~wt : -1), wv ? dec_f(wv) : 0.f, wv ? wl : 0.f);   // token (as bits), value, logit
 }
 
 // Log-normalisers of a parent from its ranges' sums; every lane gets them.
-__device__ __forceinline__ void warp_lse(const TreeArgs& a, int p, int lane, float& lse0, float& lseT) {
-  const float T = a.T, invT = T > 0.f ? 1.f / T : 1.f;
-  const float4* h = a.sums + (size_t)p * a.ntiles;
+__device__ __forceinline__ float2 warp_lse(const float4* h, const int nt, const float T, int lane) {
+  const float invT = T > 0.f ? 1.f / T : 1.f;
   float m = -INFINITY, s0 = 0.f, sT = 0.f;
-  for (int t0 = 0; t0 < a.ntiles; t0 += 5 * 32) {
+#pragma unroll 1
+  for (int t0 = 0; t0 < nt; t0 += 5 * 32) {
     float4 x[5];
 #pragma unroll
-    for (int u = 0; u < 5; ++u) { const int t = t0 + u * 32 + lane; x[u] = t < a.ntiles ? __ldcg(h + t) : make_float4(-INFINITY, 0.f, 0.f, 0.f); }
+    for (int u = 0; u < 5; ++u) { const int t = t0 + u * 32 + lane; x[u] = t < nt ? __ldcg(h + t) : make_float4(-INFINITY, 0.f, 0.f, 0.f); }
 #pragma unroll
     for (int u = 0; u < 5; ++u) {
       if (x[u].x == -INFINITY) { s0 += x[u].y; continue; }
@@ -616,8 +650,8 @@ __device__ __forceinline__ void warp_lse(const TreeArgs& a, int p, int lane, flo
   if (m > -INFINITY) { s0 *= __expf(m - gm); sT *= __expf((m - gm) * invT); }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) { s0 += __shfl_xor_sync(0xFFFFFFFFu, s0, off); sT += __shfl_xor_sync(0xFFFFFFFFu, sT, off); }
-  lse0 = gm + logf(s0);
-  lseT = T > 0.f ? gm * invT + logf(sT) : lse0;
+  const float lse0 = gm + logf(s0);
+  return make_float2(lse0, T > 0.f ? gm * invT + logf(sT) : lse0);
 }
 
 // ---- seed bounds ------------------------------------------------------------------------------------------------------
@@ -661,21 +695,23 @@ __device__ __forceinline__ void scout_piece(const TreeArgs& a, int row, int piec
 }
 
 // The seed tokens of one row: the best of its pieces, picked by one warp (lane j: the j-th).
-__device__ __forceinline__ void pick_seeds(const TreeArgs& a, const uint2* ut, int NS, int* stok, float* sval, int lane) {
+__device__ __forceinline__ void pick_seeds(const int npiece, const uint2* ut, int NS, int* stok, float* sval, int lane) {
   uint32_t ev[8], et[8];
 #pragma unroll
   for (int u = 0; u < 8; ++u) { ev[u] = 0u; et[u] = 0u; }
-  for (int i0 = 0; i0 < a.npiece; i0 += 256) {
+#pragma unroll 1
+  for (int i0 = 0; i0 < npiece; i0 += 256) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int i = i0 + u * 32 + lane;
-      if (i < a.npiece) {
+      if (i < npiece) {
         const uint2 e = __ldcg(ut + i);
         if (e.x > ev[u]) { ev[u] = e.x; et[u] = e.y; }   // (beyond 256 pieces the best of every 256th: any tokens give valid bounds)
       }
     }
   }
   int tok = -1; float val = -INFINITY;
+#pragma unroll 1
   for (int j = 0; j < NS; ++j) {
     uint32_t bv = ev[0], bt = et[0];
 #pragma unroll
@@ -802,105 +838,103 @@ __device__ __forceinline__ void tx_caps(const TreeArgs& a, int b, int& K_eff, in
   else log_theta = th > 0.f ? log((double)th) : -INFINITY;
 }
 
-// The start of a request: an empty pool and the root as the only parent of level 0 (its seed bounds come from the
-// sweep of the depth-0 row that every CTA has just finished).
-__device__ __noinline__ void tx_root(const TreeArgs& a, unsigned char* sm, const int b) {
-  const OwnerSm s = owner_carve(sm, a);
-  const int tid = threadIdx.x, NS = seed_count(a.K);
-  __shared__ int tok0; __shared__ uint64_t hash0;
-  PoolView g = pool_view(a.pool + (size_t)b * a.pool_stride, a.N);
-  for (int i = tid; i < a.N; i += TX_THREADS) g.meta[i] = 0;
-  if (tid == 0) {
-    const int t = a.anchor[b];
-    const bool ok = t >= 0 && t < a.V && a.theta[b] == a.theta[b];
-    a.status[b] = ok ? TS_OK : TS_ERR_INVALID;
-    tok0 = ok ? t : 0; hash0 = 0ull; s.npl[0] = -1;
-    a.req_npar[b] = 1; a.req_base[b] = b; a.req_nscored[b] = 0;
-    a.root_lseT[b] = nanf("");
-  }
-  if ((tid >> 5) == 1) pick_seeds(a, a.utop + (size_t)b * a.npiece, NS, s.stok, s.sval, tid & 31);
-  __syncthreads();
-  fetch_seed_columns(a, s, NS);
-  cp_async_wait_all();
-  __syncthreads();
-  make_parents(a, s, 1, b, b, b * a.D, NS, &tok0, &hash0, a.ent[0], a.ent_slot[0]);
-  __syncthreads();
-}
-
-// A given parent of ts_score_parents: list place i.
-__device__ __noinline__ void tx_given(const TreeArgs& a, unsigned char* sm, const int i) {
-  const OwnerSm s = owner_carve(sm, a);
-  const int tid = threadIdx.x, NS = seed_count(a.K);
-  __shared__ int tok0; __shared__ uint64_t hash0;
-  const int req = a.p_req[i], dep = a.p_depth[i];
-  if (tid == 0) { tok0 = a.p_token[i]; hash0 = a.p_hash[i]; }
-  if ((tid >> 5) == 1) pick_seeds(a, a.utop + (size_t)i * a.npiece, NS, s.stok, s.sval, tid & 31);
-  __syncthreads();
-  fetch_seed_columns(a, s, NS);
-  cp_async_wait_all();
-  __syncthreads();
-  make_parents(a, s, 1, i, req, req * a.D + dep, NS, &tok0, &hash0, a.ent[0], nullptr);
-  __syncthreads();
-}
-
 // One level of one request: merge of its parents, slots and cut of Algorithm 1, the next level's parents.
-// d = depth of the parents just scanned.
-__device__ __noinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, const int b, const int d) {
+// d = depth of the parents just scanned; d = -1: the start of request b (an empty pool and the root as the only parent of
+// level 0) or, for ts_score_parents, the list entry of given parent b.
+// (Inlined, once: behind a call the arguments would be read through generic addresses, some 40 cycles each.)
+__device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, const int b, const int d) {
   const OwnerSm s = owner_carve(sm, a);
   __shared__ int sh[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int N = a.N, K = a.K, cur = d & 1, nxt = cur ^ 1, NS = seed_count(K);
-  const int npar = __ldcg(a.req_npar + cur * a.B + b), base = __ldcg(a.req_base + b);
-  if (npar == 0 || __ldcg(a.status + b) != TS_OK) {   // uniform: nothing below has run yet
-    if (tid == 0) a.req_npar[nxt * a.B + b] = 0;
-    return;
-  }
-  int K_eff, N_eff; double log_theta;
-  tx_caps(a, b, K_eff, N_eff, log_theta);
-  const bool more = d + 1 < a.D;
+  int* ptok = s.ttok; uint64_t* phash = reinterpret_cast<uint64_t*>(s.tlog);   // the new parents (merged results are done with by then)
+  int cnt = 1, li0 = b, req = b, row = b * a.D + d + 1;
+  bool more = true;
+  int npar = 0, base = 0, K_eff = 0, N_eff = 0;
+  double log_theta = 0.0;
   unsigned char* gpool = a.pool + (size_t)b * a.pool_stride;
-  {
+  if (d < 0) {
+    const bool given = a.score_P > 0;
+    if (given) { req = a.p_req[b]; row = req * a.D + a.p_depth[b]; }
+    else {
+      PoolView g = pool_view(gpool, N);
+      for (int i = tid; i < N; i += TX_THREADS) g.meta[i] = 0;
+    }
+    if (tid == 0) {
+      if (given) { ptok[0] = a.p_token[b]; phash[0] = a.p_hash[b]; }
+      else {
+        const int t = a.anchor[b];
+        const bool ok = t >= 0 && t < a.V && a.theta[b] == a.theta[b];
+        a.status[b] = ok ? TS_OK : TS_ERR_INVALID;
+        ptok[0] = ok ? t : 0; phash[0] = 0ull;
+        a.req_npar[b] = 1; a.req_base[b] = b; a.req_nscored[b] = 0;
+        a.root_lseT[b] = nanf("");
+      }
+      s.npl[0] = -1;
+    }
+  } else {
+    npar = __ldcg(a.req_npar + cur * a.B + b); base = __ldcg(a.req_base + b);
+    if (npar == 0 || __ldcg(a.status + b) != TS_OK) {   // uniform: nothing below has run yet
+      if (tid == 0) a.req_npar[nxt * a.B + b] = 0;
+      return;
+    }
+    tx_caps(a, b, K_eff, N_eff, log_theta);
+    more = d + 1 < a.D;
     uint4* dst = reinterpret_cast<uint4*>(s.pv.key); const uint4* src = reinterpret_cast<const uint4*>(gpool);
     for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) dst[i] = __ldcg(src + i);
+    for (int i = tid; i < npar; i += TX_THREADS) s.pslot[i] = __ldcg(a.ent_slot[cur] + base + i);
+    if (tid < 8) sh[tid] = 0;
   }
-  for (int i = tid; i < npar; i += TX_THREADS) s.pslot[i] = __ldcg(a.ent_slot[cur] + base + i);
-  if (tid < 8) sh[tid] = 0;
-  // ---- merge: one warp per parent (the last warp picks the next level's seed tokens meanwhile) ----
+  // ---- merge: a warp each for a parent's log-normalisers, its best logits and its best keys: each is one or two memory
+  // round trips, side by side (the last warp picks the next row's seed tokens meanwhile) ----
   if (warp == TX_WARPS - 1) {
-    if (more) pick_seeds(a, a.utop + ((size_t)nxt * a.B + b) * a.npiece, NS, s.stok, s.sval, lane);
-  } else {
-    for (int i = warp; i < npar; i += TX_WARPS - 1) {
-      const int p = base + i;
-      const int P = __ldcg(a.lvl_count + d), R = mma_replicas(P);
-      const int nt = __ldcg(a.cand_cnt + p), nk = __ldcg(a.cand_cnt + a.cap + p);
-      const size_t cb = (size_t)p * a.ntiles * (R * K);
-      float l0, lT, val, lg; int tok;
-      warp_lse(a, p, lane, l0, lT);
-      warp_topk(a.cand_top + cb, nullptr, nt, K, lane, tok, val, lg);
-      const int ttok = tok; const float tlog = val;
-      int dtok = ttok; float dlog = tlog;
-      if (a.T > 0.f) { warp_topk(a.cand_key + cb, a.cand_lg + cb, nk, K, lane, tok, val, lg); dtok = tok; dlog = lg; }
-      if (lane < K) { s.ttok[i * K + lane] = ttok; s.tlog[i * K + lane] = tlog; s.dtok[i * K + lane] = dtok; s.dlog[i * K + lane] = dlog; }
-      if (lane == 0) { s.lse0[i] = l0; s.lseT[i] = lT; }
-      // the best token of q0 not among the first j draws, for every j: places of the draws in the top list, or-ed up
-      unsigned used = 0u;
-      for (int t = 0; t < K; ++t) { const int tt = __shfl_sync(0xFFFFFFFFu, ttok, t); if (lane < K && tt == dtok && tt >= 0) used |= 1u << t; }
-      if (!(a.T > 0.f)) used = lane < K ? 1u << lane : 0u;
-#pragma unroll
-      for (int o = 1; o < 16; o <<= 1) { const unsigned u = __shfl_up_sync(0xFFFFFFFFu, used, o); if (lane >= o) used |= u; }
-      const unsigned before = __shfl_up_sync(0xFFFFFFFFu, used, 1);
-      if (lane < K) { const unsigned freeb = ~(lane ? before : 0u) & ((1u << K_eff) - 1u); s.best[i * K + lane] = freeb ? (unsigned char)(__ffs(freeb) - 1) : 255u; }
+    if (more) pick_seeds(a.npiece, a.utop + ((size_t)nxt * a.B + b) * a.npiece, NS, s.stok, s.sval, lane);
+  } else if (d >= 0) {
+    const int P = __ldcg(a.lvl_count + d), R = mma_replicas(P), kinds = a.T > 0.f ? 3 : 2;
+#pragma unroll 1
+    for (int task = warp; task < npar * kinds; task += TX_WARPS - 1) {
+      const int i = task / kinds, kind = task % kinds, p = base + i;
+      if (kind == 0) {
+        const float2 l = warp_lse(a.sums + (size_t)p * a.ntiles, a.ntiles, a.T, lane);
+        if (lane == 0) { s.lse0[i] = l.x; s.lseT[i] = l.y; }
+      } else {
+        const size_t cb = (size_t)p * a.ntiles * (R * K);
+        const float3 w = warp_topk(kind == 1 ? a.cand_top + cb : a.cand_key + cb, kind == 1 ? nullptr : a.cand_lg + cb, a.cand_cnt + (kind == 1 ? 0 : a.cap) + p, K, lane);
+        if (lane < K) {
+          if (kind == 1) { s.ttok[i * K + lane] = __float_as_int(w.x); s.tlog[i * K + lane] = w.y; }
+          if (kind == 2 || kinds == 2) { s.dtok[i * K + lane] = __float_as_int(w.x); s.dlog[i * K + lane] = w.z; }
+        }
+      }
     }
   }
   __syncthreads();
   if (more) fetch_seed_columns(a, s, NS);   // lands while the slots are formed
-  // ---- slots of every scored parent, one thread per (parent, sibling rank) ----
-  for (int t = tid; t < npar * K; t += TX_THREADS) {
-    const int i = t / K, j = t % K;
+  if (d >= 0) {
+  // the best token of q0 not among the first j draws, for every j: places of the draws in the top list, or-ed up
+#pragma unroll 1
+  for (int i = warp; i < npar; i += TX_WARPS) {
+    unsigned used = 0u;
+    if (!(a.T > 0.f)) used = lane < K ? 1u << lane : 0u;
+    else if (lane < K) {
+      const int x = s.dtok[i * K + lane];
+#pragma unroll 4
+      for (int t = 0; t < K; ++t) if (x >= 0 && s.ttok[i * K + t] == x) used |= 1u << t;
+    }
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) { const unsigned u = __shfl_up_sync(0xFFFFFFFFu, used, o); if (lane >= o) used |= u; }
+    const unsigned prior = __shfl_up_sync(0xFFFFFFFFu, used, 1);
+    if (lane < K) { const unsigned fr = ~(lane ? prior : 0u) & ((1u << K_eff) - 1u); s.best[i * K + lane] = fr ? (unsigned char)(__ffs(fr) - 1) : 255u; }
+  }
+  __syncthreads();
+  // ---- slots of every scored parent: two threads per (parent, sibling rank), one for the key (the best unused token's
+  // estimate), one for the survival of the token drawn ----
+#pragma unroll 1
+  for (int t2 = tid; t2 < 2 * npar * K; t2 += TX_THREADS) {
+    const int t = t2 >> 1, which = t2 & 1, i = t / K, j = t % K;
     const double lse0 = s.lse0[i], lseT = s.lseT[i];
     const int slot = s.pslot[i];
     const bool bad = !(lse0 == lse0) || isinf(lse0);
-    if (j == 0) {
+    if (j == 0 && which == 0) {
       if (slot < 0) a.root_lseT[b] = (float)lseT; else s.pv.lseT[slot] = (float)lseT;
       if (bad) a.status[b] = TS_ERR_NUMERIC;
     }
@@ -912,15 +946,12 @@ __device__ __noinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, cons
         // the calibrator's input: the untempered conditional, or (ablation) the tempered one
         const bool tempered = a.calib_qT && a.T > 0.f;
         const double lsc = tempered ? 1.0 / (double)a.T : 1.0, lsn = tempered ? lseT : lse0;
-        const double key = logS_v + log_phat(a.calib, d, (double)s.tlog[i * K + bi] * lsc, lsn);
-        if (!(key < log_theta)) {
-          ok = 1;
-          s.ckey[t] = key;
-          s.clogS[t] = logS_v + log_phat(a.calib, d, (double)s.dlog[t] * lsc, lsn);
-        }
+        const double v = logS_v + log_phat(a.calib, d, (double)(which ? s.dlog[t] : s.tlog[i * K + bi]) * lsc, lsn);
+        if (which) s.clogS[t] = v;
+        else { s.ckey[t] = v; ok = !(v < log_theta); }
       }
     }
-    s.valid[t] = (unsigned char)ok;
+    if (which == 0) s.valid[t] = (unsigned char)ok;
   }
   __syncthreads();
   // a sibling slot exists only if the one before it was admitted (keys are non-increasing in j)
@@ -1077,31 +1108,31 @@ __device__ __noinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, cons
     const bool par = more && tid < nnew && !(s.pv.logS[s.newl[tid]] < log_theta);
     const unsigned bal = __ballot_sync(0xFFFFFFFFu, par);
     if (lane == 0 && warp < 8) s.tcnt[warp] = __popc(bal);
+    uint64_t ph = 0; int pt = 0, sl = 0;
+    if (par) { sl = s.newl[tid]; ph = s.pv.hash[sl]; pt = s.pv.tok[sl]; }
     __syncthreads();
-    int off = 0, cnt = 0;
+    int off = 0;
+    cnt = 0;
     for (int w = 0; w < 8; ++w) { if (w < warp) off += s.tcnt[w]; cnt += s.tcnt[w]; }
     if (tid == 0) {
       const int nb = cnt > 0 ? atomicAdd(a.lvl_count + d + 1, cnt) : 0;
       sh[6] = nb; a.req_base[b] = nb; a.req_npar[nxt * a.B + b] = cnt; a.req_nscored[b] += npar;
     }
-    int* ptok = s.ttok; uint64_t* phash = reinterpret_cast<uint64_t*>(s.tlog);   // (merged results are done with; tlog is 8-byte aligned: N * K * 8 bytes in)
-    uint64_t ph = 0; int pt = 0, sl = 0;
-    if (par) { sl = s.newl[tid]; ph = s.pv.hash[sl]; pt = s.pv.tok[sl]; }
-    __syncthreads();
     if (par) { const int i = off + __popc(bal & ((1u << lane) - 1u)); s.npl[i] = sl; ptok[i] = pt; phash[i] = ph; }
-    if (more) cp_async_wait_all();
-    __syncthreads();
-    if (cnt > 0) make_parents(a, s, cnt, sh[6], b, b * a.D + d + 1, NS, ptok, phash, a.ent[nxt], a.ent_slot[nxt]);
   }
-  {
-    uint4* dst = reinterpret_cast<uint4*>(gpool); const uint4* src = reinterpret_cast<const uint4*>(s.pv.key);
-    for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) dst[i] = src[i];
+  uint4* gdst = reinterpret_cast<uint4*>(gpool); const uint4* psrc = reinterpret_cast<const uint4*>(s.pv.key);
+  for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) gdst[i] = psrc[i];
   }
+  // ---- seed bounds and list entries ----
+  if (more) cp_async_wait_all();
+  __syncthreads();
+  if (d >= 0) li0 = sh[6];
+  if (more && cnt > 0) make_parents(a, s, cnt, li0, req, row, NS, ptok, phash, a.ent[nxt], a.ent_slot[nxt]);
   __syncthreads();
 }
 
 // Canonical (BFS) renumbering, outputs and ancestor bitmasks of one request, out of shared memory.
-__device__ __noinline__ void tx_finalize(const TreeArgs& a, unsigned char* sm, const int b, const bool timed_out) {
+__device__ __forceinline__ void tx_finalize(const TreeArgs& a, unsigned char* sm, const int b, const bool timed_out) {
   const OwnerSm s = owner_carve(sm, a);
   const int tid = threadIdx.x, N = a.N;
   const size_t pb = (size_t)b * N;
@@ -1200,14 +1231,13 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
   unsigned gen = 0;
   const unsigned nexpect = (unsigned)ncta + (a.lost_arrival ? 1u : 0u);
   bool dead = false;
-  WStream ws{0u, 0u};
+  WLoad wl{{0, 0}, 0, 0u};
   BlockPos pos{0, 0}, wpos{0, 0};
   int groups = 0;
   const int nreq = a.score_P > 0 ? a.score_P : a.B;
   const int piece_len = (((a.V + a.npiece - 1) / a.npiece) + 7) & ~7;
 
-  // ---- the first rows' best base logits per piece (and, for a ragged vocabulary, W with padded rows) ----------------
-  if (a.ragged) {
+  if (a.ragged) {   // W with padded rows (the bulk-tensor loads need rows of whole 16 bytes)
     const unsigned short* src = reinterpret_cast<const unsigned short*>(a.W);
     const int cpr = a.Vs / 8;
     for (int e = cta * TX_THREADS + tid; e < a.r * cpr; e += ncta * TX_THREADS) {
@@ -1222,40 +1252,14 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
     }
     asm volatile("fence.proxy.async;" ::: "memory");   // the bulk-tensor loads of W read these through the other proxy
   }
-  for (int i = cta * TX_WARPS + warp; i < nreq * a.npiece; i += ncta * TX_WARPS) {
-    const int x = i / a.npiece;
-    const int row = a.score_P > 0 ? a.p_req[x] * a.D + a.p_depth[x] : x * a.D;
-    scout_piece(a, row, i % a.npiece, piece_len, a.utop + i, lane);
-  }
-  __threadfence();
-  if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) dead = true;
-  if (a.ragged) asm volatile("fence.proxy.async;" ::: "memory");
-
-  if (!dead) {
-    if (a.score_P > 0) { for (int i = cta; i < a.score_P; i += ncta) tx_given(a, base_sm, i); }
-    else {
-      for (int b = cta; b < a.B; b += ncta) tx_root(a, base_sm, b);
-      // sweep of the depth-1 rows, by the CTAs that own no request where there are enough of them
-      const int h0 = ncta - a.B >= ncta / 4 ? a.B : 0;
-      if (a.D > 1 && cta >= h0)
-        for (int i = (cta - h0) * TX_WARPS + warp; i < a.B * a.npiece; i += (ncta - h0) * TX_WARPS)
-          scout_piece(a, (i / a.npiece) * a.D + 1, i % a.npiece, piece_len, a.utop + (size_t)a.B * a.npiece + i, lane);
-    }
-    fence_async_smem();   // (owners work in memory that the scan's bulk loads may write)
-    __threadfence();
-    if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) dead = true;
-  } else if (a.score_P == 0) {
-    for (int b = cta; b < a.B; b += ncta) {   // nothing of these requests exists yet: an empty tree
-      PoolView g = pool_view(a.pool + (size_t)b * a.pool_stride, a.N);
-      for (int i = tid; i < a.N; i += TX_THREADS) g.meta[i] = 0;
-      if (tid == 0) { a.status[b] = TS_OK; a.req_nscored[b] = 0; a.root_lseT[b] = nanf(""); }
-    }
-    __syncthreads();
-  }
-
-  for (int d = 0; !dead && d < (a.score_P > 0 ? 1 : a.D); ++d) {
-    const int P = a.score_P > 0 ? a.score_P : (d == 0 ? a.B : __ldcg(a.lvl_count + d));
-    if (d == 0 && a.score_P == 0 && cta == 0 && tid == 0) a.lvl_count[0] = a.B;   // (read by the owners, after the scan's barrier)
+  // Phases: d = -2 sweeps the depth-0 rows (given parents: theirs); d = -1 starts the requests; d >= 0 scans the parents of
+  // depth d and runs their level step.
+  int d = -2;
+  for (;; ++d) {
+    int P = nreq;
+    if (d >= 0) {
+    if (d > 0) P = __ldcg(a.lvl_count + d);
+    else if (a.score_P == 0 && cta == 0 && tid == 0) a.lvl_count[0] = a.B;   // (read by the owners, after the scan's barrier)
     if (P <= 0) break;
     // ---- scan ---------------------------------------------------------------------------------------------------------
     if (tlen > 0) {
@@ -1275,11 +1279,12 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
         __syncthreads();
         const int done_target = (groups + 1) * TX_SCAN_WARPS;
         if (warp < TX_SCAN_WARPS) tx_scan(a, sm, R, P, g, t0, tlen, tmem_base, pos);
-        else if (warp == TX_MMA) {
-          if (lane == 0) tx_issue(a, sm, &tmW, t0, tlen, tmem_base, pos, ws, groups, ngroups - g, !a.w_over && a.score_P == 0);
-          __syncwarp();
-        } else if (warp == TX_REFRESH) tx_refresh(a, sm, R, P, g, cta, done_target);
-        else if (warp == TX_SELECT) tx_drain(a, sm, R, g, cta, done_target);
+        else if (warp == TX_MMA) tx_issue(a, sm, tlen, tmem_base, pos, wpos, groups);
+        else if (warp == TX_REFRESH) {
+          const uint32_t nblk = (uint32_t)((tlen + a.BN - 1) / a.BN);
+          const uint32_t level_end = (uint32_t)(groups + ngroups - g) * nblk + ((a.w_over || a.score_P > 0) ? 0u : (uint32_t)a.nW);
+          tx_refresh(a, sm, R, P, g, cta, done_target, &tmW, t0, tlen, wl, min((uint32_t)(groups + 1) * nblk + (uint32_t)a.nW, level_end));
+        } else if (warp == TX_SELECT) tx_drain(a, sm, R, g, cta, done_target);
         else tx_copy(a, sm, R > 1 ? P : min(TX_ROWS, P - g * TX_ROWS), t0, tlen, pos, wpos);
         tc_fence_before();
         __syncthreads();
@@ -1296,37 +1301,54 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
       // given parents: merged by all CTAs, results to the caller
       const int R = mma_replicas(P), K = a.K;
       for (int p = cta + ncta * warp; p < P; p += ncta * TX_WARPS) {
-        const int nt = __ldcg(a.cand_cnt + p), nk = __ldcg(a.cand_cnt + a.cap + p);
         const size_t cb = (size_t)p * a.ntiles * (R * K);
-        float l0, lT, val, lg; int tok;
-        warp_lse(a, p, lane, l0, lT);
-        if (lane == 0) { a.o_lse0[p] = l0; a.o_lseT[p] = lT; }
-        warp_topk(a.cand_top + cb, nullptr, nt, K, lane, tok, val, lg);
-        if (lane < K) { a.o_top_tok[(size_t)p * K + lane] = tok; a.o_top_logit[(size_t)p * K + lane] = val; }
-        if (a.T > 0.f) { warp_topk(a.cand_key + cb, a.cand_lg + cb, nk, K, lane, tok, val, lg); val = lg; }
-        if (lane < K) { a.o_draw_tok[(size_t)p * K + lane] = tok; a.o_draw_logit[(size_t)p * K + lane] = val; }
+        const float2 l = warp_lse(a.sums + (size_t)p * a.ntiles, a.ntiles, a.T, lane);
+        if (lane == 0) { a.o_lse0[p] = l.x; a.o_lseT[p] = l.y; }
+        float3 w = warp_topk(a.cand_top + cb, nullptr, a.cand_cnt + p, K, lane);
+        if (lane < K) { a.o_top_tok[(size_t)p * K + lane] = __float_as_int(w.x); a.o_top_logit[(size_t)p * K + lane] = w.y; }
+        if (a.T > 0.f) w = warp_topk(a.cand_key + cb, a.cand_lg + cb, a.cand_cnt + a.cap + p, K, lane);
+        if (lane < K) { a.o_draw_tok[(size_t)p * K + lane] = __float_as_int(w.x); a.o_draw_logit[(size_t)p * K + lane] = w.z; }
       }
       break;
     }
+    }
     // ---- owners ---------------------------------------------------------------------------------------------------------
-    for (int b = cta; b < a.B; b += ncta) tx_owner(a, base_sm, b, d);
-    const int h0 = ncta - a.B >= ncta / 4 ? a.B : 0;
-    if (d + 2 < a.D && cta >= h0)
-      for (int i = (cta - h0) * TX_WARPS + warp; i < a.B * a.npiece; i += (ncta - h0) * TX_WARPS) {
-        const int b = i / a.npiece;
-        if (__ldcg(a.req_npar + (d & 1) * a.B + b) > 0)
-          scout_piece(a, b * a.D + d + 2, i % a.npiece, piece_len, a.utop + (size_t)(d & 1) * a.B * a.npiece + i, lane);
-      }
-    if (d + 1 >= a.D) break;
+    if (d >= -1)
+#pragma unroll 1
+      for (int b = cta; b < nreq; b += ncta) tx_owner(a, base_sm, b, d);
+    // best base logits of the rows after the next ones, by the CTAs that own no request where there are enough of them
+    // (given parents: of their rows, before anything else)
+    if (d == -2 || (a.score_P == 0 && d + 2 < a.D)) {
+      const int h0 = d >= -1 && ncta - a.B >= ncta / 4 ? a.B : 0;
+      uint2* ut = a.utop + (size_t)(d & 1) * a.B * a.npiece;
+      if (cta >= h0)
+#pragma unroll 1
+        for (int i = (cta - h0) * TX_WARPS + warp; i < nreq * a.npiece; i += (ncta - h0) * TX_WARPS) {
+          const int x = i / a.npiece;
+          if (d >= 0 && __ldcg(a.req_npar + (d & 1) * a.B + x) <= 0) continue;
+          const int row = a.score_P > 0 ? a.p_req[x] * a.D + a.p_depth[x] : x * a.D + d + 2;
+          scout_piece(a, row, i % a.npiece, piece_len, ut + i, lane);
+        }
+    }
+    if (d + 1 >= a.D && a.score_P == 0) break;
     fence_async_smem();   // owners work in memory that the next scan's bulk loads may write
     __threadfence();
     if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
+    if (d == -2 && a.ragged) asm volatile("fence.proxy.async;" ::: "memory");
+  }
+  if (dead && d == -2 && a.score_P == 0) {
+    for (int b = cta; b < a.B; b += ncta) {   // nothing of these requests exists yet: an empty tree
+      PoolView g = pool_view(a.pool + (size_t)b * a.pool_stride, a.N);
+      for (int i = tid; i < a.N; i += TX_THREADS) g.meta[i] = 0;
+      if (tid == 0) { a.status[b] = TS_OK; a.req_nscored[b] = 0; a.root_lseT[b] = nanf(""); }
+    }
+    __syncthreads();
   }
   // ---- no copy may still be writing this CTA's shared memory when the last phase works in it or the CTA ends -----------
   cp_async_wait_all();
-  if (a.use_tma && warp == TX_MMA && lane == 0)
-    for (; ws.issued < ws.requested; ++ws.issued) {
-      const uint32_t slot = ws.issued % (uint32_t)a.nW, use = ws.issued / (uint32_t)a.nW;
+  if (a.use_tma && warp == TX_REFRESH && lane == 0)
+    for (uint32_t x = wl.requested > (uint32_t)a.nW ? wl.requested - (uint32_t)a.nW : 0u; x < wl.requested; ++x) {
+      const uint32_t slot = x % (uint32_t)a.nW, use = x / (uint32_t)a.nW;
       bool landed = false;
       for (uint32_t i = 0; i < WAIT_LIMIT && !landed; ++i) { landed = mbar_test_wait(sm.w_full + slot, use & 1); if (!landed) __nanosleep(100); }
     }

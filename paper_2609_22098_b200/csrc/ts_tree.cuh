@@ -9,11 +9,11 @@ namespace ts {
 
 constexpr int TX_SCAN_WARPS = 16;          // warps that scan accumulators: 4 tensor-memory lane quarters x 4 splits
 constexpr int TX_SPLIT = TX_SCAN_WARPS / 4;
-constexpr int TX_MMA = TX_SCAN_WARPS;      // requests W, issues the MMAs
-constexpr int TX_REFRESH = TX_SCAN_WARPS + 1;   // keeps the rows' launch-wide bounds current
+constexpr int TX_MMA = TX_SCAN_WARPS;      // issues the MMAs
+constexpr int TX_REFRESH = TX_SCAN_WARPS + 1;   // requests W, keeps the rows' launch-wide bounds current
 constexpr int TX_SELECT = TX_SCAN_WARPS + 2;    // evaluates queued candidates exactly
 constexpr int TX_COPY = TX_SCAN_WARPS + 3;      // brings base logits into shared memory
-constexpr int TX_WARPS = TX_SCAN_WARPS + 4;
+constexpr int TX_WARPS = TX_SCAN_WARPS + 4;      // (a multiple of four: one warp more would cost every thread 16 registers)
 constexpr int TX_THREADS = TX_WARPS * 32;
 constexpr int TX_ROWS = 128;               // parent rows of one MMA tile
 constexpr int TX_QCAP = 256;               // candidate queue entries (power of two)
