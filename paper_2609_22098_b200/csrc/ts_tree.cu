@@ -28,9 +28,6 @@ namespace ts {
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool in) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
 }
-__device__ __forceinline__ void cp_async4(void* dst, const void* src, bool in) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 4 : 0) : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // arrives on `bar` when this thread's earlier cp.async have landed (the barrier counts every thread that says so)
 __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
@@ -118,29 +115,28 @@ __device__ __forceinline__ float exact_key(uint64_t seed, int req, uint64_t hash
 // counter only the index changes from call to call, and it reaches the other lane pair one round later, so one of the
 // two products of the first round and one of the second are constants of the parent.
 struct CoarseGen {
-  uint32_t x0, x1, y2, y3;   // round 1's c0 ^ , c1 ; round 2's constants
-  uint32_t k0, k1, c3;
+  uint32_t x0, y2, y3, k0, k1, c3;
   __device__ __forceinline__ void init(uint64_t seed, int req, uint64_t hash) {
     k0 = (uint32_t)seed; k1 = (uint32_t)(seed >> 32);
     c3 = (((uint32_t)req & 0xFFFFFFu) | ((uint32_t)STREAM_GUMBEL_COARSE << 24)) ^ k1;
     const uint32_t c1 = (uint32_t)hash, c2 = (uint32_t)(hash >> 32);
     const uint32_t n0 = __umulhi(0xCD9E8D57u, c2) ^ c1 ^ k0;   // round 1, word 0
-    x1 = 0xCD9E8D57u * c2;                                      // round 1, word 1
     y2 = __umulhi(0xD2511F53u, n0) ^ (k1 + 0xBB67AE85u);        // round 2, word 2 = y2 ^ (word 3 of round 1)
     y3 = 0xD2511F53u * n0;                                      // round 2, word 3
-    x0 = x1 ^ (k0 + 0x9E3779B9u);                               // round 2, word 0 = hi(M1 * word 2 of round 1) ^ x0
+    x0 = (0xCD9E8D57u * c2) ^ (k0 + 0x9E3779B9u);                               // round 2, word 0 = hi(M1 * word 2 of round 1) ^ x0
   }
   __device__ __forceinline__ uint4 words(uint32_t index) const {
     // round 1: words 2 and 3
-    const uint32_t a2 = __umulhi(0xD2511F53u, index) ^ c3, a3 = 0xD2511F53u * index;
+    const uint64_t pi = mul_wide(0xD2511F53u, index);
+    const uint32_t a2 = (uint32_t)(pi >> 32) ^ c3, a3 = (uint32_t)pi;
     // round 2
-    uint32_t c0 = __umulhi(0xCD9E8D57u, a2) ^ x0, c1 = 0xCD9E8D57u * a2, c2 = y2 ^ a3, cc3 = y3;
+    const uint64_t pa = mul_wide(0xCD9E8D57u, a2);
+    uint32_t c0 = (uint32_t)(pa >> 32) ^ x0, c1 = (uint32_t)pa, c2 = y2 ^ a3, cc3 = y3;
     uint32_t q0 = k0 + 2u * 0x9E3779B9u, q1 = k1 + 2u * 0xBB67AE85u;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const uint32_t hi0 = __umulhi(0xD2511F53u, c0), lo0 = 0xD2511F53u * c0;
-      const uint32_t hi1 = __umulhi(0xCD9E8D57u, c2), lo1 = 0xCD9E8D57u * c2;
-      c0 = hi1 ^ c1 ^ q0; c1 = lo1; c2 = hi0 ^ cc3 ^ q1; cc3 = lo0;
+      const uint64_t p0 = mul_wide(0xD2511F53u, c0), p1 = mul_wide(0xCD9E8D57u, c2);
+      c0 = (uint32_t)(p1 >> 32) ^ c1 ^ q0; c1 = (uint32_t)p1; c2 = (uint32_t)(p0 >> 32) ^ cc3 ^ q1; cc3 = (uint32_t)p0;
       q0 += 0x9E3779B9u; q1 += 0xBB67AE85u;
     }
     return make_uint4(c0, c1, c2, cc3);
@@ -183,9 +179,13 @@ __device__ __forceinline__ void tx_select(const TreeArgs& a, const TxSm& sm, con
 }
 
 // Where a role stands in the stream of blocks: every role passes every block of every group in the same order.
+// (Phases are kept per slot: with few parents a group uses more, smaller base-logit slots than with many.)
 struct BlockPos {
-  int slot, use;
-  __device__ __forceinline__ void next(int n) { if (++slot == n) { slot = 0; ++use; } }
+  int slot; uint32_t phase, seen;   // bit per slot: parity of its next "full", whether it was used before
+  __device__ __forceinline__ uint32_t full() const { return (phase >> slot) & 1u; }
+  __device__ __forceinline__ bool reused() const { return (seen >> slot) & 1u; }
+  __device__ __forceinline__ uint32_t empty() const { return full() ^ 1u; }
+  __device__ __forceinline__ void next(int n) { phase ^= 1u << slot; seen |= 1u << slot; if (++slot == n) slot = 0; }
 };
 
 __device__ __noinline__ bool tx_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort, int* err, uint32_t limit) {
@@ -211,7 +211,7 @@ __device__ __forceinline__ bool tx_wait_warp(uint64_t* bar, uint32_t parity, con
 // parent; a warp owns every (4R)-th chunk of 16 tokens, so with few parents (R = 2, 4 replicas of the rows) the
 // copies share the range.
 __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int t0, const int tlen,
-                                        const uint32_t tmem_base, BlockPos& pos) {
+                                        const uint32_t tmem_base, BlockPos& pos, const int nst, const int urows) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int q = warp & 3, s = warp >> 2, row = q * 32 + lane;
   const int per = TX_ROWS / R, K = a.K;
@@ -241,12 +241,12 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
   const int CB = a.BN / 16, nblk = (tlen + a.BN - 1) / a.BN, stride = R * TX_SPLIT, own = rho * TX_SPLIT + s;
   const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16);
   bool alive = true;
-  for (int nb = 0; nb < nblk; ++nb, pos.next(a.nU)) {
+  for (int nb = 0; nb < nblk; ++nb, pos.next(nst)) {
     const int slot = pos.slot;
-    if (!tx_wait_warp(sm.t_full + slot, pos.use & 1, sm, a) || !tx_wait_warp(sm.u_full + slot, pos.use & 1, sm, a)) { alive = false; break; }
+    if (!tx_wait_warp(sm.t_full + slot, pos.full(), sm, a) || !tx_wait_warp(sm.u_full + slot, pos.full(), sm, a)) { alive = false; break; }
     tc_fence_after();
     const int nch = min(CB, (tlen - nb * a.BN + 15) / 16);
-    const unsigned char* urow = sm.Us + (size_t)slot * (TX_ROWS * 2) * a.BN + (size_t)prow * 2 * a.BN;
+    const unsigned char* urow = sm.Us + (size_t)(slot * urows + prow) * 2 * a.BN;
     for (int c = (own - nb * CB) & (stride - 1); c < nch; c += stride) {
       uint32_t ra[16];
       __syncwarp();   // (the tensor-memory load is a warp-wide instruction)
@@ -355,18 +355,18 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
 }
 
 // ---- the copying warp: base-logit rows of every block into the ring (and W, where no tensor map could be made) ----
-__device__ __forceinline__ void tx_copy(const TreeArgs& a, const TxSm& sm, const int nrow, const int t0, const int tlen, BlockPos& pos, BlockPos& wpos) {
+__device__ __forceinline__ void tx_copy(const TreeArgs& a, const TxSm& sm, const int nrow, const int t0, const int tlen, BlockPos& pos, BlockPos& wpos, const int nst, const int urows) {
   const int lane = threadIdx.x & 31;
   const int CB8 = a.BN / 8, nblk = (tlen + a.BN - 1) / a.BN;
   const int sh = a.BN == 128 ? 4 : 3;             // log2 of the 16-byte chunks per row and block
   const int ck = lane & (CB8 - 1), r0 = lane >> sh, rstep = 32 >> sh;
   const __nv_bfloat16* Ug = reinterpret_cast<const __nv_bfloat16*>(a.Uscan);
-  for (int nb = 0; nb < nblk; ++nb, pos.next(a.nU)) {
-    if (pos.use >= 1 && !tx_wait_warp(sm.t_empty + pos.slot, (pos.use - 1) & 1, sm, a)) return;
+  for (int nb = 0; nb < nblk; ++nb, pos.next(nst)) {
+    if (pos.reused() && !tx_wait_warp(sm.t_empty + pos.slot, pos.empty(), sm, a)) return;
     const int v = t0 + nb * a.BN + ck * 8;
     const bool in = v < a.Vs;
     const __nv_bfloat16* src = in ? Ug + v : Ug;
-    unsigned char* dst = sm.Us + (size_t)pos.slot * (TX_ROWS * 2) * a.BN;
+    unsigned char* dst = sm.Us + (size_t)(pos.slot * urows) * 2 * a.BN;
     // (the row indices of eight copies are read together: one at a time the loop is a chain of shared-memory reads)
     for (int rr = r0; rr < nrow; rr += 8 * rstep) {
       int row[8];
@@ -382,7 +382,7 @@ __device__ __forceinline__ void tx_copy(const TreeArgs& a, const TxSm& sm, const
     if (!a.use_tma) {
       const int rw = (a.r + 15) / 16 * 16;
       const __nv_bfloat16* Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wscan);
-      if (wpos.use >= 1 && !tx_wait_warp(sm.w_free + wpos.slot, (wpos.use - 1) & 1, sm, a)) return;
+      if (wpos.reused() && !tx_wait_warp(sm.w_free + wpos.slot, wpos.empty(), sm, a)) return;
       unsigned char* wd = sm.Ws + (size_t)wpos.slot * rw * 2 * a.BN;
       for (int k = r0; k < rw; k += rstep) {
         const bool win = in && k < a.r;
@@ -406,9 +406,9 @@ __device__ __forceinline__ void tx_load(const TreeArgs& a, const TxSm& sm, const
   const int nblk = (tlen + a.BN - 1) / a.BN, rw = (a.r + 15) / 16 * 16;
   const uint32_t slab = (uint32_t)rw * 128u;
   for (; w.requested < upto; ++w.requested, w.pos.next(a.nW)) {
-    if (w.pos.use >= 1) {
-      if (BLOCKING) { if (!tx_wait_warp(sm.w_free + w.pos.slot, (w.pos.use - 1) & 1, sm, a)) return; }
-      else if (!__all_sync(0xFFFFFFFFu, mbar_test_wait(sm.w_free + w.pos.slot, (w.pos.use - 1) & 1))) return;
+    if (w.pos.reused()) {
+      if (BLOCKING) { if (!tx_wait_warp(sm.w_free + w.pos.slot, w.pos.empty(), sm, a)) return; }
+      else if (!__all_sync(0xFFFFFFFFu, mbar_test_wait(sm.w_free + w.pos.slot, w.pos.empty()))) return;
     }
     if (elect_one()) {
       const int ns = min(a.BN / 64, (tlen - w.nb * a.BN + 63) / 64);
@@ -422,14 +422,14 @@ __device__ __forceinline__ void tx_load(const TreeArgs& a, const TxSm& sm, const
 }
 
 // ---- the issuing warp: one tile of MMAs per block -----------------------------------------------------------------------
-__device__ __forceinline__ void tx_issue(const TreeArgs& a, const TxSm& sm, const int tlen, const uint32_t tmem_base, BlockPos& pos, BlockPos& wpos, const int group_no) {
+__device__ __forceinline__ void tx_issue(const TreeArgs& a, const TxSm& sm, const int tlen, const uint32_t tmem_base, BlockPos& pos, BlockPos& wpos, const int group_no, const int nst) {
   const int nblk = (tlen + a.BN - 1) / a.BN, ksteps = (a.r + 15) / 16;
   const uint32_t slab = (uint32_t)ksteps * 2048u;
   const uint64_t adesc0 = smem_desc(smem_u32(sm.As), 16u, 1024u), bdesc0 = smem_desc(smem_u32(sm.Ws), slab, 1024u);
   if (!tx_wait_warp(sm.a_full, group_no & 1, sm, a)) return;
-  for (int nb = 0; nb < nblk; ++nb, pos.next(a.nU), wpos.next(a.nW)) {
-    if (!tx_wait_warp(sm.w_full + wpos.slot, wpos.use & 1, sm, a)) return;
-    if (pos.use >= 1 && !tx_wait_warp(sm.t_empty + pos.slot, (pos.use - 1) & 1, sm, a)) return;
+  for (int nb = 0; nb < nblk; ++nb, pos.next(nst), wpos.next(a.nW)) {
+    if (!tx_wait_warp(sm.w_full + wpos.slot, wpos.full(), sm, a)) return;
+    if (pos.reused() && !tx_wait_warp(sm.t_empty + pos.slot, pos.empty(), sm, a)) return;
     tc_fence_after();
     if (elect_one()) {
       const int n = min(a.BN, (tlen - nb * a.BN + 63) / 64 * 64);   // whole 64-token slabs
@@ -457,6 +457,9 @@ __device__ __forceinline__ void tx_refresh(const TreeArgs& a, const TxSm& sm, co
   for (uint32_t spin = 0; spin < a.wait_limit; ++spin) {
     if (a.use_tma) tx_load<false>(a, sm, tm, t0, tlen, w, upto);
     if (*sm.done >= done_target || *sm.abort) break;
+    // (a pass is a memory round trip: steady at first, while the bounds rise, every eighth turn later, so that the end of
+    // the scan is seldom waited for)
+    if (spin >= 12u && (spin & 7u)) { __nanosleep(100); continue; }
     unsigned v = 0xFFFFFFFFu;
     if (p_own < p_hi && j < K) v = __ldcg(a.slots + (((size_t)which * a.cap + p_own) * K + j) * SLOT_STRIDE);
     unsigned rL[4], rK[4];
@@ -485,7 +488,6 @@ __device__ __forceinline__ void tx_refresh(const TreeArgs& a, const TxSm& sm, co
         sm.thr[TX_ROWS + rr] = fmaxf(dec_f(rK[k]), sm.ent[rr].thrK);
       }
     }
-    __nanosleep(spin < 16u ? 32 : 200);
   }
   __syncwarp();
   if (a.use_tma && !*sm.abort) tx_load<true>(a, sm, tm, t0, tlen, w, upto);
@@ -546,6 +548,7 @@ __device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, co
   if (row < per) {
     // the pieces' sums in a fixed order: the same bits on every run
     float m = -INFINITY, s0 = 0.f, sT = 0.f;
+#pragma unroll 1
     for (int rho = 0; rho < R; ++rho)
 #pragma unroll
       for (int s = 0; s < TX_SPLIT; ++s) {
@@ -562,21 +565,21 @@ __device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, co
   const float gL = sm.thr[prow], gK = sm.thr[TX_ROWS + prow];
   const float* L = sm.lists + (size_t)row * 5 * K;
   const int* Li = reinterpret_cast<const int*>(L);
-  int n = sm.ln[row], k = 0;
-  while (k < n && L[k] >= gL) ++k;
-  if (k) {
-    const int at = atomicAdd(a.cand_cnt + p, k);
-    for (int j = 0; j < k; ++j) a.cand_top[base + at + j] = make_uint2(__float_as_uint(L[j]), (unsigned)Li[K + j]);
+  int kt = 0, kk = 0;
+#pragma unroll 1
+  for (int n = sm.ln[row]; kt < n && L[kt] >= gL;) ++kt;
+#pragma unroll 1
+  for (int n = sm.ln[TX_ROWS + row]; kk < n && L[2 * K + kk] >= gK;) ++kk;
+  int at = 0, ak = 0;
+  if (kt) at = atomicAdd(a.cand_cnt + p, kt);
+  if (kk) ak = atomicAdd(a.cand_cnt + a.cap + p, kk);
+#pragma unroll 1
+  for (int j = 0; j < kk; ++j) {
+    a.cand_key[base + ak + j] = make_uint2(__float_as_uint(L[2 * K + j]), (unsigned)Li[3 * K + j]);
+    a.cand_lg[base + ak + j] = L[4 * K + j];
   }
-  n = sm.ln[TX_ROWS + row]; k = 0;
-  while (k < n && L[2 * K + k] >= gK) ++k;
-  if (k) {
-    const int at = atomicAdd(a.cand_cnt + a.cap + p, k);
-    for (int j = 0; j < k; ++j) {
-      a.cand_key[base + at + j] = make_uint2(__float_as_uint(L[2 * K + j]), (unsigned)Li[3 * K + j]);
-      a.cand_lg[base + at + j] = L[4 * K + j];
-    }
-  }
+#pragma unroll 1
+  for (int j = 0; j < kt; ++j) a.cand_top[base + at + j] = make_uint2(__float_as_uint(L[j]), (unsigned)Li[K + j]);
 }
 
 // ---- merge of one parent, by one warp --------------------------------------------------------------------------------
@@ -749,13 +752,27 @@ __device__ __forceinline__ OwnerSm owner_carve(unsigned char* sm, const TreeArgs
   return s;
 }
 
-// The seed tokens' columns of W on their way into shared memory (words of two tokens; rows of r + 1 words: the threads
-// that later read one k of different tokens hit different banks).  All threads; cp_async_wait_all and a barrier follow.
-__device__ __forceinline__ void fetch_seed_columns(const TreeArgs& a, const OwnerSm& s, int NS) {
-  const __nv_bfloat16* Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wscan);
-  for (int e = threadIdx.x; e < NS * a.r; e += TX_THREADS) {
-    const int j = e % NS, k = e / NS, tok = s.stok[j];
-    cp_async4(s.Wc + (size_t)j * (a.r + 1) + k, tok >= 0 ? Wg + (size_t)k * a.Vs + (tok & ~1) : Wg, tok >= 0);
+// The seed tokens' columns of W (words of two tokens; rows of r + 1 words in shared memory: the threads that later read one
+// k of different tokens hit different banks).  All threads; every word is a sector of its own, so a thread requests its
+// words together, and keeps them in registers while other work goes on (cp.async of 4 bytes took 5 us for 1024 of them).
+constexpr int SEED_REGS = 4;
+__device__ __forceinline__ void load_seed_columns(const TreeArgs& a, const OwnerSm& s, int NS, int e0, uint32_t* w) {
+  const uint32_t* Wg = reinterpret_cast<const uint32_t*>(a.Wscan);
+#pragma unroll
+  for (int u = 0; u < SEED_REGS; ++u) {
+    const int e = e0 + u * TX_THREADS + (int)threadIdx.x;
+    w[u] = 0u;
+    if (e < NS * a.r) {
+      const int j = e & (NS - 1), k = e >> seed_log2(a.K), tok = s.stok[j];
+      if (tok >= 0) w[u] = __ldg(Wg + (((size_t)k * a.Vs + tok) >> 1));
+    }
+  }
+}
+__device__ __forceinline__ void store_seed_columns(const TreeArgs& a, const OwnerSm& s, int NS, int e0, const uint32_t* w) {
+#pragma unroll
+  for (int u = 0; u < SEED_REGS; ++u) {
+    const int e = e0 + u * TX_THREADS + (int)threadIdx.x;
+    if (e < NS * a.r) s.Wc[(e & (NS - 1)) * (a.r + 1) + (e >> seed_log2(a.K))] = w[u];
   }
 }
 
@@ -763,28 +780,32 @@ __device__ __forceinline__ void fetch_seed_columns(const TreeArgs& a, const Owne
 // s.ttok[i], hash hs[i], pool slot s.npl[i]; its place in the level's list is li0 + i.
 __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s, const int cnt, const int li0, const int req, const int row, const int NS,
                                              const int* ptok, const uint64_t* phash, ParentEntry* ent, int* ent_slot) {
-  const int tid = threadIdx.x, r = a.r, K = a.K;
+  const int tid = threadIdx.x, r = a.r, K = a.K, lg = seed_log2(K);
   const float invT = a.T > 0.f ? 1.f / a.T : 1.f;
   const __nv_bfloat16* Ag = reinterpret_cast<const __nv_bfloat16*>(a.A);
   // the parents' pruning state and candidate counts start clean
+#pragma unroll 1
   for (int e = tid; e < cnt * 2 * K; e += TX_THREADS) {
     const int i = e / (2 * K), w = (e / K) & 1, j = e % K;
     a.slots[(((size_t)w * a.cap + li0 + i) * K + j) * SLOT_STRIDE] = 0u;
   }
+#pragma unroll 1
   for (int e = tid; e < cnt * 2; e += TX_THREADS) {
     a.thr[(size_t)(e & 1) * a.cap + li0 + (e >> 1)] = 0u;
     a.cand_cnt[(size_t)(e & 1) * a.cap + li0 + (e >> 1)] = 0;
   }
   // every (parent, seed token) pair exactly: eight lanes a pair, 16 bytes of the head row a lane and step
   const int sub = tid & 7;
+#pragma unroll 1
   for (int e0 = 0; e0 < cnt * NS; e0 += TX_THREADS / 8) {
     const int e = e0 + (tid >> 3);
     const bool have = e < cnt * NS;
-    const int i = have ? e / NS : 0, j = have ? e % NS : 0, tok = s.stok[j];
+    const int i = have ? e >> lg : 0, j = e & (NS - 1), tok = s.stok[j];
     float dot = 0.f;
     if (have && tok >= 0) {
       const uint32_t* wc = s.Wc + (size_t)j * (r + 1);
       const int hi = tok & 1;
+#pragma unroll 1
       for (int k = sub * 8; k < r; k += 64) {
         float av[8];
         unpack_bf16x8(__ldg(reinterpret_cast<const uint4*>(Ag + (size_t)ptok[i] * r + k)), av);
@@ -794,23 +815,26 @@ __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s
     }
     dot += __shfl_xor_sync(0xFFFFFFFFu, dot, 1); dot += __shfl_xor_sync(0xFFFFFFFFu, dot, 2); dot += __shfl_xor_sync(0xFFFFFFFFu, dot, 4);
     if (have && sub == 0) {
-      float lg = -INFINITY, key = -INFINITY;
+      float lo = -INFINITY, key = -INFINITY;
       if (tok >= 0) {
-        lg = s.sval[j] + dot;
-        key = a.T > 0.f ? exact_key(a.seed, req, phash[i], tok, lg, invT) : lg;
+        lo = s.sval[j] + dot;
+        key = a.T > 0.f ? exact_key(a.seed, req, phash[i], tok, lo, invT) : lo;
       }
-      s.res[2 * e] = lg; s.res[2 * e + 1] = key;
+      s.res[2 * e] = lo; s.res[2 * e + 1] = key;
     }
   }
   float* bL = reinterpret_cast<float*>(s.tcnt); float* bK = reinterpret_cast<float*>(s.toff); float* bM = reinterpret_cast<float*>(s.hist);
+#pragma unroll 1
   for (int i = tid; i < cnt; i += TX_THREADS) { bL[i] = -INFINITY; bK[i] = -INFINITY; bM[i] = -INFINITY; }
   __syncthreads();
+#pragma unroll 1
   for (int e = tid; e < 2 * cnt * NS; e += TX_THREADS) {
     // one thread per value: the one with exactly K - 1 values before it (ties broken by place) is the K-th best
-    const int j = e % NS, which = (e / NS) & 1, i = e / (2 * NS);
+    const int j = e & (NS - 1), which = (e >> lg) & 1, i = e >> (lg + 1);
     const float* val = s.res + (size_t)i * NS * 2 + which;
     const float mine = val[2 * j];
     int before = 0;
+#pragma unroll 1
     for (int t = 0; t < NS; ++t) before += (val[2 * t] > mine || (val[2 * t] == mine && t < j)) ? 1 : 0;
     const bool fin = mine == mine && fabsf(mine) < INFINITY;
     if (before == K - 1 && fin && !a.no_seed) {
@@ -821,6 +845,7 @@ __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s
     if (before == 0 && which == 0 && fin) bM[i] = mine;
   }
   __syncthreads();
+#pragma unroll 1
   for (int i = tid; i < cnt; i += TX_THREADS) {
     ParentEntry pe;
     pe.row = row; pe.token = ptok[i]; pe.hash = phash[i]; pe.thrL = bL[i]; pe.thrK = a.T > 0.f ? bK[i] : -INFINITY; pe.mref = bM[i]; pe.req = req;
@@ -858,6 +883,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     if (given) { req = a.p_req[b]; row = req * a.D + a.p_depth[b]; }
     else {
       PoolView g = pool_view(gpool, N);
+#pragma unroll 1
       for (int i = tid; i < N; i += TX_THREADS) g.meta[i] = 0;
     }
     if (tid == 0) {
@@ -881,7 +907,9 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     tx_caps(a, b, K_eff, N_eff, log_theta);
     more = d + 1 < a.D;
     uint4* dst = reinterpret_cast<uint4*>(s.pv.key); const uint4* src = reinterpret_cast<const uint4*>(gpool);
+#pragma unroll 1
     for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) dst[i] = __ldcg(src + i);
+#pragma unroll 1
     for (int i = tid; i < npar; i += TX_THREADS) s.pslot[i] = __ldcg(a.ent_slot[cur] + base + i);
     if (tid < 8) sh[tid] = 0;
   }
@@ -908,7 +936,8 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     }
   }
   __syncthreads();
-  if (more) fetch_seed_columns(a, s, NS);   // lands while the slots are formed
+  uint32_t wcol[SEED_REGS];
+  if (more) load_seed_columns(a, s, NS, 0, wcol);   // on their way while the draws are ranked
   if (d >= 0) {
   // the best token of q0 not among the first j draws, for every j: places of the draws in the top list, or-ed up
 #pragma unroll 1
@@ -926,6 +955,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     if (lane < K) { const unsigned fr = ~(lane ? prior : 0u) & ((1u << K_eff) - 1u); s.best[i * K + lane] = fr ? (unsigned char)(__ffs(fr) - 1) : 255u; }
   }
   __syncthreads();
+  if (more) store_seed_columns(a, s, NS, 0, wcol);
   // ---- slots of every scored parent: two threads per (parent, sibling rank), one for the key (the best unused token's
   // estimate), one for the survival of the token drawn ----
 #pragma unroll 1
@@ -957,10 +987,13 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
   // a sibling slot exists only if the one before it was admitted (keys are non-increasing in j)
   {
     int nv = 0, np = 0;
+#pragma unroll 1
     for (int i = tid; i < npar; i += TX_THREADS) {
       bool open = true;
+#pragma unroll 1
       for (int j = 0; j < K; ++j) { if (!s.valid[i * K + j]) open = false; if (open) ++nv; else s.valid[i * K + j] = 0; }
     }
+#pragma unroll 1
     for (int i = tid; i < N; i += TX_THREADS) np += s.pv.meta[i] >> 16;
     nv = __reduce_add_sync(0xFFFFFFFFu, nv); np = __reduce_add_sync(0xFFFFFFFFu, np);
     if (lane == 0) { if (np) atomicAdd(&sh[0], np); if (nv) atomicAdd(&sh[1], nv); }
@@ -988,9 +1021,11 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     // (depth, path) for the places that are left.
     uint64_t prefix = 0;
     int need = N_eff;
+#pragma unroll 1
     for (int sh8 = 56; sh8 >= 0; sh8 -= 8) {
       if (tid < 256) s.hist[tid] = 0;
       __syncthreads();
+#pragma unroll 1
       for (int e = tid; e < M; e += TX_THREADS) {
         if (!live(e)) continue;
         const uint64_t k = skey(key_of(e));
@@ -1022,11 +1057,13 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     }
     if (tid == 0) sh[4] = 0;
     __syncthreads();
+#pragma unroll 1
     for (int e = tid; e < M; e += TX_THREADS)
       if (live(e) && skey(key_of(e)) == prefix) { const int at = atomicAdd(&sh[4], 1); if (at < 256) s.newl[at] = e; }
     __syncthreads();
     const int ntie = sh[4];
     unsigned drop = 0u;   // bit per trip: M <= 17 * 256 entries, at most 7 trips
+#pragma unroll 1
     for (int e = tid, it = 0; e < M; e += TX_THREADS, ++it) {
       if (!live(e)) continue;
       const double ke = key_of(e);
@@ -1036,6 +1073,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
         int rank = 0;
         const int de = depth_of(e); const uint64_t pe = path_of(e);
         const int nn = ntie <= 256 ? ntie : M;
+#pragma unroll 1
         for (int t = 0; t < nn; ++t) {
           const int f = ntie <= 256 ? s.newl[t] : t;
           if (f == e || (ntie > 256 && !(live(f) && skey(key_of(f)) == prefix))) continue;
@@ -1046,6 +1084,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       drop |= (out ? 1u : 0u) << it;
     }
     __syncthreads();
+#pragma unroll 1
     for (int e = tid, it = 0; e < M; e += TX_THREADS, ++it)
       if ((drop >> it) & 1u) { if (e < N) s.pv.meta[e] &= 0xFFFF; else s.valid[e - N] = 0; }
     __syncthreads();
@@ -1057,6 +1096,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     if (lane == 0 && warp < 8) s.npl[warp] = __popc(bal);
     const int ntrip = (ncand + TX_THREADS - 1) / TX_THREADS;   // <= 7
     unsigned vm = 0;
+#pragma unroll 1
     for (int it = 0; it < ntrip; ++it) {
       const int c = it * TX_THREADS + tid;
       const bool v = c < ncand && s.valid[c];
@@ -1066,11 +1106,13 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     }
     __syncthreads();
     int off = 0, nfree = 0;
+#pragma unroll 1
     for (int w = 0; w < 8; ++w) { if (w < warp) off += s.npl[w]; nfree += s.npl[w]; }
     if (fr) s.hist[off + __popc(bal & ((1u << lane) - 1u))] = tid;
     const int ne = ntrip * TX_WARPS;
     if (warp == 0) {   // exclusive prefix over (trip, warp)
       int run = 0;
+#pragma unroll 1
       for (int e0 = 0; e0 < ne; e0 += 32) {
         const int e = e0 + lane, c = e < ne ? s.tcnt[e] : 0;
         int incl = c;
@@ -1083,6 +1125,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       if (lane == 0 && run > nfree) a.status[b] = TS_ERR_OVERFLOW;
     }
     __syncthreads();
+#pragma unroll 1
     for (int it = 0; it < ntrip; ++it) {
       const bool v = (vm >> it) & 1u;
       const unsigned vb = __ballot_sync(0xFFFFFFFFu, v);
@@ -1113,6 +1156,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     __syncthreads();
     int off = 0;
     cnt = 0;
+#pragma unroll 1
     for (int w = 0; w < 8; ++w) { if (w < warp) off += s.tcnt[w]; cnt += s.tcnt[w]; }
     if (tid == 0) {
       const int nb = cnt > 0 ? atomicAdd(a.lvl_count + d + 1, cnt) : 0;
@@ -1121,10 +1165,14 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     if (par) { const int i = off + __popc(bal & ((1u << lane) - 1u)); s.npl[i] = sl; ptok[i] = pt; phash[i] = ph; }
   }
   uint4* gdst = reinterpret_cast<uint4*>(gpool); const uint4* psrc = reinterpret_cast<const uint4*>(s.pv.key);
+#pragma unroll 1
   for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) gdst[i] = psrc[i];
   }
   // ---- seed bounds and list entries ----
-  if (more) cp_async_wait_all();
+  if (more && d < 0) store_seed_columns(a, s, NS, 0, wcol);
+  if (more)
+#pragma unroll 1
+    for (int e0 = SEED_REGS * TX_THREADS; e0 < NS * a.r; e0 += SEED_REGS * TX_THREADS) { load_seed_columns(a, s, NS, e0, wcol); store_seed_columns(a, s, NS, e0, wcol); }
   __syncthreads();
   if (d >= 0) li0 = sh[6];
   if (more && cnt > 0) make_parents(a, s, cnt, li0, req, row, NS, ptok, phash, a.ent[nxt], a.ent_slot[nxt]);
@@ -1140,18 +1188,21 @@ __device__ __forceinline__ void tx_finalize(const TreeArgs& a, unsigned char* sm
   __shared__ int n_sh;
   {
     uint4* dst = reinterpret_cast<uint4*>(s.pv.key); const uint4* src = reinterpret_cast<const uint4*>(a.pool + (size_t)b * a.pool_stride);
+#pragma unroll 1
     for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) dst[i] = __ldcg(src + i);
   }
   if (tid == 0) n_sh = 0;
   __syncthreads();
   // a node's places by counting; G neighbouring lanes share a node's comparisons
   const int G = N <= 80 ? 8 : (N <= 160 ? 4 : 2);
+#pragma unroll 1
   for (int q0 = 0; q0 < N; q0 += TX_THREADS / G) {
     const int x = q0 + tid / G, sub = tid % G;
     const bool have = x < N && (s.pv.meta[x] >> 16) != 0;
     int cr = 0, pr = 0;
     if (have) {
       const int dx = (s.pv.meta[x] >> 8) & 255; const uint64_t px = s.pv.path[x]; const double kx = s.pv.key[x];
+#pragma unroll 1
       for (int t = sub; t < N; t += G) {
         const int mt = s.pv.meta[t];
         if (t == x || !(mt >> 16)) continue;
@@ -1174,6 +1225,7 @@ __device__ __forceinline__ void tx_finalize(const TreeArgs& a, unsigned char* sm
     }
   }
   __syncthreads();
+#pragma unroll 1
   for (int x = tid; x < N; x += TX_THREADS) {
     const int c = canon[x];
     if (c < 0) continue;
@@ -1191,9 +1243,11 @@ __device__ __forceinline__ void tx_finalize(const TreeArgs& a, unsigned char* sm
   __syncthreads();
   // a node's mask row: its own bit and its ancestors', up the (short) chain of parents
   const int n = n_sh;
+#pragma unroll 1
   for (int e = tid; e < n * a.words; e += TX_THREADS) {
     const int i = e / a.words, w = e % a.words;
     uint64_t m = 0ull;
+#pragma unroll 1
     for (int x = i; x >= 0; x = cpar[x]) if ((x >> 6) == w) m |= 1ull << (x & 63);
     a.mask[pb * a.words + e] = m;
   }
@@ -1231,8 +1285,8 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
   unsigned gen = 0;
   const unsigned nexpect = (unsigned)ncta + (a.lost_arrival ? 1u : 0u);
   bool dead = false;
-  WLoad wl{{0, 0}, 0, 0u};
-  BlockPos pos{0, 0}, wpos{0, 0};
+  WLoad wl{{0, 0u, 0u}, 0, 0u};
+  BlockPos pos{0, 0u, 0u}, wpos{0, 0u, 0u};
   int groups = 0;
   const int nreq = a.score_P > 0 ? a.score_P : a.B;
   const int piece_len = (((a.V + a.npiece - 1) / a.npiece) + 7) & ~7;
@@ -1278,14 +1332,17 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
         if (g == 0) for (int i = tid; i < TX_QCAP; i += TX_THREADS) sm.q[i].w = 0u;   // (owners work in this memory: the queue's tags start clean)
         __syncthreads();
         const int done_target = (groups + 1) * TX_SCAN_WARPS;
-        if (warp < TX_SCAN_WARPS) tx_scan(a, sm, R, P, g, t0, tlen, tmem_base, pos);
-        else if (warp == TX_MMA) tx_issue(a, sm, tlen, tmem_base, pos, wpos, groups);
+        // with at most 64 parents a base-logit slot is half as large and the accumulators allow four stages
+        const int urows = R > 1 ? per : TX_ROWS, nst = min(a.nU * R, 512 / a.BN < TX_STAGE_MAX ? 512 / a.BN : TX_STAGE_MAX);
+        pos.slot = 0;
+        if (warp < TX_SCAN_WARPS) tx_scan(a, sm, R, P, g, t0, tlen, tmem_base, pos, nst, urows);
+        else if (warp == TX_MMA) tx_issue(a, sm, tlen, tmem_base, pos, wpos, groups, nst);
         else if (warp == TX_REFRESH) {
           const uint32_t nblk = (uint32_t)((tlen + a.BN - 1) / a.BN);
           const uint32_t level_end = (uint32_t)(groups + ngroups - g) * nblk + ((a.w_over || a.score_P > 0) ? 0u : (uint32_t)a.nW);
           tx_refresh(a, sm, R, P, g, cta, done_target, &tmW, t0, tlen, wl, min((uint32_t)(groups + 1) * nblk + (uint32_t)a.nW, level_end));
         } else if (warp == TX_SELECT) tx_drain(a, sm, R, g, cta, done_target);
-        else tx_copy(a, sm, R > 1 ? P : min(TX_ROWS, P - g * TX_ROWS), t0, tlen, pos, wpos);
+        else tx_copy(a, sm, R > 1 ? P : min(TX_ROWS, P - g * TX_ROWS), t0, tlen, pos, wpos, nst, urows);
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
@@ -1398,8 +1455,9 @@ bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
     if (total(nU, nW) > avail) continue;
     for (;;) {   // the base-logit ring first: its loads start late
       if (nU < 3 && total(nU + 1, nW) <= avail) { ++nU; continue; }
+      if (nW < 4 && total(nU, nW + 1) <= avail) { ++nW; continue; }
+      if (nU < 512 / BN && total(nU + 1, nW) <= avail) { ++nU; continue; }   // (as many accumulators as tensor memory holds)
       if (nW < TX_STAGE_MAX && total(nU, nW + 1) <= avail) { ++nW; continue; }
-      if (nU < TX_STAGE_MAX && total(nU + 1, nW) <= avail) { ++nU; continue; }
       break;
     }
     p.BN = BN; p.nU = nU; p.nW = nW;

@@ -17,7 +17,7 @@ constexpr int TX_WARPS = TX_SCAN_WARPS + 4;      // (a multiple of four: one war
 constexpr int TX_THREADS = TX_WARPS * 32;
 constexpr int TX_ROWS = 128;               // parent rows of one MMA tile
 constexpr int TX_QCAP = 256;               // candidate queue entries (power of two)
-constexpr int TX_STAGE_MAX = 4;
+constexpr int TX_STAGE_MAX = 8;
 constexpr int TX_PIECE = 1024;             // tokens of one scouting item
 
 // Everything the scan needs to know about one parent.
@@ -78,7 +78,9 @@ __device__ __forceinline__ PoolView pool_view(unsigned char* p, int N) {
 
 // Bytes of shared memory the owner of a request works in (pool, merged results, candidates, seed columns).
 struct OwnerLayout { uint32_t pool, lse, toks, cand, flags, lists, seeds, total; };
-__host__ __device__ inline int seed_count(int K) { return 2 * K < 8 ? 8 : 2 * K; }   // tokens evaluated for a parent's seed bounds, at most 32
+// tokens evaluated for a parent's seed bounds: at least 2K (K <= 16), a power of two
+__host__ __device__ inline int seed_log2(int K) { return K <= 4 ? 3 : (K <= 8 ? 4 : 5); }
+__host__ __device__ inline int seed_count(int K) { return 1 << seed_log2(K); }
 __host__ __device__ inline OwnerLayout owner_layout(int N, int K, int r) {
   OwnerLayout o; uint32_t at = 0;
   auto take = [&](size_t bytes) { uint32_t x = at; at = (uint32_t)((at + bytes + 15) & ~(size_t)15); return x; };
