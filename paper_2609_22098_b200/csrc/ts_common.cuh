@@ -342,7 +342,7 @@ __device__ __forceinline__ double log_phat(const DevCalib& c, int d, double lx, 
   t = t > 30.0 ? 30.0 : (t < -30.0 ? -30.0 : t);
   if (c.mode == 0) {
     const double x = c.a * t + c.b;
-    return x >= 0 ? -log1p(exp(-x)) : x - log1p(exp(x));
+    return (x >= 0 ? 0.0 : x) - log1p(exp(-fabs(x)));
   }
   const float* y = c.table + d * KNOTS;
   const double pos = (t - c.lo) / (c.hi - c.lo) * (KNOTS - 1);
@@ -366,16 +366,18 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned nblocks, un
   __syncthreads();
   bool ok = true;
   if (threadIdx.x == 0) {
-    __threadfence();
+    // release (what the block wrote, ordered before this by the block barrier) without waiting for the old count; then
+    // acquire: no fence of its own on either side
     const unsigned target = (gen + 1) * nblocks;
-    atomicAdd(&bar[0], 1u);
-    unsigned spins = 0;
-    while (*((volatile unsigned*)&bar[0]) < target) {
-      if (*((volatile unsigned*)&bar[1]) != 0u) { ok = false; break; }
-      if (++spins > limit) { atomicExch(&bar[1], 1u); ok = false; break; }
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    unsigned spins = 0, seen;
+    for (;;) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+      if (seen >= target) break;
+      if ((++spins & 15u) == 0u && *((volatile unsigned*)&bar[1]) != 0u) { ok = false; break; }
+      if (spins > limit) { atomicExch(&bar[1], 1u); ok = false; break; }
       if (spins > 256u) __nanosleep(32);
     }
-    __threadfence();
   }
   gen++;
   ok = __syncthreads_and((int)ok) != 0;

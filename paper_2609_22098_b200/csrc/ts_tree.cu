@@ -584,7 +584,7 @@ __device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, co
 
 // ---- merge of one parent, by one warp --------------------------------------------------------------------------------
 // The K best of n (value, token) pairs (value desc, token asc): lane j < K gets the j-th in (tok, val, lg).  Batches of
-// up to 224 entries in registers beside the winners so far; a round is two warp-wide maxima (the value's order-
+// up to 96 entries in registers beside the winners so far; a round is two warp-wide maxima (the value's order-
 // preserving image, then the inverted token among its ties) and one removal.
 __device__ __noinline__ float3 warp_topk(const uint2* cand, const float* lgs, const int* count, int K, int lane) {
   uint32_t wv = 0u, wt = 0u; float wl = 0.f;   // winner `lane` so far: 0 = none
@@ -593,12 +593,12 @@ __device__ __noinline__ float3 warp_topk(const uint2* cand, const float* lgs, co
   const uint2 pre0 = __ldcg(cand + lane), pre1 = __ldcg(cand + 32 + lane);
   const float pl0 = lgs ? __ldcg(lgs + lane) : 0.f, pl1 = lgs ? __ldcg(lgs + 32 + lane) : 0.f;
 #pragma unroll 1
-  for (int base = 0; base < n; base += 7 * 32) {
-    uint32_t ev[8], et[8]; float el[8];
+  for (int base = 0; base < n; base += 3 * 32) {
+    uint32_t ev[4], et[4]; float el[4];
     ev[0] = wv; et[0] = wt; el[0] = wl;
-    const int used = min(7, (n - base + 31) / 32);   // (warp-uniform) slots of 32 entries in this batch
+    const int used = min(3, (n - base + 31) / 32);   // (warp-uniform) slots of 32 entries in this batch
 #pragma unroll
-    for (int u = 1; u < 8; ++u) {
+    for (int u = 1; u < 4; ++u) {
       const int i = base + (u - 1) * 32 + lane;
       ev[u] = 0u; et[u] = 0u; el[u] = 0.f;
       if (u <= used && i < n) {
@@ -612,7 +612,7 @@ __device__ __noinline__ float3 warp_topk(const uint2* cand, const float* lgs, co
     for (int j = 0; j < K; ++j) {
       uint32_t bv = ev[0], bt = et[0]; float bl = el[0];
 #pragma unroll
-      for (int u = 1; u < 8; ++u)
+      for (int u = 1; u < 4; ++u)
         if (u <= used && (ev[u] > bv || (ev[u] == bv && et[u] > bt))) { bv = ev[u]; bt = et[u]; bl = el[u]; }
       const uint32_t mv = __reduce_max_sync(0xFFFFFFFFu, bv);
       if (mv == 0u) break;   // warp-uniform
@@ -622,7 +622,7 @@ __device__ __noinline__ float3 warp_topk(const uint2* cand, const float* lgs, co
       const float l = __shfl_sync(0xFFFFFFFFu, bl, __ffs(who) - 1);
       if (mine) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) if (ev[u] == mv && et[u] == mt) { ev[u] = 0u; et[u] = 0u; }
+        for (int u = 0; u < 4; ++u) if (ev[u] == mv && et[u] == mt) { ev[u] = 0u; et[u] = 0u; }
       }
       if (lane == j) { wv = mv; wt = mt; wl = l; }
     }
@@ -631,7 +631,7 @@ __device__ __noinline__ float3 warp_topk(const uint2* cand, const float* lgs, co
 }
 
 // Log-normalisers of a parent from its ranges' sums; every lane gets them.
-__device__ __forceinline__ float2 warp_lse(const float4* h, const int nt, const float T, int lane) {
+__device__ __noinline__ float2 warp_lse(const float4* h, const int nt, const float T, int lane) {
   const float invT = T > 0.f ? 1.f / T : 1.f;
   float m = -INFINITY, s0 = 0.f, sT = 0.f;
 #pragma unroll 1
@@ -738,17 +738,16 @@ struct OwnerSm {
   unsigned char *valid, *best; int *hist, *newl, *tcnt, *toff, *npl; uint32_t* Wc; int* stok; float* sval; float* res;
 };
 __device__ __forceinline__ OwnerSm owner_carve(unsigned char* sm, const TreeArgs& a) {
-  const int N = a.N, K = a.K;
-  const OwnerLayout o = owner_layout(N, K, a.r);
+  const int N = a.N, NK = a.N << slot_log2(a.K);
   OwnerSm s;
-  s.pv = pool_view(sm + o.pool, N);
-  s.lse0 = reinterpret_cast<float*>(sm + o.lse); s.lseT = s.lse0 + N; s.pslot = reinterpret_cast<int*>(s.lseT + N);
-  s.ttok = reinterpret_cast<int*>(sm + o.toks); s.dtok = s.ttok + N * K; s.tlog = reinterpret_cast<float*>(s.dtok + N * K); s.dlog = s.tlog + N * K;
-  s.ckey = reinterpret_cast<double*>(sm + o.cand); s.clogS = s.ckey + N * K; s.res = reinterpret_cast<float*>(sm + o.cand);
-  s.valid = sm + o.flags; s.best = s.valid + N * K;
-  s.hist = reinterpret_cast<int*>(sm + o.lists); s.newl = s.hist + 256; s.tcnt = s.newl + 256; s.toff = s.tcnt + 256; s.npl = s.toff + 256;
-  s.Wc = reinterpret_cast<uint32_t*>(sm + o.seeds);
-  s.stok = reinterpret_cast<int*>(s.Wc + (size_t)seed_count(K) * (a.r + 1)); s.sval = reinterpret_cast<float*>(s.stok + 32);
+  s.pv = pool_view(sm + a.own.pool, N);
+  s.lse0 = reinterpret_cast<float*>(sm + a.own.lse); s.lseT = s.lse0 + N; s.pslot = reinterpret_cast<int*>(s.lseT + N);
+  s.ttok = reinterpret_cast<int*>(sm + a.own.toks); s.dtok = s.ttok + NK; s.tlog = reinterpret_cast<float*>(s.dtok + NK); s.dlog = s.tlog + NK;
+  s.ckey = reinterpret_cast<double*>(sm + a.own.cand); s.clogS = s.ckey + NK; s.res = reinterpret_cast<float*>(sm + a.own.cand);
+  s.valid = sm + a.own.flags; s.best = s.valid + NK;
+  s.hist = reinterpret_cast<int*>(sm + a.own.lists); s.newl = s.hist + 256; s.tcnt = s.newl + 256; s.toff = s.tcnt + 256; s.npl = s.toff + 256;
+  s.Wc = reinterpret_cast<uint32_t*>(sm + a.own.seeds);
+  s.stok = reinterpret_cast<int*>(s.Wc + (size_t)seed_count(a.K) * (a.r + 1)); s.sval = reinterpret_cast<float*>(s.stok + 32);
   return s;
 }
 
@@ -856,13 +855,6 @@ __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s
   }
 }
 
-__device__ __forceinline__ void tx_caps(const TreeArgs& a, int b, int& K_eff, int& N_eff, double& log_theta) {
-  const float th = a.theta[b];
-  K_eff = a.K < a.V ? a.K : a.V; N_eff = a.N;
-  if (th >= 1.f) { K_eff = 1; N_eff = a.D < a.N ? a.D : a.N; log_theta = -INFINITY; }   // chain member of the price ladder
-  else log_theta = th > 0.f ? log((double)th) : -INFINITY;
-}
-
 // One level of one request: merge of its parents, slots and cut of Algorithm 1, the next level's parents.
 // d = depth of the parents just scanned; d = -1: the start of request b (an empty pool and the root as the only parent of
 // level 0) or, for ts_score_parents, the list entry of given parent b.
@@ -871,7 +863,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
   const OwnerSm s = owner_carve(sm, a);
   __shared__ int sh[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int N = a.N, K = a.K, cur = d & 1, nxt = cur ^ 1, NS = seed_count(K);
+  const int N = a.N, K = a.K, lk = slot_log2(K), cur = d & 1, nxt = cur ^ 1, NS = seed_count(K);
   int* ptok = s.ttok; uint64_t* phash = reinterpret_cast<uint64_t*>(s.tlog);   // the new parents (merged results are done with by then)
   int cnt = 1, li0 = b, req = b, row = b * a.D + d + 1;
   bool more = true;
@@ -895,6 +887,8 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
         ptok[0] = ok ? t : 0; phash[0] = 0ull;
         a.req_npar[b] = 1; a.req_base[b] = b; a.req_nscored[b] = 0;
         a.root_lseT[b] = nanf("");
+        const float th = a.theta[b];   // (>= 1: the chain member of the price ladder)
+        a.req_caps[b] = make_double2(th >= 1.f || !(th > 0.f) ? -INFINITY : log((double)th), th >= 1.f ? 1.0 : 0.0);
       }
       s.npl[0] = -1;
     }
@@ -904,7 +898,8 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       if (tid == 0) a.req_npar[nxt * a.B + b] = 0;
       return;
     }
-    tx_caps(a, b, K_eff, N_eff, log_theta);
+    const double2 caps = __ldcg(a.req_caps + b);   // log theta (-inf on the chain member), 1 on the chain member
+    log_theta = caps.x; K_eff = caps.y != 0.0 ? 1 : min(K, a.V); N_eff = caps.y != 0.0 ? min(a.D, N) : N;
     more = d + 1 < a.D;
     uint4* dst = reinterpret_cast<uint4*>(s.pv.key); const uint4* src = reinterpret_cast<const uint4*>(gpool);
 #pragma unroll 1
@@ -918,10 +913,11 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
   if (warp == TX_WARPS - 1) {
     if (more) pick_seeds(a.npiece, a.utop + ((size_t)nxt * a.B + b) * a.npiece, NS, s.stok, s.sval, lane);
   } else if (d >= 0) {
-    const int P = __ldcg(a.lvl_count + d), R = mma_replicas(P), kinds = a.T > 0.f ? 3 : 2;
+    const int P = __ldcg(a.lvl_count + d), R = mma_replicas(P);
 #pragma unroll 1
-    for (int task = warp; task < npar * kinds; task += TX_WARPS - 1) {
-      const int i = task / kinds, kind = task % kinds, p = base + i;
+    for (int task = warp; task < npar * 3; task += TX_WARPS - 1) {
+      const int i = task / 3, kind = task - 3 * i, p = base + i;
+      if (kind == 2 && !(a.T > 0.f)) continue;
       if (kind == 0) {
         const float2 l = warp_lse(a.sums + (size_t)p * a.ntiles, a.ntiles, a.T, lane);
         if (lane == 0) { s.lse0[i] = l.x; s.lseT[i] = l.y; }
@@ -929,8 +925,8 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
         const size_t cb = (size_t)p * a.ntiles * (R * K);
         const float3 w = warp_topk(kind == 1 ? a.cand_top + cb : a.cand_key + cb, kind == 1 ? nullptr : a.cand_lg + cb, a.cand_cnt + (kind == 1 ? 0 : a.cap) + p, K, lane);
         if (lane < K) {
-          if (kind == 1) { s.ttok[i * K + lane] = __float_as_int(w.x); s.tlog[i * K + lane] = w.y; }
-          if (kind == 2 || kinds == 2) { s.dtok[i * K + lane] = __float_as_int(w.x); s.dlog[i * K + lane] = w.z; }
+          if (kind == 1) { s.ttok[(i << lk) + lane] = __float_as_int(w.x); s.tlog[(i << lk) + lane] = w.y; }
+          if (kind == 2 || !(a.T > 0.f)) { s.dtok[(i << lk) + lane] = __float_as_int(w.x); s.dlog[(i << lk) + lane] = w.z; }
         }
       }
     }
@@ -945,22 +941,22 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     unsigned used = 0u;
     if (!(a.T > 0.f)) used = lane < K ? 1u << lane : 0u;
     else if (lane < K) {
-      const int x = s.dtok[i * K + lane];
+      const int x = s.dtok[(i << lk) + lane];
 #pragma unroll 4
-      for (int t = 0; t < K; ++t) if (x >= 0 && s.ttok[i * K + t] == x) used |= 1u << t;
+      for (int t = 0; t < K; ++t) if (x >= 0 && s.ttok[(i << lk) + t] == x) used |= 1u << t;
     }
 #pragma unroll
     for (int o = 1; o < 16; o <<= 1) { const unsigned u = __shfl_up_sync(0xFFFFFFFFu, used, o); if (lane >= o) used |= u; }
     const unsigned prior = __shfl_up_sync(0xFFFFFFFFu, used, 1);
-    if (lane < K) { const unsigned fr = ~(lane ? prior : 0u) & ((1u << K_eff) - 1u); s.best[i * K + lane] = fr ? (unsigned char)(__ffs(fr) - 1) : 255u; }
+    if (lane < K) { const unsigned fr = ~(lane ? prior : 0u) & ((1u << K_eff) - 1u); s.best[(i << lk) + lane] = fr ? (unsigned char)(__ffs(fr) - 1) : 255u; }
   }
   __syncthreads();
   if (more) store_seed_columns(a, s, NS, 0, wcol);
   // ---- slots of every scored parent: two threads per (parent, sibling rank), one for the key (the best unused token's
   // estimate), one for the survival of the token drawn ----
 #pragma unroll 1
-  for (int t2 = tid; t2 < 2 * npar * K; t2 += TX_THREADS) {
-    const int t = t2 >> 1, which = t2 & 1, i = t / K, j = t % K;
+  for (int t2 = tid; t2 < 2 * npar << lk; t2 += TX_THREADS) {
+    const int t = t2 >> 1, which = t2 & 1, i = t >> lk, j = t & ((1 << lk) - 1);
     const double lse0 = s.lse0[i], lseT = s.lseT[i];
     const int slot = s.pslot[i];
     const bool bad = !(lse0 == lse0) || isinf(lse0);
@@ -971,12 +967,12 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     int ok = 0;
     if (j < K_eff && !bad) {
       const int bi = s.best[t], x = s.dtok[t];
-      if (bi < K_eff && s.ttok[i * K + bi] >= 0 && x >= 0) {
+      if (bi < K_eff && s.ttok[(i << lk) + bi] >= 0 && x >= 0) {
         const double logS_v = slot < 0 ? 0.0 : s.pv.logS[slot];
         // the calibrator's input: the untempered conditional, or (ablation) the tempered one
         const bool tempered = a.calib_qT && a.T > 0.f;
         const double lsc = tempered ? 1.0 / (double)a.T : 1.0, lsn = tempered ? lseT : lse0;
-        const double v = logS_v + log_phat(a.calib, d, (double)(which ? s.dlog[t] : s.tlog[i * K + bi]) * lsc, lsn);
+        const double v = logS_v + log_phat(a.calib, d, (double)(which ? s.dlog[t] : s.tlog[(i << lk) + bi]) * lsc, lsn);
         if (which) s.clogS[t] = v;
         else { s.ckey[t] = v; ok = !(v < log_theta); }
       }
@@ -991,7 +987,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     for (int i = tid; i < npar; i += TX_THREADS) {
       bool open = true;
 #pragma unroll 1
-      for (int j = 0; j < K; ++j) { if (!s.valid[i * K + j]) open = false; if (open) ++nv; else s.valid[i * K + j] = 0; }
+      for (int j = 0; j < K; ++j) { if (!s.valid[(i << lk) + j]) open = false; if (open) ++nv; else s.valid[(i << lk) + j] = 0; }
     }
 #pragma unroll 1
     for (int i = tid; i < N; i += TX_THREADS) np += s.pv.meta[i] >> 16;
@@ -999,7 +995,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     if (lane == 0) { if (np) atomicAdd(&sh[0], np); if (nv) atomicAdd(&sh[1], nv); }
   }
   __syncthreads();
-  const int ncand = npar * K, shift = 60 - 4 * d;
+  const int ncand = npar << lk, shift = 60 - 4 * d;
   auto skey = [](double k) -> uint64_t {
     if (k == 0.0) k = 0.0;   // -0 and +0 compare equal: one pattern
     const uint64_t u = (uint64_t)__double_as_longlong(k);
@@ -1012,8 +1008,8 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
   auto depth_of = [&](int e) -> int { return e < N ? (s.pv.meta[e] >> 8) & 255 : d + 1; };
   auto path_of = [&](int e) -> uint64_t {
     if (e < N) return s.pv.path[e];
-    const int c = e - N, slot = s.pslot[c / K];
-    return (slot < 0 ? 0ull : s.pv.path[slot]) | ((uint64_t)(c % K) << shift);
+    const int c = e - N, slot = s.pslot[c >> lk];
+    return (slot < 0 ? 0ull : s.pv.path[slot]) | ((uint64_t)(c & ((1 << lk) - 1)) << shift);
   };
   if (sh[0] + sh[1] > N_eff) {
     // The N_eff-th largest key by radix selection over the keys' order-preserving bit patterns (eight bits a pass);
@@ -1132,7 +1128,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       if (!v) continue;
       const int c = it * TX_THREADS + tid, t = s.toff[it * TX_WARPS + warp] + __popc(vb & ((1u << lane) - 1u));
       if (t >= nfree) continue;
-      const int sl = s.hist[t], i = c / K, j = c % K, slot = s.pslot[i], x = s.dtok[c];
+      const int sl = s.hist[t], i = c >> lk, j = c & ((1 << lk) - 1), slot = s.pslot[i], x = s.dtok[c];
       const double lx = s.dlog[c], lse0 = s.lse0[i], lseT = s.lseT[i];
       s.pv.meta[sl] = (1 << 16) | ((d + 1) << 8) | j; s.pv.parent[sl] = slot; s.pv.tok[sl] = x;
       s.pv.key[sl] = s.ckey[c]; s.pv.logS[sl] = s.clogS[c];
@@ -1351,7 +1347,6 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
         __syncthreads();
       }
     }
-    __threadfence();
     if (dead) { if (tid == 0) atomicExch(a.barrier + 1, 1u); break; }
     if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
     if (a.score_P > 0) {
@@ -1389,7 +1384,6 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
     }
     if (d + 1 >= a.D && a.score_P == 0) break;
     fence_async_smem();   // owners work in memory that the next scan's bulk loads may write
-    __threadfence();
     if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
     if (d == -2 && a.ragged) asm volatile("fence.proxy.async;" ::: "memory");
   }
@@ -1474,7 +1468,7 @@ bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
 }
 
 // Workspace of one call over `nreq` requests (or given parents) whose lists hold up to `cap` parents.
-struct TreeWs { size_t head, ent[2], slot[2], sums, cnt, top, key, lg, thr, utop, pool, state, upad, wpad, total; int cap; };
+struct TreeWs { size_t head, ent[2], slot[2], sums, cnt, top, key, lg, thr, utop, pool, state, caps, upad, wpad, total; int cap; };
 static TreeWs tree_ws(const ts_ctx* ctx, int nreq, int cap, bool expand, int rows) {
   const ts_config& c = ctx->cfg; const TreePlan& p = ctx->tree;
   TreeWs w{}; size_t at = 0;
@@ -1488,7 +1482,7 @@ static TreeWs tree_ws(const ts_ctx* ctx, int nreq, int cap, bool expand, int row
   w.top = take(cands * 8); w.key = take(cands * 8); w.lg = take(cands * 4);
   w.thr = take(2 * C * 4 + 2 * C * c.K * SLOT_STRIDE * 4);
   w.utop = take((size_t)nreq * (expand ? 2 : 1) * p.npiece * 8);
-  if (expand) { w.pool = take((size_t)nreq * pool_bytes(c.Nmax)); w.state = take((size_t)nreq * 5 * 4); }
+  if (expand) { w.pool = take((size_t)nreq * pool_bytes(c.Nmax)); w.state = take((size_t)nreq * 5 * 4); w.caps = take((size_t)nreq * 16); }
   if (c.V % 8) { w.upad = take((size_t)rows * p.Vs * 2); w.wpad = take((size_t)c.r * p.Vs * 2); }
   w.total = at;
   return w;
@@ -1507,6 +1501,7 @@ size_t tree_score_bytes(const ts_ctx* ctx, int P) { return ctx->cfg.V % 8 ? 0 : 
 static void fill_args(ts_ctx* ctx, TreeArgs& a, char* base, const TreeWs& w, bool expand, const void* U, const void* A, const void* W, float T, uint64_t seed) {
   const ts_config& c = ctx->cfg; const TreePlan& p = ctx->tree;
   a.U = U; a.A = A; a.W = W; a.V = c.V; a.D = c.D; a.r = c.r; a.K = c.K; a.N = c.Nmax; a.T = T; a.seed = seed;
+  a.own = owner_layout(c.Nmax, c.K, c.r);
   a.ragged = c.V % 8 ? 1 : 0;
   a.Vs = p.Vs; a.Uscan = a.ragged ? base + w.upad : U; a.Wscan = a.ragged ? base + w.wpad : W;
   a.TV = p.TV; a.ntiles = p.ntiles; a.BN = p.BN; a.nW = p.nW; a.nU = p.nU; a.npiece = p.npiece; a.w_over = p.w_over;
@@ -1570,6 +1565,7 @@ cudaError_t tree_expand(ts_ctx* ctx, char* ws, const TreeOut& o, const void* U, 
   a.pool = (unsigned char*)ws + w.pool; a.pool_stride = pool_bytes(c.Nmax);
   int* state = (int*)(ws + w.state);
   a.req_npar = state; a.req_base = state + 2 * (size_t)B; a.req_nscored = state + 3 * (size_t)B; a.root_lseT = (float*)(state + 4 * (size_t)B);
+  a.req_caps = (double2*)(ws + w.caps);
   a.n_nodes = o.n_nodes; a.tok = o.tok; a.parent = o.parent; a.depth = o.depth; a.sib_rank = o.sib_rank; a.logS = o.logS; a.q0 = o.q0; a.logqT = o.logqT;
   a.logkey = o.logkey; a.pop_rank = o.pop_rank; a.node_hash = o.node_hash; a.node_lseT = o.node_lseT; a.mask = o.mask; a.n_scored = o.n_scored; a.status = o.status;
   a.words = (c.Nmax + 63) / 64;

@@ -31,7 +31,10 @@ struct __align__(16) ParentEntry {
 };
 static_assert(sizeof(ParentEntry) == 32, "two 16-byte loads");
 
+struct OwnerLayout { uint32_t pool, lse, toks, cand, flags, lists, seeds, total; };
+
 struct TreeArgs {
+  OwnerLayout own;
   const void *U, *A, *W;
   const void *Uscan, *Wscan;   // base logits and W as the scan reads them (a ragged vocabulary: copies with padded rows)
   int V, Vs;             // vocabulary; row stride of Uscan and Wscan
@@ -51,7 +54,7 @@ struct TreeArgs {
   unsigned *thr, *slots; int cap;
   uint2* utop;                                     // [2][B][npiece] (given parents: [P][npiece]): best base logit of every piece of a row
   unsigned char* pool; size_t pool_stride;         // per request: PoolView
-  int *req_npar, *req_base, *req_nscored; float* root_lseT;
+  int *req_npar, *req_base, *req_nscored; float* root_lseT; double2* req_caps;
   // expansion inputs and outputs
   const int* anchor; const float* theta; DevCalib calib; int calib_qT;
   int *n_nodes, *tok, *parent, *depth, *sib_rank; float *logS, *q0, *logqT, *logkey; int* pop_rank;
@@ -76,8 +79,10 @@ __device__ __forceinline__ PoolView pool_view(unsigned char* p, int N) {
   return v;
 }
 
+// Rows of a parent's K candidates are padded to a power of two (no divisions on the owner's chain of instructions).
+__host__ __device__ inline int slot_log2(int K) { return K <= 8 ? 3 : 4; }
+
 // Bytes of shared memory the owner of a request works in (pool, merged results, candidates, seed columns).
-struct OwnerLayout { uint32_t pool, lse, toks, cand, flags, lists, seeds, total; };
 // tokens evaluated for a parent's seed bounds: at least 2K (K <= 16), a power of two
 __host__ __device__ inline int seed_log2(int K) { return K <= 4 ? 3 : (K <= 8 ? 4 : 5); }
 __host__ __device__ inline int seed_count(int K) { return 1 << seed_log2(K); }
@@ -86,10 +91,11 @@ __host__ __device__ inline OwnerLayout owner_layout(int N, int K, int r) {
   auto take = [&](size_t bytes) { uint32_t x = at; at = (uint32_t)((at + bytes + 15) & ~(size_t)15); return x; };
   o.pool = take(pool_bytes(N));
   o.lse = take((size_t)N * 3 * 4);              // lse0, lseT, pool slot of every parent
-  o.toks = take((size_t)N * K * 4 * 4);         // top tokens, top logits, draw tokens, draw logits
-  const size_t cand = (size_t)N * K * 16, res = (size_t)N * seed_count(K) * 8;
+  const size_t KP = (size_t)1 << slot_log2(K);
+  o.toks = take((size_t)N * KP * 4 * 4);        // top tokens, draw tokens, top logits, draw logits
+  const size_t cand = (size_t)N * KP * 16, res = (size_t)N * seed_count(K) * 8;
   o.cand = take(cand > res ? cand : res);       // key, logS of every slot; later the seed values of the new parents
-  o.flags = take((size_t)N * K * 2);            // valid, index of the best unused token
+  o.flags = take((size_t)N * KP * 2);           // valid, index of the best unused token
   o.lists = take(256 * 4 * 5);                  // histogram / free slots, new slots, trip counts and offsets, new parents
   o.seeds = take((size_t)seed_count(K) * (r + 1) * 4 + 32 * 8);   // words of W holding the seed tokens' columns; tokens and base logits
   o.total = at;
