@@ -59,10 +59,10 @@ struct TileCfg {
 struct TreePlan {
   int TV, ntiles;        // tokens per CTA (a multiple of 64), CTAs with tokens
   int Vs;                // row stride of W and the base logits as the scan reads them (V rounded up to 8)
-  int BN, nU, nW;        // tokens per block, stages of the base-logit and W rings
+  int BN, nW;            // tokens per block, stages of the W ring
   int npiece;            // pieces of a base-logit row whose best tokens become seed candidates
   int w_over;            // owners work in the W ring too
-  uint32_t oU, oL, oW, oX;   // shared-memory offsets (bytes)
+  uint32_t oL, oW, oX;   // shared-memory offsets (bytes)
   size_t smem;
 };
 

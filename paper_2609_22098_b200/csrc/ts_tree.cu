@@ -29,11 +29,6 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool in) 
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-// arrives on `bar` when this thread's earlier cp.async have landed (the barrier counts every thread that says so)
-__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
 // one lane of a converged warp (the instruction tells the compiler that the branch is uniform)
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
@@ -43,7 +38,7 @@ __device__ __forceinline__ bool elect_one() {
 
 // Shared-memory state of a CTA.
 struct TxSm {
-  unsigned char *As, *Us, *Ws;
+  unsigned char *As, *Ws;
   uint4* q;                    // [TX_QCAP] queued candidates: token, logit, row | split << 8 | kind << 12 | c16 << 16, tag
   float* lists;                // [128][5K]: topv, topi, keyv, keyi, keyl of every row, sorted (value desc, token asc)
   int* ln;                     // [2][128] entries in use
@@ -53,7 +48,7 @@ struct TxSm {
   float* ghi;                  // [512] noise bounds
   volatile float* thr;         // [2][128] launch-wide bounds of the rows' parents
   ParentEntry* ent;            // [128] the group's parents by tile row
-  uint64_t *a_full, *t_full, *t_empty, *u_full, *w_full, *w_free;
+  uint64_t *a_full, *t_full, *t_empty, *w_full, *w_free;
   uint32_t* tmem;
   volatile int *abort, *done;
   volatile unsigned* q_head; unsigned* q_tail;
@@ -62,11 +57,11 @@ struct TxSm {
 constexpr size_t tx_select_bytes(int K) {
   return (size_t)TX_QCAP * 16 + (size_t)TX_ROWS * 5 * K * 4 + 2 * TX_ROWS * 4 + 2 * TX_ROWS * 4 + 2 * TX_SPLIT * TX_ROWS * 4 + 3 * TX_SPLIT * TX_ROWS * 4;
 }
-constexpr size_t TX_FIXED_BYTES = 512 * 4 + 2 * TX_ROWS * 4 + TX_ROWS * sizeof(ParentEntry) + (1 + 5 * TX_STAGE_MAX) * 8 + 64;
+constexpr size_t TX_FIXED_BYTES = 512 * 4 + 2 * TX_ROWS * 4 + TX_ROWS * sizeof(ParentEntry) + (1 + 4 * TX_STAGE_MAX) * 8 + 64;
 
 __device__ __forceinline__ TxSm tx_carve(unsigned char* sm, const TreeArgs& a) {
   TxSm s;
-  s.As = sm; s.Us = sm + a.oU; s.Ws = sm + a.oW;
+  s.As = sm; s.Ws = sm + a.oW;
   s.q = reinterpret_cast<uint4*>(sm + a.oL);
   s.lists = reinterpret_cast<float*>(s.q + TX_QCAP);
   s.ln = reinterpret_cast<int*>(s.lists + (size_t)TX_ROWS * 5 * a.K);
@@ -77,8 +72,7 @@ __device__ __forceinline__ TxSm tx_carve(unsigned char* sm, const TreeArgs& a) {
   s.ghi = reinterpret_cast<float*>(s.ent + TX_ROWS);
   s.thr = s.ghi + 512;
   uint64_t* bars = reinterpret_cast<uint64_t*>(const_cast<float*>(s.thr) + 2 * TX_ROWS);
-  s.a_full = bars; s.t_full = bars + 1; s.t_empty = s.t_full + TX_STAGE_MAX; s.u_full = s.t_empty + TX_STAGE_MAX;
-  s.w_full = s.u_full + TX_STAGE_MAX; s.w_free = s.w_full + TX_STAGE_MAX;
+  s.a_full = bars; s.t_full = bars + 1; s.t_empty = s.t_full + TX_STAGE_MAX; s.w_full = s.t_empty + TX_STAGE_MAX; s.w_free = s.w_full + TX_STAGE_MAX;
   s.tmem = reinterpret_cast<uint32_t*>(s.w_free + TX_STAGE_MAX);
   s.abort = reinterpret_cast<volatile int*>(s.tmem + 1);
   s.done = reinterpret_cast<volatile int*>(s.tmem + 2);
@@ -115,29 +109,25 @@ __device__ __forceinline__ float exact_key(uint64_t seed, int req, uint64_t hash
 // counter only the index changes from call to call, and it reaches the other lane pair one round later, so one of the
 // two products of the first round and one of the second are constants of the parent.
 struct CoarseGen {
-  uint32_t x0, y2, y3, k0, k1, c3;
-  __device__ __forceinline__ void init(uint64_t seed, int req, uint64_t hash) {
-    k0 = (uint32_t)seed; k1 = (uint32_t)(seed >> 32);
-    c3 = (((uint32_t)req & 0xFFFFFFu) | ((uint32_t)STREAM_GUMBEL_COARSE << 24)) ^ k1;
+  uint32_t x0, y2, y3, c3;
+  __device__ __forceinline__ void init(const uint32_t* rk, int req, uint64_t hash) {
+    c3 = (((uint32_t)req & 0xFFFFFFu) | ((uint32_t)STREAM_GUMBEL_COARSE << 24)) ^ rk[1];
     const uint32_t c1 = (uint32_t)hash, c2 = (uint32_t)(hash >> 32);
-    const uint32_t n0 = __umulhi(0xCD9E8D57u, c2) ^ c1 ^ k0;   // round 1, word 0
-    y2 = __umulhi(0xD2511F53u, n0) ^ (k1 + 0xBB67AE85u);        // round 2, word 2 = y2 ^ (word 3 of round 1)
-    y3 = 0xD2511F53u * n0;                                      // round 2, word 3
-    x0 = (0xCD9E8D57u * c2) ^ (k0 + 0x9E3779B9u);                               // round 2, word 0 = hi(M1 * word 2 of round 1) ^ x0
+    const uint32_t n0 = __umulhi(0xCD9E8D57u, c2) ^ c1 ^ rk[0];   // round 1, word 0
+    y2 = __umulhi(0xD2511F53u, n0) ^ rk[3];                        // round 2, word 2 = y2 ^ (word 3 of round 1)
+    y3 = 0xD2511F53u * n0;                                         // round 2, word 3
+    x0 = (0xCD9E8D57u * c2) ^ rk[2];                               // round 2, word 0 = hi(M1 * word 2 of round 1) ^ x0
   }
-  __device__ __forceinline__ uint4 words(uint32_t index) const {
-    // round 1: words 2 and 3
+  // rk: the twenty round keys (kernel parameters: an exclusive-or takes one as its constant operand)
+  __device__ __forceinline__ uint4 words(const uint32_t* rk, uint32_t index) const {
     const uint64_t pi = mul_wide(0xD2511F53u, index);
     const uint32_t a2 = (uint32_t)(pi >> 32) ^ c3, a3 = (uint32_t)pi;
-    // round 2
     const uint64_t pa = mul_wide(0xCD9E8D57u, a2);
     uint32_t c0 = (uint32_t)(pa >> 32) ^ x0, c1 = (uint32_t)pa, c2 = y2 ^ a3, cc3 = y3;
-    uint32_t q0 = k0 + 2u * 0x9E3779B9u, q1 = k1 + 2u * 0xBB67AE85u;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 2; i < 10; ++i) {
       const uint64_t p0 = mul_wide(0xD2511F53u, c0), p1 = mul_wide(0xCD9E8D57u, c2);
-      c0 = (uint32_t)(p1 >> 32) ^ c1 ^ q0; c1 = (uint32_t)p1; c2 = (uint32_t)(p0 >> 32) ^ cc3 ^ q1; cc3 = (uint32_t)p0;
-      q0 += 0x9E3779B9u; q1 += 0xBB67AE85u;
+      c0 = (uint32_t)(p1 >> 32) ^ c1 ^ rk[2 * i]; c1 = (uint32_t)p1; c2 = (uint32_t)(p0 >> 32) ^ cc3 ^ rk[2 * i + 1]; cc3 = (uint32_t)p0;
     }
     return make_uint4(c0, c1, c2, cc3);
   }
@@ -211,7 +201,7 @@ __device__ __forceinline__ bool tx_wait_warp(uint64_t* bar, uint32_t parity, con
 // parent; a warp owns every (4R)-th chunk of 16 tokens, so with few parents (R = 2, 4 replicas of the rows) the
 // copies share the range.
 __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int t0, const int tlen,
-                                        const uint32_t tmem_base, BlockPos& pos, const int nst, const int urows) {
+                                        const uint32_t tmem_base, BlockPos& pos, const int nst) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int q = warp & 3, s = warp >> 2, row = q * 32 + lane;
   const int per = TX_ROWS / R, K = a.K;
@@ -235,28 +225,36 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
   const float T = a.T, invT = T > 0.f ? 1.f / T : 1.f;
   const bool keys = T > 0.f, two = keys && T != 1.f;
   const float slack = 8.f * fminf(1.f, T > 0.f ? T : 1.f);   // how far a logit may exceed the sums' reference
-  CoarseGen gen; gen.init(a.seed, me.req, me.hash);
+  CoarseGen gen; gen.init(a.rk, me.req, me.hash);
   float m = me.mref, s0 = 0.f, sT = 0.f;
   const uint32_t ztag = (uint32_t)row | ((uint32_t)s << 8);
   const int CB = a.BN / 16, nblk = (tlen + a.BN - 1) / a.BN, stride = R * TX_SPLIT, own = rho * TX_SPLIT + s;
   const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16);
+  // Base logits: 32 bytes of its parent's row per lane and chunk, straight from L2 (a scan reads each once; lanes whose
+  // parents share a row read the same sector).  Through shared memory they needed a copying warp that could not keep up with
+  // 128 different rows: 3 us per block of 128 tokens by 16-byte cp.async, 6 us by one bulk copy per row.
+  const __nv_bfloat16* urow = reinterpret_cast<const __nv_bfloat16*>(a.Uscan) + (size_t)max(me.row, 0) * a.Vs + t0;
+  const int vleft = a.Vs - t0;   // tokens of the row from t0 on (whole 16 bytes)
+  int o = own * 16;              // the next chunk to request
+  uint4 nx0 = make_uint4(0u, 0u, 0u, 0u), nx1 = nx0;
+  if (o < tlen) { nx0 = __ldcg(reinterpret_cast<const uint4*>(urow + o)); if (o + 8 < vleft) nx1 = __ldcg(reinterpret_cast<const uint4*>(urow + o + 8)); }
   bool alive = true;
   for (int nb = 0; nb < nblk; ++nb, pos.next(nst)) {
     const int slot = pos.slot;
-    if (!tx_wait_warp(sm.t_full + slot, pos.full(), sm, a) || !tx_wait_warp(sm.u_full + slot, pos.full(), sm, a)) { alive = false; break; }
+    if (!tx_wait_warp(sm.t_full + slot, pos.full(), sm, a)) { alive = false; break; }
     tc_fence_after();
     const int nch = min(CB, (tlen - nb * a.BN + 15) / 16);
-    const unsigned char* urow = sm.Us + (size_t)(slot * urows + prow) * 2 * a.BN;
     for (int c = (own - nb * CB) & (stride - 1); c < nch; c += stride) {
       uint32_t ra[16];
       __syncwarp();   // (the tensor-memory load is a warp-wide instruction)
       tmem_ld16_issue(trow + (uint32_t)(slot * a.BN + c * 16), ra);
-      const uint4 u0 = *reinterpret_cast<const uint4*>(urow + (((2 * c) ^ (prow & 7)) << 4));
-      const uint4 u1 = *reinterpret_cast<const uint4*>(urow + (((2 * c + 1) ^ (prow & 7)) << 4));
+      const uint4 u0 = nx0, u1 = nx1;   // requested one owned chunk ago; the next one's are requested now
+      o += stride * 16;
+      if (o < tlen) { nx0 = __ldcg(reinterpret_cast<const uint4*>(urow + o)); if (o + 8 < vleft) nx1 = __ldcg(reinterpret_cast<const uint4*>(urow + o + 8)); }
       const int v0 = t0 + nb * a.BN + c * 16, valid = min(16, a.V - v0);
       // high halves of the sixteen uniforms: issued first, their long dependent chains overlap the rest
       uint4 cw0 = make_uint4(0, 0, 0, 0), cw1 = cw0;
-      if (keys) { cw0 = gen.words((uint32_t)v0 >> 3); cw1 = gen.words(((uint32_t)v0 >> 3) + 1u); }
+      if (keys) { cw0 = gen.words(a.rk, (uint32_t)v0 >> 3); cw1 = gen.words(a.rk, ((uint32_t)v0 >> 3) + 1u); }
       tmem_ld_wait();
       if (!active) continue;
       float acc[16];
@@ -354,48 +352,6 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
   if (lane == 0) atomicAdd((int*)sm.done, alive ? 1 : (1 << 20));   // one tick per warp per group (a large one releases the others after a failed wait)
 }
 
-// ---- the copying warp: base-logit rows of every block into the ring (and W, where no tensor map could be made) ----
-__device__ __forceinline__ void tx_copy(const TreeArgs& a, const TxSm& sm, const int nrow, const int t0, const int tlen, BlockPos& pos, BlockPos& wpos, const int nst, const int urows) {
-  const int lane = threadIdx.x & 31;
-  const int CB8 = a.BN / 8, nblk = (tlen + a.BN - 1) / a.BN;
-  const int sh = a.BN == 128 ? 4 : 3;             // log2 of the 16-byte chunks per row and block
-  const int ck = lane & (CB8 - 1), r0 = lane >> sh, rstep = 32 >> sh;
-  const __nv_bfloat16* Ug = reinterpret_cast<const __nv_bfloat16*>(a.Uscan);
-  for (int nb = 0; nb < nblk; ++nb, pos.next(nst)) {
-    if (pos.reused() && !tx_wait_warp(sm.t_empty + pos.slot, pos.empty(), sm, a)) return;
-    const int v = t0 + nb * a.BN + ck * 8;
-    const bool in = v < a.Vs;
-    const __nv_bfloat16* src = in ? Ug + v : Ug;
-    unsigned char* dst = sm.Us + (size_t)(pos.slot * urows) * 2 * a.BN;
-    // (the row indices of eight copies are read together: one at a time the loop is a chain of shared-memory reads)
-    for (int rr = r0; rr < nrow; rr += 8 * rstep) {
-      int row[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) row[u] = sm.ent[min(rr + u * rstep, nrow - 1)].row;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int x = rr + u * rstep;
-        if (x < nrow) cp_async16(dst + x * 2 * a.BN + ((ck ^ (x & 7)) << 4), src + (size_t)row[u] * a.Vs, in);
-      }
-    }
-    cp_async_arrive(sm.u_full + pos.slot);
-    if (!a.use_tma) {
-      const int rw = (a.r + 15) / 16 * 16;
-      const __nv_bfloat16* Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wscan);
-      if (wpos.reused() && !tx_wait_warp(sm.w_free + wpos.slot, wpos.empty(), sm, a)) return;
-      unsigned char* wd = sm.Ws + (size_t)wpos.slot * rw * 2 * a.BN;
-      for (int k = r0; k < rw; k += rstep) {
-        const bool win = in && k < a.r;
-        cp_async16(wd + (size_t)(ck >> 3) * rw * 128 + k * 128 + (((ck & 7) ^ (k & 7)) << 4), win ? Wg + (size_t)k * a.Vs + v : Wg, win);
-      }
-      cp_async_wait_all();
-      fence_async_smem();
-      mbar_arrive(sm.w_full + wpos.slot);
-      wpos.next(a.nW);
-    }
-  }
-}
-
 // ---- W blocks into their ring (by the refreshing warp) ----------------------------------------------------------------
 // `upto`: blocks of the whole launch that may be requested while this group runs.  Requests run on into the next scan (W
 // does not depend on which parents that will score) except where the owners work in the ring.  Not the issuing warp's
@@ -410,7 +366,19 @@ __device__ __forceinline__ void tx_load(const TreeArgs& a, const TxSm& sm, const
       if (BLOCKING) { if (!tx_wait_warp(sm.w_free + w.pos.slot, w.pos.empty(), sm, a)) return; }
       else if (!__all_sync(0xFFFFFFFFu, mbar_test_wait(sm.w_free + w.pos.slot, w.pos.empty()))) return;
     }
-    if (elect_one()) {
+    if (!a.use_tma) {   // no tensor map: 16-byte copies into the same swizzled places
+      const int CB8 = a.BN / 8, sh = a.BN == 128 ? 4 : 3, lane = threadIdx.x & 31;
+      const int ck = lane & (CB8 - 1), r0 = lane >> sh, rstep = 32 >> sh, v = t0 + w.nb * a.BN + ck * 8;
+      const __nv_bfloat16* Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wscan);
+      unsigned char* wd = sm.Ws + (size_t)(w.pos.slot * (a.BN / 64)) * slab;
+      for (int k = r0; k < rw; k += rstep) {
+        const bool in = v < a.Vs && k < a.r;
+        cp_async16(wd + (size_t)(ck >> 3) * slab + k * 128 + (((ck & 7) ^ (k & 7)) << 4), in ? Wg + (size_t)k * a.Vs + v : Wg, in);
+      }
+      cp_async_wait_all();
+      fence_async_smem();
+      mbar_arrive(sm.w_full + w.pos.slot);
+    } else if (elect_one()) {
       const int ns = min(a.BN / 64, (tlen - w.nb * a.BN + 63) / 64);
       mbar_expect_tx(sm.w_full + w.pos.slot, (uint32_t)ns * slab);
       unsigned char* dst = sm.Ws + (size_t)(w.pos.slot * (a.BN / 64)) * slab;
@@ -455,7 +423,7 @@ __device__ __forceinline__ void tx_refresh(const TreeArgs& a, const TxSm& sm, co
   const int p_own = p_lo + ((tile - p_lo % nt + nt) % nt);
   const int which = lane >> 4, j = lane & 15;
   for (uint32_t spin = 0; spin < a.wait_limit; ++spin) {
-    if (a.use_tma) tx_load<false>(a, sm, tm, t0, tlen, w, upto);
+    tx_load<false>(a, sm, tm, t0, tlen, w, upto);
     if (*sm.done >= done_target || *sm.abort) break;
     // (a pass is a memory round trip: steady at first, while the bounds rise, every eighth turn later, so that the end of
     // the scan is seldom waited for)
@@ -490,7 +458,7 @@ __device__ __forceinline__ void tx_refresh(const TreeArgs& a, const TxSm& sm, co
     }
   }
   __syncwarp();
-  if (a.use_tma && !*sm.abort) tx_load<true>(a, sm, tm, t0, tlen, w, upto);
+  if (!*sm.abort) tx_load<true>(a, sm, tm, t0, tlen, w, upto);
 }
 
 // ---- the selecting warp: drains the queue until the scan is over ----------------------------------------------------
@@ -539,7 +507,7 @@ __device__ __forceinline__ void tx_drain(const TreeArgs& a, const TxSm& sm, cons
 }
 
 // ---- end of a group: the range's sums and surviving candidates of every parent -------------------------------------
-__device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int tile) {
+__device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int tile, int* cnt) {
   const int tid = threadIdx.x, per = TX_ROWS / R, K = a.K;
   if (tid >= TX_ROWS) return;
   const int row = tid, prow = R > 1 ? row % per : row, p = R > 1 ? prow : g * TX_ROWS + row;
@@ -571,8 +539,8 @@ __device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, co
 #pragma unroll 1
   for (int n = sm.ln[TX_ROWS + row]; kk < n && L[2 * K + kk] >= gK;) ++kk;
   int at = 0, ak = 0;
-  if (kt) at = atomicAdd(a.cand_cnt + p, kt);
-  if (kk) ak = atomicAdd(a.cand_cnt + a.cap + p, kk);
+  if (kt) at = atomicAdd(cnt + p, kt);
+  if (kk) ak = atomicAdd(cnt + a.cap + p, kk);
 #pragma unroll 1
   for (int j = 0; j < kk; ++j) {
     a.cand_key[base + ak + j] = make_uint2(__float_as_uint(L[2 * K + j]), (unsigned)Li[3 * K + j]);
@@ -778,7 +746,7 @@ __device__ __forceinline__ void store_seed_columns(const TreeArgs& a, const Owne
 // Seed bounds and list entries of `cnt` parents of one row (all threads; the columns have landed).  Parent i: token
 // s.ttok[i], hash hs[i], pool slot s.npl[i]; its place in the level's list is li0 + i.
 __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s, const int cnt, const int li0, const int req, const int row, const int NS,
-                                             const int* ptok, const uint64_t* phash, ParentEntry* ent, int* ent_slot) {
+                                             const int* ptok, const uint64_t* phash, ParentEntry* ent, int* ent_slot, int* cnt_next) {
   const int tid = threadIdx.x, r = a.r, K = a.K, lg = seed_log2(K);
   const float invT = a.T > 0.f ? 1.f / a.T : 1.f;
   const __nv_bfloat16* Ag = reinterpret_cast<const __nv_bfloat16*>(a.A);
@@ -791,7 +759,7 @@ __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s
 #pragma unroll 1
   for (int e = tid; e < cnt * 2; e += TX_THREADS) {
     a.thr[(size_t)(e & 1) * a.cap + li0 + (e >> 1)] = 0u;
-    a.cand_cnt[(size_t)(e & 1) * a.cap + li0 + (e >> 1)] = 0;
+    cnt_next[(size_t)(e & 1) * a.cap + li0 + (e >> 1)] = 0;
   }
   // every (parent, seed token) pair exactly: eight lanes a pair, 16 bytes of the head row a lane and step
   const int sub = tid & 7;
@@ -923,7 +891,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
         if (lane == 0) { s.lse0[i] = l.x; s.lseT[i] = l.y; }
       } else {
         const size_t cb = (size_t)p * a.ntiles * (R * K);
-        const float3 w = warp_topk(kind == 1 ? a.cand_top + cb : a.cand_key + cb, kind == 1 ? nullptr : a.cand_lg + cb, a.cand_cnt + (kind == 1 ? 0 : a.cap) + p, K, lane);
+        const float3 w = warp_topk(kind == 1 ? a.cand_top + cb : a.cand_key + cb, kind == 1 ? nullptr : a.cand_lg + cb, a.cand_cnt[cur] + (kind == 1 ? 0 : a.cap) + p, K, lane);
         if (lane < K) {
           if (kind == 1) { s.ttok[(i << lk) + lane] = __float_as_int(w.x); s.tlog[(i << lk) + lane] = w.y; }
           if (kind == 2 || !(a.T > 0.f)) { s.dtok[(i << lk) + lane] = __float_as_int(w.x); s.dlog[(i << lk) + lane] = w.z; }
@@ -1171,7 +1139,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     for (int e0 = SEED_REGS * TX_THREADS; e0 < NS * a.r; e0 += SEED_REGS * TX_THREADS) { load_seed_columns(a, s, NS, e0, wcol); store_seed_columns(a, s, NS, e0, wcol); }
   __syncthreads();
   if (d >= 0) li0 = sh[6];
-  if (more && cnt > 0) make_parents(a, s, cnt, li0, req, row, NS, ptok, phash, a.ent[nxt], a.ent_slot[nxt]);
+  if (more && cnt > 0) make_parents(a, s, cnt, li0, req, row, NS, ptok, phash, a.ent[nxt], a.ent_slot[nxt], a.cand_cnt[nxt]);
   __syncthreads();
 }
 
@@ -1264,7 +1232,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
   if (tid == 0) {
     mbar_init(sm.a_full, TX_SCAN_WARPS * 32 + (a.lost_arrival ? 1 : 0));
     for (int i = 0; i < TX_STAGE_MAX; ++i) {
-      mbar_init(sm.t_full + i, 1); mbar_init(sm.t_empty + i, TX_SCAN_WARPS); mbar_init(sm.u_full + i, 32);
+      mbar_init(sm.t_full + i, 1); mbar_init(sm.t_empty + i, TX_SCAN_WARPS);
       mbar_init(sm.w_full + i, a.use_tma ? 1 : 32); mbar_init(sm.w_free + i, 1);
     }
     *sm.abort = 0; *sm.done = 0; *sm.q_head = 0u; *sm.q_tail = 0u;
@@ -1328,22 +1296,19 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
         if (g == 0) for (int i = tid; i < TX_QCAP; i += TX_THREADS) sm.q[i].w = 0u;   // (owners work in this memory: the queue's tags start clean)
         __syncthreads();
         const int done_target = (groups + 1) * TX_SCAN_WARPS;
-        // with at most 64 parents a base-logit slot is half as large and the accumulators allow four stages
-        const int urows = R > 1 ? per : TX_ROWS, nst = min(a.nU * R, 512 / a.BN < TX_STAGE_MAX ? 512 / a.BN : TX_STAGE_MAX);
-        pos.slot = 0;
-        if (warp < TX_SCAN_WARPS) tx_scan(a, sm, R, P, g, t0, tlen, tmem_base, pos, nst, urows);
+        const int nst = min(512 / a.BN, TX_STAGE_MAX);   // accumulator stages
+        if (warp < TX_SCAN_WARPS) tx_scan(a, sm, R, P, g, t0, tlen, tmem_base, pos, nst);
         else if (warp == TX_MMA) tx_issue(a, sm, tlen, tmem_base, pos, wpos, groups, nst);
         else if (warp == TX_REFRESH) {
           const uint32_t nblk = (uint32_t)((tlen + a.BN - 1) / a.BN);
           const uint32_t level_end = (uint32_t)(groups + ngroups - g) * nblk + ((a.w_over || a.score_P > 0) ? 0u : (uint32_t)a.nW);
           tx_refresh(a, sm, R, P, g, cta, done_target, &tmW, t0, tlen, wl, min((uint32_t)(groups + 1) * nblk + (uint32_t)a.nW, level_end));
-        } else if (warp == TX_SELECT) tx_drain(a, sm, R, g, cta, done_target);
-        else tx_copy(a, sm, R > 1 ? P : min(TX_ROWS, P - g * TX_ROWS), t0, tlen, pos, wpos, nst, urows);
+        } else tx_drain(a, sm, R, g, cta, done_target);
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
         if (*sm.abort) { dead = true; break; }
-        tx_publish(a, sm, R, P, g, cta);
+        tx_publish(a, sm, R, P, g, cta, a.cand_cnt[d & 1]);
         __syncthreads();
       }
     }
@@ -1356,9 +1321,9 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
         const size_t cb = (size_t)p * a.ntiles * (R * K);
         const float2 l = warp_lse(a.sums + (size_t)p * a.ntiles, a.ntiles, a.T, lane);
         if (lane == 0) { a.o_lse0[p] = l.x; a.o_lseT[p] = l.y; }
-        float3 w = warp_topk(a.cand_top + cb, nullptr, a.cand_cnt + p, K, lane);
+        float3 w = warp_topk(a.cand_top + cb, nullptr, a.cand_cnt[0] + p, K, lane);
         if (lane < K) { a.o_top_tok[(size_t)p * K + lane] = __float_as_int(w.x); a.o_top_logit[(size_t)p * K + lane] = w.y; }
-        if (a.T > 0.f) w = warp_topk(a.cand_key + cb, a.cand_lg + cb, a.cand_cnt + a.cap + p, K, lane);
+        if (a.T > 0.f) w = warp_topk(a.cand_key + cb, a.cand_lg + cb, a.cand_cnt[0] + a.cap + p, K, lane);
         if (lane < K) { a.o_draw_tok[(size_t)p * K + lane] = __float_as_int(w.x); a.o_draw_logit[(size_t)p * K + lane] = w.z; }
       }
       break;
@@ -1442,25 +1407,21 @@ bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
   int piece = ((c.V + 127) / 128 + 7) & ~7;
   piece = piece < 64 ? 64 : (piece > TX_PIECE ? TX_PIECE : piece);
   p.npiece = (c.V + piece - 1) / piece;
+  const size_t own = owner_layout(c.Nmax, c.K, c.r).total, sel = up(tx_select_bytes(c.K)), fix = up(TX_FIXED_BYTES), A = rp * 256;
   for (int BN = 128; BN >= 64; BN /= 2) {
-    const size_t u = (size_t)TX_ROWS * 2 * BN, w = rw * 2 * BN, sel = up(tx_select_bytes(c.K)), fix = up(TX_FIXED_BYTES), A = rp * 256;
-    int nU = 2, nW = 2;
-    auto total = [&](int nu, int nw) { return A + (size_t)nu * u + sel + fix + (size_t)nw * w; };
-    if (total(nU, nW) > avail) continue;
-    for (;;) {   // the base-logit ring first: its loads start late
-      if (nU < 3 && total(nU + 1, nW) <= avail) { ++nU; continue; }
-      if (nW < 4 && total(nU, nW + 1) <= avail) { ++nW; continue; }
-      if (nU < 512 / BN && total(nU + 1, nW) <= avail) { ++nU; continue; }   // (as many accumulators as tensor memory holds)
-      if (nW < TX_STAGE_MAX && total(nU, nW + 1) <= avail) { ++nW; continue; }
-      break;
-    }
-    p.BN = BN; p.nU = nU; p.nW = nW;
-    p.oU = (uint32_t)A; p.oL = (uint32_t)(A + (size_t)nU * u); p.oW = (uint32_t)(p.oL + sel); p.oX = (uint32_t)(p.oW + (size_t)nW * w);
-    // owners work in [A, U ring, selection state], and in the W ring too when that is not enough (the ring then does not run ahead)
-    const size_t own = owner_layout(c.Nmax, c.K, c.r).total;
-    if (own > p.oX) return false;
+    const size_t w = rw * 2 * BN;
+    int nW = 2;
+    auto total = [&](int nw) { return A + sel + fix + (size_t)nw * w; };
+    if (total(nW) > avail) continue;
+    while (nW < TX_STAGE_MAX && total(nW + 1) <= avail) ++nW;
+    p.BN = BN; p.nW = nW;
+    p.oL = (uint32_t)A; p.oW = (uint32_t)(p.oL + sel); p.oX = (uint32_t)(p.oW + (size_t)nW * w);
+    // owners work in [A, selection state] and, where that is not enough, in the W ring (which then does not run ahead);
+    // where not even that is, behind them
     p.w_over = own > p.oW ? 1 : 0;
-    p.smem = total(nU, nW) + 1024;
+    if (own > p.oX) p.oX = (uint32_t)up(own);
+    if (p.oX + fix > avail) continue;
+    p.smem = p.oX + fix + 1024;
     *out = p;
     return true;
   }
@@ -1478,7 +1439,7 @@ static TreeWs tree_ws(const ts_ctx* ctx, int nreq, int cap, bool expand, int row
   w.head = take(256);
   w.ent[0] = take(C * sizeof(ParentEntry));
   if (expand) { w.ent[1] = take(C * sizeof(ParentEntry)); w.slot[0] = take(C * 4); w.slot[1] = take(C * 4); }
-  w.sums = take(C * nt * 16); w.cnt = take(2 * C * 4);
+  w.sums = take(C * nt * 16); w.cnt = take((expand ? 4 : 2) * C * 4);
   w.top = take(cands * 8); w.key = take(cands * 8); w.lg = take(cands * 4);
   w.thr = take(2 * C * 4 + 2 * C * c.K * SLOT_STRIDE * 4);
   w.utop = take((size_t)nreq * (expand ? 2 : 1) * p.npiece * 8);
@@ -1504,13 +1465,14 @@ static void fill_args(ts_ctx* ctx, TreeArgs& a, char* base, const TreeWs& w, boo
   a.own = owner_layout(c.Nmax, c.K, c.r);
   a.ragged = c.V % 8 ? 1 : 0;
   a.Vs = p.Vs; a.Uscan = a.ragged ? base + w.upad : U; a.Wscan = a.ragged ? base + w.wpad : W;
-  a.TV = p.TV; a.ntiles = p.ntiles; a.BN = p.BN; a.nW = p.nW; a.nU = p.nU; a.npiece = p.npiece; a.w_over = p.w_over;
-  a.oU = p.oU; a.oL = p.oL; a.oW = p.oW; a.oX = p.oX;
+  a.TV = p.TV; a.ntiles = p.ntiles; a.BN = p.BN; a.nW = p.nW; a.npiece = p.npiece; a.w_over = p.w_over;
+  a.oL = p.oL; a.oW = p.oW; a.oX = p.oX;
+  for (uint32_t i = 0; i < 10; ++i) { a.rk[2 * i] = (uint32_t)seed + i * 0x9E3779B9u; a.rk[2 * i + 1] = (uint32_t)(seed >> 32) + i * 0xBB67AE85u; }
   a.no_seed = (ctx->test_mode & TS_TEST_NO_SEED) ? 1 : 0;
   int* head = (int*)(base + w.head);
   a.barrier = (unsigned*)head; a.err = head + 4; a.lvl_count = head + 8;
   for (int i = 0; i < (expand ? 2 : 1); ++i) { a.ent[i] = (ParentEntry*)(base + w.ent[i]); a.ent_slot[i] = expand ? (int*)(base + w.slot[i]) : nullptr; }
-  a.sums = (float4*)(base + w.sums); a.cand_cnt = (int*)(base + w.cnt);
+  a.sums = (float4*)(base + w.sums); for (int i = 0; i < 2; ++i) a.cand_cnt[i] = (int*)(base + w.cnt) + (expand ? i : 0) * 2 * (size_t)w.cap;
   a.cand_top = (uint2*)(base + w.top); a.cand_key = (uint2*)(base + w.key); a.cand_lg = (float*)(base + w.lg);
   a.cap = w.cap; a.thr = (unsigned*)(base + w.thr); a.slots = a.thr + 2 * (size_t)w.cap;
   a.utop = (uint2*)(base + w.utop);

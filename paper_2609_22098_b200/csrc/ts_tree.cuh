@@ -12,8 +12,7 @@ constexpr int TX_SPLIT = TX_SCAN_WARPS / 4;
 constexpr int TX_MMA = TX_SCAN_WARPS;      // issues the MMAs
 constexpr int TX_REFRESH = TX_SCAN_WARPS + 1;   // requests W, keeps the rows' launch-wide bounds current
 constexpr int TX_SELECT = TX_SCAN_WARPS + 2;    // evaluates queued candidates exactly
-constexpr int TX_COPY = TX_SCAN_WARPS + 3;      // brings base logits into shared memory
-constexpr int TX_WARPS = TX_SCAN_WARPS + 4;      // (a multiple of four: one warp more would cost every thread 16 registers)
+constexpr int TX_WARPS = TX_SCAN_WARPS + 3;
 constexpr int TX_THREADS = TX_WARPS * 32;
 constexpr int TX_ROWS = 128;               // parent rows of one MMA tile
 constexpr int TX_QCAP = 256;               // candidate queue entries (power of two)
@@ -44,13 +43,15 @@ struct TreeArgs {
   const int *p_req, *p_depth, *p_token; const uint64_t* p_hash;      // the given parents
   float *o_lse0, *o_lseT; int* o_top_tok; float* o_top_logit; int* o_draw_tok; float* o_draw_logit;
   // plan
-  int TV, ntiles, BN, nW, nU, npiece, w_over, use_tma, no_seed, ragged;
-  uint32_t oU, oL, oW, oX;   // byte offsets of the U ring, the selection state, the W ring and the fixed part
+  int TV, ntiles, BN, nW, npiece, w_over, use_tma, no_seed, ragged;
+  uint32_t oL, oW, oX;   // byte offsets of the selection state, the W ring and the fixed part
+  uint32_t rk[20];       // round keys of the sampling generator
   // workspace
   ParentEntry* ent[2]; int* ent_slot[2];
   int* lvl_count; unsigned* barrier; int* err;
   float4* sums;                                    // [cap][ntiles]: max reference, sum, tempered sum of every tile
-  int* cand_cnt; uint2 *cand_top, *cand_key; float* cand_lg;   // candidates per parent: (value, token), and the keys' logits
+  int* cand_cnt[2]; uint2 *cand_top, *cand_key; float* cand_lg;   // candidates per parent: (value, token), and the keys' logits
+                                                                 // (counts by level parity: an owner clears the next level's while others still read this one's)
   unsigned *thr, *slots; int cap;
   uint2* utop;                                     // [2][B][npiece] (given parents: [P][npiece]): best base logit of every piece of a row
   unsigned char* pool; size_t pool_stride;         // per request: PoolView
