@@ -55,6 +55,7 @@ static bool select_paths(ts_ctx* ctx) {
   ctx->use_tree = (c.dt_U == TS_DTYPE_BF16 && c.r % 8 == 0 && ctx->cc_major == 10 && !(tm & TS_TEST_FORCE_FMA) &&
                    tree_plan(c, ctx->num_sms, ctx->max_smem, &ctx->tree)) ? 1 : 0;
   ctx->tmapT_ptr = nullptr;
+  ctx->use_walk = (c.dt_U == TS_DTYPE_BF16 && c.r % 8 == 0 && ctx->cc_major == 10 && !(tm & TS_TEST_FORCE_FMA)) ? 1 : 0;
   ctx->few_ok = (few_supported(ctx) && !(tm & TS_TEST_NO_FEW)) ? 1 : 0;
   ctx->wait_limit = (tm & TS_TEST_SHORT_WAITS) ? 4096u : WAIT_LIMIT;
   return true;
@@ -121,6 +122,7 @@ extern "C" int32_t ts_create(const ts_config* cfg, ts_ctx** out) {
   e = score_setup(ctx);
   if (e == cudaSuccess && ctx->use_tree) e = tree_setup(ctx);
   if (e == cudaSuccess) e = verify_setup(ctx);
+  if (e == cudaSuccess) e = walk_setup(ctx);
   if (e == cudaSuccess) e = expand_setup(ctx);
   if (e != cudaSuccess) { cudaFree(ctx->d_table); delete (Prof*)ctx->prof; delete ctx; return set_cuda_error("ts_create", e); }
   *out = ctx;

@@ -77,6 +77,7 @@ struct ts_ctx {
   int max_smem;
   ts::TileCfg tile;
   ts::TreePlan tree;
+  int use_walk;     // 1: the walk's reductions may run on the tensor cores
   int use_tree;     // 1: expansion and scoring run on the one-launch tensor-core kernel
   int vt_TV, vt_n;  // vocabulary ranges of the verification walk, one per CTA
   int use_mma;      // 1: scoring runs on the tensor-core kernel, 0: on the fp32 FMA kernel
@@ -133,9 +134,11 @@ struct WsLayout {
   size_t vf_lists;                       // int[2][B] reduction list, int[2][B] rescan list, int[8] counters
   size_t vf_edge;                        // double[3][B][N]: per edge p(x), q(x) and the accept uniform
   size_t tree;                           // the one-launch expansion's region (ts_tree.cu lays it out)
+  size_t walk;                           // the tensor-core walk's region (ts_walk.cu)
   size_t total;
 };
 
+size_t walk_ws_bytes(const ts_ctx* ctx, int B);
 size_t tree_ws_bytes(const ts_ctx* ctx, int B);
 
 __host__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -214,6 +217,7 @@ __host__ inline WsLayout make_layout(const ts_ctx* ctx, int B) {
   L.vf_lists = take((4 * b + 8) * 4);
   L.vf_edge = take(3 * b * N * 8);
   L.tree = ctx->use_tree ? take(tree_ws_bytes(ctx, B)) : 0;
+  L.walk = take(walk_ws_bytes(ctx, B));
   L.total = off;
   return L;
 }

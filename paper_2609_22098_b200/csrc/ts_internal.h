@@ -15,6 +15,7 @@ int32_t set_cuda_error(const char* where, cudaError_t e);
 cudaError_t score_setup(ts_ctx* ctx);
 cudaError_t verify_setup(ts_ctx* ctx);
 cudaError_t expand_setup(ts_ctx* ctx);
+cudaError_t walk_setup(ts_ctx* ctx);
 size_t level_smem_bytes(const ts_config& c);
 
 struct ScoreArgs {

@@ -109,4 +109,14 @@ __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* r) {
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// Where a role stands in the stream of blocks: every role passes every block of every group in the same order.
+// (Phases are kept per slot: the number of slots in use may change between passes.)
+struct BlockPos {
+  int slot; uint32_t phase, seen;   // bit per slot: parity of its next "full", whether it was used before
+  __device__ __forceinline__ uint32_t full() const { return (phase >> slot) & 1u; }
+  __device__ __forceinline__ bool reused() const { return (seen >> slot) & 1u; }
+  __device__ __forceinline__ uint32_t empty() const { return full() ^ 1u; }
+  __device__ __forceinline__ void next(int n) { phase ^= 1u << slot; seen |= 1u << slot; if (++slot == n) slot = 0; }
+};
+
 }  // namespace ts

@@ -168,16 +168,6 @@ __device__ __forceinline__ void tx_select(const TreeArgs& a, const TxSm& sm, con
   }
 }
 
-// Where a role stands in the stream of blocks: every role passes every block of every group in the same order.
-// (Phases are kept per slot: with few parents a group uses more, smaller base-logit slots than with many.)
-struct BlockPos {
-  int slot; uint32_t phase, seen;   // bit per slot: parity of its next "full", whether it was used before
-  __device__ __forceinline__ uint32_t full() const { return (phase >> slot) & 1u; }
-  __device__ __forceinline__ bool reused() const { return (seen >> slot) & 1u; }
-  __device__ __forceinline__ uint32_t empty() const { return full() ^ 1u; }
-  __device__ __forceinline__ void next(int n) { phase ^= 1u << slot; seen |= 1u << slot; if (++slot == n) slot = 0; }
-};
-
 __device__ __noinline__ bool tx_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort, int* err, uint32_t limit) {
   for (uint32_t i = 0; i < limit; ++i) {
     if (mbar_try_wait(bar, parity)) return true;

@@ -18,6 +18,7 @@
 #include "ts_internal.h"
 #include "ts_scan.cuh"
 #include "ts_tc.cuh"
+#include "ts_walk.cuh"
 
 namespace ts {
 
@@ -1202,6 +1203,22 @@ extern "C" int32_t ts_verify_tree(ts_ctx* ctx, const void* U, const void* A, con
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_cuda_error("ts_verify_tree(greedy)", e);
     return TS_OK;
+  }
+  if (ctx->use_walk) {
+    const bool tma = c.V % 8 == 0 && w_tensor_map(ctx, W);
+    WalkPlan wp;
+    if (walk_plan(ctx, B, tma, &wp)) {
+      WalkArgs w{};
+      w.U = (const __nv_bfloat16*)U; w.A = (const __nv_bfloat16*)A; w.W = (const __nv_bfloat16*)W; w.Z = (const __nv_bfloat16*)Z; w.z_row_off = z_row_off;
+      w.B = B; w.V = c.V; w.D = c.D; w.r = c.r; w.N = c.Nmax; w.T = T; w.seed = seed;
+      w.anchor = anchor_tok; w.n_nodes = n_nodes; w.tok = tok; w.parent = parent; w.depth = depth; w.node_hash = node_hash;
+      w.logqT = logqT; w.node_lseT = node_lseT; w.z_max = z_max; w.z_logs = z_logs;
+      w.acc_len = acc_len; w.acc_node = acc_node; w.acc_tok = acc_tok; w.bonus = bonus_tok; w.edge_stat = edge_stat; w.flags = flags; w.status = status;
+      w.part = a.part; w.barrier = a.barrier; w.vt_TV = a.vt_TV; w.vt_n = a.vt_n; w.max_steps = a.max_steps;
+      w.wait_limit = a.wait_limit; w.lost_arrival = a.lost_arrival; w.use_tma = tma ? 1 : 0;
+      e = launch_walk_mma(ctx, w, ws + L.walk, wp, st);
+      return e == cudaSuccess ? TS_OK : set_cuda_error("ts_verify_tree(walk)", e);
+    }
   }
   size_t w_bytes = (size_t)c.r * ctx->vt_TV * (c.dt_W == TS_DTYPE_BF16 ? 2 : 4);
   a.w_smem = (w_bytes + 40 * 1024 <= (size_t)ctx->max_smem) ? 1 : 0;
