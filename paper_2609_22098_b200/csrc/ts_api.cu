@@ -56,7 +56,7 @@ static bool select_paths(ts_ctx* ctx) {
                    tree_plan(c, ctx->num_sms, ctx->max_smem, &ctx->tree)) ? 1 : 0;
   ctx->tmapT_ptr = nullptr;
   ctx->use_walk = (c.dt_U == TS_DTYPE_BF16 && c.r % 8 == 0 && ctx->cc_major == 10 && !(tm & TS_TEST_FORCE_FMA)) ? 1 : 0;
-  ctx->few_ok = (few_supported(ctx) && !(tm & TS_TEST_NO_FEW)) ? 1 : 0;
+  ctx->few_cap = (tm & TS_TEST_NO_FEW) ? 0 : few_capacity(c);
   ctx->wait_limit = (tm & TS_TEST_SHORT_WAITS) ? 4096u : WAIT_LIMIT;
   return true;
 }

@@ -31,7 +31,6 @@ constexpr int SLOT_STRIDE = 32;
 constexpr int SEED_PARTS_MAX = 16, SEED_SPLIT_PARENTS = 256, NSEED_MAX = 32;
 constexpr size_t SEED_CAND_WORDS = (size_t)SEED_SPLIT_PARENTS * SEED_PARTS_MAX * NSEED_MAX * 2;
 constexpr int UMMA_REQ = 32;         // requests whose base logits can ride through the tensor cores (rows of one extra B-operand slab)
-constexpr int FEW_MAX = 8;           // levels with at most this many parents go to the few-parents scoring kernel
 constexpr int SCORE_THREADS = 128;   // one parent per thread; every thread scans the CTA's whole tile
 constexpr int CHUNK = 16;            // tokens per coarse generator call
 constexpr int MMA_S = 4;             // column splits per tile in the tensor-core scoring kernel (scanning warps per row quarter)
@@ -81,7 +80,7 @@ struct ts_ctx {
   int use_tree;     // 1: expansion and scoring run on the one-launch tensor-core kernel
   int vt_TV, vt_n;  // vocabulary ranges of the verification walk, one per CTA
   int use_mma;      // 1: scoring runs on the tensor-core kernel, 0: on the fp32 FMA kernel
-  int few_ok;       // 1: levels with <= FEW_MAX parents run on the few-parents kernel instead
+  int few_cap;      // levels with at most this many parents run on the few-parents kernel instead (0: none)
   ts::DevCalib calib;
   void* prof;  // ts::Prof*, instrumentation state
   // tensor-map descriptor of the W matrix last scored with (bulk-tensor loads of the W tile); -1: the
@@ -164,12 +163,12 @@ struct VerifyState {
 };
 
 // Bytes of the scoring records for `cap` parent slots: one record per (tile, slot) of the tile kernels,
-// and room for the few-parents kernel's records (one per 256-token tile and parent, at most FEW_MAX
+// and room for the few-parents kernel's records (one per 256-token tile and parent, at most few_cap
 // parents), whichever is larger.
 __host__ inline size_t record_bytes(const ts_ctx* ctx, int cap) {
   const size_t rw = (4 + 5 * (size_t)ctx->cfg.K + 3) & ~(size_t)3;
   const size_t tile = (size_t)ctx->tile.ntiles * (size_t)cap;
-  const size_t few = (size_t)((ctx->cfg.V + 255) / 256) * FEW_MAX;
+  const size_t few = (size_t)((ctx->cfg.V + 255) / 256) * (size_t)ctx->few_cap;
   return align_up((tile > few ? tile : few) * rw * sizeof(float), 256);
 }
 

@@ -226,7 +226,7 @@ extern "C" int32_t ts_expand_tree(ts_ctx* ctx, const void* U, const void* A, con
   if (seeds_on && (ctx->test_mode & TS_TEST_PERSIST) && persistent_supported(ctx, B, 0)) coop_from = 0;
   else if (seeds_on && !(ctx->test_mode & TS_TEST_NO_TAIL)) {
     // (a handful of requests rarely has parents at the fourth level either: one level earlier there)
-    const int from = (ctx->few_ok && B <= FEW_MAX) ? TAIL_FROM - 1 : TAIL_FROM;
+    const int from = TAIL_FROM;
     if (c.D > from + 1 && persistent_supported(ctx, B, from)) coop_from = from;
   }
   long long level_bound = B;   // parents a level can have at most: B at the root, K times more per level, B * Nmax overall
@@ -236,7 +236,7 @@ extern "C" int32_t ts_expand_tree(ts_ctx* ctx, const void* U, const void* A, con
   bool scouted_prev = false;
   for (int d = 0; d < coop_from; ++d) {
     const int cur = d & 1;
-    const bool on_mma = ctx->use_mma && !(ctx->few_ok && level_bound <= FEW_MAX);
+    const bool on_mma = ctx->use_mma != 0;
     ScoreExtras ex;
     ex.thr0_ready = scouted_prev;
     ex.root_B = d == 0 ? B : 0;

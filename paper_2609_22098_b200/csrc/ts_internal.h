@@ -27,6 +27,7 @@ struct ScoreArgs {
   int seed_root_B;         // seed kernel: > 0 = the parents are the roots of that many requests (parent p = request p at depth 0)
   int pdl;                 // host side: launch with programmatic stream serialization
   int few;                 // host side: this launch runs on the few-parents kernel
+  int few_cap;             // parents its records have room for
   const int *p_req, *p_depth, *p_token; const uint64_t* p_hash;
   float T; uint64_t seed;
   int TV, ntiles, cap, S;
@@ -53,7 +54,7 @@ struct ScoreArgs {
 struct MergeArgs {
   int P; const int* P_dev; int K, ntiles, cap, S, mma; float T;
   int pdl;   // host side: launch with programmatic stream serialization
-  int few_ntiles;   // > 0: the level was scored by the few-parents kernel over this many tiles
+  int few_ntiles, few_cap;   // few_ntiles > 0: the level was scored by the few-parents kernel over this many tiles
   const float* rec; unsigned* thr; unsigned* slots; const unsigned* thr0;
   float *lse0, *lseT; int* top_tok; float* top_logit; int* draw_tok; float* draw_logit;
 };
@@ -66,7 +67,7 @@ unsigned* thr_base(const ts_ctx* ctx, float* rec, int cap);
 size_t thr_bytes(const ts_ctx* ctx, int cap);
 
 // Scoring pass + merge for a parent list whose length is P (host) or *P_dev (device) when P_dev is set;
-// p_bound: an upper bound of *P_dev the host knows (-1: none).  A list that cannot exceed FEW_MAX parents
+// p_bound: an upper bound of *P_dev the host knows (-1: none).  A list that cannot exceed few_cap parents
 // goes to the few-parents kernel where the context has one.
 // rec: record scratch of score_scratch_bytes(ctx, max parents) bytes with slot capacity cap.
 ScoreArgs make_score_args(const ts_ctx* ctx, float* rec, int cap, int* err, const void* U, const void* A, const void* W, float T,
@@ -108,7 +109,7 @@ cudaError_t launch_score_mma(const ts_ctx* ctx, const ScoreArgs& a, cudaStream_t
 cudaError_t launch_seed(const ts_ctx* ctx, const ScoreArgs& a, cudaStream_t st);
 // the few-parents kernel (ts_score_few.cu)
 int few_tiles(const ts_config& c);
-bool few_supported(const ts_ctx* ctx);
+int few_capacity(const ts_config& c);
 cudaError_t launch_score_few(const ts_ctx* ctx, const ScoreArgs& a, int p_bound, cudaStream_t st);
 // encodes (or finds cached in the context) the tensor map of W for 64-token boxes; false: not available
 bool w_tensor_map(ts_ctx* ctx, const void* W);

@@ -109,7 +109,7 @@ __device__ __forceinline__ void merge_parent(const MergeArgs& a, const int p, co
     sync();
     float m = -INFINITY, s0 = 0.f, sT = 0.f;
     auto rec_of = [&](int q) {
-      if (few) return a.rec + ((size_t)q * FEW_MAX + p) * rw;
+      if (few) return a.rec + ((size_t)q * a.few_cap + p) * rw;
       const int ts_ = q / R, rho = q % R;
       const int slot = R > 1 ? rho * (128 / R) + p : p;
       return a.rec + ((size_t)ts_ * a.cap + slot) * rw;

@@ -167,9 +167,10 @@ cudaError_t launch_score(const ts_ctx* ctx, float* rec, int cap, int* err, const
   a.p_req = p_req; a.p_depth = p_depth; a.p_token = p_token; a.p_hash = p_hash;
   cudaError_t e = cudaSuccess;
   // Which kernel scores the level: the few-parents kernel when the host knows that the list cannot hold
-  // more than FEW_MAX parents (its own P, or a bound of the device-side count), the tile kernel otherwise.
+  // more than few_cap parents (its own P, or a bound of the device-side count), the tile kernel otherwise.
   const int bound = P_dev ? p_bound : P;
-  const bool run_few = ctx->use_mma && ctx->few_ok && bound >= 0 && bound <= FEW_MAX;
+  const bool run_few = bound >= 0 && bound <= ctx->few_cap;
+  a.few_cap = ctx->few_cap;
   const bool run_tile = !run_few;
   a.few = run_few ? 1 : 0;
   if (run_tile && ctx->use_mma && !(ctx->test_mode & TS_TEST_NO_SEED)) {
@@ -209,7 +210,7 @@ cudaError_t launch_score(const ts_ctx* ctx, float* rec, int cap, int* err, const
   }
   MergeArgs m{};
   m.pdl = a.pdl;
-  m.few_ntiles = run_few ? few_tiles(c) : 0;
+  m.few_ntiles = run_few ? few_tiles(c) : 0; m.few_cap = ctx->few_cap;
   m.P = P; m.P_dev = P_dev; m.K = c.K; m.ntiles = a.ntiles; m.cap = cap; m.S = a.S; m.mma = ctx->use_mma ? 1 : 0; m.T = T;
   m.rec = rec; m.thr = a.thr; m.slots = a.slots; m.thr0 = a.thr0;
   m.lse0 = lse0; m.lseT = lseT; m.top_tok = top_tok; m.top_logit = top_logit; m.draw_tok = draw_tok; m.draw_logit = draw_logit;

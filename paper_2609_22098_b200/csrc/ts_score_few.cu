@@ -1,36 +1,39 @@
-// Scoring kernel for levels with few parents (single-request decoding, the last levels of a batch).
+// Scoring kernel for fp32 inputs when the parents of a level are few (a small model decoding a request or a handful).
 //
-// With a handful of parents the low-rank bias [parents x r] . [r x V] is no dense contraction: a
-// 128-row tensor-core tile would carry one to sixteen useful rows, and the epilogue of the tensor-core
-// kernel -- one parent per lane -- would leave most lanes idle while it walks the vocabulary.  Here the
+// With a handful of parents the low-rank bias [parents x r] . [r x V] is no dense contraction, and the tile kernel -- one
+// parent per lane, every lane over the whole tile -- would leave most lanes idle while it walks the vocabulary.  Here the
 // mapping is turned round: one warp = one (parent, 256-token tile), one lane = eight consecutive tokens.
 // The lane forms its eight logits with fused multiply-adds (U + sum_k A[x_p][k] W[k][v], k ascending),
 // every token gets its exact Gumbel key (no bounds: a tile is over before any could arrive), and the
-// warp's K best logits and K best keys come out of K rounds of a shuffle arg-max.  The whole grid works
-// on every parent at once: the launch takes a few microseconds instead of the tens the tile kernel needs
-// to get going.  W is read through L1 (the eight warps of a CTA share a tile and its lines).
+// warp's K best logits and K best keys come out of K rounds of a warp-wide arg-max.  The whole grid works
+// on every parent at once.  W is read through L1 (the eight warps of a CTA share a tile and its lines).
+// One parent at V = 32,000, r = 16: 61 us with the tile kernel, FEWTIME here.
 //
-// Records have the layout of the other scoring kernels (header (max, sum0, sumT, counts), then K logits,
-// K tokens, K keys, K tokens, K logits), one per (tile, parent) at rec[(tile * FEW_MAX + p) * rec_words];
+// Records have the layout of the tile kernel's (header (max, sum0, sumT, counts), then K logits,
+// K tokens, K keys, K tokens, K logits), one per (tile, parent) at rec[(tile * few_cap + p) * rec_words];
 // the merge kernel is told which kernel ran.  The host sends a level here when it knows that the level
-// cannot have more than FEW_MAX parents (B * K^depth and B * Nmax bound it).
+// cannot have more than few_cap parents (B * K^depth and B * Nmax bound it); few_cap is what 4 MiB of records hold, 256 at most.
 #include "ts_internal.h"
 #include "ts_scan.cuh"
 
 namespace ts {
 
+// eight consecutive elements
+__device__ __forceinline__ void load8(const float* p, float* out) {
+  const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  out[0] = a.x; out[1] = a.y; out[2] = a.z; out[3] = a.w; out[4] = b.x; out[5] = b.y; out[6] = b.z; out[7] = b.w;
+}
+
 constexpr int FEW_THREADS = 256;
 constexpr int FEW_WARPS = FEW_THREADS / 32;
 constexpr int FEW_TILE = 256;   // tokens per tile: eight per lane
 
-// (value desc, token asc) arg-max over the warp; every lane gets the winner
+// (value desc, token asc) arg-max over the warp; every lane gets the winner (two reductions of integers: the value's
+// order-preserving image, then the lowest token among those that have it)
 __device__ __forceinline__ void warp_best(float& v, int& tok) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float ov = __shfl_xor_sync(0xFFFFFFFFu, v, off);
-    const int ot = __shfl_xor_sync(0xFFFFFFFFu, tok, off);
-    if (ov > v || (ov == v && ot < tok)) { v = ov; tok = ot; }
-  }
+  const unsigned e = enc_f(v), m = __reduce_max_sync(0xFFFFFFFFu, e);
+  tok = (int)__reduce_min_sync(0xFFFFFFFFu, e == m ? (unsigned)tok : 0x7FFFFFFFu);
+  v = dec_f(m);
 }
 
 __global__ void __launch_bounds__(FEW_THREADS) score_few_kernel(const ScoreArgs a) {
@@ -39,28 +42,28 @@ __global__ void __launch_bounds__(FEW_THREADS) score_few_kernel(const ScoreArgs 
   pdl_wait();                // the parent list and its length come from the kernel before
   pdl_launch_dependents();
   const int P = a.P_dev ? *a.P_dev : a.P;
-  if (P <= 0 || P > FEW_MAX) return;   // an empty level (the host never sends a longer list here)
+  if (P <= 0 || P > a.few_cap) return;   // an empty level (the host never sends a longer list here)
   const int p = blockIdx.y * FEW_WARPS + warp;
   if (p >= P) return;                  // no block-wide barrier below
   const int V = a.V, r = a.r, K = a.K;
   const int tile = blockIdx.x, v = tile * FEW_TILE + lane * 8;
   const bool in = v < V;               // V is a multiple of 8: a lane's eight tokens are all inside or all outside
-  const __nv_bfloat16* Wg = reinterpret_cast<const __nv_bfloat16*>(a.W);
-  const __nv_bfloat16* Ug = reinterpret_cast<const __nv_bfloat16*>(a.U);
-  const __nv_bfloat16* Ag = reinterpret_cast<const __nv_bfloat16*>(a.A);
+  const float* Wg = reinterpret_cast<const float*>(a.W);
+  const float* Ug = reinterpret_cast<const float*>(a.U);
+  const float* Ag = reinterpret_cast<const float*>(a.A);
   const int req = a.p_req[p], dep = a.p_depth[p], ptok = a.p_token[p];
   const uint64_t hash = a.p_hash[p];
-  for (int k = lane; k < r; k += 32) s_a[warp][k] = __bfloat162float(Ag[(size_t)ptok * r + k]);
+  for (int k = lane; k < r; k += 32) s_a[warp][k] = Ag[(size_t)ptok * r + k];
   __syncwarp();
 
   // ---- logits of the lane's eight tokens -------------------------------------------------------------
   float l[8];
   if (in) {
-    unpack_bf16x8(__ldg(reinterpret_cast<const uint4*>(Ug + ((size_t)req * a.D + dep) * V + v)), l);
+    load8(Ug + ((size_t)req * a.D + dep) * V + v, l);
 #pragma unroll 16
     for (int k = 0; k < r; ++k) {
       float w[8];
-      unpack_bf16x8(__ldg(reinterpret_cast<const uint4*>(Wg + (size_t)k * V + v)), w);
+      load8(Wg + (size_t)k * V + v, w);
       const float ak = s_a[warp][k];
 #pragma unroll
       for (int i = 0; i < 8; ++i) l[i] = fmaf(ak, w[i], l[i]);
@@ -158,7 +161,7 @@ __global__ void __launch_bounds__(FEW_THREADS) score_few_kernel(const ScoreArgs 
 
   // ---- record ----------------------------------------------------------------------------------------------
   const int rw = rec_words(K);
-  float* rec = a.rec + ((size_t)tile * FEW_MAX + p) * rw;
+  float* rec = a.rec + ((size_t)tile * a.few_cap + p) * rw;
   const int nt = __popc(__ballot_sync(0xFFFFFFFFu, lane < K && topi >= 0));
   const int nk = __popc(__ballot_sync(0xFFFFFFFFu, lane < K && keyi >= 0));
   if (lane == 0) *reinterpret_cast<float4*>(rec) = make_float4(m, s0, sT, __int_as_float(nt | (nk << 8)));
@@ -170,10 +173,11 @@ __global__ void __launch_bounds__(FEW_THREADS) score_few_kernel(const ScoreArgs 
 
 int few_tiles(const ts_config& c) { return (c.V + FEW_TILE - 1) / FEW_TILE; }
 
-// bf16 inputs with 16-byte rows; the records of the largest level this kernel takes must fit the scratch
-bool few_supported(const ts_ctx* ctx) {
-  const ts_config& c = ctx->cfg;
-  return ctx->use_mma && c.dt_U == TS_DTYPE_BF16 && c.V % 8 == 0 && c.r <= 256 && c.K <= 32;
+// parents a launch may hold (0: the kernel does not serve this configuration)
+int few_capacity(const ts_config& c) {
+  if (c.dt_U != TS_DTYPE_F32 || c.V % 8 != 0) return 0;
+  const size_t per = (size_t)few_tiles(c) * rec_words(c.K) * 4, cap = ((size_t)4 << 20) / per;
+  return cap > 256 ? 256 : (cap < 8 ? 8 : (int)cap);
 }
 
 cudaError_t launch_score_few(const ts_ctx* ctx, const ScoreArgs& a, int p_bound, cudaStream_t st) {
