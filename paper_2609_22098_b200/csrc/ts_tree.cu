@@ -29,6 +29,16 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool in) 
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// sixteen consecutive bf16 (32-byte aligned when `wide`): read once, so not kept in L1; hi = false: only the first eight exist
+__device__ __forceinline__ void load16_bf16(const __nv_bfloat16* p, const bool wide, const bool hi, uint4& a, uint4& b) {
+  if (wide) {
+    asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
+  } else {
+    a = __ldcg(reinterpret_cast<const uint4*>(p));
+    if (hi) b = __ldcg(reinterpret_cast<const uint4*>(p) + 1);
+  }
+}
 // one lane of a converged warp (the instruction tells the compiler that the branch is uniform)
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
@@ -39,7 +49,7 @@ __device__ __forceinline__ bool elect_one() {
 // Shared-memory state of a CTA.
 struct TxSm {
   unsigned char *As, *Ws;
-  uint4* q;                    // [TX_QCAP] queued candidates: token, logit, row | split << 8 | kind << 12 | c16 << 16, tag
+  unsigned long long* q;       // [TX_QCAP] queued candidates (QEntry)
   float* lists;                // [128][5K]: topv, topi, keyv, keyi, keyl of every row, sorted (value desc, token asc)
   int* ln;                     // [2][128] entries in use
   volatile float* lthr;        // [2][128] K-th best of the row's own list (-inf until it is full)
@@ -55,14 +65,14 @@ struct TxSm {
 };
 
 constexpr size_t tx_select_bytes(int K) {
-  return (size_t)TX_QCAP * 16 + (size_t)TX_ROWS * 5 * K * 4 + 2 * TX_ROWS * 4 + 2 * TX_ROWS * 4 + 2 * TX_SPLIT * TX_ROWS * 4 + 3 * TX_SPLIT * TX_ROWS * 4;
+  return (size_t)TX_QCAP * 8 + (size_t)TX_ROWS * 5 * K * 4 + 2 * TX_ROWS * 4 + 2 * TX_ROWS * 4 + 2 * TX_SPLIT * TX_ROWS * 4 + 3 * TX_SPLIT * TX_ROWS * 4;
 }
 constexpr size_t TX_FIXED_BYTES = 512 * 4 + 2 * TX_ROWS * 4 + TX_ROWS * sizeof(ParentEntry) + (1 + 4 * TX_STAGE_MAX) * 8 + 64;
 
 __device__ __forceinline__ TxSm tx_carve(unsigned char* sm, const TreeArgs& a) {
   TxSm s;
   s.As = sm; s.Ws = sm + a.oW;
-  s.q = reinterpret_cast<uint4*>(sm + a.oL);
+  s.q = reinterpret_cast<unsigned long long*>(sm + a.oL);
   s.lists = reinterpret_cast<float*>(s.q + TX_QCAP);
   s.ln = reinterpret_cast<int*>(s.lists + (size_t)TX_ROWS * 5 * a.K);
   s.lthr = reinterpret_cast<float*>(s.ln + 2 * TX_ROWS);
@@ -79,6 +89,15 @@ __device__ __forceinline__ TxSm tx_carve(unsigned char* sm, const TreeArgs& a) {
   s.q_head = reinterpret_cast<volatile unsigned*>(s.tmem + 3);
   s.q_tail = s.tmem + 4;
   return s;
+}
+
+// A queued candidate in one 64-bit word, so that a plain store publishes it whole: logit in the high half; below it a tag
+// that changes with every turn of the queue (4 bits), kind (2), split (2), row (7), place in the range (17).  (With the tag
+// in a word of its own a fence had to stand between the two stores, and the fence waited for the scanning thread's
+// base-logit loads in flight: two microseconds a candidate.)
+__device__ __forceinline__ uint32_t q_tag(unsigned idx) { return (idx / TX_QCAP) % 15u + 1u; }   // never 0: 0 = nothing written
+__device__ __forceinline__ unsigned long long q_pack(float lg, unsigned idx, uint32_t kind, int split, int row, int off) {
+  return ((unsigned long long)__float_as_uint(lg) << 32) | (q_tag(idx) << 28) | (kind << 26) | ((uint32_t)split << 24) | ((uint32_t)row << 17) | (uint32_t)off;
 }
 
 // insertion into one sorted list of at most K entries (value desc, token asc); returns the K-th value (-inf: not full)
@@ -134,11 +153,11 @@ struct CoarseGen {
 };
 
 // One candidate, handled by one lane of the selecting warp: exact key, insertion, publication.
-__device__ __forceinline__ void tx_select(const TreeArgs& a, const TxSm& sm, const uint4 e, float invT, int tile, int R, int g) {
-  const int K = a.K, tok = (int)e.x;
-  const float lg = __uint_as_float(e.y);
-  const int row = (int)(e.z & 0xFFu), s = (int)((e.z >> 8) & 0xFu);
-  const uint32_t kind = (e.z >> 12) & 0xFu, c16 = e.z >> 16;
+__device__ __forceinline__ void tx_select(const TreeArgs& a, const TxSm& sm, const unsigned long long e, float invT, int tile, int R, int g) {
+  const int K = a.K, tok = tile * a.TV + (int)((uint32_t)e & 0x1FFFFu);
+  const float lg = __uint_as_float((uint32_t)(e >> 32));
+  const int row = (int)((uint32_t)e >> 17) & 127, s = (int)((uint32_t)e >> 24) & 3;
+  const uint32_t kind = ((uint32_t)e >> 26) & 3u;
   const int per = TX_ROWS / R;
   const int prow = R > 1 ? row % per : row, rho = R > 1 ? row / per : 0;
   const int p = R > 1 ? prow : g * TX_ROWS + row;
@@ -153,9 +172,10 @@ __device__ __forceinline__ void tx_select(const TreeArgs& a, const TxSm& sm, con
   }
   if (kind & 2u) {
     const float thr = fmaxf(sm.thr[TX_ROWS + prow], sm.lthr[TX_ROWS + row]);
-    const float bnd = lg * invT + sm.ghi[noise_bound_index(c16)];
-    if (bnd >= thr) {   // the bounds have often risen since the candidate was queued
-      const ParentEntry& pe = sm.ent[row];
+    const ParentEntry& pe = sm.ent[row];
+    const uint4 cw = stream_words(a.seed, pe.req, pe.hash, STREAM_GUMBEL_COARSE, (uint32_t)tok >> 3);
+    const uint32_t c16 = (word_of(cw, (tok & 7) >> 1) >> (16 * (tok & 1))) & 0xFFFFu;
+    if (lg * invT + sm.ghi[noise_bound_index(c16)] >= thr) {   // the bounds have often risen since the candidate was queued
       const uint4 fw = stream_words(a.seed, pe.req, pe.hash, STREAM_GUMBEL_FINE, (uint32_t)tok >> 3);
       const uint32_t f16 = (word_of(fw, (tok & 7) >> 1) >> (16 * (tok & 1))) & 0xFFFFu;
       const float key = lg * invT + gumbel_from_bits((c16 << 16) | f16);
@@ -217,7 +237,6 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
   const float slack = 8.f * fminf(1.f, T > 0.f ? T : 1.f);   // how far a logit may exceed the sums' reference
   CoarseGen gen; gen.init(a.rk, me.req, me.hash);
   float m = me.mref, s0 = 0.f, sT = 0.f;
-  const uint32_t ztag = (uint32_t)row | ((uint32_t)s << 8);
   const int CB = a.BN / 16, nblk = (tlen + a.BN - 1) / a.BN, stride = R * TX_SPLIT, own = rho * TX_SPLIT + s;
   const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16);
   // Base logits: 32 bytes of its parent's row per lane and chunk, straight from L2 (a scan reads each once; lanes whose
@@ -227,7 +246,8 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
   const int vleft = a.Vs - t0;   // tokens of the row from t0 on (whole 16 bytes)
   int o = own * 16;              // the next chunk to request
   uint4 nx0 = make_uint4(0u, 0u, 0u, 0u), nx1 = nx0;
-  if (o < tlen) { nx0 = __ldcg(reinterpret_cast<const uint4*>(urow + o)); if (o + 8 < vleft) nx1 = __ldcg(reinterpret_cast<const uint4*>(urow + o + 8)); }
+  const bool wide = a.wide_u != 0;
+  if (o < tlen) load16_bf16(urow + o, wide, o + 8 < vleft, nx0, nx1);
   bool alive = true;
   for (int nb = 0; nb < nblk; ++nb, pos.next(nst)) {
     const int slot = pos.slot;
@@ -240,7 +260,7 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
       tmem_ld16_issue(trow + (uint32_t)(slot * a.BN + c * 16), ra);
       const uint4 u0 = nx0, u1 = nx1;   // requested one owned chunk ago; the next one's are requested now
       o += stride * 16;
-      if (o < tlen) { nx0 = __ldcg(reinterpret_cast<const uint4*>(urow + o)); if (o + 8 < vleft) nx1 = __ldcg(reinterpret_cast<const uint4*>(urow + o + 8)); }
+      if (o < tlen) load16_bf16(urow + o, wide, o + 8 < vleft, nx0, nx1);
       const int v0 = t0 + nb * a.BN + c * 16, valid = min(16, a.V - v0);
       // high halves of the sixteen uniforms: issued first, their long dependent chains overlap the rest
       uint4 cw0 = make_uint4(0, 0, 0, 0), cw1 = cw0;
@@ -317,7 +337,6 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
         const int i = __ffs(mk) - 1;
         mk &= mk - 1;
         const uint32_t kind = ((mkL >> i) & 1u) | ((mkK >> i) & 1u) << 1;
-        const uint32_t c16 = (pick8(cw0, cw1, i >> 1) >> (16 * (i & 1))) & 0xFFFFu;
         const unsigned idx = atomicAdd(sm.q_tail, 1u);
         uint32_t spin = 0;
         while ((int)(idx - *sm.q_head) >= TX_QCAP) {   // queue full: the selecting warp is behind
@@ -325,11 +344,7 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
           if (++spin > a.wait_limit) { *sm.abort = 1; atomicExch(a.err, 1); break; }
           __nanosleep(64);
         }
-        uint4* e = sm.q + (idx & (TX_QCAP - 1));
-        e->x = (uint32_t)(v0 + i); e->y = __float_as_uint(pick16(acc, i));
-        e->z = ztag | (kind << 12) | (c16 << 16);
-        __threadfence_block();
-        *reinterpret_cast<volatile uint32_t*>(&e->w) = idx + 1u;   // tag: the entry is complete
+        *reinterpret_cast<volatile unsigned long long*>(sm.q + (idx & (TX_QCAP - 1))) = q_pack(pick16(acc, i), idx, kind, s, row, v0 + i - t0);
       }
     }
     tc_fence_before();
@@ -468,25 +483,23 @@ __device__ __forceinline__ void tx_drain(const TreeArgs& a, const TxSm& sm, cons
     }
     spin = 0;
     const int n = min(avail, 32);
-    uint4 e = make_uint4(0u, 0u, 0u, 0u);
+    unsigned long long e = 0ull;
     bool have = false;
     if (lane < n) {
-      uint4* slot = sm.q + ((head + lane) & (TX_QCAP - 1));
-      uint32_t w = 0;
+      volatile unsigned long long* slot = sm.q + ((head + lane) & (TX_QCAP - 1));
+      const uint32_t tag = q_tag(head + lane);
       for (uint32_t t = 0; t < a.wait_limit; ++t) {   // the producer writes right after claiming: a few cycles
-        w = *reinterpret_cast<volatile uint32_t*>(&slot->w);
-        if (w == head + lane + 1u || *sm.abort) break;
+        e = *slot;
+        have = (((uint32_t)e >> 28) & 15u) == tag;
+        if (have || *sm.abort) break;
       }
-      have = (w == head + lane + 1u);
-      __threadfence_block();
-      if (have) { e.x = slot->x; e.y = slot->y; e.z = slot->z; }
     }
     __threadfence_block();
     __syncwarp();
     head += (unsigned)n;
     if (lane == 0) *sm.q_head = head;   // the slots may be reused
     // candidates of one row are inserted one after the other (lanes of a row take turns)
-    const unsigned peers = __match_any_sync(0xFFFFFFFFu, have ? (int)(e.z & 0xFFu) : -1 - lane);
+    const unsigned peers = __match_any_sync(0xFFFFFFFFu, have ? (int)((uint32_t)e >> 17) & 127 : -1 - lane);
     const int turn = __popc(peers & ((1u << lane) - 1u));
     const int turns = __reduce_max_sync(0xFFFFFFFFu, have ? turn + 1 : 0);
     for (int t = 0; t < turns; ++t) {
@@ -1283,8 +1296,21 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
           sm.ln[tid] = 0; sm.ln[TX_ROWS + tid] = 0; sm.lthr[tid] = -INFINITY; sm.lthr[TX_ROWS + tid] = -INFINITY;
         }
         for (int i = tid; i < 2 * TX_SPLIT * TX_ROWS; i += TX_THREADS) sm.best[i] = -INFINITY;
-        if (g == 0) for (int i = tid; i < TX_QCAP; i += TX_THREADS) sm.q[i].w = 0u;   // (owners work in this memory: the queue's tags start clean)
+        if (g == 0) for (int i = tid; i < TX_QCAP; i += TX_THREADS) sm.q[i] = 0ull;   // (owners work in this memory: the queue's tags start clean)
         __syncthreads();
+        // ask L2 for this range of every base-logit row the group reads (neighbours of the list often share theirs): the scan
+        // itself asks for 32 bytes a lane one chunk ahead, which leaves DRAM waiting when the rows are many
+        {
+          const int nrow = R > 1 ? P : min(TX_ROWS, P - g * TX_ROWS), lines = (tlen * 2 + 127) / 128;
+#pragma unroll 1
+          for (int x = warp; x < nrow; x += TX_WARPS) {
+            const int rw = sm.ent[x].row;
+            if (x > 0 && sm.ent[x - 1].row == rw) continue;
+            const __nv_bfloat16* src = reinterpret_cast<const __nv_bfloat16*>(a.Uscan) + (size_t)rw * a.Vs + t0;
+#pragma unroll 1
+            for (int l = lane; l < lines; l += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + l * 64));
+          }
+        }
         const int done_target = (groups + 1) * TX_SCAN_WARPS;
         const int nst = min(512 / a.BN, TX_STAGE_MAX);   // accumulator stages
         if (warp < TX_SCAN_WARPS) tx_scan(a, sm, R, P, g, t0, tlen, tmem_base, pos, nst);
@@ -1403,7 +1429,7 @@ bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
     int nW = 2;
     auto total = [&](int nw) { return A + sel + fix + (size_t)nw * w; };
     if (total(nW) > avail) continue;
-    while (nW < TX_STAGE_MAX && total(nW + 1) <= avail) ++nW;
+    while (nW < TX_NW && total(nW + 1) <= avail) ++nW;
     p.BN = BN; p.nW = nW;
     p.oL = (uint32_t)A; p.oW = (uint32_t)(p.oL + sel); p.oX = (uint32_t)(p.oW + (size_t)nW * w);
     // owners work in [A, selection state] and, where that is not enough, in the W ring (which then does not run ahead);
@@ -1455,6 +1481,7 @@ static void fill_args(ts_ctx* ctx, TreeArgs& a, char* base, const TreeWs& w, boo
   a.own = owner_layout(c.Nmax, c.K, c.r);
   a.ragged = c.V % 8 ? 1 : 0;
   a.Vs = p.Vs; a.Uscan = a.ragged ? base + w.upad : U; a.Wscan = a.ragged ? base + w.wpad : W;
+  a.wide_u = (p.Vs % 16 == 0 && ((uintptr_t)a.Uscan & 31u) == 0) ? 1 : 0;
   a.TV = p.TV; a.ntiles = p.ntiles; a.BN = p.BN; a.nW = p.nW; a.npiece = p.npiece; a.w_over = p.w_over;
   a.oL = p.oL; a.oW = p.oW; a.oX = p.oX;
   for (uint32_t i = 0; i < 10; ++i) { a.rk[2 * i] = (uint32_t)seed + i * 0x9E3779B9u; a.rk[2 * i + 1] = (uint32_t)(seed >> 32) + i * 0xBB67AE85u; }

@@ -17,6 +17,9 @@ constexpr int TX_THREADS = TX_WARPS * 32;
 constexpr int TX_ROWS = 128;               // parent rows of one MMA tile
 constexpr int TX_QCAP = 256;               // candidate queue entries (power of two)
 constexpr int TX_STAGE_MAX = 8;
+#ifndef TX_NW
+#define TX_NW 8
+#endif
 constexpr int TX_PIECE = 1024;             // tokens of one scouting item
 
 // Everything the scan needs to know about one parent.
@@ -43,6 +46,7 @@ struct TreeArgs {
   const int *p_req, *p_depth, *p_token; const uint64_t* p_hash;      // the given parents
   float *o_lse0, *o_lseT; int* o_top_tok; float* o_top_logit; int* o_draw_tok; float* o_draw_logit;
   // plan
+  int wide_u;            // base-logit rows start on 32 bytes
   int TV, ntiles, BN, nW, npiece, w_over, use_tma, no_seed, ragged;
   uint32_t oL, oW, oX;   // byte offsets of the selection state, the W ring and the fixed part
   uint32_t rk[20];       // round keys of the sampling generator
