@@ -747,8 +747,8 @@ __device__ __forceinline__ void store_seed_columns(const TreeArgs& a, const Owne
 }
 
 // Seed bounds and list entries of `cnt` parents of one row (all threads; the columns have landed).  Parent i: token
-// s.ttok[i], hash hs[i], pool slot s.npl[i]; its place in the level's list is li0 + i.
-__device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s, const int cnt, const int li0, const int req, const int row, const int NS,
+// s.ttok[i], hash hs[i], pool slot s.npl[i]; its place in the level's list is li0 + i * step.
+__device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s, const int cnt, const int li0, const int step, const int req, const int row, const int NS,
                                              const int* ptok, const uint64_t* phash, ParentEntry* ent, int* ent_slot, int* cnt_next) {
   const int tid = threadIdx.x, r = a.r, K = a.K, lg = seed_log2(K);
   const float invT = a.T > 0.f ? 1.f / a.T : 1.f;
@@ -757,12 +757,12 @@ __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s
 #pragma unroll 1
   for (int e = tid; e < cnt * 2 * K; e += TX_THREADS) {
     const int i = e / (2 * K), w = (e / K) & 1, j = e % K;
-    a.slots[(((size_t)w * a.cap + li0 + i) * K + j) * SLOT_STRIDE] = 0u;
+    a.slots[(((size_t)w * a.cap + li0 + i * step) * K + j) * SLOT_STRIDE] = 0u;
   }
 #pragma unroll 1
   for (int e = tid; e < cnt * 2; e += TX_THREADS) {
-    a.thr[(size_t)(e & 1) * a.cap + li0 + (e >> 1)] = 0u;
-    cnt_next[(size_t)(e & 1) * a.cap + li0 + (e >> 1)] = 0;
+    a.thr[(size_t)(e & 1) * a.cap + li0 + (e >> 1) * step] = 0u;
+    cnt_next[(size_t)(e & 1) * a.cap + li0 + (e >> 1) * step] = 0;
   }
   // every (parent, seed token) pair exactly: eight lanes a pair, 16 bytes of the head row a lane and step
   const int sub = tid & 7;
@@ -820,9 +820,9 @@ __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s
     ParentEntry pe;
     pe.row = row; pe.token = ptok[i]; pe.hash = phash[i]; pe.thrL = bL[i]; pe.thrK = a.T > 0.f ? bK[i] : -INFINITY; pe.mref = bM[i]; pe.req = req;
     const uint4* src = reinterpret_cast<const uint4*>(&pe);
-    uint4* dst = reinterpret_cast<uint4*>(ent + li0 + i);
+    uint4* dst = reinterpret_cast<uint4*>(ent + li0 + i * step);
     dst[0] = src[0]; dst[1] = src[1];
-    if (ent_slot) ent_slot[li0 + i] = s.npl[i];
+    if (ent_slot) ent_slot[li0 + i * step] = s.npl[i];
   }
 }
 
@@ -830,7 +830,9 @@ __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s
 // d = depth of the parents just scanned; d = -1: the start of request b (an empty pool and the root as the only parent of
 // level 0) or, for ts_score_parents, the list entry of given parent b.
 // (Inlined, once: behind a call the arguments would be read through generic addresses, some 40 cycles each.)
-__device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, const int b, const int d) {
+// share >= 0: not the level step, but the seed bounds of every `step`-th of the new parents of request b, from the share-th
+// on (a request with many leaves them to the CTAs that own none); spread: the merge was done by all CTAs.
+__device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, const int b, const int d, const int share, const int step, const bool many, const bool spread) {
   const OwnerSm s = owner_carve(sm, a);
   __shared__ int sh[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -841,7 +843,17 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
   int npar = 0, base = 0, K_eff = 0, N_eff = 0;
   double log_theta = 0.0;
   unsigned char* gpool = a.pool + (size_t)b * a.pool_stride;
-  if (d < 0) {
+  if (share >= 0) {
+    const int np = __ldcg(a.req_npar + nxt * a.B + b);
+    cnt = np > TX_SOLO ? (np - share + step - 1) / step : 0;
+    if (cnt <= 0) return;   // uniform
+    li0 = __ldcg(a.req_base + b) + share;
+#pragma unroll 1
+    for (int i = tid; i < cnt; i += TX_THREADS) {
+      const uint4 e = __ldcg(reinterpret_cast<const uint4*>(a.ent[nxt] + li0 + i * step));
+      ptok[i] = (int)e.y; phash[i] = ((uint64_t)e.w << 32) | e.z;
+    }
+  } else if (d < 0) {
     const bool given = a.score_P > 0;
     if (given) { req = a.p_req[b]; row = req * a.D + a.p_depth[b]; }
     else {
@@ -883,7 +895,18 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
   // round trips, side by side (the last warp picks the next row's seed tokens meanwhile) ----
   if (warp == TX_WARPS - 1) {
     if (more) pick_seeds(a.npiece, a.utop + ((size_t)nxt * a.B + b) * a.npiece, NS, s.stok, s.sval, lane);
-  } else if (d >= 0) {
+  } else if (spread && share < 0) {
+#pragma unroll 1
+    for (int t = tid; t < npar << lk; t += TX_THREADS - 32) {
+      const int i = t >> lk, j = t & ((1 << lk) - 1);
+      const size_t at = (size_t)(base + i) * KMAX + j;
+      if (j < K) {
+        const uint4 e = __ldcg(a.res_cand + at);
+        s.ttok[t] = (int)e.x; s.tlog[t] = __uint_as_float(e.y); s.dtok[t] = (int)e.z; s.dlog[t] = __uint_as_float(e.w);
+      }
+      if (j == 0) { const float2 l = __ldcg(a.res_lse + base + i); s.lse0[i] = l.x; s.lseT[i] = l.y; }
+    }
+  } else if (d >= 0 && share < 0) {
     const int P = __ldcg(a.lvl_count + d), R = mma_replicas(P);
 #pragma unroll 1
     for (int task = warp; task < npar * 3; task += TX_WARPS - 1) {
@@ -905,7 +928,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
   __syncthreads();
   uint32_t wcol[SEED_REGS];
   if (more) load_seed_columns(a, s, NS, 0, wcol);   // on their way while the draws are ranked
-  if (d >= 0) {
+  if (d >= 0 && share < 0) {
   // the best token of q0 not among the first j draws, for every j: places of the draws in the top list, or-ed up
 #pragma unroll 1
   for (int i = warp; i < npar; i += TX_WARPS) {
@@ -1136,13 +1159,22 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
   for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) gdst[i] = psrc[i];
   }
   // ---- seed bounds and list entries ----
-  if (more && d < 0) store_seed_columns(a, s, NS, 0, wcol);
+  if (more && (d < 0 || share >= 0)) store_seed_columns(a, s, NS, 0, wcol);
   if (more)
 #pragma unroll 1
     for (int e0 = SEED_REGS * TX_THREADS; e0 < NS * a.r; e0 += SEED_REGS * TX_THREADS) { load_seed_columns(a, s, NS, e0, wcol); store_seed_columns(a, s, NS, e0, wcol); }
   __syncthreads();
-  if (d >= 0) li0 = sh[6];
-  if (more && cnt > 0) make_parents(a, s, cnt, li0, req, row, NS, ptok, phash, a.ent[nxt], a.ent_slot[nxt], a.cand_cnt[nxt]);
+  if (d >= 0 && share < 0) li0 = sh[6];
+  if (more && share < 0 && many && cnt > TX_SOLO) {   // many parents: entries without bounds; all CTAs make those after the next barrier
+#pragma unroll 1
+    for (int i = tid; i < cnt; i += TX_THREADS) {
+      uint4* dst = reinterpret_cast<uint4*>(a.ent[nxt] + li0 + i);
+      dst[0] = make_uint4((unsigned)row, (unsigned)ptok[i], (unsigned)phash[i], (unsigned)(phash[i] >> 32));
+      dst[1] = make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, (unsigned)req);
+      a.ent_slot[nxt][li0 + i] = s.npl[i];
+    }
+    if (tid == 0) a.seed_need[d + 1] = 1;
+  } else if (more && cnt > 0) make_parents(a, s, cnt, li0, share >= 0 ? step : 1, req, row, NS, ptok, phash, a.ent[nxt], share >= 0 ? nullptr : a.ent_slot[nxt], a.cand_cnt[nxt]);
   __syncthreads();
 }
 
@@ -1256,6 +1288,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
   BlockPos pos{0, 0u, 0u}, wpos{0, 0u, 0u};
   int groups = 0;
   const int nreq = a.score_P > 0 ? a.score_P : a.B;
+  const bool many = a.score_P == 0 && ncta >= 2 * a.B;   // several CTAs a request: they help owners with many parents
   const int piece_len = (((a.V + a.npiece - 1) / a.npiece) + 7) & ~7;
 
   if (a.ragged) {   // W with padded rows (the bulk-tensor loads need rows of whole 16 bytes)
@@ -1345,27 +1378,53 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
       break;
     }
     }
-    // ---- owners ---------------------------------------------------------------------------------------------------------
-    if (d >= -1)
+    // ---- merge by all CTAs where the owners alone would take long over it (8 requests with 60 parents each: 150 us) -------
+    const bool spread = many && d >= 0 && P > 8 * a.B;
+    if (spread) {
+      const int R = mma_replicas(P), K = a.K;
 #pragma unroll 1
-      for (int b = cta; b < nreq; b += ncta) tx_owner(a, base_sm, b, d);
-    // best base logits of the rows after the next ones, by the CTAs that own no request where there are enough of them
-    // (given parents: of their rows, before anything else)
-    if (d == -2 || (a.score_P == 0 && d + 2 < a.D)) {
-      const int h0 = d >= -1 && ncta - a.B >= ncta / 4 ? a.B : 0;
-      uint2* ut = a.utop + (size_t)(d & 1) * a.B * a.npiece;
-      if (cta >= h0)
-#pragma unroll 1
-        for (int i = (cta - h0) * TX_WARPS + warp; i < nreq * a.npiece; i += (ncta - h0) * TX_WARPS) {
-          const int x = i / a.npiece;
-          if (d >= 0 && __ldcg(a.req_npar + (d & 1) * a.B + x) <= 0) continue;
-          const int row = a.score_P > 0 ? a.p_req[x] * a.D + a.p_depth[x] : x * a.D + d + 2;
-          scout_piece(a, row, i % a.npiece, piece_len, ut + i, lane);
-        }
+      for (int p = cta + ncta * warp; p < P; p += ncta * TX_WARPS) {
+        const size_t cb = (size_t)p * a.ntiles * (R * K);
+        const int* cnt = a.cand_cnt[d & 1];
+        const float2 l = warp_lse(a.sums + (size_t)p * a.ntiles, a.ntiles, a.T, lane);
+        const float3 w = warp_topk(a.cand_top + cb, nullptr, cnt + p, K, lane);
+        float3 x = w;
+        if (a.T > 0.f) x = warp_topk(a.cand_key + cb, a.cand_lg + cb, cnt + a.cap + p, K, lane);
+        if (lane == 0) a.res_lse[p] = l;
+        if (lane < K) a.res_cand[(size_t)p * KMAX + lane] = make_uint4(__float_as_uint(w.x), __float_as_uint(w.y), __float_as_uint(x.x), __float_as_uint(x.z));
+      }
+      if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
     }
-    if (d + 1 >= a.D && a.score_P == 0) break;
-    fence_async_smem();   // owners work in memory that the next scan's bulk loads may write
-    if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
+    // ---- owners (second turn: shares of the seed bounds that owners with many new parents left) ----------------------------
+    bool over = false;
+#pragma unroll 1
+    for (int turn = 0;; ++turn) {
+      if (d >= -1) {
+        const int first = turn ? cta % nreq : cta, share = turn ? cta / nreq : -1, hstep = ncta / nreq;
+        if (share < hstep)
+#pragma unroll 1
+          for (int b = first; b < nreq; b += turn ? nreq : ncta) tx_owner(a, base_sm, b, d, share, hstep, many, spread);
+      }
+      // best base logits of the rows after the next ones, by the CTAs that own no request where there are enough of them
+      // (given parents: of their rows, before anything else)
+      if (turn == 0 && (d == -2 || (a.score_P == 0 && d + 2 < a.D))) {
+        const int h0 = d >= -1 && ncta - a.B >= ncta / 4 ? a.B : 0;
+        uint2* ut = a.utop + (size_t)(d & 1) * a.B * a.npiece;
+        if (cta >= h0)
+#pragma unroll 1
+          for (int i = (cta - h0) * TX_WARPS + warp; i < nreq * a.npiece; i += (ncta - h0) * TX_WARPS) {
+            const int x = i / a.npiece;
+            if (d >= 0 && __ldcg(a.req_npar + (d & 1) * a.B + x) <= 0) continue;
+            const int row = a.score_P > 0 ? a.p_req[x] * a.D + a.p_depth[x] : x * a.D + d + 2;
+            scout_piece(a, row, i % a.npiece, piece_len, ut + i, lane);
+          }
+      }
+      if (d + 1 >= a.D && a.score_P == 0) { over = true; break; }
+      fence_async_smem();   // owners work in memory that the next scan's bulk loads may write
+      if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
+      if (turn || d < 0 || !many || __ldcg(a.seed_need + d + 1) == 0) break;   // uniform: written before the barrier
+    }
+    if (over || dead) break;
     if (d == -2 && a.ragged) asm volatile("fence.proxy.async;" ::: "memory");
   }
   if (dead && d == -2 && a.score_P == 0) {
@@ -1445,7 +1504,7 @@ bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
 }
 
 // Workspace of one call over `nreq` requests (or given parents) whose lists hold up to `cap` parents.
-struct TreeWs { size_t head, ent[2], slot[2], sums, cnt, top, key, lg, thr, utop, pool, state, caps, upad, wpad, total; int cap; };
+struct TreeWs { size_t head, ent[2], slot[2], sums, cnt, top, key, lg, thr, utop, pool, state, caps, rlse, rcand, upad, wpad, total; int cap; };
 static TreeWs tree_ws(const ts_ctx* ctx, int nreq, int cap, bool expand, int rows) {
   const ts_config& c = ctx->cfg; const TreePlan& p = ctx->tree;
   TreeWs w{}; size_t at = 0;
@@ -1459,7 +1518,7 @@ static TreeWs tree_ws(const ts_ctx* ctx, int nreq, int cap, bool expand, int row
   w.top = take(cands * 8); w.key = take(cands * 8); w.lg = take(cands * 4);
   w.thr = take(2 * C * 4 + 2 * C * c.K * SLOT_STRIDE * 4);
   w.utop = take((size_t)nreq * (expand ? 2 : 1) * p.npiece * 8);
-  if (expand) { w.pool = take((size_t)nreq * pool_bytes(c.Nmax)); w.state = take((size_t)nreq * 5 * 4); w.caps = take((size_t)nreq * 16); }
+  if (expand) { w.pool = take((size_t)nreq * pool_bytes(c.Nmax)); w.state = take((size_t)nreq * 5 * 4); w.caps = take((size_t)nreq * 16); w.rlse = take(C * 8); w.rcand = take(C * KMAX * 16); }
   if (c.V % 8) { w.upad = take((size_t)rows * p.Vs * 2); w.wpad = take((size_t)c.r * p.Vs * 2); }
   w.total = at;
   return w;
@@ -1487,7 +1546,7 @@ static void fill_args(ts_ctx* ctx, TreeArgs& a, char* base, const TreeWs& w, boo
   for (uint32_t i = 0; i < 10; ++i) { a.rk[2 * i] = (uint32_t)seed + i * 0x9E3779B9u; a.rk[2 * i + 1] = (uint32_t)(seed >> 32) + i * 0xBB67AE85u; }
   a.no_seed = (ctx->test_mode & TS_TEST_NO_SEED) ? 1 : 0;
   int* head = (int*)(base + w.head);
-  a.barrier = (unsigned*)head; a.err = head + 4; a.lvl_count = head + 8;
+  a.barrier = (unsigned*)head; a.err = head + 4; a.lvl_count = head + 8; a.seed_need = head + 8 + DMAX + 2;
   for (int i = 0; i < (expand ? 2 : 1); ++i) { a.ent[i] = (ParentEntry*)(base + w.ent[i]); a.ent_slot[i] = expand ? (int*)(base + w.slot[i]) : nullptr; }
   a.sums = (float4*)(base + w.sums); for (int i = 0; i < 2; ++i) a.cand_cnt[i] = (int*)(base + w.cnt) + (expand ? i : 0) * 2 * (size_t)w.cap;
   a.cand_top = (uint2*)(base + w.top); a.cand_key = (uint2*)(base + w.key); a.cand_lg = (float*)(base + w.lg);
@@ -1501,7 +1560,7 @@ static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream
   memset(&tm, 0, sizeof(tm));
   a.use_tma = tree_tensor_map(ctx, a.Wscan, a.Vs, &tm) ? 1 : 0;
   cudaError_t e;
-  { ProfScope ps(ctx, K_INIT, st); e = launch_kernel(tree_init_kernel, 1, 64, 0, st, true, a.barrier, 8 + DMAX + 2); }
+  { ProfScope ps(ctx, K_INIT, st); e = launch_kernel(tree_init_kernel, 1, 64, 0, st, true, a.barrier, 8 + 2 * (DMAX + 2)); }
   if (e != cudaSuccess) return e;
   ProfScope ps(ctx, prof_id, st);
   void* kargs[] = {(void*)&a, (void*)&tm};
@@ -1544,7 +1603,7 @@ cudaError_t tree_expand(ts_ctx* ctx, char* ws, const TreeOut& o, const void* U, 
   a.pool = (unsigned char*)ws + w.pool; a.pool_stride = pool_bytes(c.Nmax);
   int* state = (int*)(ws + w.state);
   a.req_npar = state; a.req_base = state + 2 * (size_t)B; a.req_nscored = state + 3 * (size_t)B; a.root_lseT = (float*)(state + 4 * (size_t)B);
-  a.req_caps = (double2*)(ws + w.caps);
+  a.req_caps = (double2*)(ws + w.caps); a.res_lse = (float2*)(ws + w.rlse); a.res_cand = (uint4*)(ws + w.rcand);
   a.n_nodes = o.n_nodes; a.tok = o.tok; a.parent = o.parent; a.depth = o.depth; a.sib_rank = o.sib_rank; a.logS = o.logS; a.q0 = o.q0; a.logqT = o.logqT;
   a.logkey = o.logkey; a.pop_rank = o.pop_rank; a.node_hash = o.node_hash; a.node_lseT = o.node_lseT; a.mask = o.mask; a.n_scored = o.n_scored; a.status = o.status;
   a.words = (c.Nmax + 63) / 64;

@@ -20,6 +20,7 @@ constexpr int TX_STAGE_MAX = 8;
 #ifndef TX_NW
 #define TX_NW 8
 #endif
+constexpr int TX_SOLO = 16;                // new parents whose seed bounds an owner makes itself
 constexpr int TX_PIECE = 1024;             // tokens of one scouting item
 
 // Everything the scan needs to know about one parent.
@@ -52,10 +53,11 @@ struct TreeArgs {
   uint32_t rk[20];       // round keys of the sampling generator
   // workspace
   ParentEntry* ent[2]; int* ent_slot[2];
-  int* lvl_count; unsigned* barrier; int* err;
+  int *lvl_count, *seed_need; unsigned* barrier; int* err;   // seed_need[d]: some owner left the seed bounds of its parents of depth d to all CTAs
   float4* sums;                                    // [cap][ntiles]: max reference, sum, tempered sum of every tile
   int* cand_cnt[2]; uint2 *cand_top, *cand_key; float* cand_lg;   // candidates per parent: (value, token), and the keys' logits
                                                                  // (counts by level parity: an owner clears the next level's while others still read this one's)
+  float2* res_lse; uint4* res_cand;                // merged results of a level with many parents: [cap], [cap][KMAX] (top token, logit, draw, logit)
   unsigned *thr, *slots; int cap;
   uint2* utop;                                     // [2][B][npiece] (given parents: [P][npiece]): best base logit of every piece of a row
   unsigned char* pool; size_t pool_stride;         // per request: PoolView
