@@ -832,7 +832,10 @@ __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s
 // (Inlined, once: behind a call the arguments would be read through generic addresses, some 40 cycles each.)
 // share >= 0: not the level step, but the seed bounds of every `step`-th of the new parents of request b, from the share-th
 // on (a request with many leaves them to the CTAs that own none); spread: the merge was done by all CTAs.
-__device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, const int b, const int d, const int share, const int step, const bool many, const bool spread) {
+template <bool MANY>
+__device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, const int b, const int d, const int share_, const int step, const bool spread_) {
+  const int share = MANY ? share_ : -1;
+  const bool spread = MANY && spread_;
   const OwnerSm s = owner_carve(sm, a);
   __shared__ int sh[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1165,7 +1168,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     for (int e0 = SEED_REGS * TX_THREADS; e0 < NS * a.r; e0 += SEED_REGS * TX_THREADS) { load_seed_columns(a, s, NS, e0, wcol); store_seed_columns(a, s, NS, e0, wcol); }
   __syncthreads();
   if (d >= 0 && share < 0) li0 = sh[6];
-  if (more && share < 0 && many && cnt > TX_SOLO) {   // many parents: entries without bounds; all CTAs make those after the next barrier
+  if (MANY && more && share < 0 && cnt > TX_SOLO) {   // many parents: entries without bounds; all CTAs make those after the next barrier
 #pragma unroll 1
     for (int i = tid; i < cnt; i += TX_THREADS) {
       uint4* dst = reinterpret_cast<uint4*>(a.ent[nxt] + li0 + i);
@@ -1253,6 +1256,9 @@ __device__ __forceinline__ void tx_finalize(const TreeArgs& a, unsigned char* sm
   __syncthreads();
 }
 
+// MANY: owners share the work on crowded levels with the CTAs that own no request (a second instantiation: the code costs
+// the scan of the other one's launches 4 %).
+template <bool MANY>
 __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_constant__ TreeArgs a, const __grid_constant__ CUtensorMap tmW) {
   extern __shared__ unsigned char raw[];
   unsigned char* base_sm = raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u);
@@ -1288,8 +1294,6 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
   BlockPos pos{0, 0u, 0u}, wpos{0, 0u, 0u};
   int groups = 0;
   const int nreq = a.score_P > 0 ? a.score_P : a.B;
-  const bool many = a.score_P == 0 && ncta >= 2 * a.B;   // several CTAs a request: they help owners with many parents
-  const int piece_len = (((a.V + a.npiece - 1) / a.npiece) + 7) & ~7;
 
   if (a.ragged) {   // W with padded rows (the bulk-tensor loads need rows of whole 16 bytes)
     const unsigned short* src = reinterpret_cast<const unsigned short*>(a.W);
@@ -1379,7 +1383,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
     }
     }
     // ---- merge by all CTAs where the owners alone would take long over it (8 requests with 60 parents each: 150 us) -------
-    const bool spread = many && d >= 0 && P > 8 * a.B;
+    const bool spread = MANY && d >= 0 && P > 8 * a.B;
     if (spread) {
       const int R = mma_replicas(P), K = a.K;
 #pragma unroll 1
@@ -1400,15 +1404,16 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
 #pragma unroll 1
     for (int turn = 0;; ++turn) {
       if (d >= -1) {
-        const int first = turn ? cta % nreq : cta, share = turn ? cta / nreq : -1, hstep = ncta / nreq;
-        if (share < hstep)
+        const int first = MANY && turn ? cta % nreq : cta, share = MANY && turn ? cta / nreq : -1, hstep = MANY ? ncta / nreq : 1;
+        if (!MANY || share < hstep)
 #pragma unroll 1
-          for (int b = first; b < nreq; b += turn ? nreq : ncta) tx_owner(a, base_sm, b, d, share, hstep, many, spread);
+          for (int b = first; b < nreq; b += MANY && turn ? nreq : ncta) tx_owner<MANY>(a, base_sm, b, d, share, hstep, spread);
       }
       // best base logits of the rows after the next ones, by the CTAs that own no request where there are enough of them
       // (given parents: of their rows, before anything else)
       if (turn == 0 && (d == -2 || (a.score_P == 0 && d + 2 < a.D))) {
         const int h0 = d >= -1 && ncta - a.B >= ncta / 4 ? a.B : 0;
+        const int piece_len = (((a.V + a.npiece - 1) / a.npiece) + 7) & ~7;
         uint2* ut = a.utop + (size_t)(d & 1) * a.B * a.npiece;
         if (cta >= h0)
 #pragma unroll 1
@@ -1422,7 +1427,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
       if (d + 1 >= a.D && a.score_P == 0) { over = true; break; }
       fence_async_smem();   // owners work in memory that the next scan's bulk loads may write
       if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
-      if (turn || d < 0 || !many || __ldcg(a.seed_need + d + 1) == 0) break;   // uniform: written before the barrier
+      if (!MANY || turn || d < 0 || __ldcg(a.seed_need + d + 1) == 0) break;   // uniform: written before the barrier
     }
     if (over || dead) break;
     if (d == -2 && a.ragged) asm volatile("fence.proxy.async;" ::: "memory");
@@ -1563,6 +1568,8 @@ static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream
   { ProfScope ps(ctx, K_INIT, st); e = launch_kernel(tree_init_kernel, 1, 64, 0, st, true, a.barrier, 8 + 2 * (DMAX + 2)); }
   if (e != cudaSuccess) return e;
   ProfScope ps(ctx, prof_id, st);
+  // crowded levels (a request with dozens of parents) need room for them in the tree and CTAs to spare
+  const void* fn = (a.score_P == 0 && ctx->num_sms >= 2 * a.B && a.N > 96) ? (const void*)tree_kernel<true> : (const void*)tree_kernel<false>;
   void* kargs[] = {(void*)&a, (void*)&tm};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctx->num_sms); cfg.blockDim = dim3(TX_THREADS); cfg.dynamicSmemBytes = ctx->tree.smem; cfg.stream = st;
@@ -1570,17 +1577,20 @@ static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream
   attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;   // grid barriers: every CTA resident
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = ctx->persist_pdl >= 0 ? 2 : 1;
-  e = cudaLaunchKernelExC(&cfg, (const void*)tree_kernel, kargs);
+  e = cudaLaunchKernelExC(&cfg, fn, kargs);
   if (e != cudaSuccess && cfg.numAttrs == 2) {   // not accepted together: remember, and launch cooperative only
     (void)cudaGetLastError();
     ctx->persist_pdl = -1;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelExC(&cfg, (const void*)tree_kernel, kargs);
+    e = cudaLaunchKernelExC(&cfg, fn, kargs);
   }
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t tree_setup(ts_ctx* ctx) { return cudaFuncSetAttribute(tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->tree.smem); }
+cudaError_t tree_setup(ts_ctx* ctx) {
+  const cudaError_t e = cudaFuncSetAttribute(tree_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->tree.smem);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(tree_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->tree.smem);
+}
 
 cudaError_t tree_score(ts_ctx* ctx, char* scratch, const void* U, const void* A, const void* W, int P, const int* p_req, const int* p_depth, const int* p_token,
                        const uint64_t* p_hash, float T, uint64_t seed, float* lse0, float* lseT, int* top_tok, float* top_logit, int* draw_tok,
