@@ -39,13 +39,6 @@ __device__ __forceinline__ void load16_bf16(const __nv_bfloat16* p, const bool w
     if (hi) b = __ldcg(reinterpret_cast<const uint4*>(p) + 1);
   }
 }
-// one lane of a converged warp (the instruction tells the compiler that the branch is uniform)
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
-
 // Shared-memory state of a CTA.
 struct TxSm {
   unsigned char *As, *Ws;

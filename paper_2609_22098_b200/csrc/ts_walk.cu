@@ -23,10 +23,10 @@
 namespace ts {
 
 constexpr int WK_EPI = 16;                 // warps that read accumulators: 4 lane quarters x 4 sets of tiles
-constexpr int WK_MMA = WK_EPI;             // issues the MMAs and, in the streaming form, requests W
+constexpr int WK_LOAD = WK_EPI;            // tensor memory; in the streaming form it requests W and issues the MMAs
 constexpr int WK_THREADS = (WK_EPI + 1) * 32;
 constexpr int WK_REQ = 64;                 // requests of one reduction pass (columns of a tile)
-constexpr int WK_BUF = 8;                  // accumulator buffers at most
+constexpr int WK_BUF = 8;                  // accumulator buffers of WK_REQ columns: two per set of tiles
 constexpr int WK_CHUNK = 1088;             // tokens of one step of the bonus rescan: 8 tokens x 136 places x 4 slices of the rank
 
 struct RedDesc { const __nv_bfloat16 *z, *u; float C, zoff, qoff; int b; };
@@ -211,58 +211,66 @@ __device__ __forceinline__ void wk_advance(const WalkArgs& a, WalkState& st, con
 }
 
 // ---- one reduction pass: sums of max(p - C q, 0) over this CTA's tokens for up to WK_REQ requests ---------------------------
-struct WkPos { BlockPos buf; uint32_t wreq, wuse; bool resident_seen; };
-
-// the issuing warp: W blocks of 128 tokens through their ring (streaming form), one MMA tile per block
-__device__ __forceinline__ bool wk_issue(const WalkArgs& a, const WalkSm& sm, const CUtensorMap* tm, const int ncol, const int nbuf, const int t0, const int tlen,
-                                         const uint32_t tmem_base, WkPos& ps) {
-  const int lane = threadIdx.x & 31, ntile = (tlen + 127) / 128, ksteps = (a.r + 15) / 16, rp = (a.r + 63) / 64 * 64;
-  const uint32_t slab = (uint32_t)rp * 128u;
-  const uint64_t bd = smem_desc(smem_u32(sm.Bs), 16u, 1024u);
-  auto request = [&](uint32_t limit) -> bool {   // blocks follow one another round the range, on into the next pass
-    for (; ps.wreq < limit; ++ps.wreq) {
-      const uint32_t slot = ps.wreq % (uint32_t)a.ring, use = ps.wreq / (uint32_t)a.ring;
-      if (use >= 1 && !__all_sync(0xFFFFFFFFu, wk_wait(sm.w_free + slot, (use - 1) & 1, a, sm.abort))) return false;
-      const int nb = (int)(ps.wreq % (uint32_t)ntile), ns = (tlen - nb * 128 > 64) ? 2 : 1;
-      if (lane == 0) {
+// The MMAs of one tile into accumulator buffer `buf`, W from slab pair `ws`; an elected lane of the calling warp.
+// Issuing costs about 70 cycles an instruction (400 a tile of rank 64; 600 from a branch on the lane instead of an elected one,
+// and 1200 beside busy warps): one warp for all nine tiles of a pass took longer than the sums, so where W is resident the
+// first warp of every set issues its set's tiles.
+__device__ __forceinline__ void wk_mma(const WalkArgs& a, const WalkSm& sm, const int ncol, const uint32_t ws, const uint32_t buf, const uint32_t tmem_base) {
+  const int ksteps = (a.r + 15) / 16;
+  const uint32_t slab = (uint32_t)((a.r + 63) / 64 * 64) * 128u;
+  tc_fence_after();
+  if (elect_one()) {
+    const uint64_t ad = smem_desc(smem_u32(sm.Ws) + 2u * ws * slab, slab, 1024u), bd = smem_desc(smem_u32(sm.Bs), 16u, 1024u);
+    const uint32_t idesc = wk_idesc(ncol), d = tmem_base + buf * (uint32_t)WK_REQ;
+#pragma unroll 4
+    for (int ks = 0; ks < ksteps; ++ks)
+      mma_bf16(d, ad + (uint64_t)(ks * 128), bd + (uint64_t)((ks >> 2) * (WK_REQ * 128 / 16) + (ks & 3) * 2), idesc, ks > 0 ? 1u : 0u);
+    mma_commit(sm.t_full + buf);
+    if (a.ring) mma_commit(sm.w_free + ws);
+  }
+  __syncwarp();
+}
+// a set's tile number `nt` (counted over all passes) waits until the buffer's tile before last is drained
+__device__ __forceinline__ bool wk_drained(const WalkArgs& a, const WalkSm& sm, const uint32_t buf, const uint32_t nt) {
+  return nt < 2u || __all_sync(0xFFFFFFFFu, wk_wait(sm.t_empty + buf, ((nt >> 1) - 1u) & 1u, a, sm.abort));
+}
+__device__ __forceinline__ bool wk_issue(const WalkArgs& a, const WalkSm& sm, const int ncol, const int t, const int set, const uint32_t nt, const bool first_pass, const uint32_t tmem_base) {
+  const uint32_t buf = (uint32_t)set * 2u + (nt & 1u);
+  if (first_pass && a.use_tma && !__all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + t, 0, a, sm.abort))) return false;
+  if (!wk_drained(a, sm, buf, nt)) return false;
+  wk_mma(a, sm, ncol, (uint32_t)t, buf, tmem_base);
+  return true;
+}
+// Streaming form, one warp: blocks of 128 tokens of W through the ring, one after the other round the range and on into the next
+// pass (W does not depend on which requests that sums), and the tiles in the same order.  (In order, and by one warp: a wait
+// for a parity tells a slot's turns apart only while the waiter follows every one of them.)
+__device__ __forceinline__ void wk_stream(const WalkArgs& a, const WalkSm& sm, const CUtensorMap* tm, const int ncol, const int t0, const int tlen, const uint32_t pass,
+                                          uint32_t& wreq, const uint32_t tmem_base) {
+  const int ntile = (tlen + 127) / 128;
+  const uint32_t slab = (uint32_t)((a.r + 63) / 64 * 64) * 128u, ring = (uint32_t)a.ring, w0 = pass * (uint32_t)ntile;
+  for (int t = 0; t <= ntile; ++t) {
+    for (const uint32_t upto = w0 + (uint32_t)t + ring; wreq < upto; ++wreq) {
+      const uint32_t slot = wreq % ring, use = wreq / ring;
+      if (use >= 1 && !__all_sync(0xFFFFFFFFu, wk_wait(sm.w_free + slot, (use - 1) & 1, a, sm.abort))) return;
+      const int nb = (int)(wreq % (uint32_t)ntile), ns = (tlen - nb * 128 > 64) ? 2 : 1;
+      if (elect_one()) {
         mbar_expect_tx(sm.w_full + slot, (uint32_t)ns * slab);
         for (int h = 0; h < ns; ++h) tma_load_box(sm.Ws + (size_t)(2 * slot + h) * slab, tm, t0 + nb * 128 + h * 64, 0, sm.w_full + slot);
       }
       __syncwarp();
     }
-    return true;
-  };
-  for (int t = 0; t < ntile; ++t, ps.buf.next(nbuf)) {
-    uint32_t ws = (uint32_t)t;
-    if (a.ring) {
-      if (!request(ps.wuse + (uint32_t)a.ring)) return false;
-      ws = ps.wuse % (uint32_t)a.ring;
-      if (!__all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + ws, (ps.wuse / (uint32_t)a.ring) & 1, a, sm.abort))) return false;
-    } else if (!ps.resident_seen && a.use_tma) {
-      if (!__all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + t, 0, a, sm.abort))) return false;
-    }
-    if (ps.buf.reused() && !__all_sync(0xFFFFFFFFu, wk_wait(sm.t_empty + ps.buf.slot, ps.buf.empty(), a, sm.abort))) return false;
-    tc_fence_after();
-    if (lane == 0) {
-      const uint64_t ad = smem_desc(smem_u32(sm.Ws) + 2u * ws * slab, slab, 1024u);
-      const uint32_t idesc = wk_idesc(ncol), d = tmem_base + (uint32_t)(ps.buf.slot * ncol);
-#pragma unroll 4
-      for (int ks = 0; ks < ksteps; ++ks)
-        mma_bf16(d, ad + (uint64_t)(ks * 128), bd + (uint64_t)((ks >> 2) * (WK_REQ * 128 / 16) + (ks & 3) * 2), idesc, ks > 0 ? 1u : 0u);
-      mma_commit(sm.t_full + ps.buf.slot);
-      if (a.ring) mma_commit(sm.w_free + ws);
-    }
-    __syncwarp();
-    if (a.ring) ++ps.wuse;
+    if (t == ntile) break;
+    const uint32_t x = w0 + (uint32_t)t, set = (uint32_t)t & 3u, nt = pass * (uint32_t)((ntile - (int)set + 3) / 4) + (uint32_t)(t >> 2), buf = set * 2u + (nt & 1u);
+    if (!__all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + x % ring, (x / ring) & 1, a, sm.abort))) return;
+    if (!wk_drained(a, sm, buf, nt)) return;
+    wk_mma(a, sm, ncol, x % ring, buf, tmem_base);
   }
-  ps.resident_seen = true;
-  return !a.ring || request(ps.wuse + (uint32_t)a.ring);   // W does not depend on which requests the next pass sums
 }
 
 // The scanning warps.  Per tile and eight requests a thread loads its token's target and base logit of every request (a
 // warp reads 64 contiguous bytes of each row), requested one group ahead.
-__device__ __forceinline__ bool wk_epilogue(const WalkArgs& a, const WalkSm& sm, const int nreq, const int ncol, const int nbuf, const int t0, const int tlen,
-                                            const uint32_t tmem_base, WkPos& ps, const RedDesc* desc, float* s_part) {
+__device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm, const int nreq, const int ncol, const int t0, const int tlen,
+                                            const uint32_t tmem_base, uint32_t& nt, const bool first_pass, const RedDesc* desc, float* s_part) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = warp & 3, set = warp >> 2;
   const int ntile = (tlen + 127) / 128, ng = (nreq + 7) / 8;
   const float zs = (1.f / a.T) * 1.4426950408889634f;   // exponentials as powers of two
@@ -284,26 +292,30 @@ __device__ __forceinline__ bool wk_epilogue(const WalkArgs& a, const WalkSm& sm,
       }
     }
   };
-  if (set < ntile) load(set, 0);
   bool alive = true;
-  for (int t = 0; t < ntile; ++t, ps.buf.next(nbuf)) {
-    if ((t & 3) != set || !alive) continue;
-    if (!__all_sync(0xFFFFFFFFu, wk_wait(sm.t_full + ps.buf.slot, ps.buf.full(), a, sm.abort))) { alive = false; continue; }
+  const bool issues = q == 0 && !a.ring;
+  if (issues) for (int k = 0; k < 2 && alive; ++k) if (set + 4 * k < ntile) alive = wk_issue(a, sm, ncol, set + 4 * k, set, nt + (uint32_t)k, first_pass, tmem_base);
+  if (set < ntile) load(set, 0);
+  for (int t = set; t < ntile && alive; t += 4, ++nt) {
+    const uint32_t buf = (uint32_t)set * 2u + (nt & 1u);
+    if (!__all_sync(0xFFFFFFFFu, wk_wait(sm.t_full + buf, (nt >> 1) & 1u, a, sm.abort))) { alive = false; break; }
     tc_fence_after();
     for (int g = 0; g < ng; ++g) {
       uint32_t acc[8];
       __syncwarp();   // (the tensor-memory load is a warp-wide instruction)
       asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                    : "=r"(acc[0]), "=r"(acc[1]), "=r"(acc[2]), "=r"(acc[3]), "=r"(acc[4]), "=r"(acc[5]), "=r"(acc[6]), "=r"(acc[7])
-                   : "r"(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ps.buf.slot * ncol + g * 8)) : "memory");
+                   : "r"(tmem_base + ((uint32_t)(q * 32) << 16) + buf * (uint32_t)WK_REQ + (uint32_t)(g * 8)) : "memory");
       float z[8], u[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) { z[i] = __uint_as_float((uint32_t)nz[i] << 16); u[i] = __uint_as_float((uint32_t)nu[i] << 16); }
       if (g + 1 < ng) load(t, g + 1); else if (t + 4 < ntile) load(t + 4, 0);
       tmem_ld_wait();
       float s[8];
+      const bool upper = nreq - g * 8 > 4;   // (late steps have a few requests: half a group)
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
+        if (i >= 4 && !upper) { s[i] = 0.f; continue; }
         const int j = min(g * 8 + i, nreq - 1);
         const float p = ex2_approx(fmaf(z[i], zs, desc[j].zoff));
         const float qq = ex2_approx(fmaf(__uint_as_float(acc[i]) + u[i], zs, desc[j].qoff));   // C == 0: qoff = -huge, the term vanishes
@@ -328,9 +340,9 @@ __device__ __forceinline__ bool wk_epilogue(const WalkArgs& a, const WalkSm& sm,
     }
     tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive(sm.t_empty + ps.buf.slot);
+    if (lane == 0) mbar_arrive(sm.t_empty + buf);
+    if (issues && t + 8 < ntile) alive = wk_issue(a, sm, ncol, t + 8, set, nt + 2u, first_pass, tmem_base);
   }
-  return alive;
 }
 
 // ---- the bonus token of one request whose walk is over, by the CTA that owns it ----------------------------------------------
@@ -492,7 +504,7 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
   sm.t_full = bars; sm.t_empty = bars + WK_BUF; sm.w_full = bars + 2 * WK_BUF; sm.w_free = sm.w_full + 32;
   sm.tmem = reinterpret_cast<uint32_t*>(sm.w_free + 8); sm.abort = reinterpret_cast<volatile int*>(sm.tmem + 1);
   sm.st = reinterpret_cast<WalkState*>(bars + 64);
-  if (warp == WK_MMA) {
+  if (warp == WK_LOAD) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(sm.tmem)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -539,7 +551,7 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
   unsigned gen = 0;
   const unsigned nexpect = (unsigned)ncta + (a.lost_arrival ? 1u : 0u);
   bool dead = false, finished = false;
-  WkPos ps{{0, 0u, 0u}, 0u, 0u, false};
+  uint32_t nt = 0u, wreq = 0u, pass = 0u;   // tiles of this warp's set and W blocks requested, over all passes
   for (int step = 0; !dead && step < a.max_steps; ++step) {
     if (warp < WK_EPI)
       for (int i = warp; i < nown; i += WK_EPI) wk_advance(a, sm.st[i], cta + i * ncta, lane, step + 1);
@@ -570,20 +582,27 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
         __syncthreads();
       }
       if (nwk == 0) break;
-      const int nreq = min(WK_REQ, nwk - sb), ncol = (nreq + 15) & ~15, nbuf = min(WK_BUF, 512 / ncol);
+      const int nreq = min(WK_REQ, nwk - sb), ncol = (nreq + 15) & ~15;
       // head rows of the requests' nodes: the B operand, K-major with the 128-byte swizzle
       for (int idx = tid; idx < nreq * (a.r / 8); idx += WK_THREADS) {
         const int g = idx / (a.r / 8), ck = idx - g * (a.r / 8);
         *reinterpret_cast<uint4*>(sm.Bs + (ck >> 3) * (WK_REQ * 128) + g * 128 + (((ck & 7) ^ (g & 7)) << 4)) =
             __ldg(reinterpret_cast<const uint4*>(a.A + (size_t)s_tok[g] * a.r + ck * 8));
       }
+      // ask L2 for this range of the rows that will be read
+      for (int x = warp; x < 2 * nreq; x += WK_THREADS / 32) {
+        const RedDesc& d = s_desc[x >> 1];
+        const __nv_bfloat16* src = ((x & 1) ? d.u : d.z) + t0;
+        if (!(x & 1) || d.C != 0.f)
+          for (int l = lane * 64; l < tlen; l += 32 * 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + l));
+      }
       fence_async_smem();
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
-      ps.buf.slot = 0;
-      if (warp < WK_EPI) wk_epilogue(a, sm, nreq, ncol, nbuf, t0, tlen, tmem_base, ps, s_desc, s_part);
-      else wk_issue(a, sm, &tmW, ncol, nbuf, t0, tlen, tmem_base, ps);
+      if (warp < WK_EPI) wk_epilogue(a, sm, nreq, ncol, t0, tlen, tmem_base, nt, pass == 0u, s_desc, s_part);
+      else if (a.ring) wk_stream(a, sm, &tmW, ncol, t0, tlen, pass, wreq, tmem_base);
+      ++pass;
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
@@ -600,8 +619,8 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
     if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
   }
   // ---- no bulk load may still be writing this CTA's shared memory (waits bounded) -----------------------------------------
-  if (warp == WK_MMA && lane == 0 && a.use_tma) {
-    const uint32_t lo = a.ring ? ps.wuse : 0u, hi = a.ring ? ps.wreq : (uint32_t)ntile;
+  if (warp == WK_LOAD && lane == 0 && a.use_tma) {
+    const uint32_t lo = a.ring ? (wreq > (uint32_t)a.ring ? wreq - (uint32_t)a.ring : 0u) : 0u, hi = a.ring ? wreq : (uint32_t)ntile;
     for (uint32_t x = lo; x < hi; ++x) {
       uint64_t* bar = sm.w_full + (a.ring ? x % (uint32_t)a.ring : x);
       const uint32_t par = a.ring ? (x / (uint32_t)a.ring) & 1u : 0u;
@@ -617,7 +636,7 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == WK_MMA) {
+  if (warp == WK_LOAD) {
     __syncwarp();
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
