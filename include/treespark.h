@@ -91,16 +91,12 @@ int32_t ts_set_ablation(ts_ctx* ctx, uint32_t flags);
  *   TS_TEST_FORCE_FMA     bf16 inputs run on the fp32 fused-multiply-add kernels (no tensor cores)
  *   TS_TEST_NO_TMA        the tensor-core kernels stage W with plain loads (no tensor map)
  *   TS_TEST_NO_FEW        levels with few parents run on the tile kernel too
- *   TS_TEST_NO_SEED       the tensor-core scoring kernel runs without seed bounds (no seed kernel ahead of it)
- *   TS_TEST_PERSIST       ts_expand_tree runs every level inside one cooperative launch (scan, merge and level
- *                         step separated by grid barriers; nothing is launched for empty levels) instead of one
- *                         launch per step of every level, where the configuration fits that kernel
- *   TS_TEST_NO_TAIL       ts_expand_tree launches every level's kernels one by one up to the last level, instead of
- *                         handing the levels from the fifth on (mostly empty) to one cooperative launch
- *   TS_TEST_NO_UMMA       the scanning threads of the tensor-core scoring kernel load the base logits themselves
- *                         instead of receiving them through the MMA (the path of batches above 32 requests)
+ *   TS_TEST_NO_SEED       the tensor-core scoring kernel runs without seed bounds
+ *   TS_TEST_PERSIST, TS_TEST_NO_TAIL, TS_TEST_NO_UMMA
+ *                         accepted without effect: they chose between forms of the tensor-core expansion, which now
+ *                         has one form (a single cooperative launch for all levels)
  *   TS_TEST_SHORT_WAITS   bounded waits give up after 4096 polls instead of 2^22
- *   TS_TEST_LOST_ARRIVAL  the walk's grid barriers and the scoring kernel's operand barrier expect one
+ *   TS_TEST_LOST_ARRIVAL  the grid barriers of the walk and of the tensor-core scoring kernel expect one
  *                         arrival more than will come: the waits run out, the kernels return, and the
  *                         requests are reported with TS_ERR_TIMEOUT in status[] */
 #define TS_TEST_FORCE_FMA 1u

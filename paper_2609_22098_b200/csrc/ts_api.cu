@@ -46,16 +46,17 @@ static bool choose_tile(const ts_config& c, int num_sms, int max_smem, TileCfg* 
 static bool select_paths(ts_ctx* ctx) {
   const ts_config& c = ctx->cfg;
   const unsigned tm = ctx->test_mode;
-  // tensor cores for bf16 inputs whose rows allow 16-byte chunks; the fp32 FMA kernel otherwise
-  ctx->use_mma = (c.dt_U == TS_DTYPE_BF16 && c.r % 8 == 0 && c.V % 8 == 0 && ctx->cc_major == 10 && !(tm & TS_TEST_FORCE_FMA)) ? 1 : 0;
   ctx->tma_state = (tm & TS_TEST_NO_TMA) ? -1 : 0;
-  ctx->tmapW_ptr = nullptr;
-  if (ctx->use_mma && !choose_tile_mma(c, ctx->num_sms, ctx->max_smem, !(tm & TS_TEST_NO_TMA), &ctx->tile)) ctx->use_mma = 0;
-  if (!ctx->use_mma && !choose_tile(c, ctx->num_sms, ctx->max_smem, &ctx->tile)) return false;
-  ctx->use_tree = (c.dt_U == TS_DTYPE_BF16 && c.r % 8 == 0 && ctx->cc_major == 10 && !(tm & TS_TEST_FORCE_FMA) &&
-                   tree_plan(c, ctx->num_sms, ctx->max_smem, &ctx->tree)) ? 1 : 0;
-  ctx->tmapT_ptr = nullptr;
-  ctx->use_walk = (c.dt_U == TS_DTYPE_BF16 && c.r % 8 == 0 && ctx->cc_major == 10 && !(tm & TS_TEST_FORCE_FMA)) ? 1 : 0;
+  ctx->tmapW_ptr = ctx->tmapT_ptr = nullptr;
+  // tensor cores for bf16 inputs whose rows allow 16-byte chunks; the fp32 FMA kernels otherwise
+  const bool tc = c.dt_U == TS_DTYPE_BF16 && c.r % 8 == 0 && ctx->cc_major == 10 && !(tm & TS_TEST_FORCE_FMA);
+  ctx->use_walk = tc ? 1 : 0;
+  ctx->use_tree = (tc && tree_plan(c, ctx->num_sms, ctx->max_smem, &ctx->tree)) ? 1 : 0;
+  // (a context of the tensor-core kernel needs the tile only to score ragged vocabularies without a workspace)
+  if (!choose_tile(c, ctx->num_sms, ctx->max_smem, &ctx->tile)) {
+    if (!ctx->use_tree) return false;
+    ctx->tile = TileCfg{};
+  }
   ctx->few_cap = (tm & TS_TEST_NO_FEW) ? 0 : few_capacity(c);
   ctx->wait_limit = (tm & TS_TEST_SHORT_WAITS) ? 4096u : WAIT_LIMIT;
   return true;
@@ -168,7 +169,7 @@ extern "C" size_t ts_workspace_bytes(const ts_ctx* ctx, int32_t batch) {
 
 static const char* kKernelNames[K_COUNT] = {"expand_init", "score_tile", "score_merge", "expand_level", "expand_finalize",
                                             "zrow_stats", "verify_greedy", "verify_walk", "verify_check", "score_few", "allocate_select", "allocate_cut",
-                                            "calib_accumulate", "calib_refit", "attention_inputs", "score_seed", "expand_persistent"};
+                                            "calib_accumulate", "calib_refit", "attention_inputs", "expand_persistent"};
 
 extern "C" const char* ts_kernel_name(int32_t id) { return (id >= 0 && id < K_COUNT) ? kKernelNames[id] : nullptr; }
 

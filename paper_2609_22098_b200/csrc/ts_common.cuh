@@ -26,14 +26,8 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 // these words with atomicMax in the launch's first microseconds; packed together they queue up on a
 // handful of L2 lines (measured: a third of the scoring launch at stride 1).
 constexpr int SLOT_STRIDE = 32;
-// Seed kernel: a parent's base-logit row is swept by up to SEED_PARTS_MAX CTAs when there are few parents;
-// the parts of at most SEED_SPLIT_PARENTS parents meet in a scratch of NSEED_MAX candidates per part.
-constexpr int SEED_PARTS_MAX = 16, SEED_SPLIT_PARENTS = 256, NSEED_MAX = 32;
-constexpr size_t SEED_CAND_WORDS = (size_t)SEED_SPLIT_PARENTS * SEED_PARTS_MAX * NSEED_MAX * 2;
-constexpr int UMMA_REQ = 32;         // requests whose base logits can ride through the tensor cores (rows of one extra B-operand slab)
 constexpr int SCORE_THREADS = 128;   // one parent per thread; every thread scans the CTA's whole tile
 constexpr int CHUNK = 16;            // tokens per coarse generator call
-constexpr int MMA_S = 4;             // column splits per tile in the tensor-core scoring kernel (scanning warps per row quarter)
 
 enum Stream : uint32_t { STREAM_GUMBEL_COARSE = 1, STREAM_GUMBEL_FINE = 2, STREAM_ACCEPT = 3, STREAM_BONUS = 4 };
 
@@ -50,8 +44,6 @@ struct TileCfg {
   int TV;       // tokens per vocabulary tile (multiple of 64)
   int ntiles;   // tiles covering V
   size_t smem;  // dynamic shared memory of the scoring kernel
-  int umma;     // the tiling leaves room for the one-hot slab and the base-logit slab ring (base logits through the MMA)
-  int w_ring;   // 0: the W tile is resident; > 0: that many 64-token slabs of W stream through a ring (large ranks)
 };
 
 // Shared-memory and vocabulary plan of the one-launch expansion (ts_tree.cu).
@@ -79,7 +71,6 @@ struct ts_ctx {
   int use_walk;     // 1: the walk's reductions may run on the tensor cores
   int use_tree;     // 1: expansion and scoring run on the one-launch tensor-core kernel
   int vt_TV, vt_n;  // vocabulary ranges of the verification walk, one per CTA
-  int use_mma;      // 1: scoring runs on the tensor-core kernel, 0: on the fp32 FMA kernel
   int few_cap;      // levels with at most this many parents run on the few-parents kernel instead (0: none)
   ts::DevCalib calib;
   void* prof;  // ts::Prof*, instrumentation state
@@ -89,11 +80,9 @@ struct ts_ctx {
   const void* tmapW_ptr;
   alignas(64) unsigned char tmapT[128];   // the one-launch kernel's tensor map of W (boxes of 64 tokens x r rows)
   const void* tmapT_ptr;
-  alignas(64) unsigned char tmapU[128];   // tensor map of the base logits last expanded with ([request][depth][token] boxes)
-  const void* tmapU_ptr; int tmapU_B;
   int tma_state;   // 0 not tried yet, 1 encoder found, -1 unavailable
   int walk_pdl;    // -1: the driver refused a cooperative launch with programmatic serialization
-  int persist_pdl; // the same for the persistent expansion kernel
+  int tree_pdl;    // the same for the one-launch expansion
   unsigned ablation;   // TS_ABLATE_* switches (0 = the method)
   unsigned test_mode;  // TS_TEST_* switches (0 = the product's kernel selection and wait limits)
   uint32_t wait_limit; // polls before a bounded device-side wait gives up
@@ -106,16 +95,13 @@ namespace ts {
 // ------------------------------------------------------------------------------------------------
 struct WsLayout {
   int B, N, K, Pcap, ntiles, words;
-  // scoring records, [ntiles * S][rec_cap][rec_words]
+  // scoring records, [ntiles][rec_cap][rec_words]
   size_t rec; int rec_cap;
-  size_t err;            // int[4]: error word raised by a bounded wait inside the scoring kernel
   // merged per-parent results of the level being expanded, [Pcap] / [Pcap][K]
   size_t res_lse0, res_lseT, res_top_tok, res_top_logit, res_draw_tok, res_draw_logit;
   // level parent lists (two, alternating) [Pcap]
   size_t lst_req[2], lst_depth[2], lst_token[2], lst_hash[2], lst_slot[2];
   size_t lvl_count;      // int[DMAX + 2]
-  size_t ex_barrier;     // unsigned[4]: grid barrier of the persistent expansion kernel
-  size_t utop;           // uint2[B][D][ntiles]: best base logit (value, token) of every vocabulary tile of every row
   // per-request pool, [B][N]
   size_t pl_alive, pl_depth, pl_parent, pl_sib, pl_tok, pl_lidx, pl_new, pl_logkey, pl_logS, pl_q0, pl_logqT,
       pl_lseT, pl_hash, pl_path;
@@ -180,13 +166,8 @@ __host__ inline WsLayout make_layout(const ts_ctx* ctx, int B) {
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   const size_t P = (size_t)L.Pcap, K = (size_t)c.K, N = (size_t)c.Nmax, b = (size_t)B;
-  {
-    int cap = (L.Pcap + 7) / 8 * 8;
-    if (ctx->use_mma) cap = (L.Pcap + 127) / 128 * 128;
-    L.rec_cap = cap;
-    L.rec = take(record_bytes(ctx, cap) + ((size_t)cap * (4 + 2 * K * SLOT_STRIDE) + SEED_SPLIT_PARENTS + SEED_CAND_WORDS) * 4);
-    L.err = take(16);
-  }
+  L.rec_cap = (L.Pcap + 7) / 8 * 8;
+  L.rec = take(record_bytes(ctx, L.rec_cap) + 2 * (size_t)L.rec_cap * K * SLOT_STRIDE * 4);
   L.res_lse0 = take(P * 4); L.res_lseT = take(P * 4);
   L.res_top_tok = take(P * K * 4); L.res_top_logit = take(P * K * 4);
   L.res_draw_tok = take(P * K * 4); L.res_draw_logit = take(P * K * 4);
@@ -195,8 +176,6 @@ __host__ inline WsLayout make_layout(const ts_ctx* ctx, int B) {
     L.lst_hash[i] = take(P * 8); L.lst_slot[i] = take(P * 4);
   }
   L.lvl_count = take((DMAX + 2) * 4);
-  L.ex_barrier = take(64);
-  L.utop = take(b * (size_t)c.D * (size_t)ctx->tile.ntiles * 8);
   L.pl_alive = take(b * N * 4); L.pl_depth = take(b * N * 4); L.pl_parent = take(b * N * 4);
   L.pl_sib = take(b * N * 4); L.pl_tok = take(b * N * 4); L.pl_lidx = take(b * N * 4); L.pl_new = take(b * N * 4);
   L.pl_logkey = take(b * N * 8); L.pl_logS = take(b * N * 8); L.pl_q0 = take(b * N * 4);

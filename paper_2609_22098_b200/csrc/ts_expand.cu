@@ -20,12 +20,8 @@ __global__ void expand_init_kernel(ExpandArgs a) {
   pdl_wait();                // whatever ran before in the stream may still be reading what this kernel resets
   pdl_launch_dependents();   // the first scoring launch may run its preamble beside this kernel
   const int b = blockIdx.x;
-  // pruning state of the scoring launches: the threshold words, then one word per slot (the slots sit
-  // SLOT_STRIDE words apart; only the first word of each is ever used)
-  for (int i = b * blockDim.x + threadIdx.x; i < a.thr_words; i += gridDim.x * blockDim.x)
-    a.thr[i < a.thr_head ? i : a.thr_head + (size_t)(i - a.thr_head) * SLOT_STRIDE] = 0u;
-  if (b == 0) for (int i = threadIdx.x; i < SEED_SPLIT_PARENTS; i += blockDim.x) a.seed_cnt[i] = 0u;
-  if (b == 0 && threadIdx.x < 4) a.ex_barrier[threadIdx.x] = 0u;
+  // pruning slots of the scoring launches (SLOT_STRIDE words apart; only the first word of each is ever used)
+  for (int i = b * blockDim.x + threadIdx.x; i < a.nslots; i += gridDim.x * blockDim.x) a.slots[(size_t)i * SLOT_STRIDE] = 0u;
   if (b >= a.B) return;
   for (int s = threadIdx.x; s < a.N; s += blockDim.x) a.pl_alive[(size_t)b * a.N + s] = 0;
   if (threadIdx.x == 0) {
@@ -37,7 +33,6 @@ __global__ void expand_init_kernel(ExpandArgs a) {
     a.req_npar[b] = 1; a.req_base[b] = b; a.req_nscored[b] = 0;
     a.root_lseT[b] = nanf("");
     if (b == 0) {
-      a.err[0] = 0;
       a.lvl_count[0] = a.B;
       for (int d = 1; d <= DMAX + 1; ++d) a.lvl_count[d] = 0;
     }
@@ -45,12 +40,12 @@ __global__ void expand_init_kernel(ExpandArgs a) {
 }
 
 // One CTA per request; level d = depth of the parents just scored (body in ts_level.cuh).
-__global__ void __launch_bounds__(LEVEL_THREADS) expand_level_kernel(ExpandArgs a, int d, int seed_next) {
+__global__ void __launch_bounds__(LEVEL_THREADS) expand_level_kernel(ExpandArgs a, int d) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ LevelSmem sm;
   pdl_wait();               // merged scoring results of this level
   pdl_launch_dependents();
-  level_step(a, d, seed_next, (int)blockIdx.x, sm, sm_raw, (int)threadIdx.x, [] { __syncthreads(); });
+  level_step(a, d, (int)blockIdx.x, sm, sm_raw, (int)threadIdx.x, [] { __syncthreads(); });
 }
 
 struct FinalArgs {
@@ -60,7 +55,6 @@ struct FinalArgs {
   const float* root_lseT; const int* req_nscored;
   int *n_nodes, *tok, *parent, *depth, *sib_rank; float *logS, *q0, *logqT, *logkey; int* pop_rank;
   uint64_t* node_hash; float* node_lseT; uint64_t* mask; int* n_scored;
-  const int* err; int* status;   // a bounded wait that ran out during the expansion is reported for every request still marked fine
 };
 
 // Canonical (BFS) renumbering, outputs and ancestor bitmasks; one CTA per request.
@@ -110,7 +104,6 @@ __global__ void __launch_bounds__(256) expand_finalize_kernel(FinalArgs a) {
     a.parent[pb + s_canon[s]] = cp;
   }
   if (tid == 0) {
-    if (*reinterpret_cast<const volatile int*>(a.err) != 0 && a.status[b] == TS_OK) a.status[b] = TS_ERR_TIMEOUT;
     a.n_nodes[b] = s_n;
     a.node_hash[(size_t)b * (N + 1)] = 0ull;
     if (a.node_lseT) a.node_lseT[(size_t)b * (N + 1)] = a.root_lseT[b];
@@ -132,14 +125,8 @@ __global__ void __launch_bounds__(256) expand_finalize_kernel(FinalArgs a) {
 }
 
 // the level kernel ranks a request's pool and candidates out of dynamic shared memory: opt in once per context
-// dynamic shared memory of the level kernel: the ranking entries of a request's pool and candidates, later
-// reused for the seed bounds' staged W columns [2K][r], per-pair results [Nmax][2K][2] and a batch of rows of A
-size_t level_smem_bytes(const ts_config& c) {
-  const size_t entries = (size_t)(c.Nmax + c.Nmax * c.K) * sizeof(Entry);
-  const size_t ns = (size_t)(2 * c.K > NSEED_MAX ? NSEED_MAX : (2 * c.K < 8 ? 8 : 2 * c.K));
-  const size_t seeds = ns * (size_t)(c.r + 1) * 4 + (size_t)c.Nmax * ns * 2 * 4 + (size_t)SEED_PBATCH * c.r * 2;
-  return entries > seeds ? entries : seeds;
-}
+// dynamic shared memory of the level kernel: the ranking entries of a request's pool and candidates
+size_t level_smem_bytes(const ts_config& c) { return (size_t)(c.Nmax + c.Nmax * c.K) * sizeof(Entry); }
 
 cudaError_t expand_setup(ts_ctx* ctx) {
   const size_t level_smem = level_smem_bytes(ctx->cfg);
@@ -202,84 +189,25 @@ extern "C" int32_t ts_expand_tree(ts_ctx* ctx, const void* U, const void* A, con
   a.cd_valid = (int*)(ws + L.cd_valid); a.cd_parent = (int*)(ws + L.cd_parent); a.cd_sib = (int*)(ws + L.cd_sib);
   a.cd_tok = (int*)(ws + L.cd_tok); a.cd_logkey = (double*)(ws + L.cd_logkey); a.cd_logS = (double*)(ws + L.cd_logS);
   a.cd_q0 = (float*)(ws + L.cd_q0); a.cd_logqT = (float*)(ws + L.cd_logqT); a.cd_rank = (int*)(ws + L.cd_rank);
-  a.status = status; a.err = (int*)(ws + L.err);
-  a.thr = thr_base(ctx, (float*)(ws + L.rec), L.rec_cap);
-  a.thr_head = 2 * L.rec_cap; a.thr_words = a.thr_head + 2 * L.rec_cap * c.K;   // words to clear, not their span
-  a.thr0 = a.thr + 2 * (size_t)L.rec_cap + 2 * (size_t)L.rec_cap * c.K * SLOT_STRIDE;
-  a.seed_cnt = a.thr0 + 2 * (size_t)L.rec_cap;
-  a.U = U; a.A = A; a.W = W; a.r = c.r; a.ntiles = ctx->tile.ntiles; a.cap = L.rec_cap; a.seed = seed;
-  a.utop = (const uint2*)(ws + L.utop);
-  a.ex_barrier = (unsigned*)(ws + L.ex_barrier);
+  a.status = status;
+  a.slots = thr_base(ctx, (float*)(ws + L.rec), L.rec_cap); a.nslots = 2 * L.rec_cap * c.K;
 
   cudaError_t e0;
   { ProfScope ps(ctx, K_INIT, st); e0 = launch_kernel(expand_init_kernel, B > 296 ? B : 296, 256, 0, st, true, a); }
   cudaError_t e = e0 != cudaSuccess ? e0 : cudaGetLastError();
   if (e != cudaSuccess) return set_cuda_error("ts_expand_tree(init)", e);
   const size_t level_smem = level_smem_bytes(c);   // opted into at ts_create when above 48 KB
-  const bool seeds_on = ctx->use_mma && !(ctx->test_mode & TS_TEST_NO_SEED);
-  // Three forms.  Default: one launch per step of every level (score, merge, level step), chained, for the first
-  // TAIL_FROM levels, and one cooperative launch for all levels after those: trees usually end before them, and
-  // three launches per empty level (each a hop in the chain of dependent launches) become one that returns at once.
-  // TS_TEST_PERSIST: the cooperative launch runs every level.  TS_TEST_NO_TAIL: no cooperative launch at all.
-  constexpr int TAIL_FROM = 4;
-  int coop_from = c.D;   // first level of the cooperative launch (D: none)
-  if (seeds_on && (ctx->test_mode & TS_TEST_PERSIST) && persistent_supported(ctx, B, 0)) coop_from = 0;
-  else if (seeds_on && !(ctx->test_mode & TS_TEST_NO_TAIL)) {
-    // (a handful of requests rarely has parents at the fourth level either: one level earlier there)
-    const int from = TAIL_FROM;
-    if (c.D > from + 1 && persistent_supported(ctx, B, from)) coop_from = from;
-  }
   long long level_bound = B;   // parents a level can have at most: B at the root, K times more per level, B * Nmax overall
-  // Seed bounds of a level on the tensor-core kernel: made by the level kernel before it when that level's scoring
-  // launch scouted the rows (it does whenever it runs on the tensor-core kernel itself); by a seed launch otherwise
-  // (the root level, and the first tensor-core level after levels on the few-parents kernel).
-  bool scouted_prev = false;
-  for (int d = 0; d < coop_from; ++d) {
+  for (int d = 0; d < c.D; ++d) {
     const int cur = d & 1;
-    const bool on_mma = ctx->use_mma != 0;
-    ScoreExtras ex;
-    ex.thr0_ready = scouted_prev;
-    ex.root_B = d == 0 ? B : 0;
-    const bool scout = seeds_on && on_mma && d + 1 < c.D;
-    ex.u_depth = d; ex.u_B = B;
-    if (scout) { ex.utop = (uint2*)(ws + L.utop); ex.scout_live = a.req_npar; ex.scout_B = B; ex.scout_depth = d + 1; }
-    e = launch_score(ctx, (float*)(ws + L.rec), L.rec_cap, (int*)(ws + L.err), U, A, W, 0, a.lvl_count + d,
-                     a.lst_req[cur], a.lst_depth[cur], a.lst_token[cur],
+    e = launch_score(ctx, (float*)(ws + L.rec), L.rec_cap, U, A, W, 0, a.lvl_count + d, a.lst_req[cur], a.lst_depth[cur], a.lst_token[cur],
                      a.lst_hash[cur], T, seed, res_lse0, res_lseT, res_top_tok, res_top_logit, res_draw_tok,
-                     res_draw_logit, st, /*pdl=*/true, d > 0 ? a.lvl_count + d - 1 : nullptr, (int)level_bound, &ex);
+                     res_draw_logit, st, /*pdl=*/true, (int)level_bound);
     level_bound = level_bound * c.K < (long long)B * c.Nmax ? level_bound * c.K : (long long)B * c.Nmax;
     if (e != cudaSuccess) return set_cuda_error("ts_expand_tree(score)", e);
-    { ProfScope ps(ctx, K_LEVEL, st); e = launch_kernel(expand_level_kernel, B, LEVEL_THREADS, level_smem, st, true, a, d, scout ? 1 : 0); }
-    scouted_prev = scout;
+    { ProfScope ps(ctx, K_LEVEL, st); e = launch_kernel(expand_level_kernel, B, LEVEL_THREADS, level_smem, st, true, a, d); }
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return set_cuda_error("ts_expand_tree(level)", e);
-  }
-  if (coop_from < c.D) {
-    // One cooperative launch runs the remaining levels: scan, merge, level step, separated by grid barriers.  Its
-    // first level's seed bounds come from a seed launch (the root level) or from the level kernel before it.
-    ScoreArgs sa = make_score_args(ctx, (float*)(ws + L.rec), L.rec_cap, (int*)(ws + L.err), U, A, W, T, seed);
-    sa.pdl = 1; sa.P = 0; sa.P_dev = a.lvl_count + coop_from;
-    sa.P_prev_dev = coop_from > 0 ? a.lvl_count + coop_from - 1 : nullptr;
-    const int cur = coop_from & 1;
-    sa.p_req = a.lst_req[cur]; sa.p_depth = a.lst_depth[cur]; sa.p_token = a.lst_token[cur]; sa.p_hash = a.lst_hash[cur];
-    set_seed_pointers(ctx, sa);
-    if (coop_from == 0) {
-      ProfScope ps(ctx, K_SEED, st);
-      e = launch_seed(ctx, sa, st);
-      if (e != cudaSuccess) return set_cuda_error("ts_expand_tree(seed)", e);
-    }
-    sa.utop = (uint2*)(ws + L.utop); sa.scout_live = a.req_npar; sa.scout_B = B; sa.scout_depth = coop_from + 1;
-    sa.u_depth = coop_from; sa.u_B = B;
-    PersistArgs pa{};
-    pa.on = 1; pa.first = coop_from; pa.nlevels = c.D; pa.ex = a; pa.barrier = a.ex_barrier;
-    pa.lost_arrival = (ctx->test_mode & TS_TEST_LOST_ARRIVAL) ? 1 : 0;
-    MergeArgs& m = pa.mg;
-    m.pdl = 0; m.few_ntiles = 0; m.P = 0; m.P_dev = nullptr; m.K = c.K; m.ntiles = sa.ntiles; m.cap = L.rec_cap; m.S = 1; m.mma = 1; m.T = T;
-    m.rec = sa.rec; m.thr = sa.thr; m.slots = sa.slots; m.thr0 = sa.thr0;
-    m.lse0 = res_lse0; m.lseT = res_lseT; m.top_tok = res_top_tok; m.top_logit = res_top_logit; m.draw_tok = res_draw_tok;
-    m.draw_logit = res_draw_logit;
-    { ProfScope ps(ctx, K_PERSIST, st); e = launch_expand_persistent(ctx, sa, pa, st); }
-    if (e != cudaSuccess) return set_cuda_error("ts_expand_tree(cooperative)", e);
   }
   FinalArgs f{};
   f.B = B; f.N = c.Nmax; f.words = L.words;
@@ -288,7 +216,7 @@ extern "C" int32_t ts_expand_tree(ts_ctx* ctx, const void* U, const void* A, con
   f.pl_hash = a.pl_hash; f.pl_path = a.pl_path; f.root_lseT = a.root_lseT; f.req_nscored = a.req_nscored;
   f.n_nodes = n_nodes; f.tok = tok; f.parent = parent; f.depth = depth; f.sib_rank = sib_rank; f.logS = logS; f.q0 = q0;
   f.logqT = logqT; f.logkey = logkey; f.pop_rank = pop_rank; f.node_hash = node_hash; f.node_lseT = node_lseT;
-  f.mask = mask; f.n_scored = n_scored; f.err = a.err; f.status = status;
+  f.mask = mask; f.n_scored = n_scored;
   { ProfScope ps(ctx, K_FINAL, st); e = launch_kernel(expand_finalize_kernel, B, 256, 0, st, true, f); }
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return set_cuda_error("ts_expand_tree(finalize)", e);

@@ -22,47 +22,27 @@ struct ScoreArgs {
   const void *U, *A, *W;
   int V, D, r, K;
   int P; const int* P_dev;
-  const int* P_prev_dev;   // parent count of the previous level (nullptr: none); 0 there means 0 here
-  int w_ring;              // tensor-core kernel: 0 = resident W tile, > 0 = slabs of the W ring (streaming form)
-  int seed_root_B;         // seed kernel: > 0 = the parents are the roots of that many requests (parent p = request p at depth 0)
   int pdl;                 // host side: launch with programmatic stream serialization
-  int few;                 // host side: this launch runs on the few-parents kernel
-  int few_cap;             // parents its records have room for
+  int few_cap;             // parents the few-parents kernel's records have room for
   const int *p_req, *p_depth, *p_token; const uint64_t* p_hash;
   float T; uint64_t seed;
-  int TV, ntiles, cap, S;
-  float* rec; int* err;
-  unsigned* thr;    // [2][cap]: launch-wide lower bounds (logit, key) per parent, order-preserving encoding
-  unsigned* slots;  // [2][cap][K]
-  // Scouting for the next level (expansion only; utop == nullptr: none): while its first MMAs are on their
-  // way, the tensor-core kernel finds the best base logit of its vocabulary tile in row U[b][scout_depth] of
-  // every request b < scout_B that has parents in this launch (scout_live[b] > 0), and leaves (value, token)
-  // at utop[(b * D + scout_depth) * ntiles + tile]: the next level's seed bounds are made from those.
-  const int* scout_live; int scout_B, scout_depth; uint2* utop;
-  // Base logits through the tensor cores (expansion only, at most UMMA_REQ requests): all parents of the launch
-  // sit at depth u_depth (-1: not so; the persistent form takes the level instead), and the base logits of
-  // requests 0 .. u_B-1 at that depth enter the MMA as extra rows of the B operand against one-hot columns of
-  // the A operand, fetched by bulk-tensor loads: the scanning threads load no base logits at all.
-  int u_depth, u_B;
-  unsigned* seed_cnt;    // [SEED_SPLIT_PARENTS] arrival counters of the seed kernel (zero between launches)
-  unsigned* seed_cand;   // [SEED_SPLIT_PARENTS][SEED_PARTS_MAX][NSEED_MAX][2] candidates (value, token) of the parts
-  unsigned* thr0;   // [2][cap]: seed bounds (logit, key) per parent, written ahead of the launch; nullptr: none
-  uint32_t wait_limit;   // polls before a bounded device-side wait gives up
-  int lost_arrival;      // test switch: the A-tile barrier expects one arrival more than will come
+  int TV, ntiles, cap;
+  float* rec;
+  unsigned* slots;  // [2][cap][K]: launch-wide lower bounds (logit, key) per parent, order-preserving encoding
 };
 
 struct MergeArgs {
-  int P; const int* P_dev; int K, ntiles, cap, S, mma; float T;
+  int P; const int* P_dev; int K, ntiles, cap; float T;
   int pdl;   // host side: launch with programmatic stream serialization
   int few_ntiles, few_cap;   // few_ntiles > 0: the level was scored by the few-parents kernel over this many tiles
-  const float* rec; unsigned* thr; unsigned* slots; const unsigned* thr0;
+  const float* rec; unsigned* slots;
   float *lse0, *lseT; int* top_tok; float* top_logit; int* draw_tok; float* draw_logit;
 };
 
 // Bytes of record scratch a scoring pass over up to P parents needs, and the slot capacity it implies.
 size_t score_scratch_bytes(const ts_ctx* ctx, int P, int* cap_out);
-// The pruning state (thresholds + slots) sits behind the records; it must be zero before a launch and
-// the merge kernel leaves it zero again.
+// The pruning slots sit behind the records; they must be zero before a launch and
+// the merge kernel leaves them zero again.
 unsigned* thr_base(const ts_ctx* ctx, float* rec, int cap);
 size_t thr_bytes(const ts_ctx* ctx, int cap);
 
@@ -70,22 +50,11 @@ size_t thr_bytes(const ts_ctx* ctx, int cap);
 // p_bound: an upper bound of *P_dev the host knows (-1: none).  A list that cannot exceed few_cap parents
 // goes to the few-parents kernel where the context has one.
 // rec: record scratch of score_scratch_bytes(ctx, max parents) bytes with slot capacity cap.
-ScoreArgs make_score_args(const ts_ctx* ctx, float* rec, int cap, int* err, const void* U, const void* A, const void* W, float T,
-                          uint64_t seed);
-void set_seed_pointers(const ts_ctx* ctx, ScoreArgs& a);
-// What the expansion adds to a scoring pass: seed bounds that the level kernel already wrote (no seed launch),
-// and scouting of the next level's rows (see ScoreArgs).
-struct ScoreExtras {
-  bool thr0_ready = false;
-  int root_B = 0;   // > 0: the parents are the roots of requests 0 .. root_B-1 (parent p = request p, depth 0)
-  const int* scout_live = nullptr; int scout_B = 0, scout_depth = -1; uint2* utop = nullptr;
-  int u_depth = -1, u_B = 0;
-};
-cudaError_t launch_score(const ts_ctx* ctx, float* rec, int cap, int* err, const void* U, const void* A, const void* W,
+cudaError_t launch_score(const ts_ctx* ctx, float* rec, int cap, const void* U, const void* A, const void* W,
                          int P, const int* P_dev, const int* p_req, const int* p_depth, const int* p_token,
                          const uint64_t* p_hash, float T, uint64_t seed, float* lse0, float* lseT, int* top_tok,
                          float* top_logit, int* draw_tok, float* draw_logit, cudaStream_t st,
-                         bool pdl = false, const int* P_prev_dev = nullptr, int p_bound = -1, const ScoreExtras* extras = nullptr);
+                         bool pdl = false, int p_bound = -1);
 
 // Kernel launch, optionally with programmatic stream serialization: the kernel may then start while the
 // kernel before it in the stream is still running, and must execute pdl_wait() before it touches anything
@@ -102,17 +71,14 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-bool choose_tile_mma(const ts_config& c, int num_sms, int max_smem, bool allow_stream, TileCfg* out);
-cudaError_t score_mma_setup(ts_ctx* ctx);
-cudaError_t launch_score_mma(const ts_ctx* ctx, const ScoreArgs& a, cudaStream_t st);
-// seed bounds of every parent of the list (ts_seed.cu); runs ahead of the tensor-core scoring kernel
-cudaError_t launch_seed(const ts_ctx* ctx, const ScoreArgs& a, cudaStream_t st);
 // the few-parents kernel (ts_score_few.cu)
 int few_tiles(const ts_config& c);
 int few_capacity(const ts_config& c);
 cudaError_t launch_score_few(const ts_ctx* ctx, const ScoreArgs& a, int p_bound, cudaStream_t st);
-// encodes (or finds cached in the context) the tensor map of W for 64-token boxes; false: not available
+// tensor maps (ts_tmap.cu), encoded or found cached in the context; false: not available.  Of W [r][V] for the walk
+// (boxes of 64 tokens x r rows rounded up to 64), and of the one-launch kernel's [r][stride] matrix (rounded up to 16).
 bool w_tensor_map(ts_ctx* ctx, const void* W);
+bool tree_tensor_map(ts_ctx* ctx, const void* W, int stride, CUtensorMap* out);
 
 // the one-launch expansion and scoring (ts_tree.cu)
 struct TreeOut {
@@ -127,10 +93,8 @@ cudaError_t tree_score(ts_ctx* ctx, char* scratch, const void* U, const void* A,
                        float* draw_logit, int rows, cudaStream_t st);
 cudaError_t tree_expand(ts_ctx* ctx, char* ws, const TreeOut& o, const void* U, const void* A, const void* W, int B, const int* anchor, const float* theta,
                         float T, uint64_t seed, cudaStream_t st);
-// tensor map of a bf16 matrix [r][stride] for boxes of 64 tokens x r rows (rounded up to 16); false: not available
-bool tree_tensor_map(ts_ctx* ctx, const void* W, int stride, CUtensorMap* out);
 
-enum KernelId { K_INIT, K_SCORE, K_MERGE, K_LEVEL, K_FINAL, K_ZROWS, K_GREEDY, K_WALK, K_CHECK, K_SCORE_FEW, K_ALLOC_SELECT, K_ALLOC_CUT, K_CALIB_ACC, K_CALIB_FIT, K_ATTN_INPUTS, K_SEED, K_PERSIST, K_COUNT };
+enum KernelId { K_INIT, K_SCORE, K_MERGE, K_LEVEL, K_FINAL, K_ZROWS, K_GREEDY, K_WALK, K_CHECK, K_SCORE_FEW, K_ALLOC_SELECT, K_ALLOC_CUT, K_CALIB_ACC, K_CALIB_FIT, K_ATTN_INPUTS, K_PERSIST, K_COUNT };
 
 struct Prof {
   bool on = false;

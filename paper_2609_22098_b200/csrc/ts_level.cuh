@@ -1,5 +1,5 @@
-// One level step of the best-first expansion (Algorithm 1, Section 3.5) for one request: the body shared by
-// expand_level_kernel and the persistent expansion kernel.
+// One level step of the best-first expansion (Algorithm 1, Section 3.5) for one request: the body of
+// expand_level_kernel, and what the one-launch expansion shares with it.
 #pragma once
 #include <math.h>
 
@@ -25,11 +25,7 @@ struct ExpandArgs {
   float* root_lseT; int *req_npar, *req_base, *req_nscored;
   // candidates
   int *cd_valid, *cd_parent, *cd_sib, *cd_tok; double *cd_logkey, *cd_logS; float *cd_q0, *cd_logqT; int* cd_rank;
-  int* status; int* err; unsigned* thr; int thr_head, thr_words;
-  unsigned* seed_cnt;   // the seed kernel's arrival counters
-  unsigned* ex_barrier; // grid barrier words of the persistent kernel
-  // seed bounds of the next level's parents (made by the level kernel from the scoring kernel's scouting)
-  const void *U, *A, *W; int r, ntiles, cap; uint64_t seed; const uint2* utop; unsigned* thr0;
+  int* status; unsigned* slots; int nslots;   // pruning slots of the scoring launches
   int calib_qT;   // ablation: the calibrator is fed the tempered conditional when T > 0
 };
 
@@ -54,43 +50,22 @@ __device__ __forceinline__ bool before(double ka, int da, uint64_t pa, double kb
   return pa < pb;
 }
 
-// The persistent form of the kernel (one cooperative launch for all levels of an expansion): after the scan of a
-// level the grid merges the level's parents (merge_parent, parents dealt to the CTAs), runs the level step of every
-// request (level_step, requests dealt to the CTAs), and goes on to the next level while it has parents.  The W
-// tile, tensor memory and barriers are set up once; grid barriers (bounded) separate the phases.
-struct PersistArgs {
-  int on;               // 0: one scan of the parent list in ScoreArgs, nothing else
-  int first;            // first level this launch runs (levels before it were run by launches of their own)
-  int nlevels;          // D
-  ExpandArgs ex;        // level lists, pools, seeds
-  MergeArgs mg;         // merged-result arrays
-  unsigned* barrier;    // [2] counter and abort word of the grid barrier (zero at launch)
-  int lost_arrival;     // test switch: the grid barrier expects one arrival more than will come
-};
-
-// host side of the persistent form (ts_score_mma.cu)
-bool persistent_supported(const ts_ctx* ctx, int B, int first_level);
-cudaError_t launch_expand_persistent(const ts_ctx* ctx, const ScoreArgs& a, const PersistArgs& pa, cudaStream_t st);
-
 constexpr int LEVEL_THREADS = 256;
-constexpr int SEED_PBATCH = 64;    // parents whose rows of A the seed phase stages at a time
 
 // shared-memory state of one level step (beside the dynamic array of level_smem_bytes())
 struct LevelSmem {
   int s_cnt[2]; int s_base;
   int s_free[256], s_new[256], s_warp[8]; int s_run, s_nb;
-  int s_stok[NSEED_MAX], s_pli[256], s_ptok[256]; float s_sval[NSEED_MAX]; uint64_t s_phash[256];
+  int s_tcnt[128], s_toff[128];
 };
 
 // The level step of request b; level d = depth of the parents just scored.  Called by LEVEL_THREADS threads
 // (tid = 0 .. LEVEL_THREADS-1) that `sync` synchronises; sm_raw = level_smem_bytes() bytes of shared memory.
 template <class Sync>
-__device__ __forceinline__ void level_step(const ExpandArgs& a, const int d, const int seed_next, const int b, LevelSmem& sm,
+__device__ __forceinline__ void level_step(const ExpandArgs& a, const int d, const int b, LevelSmem& sm,
                                            unsigned char* sm_raw, const int tid, Sync sync) {
   int (&s_cnt)[2] = sm.s_cnt; int& s_base = sm.s_base;
   int (&s_free)[256] = sm.s_free; int (&s_new)[256] = sm.s_new; int (&s_warp)[8] = sm.s_warp; int& s_run = sm.s_run; int& s_nb = sm.s_nb;
-  int (&s_stok)[NSEED_MAX] = sm.s_stok; int (&s_pli)[256] = sm.s_pli; int (&s_ptok)[256] = sm.s_ptok;
-  float (&s_sval)[NSEED_MAX] = sm.s_sval; uint64_t (&s_phash)[256] = sm.s_phash;
   const int N = a.N, K = a.K;
   const int npar = a.req_npar[b], base = a.req_base[b];
   const int cur = d & 1, nxt = cur ^ 1;
@@ -98,7 +73,6 @@ __device__ __forceinline__ void level_step(const ExpandArgs& a, const int d, con
   request_caps(a, b, K_eff, N_eff, log_theta);
   const size_t pb = (size_t)b * N, cb = (size_t)b * N * K;
   if (tid == 0) {
-    if (*reinterpret_cast<volatile int*>(a.err) != 0 && a.status[b] == TS_OK) a.status[b] = TS_ERR_TIMEOUT;  // a wait in the scoring kernel ran out
     s_base = a.status[b];
   }
   sync();
@@ -112,7 +86,6 @@ __device__ __forceinline__ void level_step(const ExpandArgs& a, const int d, con
     const int li = base + i;
     const int slot = a.lst_slot[cur][li];
     const double logS_v = slot < 0 ? 0.0 : a.pl_logS[pb + slot];
-    // (merged results come from other CTAs, which in the persistent kernel wrote them moments ago: read around L1)
     const double lse0 = __ldcg(a.res_lse0 + li), lseT = __ldcg(a.res_lseT + li);
     if (j == 0) {
       if (slot < 0) a.root_lseT[b] = (float)lseT; else a.pl_lseT[pb + slot] = (float)lseT;
@@ -317,8 +290,8 @@ __device__ __forceinline__ void level_step(const ExpandArgs& a, const int d, con
   // place; pass 2 places.  (One trip at a time with the running total carried through shared memory cost four
   // block barriers and a chain of loads per trip: 11 trips at the wide configuration, 100 us.)
   const int ntrip = (ncand + LEVEL_THREADS - 1) / LEVEL_THREADS;   // <= Nmax * K / 256 <= 16
-  int* trip_cnt = s_pli;    // [ntrip][8] (phase 5 fills these arrays later)
-  int* trip_off = s_ptok;
+  int* trip_cnt = sm.s_tcnt;    // [ntrip][8]
+  int* trip_off = sm.s_toff;
   unsigned vm = 0;
   for (int it = 0; it < ntrip; ++it) {
     const int c = it * LEVEL_THREADS + tid;
@@ -373,115 +346,11 @@ __device__ __forceinline__ void level_step(const ExpandArgs& a, const int d, con
     }
     sync();
     if (tid == 0) a.req_base[b] = s_nb;
-    int my_li = -1;
     if (par) {
       const int sl = s_new[tid];
       const int li = s_nb + off + __popc(bal & ((1u << lane) - 1u));
       a.lst_req[nxt][li] = b; a.lst_depth[nxt][li] = d + 1; a.lst_token[nxt][li] = a.pl_tok[pb + sl];
       a.lst_hash[nxt][li] = a.pl_hash[pb + sl]; a.lst_slot[nxt][li] = sl;
-      my_li = li;
-    }
-    // ---- phase 5: seed bounds of those parents (bf16 tensor-core path; see ts_seed.cu for what they are) ----
-    // The scoring launch of this level left the best base logit of every vocabulary tile of row U[b][d+1]:
-    // the warps pick 2K good tokens from those, the tokens' columns of W are staged once for the request,
-    // every (parent, token) pair is evaluated exactly by one thread, and one thread per parent takes the
-    // K-th best logit and key, less the rounding margin.
-    if (seed_next && cnt > 0) {
-      const int r = a.r, V = a.V;
-      const int npick = max(1, min(2 * K, NSEED_MAX) / 8), NSn = 8 * npick;
-      const float invT = a.T > 0.f ? 1.f / a.T : 1.f;
-      sync();   // the Entry array in dynamic shared memory is free now
-      // (rows of r + 1 words: the threads of a warp read the same k of different picks, which an even row length
-      // puts into one bank)
-      const int rs = r + 1;
-      float* Wc = reinterpret_cast<float*>(sm_raw);            // [NSn][r + 1]
-      float* res = Wc + (size_t)NSn * rs;                       // [cnt][NSn][2]: logit, key
-      if (par) {
-        const int i = off + __popc(bal & ((1u << lane) - 1u));
-        s_pli[i] = my_li; s_ptok[i] = a.pl_tok[pb + s_new[tid]]; s_phash[i] = a.pl_hash[pb + s_new[tid]];
-      }
-      {
-        const uint2* ut = a.utop + ((size_t)b * a.D + (d + 1)) * a.ntiles;
-        float bv = -INFINITY; int bi = 0x7FFFFFFF;
-        for (int t = lane * 8 + warp; t < a.ntiles; t += LEVEL_THREADS) {   // consecutive tiles go to different warps
-          const uint2 e = __ldcg(ut + t);
-          const float v = __uint_as_float(e.x);
-          if (v > bv || (v == bv && (int)e.y < bi)) { bv = v; bi = (int)e.y; }
-        }
-        for (int i = 0; i < npick; ++i) {   // every warp hands over its npick best
-          float wv = bv; int wi = bi;
-#pragma unroll
-          for (int o2 = 16; o2 > 0; o2 >>= 1) {
-            const float ov = __shfl_xor_sync(0xFFFFFFFFu, wv, o2);
-            const int oi = __shfl_xor_sync(0xFFFFFFFFu, wi, o2);
-            if (ov > wv || (ov == wv && oi < wi)) { wv = ov; wi = oi; }
-          }
-          if (wi == bi && bv > -INFINITY) { bv = -INFINITY; bi = 0x7FFFFFFF; }
-          if (lane == 0) { s_stok[warp * npick + i] = (wv > -INFINITY && wi >= 0 && wi < V) ? wi : -1; }
-        }
-      }
-      sync();
-      const __nv_bfloat16* Wg = reinterpret_cast<const __nv_bfloat16*>(a.W);
-      const __nv_bfloat16* Ag = reinterpret_cast<const __nv_bfloat16*>(a.A);
-      const __nv_bfloat16* Urow = reinterpret_cast<const __nv_bfloat16*>(a.U) + ((size_t)b * a.D + (d + 1)) * V;
-      for (int e = tid; e < NSn * r; e += LEVEL_THREADS) {
-        const int j = e / r, k = e % r;
-        Wc[(size_t)j * rs + k] = s_stok[j] >= 0 ? __bfloat162float(Wg[(size_t)k * V + s_stok[j]]) : 0.f;
-      }
-      if (tid < NSn) s_sval[tid] = s_stok[tid] >= 0 ? __bfloat162float(Urow[s_stok[tid]]) : -INFINITY;
-      sync();
-      // The parents' rows of A are staged in shared memory a batch of SEED_PBATCH parents at a time (one coalesced
-      // sweep per batch): read per pair from global memory they were r / 8 dependent round trips per pair, and a
-      // request of the wide configuration has 5,000 pairs.
-      uint4* Ast = reinterpret_cast<uint4*>(res + (size_t)a.N * NSn * 2);   // [SEED_PBATCH][r] bf16
-      const int cpr = r / 8;                                                  // r is a multiple of 8 on this path
-      for (int i0 = 0; i0 < cnt; i0 += SEED_PBATCH) {
-        const int nbat = min(SEED_PBATCH, cnt - i0);
-        for (int e = tid; e < nbat * cpr; e += LEVEL_THREADS)
-          Ast[e] = __ldg(reinterpret_cast<const uint4*>(Ag + (size_t)s_ptok[i0 + e / cpr] * r) + e % cpr);
-        sync();
-        for (int e = tid; e < nbat * NSn; e += LEVEL_THREADS) {
-          const int il = e / NSn, i = i0 + il, j = e % NSn;
-          float lg = -INFINITY, key = -INFINITY;
-          const int tok = s_stok[j];
-          if (tok >= 0) {
-            const uint4* arow = Ast + (size_t)il * cpr;
-            float dot = 0.f;
-            for (int k8 = 0; k8 < cpr; ++k8) {
-              float av[8];
-              unpack_bf16x8(arow[k8], av);
-#pragma unroll
-              for (int u = 0; u < 8; ++u) dot = fmaf(av[u], Wc[(size_t)j * rs + k8 * 8 + u], dot);
-            }
-            lg = s_sval[j] + dot;
-            key = lg;
-            if (a.T > 0.f) {
-              const uint4 cw = stream_words(a.seed, b, s_phash[i], STREAM_GUMBEL_COARSE, (uint32_t)tok >> 3);
-              const uint4 fw = stream_words(a.seed, b, s_phash[i], STREAM_GUMBEL_FINE, (uint32_t)tok >> 3);
-              const uint32_t c16 = (word_of(cw, (tok & 7) >> 1) >> (16 * (tok & 1))) & 0xFFFFu;
-              const uint32_t f16 = (word_of(fw, (tok & 7) >> 1) >> (16 * (tok & 1))) & 0xFFFFu;
-              key = lg * invT + gumbel_from_bits((c16 << 16) | f16);
-            }
-          }
-          res[2 * ((size_t)i * NSn + j)] = lg; res[2 * ((size_t)i * NSn + j) + 1] = key;
-        }
-        sync();
-      }
-      for (int e = tid; e < 2 * cnt; e += LEVEL_THREADS) a.thr0[(size_t)(e & 1) * a.cap + s_pli[e >> 1]] = 0u;   // no bound unless K finite values turn up
-      sync();
-      for (int e = tid; e < 2 * cnt * NSn; e += LEVEL_THREADS) {
-        // one thread per value: the one with exactly K - 1 values before it (ties broken by place) is the K-th best
-        const int j = e % NSn, which = (e / NSn) & 1, i = e / (2 * NSn);
-        if (which == 1 && !(a.T > 0.f)) continue;
-        const float* val = res + (size_t)i * NSn * 2 + which;
-        const float mine = val[2 * j];
-        int before = 0;
-        for (int t = 0; t < NSn; ++t) before += (val[2 * t] > mine || (val[2 * t] == mine && t < j)) ? 1 : 0;
-        if (before == K - 1 && mine == mine && fabsf(mine) < INFINITY) {
-          const float margin = (2e-4f + 4e-5f * fabsf(mine)) * (which == 0 ? 1.f : fmaxf(invT, 1.f)) + (which == 0 ? 0.f : 2e-4f);
-          a.thr0[(size_t)which * a.cap + s_pli[i]] = enc_f(mine - margin);
-        }
-      }
     }
   }
 }

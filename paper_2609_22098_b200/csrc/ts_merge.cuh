@@ -1,5 +1,5 @@
 // Merge of the per-piece scoring records of one parent (Eq. 1 log-normalisers, the K best logits and the K
-// best sampling keys of Eq. 2): the body shared by merge_kernel and the persistent expansion kernel.
+// best sampling keys of Eq. 2): the body of merge_kernel.
 #pragma once
 #include "ts_internal.h"
 #include "ts_scan.cuh"
@@ -84,9 +84,9 @@ struct MergeSmem {
 
 // Every thread folds its share of the pieces into a private (max, sums) pair and hands the list entries that
 // survive the final bounds to shared memory; the block then ranks them (value desc, token asc).  Called by
-// MERGE_THREADS threads (tid = 0 .. MERGE_THREADS-1) that `sync` synchronises; P = parents of the launch.
+// MERGE_THREADS threads (tid = 0 .. MERGE_THREADS-1) that `sync` synchronises.
 template <int KR, class Sync>
-__device__ __forceinline__ void merge_parent(const MergeArgs& a, const int p, const int P, MergeSmem& sm, const int tid, Sync sync) {
+__device__ __forceinline__ void merge_parent(const MergeArgs& a, const int p, MergeSmem& sm, const int tid, Sync sync) {
   float (&s_v)[MERGE_WARPS] = sm.s_v; int (&s_i)[MERGE_WARPS] = sm.s_i; float (&s_l)[MERGE_WARPS] = sm.s_l;
   float (&s_m)[MERGE_WARPS] = sm.s_m; float (&s_s0)[MERGE_WARPS] = sm.s_s0; float (&s_sT)[MERGE_WARPS] = sm.s_sT;
   float (&c_v)[2][MERGE_CAP] = sm.c_v; int (&c_i)[2][MERGE_CAP] = sm.c_i; float (&c_l)[2][MERGE_CAP] = sm.c_l;
@@ -95,24 +95,17 @@ __device__ __forceinline__ void merge_parent(const MergeArgs& a, const int p, co
   const float invT = a.T > 0.f ? 1.f / a.T : 1.f;
   const int K = a.K, rw = rec_words(K);
   const bool few = a.few_ntiles > 0;   // the level was scored by the few-parents kernel
-  const int R = few ? 1 : (a.mma ? mma_replicas(P) : 1);
-  const int npieces = few ? a.few_ntiles : a.ntiles * a.S * R;
+  const int npieces = few ? a.few_ntiles : a.ntiles;
   {
     // final launch-wide lower bounds of this parent's K-th best logit / key: entries below cannot win
     const SharedThr gl{a.slots + (size_t)p * K * SLOT_STRIDE, 0}, gk{a.slots + ((size_t)a.cap + p) * K * SLOT_STRIDE, 0};
-    float bL = dec_f(slots_min(gl, K)), bK = a.T > 0.f ? dec_f(slots_min(gk, K)) : -INFINITY;
-    if (a.thr0) {   // never below the parent's seed bounds
-      bL = fmaxf(bL, dec_f(__ldcg(a.thr0 + p)));
-      if (a.T > 0.f) bK = fmaxf(bK, dec_f(__ldcg(a.thr0 + (size_t)a.cap + p)));
-    }
+    const float bL = dec_f(slots_min(gl, K)), bK = a.T > 0.f ? dec_f(slots_min(gk, K)) : -INFINITY;
     if (tid < 2) c_n[tid] = 0;
     sync();
     float m = -INFINITY, s0 = 0.f, sT = 0.f;
     auto rec_of = [&](int q) {
       if (few) return a.rec + ((size_t)q * a.few_cap + p) * rw;
-      const int ts_ = q / R, rho = q % R;
-      const int slot = R > 1 ? rho * (128 / R) + p : p;
-      return a.rec + ((size_t)ts_ * a.cap + slot) * rw;
+      return a.rec + ((size_t)q * a.cap + p) * rw;
     };
     // the header of the next record is requested before this one's entries, so that a thread with
     // several records pays one memory round trip per record, not two
@@ -186,7 +179,6 @@ __device__ __forceinline__ void merge_parent(const MergeArgs& a, const int p, co
     }
     // leave the launch-wide pruning state of this parent clean for the next launch
     if (tid < 2 * K) a.slots[(((size_t)(tid / K) * a.cap + p) * K + tid % K) * SLOT_STRIDE] = 0u;
-    if (tid < 2) a.thr[(size_t)tid * a.cap + p] = 0u;   // and its condensed copy
     const bool fits = c_n[0] <= MERGE_CAP && c_n[1] <= MERGE_CAP;   // uniform: read after the barrier above
     if (fits) {
       // the usual case: a few dozen candidates survive the bounds; half of the block ranks each list

@@ -46,10 +46,12 @@ extern "C" int32_t ts_score_parents_static(ts_ctx* ctx, const void* U, const voi
              P, tree_need, (unsigned)TS_STATIC_SCRATCH_BYTES);
     return set_error(TS_ERR_WORKSPACE, msg);
   }
-  // records of P parents over all vocabulary tiles, plus the scoring kernel's error word
+  if (tree_need == 0 && ctx->tile.ntiles == 0)   // ragged vocabulary and a rank whose W tile does not fit shared memory
+    return set_error(TS_ERR_UNSUPPORTED, "ts_score_parents_static: no vocabulary tiling fits shared memory; use ts_score_parents with a workspace instead");
+  // records of P parents over all vocabulary tiles
   int cap = 0;
   const size_t rec_bytes = align_up(score_scratch_bytes(ctx, P, &cap), 256);
-  const size_t need = rec_bytes + 256;
+  const size_t need = rec_bytes;
   if (tree_need == 0 && need > (size_t)TS_STATIC_SCRATCH_BYTES) {
     int cap1 = 0;
     const size_t unit = score_scratch_bytes(ctx, 1, &cap1);  // bytes for the smallest slot block
@@ -80,13 +82,11 @@ extern "C" int32_t ts_score_parents_static(ts_ctx* ctx, const void* U, const voi
     return e == cudaSuccess ? TS_OK : set_cuda_error("ts_score_parents_static", e);
   }
   // The records need no clearing: the scoring kernel writes every record of (piece, parent < P) before
-  // the merge kernel, next on the same stream, reads exactly those.  The error word and the pruning
-  // state behind the records must start at zero.
-  int* err = (int*)((char*)scratch + rec_bytes);
-  e = cudaMemsetAsync(err, 0, 16, (cudaStream_t)stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(thr_base(ctx, (float*)scratch, cap), 0, thr_bytes(ctx, cap), (cudaStream_t)stream);
+  // the merge kernel, next on the same stream, reads exactly those.  The pruning
+  // slots behind the records must start at zero.
+  e = cudaMemsetAsync(thr_base(ctx, (float*)scratch, cap), 0, thr_bytes(ctx, cap), (cudaStream_t)stream);
   if (e != cudaSuccess) return set_cuda_error("ts_score_parents_static(memset)", e);
-  e = launch_score(ctx, (float*)scratch, cap, err, U, A, W, P, nullptr, parent_req, parent_depth, parent_token,
+  e = launch_score(ctx, (float*)scratch, cap, U, A, W, P, nullptr, parent_req, parent_depth, parent_token,
                    parent_hash, T, seed, lse0, lseT, top_tok, top_logit, draw_tok, draw_logit, (cudaStream_t)stream);
   if (e != cudaSuccess) return set_cuda_error("ts_score_parents_static", e);
   return TS_OK;

