@@ -26,6 +26,7 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 // these words with atomicMax in the launch's first microseconds; packed together they queue up on a
 // handful of L2 lines (measured: a third of the scoring launch at stride 1).
 constexpr int SLOT_STRIDE = 32;
+constexpr int ZCTAS = 2;             // CTAs of the row-statistics kernel per SM, one piece of the target rows each
 constexpr int SCORE_THREADS = 128;   // one parent per thread; every thread scans the CTA's whole tile
 constexpr int CHUNK = 16;            // tokens per coarse generator call
 
@@ -112,6 +113,7 @@ struct WsLayout {
   size_t cd_valid, cd_parent, cd_sib, cd_tok, cd_logkey, cd_logS, cd_q0, cd_logqT, cd_rank;
   // verification
   size_t z_max, z_arg, z_lse;            // per Z row, [B*(N+1)]
+  size_t z_part; int z_np;               // row statistics by pieces (ts_zrow.cuh): [B*(N+1) + z_np] of 16 bytes
   size_t vf_state;                       // VerifyState[B]
   size_t vf_part;                        // float[B][ntiles]
   size_t vf_barrier;                     // unsigned[4]
@@ -166,28 +168,32 @@ __host__ inline WsLayout make_layout(const ts_ctx* ctx, int B) {
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   const size_t P = (size_t)L.Pcap, K = (size_t)c.K, N = (size_t)c.Nmax, b = (size_t)B;
+  // the level-by-level expansion's arrays (the one-launch expansion has a region of its own, below)
+  auto lvl = [&](size_t bytes) { return ctx->use_tree ? (size_t)0 : take(bytes); };
   L.rec_cap = (L.Pcap + 7) / 8 * 8;
-  L.rec = take(record_bytes(ctx, L.rec_cap) + 2 * (size_t)L.rec_cap * K * SLOT_STRIDE * 4);
-  L.res_lse0 = take(P * 4); L.res_lseT = take(P * 4);
-  L.res_top_tok = take(P * K * 4); L.res_top_logit = take(P * K * 4);
-  L.res_draw_tok = take(P * K * 4); L.res_draw_logit = take(P * K * 4);
+  L.rec = lvl(record_bytes(ctx, L.rec_cap) + 2 * (size_t)L.rec_cap * K * SLOT_STRIDE * 4);
+  L.res_lse0 = lvl(P * 4); L.res_lseT = lvl(P * 4);
+  L.res_top_tok = lvl(P * K * 4); L.res_top_logit = lvl(P * K * 4);
+  L.res_draw_tok = lvl(P * K * 4); L.res_draw_logit = lvl(P * K * 4);
   for (int i = 0; i < 2; ++i) {
-    L.lst_req[i] = take(P * 4); L.lst_depth[i] = take(P * 4); L.lst_token[i] = take(P * 4);
-    L.lst_hash[i] = take(P * 8); L.lst_slot[i] = take(P * 4);
+    L.lst_req[i] = lvl(P * 4); L.lst_depth[i] = lvl(P * 4); L.lst_token[i] = lvl(P * 4);
+    L.lst_hash[i] = lvl(P * 8); L.lst_slot[i] = lvl(P * 4);
   }
-  L.lvl_count = take((DMAX + 2) * 4);
-  L.pl_alive = take(b * N * 4); L.pl_depth = take(b * N * 4); L.pl_parent = take(b * N * 4);
-  L.pl_sib = take(b * N * 4); L.pl_tok = take(b * N * 4); L.pl_lidx = take(b * N * 4); L.pl_new = take(b * N * 4);
-  L.pl_logkey = take(b * N * 8); L.pl_logS = take(b * N * 8); L.pl_q0 = take(b * N * 4);
-  L.pl_logqT = take(b * N * 4); L.pl_lseT = take(b * N * 4); L.pl_hash = take(b * N * 8); L.pl_path = take(b * N * 8);
-  L.root_lseT = take(b * 4);
-  L.req_npar = take(b * 4); L.req_base = take(b * 4); L.req_nscored = take(b * 4);
+  L.lvl_count = lvl((DMAX + 2) * 4);
+  L.pl_alive = lvl(b * N * 4); L.pl_depth = lvl(b * N * 4); L.pl_parent = lvl(b * N * 4);
+  L.pl_sib = lvl(b * N * 4); L.pl_tok = lvl(b * N * 4); L.pl_lidx = lvl(b * N * 4); L.pl_new = lvl(b * N * 4);
+  L.pl_logkey = lvl(b * N * 8); L.pl_logS = lvl(b * N * 8); L.pl_q0 = lvl(b * N * 4);
+  L.pl_logqT = lvl(b * N * 4); L.pl_lseT = lvl(b * N * 4); L.pl_hash = lvl(b * N * 8); L.pl_path = lvl(b * N * 8);
+  L.root_lseT = lvl(b * 4);
+  L.req_npar = take(b * 4); L.req_base = lvl(b * 4); L.req_nscored = lvl(b * 4);
   const size_t NK = N * K;
-  L.cd_valid = take(b * NK * 4); L.cd_parent = take(b * NK * 4); L.cd_sib = take(b * NK * 4);
-  L.cd_tok = take(b * NK * 4); L.cd_logkey = take(b * NK * 8); L.cd_logS = take(b * NK * 8);
-  L.cd_q0 = take(b * NK * 4); L.cd_logqT = take(b * NK * 4); L.cd_rank = take(b * NK * 4);
+  L.cd_valid = lvl(b * NK * 4); L.cd_parent = lvl(b * NK * 4); L.cd_sib = lvl(b * NK * 4);
+  L.cd_tok = lvl(b * NK * 4); L.cd_logkey = lvl(b * NK * 8); L.cd_logS = lvl(b * NK * 8);
+  L.cd_q0 = lvl(b * NK * 4); L.cd_logqT = lvl(b * NK * 4); L.cd_rank = lvl(b * NK * 4);
   const size_t rows = b * (N + 1);
   L.z_max = take(rows * 4); L.z_arg = take(rows * 4); L.z_lse = take(rows * 4);
+  L.z_np = ZCTAS * ctx->num_sms;
+  L.z_part = take((rows + (size_t)L.z_np) * 16);
   L.vf_state = take(b * sizeof(VerifyState));
   L.vf_part = take(b * (size_t)ctx->vt_n * 4);
   L.vf_barrier = take(64);

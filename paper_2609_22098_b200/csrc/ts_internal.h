@@ -94,7 +94,7 @@ cudaError_t tree_score(ts_ctx* ctx, char* scratch, const void* U, const void* A,
 cudaError_t tree_expand(ts_ctx* ctx, char* ws, const TreeOut& o, const void* U, const void* A, const void* W, int B, const int* anchor, const float* theta,
                         float T, uint64_t seed, cudaStream_t st);
 
-enum KernelId { K_INIT, K_SCORE, K_MERGE, K_LEVEL, K_FINAL, K_ZROWS, K_GREEDY, K_WALK, K_CHECK, K_SCORE_FEW, K_ALLOC_SELECT, K_ALLOC_CUT, K_CALIB_ACC, K_CALIB_FIT, K_ATTN_INPUTS, K_PERSIST, K_COUNT };
+enum KernelId { K_INIT, K_SCORE, K_MERGE, K_LEVEL, K_FINAL, K_ZROWS, K_GREEDY, K_WALK, K_SCORE_FEW, K_ALLOC_SELECT, K_ALLOC_CUT, K_CALIB_ACC, K_CALIB_FIT, K_ATTN_INPUTS, K_PERSIST, K_COUNT };
 
 struct Prof {
   bool on = false;

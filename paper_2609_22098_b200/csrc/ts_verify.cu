@@ -19,6 +19,7 @@
 #include "ts_scan.cuh"
 #include "ts_tc.cuh"
 #include "ts_walk.cuh"
+#include "ts_zrow.cuh"
 
 namespace ts {
 
@@ -28,95 +29,135 @@ __device__ __forceinline__ float fast_ex2(float x) { float y; asm("ex2.approx.ft
 // maximum that returns NaN when either operand is NaN (fmaxf drops NaNs)
 __device__ __forceinline__ float max_nan(float a, float b) { float y; asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b)); return y; }
 
-constexpr int ZT = 512;  // threads per target row in the row-statistics kernel
-
 // ------------------------------------------------------------------------------------------------
 // Stage 1: row statistics
 // ------------------------------------------------------------------------------------------------
-template <typename TIn>
-__global__ void __launch_bounds__(ZT) zrow_stats_kernel(const TIn* Z, const int64_t* z_row_off, int B, int V, float T,
-                                                       float* z_max, int* z_arg, float* z_logs, unsigned* walk_barrier) {
-  // One CTA per target row, one sweep: every thread keeps a running (max, arg-max, sum of exp((z-max)/T))
-  // over its share of the row, four 16-byte loads in flight, and the block folds the triples.
-  __shared__ float s_v[ZT / 32]; __shared__ int s_i[ZT / 32]; __shared__ float s_s[ZT / 32];
+// 32 bytes of a row (32-byte aligned), still packed; read once, so not kept in L1
+template <typename TIn> struct ZVec {
+  static constexpr int N = 32 / (int)sizeof(TIn);
+  uint32_t q[8];
+  __device__ __forceinline__ void load(const TIn* p) {
+    asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]) : "l"(p));
+  }
+  __device__ __forceinline__ float at(int i) const {   // (i: a constant)
+    if (sizeof(TIn) == 4) return __uint_as_float(q[i]);
+    return __uint_as_float((i & 1) ? q[i >> 1] & 0xFFFF0000u : q[i >> 1] << 16);
+  }
+  __device__ __forceinline__ static uint32_t max2(uint32_t a, uint32_t b) {
+    uint32_t y;
+    if (sizeof(TIn) == 4) y = __float_as_uint(max_nan(__uint_as_float(a), __uint_as_float(b)));
+    else asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(y) : "r"(a), "r"(b));
+    return y;
+  }
+  __device__ __forceinline__ float max() const {   // NaN when one of them is
+    const uint32_t m = max2(max2(max2(q[0], q[1]), max2(q[2], q[3])), max2(max2(q[4], q[5]), max2(q[6], q[7])));
+    if (sizeof(TIn) == 4) return __uint_as_float(m);
+    return max_nan(__uint_as_float(m << 16), __uint_as_float(m & 0xFFFF0000u));
+  }
+};
+
+// One CTA per piece of the array of target rows (ts_zrow.cuh says how it is cut).  Bound by memory, with the one ex2 per
+// element close behind (18 us of a B200's special-function units for the 175 MB of a serving batch of 32, 27 us of its
+// memory).  Per element there is one fused multiply-add, one ex2 and one add, and per 32 bytes a packed maximum; what
+// would be work per new maximum is kept out of the loop: the position inside the vector is looked up once at the end,
+// and the sums keep the reference of the thread's first vectors until a maximum leaves it by 2^32 (a running maximum
+// per thread made some lane of nearly every warp rescale and search in nearly every vector).  Two CTAs of 64 registers
+// with the next 64 bytes of every thread in flight beat three of 40 without (2,000 rows: 121 us, not 126).
+// One CTA per row took (V = 151,936, launch included) 21 us for the 15 rows of one request, 47 us for 575 rows, 144 us
+// for 2,000; now 11, 42 and 121 us.  Finer pieces (4 and 8 per SM, dealt by the hardware) were slower: 45 and 49 us.
+template <typename TIn, bool SUMS>
+__global__ void __launch_bounds__(ZT, ZCTAS) zrow_stats_kernel(const TIn* Z, const int64_t* z_row_off, int B, int V, float T, ZPart* part, unsigned* walk_barrier) {
+  __shared__ unsigned s_m[2][ZT / 32], s_c[2][ZT / 32]; __shared__ float s_ref[2][ZT / 32], s_s[2][ZT / 32]; __shared__ int s_nan[2][ZT / 32];
   pdl_wait();   // the target logits (and the tree) may come from the kernel just before this one
   pdl_launch_dependents();
   // the walk's barrier words start at zero (done here rather than by a memset, which would sit between
   // this kernel and the walk in the stream and keep the walk from starting its preamble early)
   if (walk_barrier && blockIdx.x == 0 && threadIdx.x < 16) walk_barrier[threadIdx.x] = 0u;
-  const int64_t rows = z_row_off[B];
+  const int64_t total = z_row_off[B] * V, q = zrow_piece(total, V, gridDim.x);
+  const int64_t e0 = blockIdx.x * q, e1 = e0 + q < total ? e0 + q : total;
+  if (e0 >= e1) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int VEC = Elem<TIn>::VEC;
-  constexpr int UNR = 4;
-  const bool vec_ok = (V % VEC) == 0;
-  const float invT = T > 0.f ? 1.f / T : 1.f;
-  for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
-    const TIn* z = Z + row * V;
-    float bv = -INFINITY, sum = 0.f; int bi = 0x7FFFFFFF;
-    // per vector: the maximum by a compare tree (its position is looked for only when it beats the running
-    // maximum, which is rare), then one fused multiply-add and one ex2 per element
-    const float sc = invT * 1.4426950408889634f;
-    float boff = 0.f;   // -bv * sc while bv is finite
-    bool has_nan = false;
-    auto take = [&](const float* x, int c, int n) {
-      float vm = x[0];
+  constexpr int VEC = ZVec<TIn>::N, UNR = 2;
+  const float sc = SUMS ? 1.4426950408889634f / T : 1.f, reach = 32.f / sc;
+  int par = 0;
+  int64_t row = e0 / V;
+  for (int64_t s0 = e0; s0 < e1; ++row, par ^= 1) {
+    // the piece's share [s0, s1) of this row, as token numbers [lo, hi); [al, be) of it is whole aligned vectors (a row
+    // starts wherever the vocabulary and the caller's pointer put it)
+    const int64_t base = row * V, s1 = base + V < e1 ? base + V : e1;
+    const TIn* z = Z + base;
+    const int lo = (int)(s0 - base), hi = (int)(s1 - base), mis = (int)((uintptr_t)z / sizeof(TIn) % VEC);
+    const int al = min(hi, lo + (VEC - (lo + mis) % VEC) % VEC), be = max(al, hi - (hi + mis) % VEC);
+    float bv = -INFINITY, ref = -INFINITY, lim = -INFINITY, boff = 0.f, sum = 0.f;   // lim = ref + reach, boff = -ref * sc once ref is finite
+    int bc = 0x7FFFFFFF;                                                             // first token of the vector that holds bv
+    auto top = [&](float vm, int c) {
+      if (vm > bv) bc = c;   // first maximum wins: a thread's tokens increase
+      bv = max_nan(bv, vm);  // a NaN stays
+      if (SUMS && vm > lim) { sum *= fast_ex2((ref - vm) * sc); ref = vm; lim = vm + reach; boff = -vm * sc; }
+    };
+    auto one = [&](int c) { const float x = Elem<TIn>::to_f(z[c]); top(x, c); if (SUMS) sum += fast_ex2(fmaf(x, sc, boff)); };
+    auto vec = [&](const ZVec<TIn>& v, int c) {
+      top(v.max(), c);
+      if (SUMS) {
+        float s4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int i = 1; i < VEC; ++i) if (i < n) vm = max_nan(vm, x[i]);
-      has_nan |= vm != vm;   // one test per vector: a NaN anywhere in it survives the maximum
-      if (vm > bv) {   // first maximum wins: indices increase
-        int vi = 0;
-#pragma unroll
-        for (int i = VEC - 1; i >= 0; --i) if (i < n && x[i] == vm) vi = i;
-        sum *= fast_ex2((bv - vm) * sc);
-        bv = vm; bi = c + vi; boff = -vm * sc;
-      }
-      if (T > 0.f) {
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) if (i < n) sum += fast_ex2(fmaf(x[i], sc, boff));
+        for (int i = 0; i < VEC; ++i) s4[i & 3] += fast_ex2(fmaf(v.at(i), sc, boff));
+        sum += (s4[0] + s4[1]) + (s4[2] + s4[3]);
       }
     };
-    if (vec_ok) {
-      int c = tid * VEC;
-      for (; c + (UNR - 1) * ZT * VEC < V; c += UNR * ZT * VEC) {
-        float x[UNR][8];
+    if (tid < al - lo) one(lo + tid);
+    // the next vectors are requested before the present ones are worked on
+    constexpr int STEP = UNR * ZT * VEC, SPAN = (UNR - 1) * ZT * VEC;
+    int c = al + tid * VEC;
+    ZVec<TIn> v[UNR];
+    if (c + SPAN < be)
 #pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-          const TIn* pz = z + c + u * ZT * VEC;
-          if (sizeof(TIn) == 2) unpack_bf16x8(__ldg(reinterpret_cast<const uint4*>(pz)), x[u]);
-          else { const float4 v = __ldg(reinterpret_cast<const float4*>(pz)); x[u][0] = v.x; x[u][1] = v.y; x[u][2] = v.z; x[u][3] = v.w; }
-        }
+      for (int u = 0; u < UNR; ++u) v[u].load(z + c + u * ZT * VEC);
+    for (; c + SPAN < be; c += STEP) {
+      ZVec<TIn> nx[UNR];
+      if (c + STEP + SPAN < be)
 #pragma unroll
-        for (int u = 0; u < UNR; ++u) take(x[u], c + u * ZT * VEC, VEC);
+        for (int u = 0; u < UNR; ++u) nx[u].load(z + c + STEP + u * ZT * VEC);
+#pragma unroll
+      for (int u = 0; u < UNR; ++u) vec(v[u], c + u * ZT * VEC);
+#pragma unroll
+      for (int u = 0; u < UNR; ++u) v[u] = nx[u];
+    }
+    for (; c < be; c += ZT * VEC) { v[0].load(z + c); vec(v[0], c); }
+    if (tid < hi - be) one(be + tid);
+    // fold: value descending (-0 equals 0), ties to the lowest token; sums to the largest reference
+    auto fold = [&](unsigned& m, unsigned& cc, float& r, float& s, int& nan) {
+      const unsigned wm = __reduce_max_sync(0xFFFFFFFFu, m);
+      cc = __reduce_min_sync(0xFFFFFFFFu, m == wm ? cc : 0x7FFFFFFFu);
+      m = wm;
+      nan = __any_sync(0xFFFFFFFFu, nan);
+      const float wr = dec_f(__reduce_max_sync(0xFFFFFFFFu, enc_f(r)));
+      s = r > -INFINITY ? s * fast_ex2((r - wr) * sc) : 0.f;
+      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+      r = wr;
+    };
+    int nan = bv != bv ? 1 : 0;
+    unsigned m = enc_f((nan ? -INFINITY : bv) + 0.f), cc = (unsigned)bc;
+    fold(m, cc, ref, sum, nan);
+    if (lane == 0) { s_m[par][warp] = m; s_c[par][warp] = cc; s_ref[par][warp] = ref; s_s[par][warp] = sum; s_nan[par][warp] = nan; }
+    __syncthreads();   // (the arrays of the share before last are free: warp 0 has come through this barrier twice since)
+    if (warp == 0) {
+      const bool in = lane < ZT / 32;
+      m = in ? s_m[par][lane] : 0u; cc = in ? s_c[par][lane] : 0x7FFFFFFFu; ref = in ? s_ref[par][lane] : -INFINITY; sum = in ? s_s[par][lane] : 0.f;
+      nan = in ? s_nan[par][lane] : 0;
+      fold(m, cc, ref, sum, nan);
+      const float gv = dec_f(m);
+      // the first token of the winning vector that has the maximum
+      const unsigned t = cc + (unsigned)lane;
+      const unsigned hit = __ballot_sync(0xFFFFFFFFu, lane < VEC && cc != 0x7FFFFFFFu && t < (unsigned)hi && Elem<TIn>::to_f(z[t]) == gv);
+      if (lane == 0) {
+        ZPart o;
+        o.m = nan ? nanf("") : gv; o.arg = hit ? (int)cc + __ffs(hit) - 1 : 0x7FFFFFFF; o.ref = ref; o.sum = sum;
+        part[row + blockIdx.x] = o;
       }
-      for (; c < V; c += ZT * VEC) {
-        float x[8];
-        if (sizeof(TIn) == 2) unpack_bf16x8(__ldg(reinterpret_cast<const uint4*>(z + c)), x);
-        else { const float4 v = __ldg(reinterpret_cast<const float4*>(z + c)); x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; }
-        take(x, c, VEC);
-      }
-    } else {
-      for (int c = tid; c < V; c += ZT) { float x[8]; x[0] = Elem<TIn>::to_f(z[c]); take(x, c, 1); }
     }
-    // fold (max, arg-max, sum): value descending, ties to the lowest token
-    for (int off = 16; off > 0; off >>= 1) {
-      const float ov = __shfl_xor_sync(0xFFFFFFFFu, bv, off); const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, off);
-      const float os = __shfl_xor_sync(0xFFFFFFFFu, sum, off);
-      const float nm = fmaxf(bv, ov);
-      const float ns = (nm > -INFINITY) ? sum * __expf((bv - nm) * invT) + os * __expf((ov - nm) * invT) : 0.f;
-      if (ov > bv || (ov == bv && oi < bi)) { bi = oi; }
-      bv = nm; sum = ns;
-    }
-    if (lane == 0) { s_v[warp] = bv; s_i[warp] = bi; s_s[warp] = sum; }
-    const int row_nan = __syncthreads_or(has_nan ? 1 : 0);
-    if (tid == 0) {
-      float gv = s_v[0]; int gi = s_i[0];
-      for (int w = 1; w < ZT / 32; ++w) if (s_v[w] > gv || (s_v[w] == gv && s_i[w] < gi)) { gv = s_v[w]; gi = s_i[w]; }
-      float gs = 0.f;
-      for (int w = 0; w < ZT / 32; ++w) if (s_v[w] > -INFINITY) gs += s_s[w] * __expf((s_v[w] - gv) * invT);
-      z_max[row] = row_nan ? nanf("") : gv; z_arg[row] = gi;   // a NaN maximum marks a row that holds a NaN
-      if (T > 0.f) z_logs[row] = logf(gs);
-    }
-    __syncthreads();
+    s0 = s1;
   }
 }
 
@@ -125,7 +166,8 @@ struct VerifyArgs {
   int B, V, D, r, K, N; float T; uint64_t seed;
   const int *anchor, *n_nodes, *tok, *parent, *depth, *sib; const uint64_t* node_hash;
   const float *logqT, *node_lseT;
-  const float* z_max; const int* z_arg; const float* z_logs;
+  float* z_max; int* z_arg; float* z_logs;   // per row, folded from its pieces by the CTA that owns the request
+  const ZPart* z_part; int z_np;             // the row statistics and the number of pieces they were cut into
   int *acc_len, *acc_node, *acc_tok, *bonus; float* edge_stat; uint32_t* flags; int* status;
   double *edge_px, *edge_qx, *edge_u;   // per edge: target and draft probability of its token, its accept uniform
   VerifyState* state; float* part; unsigned* barrier;
@@ -142,6 +184,7 @@ struct VerifyArgs {
 // Stage 2, T == 0
 // ------------------------------------------------------------------------------------------------
 __global__ void verify_greedy_kernel(VerifyArgs a) {
+  pdl_wait();   // the row statistics
   const int b = blockIdx.x, N = a.N;
   const int n_in = a.n_nodes[b];
   const bool okn = n_in >= 0 && n_in <= N;
@@ -150,9 +193,11 @@ __global__ void verify_greedy_kernel(VerifyArgs a) {
   const size_t nb = (size_t)b * N;
   // a target row that holds a NaN (its maximum is NaN) or nothing finite has no arg-max
   int bad = 0;
-  for (int i = threadIdx.x; i <= n; i += blockDim.x) {
-    const float zm = a.z_max[row0 + i];
-    bad |= (zm != zm || zm == -INFINITY) ? 1 : 0;
+  const int64_t zq = zrow_piece(a.z_row_off[a.B] * a.V, a.V, a.z_np);
+  for (int i = threadIdx.x; okn && i <= n; i += blockDim.x) {
+    const ZRow z = zrow_fold(a.z_part, row0 + i, a.V, zq, a.z_np, a.T);
+    a.z_arg[row0 + i] = z.arg;
+    bad |= (z.m != z.m || z.m == -INFINITY) ? 1 : 0;
   }
   bad = __syncthreads_or(okn ? bad : 0);
   if (a.edge_stat)
@@ -516,6 +561,7 @@ __device__ __forceinline__ bool walk_body(const VerifyArgs& a, unsigned char* w_
   const bool ws_ok = a.w_smem && vec_ok;
 
   // ---- per-edge statistics, child ranges and state initialisation (owner CTA of each request) ------
+  const int64_t zq = zrow_piece(a.z_row_off[a.B] * a.V, a.V, a.z_np);
   if (blockIdx.x == 0 && tid < 5) a.ctr[tid] = tid == 4 ? a.B : 0;
   for (int b = blockIdx.x; b < a.B; b += nblocks) {
     const int n = a.n_nodes[b];
@@ -528,8 +574,9 @@ __device__ __forceinline__ bool walk_body(const VerifyArgs& a, unsigned char* w_
     int bad = 0;
     if (okn) {
       for (int i = tid; i <= n; i += WT) {
-        const float zm = a.z_max[row0 + i], zl = a.z_logs[row0 + i];
-        bad |= (zm != zm || isinf(zm) || zl != zl || isinf(zl)) ? 1 : 0;
+        const ZRow z = zrow_fold(a.z_part, row0 + i, a.V, zq, a.z_np, a.T);
+        a.z_max[row0 + i] = z.m; a.z_logs[row0 + i] = z.logs;
+        bad |= (z.m != z.m || isinf(z.m) || z.logs != z.logs || isinf(z.logs)) ? 1 : 0;
       }
       for (int i = tid; i < n; i += WT) { const float lq = a.logqT[nb + i]; bad |= (lq != lq) ? 1 : 0; }
     }
@@ -804,14 +851,10 @@ template <typename TIn>
 __global__ void __launch_bounds__(WT, 1) verify_walk_kernel(const VerifyArgs a) {
   extern __shared__ __align__(16) unsigned char w_raw[];
   pdl_wait();   // row statistics and the tree come from earlier kernels
-  walk_body<TIn>(a, w_raw);
-}
-
-// after a barrier timeout the kernel returns early; this marks every unfinished request
-__global__ void verify_check_kernel(VerifyArgs a) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= a.B) return;
-  if (a.barrier[1] != 0u && a.state[b].need != 3) a.status[b] = TS_ERR_TIMEOUT;
+  if (walk_body<TIn>(a, w_raw)) return;
+  // a barrier gave up: the owners mark what they had not finished
+  for (int b = blockIdx.x; b < a.B; b += gridDim.x)
+    if (threadIdx.x == 0 && a.state[b].need != 3) a.status[b] = TS_ERR_TIMEOUT;
 }
 
 cudaError_t verify_setup(ts_ctx* ctx) {
@@ -852,8 +895,9 @@ extern "C" int32_t ts_verify_tree(ts_ctx* ctx, const void* U, const void* A, con
   a.U = U; a.A = A; a.W = W; a.Z = Z; a.z_row_off = z_row_off; a.B = B; a.V = c.V; a.D = c.D; a.r = c.r; a.K = c.K;
   a.N = c.Nmax; a.T = T; a.seed = seed; a.anchor = anchor_tok; a.n_nodes = n_nodes; a.tok = tok; a.parent = parent;
   a.depth = depth; a.sib = sib_rank; a.node_hash = node_hash; a.logqT = logqT; a.node_lseT = node_lseT;
-  float* z_max = (float*)(ws + L.z_max); int* z_arg = (int*)(ws + L.z_arg); float* z_logs = (float*)(ws + L.z_lse);
-  a.z_max = z_max; a.z_arg = z_arg; a.z_logs = z_logs;
+  a.z_max = (float*)(ws + L.z_max); a.z_arg = (int*)(ws + L.z_arg); a.z_logs = (float*)(ws + L.z_lse);
+  ZPart* z_part = (ZPart*)(ws + L.z_part);
+  a.z_part = z_part; a.z_np = L.z_np;
   a.acc_len = acc_len; a.acc_node = acc_node; a.acc_tok = acc_tok; a.bonus = bonus_tok; a.edge_stat = edge_stat;
   a.flags = flags; a.status = status;
   a.state = (VerifyState*)(ws + L.vf_state); a.part = (float*)(ws + L.vf_part); a.barrier = (unsigned*)(ws + L.vf_barrier);
@@ -863,21 +907,19 @@ extern "C" int32_t ts_verify_tree(ts_ctx* ctx, const void* U, const void* A, con
   a.vt_TV = ctx->vt_TV; a.vt_n = ctx->vt_n; a.max_steps = 2 * (c.Nmax + c.D) + 10;
   a.wait_limit = ctx->wait_limit; a.lost_arrival = (ctx->test_mode & TS_TEST_LOST_ARRIVAL) ? 1 : 0;
 
-  const int max_rows = B * (c.Nmax + 1);
-  int grid_rows = max_rows < 8 * ctx->num_sms ? max_rows : 8 * ctx->num_sms;
   cudaError_t ez;
   {
     ProfScope ps(ctx, K_ZROWS, st);
-    if (c.dt_Z == TS_DTYPE_BF16)
-      ez = launch_kernel(zrow_stats_kernel<__nv_bfloat16>, grid_rows, ZT, 0, st, true, (const __nv_bfloat16*)Z, z_row_off, B, c.V, T, z_max, z_arg, z_logs, T > 0.f ? a.barrier : (unsigned*)nullptr);
-    else
-      ez = launch_kernel(zrow_stats_kernel<float>, grid_rows, ZT, 0, st, true, (const float*)Z, z_row_off, B, c.V, T, z_max, z_arg, z_logs, T > 0.f ? a.barrier : (unsigned*)nullptr);
+    unsigned* bar = T > 0.f ? a.barrier : (unsigned*)nullptr;
+    auto stats = [&](auto* kernel, auto* z) { return launch_kernel(kernel, L.z_np, ZT, 0, st, true, z, z_row_off, B, c.V, T, z_part, bar); };
+    if (c.dt_Z == TS_DTYPE_BF16) ez = stats(T > 0.f ? zrow_stats_kernel<__nv_bfloat16, true> : zrow_stats_kernel<__nv_bfloat16, false>, (const __nv_bfloat16*)Z);
+    else ez = stats(T > 0.f ? zrow_stats_kernel<float, true> : zrow_stats_kernel<float, false>, (const float*)Z);
   }
   cudaError_t e = ez != cudaSuccess ? ez : cudaGetLastError();
   if (e != cudaSuccess) return set_cuda_error("ts_verify_tree(rows)", e);
   if (T == 0.f) {
-    { ProfScope ps(ctx, K_GREEDY, st); verify_greedy_kernel<<<B, 128, 0, st>>>(a); }
-    e = cudaGetLastError();
+    { ProfScope ps(ctx, K_GREEDY, st); e = launch_kernel(verify_greedy_kernel, B, 128, 0, st, true, a); }
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return set_cuda_error("ts_verify_tree(greedy)", e);
     return TS_OK;
   }
@@ -889,7 +931,7 @@ extern "C" int32_t ts_verify_tree(ts_ctx* ctx, const void* U, const void* A, con
       w.U = (const __nv_bfloat16*)U; w.A = (const __nv_bfloat16*)A; w.W = (const __nv_bfloat16*)W; w.Z = (const __nv_bfloat16*)Z; w.z_row_off = z_row_off;
       w.B = B; w.V = c.V; w.D = c.D; w.r = c.r; w.N = c.Nmax; w.T = T; w.seed = seed;
       w.anchor = anchor_tok; w.n_nodes = n_nodes; w.tok = tok; w.parent = parent; w.depth = depth; w.node_hash = node_hash;
-      w.logqT = logqT; w.node_lseT = node_lseT; w.z_max = z_max; w.z_logs = z_logs;
+      w.logqT = logqT; w.node_lseT = node_lseT; w.z_part = a.z_part; w.z_np = a.z_np;
       w.acc_len = acc_len; w.acc_node = acc_node; w.acc_tok = acc_tok; w.bonus = bonus_tok; w.edge_stat = edge_stat; w.flags = flags; w.status = status;
       w.part = a.part; w.barrier = a.barrier; w.vt_TV = a.vt_TV; w.vt_n = a.vt_n; w.max_steps = a.max_steps;
       w.wait_limit = a.wait_limit; w.lost_arrival = a.lost_arrival; w.use_tma = tma ? 1 : 0;
@@ -920,8 +962,5 @@ extern "C" int32_t ts_verify_tree(ts_ctx* ctx, const void* U, const void* A, con
     }
   }
   if (e != cudaSuccess) return set_cuda_error("ts_verify_tree(walk)", e);
-  { ProfScope ps(ctx, K_CHECK, st); verify_check_kernel<<<(B + 127) / 128, 128, 0, st>>>(a); }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return set_cuda_error("ts_verify_tree(check)", e);
   return TS_OK;
 }

@@ -54,7 +54,7 @@ __device__ __forceinline__ uint32_t wk_idesc(int n) {
 }
 
 // ---- set-up of one request, by the whole CTA: child ranges, accept-test inputs of every edge, what a reduction at a node needs ----
-__device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const int b, int* s_par) {
+__device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const int b, int* s_par, float2* s_z) {
   const int tid = threadIdx.x, N = a.N;
   const size_t nb = (size_t)b * N, cb = (size_t)b * (N + 1);
   const int n = a.n_nodes[b];
@@ -62,13 +62,17 @@ __device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const
   const int64_t row0 = a.z_row_off[b];
   const float invT = 1.f / a.T;
   constexpr float LOG2E = 1.4426950408889634f;
+  const int64_t zq = zrow_piece(a.z_row_off[a.B] * a.V, a.V, a.z_np);
   // non-finite inputs: a target row with a NaN (its maximum is NaN), without finite mass, or a node whose proposal
   // log-probability is NaN (its expansion was reported TS_ERR_NUMERIC) -- the request is not walked
   int bad = 0;
   if (okn) {
     for (int i = tid; i <= n; i += WK_THREADS) {
       const int par = i ? a.parent[nb + i - 1] : -1, dep = i ? a.depth[nb + i - 1] : 0, tok = i ? a.tok[nb + i - 1] : a.anchor[b];
-      const float zm = a.z_max[row0 + i], zl = a.z_logs[row0 + i], ls = a.node_lseT[cb + i], lq = i ? a.logqT[nb + i - 1] : 0.f;
+      const float ls = a.node_lseT[cb + i], lq = i ? a.logqT[nb + i - 1] : 0.f;
+      const ZRow zr = zrow_fold(a.z_part, row0 + i, a.V, zq, a.z_np, a.T);
+      const float zm = zr.m, zl = zr.logs;
+      s_z[i] = make_float2(zm, zl);
       bad |= (zm != zm || isinf(zm) || zl != zl || isinf(zl) || lq != lq) ? 1 : 0;
       if (i) s_par[i - 1] = par;
       NodeDesc nd;
@@ -92,7 +96,7 @@ __device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const
     }
     const int64_t row = row0 + par + 1;
     const int x = a.tok[nb + i];
-    const double lp = ((double)__bfloat162float(a.Z[row * a.V + x]) - (double)a.z_max[row]) / (double)a.T - (double)a.z_logs[row];
+    const double lp = ((double)__bfloat162float(a.Z[row * a.V + x]) - (double)s_z[par + 1].x) / (double)a.T - (double)s_z[par + 1].y;
     const double lq = (double)a.logqT[nb + i];
     WalkEdge e;
     e.px = exp(lp); e.qx = exp(lq); e.x = x; e.pad = 0;
@@ -494,6 +498,7 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
   __shared__ RedDesc s_desc[WK_REQ];
   __shared__ int s_tok[WK_REQ], s_par[256], s_cnt[WK_EPI + 1];
   __shared__ float s_part[WK_EPI * WK_REQ];
+  __shared__ float2 s_z[257];   // (maximum, log-sum-exp) of a request's rows
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = (int)blockIdx.x, ncta = (int)gridDim.x;
   const int rp = (a.r + 63) / 64 * 64, t0 = cta * a.vt_TV, tlen = min(a.vt_TV, a.V - t0), ntile = (tlen + 127) / 128;
   const uint32_t slab = (uint32_t)rp * 128u;
@@ -547,7 +552,7 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
   pdl_launch_dependents();
 
   const int nown = a.B > cta ? (a.B - cta + ncta - 1) / ncta : 0;   // requests cta, cta + ncta, ...
-  for (int i = 0; i < nown; ++i) wk_setup(a, sm.st[i], cta + i * ncta, s_par);
+  for (int i = 0; i < nown; ++i) wk_setup(a, sm.st[i], cta + i * ncta, s_par, s_z);
   unsigned gen = 0;
   const unsigned nexpect = (unsigned)ncta + (a.lost_arrival ? 1u : 0u);
   bool dead = false, finished = false;

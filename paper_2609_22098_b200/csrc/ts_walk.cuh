@@ -3,6 +3,7 @@
 #include "ts_internal.h"
 #include "ts_scan.cuh"
 #include "ts_tc.cuh"
+#include "ts_zrow.cuh"
 
 namespace ts {
 
@@ -19,7 +20,7 @@ struct WalkArgs {
   const __nv_bfloat16 *U, *A, *W, *Z; const int64_t* z_row_off;
   int B, V, D, r, N; float T; uint64_t seed;
   const int *anchor, *n_nodes, *tok, *parent, *depth; const uint64_t* node_hash;
-  const float *logqT, *node_lseT, *z_max, *z_logs;
+  const float *logqT, *node_lseT; const ZPart* z_part; int z_np;
   int *acc_len, *acc_node, *acc_tok, *bonus; float* edge_stat; uint32_t* flags; int* status;
   NodeDesc* node; int2* child; WalkEdge* edge; WalkRec* rec; float* part; unsigned* barrier;
   int vt_TV, vt_n, max_steps, ring, use_tma; uint32_t oB, oS;   // ring > 0: blocks of 128 tokens of W stream through that many slots

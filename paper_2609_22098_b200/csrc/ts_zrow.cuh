@@ -6,7 +6,6 @@
 namespace ts {
 
 constexpr int ZT = 512;        // threads per piece
-constexpr int ZCTAS = 3;       // pieces (CTAs) per SM
 constexpr int ZSPLIT = 8;      // a row is cut into at most this many pieces by length ...
 constexpr int ZPIECES = ZSPLIT + 2;   // ... and so lies in at most this many
 

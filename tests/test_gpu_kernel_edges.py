@@ -1,0 +1,103 @@
+"""The kernels' own edges: sizes at which a tile, a piece, a replica count or a dispatch rule changes."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import test_gpu_parity as parity
+from gpu_harness import Round, check_round, close, make_gpu, make_oracle, to_cpu
+from paper_2609_22098_b200 import binding
+from paper_2609_22098_b200.binding import TreeSpark
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V,B", [(1, 3), (7, 5), (31, 300), (4095, 2), (4097, 9), (33000, 1), (50257, 40)])
+def test_row_statistics_by_pieces(dtype, V, B):
+    """One-node trees with proposal probability 1: the edge statistic is p(x) itself, that is the row's maximum and
+    log-sum-exp; greedy bonus tokens are the first of planted equal maxima.  Rows and pieces start anywhere."""
+    ts = TreeSpark(V, 2, 8, 1, 2, B, dtype=dtype)
+    g = torch.Generator().manual_seed(V)
+    Z = (torch.randn(2 * B, V, generator=g) * 4).to(dtype)
+    Z[::3] -= torch.linspace(3e3, 0.0, V).to(dtype)   # rising rows: the sums' reference moves many times
+    for i in range(2 * B):
+        Z[i, torch.randint(0, V, (3,), generator=g)] = 20.0   # equal maxima
+    Z[0, 0] = Z[0, V - 1] = 20.0
+    if B > 1:
+        Z[2] = torch.where(torch.rand(V, generator=g) < 0.5, -0.0, 0.0).to(dtype)   # -0 equals 0
+    tree = ts.alloc_tree(B)
+    x = torch.randint(0, V, (B,), generator=g, dtype=torch.int32)
+    for k, v in (("n_nodes", 1), ("parent", -1), ("depth", 1), ("sib_rank", 0), ("logqT", 0.0), ("node_hash", 0), ("node_lseT", 0.0)):
+        tree[k].fill_(v)
+    tree["tok"][:, 0] = x.cuda()
+    U, A, W = (torch.zeros(s, dtype=dtype, device="cuda") for s in ((B, 2, V), (V, 8), (8, V)))
+    off = torch.arange(0, 2 * B + 1, 2, dtype=torch.int64).cuda()
+    anchor = torch.zeros(B, dtype=torch.int32, device="cuda")
+    first = Z.float().numpy().argmax(1)
+    out = ts.verify_tree(U, A, W, Z.cuda(), off, anchor, tree, 0.0, 5)
+    for b in range(B):
+        hit = int(first[2 * b]) == int(x[b])
+        assert int(out["bonus_tok"][b]) == int(first[2 * b + (1 if hit else 0)])
+    for T in (1.0, 0.05):
+        out = ts.verify_tree(U, A, W, Z.cuda(), off, anchor, tree, T, 5)
+        assert (out["status"] == 0).all()
+        lp = torch.log_softmax(Z[::2].double() / T, 1)[torch.arange(B), x.long()].numpy()
+        e = out["edge_stat"][:, 0].double().cpu().numpy()
+        # fp32 exponents of size |z| / T carry half an ulp each, the sum of positive terms a few more
+        rel = 2.0 ** -23 * (2 * 20.0 / T + 16)
+        assert np.all(np.abs(e - np.exp(lp)) <= rel * np.exp(lp) + 1e-37)
+
+
+def check_scores(dtype, V, r, K, P, T, mode=0):
+    wl = parity.small("tiny", V=V, r=r, K=K, D=3, Nmax=100, dtype=dtype, B=3, calib_mode=0)
+    rnd = Round(wl, seed=3 + V)
+    ts, orc = make_gpu(wl, None, max_batch=3, test_mode=mode), make_oracle(wl, None)
+    g = torch.Generator().manual_seed(P)
+    req, dep, tok, hsh = (torch.randint(0, n, (P,), generator=g) for n in (3, 3, V, 2 ** 62))
+    out = to_cpu(ts.score_parents(rnd.U, rnd.A, rnd.W, req.int().cuda(), dep.int().cuda(), tok.int().cuda(), hsh.cuda(), T, seed=99))
+    c = rnd.cpu()
+    Af, Wf, Uf = c["A"].float().numpy(), c["W"].float().numpy(), c["U"].float().numpy()
+    n, near = min(K, V), 0
+    for i in range(P):
+        o = orc.score_parent(Uf[req[i], dep[i]], Af[tok[i]], Wf, T, 99, int(req[i]), int(hsh[i]))
+        assert close(out["lse0"][i], o["lse0"]) and close(out["lseT"][i], o["lseT"]), i
+        for margin, name in zip(o["margins"], ("top", "draw")):
+            if margin < oracle.TOPK_MARGIN:
+                near += 1
+                continue
+            assert out[name + "_tok"][i, :n].tolist() == o[name + "_tok"][:n].tolist(), (i, name)
+            assert all(close(out[name + "_logit"][i, j], o[name + "_logit"][j]) for j in range(n)), (i, name)
+    assert near <= 2 + 0.02 * P
+
+
+# parents at the replica counts' borders (32, 64, 128 rows of a tile) and beyond one group; ranks that are no multiple of 16
+# or 64; vocabularies with 32-byte rows, with 16-byte rows only, and ragged ones (padded copies)
+@pytest.mark.parametrize("P", [1, 32, 33, 64, 65, 128, 129, 260])
+@pytest.mark.parametrize("V,r,K,mode", [(2048, 8, 8, 0), (2056, 24, 16, 0), (2049, 72, 4, 0), (2044, 64, 8, binding.TEST_NO_TMA), (65, 16, 8, 0)])
+def test_scoring_tile_edges(V, r, K, mode, P):
+    check_scores("bf16", V, r, K, P, 0.7, mode)
+
+
+# fp32 lists up to what the few-parents kernel's records hold (95 at this size), and one more
+@pytest.mark.parametrize("V,P", [(64000, 1), (64000, 9), (64000, 95), (64000, 96), (264, 8), (260, 8)])
+def test_few_parents_edges(V, P):
+    check_scores("f32", V, 4, 8, P, 1.0)
+
+
+@pytest.mark.parametrize("over,theta,T,mode", [
+    (dict(V=3000, B=3, Nmax=96, K=8, D=6, r=16), 0.005, 0.7, 0),            # the last size of the single-owner form
+    (dict(V=3001, B=3, Nmax=97, K=16, D=6, r=16), 0.005, 0.7, 0),           # shared merges and seed bounds, ragged rows
+    (dict(V=4104, B=5, Nmax=256, K=16, D=16, r=40), 0.002, 1.0, 0),
+    (dict(V=4104, B=2, Nmax=200, K=16, D=16, r=256), 0.002, 1.0, binding.TEST_NO_TMA),
+    (dict(V=2500, B=70, Nmax=12, K=4, D=4, r=8), 0.02, 1.0, 0),             # the walk: more than 64 requests in a step
+    (dict(V=5003, B=1, Nmax=24, K=8, D=5, r=64), 0.02, 0.7, 0),             # one request, ragged
+    (dict(V=60008, B=9, Nmax=24, K=8, D=5, r=256), 0.02, 1.0, 0),           # the walk streams its range of W
+])
+def test_round_edges(over, theta, T, mode):
+    wl = parity.small("wide", dtype="bf16", **over)
+    rnd = Round(wl, seed=over["V"])
+    rnd.theta.fill_(theta)
+    ts = make_gpu(wl, rnd.table, max_batch=rnd.B, test_mode=mode)
+    st = check_round(ts, make_oracle(wl, rnd.table), rnd, T, round_seed=9)
+    assert st["nodes"] > rnd.B and st["trees_exempt"] <= 0.05 * st["trees"] + 2
