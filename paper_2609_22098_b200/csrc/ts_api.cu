@@ -47,7 +47,7 @@ static bool select_paths(ts_ctx* ctx) {
   const ts_config& c = ctx->cfg;
   const unsigned tm = ctx->test_mode;
   ctx->tma_state = (tm & TS_TEST_NO_TMA) ? -1 : 0;
-  ctx->tmapW_ptr = ctx->tmapT_ptr = nullptr;
+  ctx->tmapW_ptr = ctx->tmapT_ptr = ctx->tmapU_ptr = nullptr;
   // tensor cores for bf16 inputs whose rows allow 16-byte chunks; the fp32 FMA kernels otherwise
   const bool tc = c.dt_U == TS_DTYPE_BF16 && c.r % 8 == 0 && ctx->cc_major == 10 && !(tm & TS_TEST_FORCE_FMA);
   ctx->use_walk = tc ? 1 : 0;

@@ -54,6 +54,9 @@ struct TreePlan {
   int BN, nW;            // tokens per block, stages of the W ring
   int npiece;            // pieces of a base-logit row whose best tokens become seed candidates
   int w_over;            // owners work in the W ring too
+  int rowsU;             // requests a stage of the base-logit ring holds
+  int ring_nW;           // the form with that ring: stages of the W ring (0: does not fit), offsets, size
+  uint32_t ring_oX, ring_oU; size_t ring_smem;
   uint32_t oL, oW, oX;   // shared-memory offsets (bytes)
   size_t smem;
 };
@@ -81,6 +84,8 @@ struct ts_ctx {
   const void* tmapW_ptr;
   alignas(64) unsigned char tmapT[128];   // the one-launch kernel's tensor map of W (boxes of 64 tokens x r rows)
   const void* tmapT_ptr;
+  alignas(64) unsigned char tmapU[128];   // tensor map of the base logits last expanded with ([request][depth][token] boxes)
+  const void* tmapU_ptr; int tmapU_B;
   int tma_state;   // 0 not tried yet, 1 encoder found, -1 unavailable
   int walk_pdl;    // -1: the driver refused a cooperative launch with programmatic serialization
   int tree_pdl;    // the same for the one-launch expansion

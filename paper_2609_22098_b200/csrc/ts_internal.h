@@ -79,6 +79,8 @@ cudaError_t launch_score_few(const ts_ctx* ctx, const ScoreArgs& a, int p_bound,
 // (boxes of 64 tokens x r rows rounded up to 64), and of the one-launch kernel's [r][stride] matrix (rounded up to 16).
 bool w_tensor_map(ts_ctx* ctx, const void* W);
 bool tree_tensor_map(ts_ctx* ctx, const void* W, int stride, CUtensorMap* out);
+// of base logits [B][D][stride], boxes of 64 tokens x one depth x `rows` requests
+bool u_tensor_map(ts_ctx* ctx, const void* U, int stride, int B, int rows, CUtensorMap* out);
 
 // the one-launch expansion and scoring (ts_tree.cu)
 struct TreeOut {

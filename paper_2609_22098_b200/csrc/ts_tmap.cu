@@ -12,17 +12,21 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 static EncodeTiledFn g_encode = nullptr;
 
+static bool encoder() {
+  if (g_encode) return true;
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || !fn || q != cudaDriverEntryPointSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  g_encode = (EncodeTiledFn)fn;
+  return true;
+}
+
 // tensor map of a matrix [ctx r][stride] for boxes of 64 x box_rows
 static bool encode(const ts_ctx* ctx, const void* W, int stride, int box_rows, CUtensorMap* out) {
-  if (!g_encode) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || !fn || q != cudaDriverEntryPointSuccess) {
-      (void)cudaGetLastError();
-      return false;
-    }
-    g_encode = (EncodeTiledFn)fn;
-  }
+  if (!encoder()) return false;
   const cuuint64_t gdim[2] = {(cuuint64_t)stride, (cuuint64_t)ctx->cfg.r};
   const cuuint64_t gstride[1] = {(cuuint64_t)stride * 2};
   const cuuint32_t box[2] = {64u, (cuuint32_t)box_rows}, estr[2] = {1u, 1u};
@@ -47,6 +51,20 @@ bool tree_tensor_map(ts_ctx* ctx, const void* W, int stride, CUtensorMap* out) {
   if (!encode(ctx, W, stride, (ctx->cfg.r + 15) / 16 * 16, out)) return false;
   memcpy(ctx->tmapT, out, sizeof(*out));
   ctx->tmapT_ptr = W;
+  return true;
+}
+
+bool u_tensor_map(ts_ctx* ctx, const void* U, int stride, int B, int rows, CUtensorMap* out) {
+  if (ctx->test_mode & TS_TEST_NO_TMA) return false;
+  if (ctx->tmapU_ptr == U && ctx->tmapU_B == B) { memcpy(out, ctx->tmapU, sizeof(*out)); return true; }
+  if (!encoder()) return false;
+  const cuuint64_t gdim[3] = {(cuuint64_t)stride, (cuuint64_t)ctx->cfg.D, (cuuint64_t)B};
+  const cuuint64_t gstride[2] = {(cuuint64_t)stride * 2, (cuuint64_t)stride * 2 * (cuuint64_t)ctx->cfg.D};
+  const cuuint32_t box[3] = {64u, 1u, (cuuint32_t)rows}, estr[3] = {1u, 1u, 1u};
+  if (g_encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(U), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return false;
+  memcpy(ctx->tmapU, out, sizeof(*out));
+  ctx->tmapU_ptr = U; ctx->tmapU_B = B;
   return true;
 }
 

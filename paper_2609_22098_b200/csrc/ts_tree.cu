@@ -41,7 +41,7 @@ __device__ __forceinline__ void load16_bf16(const __nv_bfloat16* p, const bool w
 }
 // Shared-memory state of a CTA.
 struct TxSm {
-  unsigned char *As, *Ws;
+  unsigned char *As, *Ws, *Us;
   unsigned long long* q;       // [TX_QCAP] queued candidates (QEntry)
   float* lists;                // [128][5K]: topv, topi, keyv, keyi, keyl of every row, sorted (value desc, token asc)
   int* ln;                     // [2][128] entries in use
@@ -51,7 +51,7 @@ struct TxSm {
   float* ghi;                  // [512] noise bounds
   volatile float* thr;         // [2][128] launch-wide bounds of the rows' parents
   ParentEntry* ent;            // [128] the group's parents by tile row
-  uint64_t *a_full, *t_full, *t_empty, *w_full, *w_free;
+  uint64_t *a_full, *t_full, *t_empty, *w_full, *w_free, *u_full, *u_free;
   uint32_t* tmem;
   volatile int *abort, *done;
   volatile unsigned* q_head; unsigned* q_tail;
@@ -60,11 +60,11 @@ struct TxSm {
 constexpr size_t tx_select_bytes(int K) {
   return (size_t)TX_QCAP * 8 + (size_t)TX_ROWS * 5 * K * 4 + 2 * TX_ROWS * 4 + 2 * TX_ROWS * 4 + 2 * TX_SPLIT * TX_ROWS * 4 + 3 * TX_SPLIT * TX_ROWS * 4;
 }
-constexpr size_t TX_FIXED_BYTES = 512 * 4 + 2 * TX_ROWS * 4 + TX_ROWS * sizeof(ParentEntry) + (1 + 4 * TX_STAGE_MAX) * 8 + 64;
+constexpr size_t TX_FIXED_BYTES = 512 * 4 + 2 * TX_ROWS * 4 + TX_ROWS * sizeof(ParentEntry) + (1 + 4 * TX_STAGE_MAX + 2 * TX_USTAGES) * 8 + 64;
 
 __device__ __forceinline__ TxSm tx_carve(unsigned char* sm, const TreeArgs& a) {
   TxSm s;
-  s.As = sm; s.Ws = sm + a.oW;
+  s.As = sm; s.Ws = sm + a.oW; s.Us = sm + a.oU;
   s.q = reinterpret_cast<unsigned long long*>(sm + a.oL);
   s.lists = reinterpret_cast<float*>(s.q + TX_QCAP);
   s.ln = reinterpret_cast<int*>(s.lists + (size_t)TX_ROWS * 5 * a.K);
@@ -76,7 +76,8 @@ __device__ __forceinline__ TxSm tx_carve(unsigned char* sm, const TreeArgs& a) {
   s.thr = s.ghi + 512;
   uint64_t* bars = reinterpret_cast<uint64_t*>(const_cast<float*>(s.thr) + 2 * TX_ROWS);
   s.a_full = bars; s.t_full = bars + 1; s.t_empty = s.t_full + TX_STAGE_MAX; s.w_full = s.t_empty + TX_STAGE_MAX; s.w_free = s.w_full + TX_STAGE_MAX;
-  s.tmem = reinterpret_cast<uint32_t*>(s.w_free + TX_STAGE_MAX);
+  s.u_full = s.w_free + TX_STAGE_MAX; s.u_free = s.u_full + TX_USTAGES;
+  s.tmem = reinterpret_cast<uint32_t*>(s.u_free + TX_USTAGES);
   s.abort = reinterpret_cast<volatile int*>(s.tmem + 1);
   s.done = reinterpret_cast<volatile int*>(s.tmem + 2);
   s.q_head = reinterpret_cast<volatile unsigned*>(s.tmem + 3);
@@ -203,8 +204,9 @@ __device__ __forceinline__ bool tx_wait_warp(uint64_t* bar, uint32_t parity, con
 // Cost: two generator calls (76 multiply-xor steps), 16 ex2 and about 100 other instructions per 16 tokens and
 // parent; a warp owns every (4R)-th chunk of 16 tokens, so with few parents (R = 2, 4 replicas of the rows) the
 // copies share the range.
+template <bool RING>
 __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int t0, const int tlen,
-                                        const uint32_t tmem_base, BlockPos& pos, const int nst) {
+                                        const uint32_t tmem_base, BlockPos& pos, const int nst, const uint32_t ub0) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int q = warp & 3, s = warp >> 2, row = q * 32 + lane;
   const int per = TX_ROWS / R, K = a.K;
@@ -232,28 +234,42 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
   float m = me.mref, s0 = 0.f, sT = 0.f;
   const int CB = a.BN / 16, nblk = (tlen + a.BN - 1) / a.BN, stride = R * TX_SPLIT, own = rho * TX_SPLIT + s;
   const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16);
-  // Base logits: 32 bytes of its parent's row per lane and chunk, straight from L2 (a scan reads each once; lanes whose
-  // parents share a row read the same sector).  Through shared memory they needed a copying warp that could not keep up with
-  // 128 different rows: 3 us per block of 128 tokens by 16-byte cp.async, 6 us by one bulk copy per row.
+  // Base logits, straight from L2: 32 bytes of its parent's row per lane and chunk (a scan reads each once; lanes whose
+  // parents share a row read the same sector).  A copying warp could not keep up with 128 different rows: 3 us per block
+  // of 128 tokens by 16-byte cp.async, 6 us by one bulk copy per row.
+  // RING: by bulk-tensor boxes of 64 tokens of every request at the level's depth, swizzled so that lanes of any eight
+  // neighbouring requests read different banks.  A warp whose lanes read 32 different rows touches 32 pages with every
+  // load: a scan of 128 parents on 128 rows took 50 us in the median CTA and 72 us in the slowest, against 34 and 36 when
+  // all lanes read one row; the box costs about 33 cycles a row, 40 us a scan of the same level.  Batches of 32 were
+  // slower this way (383 -> 396 us a round), a batch of 128 with three groups of parents a level the same.
   const __nv_bfloat16* urow = reinterpret_cast<const __nv_bfloat16*>(a.Uscan) + (size_t)max(me.row, 0) * a.Vs + t0;
   const int vleft = a.Vs - t0;   // tokens of the row from t0 on (whole 16 bytes)
   int o = own * 16;              // the next chunk to request
   uint4 nx0 = make_uint4(0u, 0u, 0u, 0u), nx1 = nx0;
   const bool wide = a.wide_u != 0;
-  if (o < tlen) load16_bf16(urow + o, wide, o + 8 < vleft, nx0, nx1);
+  if (!RING && o < tlen) load16_bf16(urow + o, wide, o + 8 < vleft, nx0, nx1);
+  const uint32_t uoff = (uint32_t)me.req * 128u, usw = (uint32_t)me.req & 7u, uslab = (uint32_t)a.rowsU * 128u;
   bool alive = true;
   for (int nb = 0; nb < nblk; ++nb, pos.next(nst)) {
     const int slot = pos.slot;
     if (!tx_wait_warp(sm.t_full + slot, pos.full(), sm, a)) { alive = false; break; }
+    const uint32_t ust = RING ? (ub0 + (uint32_t)nb) & (uint32_t)(TX_USTAGES - 1) : 0u;
+    if (RING && !tx_wait_warp(sm.u_full + ust, ((ub0 + (uint32_t)nb) / TX_USTAGES) & 1u, sm, a)) { alive = false; break; }
+    const unsigned char* ublk = sm.Us + (size_t)ust * (a.BN / 64) * uslab + uoff;
     tc_fence_after();
     const int nch = min(CB, (tlen - nb * a.BN + 15) / 16);
     for (int c = (own - nb * CB) & (stride - 1); c < nch; c += stride) {
       uint32_t ra[16];
       __syncwarp();   // (the tensor-memory load is a warp-wide instruction)
       tmem_ld16_issue(trow + (uint32_t)(slot * a.BN + c * 16), ra);
-      const uint4 u0 = nx0, u1 = nx1;   // requested one owned chunk ago; the next one's are requested now
+      uint4 u0 = nx0, u1 = nx1;   // requested one owned chunk ago; the next one's are requested now
+      if (RING) {
+        const unsigned char* up = ublk + (uint32_t)(c >> 2) * uslab;
+        const uint32_t j = (uint32_t)(c & 3) * 2u;
+        u0 = *reinterpret_cast<const uint4*>(up + ((j ^ usw) << 4)); u1 = *reinterpret_cast<const uint4*>(up + (((j + 1u) ^ usw) << 4));
+      }
       o += stride * 16;
-      if (o < tlen) load16_bf16(urow + o, wide, o + 8 < vleft, nx0, nx1);
+      if (!RING && o < tlen) load16_bf16(urow + o, wide, o + 8 < vleft, nx0, nx1);
       const int v0 = t0 + nb * a.BN + c * 16, valid = min(16, a.V - v0);
       // high halves of the sixteen uniforms: issued first, their long dependent chains overlap the rest
       uint4 cw0 = make_uint4(0, 0, 0, 0), cw1 = cw0;
@@ -342,7 +358,7 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
     }
     tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive(sm.t_empty + slot);
+    if (lane == 0) { mbar_arrive(sm.t_empty + slot); if (RING) mbar_arrive(sm.u_free + ust); }
   }
   sm.part[(0 * TX_SPLIT + s) * TX_ROWS + row] = m; sm.part[(1 * TX_SPLIT + s) * TX_ROWS + row] = s0; sm.part[(2 * TX_SPLIT + s) * TX_ROWS + row] = sT;
   __threadfence_block();
@@ -387,6 +403,23 @@ __device__ __forceinline__ void tx_load(const TreeArgs& a, const TxSm& sm, const
   }
 }
 
+// ---- base logits of a block of tokens, of every request at the level's depth, into their ring (by the same warp) --------
+// `uend`: blocks of the whole launch up to the end of the group's.
+struct ULoad { uint32_t requested; };
+__device__ __forceinline__ void tx_load_u(const TreeArgs& a, const TxSm& sm, const CUtensorMap* tm, const int t0, const int tlen, const int depth, ULoad& u, const uint32_t uend) {
+  const uint32_t nblk = (uint32_t)((tlen + a.BN - 1) / a.BN), uslab = (uint32_t)a.rowsU * 128u;
+  for (; u.requested < uend; ++u.requested) {
+    const uint32_t st = u.requested & (uint32_t)(TX_USTAGES - 1), use = u.requested / TX_USTAGES;
+    if (use > 0u && !__all_sync(0xFFFFFFFFu, mbar_test_wait(sm.u_free + st, (use - 1u) & 1u))) return;
+    if (elect_one()) {
+      const int off = (int)(nblk - (uend - u.requested)) * a.BN, ns = min(a.BN / 64, (tlen - off + 63) / 64);
+      mbar_expect_tx(sm.u_full + st, (uint32_t)ns * uslab);
+      for (int h = 0; h < ns; ++h) tma_load_box3(sm.Us + ((size_t)st * (a.BN / 64) + h) * uslab, tm, t0 + off + h * 64, depth, 0, sm.u_full + st);
+    }
+    __syncwarp();
+  }
+}
+
 // ---- the issuing warp: one tile of MMAs per block -----------------------------------------------------------------------
 __device__ __forceinline__ void tx_issue(const TreeArgs& a, const TxSm& sm, const int tlen, const uint32_t tmem_base, BlockPos& pos, BlockPos& wpos, const int group_no, const int nst) {
   const int nblk = (tlen + a.BN - 1) / a.BN, ksteps = (a.r + 15) / 16;
@@ -414,13 +447,16 @@ __device__ __forceinline__ void tx_issue(const TreeArgs& a, const TxSm& sm, cons
 // ---- the refreshing warp -----------------------------------------------------------------------------------------
 // Condenses the slots of the parents this CTA is responsible for (parent p belongs to range p mod ntiles) into two
 // words per parent and copies the condensed words of its rows into shared memory, until the scan is over.
+template <bool RING>
 __device__ __forceinline__ void tx_refresh(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int tile, const int done_target,
-                                           const CUtensorMap* tm, const int t0, const int tlen, WLoad& w, const uint32_t upto) {
+                                           const CUtensorMap* tm, const int t0, const int tlen, WLoad& w, const uint32_t upto,
+                                           const CUtensorMap* tmU, const int depth, ULoad& u, const uint32_t uend) {
   const int lane = threadIdx.x & 31, per = TX_ROWS / R, K = a.K;
   const int p_lo = R > 1 ? 0 : g * TX_ROWS, p_hi = min(P, p_lo + per), nt = a.ntiles;
   const int p_own = p_lo + ((tile - p_lo % nt + nt) % nt);
   const int which = lane >> 4, j = lane & 15;
   for (uint32_t spin = 0; spin < a.wait_limit; ++spin) {
+    if (RING) tx_load_u(a, sm, tmU, t0, tlen, depth, u, uend);
     tx_load<false>(a, sm, tm, t0, tlen, w, upto);
     if (*sm.done >= done_target || *sm.abort) break;
     // (a pass is a memory round trip: steady at first, while the bounds rise, every eighth turn later, so that the end of
@@ -1251,8 +1287,8 @@ __device__ __forceinline__ void tx_finalize(const TreeArgs& a, unsigned char* sm
 
 // MANY: owners share the work on crowded levels with the CTAs that own no request (a second instantiation: the code costs
 // the scan of the other one's launches 4 %).
-template <bool MANY>
-__global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_constant__ TreeArgs a, const __grid_constant__ CUtensorMap tmW) {
+template <bool MANY, bool RING>
+__global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_constant__ TreeArgs a, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmU) {
   extern __shared__ unsigned char raw[];
   unsigned char* base_sm = raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u);
   const TxSm sm = tx_carve(base_sm, a);
@@ -1269,6 +1305,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
       mbar_init(sm.t_full + i, 1); mbar_init(sm.t_empty + i, TX_SCAN_WARPS);
       mbar_init(sm.w_full + i, a.use_tma ? 1 : 32); mbar_init(sm.w_free + i, 1);
     }
+    for (int i = 0; i < TX_USTAGES; ++i) { mbar_init(sm.u_full + i, 1); mbar_init(sm.u_free + i, TX_SCAN_WARPS); }
     *sm.abort = 0; *sm.done = 0; *sm.q_head = 0u; *sm.q_tail = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -1284,6 +1321,8 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
   const unsigned nexpect = (unsigned)ncta + (a.lost_arrival ? 1u : 0u);
   bool dead = false;
   WLoad wl{{0, 0u, 0u}, 0, 0u};
+  ULoad ul{0u};
+  uint32_t ub0 = 0u;          // blocks that went through the base-logit ring
   BlockPos pos{0, 0u, 0u}, wpos{0, 0u, 0u};
   int groups = 0;
   const int nreq = a.score_P > 0 ? a.score_P : a.B;
@@ -1330,7 +1369,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
         __syncthreads();
         // ask L2 for this range of every base-logit row the group reads (neighbours of the list often share theirs): the scan
         // itself asks for 32 bytes a lane one chunk ahead, which leaves DRAM waiting when the rows are many
-        {
+        if (!RING) {
           const int nrow = R > 1 ? P : min(TX_ROWS, P - g * TX_ROWS), lines = (tlen * 2 + 127) / 128;
 #pragma unroll 1
           for (int x = warp; x < nrow; x += TX_WARPS) {
@@ -1343,13 +1382,15 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
         }
         const int done_target = (groups + 1) * TX_SCAN_WARPS;
         const int nst = min(512 / a.BN, TX_STAGE_MAX);   // accumulator stages
-        if (warp < TX_SCAN_WARPS) tx_scan(a, sm, R, P, g, t0, tlen, tmem_base, pos, nst);
+        const uint32_t ublocks = RING ? (uint32_t)((tlen + a.BN - 1) / a.BN) : 0u;
+        if (warp < TX_SCAN_WARPS) tx_scan<RING>(a, sm, R, P, g, t0, tlen, tmem_base, pos, nst, ub0);
         else if (warp == TX_MMA) tx_issue(a, sm, tlen, tmem_base, pos, wpos, groups, nst);
         else if (warp == TX_REFRESH) {
           const uint32_t nblk = (uint32_t)((tlen + a.BN - 1) / a.BN);
           const uint32_t level_end = (uint32_t)(groups + ngroups - g) * nblk + ((a.w_over || a.score_P > 0) ? 0u : (uint32_t)a.nW);
-          tx_refresh(a, sm, R, P, g, cta, done_target, &tmW, t0, tlen, wl, min((uint32_t)(groups + 1) * nblk + (uint32_t)a.nW, level_end));
+          tx_refresh<RING>(a, sm, R, P, g, cta, done_target, &tmW, t0, tlen, wl, min((uint32_t)(groups + 1) * nblk + (uint32_t)a.nW, level_end), &tmU, d, ul, ub0 + ublocks);
         } else tx_drain(a, sm, R, g, cta, done_target);
+        ub0 += ublocks;
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
@@ -1418,12 +1459,13 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
           }
       }
       if (d + 1 >= a.D && a.score_P == 0) { over = true; break; }
+      if (RING && a.ragged) asm volatile("fence.proxy.async;" ::: "memory");   // the padded rows written here are read by bulk-tensor loads
       fence_async_smem();   // owners work in memory that the next scan's bulk loads may write
       if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
       if (!MANY || turn || d < 0 || __ldcg(a.seed_need + d + 1) == 0) break;   // uniform: written before the barrier
     }
     if (over || dead) break;
-    if (d == -2 && a.ragged) asm volatile("fence.proxy.async;" ::: "memory");
+    if (a.ragged && (RING || d == -2)) asm volatile("fence.proxy.async;" ::: "memory");   // (and after it, for the warp that requests them)
   }
   if (dead && d == -2 && a.score_P == 0) {
     for (int b = cta; b < a.B; b += ncta) {   // nothing of these requests exists yet: an empty tree
@@ -1440,6 +1482,11 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
       const uint32_t slot = x % (uint32_t)a.nW, use = x / (uint32_t)a.nW;
       bool landed = false;
       for (uint32_t i = 0; i < WAIT_LIMIT && !landed; ++i) { landed = mbar_test_wait(sm.w_full + slot, use & 1); if (!landed) __nanosleep(100); }
+    }
+  if (RING && warp == TX_REFRESH && lane == 0)
+    for (uint32_t x = ul.requested > (uint32_t)TX_USTAGES ? ul.requested - (uint32_t)TX_USTAGES : 0u; x < ul.requested; ++x) {
+      bool landed = false;
+      for (uint32_t i = 0; i < WAIT_LIMIT && !landed; ++i) { landed = mbar_test_wait(sm.u_full + (x & (uint32_t)(TX_USTAGES - 1)), (x / TX_USTAGES) & 1u); if (!landed) __nanosleep(100); }
     }
   if (dead && tid == 0) { atomicExch(a.barrier + 1, 1u); atomicExch(a.err, 1); }
   __syncthreads();
@@ -1495,6 +1542,13 @@ bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
     if (own > p.oX) p.oX = (uint32_t)up(own);
     if (p.oX + fix > avail) continue;
     p.smem = p.oX + fix + 1024;
+    // The form with the base-logit ring: RU stages of it beside what W stages then fit.
+    p.rowsU = ((c.max_batch < TX_ROWS ? c.max_batch : TX_ROWS) + 7) & ~7;
+    const size_t ring = (size_t)TX_USTAGES * (BN / 64) * p.rowsU * 128;
+    auto behind = [&](int nw) { const size_t x = p.oW + (size_t)nw * w; return up(own > x ? own : x); };
+    p.ring_nW = 0;
+    for (int nw = 2; nw <= TX_STAGE_MAX && behind(nw) + fix + ring <= avail; ++nw) p.ring_nW = nw;
+    if (p.ring_nW) { p.ring_oX = (uint32_t)behind(p.ring_nW); p.ring_oU = (uint32_t)(p.ring_oX + fix); p.ring_smem = p.ring_oU + ring + 1024; }
     *out = p;
     return true;
   }
@@ -1540,7 +1594,7 @@ static void fill_args(ts_ctx* ctx, TreeArgs& a, char* base, const TreeWs& w, boo
   a.Vs = p.Vs; a.Uscan = a.ragged ? base + w.upad : U; a.Wscan = a.ragged ? base + w.wpad : W;
   a.wide_u = (p.Vs % 16 == 0 && ((uintptr_t)a.Uscan & 31u) == 0) ? 1 : 0;
   a.TV = p.TV; a.ntiles = p.ntiles; a.BN = p.BN; a.nW = p.nW; a.npiece = p.npiece; a.w_over = p.w_over;
-  a.oL = p.oL; a.oW = p.oW; a.oX = p.oX;
+  a.oL = p.oL; a.oW = p.oW; a.oX = p.oX; a.oU = 0; a.rowsU = p.rowsU;
   for (uint32_t i = 0; i < 10; ++i) { a.rk[2 * i] = (uint32_t)seed + i * 0x9E3779B9u; a.rk[2 * i + 1] = (uint32_t)(seed >> 32) + i * 0xBB67AE85u; }
   a.no_seed = (ctx->test_mode & TS_TEST_NO_SEED) ? 1 : 0;
   int* head = (int*)(base + w.head);
@@ -1554,18 +1608,23 @@ static void fill_args(ts_ctx* ctx, TreeArgs& a, char* base, const TreeWs& w, boo
 }
 
 static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream_t st) {
-  CUtensorMap tm;
-  memset(&tm, 0, sizeof(tm));
+  // crowded levels (a request with dozens of parents) need room for them in the tree and CTAs to spare
+  const bool many = a.score_P == 0 && ctx->num_sms >= 2 * a.B && a.N > 96;
+  CUtensorMap tm, tmU;
+  memset(&tm, 0, sizeof(tm)); memset(&tmU, 0, sizeof(tmU));
   a.use_tma = tree_tensor_map(ctx, a.Wscan, a.Vs, &tm) ? 1 : 0;
+  // (given parents lie at mixed depths, and a box holds 128 requests)
+  const TreePlan& p = ctx->tree;
+  const bool ring = p.ring_nW > 0 && a.score_P == 0 && !many && a.B >= TX_RING_MIN && a.B <= a.rowsU && u_tensor_map(ctx, a.Uscan, a.Vs, a.B, a.rowsU, &tmU);
+  if (ring) { a.nW = p.ring_nW; a.oX = p.ring_oX; a.oU = p.ring_oU; }
   cudaError_t e;
   { ProfScope ps(ctx, K_INIT, st); e = launch_kernel(tree_init_kernel, 1, 64, 0, st, true, a.barrier, 8 + 2 * (DMAX + 2)); }
   if (e != cudaSuccess) return e;
   ProfScope ps(ctx, prof_id, st);
-  // crowded levels (a request with dozens of parents) need room for them in the tree and CTAs to spare
-  const void* fn = (a.score_P == 0 && ctx->num_sms >= 2 * a.B && a.N > 96) ? (const void*)tree_kernel<true> : (const void*)tree_kernel<false>;
-  void* kargs[] = {(void*)&a, (void*)&tm};
+  const void* fn = many ? (const void*)tree_kernel<true, false> : (ring ? (const void*)tree_kernel<false, true> : (const void*)tree_kernel<false, false>);
+  void* kargs[] = {(void*)&a, (void*)&tm, (void*)&tmU};
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ctx->num_sms); cfg.blockDim = dim3(TX_THREADS); cfg.dynamicSmemBytes = ctx->tree.smem; cfg.stream = st;
+  cfg.gridDim = dim3(ctx->num_sms); cfg.blockDim = dim3(TX_THREADS); cfg.dynamicSmemBytes = ring ? p.ring_smem : p.smem; cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;   // grid barriers: every CTA resident
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[1].val.programmaticStreamSerializationAllowed = 1;
@@ -1581,8 +1640,10 @@ static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream
 }
 
 cudaError_t tree_setup(ts_ctx* ctx) {
-  const cudaError_t e = cudaFuncSetAttribute(tree_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->tree.smem);
-  return e != cudaSuccess ? e : cudaFuncSetAttribute(tree_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->tree.smem);
+  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(tree_kernel<false, false>, at, (int)ctx->tree.smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<true, false>, at, (int)ctx->tree.smem);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(tree_kernel<false, true>, at, (int)(ctx->tree.ring_nW ? ctx->tree.ring_smem : ctx->tree.smem));
 }
 
 cudaError_t tree_score(ts_ctx* ctx, char* scratch, const void* U, const void* A, const void* W, int P, const int* p_req, const int* p_depth, const int* p_token,

@@ -17,6 +17,8 @@ constexpr int TX_THREADS = TX_WARPS * 32;
 constexpr int TX_ROWS = 128;               // parent rows of one MMA tile
 constexpr int TX_QCAP = 256;               // candidate queue entries (power of two)
 constexpr int TX_STAGE_MAX = 8;            // stages of the W ring
+constexpr int TX_USTAGES = 4;              // stages of the base-logit ring (two: the chain of 128 requests 674 us, four: 581)
+constexpr int TX_RING_MIN = TX_ROWS / 2 + 1;   // smallest batch that takes it: from here on a root level fills a tile's 128 rows alone
 constexpr int TX_SOLO = 16;                // new parents whose seed bounds an owner makes itself
 constexpr int TX_PIECE = 1024;             // tokens of one scouting item
 
@@ -46,7 +48,8 @@ struct TreeArgs {
   // plan
   int wide_u;            // base-logit rows start on 32 bytes
   int TV, ntiles, BN, nW, npiece, w_over, use_tma, no_seed, ragged;
-  uint32_t oL, oW, oX;   // byte offsets of the selection state, the W ring and the fixed part
+  int rowsU;             // requests a stage of the base-logit ring holds
+  uint32_t oL, oW, oX, oU;   // byte offsets of the selection state, the W ring, the fixed part and the base-logit ring
   uint32_t rk[20];       // round keys of the sampling generator
   // workspace
   ParentEntry* ent[2]; int* ent_slot[2];

@@ -92,6 +92,10 @@ def test_few_parents_edges(V, P):
     (dict(V=4104, B=2, Nmax=200, K=16, D=16, r=256), 0.002, 1.0, binding.TEST_NO_TMA),
     (dict(V=2500, B=70, Nmax=12, K=4, D=4, r=8), 0.02, 1.0, 0),             # the walk: more than 64 requests in a step
     (dict(V=5003, B=1, Nmax=24, K=8, D=5, r=64), 0.02, 0.7, 0),             # one request, ragged
+    (dict(V=19000, B=65, Nmax=12, K=4, D=4, r=8), 0.03, 1.0, 0),            # base logits by boxes of all requests: a partial last slab,
+    (dict(V=2501, B=128, Nmax=12, K=4, D=4, r=16), 0.03, 1.0, 0),           # padded rows and several groups of parents,
+    (dict(V=2504, B=128, Nmax=12, K=4, D=4, r=256), 1.0, 0.7, 0),           # the chain,
+    (dict(V=2504, B=129, Nmax=12, K=4, D=4, r=16), 0.03, 1.0, 0),           # and one request more than a box holds
     (dict(V=60008, B=9, Nmax=24, K=8, D=5, r=256), 0.02, 1.0, 0),           # the walk streams its range of W
 ])
 def test_round_edges(over, theta, T, mode):
