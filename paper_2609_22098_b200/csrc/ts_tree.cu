@@ -862,11 +862,12 @@ __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s
 // share >= 0: not the level step, but the seed bounds of every `step`-th of the new parents of request b, from the share-th
 // on (a request with many leaves them to the CTAs that own none); spread: the merge was done by all CTAs.
 template <bool MANY>
-__device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, const int b, const int d, const int share_, const int step, const bool spread_) {
+__device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, const int b, const int d, const int share_, const int step, const bool spread_, const int P) {
   const int share = MANY ? share_ : -1;
   const bool spread = MANY && spread_;
   const OwnerSm s = owner_carve(sm, a);
   __shared__ int sh[8];
+  __shared__ int own[3];   // of request blockIdx.x: parents of its current level, their base in the list, status fine (kept here: a memory round trip less)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int N = a.N, K = a.K, lk = slot_log2(K), cur = d & 1, nxt = cur ^ 1, NS = seed_count(K);
   int* ptok = s.ttok; uint64_t* phash = reinterpret_cast<uint64_t*>(s.tlog);   // the new parents (merged results are done with by then)
@@ -901,6 +902,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
         a.status[b] = ok ? TS_OK : TS_ERR_INVALID;
         ptok[0] = ok ? t : 0; phash[0] = 0ull;
         a.req_npar[b] = 1; a.req_base[b] = b; a.req_nscored[b] = 0;
+        if (b == (int)blockIdx.x) { own[0] = 1; own[1] = b; own[2] = ok ? 1 : 0; }
         a.root_lseT[b] = nanf("");
         const float th = a.theta[b];   // (>= 1: the chain member of the price ladder)
         a.req_caps[b] = make_double2(th >= 1.f || !(th > 0.f) ? -INFINITY : log((double)th), th >= 1.f ? 1.0 : 0.0);
@@ -908,10 +910,12 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       s.npl[0] = -1;
     }
   } else {
-    npar = __ldcg(a.req_npar + cur * a.B + b); base = __ldcg(a.req_base + b);
-    if (npar == 0 || __ldcg(a.status + b) != TS_OK) {   // uniform: nothing below has run yet
+    bool fine;
+    if (b == (int)blockIdx.x) { npar = own[0]; base = own[1]; fine = own[2] != 0; }
+    else { npar = __ldcg(a.req_npar + cur * a.B + b); base = __ldcg(a.req_base + b); fine = __ldcg(a.status + b) == TS_OK; }
+    if (npar == 0 || !fine) {   // uniform: nothing below has run yet
       if (tid == 0) a.req_npar[nxt * a.B + b] = 0;
-      return;
+      return;   // (own[] stays: no parents, or not fine)
     }
     const double2 caps = __ldcg(a.req_caps + b);   // log theta (-inf on the chain member), 1 on the chain member
     log_theta = caps.x; K_eff = caps.y != 0.0 ? 1 : min(K, a.V); N_eff = caps.y != 0.0 ? min(a.D, N) : N;
@@ -939,7 +943,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       if (j == 0) { const float2 l = __ldcg(a.res_lse + base + i); s.lse0[i] = l.x; s.lseT[i] = l.y; }
     }
   } else if (d >= 0 && share < 0) {
-    const int P = __ldcg(a.lvl_count + d), R = mma_replicas(P);
+    const int R = mma_replicas(P);
 #pragma unroll 1
     for (int task = warp; task < npar * 3; task += TX_WARPS - 1) {
       const int i = task / 3, kind = task - 3 * i, p = base + i;
@@ -988,7 +992,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     const bool bad = !(lse0 == lse0) || isinf(lse0);
     if (j == 0 && which == 0) {
       if (slot < 0) a.root_lseT[b] = (float)lseT; else s.pv.lseT[slot] = (float)lseT;
-      if (bad) a.status[b] = TS_ERR_NUMERIC;
+      if (bad) { a.status[b] = TS_ERR_NUMERIC; if (b == (int)blockIdx.x) own[2] = 0; }
     }
     int ok = 0;
     if (j < K_eff && !bad) {
@@ -1070,20 +1074,23 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
             if (cum + h >= need) { bin = 255 - 8 * lane - j; break; }
             cum += h;
           }
-          sh[2] = bin; sh[3] = need - cum;
+          sh[2] = bin; sh[3] = need - cum; sh[7] = s.hist[bin] == need - cum ? 1 : 0;
         }
       }
       __syncthreads();
       prefix |= (uint64_t)sh[2] << sh8;
       need = sh[3];
+      if (sh[7]) break;   // the whole bin stays: its lower end is the threshold, nothing ties with it from below
     }
+    const bool whole = sh[7] != 0;   // (thousands of distinct keys: after three or four passes)
     if (tid == 0) sh[4] = 0;
     __syncthreads();
+    if (!whole)
 #pragma unroll 1
     for (int e = tid; e < M; e += TX_THREADS)
       if (live(e) && skey(key_of(e)) == prefix) { const int at = atomicAdd(&sh[4], 1); if (at < 256) s.newl[at] = e; }
     __syncthreads();
-    const int ntie = sh[4];
+    const int ntie = whole ? 0 : sh[4];
     unsigned drop = 0u;   // bit per trip: M <= 17 * 256 entries, at most 7 trips
 #pragma unroll 1
     for (int e = tid, it = 0; e < M; e += TX_THREADS, ++it) {
@@ -1144,7 +1151,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
         run += __shfl_sync(0xFFFFFFFFu, incl, 31);
       }
       if (lane == 0) sh[5] = min(run, nfree);
-      if (lane == 0 && run > nfree) a.status[b] = TS_ERR_OVERFLOW;
+      if (lane == 0 && run > nfree) { a.status[b] = TS_ERR_OVERFLOW; if (b == (int)blockIdx.x) own[2] = 0; }
     }
     __syncthreads();
 #pragma unroll 1
@@ -1182,7 +1189,9 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
     for (int w = 0; w < 8; ++w) { if (w < warp) off += s.tcnt[w]; cnt += s.tcnt[w]; }
     if (tid == 0) {
       const int nb = cnt > 0 ? atomicAdd(a.lvl_count + d + 1, cnt) : 0;
-      sh[6] = nb; a.req_base[b] = nb; a.req_npar[nxt * a.B + b] = cnt; a.req_nscored[b] += npar;
+      sh[6] = nb; a.req_base[b] = nb;
+      if (b == (int)blockIdx.x) { own[0] = cnt; own[1] = nb; }
+      a.req_npar[nxt * a.B + b] = cnt; a.req_nscored[b] += npar;
     }
     if (par) { const int i = off + __popc(bal & ((1u << lane) - 1u)); s.npl[i] = sl; ptok[i] = pt; phash[i] = ph; }
   }
@@ -1441,7 +1450,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
         const int first = MANY && turn ? cta % nreq : cta, share = MANY && turn ? cta / nreq : -1, hstep = MANY ? ncta / nreq : 1;
         if (!MANY || share < hstep)
 #pragma unroll 1
-          for (int b = first; b < nreq; b += MANY && turn ? nreq : ncta) tx_owner<MANY>(a, base_sm, b, d, share, hstep, spread);
+          for (int b = first; b < nreq; b += MANY && turn ? nreq : ncta) tx_owner<MANY>(a, base_sm, b, d, share, hstep, spread, P);
       }
       // best base logits of the rows after the next ones, by the CTAs that own no request where there are enough of them
       // (given parents: of their rows, before anything else)
