@@ -5,7 +5,8 @@
 //   scan   every CTA scores all of the level's parents on its range: the low-rank bias [128 parents x r].[r x BN
 //          tokens] is a tcgen05 tile per block of BN tokens, W streams through a ring of bulk-tensor loads (and runs
 //          ahead across levels: it does not depend on them), and 16 warps read the accumulators (one tensor-memory
-//          lane = one parent), add the base logits, read from L2 where a prefetch of the group's rows put them, and keep (max reference, sums) and the few tokens that can be among a parent's K best.
+//          lane = one parent), add the base logits (from L2, where a prefetch of the group's rows put them, or from a
+//          ring of their own), and keep (max reference, sums) and the few tokens that can be among a parent's K best.
 //   owner  the CTA that owns a request merges the request's parents (one warp each), runs the level step and makes
 //          the next level's parent list with its seed bounds; the CTAs without a request meanwhile sweep the base
 //          logits of the level after (best token of every 1024: where the next seed bounds come from).

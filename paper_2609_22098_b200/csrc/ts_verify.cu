@@ -1,10 +1,11 @@
 // Lossless tree verification (Section 3.2 item 3, Section 3.3).
 //
 // Stage 1 (all rows, fully parallel): max, arg-max and log-sum-exp at temperature T of every target
-//   row, one CTA per row.  With these, the first-sibling accept ratio of every edge is a scalar
+//   row, in equal pieces of the array of rows.  With these, the first-sibling accept ratio of every edge is a scalar
 //   expression, so per-edge statistics and greedy walks need no further vocabulary pass.
 // Stage 2, T == 0: pointer chase along arg-max matches.
-// Stage 2, T > 0: one persistent cooperative kernel.  The recursive-rejection walk is run as a
+// Stage 2, T > 0: one persistent cooperative kernel (bf16: ts_walk.cu; here the form for fp32, ranks that are no multiple
+//   of 8 and ranges of W that fit neither shared memory nor a tensor map).  The recursive-rejection walk is run as a
 //   scalar sequence: with R(w) = max(p(w) - C q(w), 0) the unnormalised residual after rejections,
 //   sibling j is accepted with probability min(1, max(p(x)/q(x) - C, 0) / c_j), c_j = Z_j / (1 - Q),
 //   and a rejection moves C to C + c_j and needs Z_{j+1} = sum_w R(w), one reduction over the
