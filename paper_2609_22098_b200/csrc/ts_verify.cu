@@ -229,12 +229,6 @@ __device__ __forceinline__ float z_elem(const VerifyArgs& a, int64_t row, int w)
   return Elem<TIn>::to_f(reinterpret_cast<const TIn*>(a.Z)[row * a.V + w]);
 }
 
-// probability of token w under softmax(Z[row]/T), double
-template <typename TIn>
-__device__ __forceinline__ double p_of(const VerifyArgs& a, int64_t row, int w) {
-  return exp(((double)z_elem<TIn>(a, row, w) - (double)a.z_max[row]) / (double)a.T - (double)a.z_logs[row]);
-}
-
 // Scalar state machine of one request, run by one warp of the request's owner CTA.
 // need: 0 walking, 1 reduction after a rejection, 4 reduction for the bonus draw, 5 walk over (bonus token
 // still to be drawn), 2 range rescan, 3 finished.  The bonus draws of all requests are left to the end of
