@@ -183,7 +183,7 @@ cudaError_t launch_score(const ts_ctx* ctx, float* rec, int cap, const void* U, 
 }
 
 cudaError_t score_setup(ts_ctx* ctx) {
-  if (ctx->use_tree) return cudaSuccess;   // (a tile may not even exist then)
+  if (ctx->tile.ntiles == 0) return cudaSuccess;   // no tile: never launched.  (A tensor-core context uses its tile to score ragged vocabularies without a workspace.)
   const int sm = (int)ctx->tile.smem;
   cudaError_t e = cudaFuncSetAttribute(score_tile_kernel<__nv_bfloat16, RegLists<8>>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(score_tile_kernel<__nv_bfloat16, MemLists>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);

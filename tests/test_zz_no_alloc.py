@@ -6,6 +6,9 @@ second call must not see anything of the first), and that it refuses what does n
 
 Collected last on purpose: a failure here cannot hide the result of any other test."""
 import dataclasses
+import os
+import subprocess
+import sys
 
 import pytest
 import torch
@@ -45,6 +48,26 @@ def test_static_scratch_scoring_matches_workspace_scoring_twice(T):
                                       out=ts.alloc_score_outputs(P))
         torch.cuda.synchronize()
         same(got, want, wl.K)
+
+
+def ragged_vocabulary():
+    wl = dataclasses.replace(synth.WORKLOADS["serve32"], V=30001, B=4)   # 65 KB of shared memory for a tile of W
+    rnd = Round(wl, seed=8)
+    ts = make_gpu(wl, rnd.table, max_batch=4)
+    for T in (0.0, 1.0):
+        req, dep, tok, hsh = parent_list(11, 4, wl.D, wl.V, seed=3)
+        got = ts.score_parents_static(rnd.U, rnd.A, rnd.W, req, dep, tok, hsh, T, seed=4, out=ts.alloc_score_outputs(11))
+        same(got, ts.score_parents(rnd.U, rnd.A, rnd.W, req, dep, tok, hsh, T, seed=4), wl.K)
+
+
+def test_static_scratch_scoring_of_a_ragged_vocabulary():
+    """A vocabulary that is no multiple of 8 has no padded copies here: the call runs on the tile kernel.  In a process of
+    its own, so that no other context has raised that kernel's shared-memory limit."""
+    here = os.path.dirname(os.path.abspath(__file__))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([here, os.path.dirname(here)]))
+    run = subprocess.run([sys.executable, "-c", "import test_zz_no_alloc as t; t.ragged_vocabulary()"], env=env,
+                         capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stderr[-2000:]
 
 
 def test_static_scratch_refuses_what_does_not_fit():
