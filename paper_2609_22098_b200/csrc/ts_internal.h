@@ -71,6 +71,15 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Lets a kernel ask for all the dynamic shared memory that its static arrays leave.  The limit is the process's, not a
+// context's: a context's own plan as the limit would lower it for the contexts made before.
+template <typename... KArgs>
+inline cudaError_t allow_all_smem(void (*kernel)(KArgs...), int max_smem) {
+  cudaFuncAttributes fa;
+  const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem - (int)fa.sharedSizeBytes);
+}
+
 // the few-parents kernel (ts_score_few.cu)
 int few_tiles(const ts_config& c);
 int few_capacity(const ts_config& c);

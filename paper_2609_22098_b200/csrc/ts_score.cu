@@ -183,12 +183,12 @@ cudaError_t launch_score(const ts_ctx* ctx, float* rec, int cap, const void* U, 
 }
 
 cudaError_t score_setup(ts_ctx* ctx) {
-  if (ctx->tile.ntiles == 0) return cudaSuccess;   // no tile: never launched.  (A tensor-core context uses its tile to score ragged vocabularies without a workspace.)
-  const int sm = (int)ctx->tile.smem;
-  cudaError_t e = cudaFuncSetAttribute(score_tile_kernel<__nv_bfloat16, RegLists<8>>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(score_tile_kernel<__nv_bfloat16, MemLists>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(score_tile_kernel<float, RegLists<8>>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(score_tile_kernel<float, MemLists>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  // never launched here: a tensor-core context needs its tile only to score ragged vocabularies without a workspace
+  if (ctx->use_tree && ctx->cfg.V % 8 == 0) return cudaSuccess;
+  cudaError_t e = allow_all_smem(score_tile_kernel<__nv_bfloat16, RegLists<8>>, ctx->max_smem);
+  if (e == cudaSuccess) e = allow_all_smem(score_tile_kernel<__nv_bfloat16, MemLists>, ctx->max_smem);
+  if (e == cudaSuccess) e = allow_all_smem(score_tile_kernel<float, RegLists<8>>, ctx->max_smem);
+  if (e == cudaSuccess) e = allow_all_smem(score_tile_kernel<float, MemLists>, ctx->max_smem);
   return e;
 }
 

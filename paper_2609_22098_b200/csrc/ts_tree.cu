@@ -1650,10 +1650,9 @@ static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream
 }
 
 cudaError_t tree_setup(ts_ctx* ctx) {
-  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(tree_kernel<false, false>, at, (int)ctx->tree.smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_kernel<true, false>, at, (int)ctx->tree.smem);
-  return e != cudaSuccess ? e : cudaFuncSetAttribute(tree_kernel<false, true>, at, (int)(ctx->tree.ring_nW ? ctx->tree.ring_smem : ctx->tree.smem));
+  cudaError_t e = allow_all_smem(tree_kernel<false, false>, ctx->max_smem);
+  if (e == cudaSuccess) e = allow_all_smem(tree_kernel<true, false>, ctx->max_smem);
+  return e != cudaSuccess ? e : allow_all_smem(tree_kernel<false, true>, ctx->max_smem);
 }
 
 cudaError_t tree_score(ts_ctx* ctx, char* scratch, const void* U, const void* A, const void* W, int P, const int* p_req, const int* p_depth, const int* p_token,

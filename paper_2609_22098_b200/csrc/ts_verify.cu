@@ -853,10 +853,9 @@ __global__ void __launch_bounds__(WT, 1) verify_walk_kernel(const VerifyArgs a) 
 }
 
 cudaError_t verify_setup(ts_ctx* ctx) {
-  // the walk kernel may keep its range of W in shared memory: allow the full opt-in size
-  const cudaError_t e = cudaFuncSetAttribute(verify_walk_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem - 40 * 1024);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(verify_walk_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem - 40 * 1024);
+  // the walk kernel may keep its range of W in shared memory
+  const cudaError_t e = allow_all_smem(verify_walk_kernel<__nv_bfloat16>, ctx->max_smem);
+  return e != cudaSuccess ? e : allow_all_smem(verify_walk_kernel<float>, ctx->max_smem);
 }
 
 }  // namespace ts

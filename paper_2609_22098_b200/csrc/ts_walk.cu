@@ -679,7 +679,7 @@ size_t walk_ws_bytes(const ts_ctx* ctx, int B) {
   return align_up(b * (n + 1) * sizeof(NodeDesc), 256) + align_up(b * (n + 1) * 8, 256) + align_up(b * n * sizeof(WalkEdge), 256) + align_up(b * sizeof(WalkRec), 256);
 }
 
-cudaError_t walk_setup(ts_ctx* ctx) { return cudaFuncSetAttribute(walk_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem - 16 * 1024); }
+cudaError_t walk_setup(ts_ctx* ctx) { return allow_all_smem(walk_mma_kernel, ctx->max_smem); }
 
 cudaError_t launch_walk_mma(ts_ctx* ctx, WalkArgs& a, char* ws, const WalkPlan& p, cudaStream_t st) {
   const size_t b = (size_t)a.B, n = (size_t)a.N;

@@ -105,3 +105,27 @@ def test_round_edges(over, theta, T, mode):
     ts = make_gpu(wl, rnd.table, max_batch=rnd.B, test_mode=mode)
     st = check_round(ts, make_oracle(wl, rnd.table), rnd, T, round_seed=9)
     assert st["nodes"] > rnd.B and st["trees_exempt"] <= 0.05 * st["trees"] + 2
+
+
+@pytest.mark.parametrize("big,small", [
+    (dict(V=19000, r=64, B=128), dict(V=19000, r=64, B=4)),                     # the form with the base-logit ring
+    (dict(V=19000, r=64, B=3), dict(V=19000, r=32, B=3)),                       # one-launch expansion
+    (dict(V=50001, r=64, B=2, dtype="f32"), dict(V=9001, r=4, B=2, dtype="f32")),   # fp32 tiles
+    (dict(V=3000, r=4, B=2, dtype="f32", Nmax=256, K=16), dict(V=3000, r=4, B=2, dtype="f32", Nmax=160, K=16)),   # fp32 level step
+    (dict(V=3000, r=4, B=2, dtype="f32", Nmax=128, K=15), dict(V=3000, r=4, B=2, dtype="f32", Nmax=8, K=2)),      # its 48 KB beside static arrays
+])
+def test_a_context_still_runs_after_another_one_was_made(big, small):
+    """A kernel's shared-memory limit belongs to the process: a context with a smaller plan must not lower it."""
+    def make(over):
+        wl = parity.small("serve32", **dict(dict(D=4, Nmax=24, K=4), **over))
+        rnd = Round(wl, seed=12)
+        return rnd, make_gpu(wl, rnd.table, max_batch=rnd.B)
+    rnd, ts = make(big)
+    want = to_cpu(ts.expand_tree(rnd.U, rnd.A, rnd.W, rnd.anchor, rnd.theta, 1.0, 5))
+    other = make(small)
+    got = to_cpu(ts.expand_tree(rnd.U, rnd.A, rnd.W, rnd.anchor, rnd.theta, 1.0, 5))
+    assert int(want["n_nodes"].sum()) > rnd.B and torch.equal(got["n_nodes"], want["n_nodes"])
+    for b in range(rnd.B):
+        n = int(want["n_nodes"][b])
+        assert torch.equal(got["tok"][b, :n], want["tok"][b, :n])
+    other[1].expand_tree(other[0].U, other[0].A, other[0].W, other[0].anchor, other[0].theta, 1.0, 5)
