@@ -87,8 +87,8 @@ struct ts_ctx {
   alignas(64) unsigned char tmapU[128];   // tensor map of the base logits last expanded with ([request][depth][token] boxes)
   const void* tmapU_ptr; int tmapU_B;
   int tma_state;   // 0 not tried yet, 1 encoder found, -1 unavailable
-  int walk_pdl;    // -1: the driver refused a cooperative launch with programmatic serialization
-  int tree_pdl;    // the same for the one-launch expansion
+  int walk_unchained;   // 1: the driver refuses a cooperative launch with programmatic serialization
+  int tree_unchained;   // the same for the one-launch expansion
   unsigned ablation;   // TS_ABLATE_* switches (0 = the method)
   unsigned test_mode;  // TS_TEST_* switches (0 = the product's kernel selection and wait limits)
   uint32_t wait_limit; // polls before a bounded device-side wait gives up

@@ -6,6 +6,7 @@
 #include <cuda.h>
 
 #include "ts_common.cuh"
+#include "ts_launch.h"
 
 namespace ts {
 
@@ -69,6 +70,22 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// Cooperative launch (grid barriers: every CTA resident), chained to the kernel before it where the driver takes both
+// attributes.
+inline cudaError_t launch_cooperative(int& refused, const void* kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st, void** kargs) {
+  return launch_chained(refused, [&](bool chained) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = chained ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, kernel, kargs);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+  });
 }
 
 // Lets a kernel ask for all the dynamic shared memory that its static arrays leave.  The limit is the process's, not a

@@ -1633,20 +1633,7 @@ static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream
   ProfScope ps(ctx, prof_id, st);
   const void* fn = many ? (const void*)tree_kernel<true, false> : (ring ? (const void*)tree_kernel<false, true> : (const void*)tree_kernel<false, false>);
   void* kargs[] = {(void*)&a, (void*)&tm, (void*)&tmU};
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ctx->num_sms); cfg.blockDim = dim3(TX_THREADS); cfg.dynamicSmemBytes = ring ? p.ring_smem : p.smem; cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;   // grid barriers: every CTA resident
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = ctx->tree_pdl >= 0 ? 2 : 1;
-  e = cudaLaunchKernelExC(&cfg, fn, kargs);
-  if (e != cudaSuccess && cfg.numAttrs == 2) {   // not accepted together: remember, and launch cooperative only
-    (void)cudaGetLastError();
-    ctx->tree_pdl = -1;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelExC(&cfg, fn, kargs);
-  }
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return launch_cooperative(ctx->tree_unchained, fn, dim3(ctx->num_sms), dim3(TX_THREADS), ring ? p.ring_smem : p.smem, st, kargs);
 }
 
 cudaError_t tree_setup(ts_ctx* ctx) {

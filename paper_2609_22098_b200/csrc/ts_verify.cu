@@ -939,21 +939,7 @@ extern "C" int32_t ts_verify_tree(ts_ctx* ctx, const void* U, const void* A, con
   const void* fn = c.dt_Z == TS_DTYPE_BF16 ? (const void*)verify_walk_kernel<__nv_bfloat16> : (const void*)verify_walk_kernel<float>;
   {
     ProfScope ps(ctx, K_WALK, st);
-    // cooperative (the grid barriers need every CTA resident) and, where the driver takes both attributes,
-    // chained to the row statistics so that the W load and the tensor-memory allocation run beside them
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.vt_n); cfg.blockDim = dim3(WT); cfg.dynamicSmemBytes = a.w_smem ? w_bytes : 0; cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = ctx->walk_pdl >= 0 ? 2 : 1;
-    e = cudaLaunchKernelExC(&cfg, fn, kargs);
-    if (e != cudaSuccess && cfg.numAttrs == 2) {   // not accepted together: remember, and launch cooperative only
-      (void)cudaGetLastError();
-      ctx->walk_pdl = -1;
-      cfg.numAttrs = 1;
-      e = cudaLaunchKernelExC(&cfg, fn, kargs);
-    }
+    e = launch_cooperative(ctx->walk_unchained, fn, dim3(a.vt_n), dim3(WT), a.w_smem ? w_bytes : 0, st, kargs);
   }
   if (e != cudaSuccess) return set_cuda_error("ts_verify_tree(walk)", e);
   return TS_OK;

@@ -692,23 +692,9 @@ cudaError_t launch_walk_mma(ts_ctx* ctx, WalkArgs& a, char* ws, const WalkPlan& 
   memset(&tm, 0, sizeof(tm));
   if (a.use_tma) memcpy(&tm, ctx->tmapW, sizeof(tm));
   ProfScope ps(ctx, K_WALK, st);
-  // cooperative (the grid barriers need every CTA resident) and, where the driver takes both attributes, chained to the
-  // row statistics so that the W load and the tensor-memory allocation run beside them
+  // (chained to the row statistics: the W load and the tensor-memory allocation run beside them)
   void* kargs[] = {(void*)&a, (void*)&tm};
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.vt_n); cfg.blockDim = dim3(WK_THREADS); cfg.dynamicSmemBytes = p.smem; cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = ctx->walk_pdl >= 0 ? 2 : 1;
-  cudaError_t e = cudaLaunchKernelExC(&cfg, (const void*)walk_mma_kernel, kargs);
-  if (e != cudaSuccess && cfg.numAttrs == 2) {   // not accepted together: remember, and launch cooperative only
-    (void)cudaGetLastError();
-    ctx->walk_pdl = -1;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelExC(&cfg, (const void*)walk_mma_kernel, kargs);
-  }
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return launch_cooperative(ctx->walk_unchained, (const void*)walk_mma_kernel, dim3(a.vt_n), dim3(WK_THREADS), p.smem, st, kargs);
 }
 
 }  // namespace ts
