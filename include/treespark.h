@@ -127,6 +127,8 @@ const char* ts_last_error_string(void);
  * Layout: U DEVICE [B][D][V], A DEVICE [V][r], W DEVICE [r][V], all row-major in the context's
  * dtype.  parent_* DEVICE [P]; parent_hash = path hash of the parent node.  Outputs DEVICE.
  * P <= max_batch * Nmax.  Entries beyond the vocabulary size (K > V) hold token -1.
+ * When a bounded device-side wait runs out (TS_ERR_TIMEOUT of the calls that have a status array), lse0 and lseT
+ * of the parents that got no result are NaN and their tokens are -1.
  */
 int32_t ts_score_parents(ts_ctx* ctx, const void* U, const void* A, const void* W,
                          int32_t P, const int32_t* parent_req, const int32_t* parent_depth,

@@ -1500,9 +1500,17 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
     }
   if (dead && tid == 0) { atomicExch(a.barrier + 1, 1u); atomicExch(a.err, 1); }
   __syncthreads();
+  const bool late = dead || *reinterpret_cast<volatile int*>(a.err) != 0;
   if (a.score_P == 0) {
-    const bool late = dead || *reinterpret_cast<volatile int*>(a.err) != 0;
     for (int b = cta; b < a.B; b += ncta) tx_finalize(a, base_sm, b, late);
+  } else if (late) {   // (there is no status array to report it in)
+    for (int p = cta; p < a.score_P; p += ncta) {
+      if (tid == 0) a.o_lse0[p] = a.o_lseT[p] = nanf("");
+      if (tid < a.K) {
+        const size_t o = (size_t)p * a.K + tid;
+        a.o_top_tok[o] = a.o_draw_tok[o] = -1; a.o_top_logit[o] = a.o_draw_logit[o] = 0.f;
+      }
+    }
   }
   tc_fence_before();
   __syncthreads();

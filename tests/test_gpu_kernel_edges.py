@@ -129,3 +129,27 @@ def test_a_context_still_runs_after_another_one_was_made(big, small):
         n = int(want["n_nodes"][b])
         assert torch.equal(got["tok"][b, :n], want["tok"][b, :n])
     other[1].expand_tree(other[0].U, other[0].A, other[0].W, other[0].anchor, other[0].theta, 1.0, 5)
+
+
+def test_scoring_that_gives_up_says_so_in_its_outputs():
+    """ts_score_parents has no status array: when a bounded wait runs out, log-normalisers are NaN and tokens -1."""
+    wl = parity.small("serve32", V=20000, B=3)
+    rnd = Round(wl, seed=14)
+    ts = make_gpu(wl, rnd.table, max_batch=3)
+    P = 150
+    g = torch.Generator().manual_seed(1)
+    req, dep, tok, hsh = (torch.randint(0, n, (P,), generator=g) for n in (3, wl.D, wl.V, 2 ** 62))
+    args = (rnd.U, rnd.A, rnd.W, req.int().cuda(), dep.int().cuda(), tok.int().cuda(), hsh.cuda(), 1.0, 3)
+    want = to_cpu(ts.score_parents(*args))
+    for call in (ts.score_parents, ts.score_parents_static):
+        out = ts.alloc_score_outputs(P)
+        for t in out.values():
+            t.fill_(1)
+        ts.set_test_mode(binding.TEST_SHORT_WAITS | binding.TEST_LOST_ARRIVAL)
+        bad = to_cpu(call(*args, out=out))
+        ts.set_test_mode(0)
+        assert torch.isnan(bad["lse0"]).all() and torch.isnan(bad["lseT"]).all()
+        assert (bad["top_tok"] == -1).all() and (bad["draw_tok"] == -1).all()
+    again = to_cpu(ts.score_parents(*args))
+    for k in want:
+        assert torch.equal(again[k], want[k]), k
