@@ -201,6 +201,9 @@ __device__ __forceinline__ bool tx_wait_warp(uint64_t* bar, uint32_t parity, con
   return __all_sync(0xFFFFFFFFu, tx_wait(bar, parity, sm, a));
 }
 
+// a polling loop that ran out: the scan is given up and the call reports it
+__device__ __forceinline__ void tx_give_up(const TxSm& sm, const TreeArgs& a) { *sm.abort = 1; atomicExch(a.err, 1); }
+
 // ---- scanning warps: one group of up to 128 parents over this CTA's range ---------------------------------
 // Cost: two generator calls (76 multiply-xor steps), 16 ex2 and about 100 other instructions per 16 tokens and
 // parent; a warp owns every (4R)-th chunk of 16 tokens, so with few parents (R = 2, 4 replicas of the rows) the
@@ -493,6 +496,8 @@ __device__ __forceinline__ void tx_refresh(const TreeArgs& a, const TxSm& sm, co
     }
   }
   __syncwarp();
+  if (lane == 0 && *sm.done < done_target && !*sm.abort) tx_give_up(sm, a);
+  __syncwarp();
   if (!*sm.abort) tx_load<true>(a, sm, tm, t0, tlen, w, upto);
 }
 
@@ -501,8 +506,9 @@ __device__ __forceinline__ void tx_drain(const TreeArgs& a, const TxSm& sm, cons
   const int lane = threadIdx.x & 31;
   const float invT = a.T > 0.f ? 1.f / a.T : 1.f;
   unsigned head = *sm.q_head;
-  for (uint32_t spin = 0; spin < a.wait_limit; ++spin) {
+  for (uint32_t spin = 0;; ++spin) {
     if (*sm.abort) break;
+    if (spin >= a.wait_limit) { if (lane == 0) tx_give_up(sm, a); break; }
     const bool finished = *sm.done >= done_target;   // read before the tail: pushes precede the tick
     const unsigned tail = *reinterpret_cast<volatile unsigned*>(sm.q_tail);
     const int avail = (int)(tail - head);
@@ -525,7 +531,7 @@ __device__ __forceinline__ void tx_drain(const TreeArgs& a, const TxSm& sm, cons
       }
     }
     __threadfence_block();
-    __syncwarp();
+    if (__any_sync(0xFFFFFFFFu, lane < n && !have)) { if (lane == 0) tx_give_up(sm, a); break; }   // (or given up elsewhere)
     head += (unsigned)n;
     if (lane == 0) *sm.q_head = head;   // the slots may be reused
     // candidates of one row are inserted one after the other (lanes of a row take turns)

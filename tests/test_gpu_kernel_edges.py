@@ -153,3 +153,25 @@ def test_scoring_that_gives_up_says_so_in_its_outputs():
     again = to_cpu(ts.score_parents(*args))
     for k in want:
         assert torch.equal(again[k], want[k]), k
+
+
+def test_candidates_that_nobody_waits_for_any_more_are_reported():
+    """With waits of 4096 polls the warp that takes the candidates loses patience in ranges of 100,000 tokens when the only
+    ones (planted far above the rest) stand at the ranges' ends.  They would be missing from the lists: the call says so."""
+    V, P = 1 << 24, 128
+    ts = TreeSpark(V, 1, 8, 4, P, 1)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    TV = ((V + sms - 1) // sms + 63) // 64 * 64
+    g = torch.Generator(device="cuda").manual_seed(4)
+    U, A, W = ((torch.randn(s, generator=g, device="cuda") * x).bfloat16() for s, x in (((1, 1, V), 2.0), ((V, 8), 0.3), ((8, V), 0.3)))
+    for i in range(16):
+        U[0, 0, (i * (sms // 16) + 1) * TV - 3 - i] = 64.0 + i
+    tok = torch.randint(0, V, (P,), generator=g, device="cuda", dtype=torch.int32)
+    hsh = torch.randint(0, 2 ** 62, (P,), generator=g, device="cuda", dtype=torch.int64)
+    zero = torch.zeros(P, dtype=torch.int32, device="cuda")
+    want = to_cpu(ts.score_parents(U, A, W, zero, zero, tok, hsh, 1.0, 3))
+    assert (want["top_tok"] >= 0).all()
+    ts.set_test_mode(binding.TEST_SHORT_WAITS)
+    got = to_cpu(ts.score_parents(U, A, W, zero, zero, tok, hsh, 1.0, 3))
+    lost = (got["top_tok"] != want["top_tok"]).any(1) | (got["draw_tok"] != want["draw_tok"]).any(1)
+    assert torch.isnan(got["lse0"][lost]).all(), f"{int(lost.sum())} lists are incomplete without a word"
