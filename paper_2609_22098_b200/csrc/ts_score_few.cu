@@ -177,7 +177,7 @@ int few_tiles(const ts_config& c) { return (c.V + FEW_TILE - 1) / FEW_TILE; }
 int few_capacity(const ts_config& c) {
   if (c.dt_U != TS_DTYPE_F32 || c.V % 8 != 0) return 0;
   const size_t per = (size_t)few_tiles(c) * rec_words(c.K) * 4, cap = ((size_t)4 << 20) / per;
-  return cap > 256 ? 256 : (cap < 8 ? 8 : (int)cap);
+  return cap > 256 ? 256 : (int)cap;
 }
 
 cudaError_t launch_score_few(const ts_ctx* ctx, const ScoreArgs& a, int p_bound, cudaStream_t st) {

@@ -70,6 +70,20 @@ def test_static_scratch_scoring_of_a_ragged_vocabulary():
     assert run.returncode == 0, run.stderr[-2000:]
 
 
+def test_static_scratch_takes_few_parents_over_a_large_fp32_vocabulary():
+    """The few-parents kernel's records never need more than their 4 MiB, however large a vocabulary's are."""
+    V, P = 1600000, 2
+    wl = dataclasses.replace(synth.WORKLOADS["tiny"], V=V, B=1, D=1, r=4, K=8, Nmax=8, dtype="f32", calib_mode=0)
+    ts = make_gpu(wl, None, max_batch=1)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    U, A, W = (torch.randn(s, generator=g, device="cuda") for s in ((1, 1, V), (V, 4), (4, V)))
+    req, dep, tok, hsh = parent_list(P, 1, 1, V, seed=6)
+    got = ts.score_parents_static(U, A, W, req, dep, tok, hsh, 1.0, seed=4, out=ts.alloc_score_outputs(P))
+    same(got, ts.score_parents(U, A, W, req, dep, tok, hsh, 1.0, seed=4), 8)
+    lse = torch.logsumexp(U[0, 0].double() + A[tok.long()].double() @ W.double(), 1)
+    assert all(close(got["lse0"][i], lse[i]) for i in range(P))
+
+
 def test_static_scratch_refuses_what_does_not_fit():
     wl = dataclasses.replace(synth.WORKLOADS["serve32"], V=30000 + 16, B=64)
     rnd = Round(wl, seed=6, B=2)
