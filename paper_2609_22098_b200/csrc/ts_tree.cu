@@ -770,7 +770,7 @@ __device__ __forceinline__ void load_seed_columns(const TreeArgs& a, const Owner
     w[u] = 0u;
     if (e < NS * a.r) {
       const int j = e & (NS - 1), k = e >> seed_log2(a.K), tok = s.stok[j];
-      if (tok >= 0) w[u] = __ldg(Wg + (((size_t)k * a.Vs + tok) >> 1));
+      if (tok >= 0) w[u] = __ldcg(Wg + (((size_t)k * a.Vs + tok) >> 1));   // (a ragged vocabulary's padded W is written by this launch: not the read-only path)
     }
   }
 }
