@@ -87,12 +87,12 @@ __device__ __forceinline__ TxSm tx_carve(unsigned char* sm, const TreeArgs& a) {
 }
 
 // A queued candidate in one 64-bit word, so that a plain store publishes it whole: logit in the high half; below it a tag
-// that changes with every turn of the queue (4 bits), kind (2), split (2), row (7), place in the range (17).  (With the tag
+// that changes with every turn of the queue (4 bits), kind (2), split (2), row (7), place in the range (TX_PLACE_BITS).  (With the tag
 // in a word of its own a fence had to stand between the two stores, and the fence waited for the scanning thread's
 // base-logit loads in flight: two microseconds a candidate.)
 __device__ __forceinline__ uint32_t q_tag(unsigned idx) { return (idx / TX_QCAP) % 15u + 1u; }   // never 0: 0 = nothing written
 __device__ __forceinline__ unsigned long long q_pack(float lg, unsigned idx, uint32_t kind, int split, int row, int off) {
-  return ((unsigned long long)__float_as_uint(lg) << 32) | (q_tag(idx) << 28) | (kind << 26) | ((uint32_t)split << 24) | ((uint32_t)row << 17) | (uint32_t)off;
+  return ((unsigned long long)__float_as_uint(lg) << 32) | (q_tag(idx) << 28) | (kind << 26) | ((uint32_t)split << 24) | ((uint32_t)row << TX_PLACE_BITS) | (uint32_t)off;
 }
 
 // insertion into one sorted list of at most K entries (value desc, token asc); returns the K-th value (-inf: not full)
@@ -149,9 +149,9 @@ struct CoarseGen {
 
 // One candidate, handled by one lane of the selecting warp: exact key, insertion, publication.
 __device__ __forceinline__ void tx_select(const TreeArgs& a, const TxSm& sm, const unsigned long long e, float invT, int tile, int R, int g) {
-  const int K = a.K, tok = tile * a.TV + (int)((uint32_t)e & 0x1FFFFu);
+  const int K = a.K, tok = tile * a.TV + (int)((uint32_t)e & ((1u << TX_PLACE_BITS) - 1u));
   const float lg = __uint_as_float((uint32_t)(e >> 32));
-  const int row = (int)((uint32_t)e >> 17) & 127, s = (int)((uint32_t)e >> 24) & 3;
+  const int row = (int)((uint32_t)e >> TX_PLACE_BITS) & 127, s = (int)((uint32_t)e >> 24) & 3;
   const uint32_t kind = ((uint32_t)e >> 26) & 3u;
   const int per = TX_ROWS / R;
   const int prow = R > 1 ? row % per : row, rho = R > 1 ? row / per : 0;
@@ -535,7 +535,7 @@ __device__ __forceinline__ void tx_drain(const TreeArgs& a, const TxSm& sm, cons
     head += (unsigned)n;
     if (lane == 0) *sm.q_head = head;   // the slots may be reused
     // candidates of one row are inserted one after the other (lanes of a row take turns)
-    const unsigned peers = __match_any_sync(0xFFFFFFFFu, have ? (int)((uint32_t)e >> 17) & 127 : -1 - lane);
+    const unsigned peers = __match_any_sync(0xFFFFFFFFu, have ? (int)((uint32_t)e >> TX_PLACE_BITS) & 127 : -1 - lane);
     const int turn = __popc(peers & ((1u << lane) - 1u));
     const int turns = __reduce_max_sync(0xFFFFFFFFu, have ? turn + 1 : 0);
     for (int t = 0; t < turns; ++t) {
@@ -1548,6 +1548,7 @@ bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
   TreePlan p{};
   p.TV = ((c.V + num_sms - 1) / num_sms + 63) / 64 * 64;
   p.ntiles = (c.V + p.TV - 1) / p.TV;
+  if (p.TV > 1 << TX_PLACE_BITS) return false;   // (never on 148 SMs: V <= 2^24)
   p.Vs = (c.V + 7) & ~7;
   int piece = ((c.V + 127) / 128 + 7) & ~7;
   piece = piece < 64 ? 64 : (piece > TX_PIECE ? TX_PIECE : piece);

@@ -16,6 +16,7 @@ constexpr int TX_WARPS = TX_SCAN_WARPS + 3;
 constexpr int TX_THREADS = TX_WARPS * 32;
 constexpr int TX_ROWS = 128;               // parent rows of one MMA tile
 constexpr int TX_QCAP = 256;               // candidate queue entries (power of two)
+constexpr int TX_PLACE_BITS = 17;          // of a queued candidate's place in the CTA's range
 constexpr int TX_STAGE_MAX = 8;            // stages of the W ring
 constexpr int TX_USTAGES = 4;              // stages of the base-logit ring (two: the chain of 128 requests 674 us, four: 581)
 constexpr int TX_RING_MIN = TX_ROWS / 2 + 1;   // smallest batch that takes it: from here on a root level fills a tile's 128 rows alone

@@ -41,3 +41,14 @@ def test_host_side_argument_checks_need_no_device():
     cfg = binding.TsConfig(100, 4, 8, 4, 16, 1, 0, 1, 0, 0, 0, 0.67, -0.46, -10, 10, None)
     assert lib.ts_create(C.byref(cfg), C.byref(out)) == -2          # mixed dtypes
     assert lib.ts_workspace_bytes(None, 1) == 0
+
+
+def test_expansion_plan_refuses_a_range_its_queue_cannot_address():
+    """A queued candidate carries 17 bits of place in its CTA's vocabulary range: fewer SMs mean longer ranges."""
+    import ctypes as C
+    plan = binding.load_library()._ZN2ts9tree_planERK9ts_configiiPNS_8TreePlanE
+    plan.restype = C.c_bool
+    cfg = binding.TsConfig(1 << 24, 4, 8, 4, 16, 1, 1, 1, 1, 1, 0, 0.67, -0.46, -10, 10, None)
+    out = (C.c_uint64 * 64)()   # (larger than the plan)
+    assert plan(C.byref(cfg), 148, 227 * 1024, out) and plan(C.byref(cfg), 128, 227 * 1024, out)
+    assert not plan(C.byref(cfg), 127, 227 * 1024, out)
