@@ -57,7 +57,7 @@ static bool select_paths(ts_ctx* ctx) {
     if (!ctx->use_tree) return false;
     ctx->tile = TileCfg{};
   }
-  ctx->few_cap = (tm & TS_TEST_NO_FEW) ? 0 : few_capacity(c);
+  ctx->few_cap = (tm & TS_TEST_NO_FEW) ? 0 : few_capacity(c, ctx->use_tree != 0);
   ctx->wait_limit = (tm & TS_TEST_SHORT_WAITS) ? 4096u : WAIT_LIMIT;
   return true;
 }

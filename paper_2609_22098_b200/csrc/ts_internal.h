@@ -99,7 +99,7 @@ inline cudaError_t allow_all_smem(void (*kernel)(KArgs...), int max_smem) {
 
 // the few-parents kernel (ts_score_few.cu)
 int few_tiles(const ts_config& c);
-int few_capacity(const ts_config& c);
+int few_capacity(const ts_config& c, bool use_tree);
 cudaError_t launch_score_few(const ts_ctx* ctx, const ScoreArgs& a, int p_bound, cudaStream_t st);
 // tensor maps (ts_tmap.cu), encoded or found cached in the context; false: not available.  Of W [r][V] for the walk
 // (boxes of 64 tokens x r rows rounded up to 64), and of the one-launch kernel's [r][stride] matrix (rounded up to 16).

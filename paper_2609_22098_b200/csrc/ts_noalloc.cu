@@ -38,7 +38,7 @@ extern "C" int32_t ts_score_parents_static(ts_ctx* ctx, const void* U, const voi
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return set_cuda_error("ts_score_parents_static(device)", e);
-  const size_t tree_need = ctx->use_tree ? tree_score_bytes(ctx, P) : 0;   // 0: this context scores on the fp32 kernels here
+  const size_t tree_need = ctx->use_tree && P > ctx->few_cap ? tree_score_bytes(ctx, P) : 0;   // 0: this list is scored by fused multiply-adds
   if (tree_need > (size_t)TS_STATIC_SCRATCH_BYTES) {
     char msg[256];
     snprintf(msg, sizeof(msg),
@@ -46,7 +46,7 @@ extern "C" int32_t ts_score_parents_static(ts_ctx* ctx, const void* U, const voi
              P, tree_need, (unsigned)TS_STATIC_SCRATCH_BYTES);
     return set_error(TS_ERR_WORKSPACE, msg);
   }
-  if (tree_need == 0 && ctx->tile.ntiles == 0)   // ragged vocabulary and a rank whose W tile does not fit shared memory
+  if (tree_need == 0 && P > ctx->few_cap && ctx->tile.ntiles == 0)   // ragged vocabulary and a rank whose W tile does not fit shared memory
     return set_error(TS_ERR_UNSUPPORTED, "ts_score_parents_static: no vocabulary tiling fits shared memory; use ts_score_parents with a workspace instead");
   // records of P parents over all vocabulary tiles
   int cap = 0;

@@ -211,16 +211,19 @@ extern "C" int32_t ts_score_parents(ts_ctx* ctx, const void* U, const void* A, c
   if (!(T >= 0.f)) return set_error(TS_ERR_INVALID, "ts_score_parents: T must be >= 0");
   if (ws_bytes < L.total) return set_error(TS_ERR_WORKSPACE, "ts_score_parents: workspace too small");
   if (P == 0) return TS_OK;
-  if (ctx->use_tree) {
+  const cudaStream_t st = (cudaStream_t)stream;
+  if (ctx->use_tree && P > ctx->few_cap) {
     const cudaError_t et = tree_score(ctx, (char*)ws + L.tree, U, A, W, P, parent_req, parent_depth, parent_token, parent_hash, T, seed, lse0, lseT, top_tok,
-                                      top_logit, draw_tok, draw_logit, ctx->cfg.max_batch * ctx->cfg.D, (cudaStream_t)stream);
+                                      top_logit, draw_tok, draw_logit, ctx->cfg.max_batch * ctx->cfg.D, st);
     return et == cudaSuccess ? TS_OK : set_cuda_error("ts_score_parents", et);
   }
-  cudaError_t e = cudaMemsetAsync(thr_base(ctx, (float*)((char*)ws + L.rec), L.rec_cap), 0, thr_bytes(ctx, L.rec_cap), (cudaStream_t)stream);
+  float* rec = (float*)((char*)ws + (ctx->use_tree ? L.tree : L.rec));
+  int cap = L.rec_cap;
+  if (ctx->use_tree) (void)score_scratch_bytes(ctx, P, &cap);
+  cudaError_t e = cudaMemsetAsync(thr_base(ctx, rec, cap), 0, thr_bytes(ctx, cap), st);
   if (e != cudaSuccess) return set_cuda_error("ts_score_parents(memset)", e);
-  e = launch_score(ctx, (float*)((char*)ws + L.rec), L.rec_cap, U, A, W, P, nullptr,
-                               parent_req, parent_depth, parent_token, parent_hash, T, seed, lse0, lseT, top_tok,
-                               top_logit, draw_tok, draw_logit, (cudaStream_t)stream);
+  e = launch_score(ctx, rec, cap, U, A, W, P, nullptr, parent_req, parent_depth, parent_token, parent_hash, T, seed, lse0, lseT, top_tok,
+                   top_logit, draw_tok, draw_logit, st);
   if (e != cudaSuccess) return set_cuda_error("ts_score_parents", e);
   return TS_OK;
 }

@@ -1,4 +1,5 @@
-// Scoring kernel for fp32 inputs when the parents of a level are few (a small model decoding a request or a handful).
+// Scoring kernel for lists of few parents: the levels of an fp32 expansion (a small model decoding a request or a handful)
+// and short lists given to the stand-alone call, in fp32 and bf16.
 //
 // With a handful of parents the low-rank bias [parents x r] . [r x V] is no dense contraction, and the tile kernel -- one
 // parent per lane, every lane over the whole tile -- would leave most lanes idle while it walks the vocabulary.  Here the
@@ -24,9 +25,17 @@ __device__ __forceinline__ void load8(const float* p, float* out) {
   out[0] = a.x; out[1] = a.y; out[2] = a.z; out[3] = a.w; out[4] = b.x; out[5] = b.y; out[6] = b.z; out[7] = b.w;
 }
 
+__device__ __forceinline__ void load8(const __nv_bfloat16* p, float* out) { unpack_bf16x8(__ldg(reinterpret_cast<const uint4*>(p)), out); }
+
 constexpr int FEW_THREADS = 256;
 constexpr int FEW_WARPS = FEW_THREADS / 32;
 constexpr int FEW_TILE = 256;   // tokens per tile: eight per lane
+// bf16 lists that the one-launch kernel (ts_tree.cu) would score too: at most so many parents, (parent, tile) pairs and ranks.
+// That kernel takes 30 to 50 us for one parent as for 32 (its set-up, seed bounds and grid barriers); here a list costs 22 us
+// and grows with its pairs.  Cold caches, T = 1, here / there (us): V = 32,000, r = 64: 36 / 44 for 1 parent, 36 / 46 for 16,
+// 42 / 48 for 32, 56 / 52 for 64; V = 151,936: 36 / 50 for 1, 40 / 50 for 4, 48 / 52 for 8, 71 / 52 for 16; V = 1,000: 32 / 56
+// for 64.  r = 128, K = 16, V = 128,256: 60 / 71 for 4, 71 / 73 for 8.  r = 256, V = 32,000: 65 / 58 for 1 (warm 34 / 40).
+constexpr int FEW_TREE_MAX = 64, FEW_TREE_ITEMS = 3000, FEW_TREE_RANK = 128;
 
 // (value desc, token asc) arg-max over the warp; every lane gets the winner (two reductions of integers: the value's
 // order-preserving image, then the lowest token among those that have it)
@@ -36,6 +45,7 @@ __device__ __forceinline__ void warp_best(float& v, int& tok) {
   v = dec_f(m);
 }
 
+template <typename TIn>
 __global__ void __launch_bounds__(FEW_THREADS) score_few_kernel(const ScoreArgs a) {
   __shared__ float s_a[FEW_WARPS][256];   // head row A[x_p] of each warp's parent (r <= 256)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -48,12 +58,12 @@ __global__ void __launch_bounds__(FEW_THREADS) score_few_kernel(const ScoreArgs 
   const int V = a.V, r = a.r, K = a.K;
   const int tile = blockIdx.x, v = tile * FEW_TILE + lane * 8;
   const bool in = v < V;               // V is a multiple of 8: a lane's eight tokens are all inside or all outside
-  const float* Wg = reinterpret_cast<const float*>(a.W);
-  const float* Ug = reinterpret_cast<const float*>(a.U);
-  const float* Ag = reinterpret_cast<const float*>(a.A);
+  const TIn* Wg = reinterpret_cast<const TIn*>(a.W);
+  const TIn* Ug = reinterpret_cast<const TIn*>(a.U);
+  const TIn* Ag = reinterpret_cast<const TIn*>(a.A);
   const int req = a.p_req[p], dep = a.p_depth[p], ptok = a.p_token[p];
   const uint64_t hash = a.p_hash[p];
-  for (int k = lane; k < r; k += 32) s_a[warp][k] = Ag[(size_t)ptok * r + k];
+  for (int k = lane; k < r; k += 32) s_a[warp][k] = Elem<TIn>::to_f(Ag[(size_t)ptok * r + k]);
   __syncwarp();
 
   // ---- logits of the lane's eight tokens -------------------------------------------------------------
@@ -174,15 +184,18 @@ __global__ void __launch_bounds__(FEW_THREADS) score_few_kernel(const ScoreArgs 
 int few_tiles(const ts_config& c) { return (c.V + FEW_TILE - 1) / FEW_TILE; }
 
 // parents a launch may hold (0: the kernel does not serve this configuration)
-int few_capacity(const ts_config& c) {
-  if (c.dt_U != TS_DTYPE_F32 || c.V % 8 != 0) return 0;
+int few_capacity(const ts_config& c, bool use_tree) {
+  if (c.V % 8 != 0 || (c.dt_U != TS_DTYPE_F32 && !use_tree)) return 0;
+  if (use_tree && c.r > FEW_TREE_RANK) return 0;
+  if (use_tree) return FEW_TREE_ITEMS / few_tiles(c) < FEW_TREE_MAX ? FEW_TREE_ITEMS / few_tiles(c) : FEW_TREE_MAX;
   const size_t per = (size_t)few_tiles(c) * rec_words(c.K) * 4, cap = ((size_t)4 << 20) / per;
   return cap > 256 ? 256 : (int)cap;
 }
 
 cudaError_t launch_score_few(const ts_ctx* ctx, const ScoreArgs& a, int p_bound, cudaStream_t st) {
   const dim3 grid(few_tiles(ctx->cfg), (p_bound + FEW_WARPS - 1) / FEW_WARPS > 0 ? (p_bound + FEW_WARPS - 1) / FEW_WARPS : 1);
-  const cudaError_t e = launch_kernel(score_few_kernel, grid, dim3(FEW_THREADS), 0, st, a.pdl != 0, a);
+  const cudaError_t e = ctx->cfg.dt_U == TS_DTYPE_F32 ? launch_kernel(score_few_kernel<float>, grid, dim3(FEW_THREADS), 0, st, a.pdl != 0, a)
+                                                      : launch_kernel(score_few_kernel<__nv_bfloat16>, grid, dim3(FEW_THREADS), 0, st, a.pdl != 0, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -1606,7 +1606,8 @@ static TreeWs tree_ws(const ts_ctx* ctx, int nreq, int cap, bool expand, int row
 size_t tree_ws_bytes(const ts_ctx* ctx, int B) {
   const int cap = B * ctx->cfg.Nmax > B ? B * ctx->cfg.Nmax : B;
   const size_t e = tree_ws(ctx, B, cap, true, B * ctx->cfg.D).total, g = tree_ws(ctx, cap, cap, false, B * ctx->cfg.D).total;
-  return e > g ? e : g;
+  const size_t t = e > g ? e : g, f = ctx->few_cap > 0 ? score_scratch_bytes(ctx, ctx->few_cap, nullptr) : 0;   // (short lists: ts_score_few.cu)
+  return t > f ? t : f;
 }
 
 // scratch of a scoring call over P given parents; 0: not possible without the caller's workspace (padded copies)

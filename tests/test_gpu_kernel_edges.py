@@ -85,6 +85,15 @@ def test_few_parents_edges(V, P):
     check_scores("f32", V, 4, 8, P, 1.0)
 
 
+# bf16 lists up to what goes to the few-parents kernel (by parents, by pairs of parent and tile, by rank), and one more; the
+# same lengths on the tensor cores
+@pytest.mark.parametrize("V,r,P,mode", [(2048, 8, 64, 0), (2048, 8, 65, 0), (64000, 24, 11, 0), (64000, 24, 12, 0), (64000, 24, 13, 0), (1000, 128, 5, 0),
+                                        (1000, 136, 5, 0), (1001, 64, 5, 0), (2048, 8, 1, binding.TEST_NO_FEW), (2048, 8, 32, binding.TEST_NO_FEW)])
+def test_short_bf16_lists(V, r, P, mode):
+    for T in (0.0, 0.7):
+        check_scores("bf16", V, r, 8, P, T, mode)
+
+
 @pytest.mark.parametrize("over,theta,T,mode", [
     (dict(V=3000, B=3, Nmax=96, K=8, D=6, r=16), 0.005, 0.7, 0),            # the last size of the single-owner form
     (dict(V=3001, B=3, Nmax=97, K=16, D=6, r=16), 0.005, 0.7, 0),           # shared merges and seed bounds, ragged rows
