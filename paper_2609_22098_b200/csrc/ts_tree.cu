@@ -1365,7 +1365,6 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
     int P = nreq;
     if (d >= 0) {
     if (d > 0) P = __ldcg(a.lvl_count + d);
-    else if (a.score_P == 0 && cta == 0 && tid == 0) a.lvl_count[0] = a.B;   // (read by the owners, after the scan's barrier)
     if (P <= 0) break;
     // ---- scan ---------------------------------------------------------------------------------------------------------
     if (tlen > 0) {

@@ -13,7 +13,6 @@
 //   runs that reduction for all requests that just rejected, each CTA owning a vocabulary range;
 //   q is recomputed from U, A, W, no per-node vocabulary vector is stored.  The bonus token is the
 //   inverse CDF of the final residual in token order: range sums locate the range, one CTA rescans it.
-#include <cooperative_groups.h>
 #include <math.h>
 
 #include "ts_internal.h"
@@ -406,34 +405,6 @@ __device__ void advance(const VerifyArgs& a, int b, int lane, int parity, bool c
   __syncwarp();
 }
 
-// logits of up to G parents for the VEC tokens at v (global W, coalesced 16-byte loads)
-template <typename TIn, int G>
-__device__ __forceinline__ void logits_group(const VerifyArgs& a, const float* as, int ng, const int* rq_req,
-                                             const int* rq_dep, int v, float (*acc)[8], const TIn* Wsrc, size_t wstride,
-                                             int woff) {
-  constexpr int VEC = Elem<TIn>::VEC;
-  const TIn* Ug = reinterpret_cast<const TIn*>(a.U);
-  for (int g = 0; g < G; ++g) {
-    if (g < ng) {
-      const TIn* u = Ug + ((size_t)rq_req[g] * a.D + rq_dep[g]) * a.V + v;
-      if (sizeof(TIn) == 2) { const uint4 x = __ldg(reinterpret_cast<const uint4*>(u)); unpack_bf16x8(x, acc[g]); }
-      else { const float4 x = __ldg(reinterpret_cast<const float4*>(u)); acc[g][0] = x.x; acc[g][1] = x.y; acc[g][2] = x.z; acc[g][3] = x.w; }
-    }
-  }
-  for (int k = 0; k < a.r; ++k) {
-    float w[8];
-    // W comes from the CTA's shared-memory copy of its vocabulary range when that fits, else from global
-    if (sizeof(TIn) == 2) { const uint4 x = *reinterpret_cast<const uint4*>(Wsrc + (size_t)k * wstride + woff); unpack_bf16x8(x, w); }
-    else { const float4 x = *reinterpret_cast<const float4*>(Wsrc + (size_t)k * wstride + woff); w[0] = x.x; w[1] = x.y; w[2] = x.z; w[3] = x.w; }
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const float ak = as[g * RMAX + k];
-#pragma unroll
-      for (int i = 0; i < VEC; ++i) acc[g][i] = fmaf(ak, w[i], acc[g][i]);
-    }
-  }
-}
-
 template <typename TIn>
 __device__ __forceinline__ float logit_scalar(const VerifyArgs& a, int req, int dep, int ptok, int w) {
   const TIn* Wg = reinterpret_cast<const TIn*>(a.W);
@@ -521,7 +492,6 @@ constexpr int WT = 288;       // threads of the walk kernel
 // The walk proper.  Returns false when a bounded wait ran out (every thread of the CTA returns the same).
 template <typename TIn>
 __device__ __forceinline__ bool walk_body(const VerifyArgs& a, unsigned char* w_raw) {
-  __shared__ float s_a[VG * RMAX];
   __shared__ int s_req[VG], s_dep[VG], s_node[VG];
   __shared__ float s_C[VG], s_zmax[VG], s_zlogs[VG], s_lseT[VG];
   __shared__ float s_red[VG][WT / 32];
@@ -694,52 +664,20 @@ __device__ __forceinline__ bool walk_body(const VerifyArgs& a, unsigned char* w_
         s_lseT[tid] = a.node_lseT[(size_t)b * (N + 1) + v + 1];
       }
       __syncthreads();
-      for (int i = tid; i < ng * a.r; i += WT) {
-        const int g = i / a.r, k = i % a.r;
-        const int v = s_node[g];
-        const int ptok = v < 0 ? a.anchor[s_req[g]] : a.tok[(size_t)s_req[g] * N + v];
-        s_a[g * RMAX + k] = Elem<TIn>::to_f(Ag[(size_t)ptok * a.r + k]);
-      }
-      __syncthreads();
       float sum[VG];
 #pragma unroll
       for (int g = 0; g < VG; ++g) sum[g] = 0.f;
-      bool need_q = false;
-      for (int g = 0; g < ng; ++g) need_q |= (s_C[g] != 0.f);
-      if (vec_ok) {
-        for (int v = v_lo + tid * VEC; v < v_hi; v += WT * VEC) {
-          float acc[VG][8];
-          if (need_q) logits_group<TIn, VG>(a, s_a, ng, s_req, s_dep, v, acc, ws_ok ? Ws : Wg,
-                                            ws_ok ? (size_t)a.vt_TV : (size_t)a.V, ws_ok ? v - v_lo : v);
-#pragma unroll
-          for (int g = 0; g < VG; ++g) {
-            if (g < ng) {
-              const int64_t row = a.z_row_off[s_req[g]] + s_node[g] + 1;
-              float z[8];
-              if (sizeof(TIn) == 2) { const uint4 x = __ldg(reinterpret_cast<const uint4*>(Zg + row * a.V + v)); unpack_bf16x8(x, z); }
-              else { const float4 x = __ldg(reinterpret_cast<const float4*>(Zg + row * a.V + v)); z[0] = x.x; z[1] = x.y; z[2] = x.z; z[3] = x.w; }
-#pragma unroll
-              for (int i = 0; i < VEC; ++i) {
-                const float p = __expf((z[i] - s_zmax[g]) * invT - s_zlogs[g]);
-                const float q = s_C[g] != 0.f ? __expf(acc[g][i] * invT - s_lseT[g]) : 0.f;
-                sum[g] += fmaxf(p - s_C[g] * q, 0.f);
-              }
-            }
+      for (int v = v_lo + tid; v < v_hi; v += WT) {
+        for (int g = 0; g < ng; ++g) {
+          const int b = s_req[g];
+          const int64_t row = a.z_row_off[b] + s_node[g] + 1;
+          const float p = __expf((z_elem<TIn>(a, row, v) - s_zmax[g]) * invT - s_zlogs[g]);
+          float q = 0.f;
+          if (s_C[g] != 0.f) {
+            const int ptok = s_node[g] < 0 ? a.anchor[b] : a.tok[(size_t)b * N + s_node[g]];
+            q = __expf(logit_scalar<TIn>(a, b, s_dep[g], ptok, v) * invT - s_lseT[g]);
           }
-        }
-      } else {
-        for (int v = v_lo + tid; v < v_hi; v += WT) {
-          for (int g = 0; g < ng; ++g) {
-            const int b = s_req[g];
-            const int64_t row = a.z_row_off[b] + s_node[g] + 1;
-            const float p = __expf((z_elem<TIn>(a, row, v) - s_zmax[g]) * invT - s_zlogs[g]);
-            float q = 0.f;
-            if (s_C[g] != 0.f) {
-              const int ptok = s_node[g] < 0 ? a.anchor[b] : a.tok[(size_t)b * N + s_node[g]];
-              q = __expf(logit_scalar<TIn>(a, b, s_dep[g], ptok, v) * invT - s_lseT[g]);
-            }
-            sum[g] += fmaxf(p - s_C[g] * q, 0.f);
-          }
+          sum[g] += fmaxf(p - s_C[g] * q, 0.f);
         }
       }
 #pragma unroll
