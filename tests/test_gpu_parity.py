@@ -26,7 +26,7 @@ def small(name, **kw):
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("V,r,K", [(1000, 7, 4), (1003, 16, 8), (4096 + 40, 64, 8), (70000, 32, 16), (8, 4, 4), (5, 3, 8),
                                    (9000 + 16, 256, 8), (3000, 200, 4),     # the paper's rank, and one that pads to it
-                                   (45000 + 8, 256, 8)])                   # more vocabulary tiles than SMs: a CTA takes several in turn
+                                   (45000 + 8, 256, 8)])                   # ranges of several blocks of W at the largest rank
 @pytest.mark.parametrize("T", [0.0, 0.7, 1.0])
 @pytest.mark.parametrize("P", [11, 3])   # 3: the few-parents kernel where the context has one
 def test_score_parents_matches_oracle(dtype, V, r, K, T, P, test_mode=0):
@@ -195,14 +195,19 @@ def test_a_request_that_accepts_a_full_depth_path_beside_requests_that_reject(dt
     assert full >= 1, "no round accepted the whole chain: the case under test was not reached"
 
 
-@pytest.mark.parametrize("mode", ["TEST_FORCE_FMA", "TEST_NO_TMA", "TEST_NO_FEW", "TEST_NO_SEED", "TEST_PERSIST", "TEST_NO_UMMA", "TEST_NO_TAIL"])
-def test_alternative_kernel_paths_match_oracle(mode):
-    """bf16 inputs on the fp32-FMA kernels; the tensor-core kernels with W staged by plain loads (the path
-    taken when no tensor map can be encoded); every level on the tile kernel; the tile kernel without seeded
-    bounds; every level inside one cooperative launch, or none of them (by default the levels from the fifth on): chosen by the library's
-    test switches."""
+@pytest.mark.parametrize("mode,over", [
+    ("TEST_FORCE_FMA", {}), ("TEST_FORCE_FMA", dict(V=20001)), ("TEST_NO_TMA", {}), ("TEST_NO_SEED", {}),
+    ("TEST_NO_FEW", dict(dtype="f32", B=1)),
+    ("TEST_NO_SEED", dict(Nmax=128)), ("TEST_NO_TMA", dict(Nmax=128)),
+    ("TEST_NO_SEED", dict(V=9000, B=66, Nmax=16, D=4)), ("TEST_NO_TMA", dict(V=9000, B=66, Nmax=16, D=4)),
+])
+def test_alternative_kernel_paths_match_oracle(mode, over):
+    """bf16 inputs on the fp32-FMA kernels (aligned and ragged rows); the tensor-core kernels with W staged by plain loads
+    (the path taken when no tensor map can be encoded) or without seeded bounds, in each of the expansion's three
+    instantiations (few nodes, shared owners, base logits through a ring -- without a tensor map the last is not taken); fp32
+    levels of few parents on the tile kernel: chosen by the library's test switches."""
     from paper_2609_22098_b200 import binding
-    wl = small("serve32", V=20000, B=5)
+    wl = small("serve32", **dict(dict(V=20000, B=5), **over))
     rnd = Round(wl, seed=77)
     ts = make_gpu(wl, rnd.table, max_batch=rnd.B, test_mode=getattr(binding, mode))
     orc = make_oracle(wl, rnd.table)
@@ -534,21 +539,20 @@ def test_gpu_losslessness_chi_square():
 
 
 @pytest.mark.parametrize("T", [0.0, 1.0])
-@pytest.mark.parametrize("persist", [True, False])
-def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(T, persist):
+@pytest.mark.parametrize("over", [{}, dict(Nmax=128), dict(V=9000, B=66, Nmax=16, D=4)])   # the expansion's three instantiations
+def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(T, over):
     """Bounded device-side waits: with the test switch that makes barriers expect one arrival more than will ever
     come (and shortens the limit to a few thousand polls) the kernels give up, every call returns, the requests
     are reported with TS_ERR_TIMEOUT, and the same context then runs an ordinary round correctly."""
     from paper_2609_22098_b200 import binding
-    wl = small("serve32", V=20000, B=6)
+    wl = small("serve32", **dict(dict(V=20000, B=6), **over))
     rnd = Round(wl, seed=91)
-    base = binding.TEST_PERSIST if persist else 0
-    ts = make_gpu(wl, rnd.table, max_batch=rnd.B, test_mode=base)
+    ts = make_gpu(wl, rnd.table, max_batch=rnd.B)
     orc = make_oracle(wl, rnd.table)
     good = ts.expand_tree(rnd.U, rnd.A, rnd.W, rnd.anchor, rnd.theta, T, 5)
     Z, off = rnd.target_logits(good)
     torch.cuda.synchronize()
-    ts.set_test_mode(base | binding.TEST_SHORT_WAITS | binding.TEST_LOST_ARRIVAL)
+    ts.set_test_mode(binding.TEST_SHORT_WAITS | binding.TEST_LOST_ARRIVAL)
     bad_tree = ts.expand_tree(rnd.U, rnd.A, rnd.W, rnd.anchor, rnd.theta, T, 5)
     torch.cuda.synchronize()
     assert (bad_tree["status"].cpu() == -5).all(), bad_tree["status"]          # TS_ERR_TIMEOUT, and the call came back
@@ -556,7 +560,7 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(T, persis
         bad_verdict = ts.verify_tree(rnd.U, rnd.A, rnd.W, Z, off, rnd.anchor, good, T, 5)
         torch.cuda.synchronize()
         assert (bad_verdict["status"].cpu() == -5).all(), bad_verdict["status"]
-    ts.set_test_mode(base)
+    ts.set_test_mode(0)
     for rs in range(2):
         st = check_round(ts, orc, rnd, T, round_seed=40 + rs)
         assert st["nodes"] > 0
