@@ -10,6 +10,9 @@
  *   - Every function returns a status (TS_OK = 0, negative = error).  No exception crosses the ABI.
  *   - Pointers marked DEVICE are CUDA device addresses owned by the caller and must be 16-byte
  *     aligned; pointers marked HOST are host addresses read during the call only.
+ *   - Cooperative launches with one block per SM of the device: the walk of ts_verify_tree (T > 0), and in bf16
+ *     ts_expand_tree and ts_score_parents (lists of more than a few parents; ranks that are multiples of 8).  A
+ *     stream whose partition has fewer SMs than the device gets TS_ERR_CUDA from them.
  *   - The three hot calls allocate nothing, never synchronise with the host and enqueue all work on
  *     the caller's stream (a cudaStream_t passed as void*).  Scratch memory is the caller's
  *     workspace of at least ts_workspace_bytes() bytes; its contents are undefined between calls.
@@ -90,7 +93,7 @@ int32_t ts_set_ablation(ts_ctx* ctx, uint32_t flags);
  * TS_ERR_UNSUPPORTED (the forced path has no tiling for this configuration), TS_ERR_CUDA.
  *   TS_TEST_FORCE_FMA     bf16 inputs run on the fp32 fused-multiply-add kernels (no tensor cores)
  *   TS_TEST_NO_TMA        the tensor-core kernels stage W with plain loads (no tensor map)
- *   TS_TEST_NO_FEW        levels with few parents run on the tile kernel too
+ *   TS_TEST_NO_FEW        short lists run on the tile kernel (fp32) or the tensor cores (bf16) too
  *   TS_TEST_NO_SEED       the tensor-core scoring kernel runs without seed bounds
  *   TS_TEST_PERSIST, TS_TEST_NO_TAIL, TS_TEST_NO_UMMA
  *                         accepted without effect: they chose between forms of the tensor-core expansion, which now
@@ -98,7 +101,7 @@ int32_t ts_set_ablation(ts_ctx* ctx, uint32_t flags);
  *   TS_TEST_SHORT_WAITS   bounded waits give up after 4096 polls instead of 2^22
  *   TS_TEST_LOST_ARRIVAL  the grid barriers of the walk and of the tensor-core scoring kernel expect one
  *                         arrival more than will come: the waits run out, the kernels return, and the
- *                         requests are reported with TS_ERR_TIMEOUT in status[] */
+ *                         requests are reported with TS_ERR_TIMEOUT in status[] (given parents: by NaN) */
 #define TS_TEST_FORCE_FMA 1u
 #define TS_TEST_NO_TMA 2u
 #define TS_TEST_NO_FEW 4u
@@ -155,11 +158,13 @@ int32_t ts_score_parents(ts_ctx* ctx, const void* U, const void* A, const void* 
  * cudaFree or other allocating call, and the results are the same as ts_score_parents'.
  *
  * Limits and rules:
- *   - The array bounds P: every parent slot needs one record of (4 + 5K) words (rounded up to 16 bytes)
- *     per vocabulary tile, plus its pruning-bound words (2K lines of 128 bytes), the array also holds 1 MiB
- *     of scratch for the seed-bound kernel, and slots come in blocks of 128 on the tensor-core path: 256
- *     parents for a 152k vocabulary with K = 8 in bf16 (140 tiles), a few hundred on the fp32 path.  A
- *     larger P is refused with TS_ERR_WORKSPACE and a message that names the limit; nothing is launched.
+ *   - The array bounds P.  Every parent needs 2K lines of 128 bytes for its pruning bounds and, on the tensor
+ *     cores, 16 + 20K bytes per vocabulary range (one range per SM at most; room for 128 parents at least) and
+ *     8 bytes per 1024 tokens; on the other kernels a record of (4 + 5K) words (rounded up to 16 bytes) per
+ *     vocabulary tile.  That is about 300 parents for a 152k vocabulary with K = 8 in bf16, a few hundred in
+ *     fp32.  A larger P is refused with TS_ERR_WORKSPACE and a message that names the limit; nothing is launched.
+ *   - bf16 vocabularies that are no multiple of 8 are scored by fused multiply-adds here (there is no room for
+ *     padded copies); TS_ERR_UNSUPPORTED where no tile of W fits shared memory.
  *   - The context's device must be the current device.
  *   - The first call on a device looks up the array's device address (cudaGetSymbolAddress) and
  *     remembers it; make that first call before starting any stream capture.

@@ -75,7 +75,7 @@ struct ts_ctx {
   int use_walk;     // 1: the walk's reductions may run on the tensor cores
   int use_tree;     // 1: expansion and scoring run on the one-launch tensor-core kernel
   int vt_TV, vt_n;  // vocabulary ranges of the verification walk, one per CTA
-  int few_cap;      // levels with at most this many parents run on the few-parents kernel instead (0: none)
+  int few_cap;      // lists of at most this many parents run on the few-parents kernel instead (0: none)
   ts::DevCalib calib;
   void* prof;  // ts::Prof*, instrumentation state
   // tensor-map descriptor of the W matrix last scored with (bulk-tensor loads of the W tile); -1: the

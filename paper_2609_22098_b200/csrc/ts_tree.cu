@@ -12,7 +12,7 @@
 //          logits of the level after (best token of every 1024: where the next seed bounds come from).
 // Before this, a level was three dependent launches (scan with its own set-up, merge of fixed-size records, level
 // step on global-memory state): about 70 us per level at 32 requests, V = 151,936, r = 64, of which the arithmetic
-// needs less than ten.  Now (serve shape: 32 requests, 16 nodes): about 9 to 28 us of scan, 17 us of owner phase and two
+// needs less than ten.  Now (serve shape: 32 requests, 16 nodes): 9 to 31 us of scan, 13 to 20 us of owner phase and two
 // grid barriers of 1.2 to 2.3 us per level, 206 us for the expansion with its set-up launch (365 before).
 //
 // Bounds.  Per parent K slots in global memory, slot j = best value published by the pieces (range, split, replica)
@@ -595,7 +595,8 @@ __device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, co
 // preserving image, then the inverted token among its ties) and one removal.
 __device__ __noinline__ float3 warp_topk(const uint2* cand, const float* lgs, const int* count, int K, int lane) {
   uint32_t wv = 0u, wt = 0u; float wl = 0.f;   // winner `lane` so far: 0 = none
-  // the first 64 entries are requested together with the count (there is always room for 128 of them)
+  // the first 64 entries are requested together with the count (past a short segment they are a neighbour's, and past the
+  // last one's another array of the workspace: not used, and always inside it)
   const int n = __ldcg(count);
   const uint2 pre0 = __ldcg(cand + lane), pre1 = __ldcg(cand + 32 + lane);
   const float pl0 = lgs ? __ldcg(lgs + lane) : 0.f, pl1 = lgs ? __ldcg(lgs + 32 + lane) : 0.f;
@@ -1098,7 +1099,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       if (live(e) && skey(key_of(e)) == prefix) { const int at = atomicAdd(&sh[4], 1); if (at < 256) s.newl[at] = e; }
     __syncthreads();
     const int ntie = whole ? 0 : sh[4];
-    unsigned drop = 0u;   // bit per trip: M <= 17 * 256 entries, at most 7 trips
+    unsigned drop = 0u;   // bit per trip: M <= 17 * 256 entries, at most 8 trips
 #pragma unroll 1
     for (int e = tid, it = 0; e < M; e += TX_THREADS, ++it) {
       if (!live(e)) continue;
@@ -1431,7 +1432,8 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
       break;
     }
     }
-    // ---- merge by all CTAs where the owners alone would take long over it (8 requests with 60 parents each: 150 us) -------
+    // ---- merge by all CTAs where the owners alone would take long over it (8 requests with 60 parents each: 150 us; from 4
+    // parents a request on instead of 8 the extra barrier costs up to 7 %, from 16 on within 2 % either way) ---------------
     const bool spread = MANY && d >= 0 && P > 8 * a.B;
     if (spread) {
       const int R = mma_replicas(P), K = a.K;
@@ -1634,7 +1636,10 @@ static void fill_args(ts_ctx* ctx, TreeArgs& a, char* base, const TreeWs& w, boo
 }
 
 static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream_t st) {
-  // crowded levels (a request with dozens of parents) need room for them in the tree and CTAs to spare
+  // Crowded levels (a request with dozens of parents) need room for them in the tree and CTAs to spare.  Expansion, owners
+  // alone / sharing (us): K = 16, flat logits, Nmax 96: 331 / 257 for 1 request, 591 / 520 for 8, 1,916 / 1,918 for 64; Nmax
+  // 256: 607 / 378, 1,140 / 894, 3,824 / 3,693.  Where levels are not crowded sharing costs 2 to 8 %, at any Nmax: 222 / 239 for
+  // 32 requests of 16 nodes at Nmax 96, 226 / 245 at 128; with K = 8 it does not pay up to Nmax 128 (640 / 679 and 759 / 792 for 32).
   const bool many = a.score_P == 0 && ctx->num_sms >= 2 * a.B && a.N > 96;
   CUtensorMap tm, tmU;
   memset(&tm, 0, sizeof(tm)); memset(&tmU, 0, sizeof(tmU));

@@ -20,7 +20,9 @@ constexpr int TX_PLACE_BITS = 17;          // of a queued candidate's place in t
 constexpr int TX_STAGE_MAX = 8;            // stages of the W ring
 constexpr int TX_USTAGES = 4;              // stages of the base-logit ring (two: the chain of 128 requests 674 us, four: 581)
 constexpr int TX_RING_MIN = TX_ROWS / 2 + 1;   // smallest batch that takes it: from here on a root level fills a tile's 128 rows alone
-constexpr int TX_SOLO = 16;                // new parents whose seed bounds an owner makes itself
+                                              // (direct / ring, us, V = 151,936, r = 64: 64 requests 280 / 296, chains 353 / 382; 80: 327 / 304,
+                                              // 572 / 458; 128: 458 / 429, 763 / 556; r = 256: 80 452 / 468, 128 646 / 655; V = 32,000: equal)
+constexpr int TX_SOLO = 16;                // new parents whose seed bounds an owner makes itself (8: up to 6 % slower, 384 -> 409 us at 32 requests, Nmax 128; 32: within 1 %)
 constexpr int TX_PIECE = 1024;             // tokens of one scouting item
 
 // Everything the scan needs to know about one parent.

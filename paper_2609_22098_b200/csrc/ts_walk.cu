@@ -14,7 +14,8 @@
 // When no request asks any more, every owner draws its requests' bonus tokens by itself: the range from the stored
 // range sums, then the token inside it.  Two barriers a step and none at the start and the end.
 //
-// Measured at 32 requests, V = 151,936, r = 64 (8 steps): see the notes at the phases.
+// Measured at 32 requests, V = 151,936, r = 64 (11 to 12 steps): 11.5 us a step -- advance 2 to 3, barriers 1.1 and 1.5,
+// operands 1.5, the pass about 5.
 #include <math.h>
 #include <string.h>
 
