@@ -865,7 +865,7 @@ extern "C" int32_t ts_verify_tree(ts_ctx* ctx, const void* U, const void* A, con
       w.anchor = anchor_tok; w.n_nodes = n_nodes; w.tok = tok; w.parent = parent; w.depth = depth; w.node_hash = node_hash;
       w.logqT = logqT; w.node_lseT = node_lseT; w.z_part = a.z_part; w.z_np = a.z_np;
       w.acc_len = acc_len; w.acc_node = acc_node; w.acc_tok = acc_tok; w.bonus = bonus_tok; w.edge_stat = edge_stat; w.flags = flags; w.status = status;
-      w.part = a.part; w.barrier = a.barrier; w.vt_TV = a.vt_TV; w.vt_n = a.vt_n; w.max_steps = a.max_steps;
+      w.barrier = a.barrier; w.vt_TV = a.vt_TV; w.vt_n = a.vt_n; w.max_steps = a.max_steps;
       w.wait_limit = a.wait_limit; w.lost_arrival = a.lost_arrival; w.use_tma = tma ? 1 : 0;
       e = launch_walk_mma(ctx, w, ws + L.walk, wp, st);
       return e == cudaSuccess ? TS_OK : set_cuda_error("ts_verify_tree(walk)", e);

@@ -3,8 +3,8 @@
 //
 // A request's walk is a scalar sequence (see ts_verify.cu for the algebra): sibling tests until one is accepted or a
 // rejection needs Z = sum_w max(p(w) - C q(w), 0).  A step of the kernel is
-//   advance   one warp per request, in the CTA that owns it, runs the scalar sequence on state in shared memory and
-//             publishes what its next reduction needs (48 bytes a request, no list and no counter);
+//   advance   the CTA that owns a request adds up its range sums, and one of its warps runs the scalar sequence on state in
+//             shared memory and publishes what its next reduction needs (80 bytes a request, no list and no counter);
 //   barrier
 //   reduce    every CTA reads those records and sums its range for all requests that asked: the draft logits are one MMA
 //             tile per 128 tokens with the TOKENS on the 128 rows (W is the A operand, as it lies in memory) and the
@@ -14,8 +14,9 @@
 // When no request asks any more, every owner draws its requests' bonus tokens by itself: the range from the stored
 // range sums, then the token inside it.  Two barriers a step and none at the start and the end.
 //
-// Measured at 32 requests, V = 151,936, r = 64 (11 to 12 steps): 11.5 us a step -- advance 2 to 3, barriers 1.1 and 1.5,
-// operands 1.5, the pass about 5.
+// Measured at 32 requests, V = 151,936, r = 64 (one of them rejects eight siblings): 108 us in five steps, 146 in nine with one
+// coefficient a reduction.  A step: sums and advance 3 to 7 (predictions), barriers 1.1 and 1.5, operands 2, the pass 18 (all requests, grid),
+// 12 and 10 (a few, eight coefficients), 3 (one request, one coefficient).  Set-up 6, bonus draws 12.
 #include <math.h>
 #include <string.h>
 
@@ -26,23 +27,33 @@ namespace ts {
 constexpr int WK_EPI = 16;                 // warps that read accumulators: 4 lane quarters x 4 sets of tiles
 constexpr int WK_LOAD = WK_EPI;            // tensor memory; in the streaming form it requests W and issues the MMAs
 constexpr int WK_THREADS = (WK_EPI + 1) * 32;
-constexpr int WK_REQ = 64;                 // requests of one reduction pass (columns of a tile)
-constexpr int WK_BUF = 8;                  // accumulator buffers of WK_REQ columns: two per set of tiles
+constexpr int WK_REQ = 32;                 // requests of one reduction pass (columns of a tile)
+constexpr int WK_TR = 3;                   // tiles of a set in tensor memory together: a round is 12 tiles of 32 columns
+constexpr int WK_ROUND = 4 * WK_TR;
+constexpr int WK_VALS = 2 * WK_COLS;       // sums of a request: residual and proposal mass at every coefficient
+constexpr int WK_SLOTS = 6;                // requests whose rows a warp has in flight or in work: three pairs
+constexpr int WK_GRID = 16;                // beside the number of coefficients: all but the first are guesses from the grid
+__host__ __device__ constexpr int wk_seg(bool aligned) { return aligned ? 64 : 80; }   // bytes of a staged segment: 32 tokens that, unaligned, may start anywhere in a 16-byte chunk
+__host__ __device__ constexpr int wk_slot(bool aligned) { return 2 * WK_TR * wk_seg(aligned); }
 constexpr int WK_CHUNK = 1088;             // tokens of one step of the bonus rescan: 8 tokens x 136 places x 4 slices of the rank
+constexpr double WK_TOL = 9.5367431640625e-7;   // 2^-20: a coefficient this close (relative) to an evaluated one counts as evaluated
 
-struct RedDesc { const __nv_bfloat16 *z, *u; float C, zoff, qoff; int b; };
-static_assert(sizeof(RedDesc) == 32, "two 16-byte loads");
+struct __align__(16) RedDesc { const __nv_bfloat16 *z, *u; float zoff, qoff; int b, nC; float C[WK_COLS]; };
+static_assert(sizeof(RedDesc) == 64, "four 16-byte loads");
 
 // The walk of one request.
 struct WalkState {
   int cur, j, acc, nf, npass, phase;       // phase: 0 walking, 1 waits for the sum after a rejection, 2 waits for the sum of the bonus draw, 3 walk over, 4 not walked
   int cfirst, ccnt;
+  int nC, pcol;                            // coefficients of the last reduction (| WK_GRID); the one that the bonus draw's range sums belong to
+  float col[WK_COLS];
   double C, Zj, Qused, passC, partsC;      // partsC: the C that the stored range sums were computed for (-1: none)
+  double S[WK_VALS];                       // the last reduction's sums
   int fx[KMAX]; double fC[KMAX], fp[KMAX], fq[KMAX];
 };
 
 struct WalkSm {
-  unsigned char *Ws, *Bs; WalkState* st;
+  unsigned char *Ws, *Bs, *stage; float* part; WalkState* st;
   uint64_t *t_full, *t_empty, *w_full, *w_free; uint32_t* tmem; volatile int* abort;
 };
 
@@ -111,7 +122,7 @@ __device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const
   if (tid == 0) {
     st.cur = -1; st.j = 0; st.acc = 0; st.nf = 0; st.npass = 0; st.phase = 0;
     st.C = 0.0; st.Zj = 1.0; st.Qused = 0.0; st.passC = 0.0; st.partsC = -1.0;
-    st.cfirst = -1; st.ccnt = 0;
+    st.cfirst = -1; st.ccnt = 0; st.nC = 0; st.pcol = 0;
     if (okn && !bad) { const int2 c = a.child[cb]; st.cfirst = c.x; st.ccnt = c.y; }
     a.flags[b] = 0u;
     a.status[b] = !okn ? TS_ERR_INVALID : (bad ? TS_ERR_NUMERIC : TS_OK);
@@ -121,136 +132,213 @@ __device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const
 }
 
 // ---- one request's scalar sequence, by one warp ------------------------------------------------------------------------
-// Everything it may need -- the range sums, the current node's children, the record of the current node -- is requested
-// together: one memory round trip a step, and one more for every node it descends to.
+// Everything it may need -- the reduction's sums, the current node's children, the record of the current node -- is
+// requested together: one memory round trip a step, and one more for every node it descends to.
+//
+// Several coefficients a reduction.  Rejecting sibling after sibling at one node needs F(C) = sum_w max(p - C q, 0) at
+// C_1 = 1 < C_2 < ..., and C_(i+1) follows from F(C_i): one reduction after the other, 8 (K = 8) or 16 steps for a request
+// that rejects all children, and the slowest request sets the length of the launch.  But F is convex with slope -G(C),
+// G = the proposal mass where the residual is positive, and nothing in the sequence depends on the uniforms.  So a reduction evaluates
+// F and G at several coefficients: the one that is needed, and guesses of the ones after it.  At first the guesses are a
+// fixed grid (there the sums are of |p - C q|, two instructions a token and coefficient: F = (1 - C + sum |p - C q|) / 2, good
+// enough for guesses); from its values (cubic interpolation of what the node's other tokens give; the children's own terms are known
+// exactly) the rest of the sequence is predicted, evaluated, and where a prediction was within 2^-20 of what its
+// predecessors turn out to give, F there is F and G at the prediction, to first order: the term left out is at most the step times the mass
+// whose ratio p / q lies inside the step, less than the rounding of the exponentials in any case.  Where it was not, the next reduction
+// evaluates the corrected predictions (errors go down quadratically).  A node's eight rejections take three reductions, sixteen take four or five.
+__device__ __forceinline__ double wk_lanes_sum(double x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
+  return x;
+}
 __device__ __forceinline__ void wk_advance(const WalkArgs& a, WalkState& st, const int b, const int lane, const int stamp) {
   const int N = a.N;
   const size_t nb = (size_t)b * N, cb = (size_t)b * (N + 1);
   WalkRec* rec = a.rec + b;
   if (st.phase >= 3) { if (lane == 0) rec->stamp = 0; return; }
   int v = st.cur, first = st.cfirst, m = st.ccnt;
-  WalkEdge e; e.px = 0.0; e.qx = 1.0; e.u = 0.0; e.x = -1;
+  WalkEdge e;
   auto fetch = [&]() {
+    e.px = 0.0; e.qx = 1.0; e.u = 0.0; e.x = -1;
     if (lane < m) { const uint4* s = reinterpret_cast<const uint4*>(a.edge + nb + first + lane); uint4* d = reinterpret_cast<uint4*>(&e); d[0] = __ldcg(s); d[1] = __ldcg(s + 1); }
   };
   fetch();
   uint4 nd = make_uint4(0u, 0u, 0u, 0u);
   if (lane < 2) nd = __ldcg(reinterpret_cast<const uint4*>(a.node + cb + v + 1) + lane);
-  const int phase = st.phase;
-  if (phase) {   // ---- fold in the sum that just ran ----
-    double f = 0.0;
-    const float* part = a.part + (size_t)b * a.vt_n;
-    for (int t0 = 0; t0 < a.vt_n; t0 += 5 * 32) {
-      float pv[5];
-#pragma unroll
-      for (int k = 0; k < 5; ++k) pv[k] = (t0 + k * 32 + lane < a.vt_n) ? __ldcg(part + t0 + k * 32 + lane) : 0.f;
-#pragma unroll
-      for (int k = 0; k < 5; ++k) f += (double)pv[k];
+  const bool grid = (st.nC & WK_GRID) != 0;
+  int kind = st.phase, have = kind ? st.nC & (WK_GRID - 1) : 0;
+  bool fresh = true;   // the first coefficient is passC's own, whatever its value
+  // lane k: the k-th coefficient of the reduction that just ran, and its sums over all tokens but the children
+  double ck = 0.0, Fk = 0.0, Gk = 0.0;
+  if (have) {
+    if (lane < have) { ck = (double)st.col[lane]; Fk = st.S[lane]; Gk = st.S[WK_COLS + lane]; }
+    if (grid && lane > 0 && lane < have) Fk = 0.5 * (1.0 - ck + Fk);   // (both distributions sum to one)
+#pragma unroll 1
+    for (int i = 0; i < m; ++i) {
+      const double p = __shfl_sync(0xFFFFFFFFu, e.px, i), q = __shfl_sync(0xFFFFFFFFu, e.qx, i), t = p - ck * q;
+      if (t > 0.0) { Fk -= t; Gk -= q; }
     }
-    // the pass used passC for every token; tested siblings keep the residual they had when tested
-    if (lane < st.nf) f += fmax(st.fp[lane] - st.fC[lane] * st.fq[lane], 0.0) - fmax(st.fp[lane] - st.passC * st.fq[lane], 0.0);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) f += __shfl_xor_sync(0xFFFFFFFFu, f, off);
-    __syncwarp();
-    if (lane == 0) {
-      if (phase == 1) {
-        if (f <= 1e-30 * st.Zj) {   // the residual lost its mass: keep the previous one
-          a.flags[b] |= TS_FLAG_ZERO_MASS;
-          st.fC[st.nf - 1] = st.C;
-          st.partsC = -1.0;
-        } else { st.C = st.passC; st.Zj = f; st.partsC = st.passC; }
-      } else { st.Zj = f; st.partsC = st.passC; }
-      st.phase = 0;
+    if (have == 1) Gk = 0.0;   // (not computed: the step is the rounding of one coefficient to fp32)
+    else if (grid) {           // slopes by the parabola through a coefficient and its neighbours
+      const int k0 = min(max(lane - 1, 0), have - 3);
+      const double c0 = __shfl_sync(0xFFFFFFFFu, ck, k0), c1 = __shfl_sync(0xFFFFFFFFu, ck, k0 + 1), c2 = __shfl_sync(0xFFFFFFFFu, ck, k0 + 2);
+      const double f0 = __shfl_sync(0xFFFFFFFFu, Fk, k0), f1 = __shfl_sync(0xFFFFFFFFu, Fk, k0 + 1), f2 = __shfl_sync(0xFFFFFFFFu, Fk, k0 + 2);
+      const double d01 = (f1 - f0) / (c1 - c0), d12 = (f2 - f1) / (c2 - c1);
+      Gk = fmax(-(d01 + (d12 - d01) / (c2 - c0) * (2.0 * ck - c0 - c1)), 0.0);
     }
-    __syncwarp();
   }
   for (;;) {
+    if (kind) {   // ---- the sum at passC: from the reduction that just ran, or by another one ----
+      const double C = st.passC;
+      const int nf = st.nf;
+      const unsigned hit = __ballot_sync(0xFFFFFFFFu, lane < have && ((lane == 0 && fresh) || ((lane == 0 || !grid) && fabs(C - ck) <= WK_TOL * C)));
+      fresh = false;
+      // a child's own term: the residual it had when it was tested, or the one it has
+      double own = lane < m ? fmax(e.px - (lane < nf && lane < KMAX ? st.fC[lane] : C) * e.qx, 0.0) : 0.0;
+      if (!hit) {
+        int nC = 1;
+        float mine = (float)C;   // lane k: coefficient k
+        const int need = kind == 2 ? 1 : m - nf + 1;   // sums that this node can still ask for
+        if (need > 1 && !have) {
+          nC = WK_COLS | WK_GRID;
+          constexpr float places[WK_COLS] = {1.f, 1.2f, 1.45f, 1.75f, 2.15f, 2.7f, 3.6f, 5.5f};
+          float g = 1.f;
+#pragma unroll
+          for (int k = 1; k < WK_COLS; ++k) g = lane == k ? places[k] : g;
+          mine = (float)C * g;
+        } else if (need > 1) {
+          // what does not depend on the sequence, by all lanes at once: lane i's 1 / (1 - proposal mass of the siblings before
+          // it), lane k's 1 / (width of interval k)
+          double Q = e.qx;
+          if (lane >= m) Q = 0.0;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) { const double x = __shfl_up_sync(0xFFFFFFFFu, Q, o); if (lane >= o) Q += x; }
+          Q = __shfl_up_sync(0xFFFFFFFFu, Q, 1);
+          if (lane == 0) Q = 0.0;
+          const double inv = Q < 1.0 ? 1.0 / (1.0 - Q) : 0.0;
+          const double next = __shfl_down_sync(0xFFFFFFFFu, ck, 1), rh = lane + 1 < have && next > ck ? 1.0 / (next - ck) : 0.0;
+          double c = C;
+#pragma unroll 1
+          for (int i = nf; i < m && nC < WK_COLS; ++i) {
+            // the other tokens' share at c: between two evaluated coefficients by Hermite's cubic, beyond the last by the decay there
+            const int n = __popc(__ballot_sync(0xFFFFFFFFu, lane < have && ck <= c));
+            const int k0 = n > 0 ? n - 1 : 0, k1 = n < have ? n : have - 1;
+            const double c0 = __shfl_sync(0xFFFFFFFFu, ck, k0), f0 = __shfl_sync(0xFFFFFFFFu, Fk, k0), g0 = __shfl_sync(0xFFFFFFFFu, Gk, k0);
+            const double c1 = __shfl_sync(0xFFFFFFFFu, ck, k1), f1 = __shfl_sync(0xFFFFFFFFu, Fk, k1), g1 = __shfl_sync(0xFFFFFFFFu, Gk, k1);
+            const double w = __shfl_sync(0xFFFFFFFFu, rh, k0), own_sum = wk_lanes_sum(own), scale = __shfl_sync(0xFFFFFFFFu, inv, i);
+            double f;
+            if (n == 0) f = f0 - (c - c0) * g0;
+            else if (n == have) f = f0 > 1e-30 ? f0 * (double)__expf((float)(-(c - c0) * g0) / (float)f0) : 0.0;
+            else {
+              const double h = c1 - c0, t = (c - c0) * w, r = 1.0 - t;
+              f = r * r * (f0 * (1.0 + 2.0 * t) - g0 * h * t) + t * t * (f1 * (3.0 - 2.0 * t) + g1 * h * r);
+            }
+            const double z = fmax(f, 0.0) + own_sum;
+            if (!(z > 1e-30) || scale == 0.0) break;   // uniform
+            c += z * scale;
+            if (lane < m && lane >= i) own = fmax(e.px - c * e.qx, 0.0);   // (sibling i keeps this from now on)
+            if (lane == nC) mine = (float)c;
+            ++nC;
+          }
+        }
+        const int cols = nC & (WK_GRID - 1);
+        if (lane < 2) reinterpret_cast<uint4*>(rec)[lane] = nd;
+        if (lane < WK_COLS) { const float x = lane < cols ? mine : 0.f; rec->C[lane] = x; st.col[lane] = x; }
+        if (lane == 0) { rec->nC = nC; rec->stamp = stamp; st.nC = nC; st.phase = kind; }
+        __syncwarp();
+        return;
+      }
+      const int k = __ffs(hit) - 1;
+      const double c0 = __shfl_sync(0xFFFFFFFFu, ck, k), f0 = __shfl_sync(0xFFFFFFFFu, Fk, k), g0 = __shfl_sync(0xFFFFFFFFu, Gk, k);
+      const double Cf = (double)(float)C;   // (sums are of the coefficient as fp32 holds it, by whichever way they come)
+      const double step = fabs(Cf - c0) <= 2.0 * WK_TOL * Cf ? Cf - c0 : 0.0;   // (one beyond what fp32 holds: no step)
+      const double f = f0 - step * g0 + wk_lanes_sum(own);
+      __syncwarp();
+      if (lane == 0) {
+        st.npass++;
+        if (kind == 1) {
+          if (f <= 1e-30 * st.Zj) {   // the residual lost its mass: keep the previous one
+            a.flags[b] |= TS_FLAG_ZERO_MASS;
+            st.fC[st.nf - 1] = st.C;
+            st.partsC = -1.0;
+          } else { st.C = C; st.Zj = f; st.partsC = C; st.pcol = k; }
+        } else { st.Zj = f; st.partsC = C; st.pcol = k; }
+        st.phase = 0;
+      }
+      kind = 0;
+      __syncwarp();
+    }
     // the sibling chain at node v until one is accepted, a sum is needed, or they run out; all lanes follow it together
-    int j = st.j;
+    const int j = st.j;
     const double C = st.C, c0 = st.Zj, Q = st.Qused;
-    int out = 0;   // 1 accepted, 2 sum after a rejection, 3 sum for the bonus draw, 4 walk over
     if (j < m && st.acc < a.D) {
       const double px = __shfl_sync(0xFFFFFFFFu, e.px, j), qx = __shfl_sync(0xFFFFFFFFu, e.qx, j), u = __shfl_sync(0xFFFFFFFFu, e.u, j);
       const int x = __shfl_sync(0xFFFFFFFFu, e.x, j);
       const double cj = c0 / (1.0 - Q);
       const double rho = fmin(1.0, fmax(px / qx - C, 0.0) / cj);
       __syncwarp();
-      if (u < rho) {
-        out = 1;
+      if (u < rho) {   // descend
         if (lane == 0) {
           a.acc_node[(size_t)b * a.D + st.acc] = first + j; a.acc_tok[(size_t)b * a.D + st.acc] = x;
           st.acc++; st.cur = first + j; st.j = 0; st.C = 0.0; st.Zj = 1.0; st.Qused = 0.0; st.nf = 0; st.partsC = -1.0;
         }
+        v = first + j;
+        const int2 c = __ldcg(a.child + cb + v + 1);
+        first = c.x; m = c.y; have = 0;
+        if (lane < 2) nd = __ldcg(reinterpret_cast<const uint4*>(a.node + cb + v + 1) + lane);
+        if (lane == 0) { st.cfirst = first; st.ccnt = m; }
+        fetch();
       } else {
-        out = 2;
         if (lane == 0) {
           const int k = st.nf;
           st.fx[k] = x; st.fp[k] = px; st.fq[k] = qx; st.fC[k] = C + cj; st.nf = k + 1;
           st.Qused = Q + qx; st.j = j + 1; st.passC = C + cj;
         }
+        kind = 1;
       }
-    } else {
-      out = st.partsC != C ? 3 : 4;
+    } else if (st.partsC != C) {
       __syncwarp();
-      if (lane == 0) { if (out == 3) st.passC = C; else st.phase = 3; }
-    }
-    __syncwarp();
-    if (out != 1) {
-      if (out == 4) { if (lane == 0) rec->stamp = 0; }
-      else {
-        if (lane < 2) reinterpret_cast<uint4*>(rec)[lane] = nd;
-        if (lane == 0) { rec->C = (float)st.passC; rec->stamp = stamp; st.npass++; st.phase = out == 2 ? 1 : 2; }
-      }
+      if (lane == 0) st.passC = C;
+      kind = 2;
+    } else {
+      __syncwarp();
+      if (lane == 0) { st.phase = 3; rec->stamp = 0; }
       __syncwarp();
       return;
     }
-    // descend
-    v = st.cur;
-    const int2 c = __ldcg(a.child + cb + v + 1);
-    first = c.x; m = c.y;
-    if (lane < 2) nd = __ldcg(reinterpret_cast<const uint4*>(a.node + cb + v + 1) + lane);
-    if (lane == 0) { st.cfirst = first; st.ccnt = m; }
-    fetch();
     __syncwarp();
   }
 }
 
-// ---- one reduction pass: sums of max(p - C q, 0) over this CTA's tokens for up to WK_REQ requests ---------------------------
-// The MMAs of one tile into accumulator buffer `buf`, W from slab pair `ws`; an elected lane of the calling warp.
+// ---- one reduction pass: sums over this CTA's tokens for up to WK_REQ requests ------------------------------------------------
+// The MMAs of one tile into accumulator place `slot` of the round, W from slab pair `ws`; an elected lane of the calling warp.
 // Issuing costs about 70 cycles an instruction (400 a tile of rank 64; 600 from a branch on the lane instead of an elected one,
 // and 1200 beside busy warps): one warp for all nine tiles of a pass took longer than the sums, so where W is resident the
 // first warp of every set issues its set's tiles.
-__device__ __forceinline__ void wk_mma(const WalkArgs& a, const WalkSm& sm, const int ncol, const uint32_t ws, const uint32_t buf, const uint32_t tmem_base) {
+__device__ __forceinline__ void wk_mma(const WalkArgs& a, const WalkSm& sm, const int ncol, const uint32_t ws, const uint32_t slot, const uint32_t tmem_base) {
   const int ksteps = (a.r + 15) / 16;
   const uint32_t slab = (uint32_t)((a.r + 63) / 64 * 64) * 128u;
   tc_fence_after();
   if (elect_one()) {
     const uint64_t ad = smem_desc(smem_u32(sm.Ws) + 2u * ws * slab, slab, 1024u), bd = smem_desc(smem_u32(sm.Bs), 16u, 1024u);
-    const uint32_t idesc = wk_idesc(ncol), d = tmem_base + buf * (uint32_t)WK_REQ;
+    const uint32_t idesc = wk_idesc(ncol), d = tmem_base + slot * (uint32_t)WK_REQ;
 #pragma unroll 4
     for (int ks = 0; ks < ksteps; ++ks)
       mma_bf16(d, ad + (uint64_t)(ks * 128), bd + (uint64_t)((ks >> 2) * (WK_REQ * 128 / 16) + (ks & 3) * 2), idesc, ks > 0 ? 1u : 0u);
-    mma_commit(sm.t_full + buf);
+    mma_commit(sm.t_full + slot);
     if (a.ring) mma_commit(sm.w_free + ws);
   }
   __syncwarp();
 }
-// a set's tile number `nt` (counted over all passes) waits until the buffer's tile before last is drained
-__device__ __forceinline__ bool wk_drained(const WalkArgs& a, const WalkSm& sm, const uint32_t buf, const uint32_t nt) {
-  return nt < 2u || __all_sync(0xFFFFFFFFu, wk_wait(sm.t_empty + buf, ((nt >> 1) - 1u) & 1u, a, sm.abort));
-}
-__device__ __forceinline__ bool wk_issue(const WalkArgs& a, const WalkSm& sm, const int ncol, const int t, const int set, const uint32_t nt, const bool first_pass, const uint32_t tmem_base) {
-  const uint32_t buf = (uint32_t)set * 2u + (nt & 1u);
-  if (first_pass && a.use_tma && !__all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + t, 0, a, sm.abort))) return false;
-  if (!wk_drained(a, sm, buf, nt)) return false;
-  wk_mma(a, sm, ncol, (uint32_t)t, buf, tmem_base);
-  return true;
+// a set's accumulators are free for round `rnd` (counted over all passes) when its four warps are done with the round before
+__device__ __forceinline__ bool wk_drained(const WalkArgs& a, const WalkSm& sm, const int set, const uint32_t rnd) {
+  return rnd == 0u || __all_sync(0xFFFFFFFFu, wk_wait(sm.t_empty + set, (rnd - 1u) & 1u, a, sm.abort));
 }
 // Streaming form, one warp: blocks of 128 tokens of W through the ring, one after the other round the range and on into the next
 // pass (W does not depend on which requests that sums), and the tiles in the same order.  (In order, and by one warp: a wait
 // for a parity tells a slot's turns apart only while the waiter follows every one of them.)
 __device__ __forceinline__ void wk_stream(const WalkArgs& a, const WalkSm& sm, const CUtensorMap* tm, const int ncol, const int t0, const int tlen, const uint32_t pass,
-                                          uint32_t& wreq, const uint32_t tmem_base) {
+                                          uint32_t& wreq, uint32_t rnd, const uint32_t tmem_base) {
   const int ntile = (tlen + 127) / 128;
   const uint32_t slab = (uint32_t)((a.r + 63) / 64 * 64) * 128u, ring = (uint32_t)a.ring, w0 = pass * (uint32_t)ntile;
   for (int t = 0; t <= ntile; ++t) {
@@ -265,88 +353,211 @@ __device__ __forceinline__ void wk_stream(const WalkArgs& a, const WalkSm& sm, c
       __syncwarp();
     }
     if (t == ntile) break;
-    const uint32_t x = w0 + (uint32_t)t, set = (uint32_t)t & 3u, nt = pass * (uint32_t)((ntile - (int)set + 3) / 4) + (uint32_t)(t >> 2), buf = set * 2u + (nt & 1u);
+    const uint32_t x = w0 + (uint32_t)t;
+    const int i = t % WK_ROUND;
+    if (i == 0 && t > 0) ++rnd;
+    if (i < 4 && !wk_drained(a, sm, i, rnd)) return;
     if (!__all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + x % ring, (x / ring) & 1, a, sm.abort))) return;
-    if (!wk_drained(a, sm, buf, nt)) return;
-    wk_mma(a, sm, ncol, x % ring, buf, tmem_base);
+    wk_mma(a, sm, ncol, x % ring, (uint32_t)i, tmem_base);
   }
 }
 
-// The scanning warps.  Per tile and eight requests a thread loads its token's target and base logit of every request (a
-// warp reads 64 contiguous bytes of each row), requested one group ahead.
+// Sums of N values over the lanes: halve the values while halving the lanes; lane (32 / N) v ends with value v.
+template <int N>
+__device__ __forceinline__ float wk_fold(float* x, const int lane) {
+#pragma unroll
+  for (int h = N / 2, o = 16; o > 0; h >>= 1, o >>= 1) {
+    if (h >= 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int k = 0; k < N / 2; ++k)
+        if (k < h) {
+          const float give = up ? x[k] : x[k + h], keep = up ? x[k + h] : x[k];
+          x[k] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+        }
+    } else x[0] += __shfl_xor_sync(0xFFFFFFFFu, x[0], o);
+  }
+  return x[0];
+}
+
+// Number of sums of a request with so many coefficients (values 0 .. WK_COLS-1: residuals, or on the grid absolute differences;
+// from WK_COLS on: proposal masses).
+__device__ __forceinline__ bool wk_has(const int nC, const int val) {
+  const int cols = nC & (WK_GRID - 1);
+  return val < WK_COLS ? val < cols : (cols > 1 && !(nC & WK_GRID) && val - WK_COLS < cols);
+}
+
+// The scanning warps.  A warp holds the accumulators of 32 tokens in each of up to three tiles and goes through the requests;
+// the two rows of a request come through a ring of 16-byte copies, two pairs ahead (AL: rows start on 16 bytes).  A request's chain
+// of waits, loads and exponentials is some 600 cycles, so two requests go through it together, and what does not depend on the request
+// is worked out before the loop.  A pass of 32 requests and one coefficient: 13.8 us; one request at a time 17, with the copies' addresses
+// and sizes worked out for every one 23; two-byte loads by every token's
+// thread, one group of eight requests ahead, took 18 us for 32 and 32 us for 64.
+template <bool AL>
 __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm, const int nreq, const int ncol, const int t0, const int tlen,
-                                            const uint32_t tmem_base, uint32_t& nt, const bool first_pass, const RedDesc* desc, float* s_part) {
+                                            const uint32_t tmem_base, uint32_t& used, uint32_t& rnd, const bool first_pass, const RedDesc* desc) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = warp & 3, set = warp >> 2;
-  const int ntile = (tlen + 127) / 128, ng = (nreq + 7) / 8;
+  const int ntile = (tlen + 127) / 128;
   const float zs = (1.f / a.T) * 1.4426950408889634f;   // exponentials as powers of two
-  float* mine = s_part + warp * WK_REQ;
-  for (int j = lane; j < WK_REQ; j += 32) mine[j] = 0.f;
-  __syncwarp();
-  unsigned short nz[8], nu[8];
-  auto load = [&](int t, int g) {
-    const int o = t * 128 + q * 32 + lane;
-    const bool in = o < tlen;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int j = g * 8 + i;
-      nz[i] = 0xFF80; nu[i] = 0;   // -inf: p = 0 and the term vanishes
-      if (in && j < nreq) {
-        const RedDesc& d = desc[j];
-        nz[i] = __ldg(reinterpret_cast<const unsigned short*>(d.z) + t0 + o);
-        if (d.C != 0.f) nu[i] = __ldg(reinterpret_cast<const unsigned short*>(d.u) + t0 + o);
-      }
-    }
-  };
+  float* mine = sm.part + (size_t)warp * WK_REQ * WK_VALS;
+  constexpr uint32_t SEG = wk_seg(AL), SLOT = wk_slot(AL);
+  const uint32_t ring = smem_u32(sm.stage) + (uint32_t)warp * (WK_SLOTS * SLOT), dbase = smem_u32(desc);
+  constexpr int CPS = AL ? 4 : 5;                       // 16-byte copies of a segment
+  const int seg = lane / CPS, ch = lane - seg * CPS;    // lane's copy of a request: 16 bytes of one segment (tile, row)
   bool alive = true;
-  const bool issues = q == 0 && !a.ring;
-  if (issues) for (int k = 0; k < 2 && alive; ++k) if (set + 4 * k < ntile) alive = wk_issue(a, sm, ncol, set + 4 * k, set, nt + (uint32_t)k, first_pass, tmem_base);
-  if (set < ntile) load(set, 0);
-  for (int t = set; t < ntile && alive; t += 4, ++nt) {
-    const uint32_t buf = (uint32_t)set * 2u + (nt & 1u);
-    if (!__all_sync(0xFFFFFFFFu, wk_wait(sm.t_full + buf, (nt >> 1) & 1u, a, sm.abort))) { alive = false; break; }
-    tc_fence_after();
-    for (int g = 0; g < ng; ++g) {
-      uint32_t acc[8];
-      __syncwarp();   // (the tensor-memory load is a warp-wide instruction)
-      asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                   : "=r"(acc[0]), "=r"(acc[1]), "=r"(acc[2]), "=r"(acc[3]), "=r"(acc[4]), "=r"(acc[5]), "=r"(acc[6]), "=r"(acc[7])
-                   : "r"(tmem_base + ((uint32_t)(q * 32) << 16) + buf * (uint32_t)WK_REQ + (uint32_t)(g * 8)) : "memory");
-      float z[8], u[8];
+  for (int r0 = 0; r0 < ntile; r0 += WK_ROUND, ++rnd) {
+    const int left = min(ntile - r0, WK_ROUND) - set, ntl = left > 0 ? (left + 3) / 4 : 0;   // the set's tiles: r0 + set + 4 i
+    const int tok = (r0 + set) * 128 + q * 32;                                              // the warp's first token in the first of them; then + 512 i
+    int nt = 0;                                                                             // its tiles with any token
 #pragma unroll
-      for (int i = 0; i < 8; ++i) { z[i] = __uint_as_float((uint32_t)nz[i] << 16); u[i] = __uint_as_float((uint32_t)nu[i] << 16); }
-      if (g + 1 < ng) load(t, g + 1); else if (t + 4 < ntile) load(t + 4, 0);
-      tmem_ld_wait();
-      float s[8];
-      const bool upper = nreq - g * 8 > 4;   // (late steps have a few requests: half a group)
+    for (int i = 0; i < WK_TR; ++i) if (i < ntl && tok + 512 * i < tlen) nt = i + 1;
+    const bool tail = nt > 0 && tok + 512 * (nt - 1) + 32 > tlen;                           // (uniform) the last of them is cut short
+    const int o = tok + 512 * (seg >> 1), nv = min(32, tlen - o);
+    const bool act = seg < 2 * nt && (!AL || 8 * ch < nv);
+    const uint64_t off = 2ull * (uint64_t)(uint32_t)(t0 + o) + (AL ? 16u * (uint32_t)ch : 0u);
+    const uint32_t from = dbase + (uint32_t)(seg & 1) * 8u, to = ring + (uint32_t)seg * SEG + (uint32_t)ch * 16u;
+    auto stage = [&](int j, uint32_t at) {   // requests j and j + 1 into the places at `at`
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        if (i >= 4 && !upper) { s[i] = 0.f; continue; }
-        const int j = min(g * 8 + i, nreq - 1);
-        const float p = ex2_approx(fmaf(z[i], zs, desc[j].zoff));
-        const float qq = ex2_approx(fmaf(__uint_as_float(acc[i]) + u[i], zs, desc[j].qoff));   // C == 0: qoff = -huge, the term vanishes
-        s[i] = fmaxf(fmaf(-desc[j].C, qq, p), 0.f);
-        if (z[i] == -INFINITY) s[i] = 0.f;   // (outside the range the accumulator may hold anything)
-      }
-      // sums over the lanes: halve the eight values three times, then two plain steps; lane 4i ends with value i
-#pragma unroll
-      for (int h = 4, off = 16; h >= 1; h >>= 1, off >>= 1) {
-        const bool up = (lane & off) != 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (i < h) {
-            const float give = up ? s[i] : s[i + h], keep = up ? s[i + h] : s[i];
-            s[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, off);
+      for (int h = 0; h < 2; ++h)
+        if (act && j + h < nreq) {
+          uint64_t row;
+          asm volatile("ld.shared.u64 %0, [%1];" : "=l"(row) : "r"(from + (uint32_t)(j + h) * (uint32_t)sizeof(RedDesc)));
+          const uint32_t dst = to + at + (uint32_t)h * SLOT;
+          if (AL) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(row + off) : "memory");
+          else {   // 32 tokens that start anywhere: up to five whole chunks, cut at the last token's end
+            const uint64_t x = row + off, src = (x & ~15ull) + 16u * (uint32_t)ch, end = x + 2u * (uint32_t)nv;
+            const int bytes = src < end ? (end - src < 16 ? (int)(end - src) : 16) : 0;
+            if (bytes) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
           }
+        }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    stage(0, 0u);
+    stage(2, 2u * SLOT);
+    if (q == 0 && !a.ring) {
+      if (alive) alive = wk_drained(a, sm, set, rnd);
+      for (int i = 0; i < ntl && alive; ++i) {
+        const int t = r0 + set + 4 * i;
+        if (first_pass && a.use_tma) alive = __all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + t, 0, a, sm.abort));
+        if (alive) wk_mma(a, sm, ncol, (uint32_t)t, (uint32_t)(set + 4 * i), tmem_base);
       }
-      float v = s[0];
-      v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
-      v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
-      if ((lane & 3) == 0) mine[g * 8 + (lane >> 2)] += v;
     }
+    for (int i = 0; i < ntl; ++i) {
+      const uint32_t slot = (uint32_t)(set + 4 * i);
+      if (alive) alive = __all_sync(0xFFFFFFFFu, wk_wait(sm.t_full + slot, (used >> slot) & 1u, a, sm.abort));
+      used ^= 1u << slot;
+    }
+    tc_fence_after();
+    const uint32_t tcol = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(set * WK_REQ);
+    uint32_t at = 0u, ahead = 4u * SLOT;   // places of this pair and of the one to be requested
+#pragma unroll 1
+    for (int j = 0; j < nreq && alive; j += 2) {
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncwarp();   // the lanes' copies of this pair are all there, and nobody reads the places the next copies go to
+      stage(j + 4, ahead);
+      uint32_t acc[2 * WK_TR];
+#pragma unroll
+      for (int i = 0; i < WK_TR; ++i)
+        if (i < nt) asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(acc[2 * i]), "=r"(acc[2 * i + 1]) : "r"(tcol + (uint32_t)(4 * i * WK_REQ + j)) : "memory");
+      float p[2 * WK_TR], qq[2 * WK_TR], c0[2]; int nC[2];
+      const int two = j + 1 < nreq ? 1 : 0;
+      const uint32_t dj = dbase + (uint32_t)j * (uint32_t)sizeof(RedDesc);
+      float zoff[2], qoff[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        int b;
+        const uint32_t dh = dj + (uint32_t)(h * two) * (uint32_t)sizeof(RedDesc);   // (a lone request stands in for its partner)
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=f"(zoff[h]), "=f"(qoff[h]), "=r"(b), "=r"(nC[h]) : "r"(dh + 16u));
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(c0[h]) : "r"(dh + 32u));
+      }
+      tmem_ld_wait();
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t zr = ring + at + (uint32_t)h * SLOT + (uint32_t)lane * 2u, ur = zr + SEG;
+        if (!AL) { zr += (uint32_t)(uintptr_t)desc[j + h * two].z & 15u; ur += (uint32_t)(uintptr_t)desc[j + h * two].u & 15u; }
+#pragma unroll
+        for (int i = 0; i < WK_TR; ++i) {
+          const int e = h * WK_TR + i;
+          p[e] = qq[e] = 0.f;
+          if (i < nt && h <= two) {
+            uint32_t z, u;
+            asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(z) : "r"(zr + 2u * (uint32_t)i * SEG));
+            asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(u) : "r"(ur + 2u * (uint32_t)i * SEG));
+            p[e] = ex2_approx(fmaf(__uint_as_float(z << 16), zs, zoff[h]));
+            qq[e] = ex2_approx(fmaf(__uint_as_float(acc[2 * i + h]) + __uint_as_float(u << 16), zs, qoff[h]));   // C == 0: qoff = -huge, the term vanishes
+          }
+        }
+      }
+      at = ahead == 4u * SLOT ? 2u * SLOT : (ahead == 0u ? 4u * SLOT : 0u);
+      ahead = ahead == 4u * SLOT ? 0u : ahead + 2u * SLOT;
+      if (tail) {
+#pragma unroll
+        for (int e = 0; e < 2 * WK_TR; ++e) if (tok + 512 * (e % WK_TR) + lane >= tlen) { p[e] = 0.f; qq[e] = 0.f; }   // (the accumulator may hold anything)
+      }
+      float* to_part = mine + j * WK_VALS;
+      if (nC[0] == 1 && nC[1] == 1) {
+        // a tile's lanes first, then the tiles in order (the bits of the bonus draw's range sums hang on it)
+        float x[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = (e & 3) < WK_TR ? fmaxf(fmaf(-c0[e >> 2], qq[(e >> 2) * WK_TR + ((e & 3) < WK_TR ? (e & 3) : 0)], p[(e >> 2) * WK_TR + ((e & 3) < WK_TR ? (e & 3) : 0)]), 0.f) : 0.f;
+        const float v0 = wk_fold<8>(x, lane), v1 = __shfl_down_sync(0xFFFFFFFFu, v0, 4), v2 = __shfl_down_sync(0xFFFFFFFFu, v0, 8);
+        if ((lane & 15) == 0 && (lane >> 4) <= two) { float* d = to_part + (lane >> 4) * WK_VALS; *d = r0 == 0 ? (v0 + v1) + v2 : ((*d + v0) + v1) + v2; }
+        continue;
+      }
+#pragma unroll 1
+      for (int h = 0; h <= two; ++h, to_part += WK_VALS) {
+        float ph[WK_TR], qh[WK_TR];
+#pragma unroll
+        for (int i = 0; i < WK_TR; ++i) { ph[i] = h ? p[WK_TR + i] : p[i]; qh[i] = h ? qq[WK_TR + i] : qq[i]; }
+        const int n = h ? nC[1] : nC[0];
+        if (n == 1) {
+          const float c = h ? c0[1] : c0[0];
+          float x[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) x[i] = i < WK_TR ? fmaxf(fmaf(-c, qh[i < WK_TR ? i : 0], ph[i < WK_TR ? i : 0]), 0.f) : 0.f;
+          const float v0 = wk_fold<4>(x, lane), v1 = __shfl_sync(0xFFFFFFFFu, v0, 8), v2 = __shfl_sync(0xFFFFFFFFu, v0, 16);
+          if (lane == 0) *to_part = r0 == 0 ? (v0 + v1) + v2 : ((*to_part + v0) + v1) + v2;
+          continue;
+        }
+        float c[WK_COLS];
+        const uint32_t dc = dj + (uint32_t)h * (uint32_t)sizeof(RedDesc) + 32u;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3]) : "r"(dc));
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(c[4]), "=f"(c[5]), "=f"(c[6]), "=f"(c[7]) : "r"(dc + 16u));
+        if (n & WK_GRID) {
+          float x[WK_COLS];
+#pragma unroll
+          for (int k = 0; k < WK_COLS; ++k) x[k] = 0.f;
+#pragma unroll
+          for (int i = 0; i < WK_TR; ++i)
+            if (i < nt) {
+              x[0] += fmaxf(fmaf(-c[0], qh[i], ph[i]), 0.f);
+#pragma unroll
+              for (int k = 1; k < WK_COLS; ++k) x[k] += fabsf(fmaf(-c[k], qh[i], ph[i]));
+            }
+          const float v = wk_fold<WK_COLS>(x, lane);
+          if ((lane & 3) == 0) { float* d = to_part + (lane >> 2); *d = r0 == 0 ? v : *d + v; }
+        } else {
+          float x[WK_VALS];
+#pragma unroll
+          for (int k = 0; k < WK_VALS; ++k) x[k] = 0.f;
+#pragma unroll
+          for (int i = 0; i < WK_TR; ++i)
+            if (i < nt) {
+#pragma unroll
+              for (int k = 0; k < WK_COLS; ++k) {
+                const float t = fmaf(-c[k], qh[i], ph[i]);
+                if (t > 0.f) { x[k] += t; x[WK_COLS + k] += qh[i]; }
+              }
+            }
+          const float v = wk_fold<WK_VALS>(x, lane);
+          if ((lane & 1) == 0) { float* d = to_part + (lane >> 1); *d = r0 == 0 ? v : *d + v; }
+        }
+      }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive(sm.t_empty + buf);
-    if (issues && t + 8 < ntile) alive = wk_issue(a, sm, ncol, t + 8, set, nt + 2u, first_pass, tmem_base);
+    if (lane == 0) mbar_arrive(sm.t_empty + set);
   }
 }
 
@@ -359,46 +570,44 @@ __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st,
   const size_t cb = (size_t)b * (a.N + 1);
   const int v = st.cur, nf = st.nf;
   const double C = st.C;
-  if (warp == 0) {
-    // the range that holds the token: cumulative range sums, corrected for the tested siblings
-    const double u = u01(stream_words(a.seed, b, a.node_hash[cb + v + 1], STREAM_BONUS, 0u).x);
-    const double target = u * st.Zj;
-    int f_tile = -1; double f_delta = 0.0;
-    if (lane < nf) { f_tile = st.fx[lane] / a.vt_TV; f_delta = fmax(st.fp[lane] - st.fC[lane] * st.fq[lane], 0.0) - fmax(st.fp[lane] - C * st.fq[lane], 0.0); }
-    double carry = 0.0, before = 0.0; int found = -1, last_pos = -1;
-    const float* part = a.part + (size_t)b * a.vt_n;
-    for (int t1 = 0; t1 < a.vt_n && found < 0; t1 += 5 * 32) {
-      float pre[5];
-#pragma unroll
-      for (int k = 0; k < 5; ++k) pre[k] = (t1 + k * 32 + lane < a.vt_n) ? __ldcg(part + t1 + k * 32 + lane) : 0.f;
-#pragma unroll 1
-      for (int k = 0; k < 5 && found < 0; ++k) {
-        const int t = t1 + k * 32 + lane;
-        double pt = (double)pre[0];
-#pragma unroll
-        for (int e = 1; e < 5; ++e) pt = k == e ? (double)pre[e] : pt;
-        for (int i = 0; i < nf; ++i) {   // tested siblings keep the residual they had when tested
-          const int ti = __shfl_sync(0xFFFFFFFFu, f_tile, i);
-          const double di = __shfl_sync(0xFFFFFFFFu, f_delta, i);
-          if (t == ti) pt += di;
-        }
-        if (pt < 0.0) pt = 0.0;
-        double inc = pt;
-        for (int off = 1; off < 32; off <<= 1) { const double o = __shfl_up_sync(0xFFFFFFFFu, inc, off); if (lane >= off) inc += o; }
-        const unsigned bal = __ballot_sync(0xFFFFFFFFu, t < a.vt_n && carry + inc > target);
-        const unsigned pos = __ballot_sync(0xFFFFFFFFu, pt > 0.0);
-        if (pos) last_pos = t1 + k * 32 + 31 - __clz(pos);
-        if (bal) { const int src = __ffs(bal) - 1; found = t1 + k * 32 + src; before = carry + __shfl_sync(0xFFFFFFFFu, inc - pt, src); }
-        carry += __shfl_sync(0xFFFFFFFFu, inc, 31);
-      }
+  const NodeDesc nd = a.node[cb + v + 1];
+  // the range that holds the token: cumulative range sums at C (to first order from the coefficient they were evaluated at),
+  // corrected for the tested siblings, which keep the residual they had when tested
+  double* s_pt = reinterpret_cast<double*>(s_dot);
+  {
+    const float col = st.col[st.pcol];
+    const double Ce = (double)col, Cf = (double)(float)C, step = st.nC > 1 && !(st.nC & WK_GRID) && fabs(Cf - Ce) <= 2.0 * WK_TOL * Cf ? Cf - Ce : 0.0;
+    const float* part = a.part + ((size_t)b * WK_VALS + st.pcol) * a.vt_n;
+    for (int t = tid; t < a.vt_n; t += WK_THREADS) {
+      double pt = (double)__ldcg(part + t);
+      if (step != 0.0) pt -= step * (double)__ldcg(part + (size_t)WK_COLS * a.vt_n + t);
+      for (int i = 0; i < nf; ++i)
+        if (st.fx[i] >= t * a.vt_TV && st.fx[i] < (t + 1) * a.vt_TV) pt += fmax(st.fp[i] - st.fC[i] * st.fq[i], 0.0) - fmax(st.fp[i] - Ce * st.fq[i], 0.0) + (st.fp[i] > Ce * st.fq[i] ? step * st.fq[i] : 0.0);
+      s_pt[t] = fmax(pt, 0.0);
     }
-    if (lane == 0) {
-      if (found < 0) { found = last_pos >= 0 ? last_pos : 0; before = -1.0; }   // rounding: take the last range with mass
+  }
+  for (int k = tid; k < a.r; k += WK_THREADS) s_a[k] = __bfloat162float(a.A[(size_t)nd.tok * a.r + k]);
+  __syncthreads();
+  if (warp == 0) {
+    const double u = u01(stream_words(a.seed, b, a.node_hash[cb + v + 1], STREAM_BONUS, 0u).x);
+    // a lane adds up neighbouring ranges, the warp scans the lanes, the lane with the crossing looks closer
+    const double target = u * st.Zj;
+    const int per = (a.vt_n + 31) / 32, r0 = min(a.vt_n, lane * per), r1 = min(a.vt_n, r0 + per);
+    double sum = 0.0; int last = -1;
+    for (int t = r0; t < r1; ++t) { const double p = s_pt[t]; sum += p; if (p > 0.0) last = t; }
+    double inc = sum;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) { const double o = __shfl_up_sync(0xFFFFFFFFu, inc, off); if (lane >= off) inc += o; }
+    last = __reduce_max_sync(0xFFFFFFFFu, last);
+    int found = -1; double before = inc - sum;
+    if (inc > target)
+      for (int t = r0; t < r1 && found < 0; ++t) { const double p = s_pt[t]; if (before + p > target) found = t; else before += p; }
+    const unsigned who = __ballot_sync(0xFFFFFFFFu, found >= 0);
+    if (lane == (who ? __ffs(who) - 1 : 0)) {
+      if (!who) { found = last >= 0 ? last : 0; before = -1.0; }   // rounding: take the last range with mass
       s_tile = found; s_target = target; s_before = before; s_found = 0x7FFFFFFF; s_last = -1;
     }
   }
-  const NodeDesc nd = a.node[cb + v + 1];
-  for (int k = tid; k < a.r; k += WK_THREADS) s_a[k] = __bfloat162float(a.A[(size_t)nd.tok * a.r + k]);
   __syncthreads();
   const int s_lo = s_tile * a.vt_TV, s_hi = min(a.V, s_lo + a.vt_TV);
   const double want = s_before >= 0.0 ? s_target - s_before : 1e300;
@@ -494,20 +703,20 @@ __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st,
   __syncthreads();
 }
 
+template <bool AL>
 __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_constant__ WalkArgs a, const __grid_constant__ CUtensorMap tmW) {
   extern __shared__ __align__(16) unsigned char raw[];
   __shared__ RedDesc s_desc[WK_REQ];
   __shared__ int s_tok[WK_REQ], s_par[256], s_cnt[WK_EPI + 1];
-  __shared__ float s_part[WK_EPI * WK_REQ];
   __shared__ float2 s_z[257];   // (maximum, log-sum-exp) of a request's rows
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = (int)blockIdx.x, ncta = (int)gridDim.x;
   const int rp = (a.r + 63) / 64 * 64, t0 = cta * a.vt_TV, tlen = min(a.vt_TV, a.V - t0), ntile = (tlen + 127) / 128;
   const uint32_t slab = (uint32_t)rp * 128u;
   unsigned char* base = raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u);
   WalkSm sm;
-  sm.Ws = base; sm.Bs = base + a.oB;
+  sm.Ws = base; sm.Bs = base + a.oB; sm.stage = base + a.oT; sm.part = reinterpret_cast<float*>(base + a.oP);
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + a.oS);
-  sm.t_full = bars; sm.t_empty = bars + WK_BUF; sm.w_full = bars + 2 * WK_BUF; sm.w_free = sm.w_full + 32;
+  sm.t_full = bars; sm.t_empty = bars + WK_ROUND; sm.w_full = bars + WK_ROUND + 4; sm.w_free = sm.w_full + 32;
   sm.tmem = reinterpret_cast<uint32_t*>(sm.w_free + 8); sm.abort = reinterpret_cast<volatile int*>(sm.tmem + 1);
   sm.st = reinterpret_cast<WalkState*>(bars + 64);
   if (warp == WK_LOAD) {
@@ -515,7 +724,8 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    for (int i = 0; i < WK_BUF; ++i) { mbar_init(sm.t_full + i, 1); mbar_init(sm.t_empty + i, 4); }
+    for (int i = 0; i < WK_ROUND; ++i) mbar_init(sm.t_full + i, 1);
+    for (int i = 0; i < 4; ++i) mbar_init(sm.t_empty + i, 4);
     for (int i = 0; i < (a.ring ? a.ring : ntile); ++i) mbar_init(sm.w_full + i, 1);
     for (int i = 0; i < a.ring; ++i) mbar_init(sm.w_free + i, 1);
     *sm.abort = 0;
@@ -543,7 +753,7 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
       *reinterpret_cast<uint4*>(sm.Ws + (size_t)sl * slab + k * 128 + ((j ^ (k & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
-  for (int i = tid; i < (int)slab / 16; i += WK_THREADS) reinterpret_cast<uint4*>(sm.Bs)[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = tid; i < rp / 64 * WK_REQ * 8; i += WK_THREADS) reinterpret_cast<uint4*>(sm.Bs)[i] = make_uint4(0u, 0u, 0u, 0u);
   fence_async_smem();
   tc_fence_before();
   __syncthreads();
@@ -557,8 +767,27 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
   unsigned gen = 0;
   const unsigned nexpect = (unsigned)ncta + (a.lost_arrival ? 1u : 0u);
   bool dead = false, finished = false;
-  uint32_t nt = 0u, wreq = 0u, pass = 0u;   // tiles of this warp's set and W blocks requested, over all passes
+  uint32_t used = 0u, rnd = 0u, wreq = 0u, pass = 0u;   // parities of the accumulator places, rounds and W blocks requested, over all passes
   for (int step = 0; !dead && step < a.max_steps; ++step) {
+    // the sums that the owners' requests asked for, a warp each: range sums in a fixed order
+    for (int x = warp; x < nown * WK_VALS; x += WK_THREADS / 32) {
+      WalkState& st = sm.st[x / WK_VALS];
+      const int val = x % WK_VALS;
+      if ((st.phase == 1 || st.phase == 2) && wk_has(st.nC, val)) {
+        const float* part = a.part + ((size_t)(cta + x / WK_VALS * ncta) * WK_VALS + val) * a.vt_n;
+        double f = 0.0;
+        for (int r0 = 0; r0 < a.vt_n; r0 += 5 * 32) {
+          float pv[5];
+#pragma unroll
+          for (int k = 0; k < 5; ++k) pv[k] = (r0 + k * 32 + lane < a.vt_n) ? __ldcg(part + r0 + k * 32 + lane) : 0.f;
+#pragma unroll
+          for (int k = 0; k < 5; ++k) f += (double)pv[k];
+        }
+        f = wk_lanes_sum(f);
+        if (lane == 0) st.S[val] = f;
+      }
+    }
+    if (nown > 0) __syncthreads();   // (uniform)
     if (warp < WK_EPI)
       for (int i = warp; i < nown; i += WK_EPI) wk_advance(a, sm.st[i], cta + i * ncta, lane, step + 1);
     if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
@@ -568,9 +797,12 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
       nwk = 0;
       for (int c0 = 0; c0 < a.B; c0 += WK_EPI * 32) {
         const int b = c0 + tid;
-        uint4 r0 = make_uint4(0u, 0u, 0u, 0u), r1 = r0, r2 = r0;
-        if (tid < WK_EPI * 32 && b < a.B) { const uint4* src = reinterpret_cast<const uint4*>(a.rec + b); r0 = __ldcg(src); r1 = __ldcg(src + 1); r2 = __ldcg(src + 2); }
-        const bool want = (int)r2.y == step + 1;
+        uint4 r0 = make_uint4(0u, 0u, 0u, 0u), r1 = r0, r2 = r0, r3 = r0, r4 = r0;
+        if (tid < WK_EPI * 32 && b < a.B) {
+          const uint4* src = reinterpret_cast<const uint4*>(a.rec + b);
+          r0 = __ldcg(src); r1 = __ldcg(src + 1); r2 = __ldcg(src + 2); r3 = __ldcg(src + 3); r4 = __ldcg(src + 4);
+        }
+        const bool want = (int)r4.y == step + 1;
         const unsigned bal = __ballot_sync(0xFFFFFFFFu, want);
         if (lane == 0) s_cnt[warp] = __popc(bal);
         __syncthreads();
@@ -580,10 +812,12 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
         if (want && at >= 0 && at < WK_REQ) {
           RedDesc d;
           const int64_t zrow = (int64_t)(((uint64_t)r0.y << 32) | r0.x);
-          d.z = a.Z + zrow * a.V; d.u = a.U + (size_t)(int)r0.z * a.V;
-          d.C = __uint_as_float(r2.x); d.zoff = __uint_as_float(r1.x); d.qoff = d.C != 0.f ? __uint_as_float(r1.y) : -1e30f;   // (lseT may be NaN where it is not needed)
-          d.b = b;
-          s_desc[at] = d; s_tok[at] = (int)r0.w;
+          d.z = a.Z + zrow * a.V; d.u = __uint_as_float(r2.x) != 0.f ? a.U + (size_t)(int)r0.z * a.V : d.z;   // (no proposal in the sum: its base row is not touched)
+          d.zoff = __uint_as_float(r1.x); d.qoff = __uint_as_float(r2.x) != 0.f ? __uint_as_float(r1.y) : -1e30f;   // (lseT may be NaN where it is not needed)
+          d.b = b; d.nC = (int)r4.x;
+          s_desc[at].z = d.z; s_desc[at].u = d.u; s_desc[at].zoff = d.zoff; s_desc[at].qoff = d.qoff; s_desc[at].b = d.b; s_desc[at].nC = d.nC;
+          reinterpret_cast<uint4*>(s_desc[at].C)[0] = r2; reinterpret_cast<uint4*>(s_desc[at].C)[1] = r3;
+          s_tok[at] = (int)r0.w;
         }
         __syncthreads();
       }
@@ -599,24 +833,29 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
       for (int x = warp; x < 2 * nreq; x += WK_THREADS / 32) {
         const RedDesc& d = s_desc[x >> 1];
         const __nv_bfloat16* src = ((x & 1) ? d.u : d.z) + t0;
-        if (!(x & 1) || d.C != 0.f)
+        if (!(x & 1) || d.u != d.z)
           for (int l = lane * 64; l < tlen; l += 32 * 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + l));
       }
       fence_async_smem();
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
-      if (warp < WK_EPI) wk_epilogue(a, sm, nreq, ncol, t0, tlen, tmem_base, nt, pass == 0u, s_desc, s_part);
-      else if (a.ring) wk_stream(a, sm, &tmW, ncol, t0, tlen, pass, wreq, tmem_base);
+      if (warp < WK_EPI) wk_epilogue<AL>(a, sm, nreq, ncol, t0, tlen, tmem_base, used, rnd, pass == 0u, s_desc);
+      else if (a.ring) wk_stream(a, sm, &tmW, ncol, t0, tlen, pass, wreq, pass * (uint32_t)((ntile + WK_ROUND - 1) / WK_ROUND), tmem_base);
       ++pass;
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
       if (*sm.abort) { dead = true; break; }
-      if (tid < nreq) {
-        float s = 0.f;
-        for (int w = 0; w < WK_EPI; ++w) s += s_part[w * WK_REQ + tid];
-        a.part[(size_t)s_desc[tid].b * a.vt_n + cta] = s;
+      for (int x = tid; x < nreq * WK_VALS; x += WK_THREADS) {
+        const RedDesc& d = s_desc[x / WK_VALS];
+        const int val = x % WK_VALS;
+        if (wk_has(d.nC, val)) {
+          float s = 0.f;
+#pragma unroll
+          for (int w = 0; w < WK_EPI; ++w) s += sm.part[w * WK_REQ * WK_VALS + x];
+          a.part[((size_t)d.b * WK_VALS + val) * a.vt_n + cta] = s;
+        }
       }
       __syncthreads();
     }
@@ -656,8 +895,9 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
 bool walk_plan(const ts_ctx* ctx, int B, bool tma, WalkPlan* out) {
   const ts_config& c = ctx->cfg;
   const size_t rp = (size_t)(c.r + 63) / 64 * 64, slab = rp * 128;
-  const size_t fixed = slab + 64 * 8 + (size_t)((B + ctx->vt_n - 1) / ctx->vt_n) * sizeof(WalkState) + 1024;
-  const size_t avail = (size_t)ctx->max_smem - 16 * 1024;   // static shared memory
+  const size_t head = rp / 64 * WK_REQ * 128, stage = (size_t)WK_EPI * WK_SLOTS * wk_slot(c.V % 8 == 0), part = (size_t)WK_EPI * WK_REQ * WK_VALS * 4;
+  const size_t fixed = head + stage + part + 64 * 8 + (size_t)((B + ctx->vt_n - 1) / ctx->vt_n) * sizeof(WalkState) + 1024;
+  const size_t avail = (size_t)ctx->max_smem - 10 * 1024;   // static shared memory
   const size_t dot = 4 * WK_CHUNK * sizeof(float);
   WalkPlan p{};
   size_t w = (size_t)(ctx->vt_TV / 64) * slab;
@@ -670,32 +910,37 @@ bool walk_plan(const ts_ctx* ctx, int B, bool tma, WalkPlan* out) {
   }
   if (w < dot) w = (dot + 1023) & ~(size_t)1023;
   if (w + fixed > avail) return false;
-  p.oB = (uint32_t)w; p.oS = (uint32_t)(w + slab); p.smem = w + fixed;
+  p.oB = (uint32_t)w; p.oT = (uint32_t)(w + head); p.oP = (uint32_t)(p.oT + stage); p.oS = (uint32_t)(p.oP + part); p.smem = w + fixed;
   *out = p;
   return true;
 }
 
 size_t walk_ws_bytes(const ts_ctx* ctx, int B) {
   const size_t b = (size_t)B, n = (size_t)ctx->cfg.Nmax;
-  return align_up(b * (n + 1) * sizeof(NodeDesc), 256) + align_up(b * (n + 1) * 8, 256) + align_up(b * n * sizeof(WalkEdge), 256) + align_up(b * sizeof(WalkRec), 256);
+  return align_up(b * (n + 1) * sizeof(NodeDesc), 256) + align_up(b * (n + 1) * 8, 256) + align_up(b * n * sizeof(WalkEdge), 256) + align_up(b * sizeof(WalkRec), 256) +
+         align_up(b * WK_VALS * (size_t)ctx->vt_n * 4, 256);
 }
 
-cudaError_t walk_setup(ts_ctx* ctx) { return allow_all_smem(walk_mma_kernel, ctx->max_smem); }
+cudaError_t walk_setup(ts_ctx* ctx) {
+  const cudaError_t e = allow_all_smem(walk_mma_kernel<true>, ctx->max_smem);
+  return e != cudaSuccess ? e : allow_all_smem(walk_mma_kernel<false>, ctx->max_smem);
+}
 
 cudaError_t launch_walk_mma(ts_ctx* ctx, WalkArgs& a, char* ws, const WalkPlan& p, cudaStream_t st) {
   const size_t b = (size_t)a.B, n = (size_t)a.N;
   a.node = (NodeDesc*)ws; ws += align_up(b * (n + 1) * sizeof(NodeDesc), 256);
   a.child = (int2*)ws; ws += align_up(b * (n + 1) * 8, 256);
   a.edge = (WalkEdge*)ws; ws += align_up(b * n * sizeof(WalkEdge), 256);
-  a.rec = (WalkRec*)ws;
-  a.ring = p.ring; a.oB = p.oB; a.oS = p.oS;
+  a.rec = (WalkRec*)ws; ws += align_up(b * sizeof(WalkRec), 256);
+  a.part = (float*)ws;
+  a.ring = p.ring; a.oB = p.oB; a.oT = p.oT; a.oP = p.oP; a.oS = p.oS;
   CUtensorMap tm;
   memset(&tm, 0, sizeof(tm));
   if (a.use_tma) memcpy(&tm, ctx->tmapW, sizeof(tm));
   ProfScope ps(ctx, K_WALK, st);
   // (chained to the row statistics: the W load and the tensor-memory allocation run beside them)
   void* kargs[] = {(void*)&a, (void*)&tm};
-  return launch_cooperative(ctx->walk_unchained, (const void*)walk_mma_kernel, dim3(a.vt_n), dim3(WK_THREADS), p.smem, st, kargs);
+  return launch_cooperative(ctx->walk_unchained, a.V % 8 == 0 ? (const void*)walk_mma_kernel<true> : (const void*)walk_mma_kernel<false>, dim3(a.vt_n), dim3(WK_THREADS), p.smem, st, kargs);
 }
 
 }  // namespace ts

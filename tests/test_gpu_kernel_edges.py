@@ -184,3 +184,49 @@ def test_candidates_that_nobody_waits_for_any_more_are_reported():
     got = to_cpu(ts.score_parents(U, A, W, zero, zero, tok, hsh, 1.0, 3))
     lost = (got["top_tok"] != want["top_tok"]).any(1) | (got["draw_tok"] != want["draw_tok"]).any(1)
     assert torch.isnan(got["lse0"][lost]).all(), f"{int(lost.sum())} lists are incomplete without a word"
+
+
+class HardRound(Round):
+    """A round whose target avoids what was drafted, so that walks reject sibling after sibling."""
+
+    def target_logits(self, tree, sigma=None):
+        Z, off = super().target_logits(tree, sigma)
+        for b in range(self.B):
+            n = int(tree["n_nodes"][b])
+            rows, cols = int(off[b]) + tree["parent"][b, :n].long() + 1, tree["tok"][b, :n].long()
+            Z[rows, cols] -= 3.0
+        return Z, off
+
+
+@pytest.mark.parametrize("over,T", [
+    (dict(V=4104, B=33, Nmax=24, K=8, D=3, r=64), 1.0),       # more requests than one pass holds, a partial second one
+    (dict(V=3001, B=3, Nmax=40, K=16, D=3, r=16), 0.7),       # sixteen rejections: more coefficients than one reduction evaluates; ragged rows
+    (dict(V=3003, B=2, Nmax=8, K=2, D=3, r=8), 1.3),          # two children
+    (dict(V=60008, B=2, Nmax=24, K=8, D=3, r=256), 1.0),      # W through the ring
+    (dict(V=240008, B=2, Nmax=12, K=8, D=2, r=8), 1.0),       # a range of more tiles than tensor memory holds at a time
+])
+def test_walks_that_reject_every_sibling(over, T):
+    """The residual masses after several rejections come from one reduction at guessed coefficients: the walk has to be the
+    oracle's, sibling by sibling, and it has to count the sums that it needed."""
+    wl = parity.small("wide", dtype="bf16", **over)
+    rnd = HardRound(wl, seed=over["V"])
+    rnd.theta.fill_(0.01)
+    ts = make_gpu(wl, rnd.table, max_batch=rnd.B)
+    st = check_round(ts, make_oracle(wl, rnd.table), rnd, T, round_seed=4)
+    assert st["walks_exempt"] <= 0.1 * st["walks"] + 1
+    tree = ts.expand_tree(rnd.U, rnd.A, rnd.W, rnd.anchor, rnd.theta, T, 4)
+    Z, off = rnd.target_logits(tree)
+    v = ts.verify_tree(rnd.U, rnd.A, rnd.W, Z, off, rnd.anchor, tree, T, 4)
+    sums = (v["flags"] >> 8).cpu()
+    for b in range(rnd.B):   # one sum a rejection, and the bonus draw's at a node without children
+        n, kids = int(tree["n_nodes"][b]), {}
+        for i in range(n):
+            kids.setdefault(int(tree["parent"][b, i]), []).append(i)
+        cur, want = -1, 0
+        for i in range(int(v["acc_len"][b])):
+            x = int(v["acc_node"][b, i])
+            want += kids[cur].index(x)
+            cur = x
+        want += max(len(kids.get(cur, [])), 1)
+        assert int(sums[b]) == want
+    assert int(sums.max()) >= wl.K   # the case was reached
