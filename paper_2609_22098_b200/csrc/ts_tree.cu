@@ -44,7 +44,7 @@ __device__ __forceinline__ void load16_bf16(const __nv_bfloat16* p, const bool w
 struct TxSm {
   unsigned char *As, *Ws, *Us;
   unsigned long long* q;       // [TX_QCAP] queued candidates (QEntry)
-  float* lists;                // [128][5K]: topv, topi, keyv, keyi, keyl of every row, sorted (value desc, token asc)
+  float* lists;                // [128][list_stride(K)]: topv, topi, keyv, keyi, keyl of every row, sorted (value desc, token asc)
   int* ln;                     // [2][128] entries in use
   volatile float* lthr;        // [2][128] K-th best of the row's own list (-inf until it is full)
   volatile float* best;        // [2][TX_SPLIT][128] best value published by the piece (row, split)
@@ -58,8 +58,10 @@ struct TxSm {
   volatile unsigned* q_head; unsigned* q_tail;
 };
 
+// words between two rows' lists: odd, so that the threads of neighbouring rows read different banks
+__host__ __device__ constexpr int list_stride(int K) { return (5 * K) | 1; }
 constexpr size_t tx_select_bytes(int K) {
-  return (size_t)TX_QCAP * 8 + (size_t)TX_ROWS * 5 * K * 4 + 2 * TX_ROWS * 4 + 2 * TX_ROWS * 4 + 2 * TX_SPLIT * TX_ROWS * 4 + 3 * TX_SPLIT * TX_ROWS * 4;
+  return (size_t)TX_QCAP * 8 + (size_t)TX_ROWS * list_stride(K) * 4 + 2 * TX_ROWS * 4 + 2 * TX_ROWS * 4 + 2 * TX_SPLIT * TX_ROWS * 4 + 3 * TX_SPLIT * TX_ROWS * 4;
 }
 constexpr size_t TX_FIXED_BYTES = 512 * 4 + 2 * TX_ROWS * 4 + TX_ROWS * sizeof(ParentEntry) + (1 + 4 * TX_STAGE_MAX + 2 * TX_USTAGES) * 8 + 64;
 
@@ -68,7 +70,7 @@ __device__ __forceinline__ TxSm tx_carve(unsigned char* sm, const TreeArgs& a) {
   s.As = sm; s.Ws = sm + a.oW; s.Us = sm + a.oU;
   s.q = reinterpret_cast<unsigned long long*>(sm + a.oL);
   s.lists = reinterpret_cast<float*>(s.q + TX_QCAP);
-  s.ln = reinterpret_cast<int*>(s.lists + (size_t)TX_ROWS * 5 * a.K);
+  s.ln = reinterpret_cast<int*>(s.lists + (size_t)TX_ROWS * list_stride(a.K));
   s.lthr = reinterpret_cast<float*>(s.ln + 2 * TX_ROWS);
   s.best = s.lthr + 2 * TX_ROWS;
   s.part = const_cast<float*>(s.best) + 2 * TX_SPLIT * TX_ROWS;
@@ -155,9 +157,9 @@ __device__ __forceinline__ void tx_select(const TreeArgs& a, const TxSm& sm, con
   const uint32_t kind = ((uint32_t)e >> 26) & 3u;
   const int per = TX_ROWS / R;
   const int prow = R > 1 ? row % per : row, rho = R > 1 ? row / per : 0;
-  const int p = R > 1 ? prow : g * TX_ROWS + row;
+  const int p = g * TX_ROWS + prow;
   const int pid = ((tile * TX_SPLIT + s) * R + rho) % K;
-  float* L = sm.lists + (size_t)row * 5 * K;
+  float* L = sm.lists + (size_t)row * list_stride(K);
   if (kind & 1u) {
     if (lg >= sm.thr[prow] && lg >= sm.lthr[row]) {
       sm.lthr[row] = tx_insert(L, reinterpret_cast<int*>(L) + K, nullptr, sm.ln[row], K, lg, tok, 0.f);
@@ -212,7 +214,7 @@ template <bool RING>
 __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int t0, const int tlen,
                                         const uint32_t tmem_base, BlockPos& pos, const int nst, const uint32_t ub0) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int q = warp & 3, s = warp >> 2, row = q * 32 + lane;
+  const int q = warp & 3, s = warp >> 2;
   const int per = TX_ROWS / R, K = a.K;
   (void)K;
   {
@@ -228,6 +230,7 @@ __device__ __forceinline__ void tx_scan(const TreeArgs& a, const TxSm& sm, const
     fence_async_smem();
     mbar_arrive(sm.a_full);
   }
+  const int row = q * 32 + lane;
   const ParentEntry& me = sm.ent[row];
   const bool active = me.row >= 0;
   const int prow = R > 1 ? row % per : row, rho = R > 1 ? row / per : 0;   // rho is uniform within a warp
@@ -456,7 +459,7 @@ __device__ __forceinline__ void tx_refresh(const TreeArgs& a, const TxSm& sm, co
                                            const CUtensorMap* tm, const int t0, const int tlen, WLoad& w, const uint32_t upto,
                                            const CUtensorMap* tmU, const int depth, ULoad& u, const uint32_t uend) {
   const int lane = threadIdx.x & 31, per = TX_ROWS / R, K = a.K;
-  const int p_lo = R > 1 ? 0 : g * TX_ROWS, p_hi = min(P, p_lo + per), nt = a.ntiles;
+  const int p_lo = g * TX_ROWS, p_hi = min(P, p_lo + per), nt = a.ntiles;
   const int p_own = p_lo + ((tile - p_lo % nt + nt) % nt);
   const int which = lane >> 4, j = lane & 15;
   for (uint32_t spin = 0; spin < a.wait_limit; ++spin) {
@@ -545,16 +548,27 @@ __device__ __forceinline__ void tx_drain(const TreeArgs& a, const TxSm& sm, cons
   }
 }
 
+// where the candidates of parent p start
+__device__ __forceinline__ size_t cand_base(const TreeArgs& a, const int P, const int p) { return (size_t)p * a.ntiles * (mma_replicas(P) * a.K); }
+
 // ---- end of a group: the range's sums and surviving candidates of every parent -------------------------------------
+// A row's sums, best logits and best keys by three threads side by side (one after the other, with the lists' atomics behind
+// the sums, it took 2 us a group).
 __device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, const int R, const int P, const int g, const int tile, int* cnt) {
-  const int tid = threadIdx.x, per = TX_ROWS / R, K = a.K;
-  if (tid >= TX_ROWS) return;
-  const int row = tid, prow = R > 1 ? row % per : row, p = R > 1 ? prow : g * TX_ROWS + row;
+  const int role = (int)threadIdx.x / TX_ROWS, row = (int)threadIdx.x % TX_ROWS, per = TX_ROWS / R, K = a.K;
+  if (role > 2) return;
+  const int prow = R > 1 ? row % per : row, p = g * TX_ROWS + prow;
   if (p >= P) return;
-  const float T = a.T, invT = T > 0.f ? 1.f / T : 1.f;
-  if (row < per) {
-    // the pieces' sums in a fixed order: the same bits on every run
+  if (role == 0) {
+    if (row >= per) return;
+    const float T = a.T, invT = T > 0.f ? 1.f / T : 1.f;
+    // the pieces' sums in a fixed order: the same bits on every run (the largest reference first: the exponentials do not wait
+    // for one another; with a running reference four copies of a row took 1.1 us longer)
     float m = -INFINITY, s0 = 0.f, sT = 0.f;
+#pragma unroll 1
+    for (int rho = 0; rho < R; ++rho)
+#pragma unroll
+      for (int s = 0; s < TX_SPLIT; ++s) m = fmaxf(m, sm.part[(0 * TX_SPLIT + s) * TX_ROWS + rho * per + row]);
 #pragma unroll 1
     for (int rho = 0; rho < R; ++rho)
 #pragma unroll
@@ -562,37 +576,35 @@ __device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, co
         const int rr = rho * per + row;
         const float hm = sm.part[(0 * TX_SPLIT + s) * TX_ROWS + rr], h0 = sm.part[(1 * TX_SPLIT + s) * TX_ROWS + rr], hT = sm.part[(2 * TX_SPLIT + s) * TX_ROWS + rr];
         if (hm == -INFINITY) { s0 += h0; continue; }   // (nothing finite: h0 is 0, or NaN if the piece met one)
-        if (hm > m) { const float d = m == -INFINITY ? 0.f : m - hm; s0 *= __expf(d); sT *= __expf(d * invT); m = hm; }
         const float d = hm - m;
         s0 += h0 * __expf(d); sT += hT * __expf(d * invT);
       }
     a.sums[(size_t)p * a.ntiles + tile] = make_float4(m, s0, sT, 0.f);
+    return;
   }
-  const size_t base = (size_t)p * a.ntiles * (R * K);
-  const float gL = sm.thr[prow], gK = sm.thr[TX_ROWS + prow];
-  const float* L = sm.lists + (size_t)row * 5 * K;
-  const int* Li = reinterpret_cast<const int*>(L);
-  int kt = 0, kk = 0;
-#pragma unroll 1
-  for (int n = sm.ln[row]; kt < n && L[kt] >= gL;) ++kt;
-#pragma unroll 1
-  for (int n = sm.ln[TX_ROWS + row]; kk < n && L[2 * K + kk] >= gK;) ++kk;
-  int at = 0, ak = 0;
-  if (kt) at = atomicAdd(cnt + p, kt);
-  if (kk) ak = atomicAdd(cnt + a.cap + p, kk);
-#pragma unroll 1
-  for (int j = 0; j < kk; ++j) {
-    a.cand_key[base + ak + j] = make_uint2(__float_as_uint(L[2 * K + j]), (unsigned)Li[3 * K + j]);
-    a.cand_lg[base + ak + j] = L[4 * K + j];
+  const size_t base = cand_base(a, P, p);
+  const float* L = sm.lists + (size_t)row * list_stride(K) + (role == 2 ? 2 * K : 0);
+  const float bound = sm.thr[(role == 2 ? TX_ROWS : 0) + prow];
+  const int n = sm.ln[(role == 2 ? TX_ROWS : 0) + row];
+  int k = 0;
+#pragma unroll 4
+  for (int j = 0; j < K; ++j) k += (j < n && L[j] >= bound) ? 1 : 0;   // (sorted: the first k)
+  if (k == 0) return;
+  const int at = atomicAdd(cnt + (role == 2 ? a.cap : 0) + p, k);
+  const int* Li = reinterpret_cast<const int*>(L) + K;
+  uint2* out = (role == 2 ? a.cand_key : a.cand_top) + base + at;
+#pragma unroll 2
+  for (int j = 0; j < k; ++j) {
+    out[j] = make_uint2(__float_as_uint(L[j]), (unsigned)Li[j]);
+    if (role == 2) a.cand_lg[base + at + j] = L[2 * K + j];
   }
-#pragma unroll 1
-  for (int j = 0; j < kt; ++j) a.cand_top[base + at + j] = make_uint2(__float_as_uint(L[j]), (unsigned)Li[K + j]);
 }
 
 // ---- merge of one parent, by one warp --------------------------------------------------------------------------------
-// The K best of n (value, token) pairs (value desc, token asc): lane j < K gets the j-th in (tok, val, lg).  Batches of
-// up to 96 entries in registers beside the winners so far; a round is two warp-wide maxima (the value's order-
-// preserving image, then the inverted token among its ties) and one removal.
+// The K best of n (value, token) pairs (value desc, token asc): lane j < K gets the j-th in (tok, val, lg).  The first 96
+// entries are picked by rounds of two warp-wide maxima (the value's order-preserving image, then the inverted token among its
+// ties) and one removal; of what follows only the few that beat the K-th so far are inserted, one by one.  (Rounds for every
+// 96 entries: crowded levels hold several hundred per parent, 24 to 28 us for a parent's three merges at K = 16.)
 __device__ __noinline__ float3 warp_topk(const uint2* cand, const float* lgs, const int* count, int K, int lane) {
   uint32_t wv = 0u, wt = 0u; float wl = 0.f;   // winner `lane` so far: 0 = none
   // the first 64 entries are requested together with the count (past a short segment they are a neighbour's, and past the
@@ -602,37 +614,55 @@ __device__ __noinline__ float3 warp_topk(const uint2* cand, const float* lgs, co
   const float pl0 = lgs ? __ldcg(lgs + lane) : 0.f, pl1 = lgs ? __ldcg(lgs + 32 + lane) : 0.f;
 #pragma unroll 1
   for (int base = 0; base < n; base += 3 * 32) {
-    uint32_t ev[4], et[4]; float el[4];
-    ev[0] = wv; et[0] = wt; el[0] = wl;
+    uint32_t ev[3], et[3]; float el[3];
     const int used = min(3, (n - base + 31) / 32);   // (warp-uniform) slots of 32 entries in this batch
 #pragma unroll
-    for (int u = 1; u < 4; ++u) {
-      const int i = base + (u - 1) * 32 + lane;
+    for (int u = 0; u < 3; ++u) {
+      const int i = base + u * 32 + lane;
       ev[u] = 0u; et[u] = 0u; el[u] = 0.f;
-      if (u <= used && i < n) {
-        const uint2 c = (u == 1 && base == 0) ? pre0 : ((u == 2 && base == 0) ? pre1 : __ldcg(cand + i));
+      if (u < used && i < n) {
+        const uint2 c = (u == 0 && base == 0) ? pre0 : ((u == 1 && base == 0) ? pre1 : __ldcg(cand + i));
         ev[u] = enc_f(__uint_as_float(c.x)); et[u] = ~c.y;
-        el[u] = !lgs ? __uint_as_float(c.x) : ((u == 1 && base == 0) ? pl0 : ((u == 2 && base == 0) ? pl1 : __ldcg(lgs + i)));
+        el[u] = !lgs ? __uint_as_float(c.x) : ((u == 0 && base == 0) ? pl0 : ((u == 1 && base == 0) ? pl1 : __ldcg(lgs + i)));
       }
     }
-    wv = 0u; wt = 0u; wl = 0.f;
+    if (base == 0) {
 #pragma unroll 1
-    for (int j = 0; j < K; ++j) {
-      uint32_t bv = ev[0], bt = et[0]; float bl = el[0];
+      for (int j = 0; j < K; ++j) {
+        uint32_t bv = ev[0], bt = et[0]; float bl = el[0];
 #pragma unroll
-      for (int u = 1; u < 4; ++u)
-        if (u <= used && (ev[u] > bv || (ev[u] == bv && et[u] > bt))) { bv = ev[u]; bt = et[u]; bl = el[u]; }
-      const uint32_t mv = __reduce_max_sync(0xFFFFFFFFu, bv);
-      if (mv == 0u) break;   // warp-uniform
-      const uint32_t mt = __reduce_max_sync(0xFFFFFFFFu, bv == mv ? bt : 0u);
-      const bool mine = bv == mv && bt == mt;
-      const unsigned who = __ballot_sync(0xFFFFFFFFu, mine);
-      const float l = __shfl_sync(0xFFFFFFFFu, bl, __ffs(who) - 1);
-      if (mine) {
+        for (int u = 1; u < 3; ++u)
+          if (u < used && (ev[u] > bv || (ev[u] == bv && et[u] > bt))) { bv = ev[u]; bt = et[u]; bl = el[u]; }
+        const uint32_t mv = __reduce_max_sync(0xFFFFFFFFu, bv);
+        if (mv == 0u) break;   // warp-uniform
+        const uint32_t mt = __reduce_max_sync(0xFFFFFFFFu, bv == mv ? bt : 0u);
+        const bool mine = bv == mv && bt == mt;
+        const unsigned who = __ballot_sync(0xFFFFFFFFu, mine);
+        const float l = __shfl_sync(0xFFFFFFFFu, bl, __ffs(who) - 1);
+        if (mine) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) if (ev[u] == mv && et[u] == mt) { ev[u] = 0u; et[u] = 0u; }
+          for (int u = 0; u < 3; ++u) if (ev[u] == mv && et[u] == mt) { ev[u] = 0u; et[u] = 0u; }
+        }
+        if (lane == j) { wv = mv; wt = mt; wl = l; }
       }
-      if (lane == j) { wv = mv; wt = mt; wl = l; }
+      continue;
+    }
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      uint32_t tv = __shfl_sync(0xFFFFFFFFu, wv, K - 1), tt = __shfl_sync(0xFFFFFFFFu, wt, K - 1);
+      unsigned todo = __ballot_sync(0xFFFFFFFFu, ev[u] > tv || (ev[u] == tv && et[u] > tt));
+#pragma unroll 1
+      while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const uint32_t v = __shfl_sync(0xFFFFFFFFu, ev[u], src), t = __shfl_sync(0xFFFFFFFFu, et[u], src);
+        const float l = __shfl_sync(0xFFFFFFFFu, el[u], src);
+        const int pos = __popc(__ballot_sync(0xFFFFFFFFu, lane < K && (wv > v || (wv == v && wt > t))));   // (K: beaten by now)
+        const uint32_t pv = __shfl_up_sync(0xFFFFFFFFu, wv, 1), pt = __shfl_up_sync(0xFFFFFFFFu, wt, 1);
+        const float pl = __shfl_up_sync(0xFFFFFFFFu, wl, 1);
+        if (lane < K && lane > pos) { wv = pv; wt = pt; wl = pl; }
+        if (lane < K && lane == pos) { wv = v; wt = t; wl = l; }
+      }
     }
   }
   return make_float3(__int_as_float(wv ? (int)~wt : -1), wv ? dec_f(wv) : 0.f, wv ? wl : 0.f);   // token (as bits), value, logit
@@ -705,39 +735,23 @@ __device__ __forceinline__ void scout_piece(const TreeArgs& a, int row, int piec
   if (lane == 0) *out = make_uint2(mv, mt);   // (0: nothing above -inf in the piece)
 }
 
-// The seed tokens of one row: the best of its pieces, picked by one warp (lane j: the j-th).
+// The seed tokens of one row, by one warp: a lane's best of the pieces it reads, ranked among the lanes' by counting (any
+// tokens give valid bounds, so the second best of a lane is not missed; picking the best 16 of all pieces one after the
+// other took 3.5 us and was what the owner's other warps waited for).
 __device__ __forceinline__ void pick_seeds(const int npiece, const uint2* ut, int NS, int* stok, float* sval, int lane) {
-  uint32_t ev[8], et[8];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) { ev[u] = 0u; et[u] = 0u; }
+  uint32_t bv = 0u, bt = 0u;
 #pragma unroll 1
-  for (int i0 = 0; i0 < npiece; i0 += 256) {
+  for (int i0 = 0; i0 < npiece; i0 += 160) {
+    uint2 e[5];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u * 32 + lane;
-      if (i < npiece) {
-        const uint2 e = __ldcg(ut + i);
-        if (e.x > ev[u]) { ev[u] = e.x; et[u] = e.y; }   // (beyond 256 pieces the best of every 256th: any tokens give valid bounds)
-      }
-    }
+    for (int u = 0; u < 5; ++u) { const int i = i0 + u * 32 + lane; e[u] = i < npiece ? __ldcg(ut + i) : make_uint2(0u, 0u); }
+#pragma unroll
+    for (int u = 0; u < 5; ++u) if (e[u].x > bv) { bv = e[u].x; bt = e[u].y; }
   }
-  int tok = -1; float val = -INFINITY;
-#pragma unroll 1
-  for (int j = 0; j < NS; ++j) {
-    uint32_t bv = ev[0], bt = et[0];
+  int rank = 0;
 #pragma unroll
-    for (int u = 1; u < 8; ++u) if (ev[u] > bv) { bv = ev[u]; bt = et[u]; }
-    const uint32_t mv = __reduce_max_sync(0xFFFFFFFFu, bv);
-    if (mv == 0u) break;
-    const int src = __ffs(__ballot_sync(0xFFFFFFFFu, bv == mv)) - 1;
-    const uint32_t t = __shfl_sync(0xFFFFFFFFu, bt, src);
-    if (lane == src) {
-#pragma unroll
-      for (int u = 0; u < 8; ++u) if (ev[u] == mv && et[u] == t) ev[u] = 0u;
-    }
-    if (lane == j) { tok = (int)t; val = dec_f(mv); }
-  }
-  if (lane < NS) { stok[lane] = tok; sval[lane] = val; }
+  for (int l = 0; l < 32; ++l) { const uint32_t o = __shfl_sync(0xFFFFFFFFu, bv, l); rank += (o > bv || (o == bv && l < lane)) ? 1 : 0; }
+  if (rank < NS) { stok[rank] = bv ? (int)bt : -1; sval[rank] = bv ? dec_f(bv) : -INFINITY; }
 }
 
 // Shared-memory pieces of an owner (offsets of OwnerLayout).
@@ -784,23 +798,12 @@ __device__ __forceinline__ void store_seed_columns(const TreeArgs& a, const Owne
 }
 
 // Seed bounds and list entries of `cnt` parents of one row (all threads; the columns have landed).  Parent i: token
-// s.ttok[i], hash hs[i], pool slot s.npl[i]; its place in the level's list is li0 + i * step.
-__device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s, const int cnt, const int li0, const int step, const int req, const int row, const int NS,
+// ptok[i], hash phash[i], pool slot s.npl[i]; its place in the level's list is li0 + i * step (place != null: *place, known after the first barrier).
+__device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s, const int cnt, int li0, const int* place, const int step, const int req, const int row, const int NS,
                                              const int* ptok, const uint64_t* phash, ParentEntry* ent, int* ent_slot, int* cnt_next) {
   const int tid = threadIdx.x, r = a.r, K = a.K, lg = seed_log2(K);
   const float invT = a.T > 0.f ? 1.f / a.T : 1.f;
   const __nv_bfloat16* Ag = reinterpret_cast<const __nv_bfloat16*>(a.A);
-  // the parents' pruning state and candidate counts start clean
-#pragma unroll 1
-  for (int e = tid; e < cnt * 2 * K; e += TX_THREADS) {
-    const int i = e / (2 * K), w = (e / K) & 1, j = e % K;
-    a.slots[(((size_t)w * a.cap + li0 + i * step) * K + j) * SLOT_STRIDE] = 0u;
-  }
-#pragma unroll 1
-  for (int e = tid; e < cnt * 2; e += TX_THREADS) {
-    a.thr[(size_t)(e & 1) * a.cap + li0 + (e >> 1) * step] = 0u;
-    cnt_next[(size_t)(e & 1) * a.cap + li0 + (e >> 1) * step] = 0;
-  }
   // every (parent, seed token) pair exactly: eight lanes a pair, 16 bytes of the head row a lane and step
   const int sub = tid & 7;
 #pragma unroll 1
@@ -834,6 +837,18 @@ __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s
 #pragma unroll 1
   for (int i = tid; i < cnt; i += TX_THREADS) { bL[i] = -INFINITY; bK[i] = -INFINITY; bM[i] = -INFINITY; }
   __syncthreads();
+  if (place) li0 = *place;
+  // the parents' pruning state and candidate counts start clean
+#pragma unroll 1
+  for (int e = tid; e < cnt * 2 * K; e += TX_THREADS) {
+    const int i = e / (2 * K), w = (e / K) & 1, j = e % K;
+    a.slots[(((size_t)w * a.cap + li0 + i * step) * K + j) * SLOT_STRIDE] = 0u;
+  }
+#pragma unroll 1
+  for (int e = tid; e < cnt * 2; e += TX_THREADS) {
+    a.thr[(size_t)(e & 1) * a.cap + li0 + (e >> 1) * step] = 0u;
+    cnt_next[(size_t)(e & 1) * a.cap + li0 + (e >> 1) * step] = 0;
+  }
 #pragma unroll 1
   for (int e = tid; e < 2 * cnt * NS; e += TX_THREADS) {
     // one thread per value: the one with exactly K - 1 values before it (ties broken by place) is the K-th best
@@ -881,8 +896,9 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
   int* ptok = s.ttok; uint64_t* phash = reinterpret_cast<uint64_t*>(s.tlog);   // the new parents (merged results are done with by then)
   int cnt = 1, li0 = b, req = b, row = b * a.D + d + 1;
   bool more = true;
-  int npar = 0, base = 0, K_eff = 0, N_eff = 0;
-  double log_theta = 0.0;
+  int npar = 0, base = 0, K_eff = 0, N_eff = 0, pslot = -1;
+  double2 caps = make_double2(0.0, 0.0);
+  int place = 0;
   unsigned char* gpool = a.pool + (size_t)b * a.pool_stride;
   if (share >= 0) {
     const int np = __ldcg(a.req_npar + nxt * a.B + b);
@@ -925,14 +941,12 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       if (tid == 0) a.req_npar[nxt * a.B + b] = 0;
       return;   // (own[] stays: no parents, or not fine)
     }
-    const double2 caps = __ldcg(a.req_caps + b);   // log theta (-inf on the chain member), 1 on the chain member
-    log_theta = caps.x; K_eff = caps.y != 0.0 ? 1 : min(K, a.V); N_eff = caps.y != 0.0 ? min(a.D, N) : N;
+    caps = __ldcg(a.req_caps + b);   // log theta (-inf on the chain member), 1 on the chain member (not looked at before the merge)
     more = d + 1 < a.D;
     uint4* dst = reinterpret_cast<uint4*>(s.pv.key); const uint4* src = reinterpret_cast<const uint4*>(gpool);
 #pragma unroll 1
-    for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) dst[i] = __ldcg(src + i);
-#pragma unroll 1
-    for (int i = tid; i < npar; i += TX_THREADS) s.pslot[i] = __ldcg(a.ent_slot[cur] + base + i);
+    for (int i = tid; i < (int)(pool_bytes(N) / 16); i += TX_THREADS) cp_async16(dst + i, src + i, true);   // (lands while the merge runs)
+    if (tid < npar) pslot = __ldcg(a.ent_slot[cur] + base + tid);   // (at most 256 parents)
     if (tid < 8) sh[tid] = 0;
   }
   // ---- merge: a warp each for a parent's log-normalisers, its best logits and its best keys: each is one or two memory
@@ -951,7 +965,6 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       if (j == 0) { const float2 l = __ldcg(a.res_lse + base + i); s.lse0[i] = l.x; s.lseT[i] = l.y; }
     }
   } else if (d >= 0 && share < 0) {
-    const int R = mma_replicas(P);
 #pragma unroll 1
     for (int task = warp; task < npar * 3; task += TX_WARPS - 1) {
       const int i = task / 3, kind = task - 3 * i, p = base + i;
@@ -960,7 +973,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
         const float2 l = warp_lse(a.sums + (size_t)p * a.ntiles, a.ntiles, a.T, lane);
         if (lane == 0) { s.lse0[i] = l.x; s.lseT[i] = l.y; }
       } else {
-        const size_t cb = (size_t)p * a.ntiles * (R * K);
+        const size_t cb = cand_base(a, P, p);
         const float3 w = warp_topk(kind == 1 ? a.cand_top + cb : a.cand_key + cb, kind == 1 ? nullptr : a.cand_lg + cb, a.cand_cnt[cur] + (kind == 1 ? 0 : a.cap) + p, K, lane);
         if (lane < K) {
           if (kind == 1) { s.ttok[(i << lk) + lane] = __float_as_int(w.x); s.tlog[(i << lk) + lane] = w.y; }
@@ -969,7 +982,11 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       }
     }
   }
+  if (tid < npar) s.pslot[tid] = pslot;
+  cp_async_wait_all();
   __syncthreads();
+  const double log_theta = caps.x;
+  K_eff = caps.y != 0.0 ? 1 : min(K, a.V); N_eff = caps.y != 0.0 ? min(a.D, N) : N;
   uint32_t wcol[SEED_REGS];
   if (more) load_seed_columns(a, s, NS, 0, wcol);   // on their way while the draws are ranked
   if (d >= 0 && share < 0) {
@@ -1170,6 +1187,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       const int c = it * TX_THREADS + tid, t = s.toff[it * TX_WARPS + warp] + __popc(vb & ((1u << lane) - 1u));
       if (t >= nfree) continue;
       const int sl = s.hist[t], i = c >> lk, j = c & ((1 << lk) - 1), slot = s.pslot[i], x = s.dtok[c];
+      if (more) asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const __nv_bfloat16*>(a.A) + (size_t)x * a.r));   // (its head row is needed soon)
       const double lx = s.dlog[c], lse0 = s.lse0[i], lseT = s.lseT[i];
       s.pv.meta[sl] = (1 << 16) | ((d + 1) << 8) | j; s.pv.parent[sl] = slot; s.pv.tok[sl] = x;
       s.pv.key[sl] = s.ckey[c]; s.pv.logS[sl] = s.clogS[c];
@@ -1196,9 +1214,8 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
 #pragma unroll 1
     for (int w = 0; w < 8; ++w) { if (w < warp) off += s.tcnt[w]; cnt += s.tcnt[w]; }
     if (tid == 0) {
-      const int nb = cnt > 0 ? atomicAdd(a.lvl_count + d + 1, cnt) : 0;
-      sh[6] = nb; a.req_base[b] = nb;
-      if (b == (int)blockIdx.x) { own[0] = cnt; own[1] = nb; }
+      if (cnt > 0) place = atomicAdd(a.lvl_count + d + 1, cnt);   // (asked for here, waited for after the seed products)
+      if (b == (int)blockIdx.x) own[0] = cnt;
       a.req_npar[nxt * a.B + b] = cnt; a.req_nscored[b] += npar;
     }
     if (par) { const int i = off + __popc(bal & ((1u << lane) - 1u)); s.npl[i] = sl; ptok[i] = pt; phash[i] = ph; }
@@ -1213,8 +1230,11 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
 #pragma unroll 1
     for (int e0 = SEED_REGS * TX_THREADS; e0 < NS * a.r; e0 += SEED_REGS * TX_THREADS) { load_seed_columns(a, s, NS, e0, wcol); store_seed_columns(a, s, NS, e0, wcol); }
   __syncthreads();
-  if (d >= 0 && share < 0) li0 = sh[6];
+  const bool placed = d >= 0 && share < 0;
+  if (placed && tid == 0) { sh[6] = place; a.req_base[b] = place; if (b == (int)blockIdx.x) own[1] = place; }   // (visible after the barrier in make_parents, or the one here)
   if (MANY && more && share < 0 && cnt > TX_SOLO) {   // many parents: entries without bounds; all CTAs make those after the next barrier
+    __syncthreads();
+    if (placed) li0 = sh[6];
 #pragma unroll 1
     for (int i = tid; i < cnt; i += TX_THREADS) {
       uint4* dst = reinterpret_cast<uint4*>(a.ent[nxt] + li0 + i);
@@ -1223,7 +1243,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       a.ent_slot[nxt][li0 + i] = s.npl[i];
     }
     if (tid == 0) a.seed_need[d + 1] = 1;
-  } else if (more && cnt > 0) make_parents(a, s, cnt, li0, share >= 0 ? step : 1, req, row, NS, ptok, phash, a.ent[nxt], share >= 0 ? nullptr : a.ent_slot[nxt], a.cand_cnt[nxt]);
+  } else if (more && cnt > 0) make_parents(a, s, cnt, li0, placed ? sh + 6 : nullptr, share >= 0 ? step : 1, req, row, NS, ptok, phash, a.ent[nxt], share >= 0 ? nullptr : a.ent_slot[nxt], a.cand_cnt[nxt]);
   __syncthreads();
 }
 
@@ -1372,7 +1392,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
       const int R = mma_replicas(P), per = TX_ROWS / R, ngroups = R > 1 ? 1 : (P + TX_ROWS - 1) / TX_ROWS;
       for (int g = 0; g < ngroups; ++g, ++groups) {
         if (tid < TX_ROWS) {
-          const int p = R > 1 ? tid % per : g * TX_ROWS + tid;
+          const int p = g * TX_ROWS + (R > 1 ? tid % per : tid);
           uint4 e0 = make_uint4(0xFFFFFFFFu, 0u, 0u, 0u), e1 = make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0u);   // row -1: unused
           if (p < P) { const uint4* src = reinterpret_cast<const uint4*>(a.ent[d & 1] + p); e0 = __ldcg(src); e1 = __ldcg(src + 1); }
           uint4* dst = reinterpret_cast<uint4*>(sm.ent + tid);
@@ -1386,7 +1406,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
         // ask L2 for this range of every base-logit row the group reads (neighbours of the list often share theirs): the scan
         // itself asks for 32 bytes a lane one chunk ahead, which leaves DRAM waiting when the rows are many
         if (!RING) {
-          const int nrow = R > 1 ? P : min(TX_ROWS, P - g * TX_ROWS), lines = (tlen * 2 + 127) / 128;
+          const int nrow = min(TX_ROWS, P - g * TX_ROWS), lines = (tlen * 2 + 127) / 128;
 #pragma unroll 1
           for (int x = warp; x < nrow; x += TX_WARPS) {
             const int rw = sm.ent[x].row;
@@ -1399,7 +1419,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
         const int done_target = (groups + 1) * TX_SCAN_WARPS;
         const int nst = min(512 / a.BN, TX_STAGE_MAX);   // accumulator stages
         const uint32_t ublocks = RING ? (uint32_t)((tlen + a.BN - 1) / a.BN) : 0u;
-        if (warp < TX_SCAN_WARPS) tx_scan<RING>(a, sm, R, P, g, t0, tlen, tmem_base, pos, nst, ub0);
+        if (warp < TX_SCAN_WARPS) tx_scan<RING>(a, sm, R, min(TX_ROWS, P - g * TX_ROWS), g, t0, tlen, tmem_base, pos, nst, ub0);
         else if (warp == TX_MMA) tx_issue(a, sm, tlen, tmem_base, pos, wpos, groups, nst);
         else if (warp == TX_REFRESH) {
           const uint32_t nblk = (uint32_t)((tlen + a.BN - 1) / a.BN);
@@ -1419,15 +1439,22 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
     if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
     if (a.score_P > 0) {
       // given parents: merged by all CTAs, results to the caller
-      const int R = mma_replicas(P), K = a.K;
-      for (int p = cta + ncta * warp; p < P; p += ncta * TX_WARPS) {
-        const size_t cb = (size_t)p * a.ntiles * (R * K);
-        const float2 l = warp_lse(a.sums + (size_t)p * a.ntiles, a.ntiles, a.T, lane);
-        if (lane == 0) { a.o_lse0[p] = l.x; a.o_lseT[p] = l.y; }
-        float3 w = warp_topk(a.cand_top + cb, nullptr, a.cand_cnt[0] + p, K, lane);
-        if (lane < K) { a.o_top_tok[(size_t)p * K + lane] = __float_as_int(w.x); a.o_top_logit[(size_t)p * K + lane] = w.y; }
-        if (a.T > 0.f) w = warp_topk(a.cand_key + cb, a.cand_lg + cb, a.cand_cnt[0] + a.cap + p, K, lane);
-        if (lane < K) { a.o_draw_tok[(size_t)p * K + lane] = __float_as_int(w.x); a.o_draw_logit[(size_t)p * K + lane] = w.z; }
+      const int K = a.K;
+      for (int x = cta + ncta * warp; x < 3 * P; x += ncta * TX_WARPS) {
+        const int kind = x / P, p = x - kind * P;
+        const size_t cb = cand_base(a, P, p);
+        if (kind == 0) {
+          const float2 l = warp_lse(a.sums + (size_t)p * a.ntiles, a.ntiles, a.T, lane);
+          if (lane == 0) { a.o_lse0[p] = l.x; a.o_lseT[p] = l.y; }
+          continue;
+        }
+        if (kind == 2 && !(a.T > 0.f)) continue;
+        const float3 w = warp_topk(kind == 1 ? a.cand_top + cb : a.cand_key + cb, kind == 1 ? nullptr : a.cand_lg + cb, a.cand_cnt[0] + (kind == 1 ? 0 : a.cap) + p, K, lane);
+        if (lane < K) {
+          const size_t o = (size_t)p * K + lane;
+          if (kind == 1) { a.o_top_tok[o] = __float_as_int(w.x); a.o_top_logit[o] = w.y; }
+          if (kind == 2 || !(a.T > 0.f)) { a.o_draw_tok[o] = __float_as_int(w.x); a.o_draw_logit[o] = w.z; }
+        }
       }
       break;
     }
@@ -1436,17 +1463,23 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
     // parents a request on instead of 8 the extra barrier costs up to 7 %, from 16 on within 2 % either way) ---------------
     const bool spread = MANY && d >= 0 && P > 8 * a.B;
     if (spread) {
-      const int R = mma_replicas(P), K = a.K;
+      const int K = a.K;
 #pragma unroll 1
-      for (int p = cta + ncta * warp; p < P; p += ncta * TX_WARPS) {
-        const size_t cb = (size_t)p * a.ntiles * (R * K);
-        const int* cnt = a.cand_cnt[d & 1];
-        const float2 l = warp_lse(a.sums + (size_t)p * a.ntiles, a.ntiles, a.T, lane);
-        const float3 w = warp_topk(a.cand_top + cb, nullptr, cnt + p, K, lane);
-        float3 x = w;
-        if (a.T > 0.f) x = warp_topk(a.cand_key + cb, a.cand_lg + cb, cnt + a.cap + p, K, lane);
-        if (lane == 0) a.res_lse[p] = l;
-        if (lane < K) a.res_cand[(size_t)p * KMAX + lane] = make_uint4(__float_as_uint(w.x), __float_as_uint(w.y), __float_as_uint(x.x), __float_as_uint(x.z));
+      for (int x = cta + ncta * warp; x < 3 * P; x += ncta * TX_WARPS) {   // (a parent's three parts side by side)
+        const int kind = x / P, p = x - kind * P;
+        const size_t cb = cand_base(a, P, p);
+        if (kind == 0) {
+          const float2 l = warp_lse(a.sums + (size_t)p * a.ntiles, a.ntiles, a.T, lane);
+          if (lane == 0) a.res_lse[p] = l;
+          continue;
+        }
+        if (kind == 2 && !(a.T > 0.f)) continue;
+        const float3 w = warp_topk(kind == 1 ? a.cand_top + cb : a.cand_key + cb, kind == 1 ? nullptr : a.cand_lg + cb, a.cand_cnt[d & 1] + (kind == 1 ? 0 : a.cap) + p, K, lane);
+        uint2* out = reinterpret_cast<uint2*>(a.res_cand + (size_t)p * KMAX + lane);
+        if (lane < K) {
+          if (kind == 1) out[0] = make_uint2(__float_as_uint(w.x), __float_as_uint(w.y));
+          if (kind == 2 || !(a.T > 0.f)) out[1] = make_uint2(__float_as_uint(w.x), __float_as_uint(w.z));
+        }
       }
       if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
     }
