@@ -548,8 +548,14 @@ __device__ __forceinline__ void tx_drain(const TreeArgs& a, const TxSm& sm, cons
   }
 }
 
+// Copies of the rows in group g: the last group of a list may have few parents (a list of 150: its 22 took as long as the 128
+// before them, 26 us).  Not without room for the copies' candidates (a.tail_copies).
+__device__ __forceinline__ int group_replicas(const TreeArgs& a, const int P, const int g) { return g == 0 || a.tail_copies ? mma_replicas(P - g * TX_ROWS) : 1; }
 // where the candidates of parent p start
-__device__ __forceinline__ size_t cand_base(const TreeArgs& a, const int P, const int p) { return (size_t)p * a.ntiles * (mma_replicas(P) * a.K); }
+__device__ __forceinline__ size_t cand_base(const TreeArgs& a, const int P, const int p) {
+  const int g = p / TX_ROWS;
+  return (size_t)(g * TX_ROWS + (p - g * TX_ROWS) * group_replicas(a, P, g)) * a.ntiles * a.K;
+}
 
 // ---- end of a group: the range's sums and surviving candidates of every parent -------------------------------------
 // A row's sums, best logits and best keys by three threads side by side (one after the other, with the lists' atomics behind
@@ -1389,8 +1395,9 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
     if (P <= 0) break;
     // ---- scan ---------------------------------------------------------------------------------------------------------
     if (tlen > 0) {
-      const int R = mma_replicas(P), per = TX_ROWS / R, ngroups = R > 1 ? 1 : (P + TX_ROWS - 1) / TX_ROWS;
+      const int ngroups = (P + TX_ROWS - 1) / TX_ROWS;
       for (int g = 0; g < ngroups; ++g, ++groups) {
+        const int R = group_replicas(a, P, g), per = TX_ROWS / R;
         if (tid < TX_ROWS) {
           const int p = g * TX_ROWS + (R > 1 ? tid % per : tid);
           uint4 e0 = make_uint4(0xFFFFFFFFu, 0u, 0u, 0u), e1 = make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0u);   // row -1: unused
@@ -1617,12 +1624,14 @@ bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
 
 // Workspace of one call over `nreq` requests (or given parents) whose lists hold up to `cap` parents.
 struct TreeWs { size_t head, ent[2], slot[2], sums, cnt, top, key, lg, thr, utop, pool, state, caps, rlse, rcand, upad, wpad, total; int cap; };
+// the built-in scratch array has no room for them
+static bool tail_copies(bool expand, int rows) { return expand || rows > 0; }
 static TreeWs tree_ws(const ts_ctx* ctx, int nreq, int cap, bool expand, int rows) {
   const ts_config& c = ctx->cfg; const TreePlan& p = ctx->tree;
   TreeWs w{}; size_t at = 0;
   auto take = [&](size_t bytes) { const size_t o = at; at = align_up(at + bytes, 256); return o; };
   w.cap = cap = (cap + 7) / 8 * 8;
-  const size_t C = (size_t)cap, nt = (size_t)p.ntiles, cands = (C > TX_ROWS ? C : (size_t)TX_ROWS) * nt * c.K;   // (replicated rows: R * P <= 128)
+  const size_t C = (size_t)cap, nt = (size_t)p.ntiles, cands = (tail_copies(expand, rows) ? (C + TX_ROWS - 1) / TX_ROWS * TX_ROWS : C > TX_ROWS ? C : (size_t)TX_ROWS) * nt * c.K;   // (copies of rows: at most 128 a group)
   w.head = take(256);
   w.ent[0] = take(C * sizeof(ParentEntry));
   if (expand) { w.ent[1] = take(C * sizeof(ParentEntry)); w.slot[0] = take(C * 4); w.slot[1] = take(C * 4); }
@@ -1701,7 +1710,7 @@ cudaError_t tree_score(ts_ctx* ctx, char* scratch, const void* U, const void* A,
                        float* draw_logit, int rows, cudaStream_t st) {
   TreeArgs a{};
   fill_args(ctx, a, scratch, tree_ws(ctx, P, P, false, rows), false, U, A, W, T, seed);
-  a.score_P = P; a.B = 1;
+  a.score_P = P; a.B = 1; a.tail_copies = tail_copies(false, rows) ? 1 : 0;
   a.p_req = p_req; a.p_depth = p_depth; a.p_token = p_token; a.p_hash = p_hash;
   a.o_lse0 = lse0; a.o_lseT = lseT; a.o_top_tok = top_tok; a.o_top_logit = top_logit; a.o_draw_tok = draw_tok; a.o_draw_logit = draw_logit;
   return launch_tree(ctx, a, K_SCORE, st);
@@ -1713,7 +1722,7 @@ cudaError_t tree_expand(ts_ctx* ctx, char* ws, const TreeOut& o, const void* U, 
   TreeArgs a{};
   const TreeWs w = tree_ws(ctx, B, B * c.Nmax > B ? B * c.Nmax : B, true, B * c.D);
   fill_args(ctx, a, ws, w, true, U, A, W, T, seed);
-  a.B = B; a.anchor = anchor; a.theta = theta; a.calib = ctx->calib; a.calib_qT = (ctx->ablation & TS_ABLATE_CALIB_QT) ? 1 : 0;
+  a.B = B; a.tail_copies = 1; a.anchor = anchor; a.theta = theta; a.calib = ctx->calib; a.calib_qT = (ctx->ablation & TS_ABLATE_CALIB_QT) ? 1 : 0;
   a.pool = (unsigned char*)ws + w.pool; a.pool_stride = pool_bytes(c.Nmax);
   int* state = (int*)(ws + w.state);
   a.req_npar = state; a.req_base = state + 2 * (size_t)B; a.req_nscored = state + 3 * (size_t)B; a.root_lseT = (float*)(state + 4 * (size_t)B);

@@ -230,3 +230,9 @@ def test_walks_that_reject_every_sibling(over, T):
         want += max(len(kids.get(cur, [])), 1)
         assert int(sums[b]) == want
     assert int(sums.max()) >= wl.K   # the case was reached
+
+
+# several groups of 128 parents whose last is held once, twice or four times over
+@pytest.mark.parametrize("P", [129, 160, 161, 192, 193])
+def test_last_group_of_a_list(P):
+    check_scores("bf16", 2048, 8, 8, P, 0.7)
