@@ -427,13 +427,17 @@ __device__ __forceinline__ void tx_load_u(const TreeArgs& a, const TxSm& sm, con
   }
 }
 
-// ---- the issuing warp: one tile of MMAs per block -----------------------------------------------------------------------
-__device__ __forceinline__ void tx_issue(const TreeArgs& a, const TxSm& sm, const int tlen, const uint32_t tmem_base, BlockPos& pos, BlockPos& wpos, const int group_no, const int nst) {
+// ---- the issuing warps: one tile of MMAs per block, in turn ---------------------------------------------------------------
+// (Waiting, issuing and committing a block of four MMAs takes a warp 0.75 us, of sixteen 0.9: one warp for the nine blocks of 128 tokens,
+// or the seventeen of 64 at rank 256, was what scans of few parents waited for.  An accumulator stage may change hands: who
+// issues block j has waited, at most three blocks earlier, until a block after j - 2 stages was drained, so that its parity is never two turns off.)
+__device__ __forceinline__ void tx_issue(const TreeArgs& a, const TxSm& sm, const int which, const int tlen, const uint32_t tmem_base, BlockPos& pos, BlockPos& wpos, const int group_no, const int nst) {
   const int nblk = (tlen + a.BN - 1) / a.BN, ksteps = (a.r + 15) / 16;
   const uint32_t slab = (uint32_t)ksteps * 2048u;
   const uint64_t adesc0 = smem_desc(smem_u32(sm.As), 16u, 1024u), bdesc0 = smem_desc(smem_u32(sm.Ws), slab, 1024u);
   if (!tx_wait_warp(sm.a_full, group_no & 1, sm, a)) return;
   for (int nb = 0; nb < nblk; ++nb, pos.next(nst), wpos.next(a.nW)) {
+    if (wpos.slot % TX_ISSUERS != which) continue;   // (by the ring's slots: a wait for a parity is right only for who follows every turn of a slot)
     if (!tx_wait_warp(sm.w_full + wpos.slot, wpos.full(), sm, a)) return;
     if (pos.reused() && !tx_wait_warp(sm.t_empty + pos.slot, pos.empty(), sm, a)) return;
     tc_fence_after();
@@ -1427,7 +1431,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
         const int nst = min(512 / a.BN, TX_STAGE_MAX);   // accumulator stages
         const uint32_t ublocks = RING ? (uint32_t)((tlen + a.BN - 1) / a.BN) : 0u;
         if (warp < TX_SCAN_WARPS) tx_scan<RING>(a, sm, R, min(TX_ROWS, P - g * TX_ROWS), g, t0, tlen, tmem_base, pos, nst, ub0);
-        else if (warp == TX_MMA) tx_issue(a, sm, tlen, tmem_base, pos, wpos, groups, nst);
+        else if (warp < TX_REFRESH) tx_issue(a, sm, warp - TX_MMA, tlen, tmem_base, pos, wpos, groups, nst);
         else if (warp == TX_REFRESH) {
           const uint32_t nblk = (uint32_t)((tlen + a.BN - 1) / a.BN);
           const uint32_t level_end = (uint32_t)(groups + ngroups - g) * nblk + ((a.w_over || a.score_P > 0) ? 0u : (uint32_t)a.nW);

@@ -9,10 +9,11 @@ namespace ts {
 
 constexpr int TX_SCAN_WARPS = 16;          // warps that scan accumulators: 4 tensor-memory lane quarters x 4 splits
 constexpr int TX_SPLIT = TX_SCAN_WARPS / 4;
-constexpr int TX_MMA = TX_SCAN_WARPS;      // issues the MMAs
-constexpr int TX_REFRESH = TX_SCAN_WARPS + 1;   // requests W, keeps the rows' launch-wide bounds current
-constexpr int TX_SELECT = TX_SCAN_WARPS + 2;    // evaluates queued candidates exactly
-constexpr int TX_WARPS = TX_SCAN_WARPS + 3;
+constexpr int TX_ISSUERS = 2;
+constexpr int TX_MMA = TX_SCAN_WARPS;      // this and the next issue the MMAs
+constexpr int TX_REFRESH = TX_MMA + TX_ISSUERS;   // requests W, keeps the rows' launch-wide bounds current
+constexpr int TX_SELECT = TX_REFRESH + 1;       // evaluates queued candidates exactly
+constexpr int TX_WARPS = TX_SELECT + 1;
 constexpr int TX_THREADS = TX_WARPS * 32;
 constexpr int TX_ROWS = 128;               // parent rows of one MMA tile
 constexpr int TX_QCAP = 256;               // candidate queue entries (power of two)
