@@ -572,23 +572,32 @@ __device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, co
   if (role == 0) {
     if (row >= per) return;
     const float T = a.T, invT = T > 0.f ? 1.f / T : 1.f;
-    // the pieces' sums in a fixed order: the same bits on every run (the largest reference first: the exponentials do not wait
-    // for one another; with a running reference four copies of a row took 1.1 us longer)
-    float m = -INFINITY, s0 = 0.f, sT = 0.f;
+    // the pieces' sums in a fixed order: the same bits on every run
+    float m = -INFINITY, lo = INFINITY, s0 = 0.f, sT = 0.f;
 #pragma unroll 1
     for (int rho = 0; rho < R; ++rho)
 #pragma unroll
-      for (int s = 0; s < TX_SPLIT; ++s) m = fmaxf(m, sm.part[(0 * TX_SPLIT + s) * TX_ROWS + rho * per + row]);
+      for (int s = 0; s < TX_SPLIT; ++s) { const float hm = sm.part[(0 * TX_SPLIT + s) * TX_ROWS + rho * per + row]; m = fmaxf(m, hm); lo = fminf(lo, hm); }
+    if (lo == m) {   // nearly always (no piece left the parent's reference): plain sums (a running reference takes four copies of a row 1.1 us longer)
 #pragma unroll 1
-    for (int rho = 0; rho < R; ++rho)
+      for (int rho = 0; rho < R; ++rho)
 #pragma unroll
-      for (int s = 0; s < TX_SPLIT; ++s) {
-        const int rr = rho * per + row;
-        const float hm = sm.part[(0 * TX_SPLIT + s) * TX_ROWS + rr], h0 = sm.part[(1 * TX_SPLIT + s) * TX_ROWS + rr], hT = sm.part[(2 * TX_SPLIT + s) * TX_ROWS + rr];
-        if (hm == -INFINITY) { s0 += h0; continue; }   // (nothing finite: h0 is 0, or NaN if the piece met one)
-        const float d = hm - m;
-        s0 += h0 * __expf(d); sT += hT * __expf(d * invT);
-      }
+        for (int s = 0; s < TX_SPLIT; ++s) { s0 += sm.part[(1 * TX_SPLIT + s) * TX_ROWS + rho * per + row]; sT += sm.part[(2 * TX_SPLIT + s) * TX_ROWS + rho * per + row]; }
+      if (m == -INFINITY) sT = 0.f;   // (nothing finite: the sums are 0, or NaN if a piece met one)
+    } else {
+      m = -INFINITY;
+#pragma unroll 1
+      for (int rho = 0; rho < R; ++rho)
+#pragma unroll
+        for (int s = 0; s < TX_SPLIT; ++s) {
+          const int rr = rho * per + row;
+          const float hm = sm.part[(0 * TX_SPLIT + s) * TX_ROWS + rr], h0 = sm.part[(1 * TX_SPLIT + s) * TX_ROWS + rr], hT = sm.part[(2 * TX_SPLIT + s) * TX_ROWS + rr];
+          if (hm == -INFINITY) { s0 += h0; continue; }
+          if (hm > m) { const float d = m == -INFINITY ? 0.f : m - hm; s0 *= __expf(d); sT *= __expf(d * invT); m = hm; }
+          const float d = hm - m;
+          s0 += h0 * __expf(d); sT += hT * __expf(d * invT);
+        }
+    }
     a.sums[(size_t)p * a.ntiles + tile] = make_float4(m, s0, sT, 0.f);
     return;
   }
@@ -888,6 +897,10 @@ __device__ __forceinline__ void make_parents(const TreeArgs& a, const OwnerSm& s
   }
 }
 
+// The calibrated estimate as one copy of code, so that one warp can bring it into the instruction caches while the others sweep: met
+// for the first time in the first owner phase it took 5 us instead of 1.6.
+__device__ __noinline__ double tx_estimate(const DevCalib& c, int d, double lx, double lse0) { return log_phat(c, d, lx, lse0); }
+
 // One level of one request: merge of its parents, slots and cut of Algorithm 1, the next level's parents.
 // d = depth of the parents just scanned; d = -1: the start of request b (an empty pool and the root as the only parent of
 // level 0) or, for ts_score_parents, the list entry of given parent b.
@@ -1037,7 +1050,7 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
         // the calibrator's input: the untempered conditional, or (ablation) the tempered one
         const bool tempered = a.calib_qT && a.T > 0.f;
         const double lsc = tempered ? 1.0 / (double)a.T : 1.0, lsn = tempered ? lseT : lse0;
-        const double v = logS_v + log_phat(a.calib, d, (double)(which ? s.dlog[t] : s.tlog[(i << lk) + bi]) * lsc, lsn);
+        const double v = logS_v + tx_estimate(a.calib, d, (double)(which ? s.dlog[t] : s.tlog[(i << lk) + bi]) * lsc, lsn);
         if (which) s.clogS[t] = v;
         else { s.ckey[t] = v; ok = !(v < log_theta); }
       }
@@ -1090,7 +1103,12 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
       for (int e = tid; e < M; e += TX_THREADS) {
         if (!live(e)) continue;
         const uint64_t k = skey(key_of(e));
-        if (sh8 == 56 || (k >> (sh8 + 8)) == (prefix >> (sh8 + 8))) atomicAdd(&s.hist[(int)((k >> sh8) & 255u)], 1);
+        if (sh8 == 56 || (k >> (sh8 + 8)) == (prefix >> (sh8 + 8))) {
+          // (one addition per bin and warp: the first pass, over sign and exponent, has two or three bins for 1,700 keys)
+          const int bin = (int)((k >> sh8) & 255u);
+          const unsigned peers = __match_any_sync(__activemask(), bin);
+          if (lane == __ffs(peers) - 1) atomicAdd(&s.hist[bin], __popc(peers));
+        }
       }
       __syncthreads();
       if (warp == 0) {
@@ -1280,13 +1298,13 @@ __device__ __forceinline__ void tx_finalize(const TreeArgs& a, unsigned char* sm
     int cr = 0, pr = 0;
     if (have) {
       const int dx = (s.pv.meta[x] >> 8) & 255; const uint64_t px = s.pv.path[x]; const double kx = s.pv.key[x];
-#pragma unroll 1
+#pragma unroll 4
       for (int t = sub; t < N; t += G) {
-        const int mt = s.pv.meta[t];
-        if (t == x || !(mt >> 16)) continue;
-        const int dt = (mt >> 8) & 255; const uint64_t pt = s.pv.path[t];
-        if (dt < dx || (dt == dx && pt < px)) ++cr;
-        if (before(s.pv.key[t], dt, pt, kx, dx, px)) ++pr;
+        const int mt = s.pv.meta[t], dt = (mt >> 8) & 255;   // (no branches: the loads of four rounds go out together)
+        const uint64_t pt = s.pv.path[t]; const double kt = s.pv.key[t];
+        const bool other = t != x && (mt >> 16) != 0, first = dt < dx || (dt == dx && pt < px);
+        cr += other && first ? 1 : 0;
+        pr += other && (kt > kx || (kt == kx && first)) ? 1 : 0;
       }
     }
     for (int o = 1; o < G; o <<= 1) { cr += __shfl_xor_sync(0xFFFFFFFFu, cr, o); pr += __shfl_xor_sync(0xFFFFFFFFu, pr, o); }
@@ -1392,6 +1410,12 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
   // Phases: d = -2 sweeps the depth-0 rows (given parents: theirs); d = -1 starts the requests; d >= 0 scans the parents of
   // depth d and runs their level step.
   int d = -2;
+  if (tid == 0 && a.score_P == 0)   // the anchors' head rows: on their way while the first rows are swept
+    for (int b = cta; b < a.B; b += ncta) {
+      const int t = a.anchor[b];
+      if (t >= 0 && t < a.V) asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const __nv_bfloat16*>(a.A) + (size_t)t * a.r));
+    }
+  if (warp == TX_REFRESH && a.score_P == 0 && cta < a.B) { const double x = tx_estimate(a.calib, 0, -1.0, 0.5); asm volatile("" ::"d"(x)); }   // (for the instruction caches)
   for (;; ++d) {
     int P = nreq;
     if (d >= 0) {
