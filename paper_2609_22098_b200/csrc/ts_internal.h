@@ -102,7 +102,7 @@ int few_tiles(const ts_config& c);
 int few_capacity(const ts_config& c, bool use_tree);
 cudaError_t launch_score_few(const ts_ctx* ctx, const ScoreArgs& a, int p_bound, cudaStream_t st);
 // tensor maps (ts_tmap.cu), encoded or found cached in the context; false: not available.  Of W [r][V] for the walk
-// (boxes of 64 tokens x r rows rounded up to 64), and of the one-launch kernel's [r][stride] matrix (rounded up to 16).
+// and of the one-launch kernel's [r][stride] matrix: boxes of 64 tokens x r rows rounded up to 16.
 bool w_tensor_map(ts_ctx* ctx, const void* W);
 bool tree_tensor_map(ts_ctx* ctx, const void* W, int stride, CUtensorMap* out);
 // of base logits [B][D][stride], boxes of 64 tokens x one depth x `rows` requests

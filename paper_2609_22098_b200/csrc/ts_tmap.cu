@@ -38,7 +38,7 @@ bool w_tensor_map(ts_ctx* ctx, const void* W) {
   if (ctx->tma_state < 0 || ((uintptr_t)W & 15u) != 0) return false;
   if (ctx->tma_state == 1 && ctx->tmapW_ptr == W) return true;
   CUtensorMap tm;
-  if (!encode(ctx, W, ctx->cfg.V, (ctx->cfg.r + 63) / 64 * 64, &tm)) { ctx->tma_state = -1; return false; }   // (r <= 256 = the most rows a box may have)
+  if (!encode(ctx, W, ctx->cfg.V, (ctx->cfg.r + 15) / 16 * 16, &tm)) { ctx->tma_state = -1; return false; }   // (r <= 256 = the most rows a box may have)
   memcpy(ctx->tmapW, &tm, sizeof(tm));
   ctx->tmapW_ptr = W;
   ctx->tma_state = 1;

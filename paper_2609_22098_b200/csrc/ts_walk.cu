@@ -27,8 +27,8 @@ namespace ts {
 constexpr int WK_EPI = 16;                 // warps that read accumulators: 4 lane quarters x 4 sets of tiles
 constexpr int WK_LOAD = WK_EPI;            // tensor memory; in the streaming form it requests W and issues the MMAs
 constexpr int WK_THREADS = (WK_EPI + 1) * 32;
-constexpr int WK_REQ = 32;                 // requests of one reduction pass (columns of a tile)
-constexpr int WK_TR = 3;                   // tiles of a set in tensor memory together: a round is 12 tiles of 32 columns
+constexpr int WK_REQ = 64;                 // requests of one reduction pass (columns of a tile) at most: WalkArgs::req of them, 16, 32 or 64
+constexpr int WK_TR = 3;                   // tiles of a set in tensor memory together at most: WalkArgs::tr of them; a round is four sets' (512 columns)
 constexpr int WK_ROUND = 4 * WK_TR;
 constexpr int WK_VALS = 2 * WK_COLS;       // sums of a request: residual and proposal mass at every coefficient
 constexpr int WK_SLOTS = 6;                // requests whose rows a warp has in flight or in work: three pairs
@@ -66,7 +66,7 @@ __device__ __forceinline__ uint32_t wk_idesc(int n) {
 }
 
 // ---- set-up of one request, by the whole CTA: child ranges, accept-test inputs of every edge, what a reduction at a node needs ----
-__device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const int b, int* s_par, float2* s_z) {
+__device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const int b, int* s_par, int* s_tok, float2* s_z) {
   const int tid = threadIdx.x, N = a.N;
   const size_t nb = (size_t)b * N, cb = (size_t)b * (N + 1);
   const int n = a.n_nodes[b];
@@ -86,7 +86,7 @@ __device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const
       const float zm = zr.m, zl = zr.logs;
       s_z[i] = make_float2(zm, zl);
       bad |= (zm != zm || isinf(zm) || zl != zl || isinf(zl) || lq != lq) ? 1 : 0;
-      if (i) s_par[i - 1] = par;
+      if (i) { s_par[i - 1] = par; s_tok[i - 1] = tok; }
       NodeDesc nd;
       nd.zrow = row0 + i; nd.urow = b * a.D + min(dep, a.D - 1);   // (a leaf at depth D asks only for its target row: keep the base row inside U)
       nd.tok = tok; nd.zoff = (-zm * invT - zl) * LOG2E; nd.qoff = -ls * LOG2E; nd.zmax = zm; nd.zlogs = zl;
@@ -95,6 +95,7 @@ __device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const
       a.child[cb + i] = make_int2(-1, 0);
     }
   }
+  if (tid == 0) { st.cfirst = -1; st.ccnt = 0; }
   bad = __syncthreads_or(bad);
   for (int i = tid; okn && i < n; i += WK_THREADS) {
     if (bad) { if (a.edge_stat) a.edge_stat[nb + i] = 0.f; continue; }
@@ -105,9 +106,10 @@ __device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const
       int m = 1;
       while (i + m < n && s_par[i + m] == par) ++m;
       a.child[cb + par + 1] = make_int2(i, m);
+      if (par < 0) { st.cfirst = i; st.ccnt = m; }
     }
     const int64_t row = row0 + par + 1;
-    const int x = a.tok[nb + i];
+    const int x = s_tok[i];
     const double lp = ((double)__bfloat162float(a.Z[row * a.V + x]) - (double)s_z[par + 1].x) / (double)a.T - (double)s_z[par + 1].y;
     const double lq = (double)a.logqT[nb + i];
     WalkEdge e;
@@ -122,8 +124,7 @@ __device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const
   if (tid == 0) {
     st.cur = -1; st.j = 0; st.acc = 0; st.nf = 0; st.npass = 0; st.phase = 0;
     st.C = 0.0; st.Zj = 1.0; st.Qused = 0.0; st.passC = 0.0; st.partsC = -1.0;
-    st.cfirst = -1; st.ccnt = 0; st.nC = 0; st.pcol = 0;
-    if (okn && !bad) { const int2 c = a.child[cb]; st.cfirst = c.x; st.ccnt = c.y; }
+    st.nC = 0; st.pcol = 0;
     a.flags[b] = 0u;
     a.status[b] = !okn ? TS_ERR_INVALID : (bad ? TS_ERR_NUMERIC : TS_OK);
     if (!okn || bad) { st.phase = 4; a.acc_len[b] = 0; a.bonus[b] = -1; }
@@ -215,28 +216,36 @@ __device__ __forceinline__ void wk_advance(const WalkArgs& a, WalkState& st, con
           for (int o = 1; o < 32; o <<= 1) { const double x = __shfl_up_sync(0xFFFFFFFFu, Q, o); if (lane >= o) Q += x; }
           Q = __shfl_up_sync(0xFFFFFFFFu, Q, 1);
           if (lane == 0) Q = 0.0;
-          const double inv = Q < 1.0 ? 1.0 / (1.0 - Q) : 0.0;
-          const double next = __shfl_down_sync(0xFFFFFFFFu, ck, 1), rh = lane + 1 < have && next > ck ? 1.0 / (next - ck) : 0.0;
+          const float inv = Q < 1.0 ? (float)(1.0 / (1.0 - Q)) : 0.f, ckf = (float)ck, Fkf = (float)Fk, Gkf = (float)Gk;
+          const float next = __shfl_down_sync(0xFFFFFFFFu, ckf, 1), rh = lane + 1 < have && next > ckf ? 1.f / (next - ckf) : 0.f;
+          // (guesses in fp32, the sum of the steps in double: some 2e-7 of rounding, a quarter of what WK_TOL allows)
+          const float pf = lane < m ? (float)e.px : 0.f, qf = lane < m ? (float)e.qx : 1.f;
+          float mass = (float)own;
           double c = C;
 #pragma unroll 1
           for (int i = nf; i < m && nC < WK_COLS; ++i) {
             // the other tokens' share at c: between two evaluated coefficients by Hermite's cubic, beyond the last by the decay there
-            const int n = __popc(__ballot_sync(0xFFFFFFFFu, lane < have && ck <= c));
+            const float cf = (float)c;
+            const int n = __popc(__ballot_sync(0xFFFFFFFFu, lane < have && ckf <= cf));
             const int k0 = n > 0 ? n - 1 : 0, k1 = n < have ? n : have - 1;
-            const double c0 = __shfl_sync(0xFFFFFFFFu, ck, k0), f0 = __shfl_sync(0xFFFFFFFFu, Fk, k0), g0 = __shfl_sync(0xFFFFFFFFu, Gk, k0);
-            const double c1 = __shfl_sync(0xFFFFFFFFu, ck, k1), f1 = __shfl_sync(0xFFFFFFFFu, Fk, k1), g1 = __shfl_sync(0xFFFFFFFFu, Gk, k1);
-            const double w = __shfl_sync(0xFFFFFFFFu, rh, k0), own_sum = wk_lanes_sum(own), scale = __shfl_sync(0xFFFFFFFFu, inv, i);
-            double f;
-            if (n == 0) f = f0 - (c - c0) * g0;
-            else if (n == have) f = f0 > 1e-30 ? f0 * (double)__expf((float)(-(c - c0) * g0) / (float)f0) : 0.0;
+            const float c0 = __shfl_sync(0xFFFFFFFFu, ckf, k0), f0 = __shfl_sync(0xFFFFFFFFu, Fkf, k0), g0 = __shfl_sync(0xFFFFFFFFu, Gkf, k0);
+            const float c1 = __shfl_sync(0xFFFFFFFFu, ckf, k1), f1 = __shfl_sync(0xFFFFFFFFu, Fkf, k1), g1 = __shfl_sync(0xFFFFFFFFu, Gkf, k1);
+            const float w = __shfl_sync(0xFFFFFFFFu, rh, k0), scale = __shfl_sync(0xFFFFFFFFu, inv, i);
+            float sum = mass;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+            const float dc = (float)(c - (double)c0);
+            float f;
+            if (n == 0) f = f0 - dc * g0;
+            else if (n == have) f = f0 > 1e-30f ? f0 * __expf(-dc * g0 / f0) : 0.f;
             else {
-              const double h = c1 - c0, t = (c - c0) * w, r = 1.0 - t;
-              f = r * r * (f0 * (1.0 + 2.0 * t) - g0 * h * t) + t * t * (f1 * (3.0 - 2.0 * t) + g1 * h * r);
+              const float h = c1 - c0, t = dc * w, r = 1.f - t;
+              f = r * r * (f0 * (1.f + 2.f * t) - g0 * h * t) + t * t * (f1 * (3.f - 2.f * t) + g1 * h * r);
             }
-            const double z = fmax(f, 0.0) + own_sum;
-            if (!(z > 1e-30) || scale == 0.0) break;   // uniform
-            c += z * scale;
-            if (lane < m && lane >= i) own = fmax(e.px - c * e.qx, 0.0);   // (sibling i keeps this from now on)
+            const float z = fmaxf(f, 0.f) + sum;
+            if (!(z > 1e-30f) || scale == 0.f) break;   // uniform
+            c += (double)(z * scale);
+            if (lane < m && lane >= i) mass = fmaxf(fmaf(-(float)c, qf, pf), 0.f);   // (sibling i keeps this from now on)
             if (lane == nC) mine = (float)c;
             ++nC;
           }
@@ -317,14 +326,14 @@ __device__ __forceinline__ void wk_advance(const WalkArgs& a, WalkState& st, con
 // first warp of every set issues its set's tiles.
 __device__ __forceinline__ void wk_mma(const WalkArgs& a, const WalkSm& sm, const int ncol, const uint32_t ws, const uint32_t slot, const uint32_t tmem_base) {
   const int ksteps = (a.r + 15) / 16;
-  const uint32_t slab = (uint32_t)((a.r + 63) / 64 * 64) * 128u;
+  const uint32_t slab = (uint32_t)ksteps * 2048u;
   tc_fence_after();
   if (elect_one()) {
     const uint64_t ad = smem_desc(smem_u32(sm.Ws) + 2u * ws * slab, slab, 1024u), bd = smem_desc(smem_u32(sm.Bs), 16u, 1024u);
-    const uint32_t idesc = wk_idesc(ncol), d = tmem_base + slot * (uint32_t)WK_REQ;
+    const uint32_t idesc = wk_idesc(ncol), d = tmem_base + slot * (uint32_t)a.req;
 #pragma unroll 4
     for (int ks = 0; ks < ksteps; ++ks)
-      mma_bf16(d, ad + (uint64_t)(ks * 128), bd + (uint64_t)((ks >> 2) * (WK_REQ * 128 / 16) + (ks & 3) * 2), idesc, ks > 0 ? 1u : 0u);
+      mma_bf16(d, ad + (uint64_t)(ks * 128), bd + (uint64_t)((ks >> 2) * (a.req * 8) + (ks & 3) * 2), idesc, ks > 0 ? 1u : 0u);
     mma_commit(sm.t_full + slot);
     if (a.ring) mma_commit(sm.w_free + ws);
   }
@@ -340,7 +349,7 @@ __device__ __forceinline__ bool wk_drained(const WalkArgs& a, const WalkSm& sm, 
 __device__ __forceinline__ void wk_stream(const WalkArgs& a, const WalkSm& sm, const CUtensorMap* tm, const int ncol, const int t0, const int tlen, const uint32_t pass,
                                           uint32_t& wreq, uint32_t rnd, const uint32_t tmem_base) {
   const int ntile = (tlen + 127) / 128;
-  const uint32_t slab = (uint32_t)((a.r + 63) / 64 * 64) * 128u, ring = (uint32_t)a.ring, w0 = pass * (uint32_t)ntile;
+  const uint32_t slab = (uint32_t)((a.r + 15) / 16) * 2048u, ring = (uint32_t)a.ring, w0 = pass * (uint32_t)ntile;
   for (int t = 0; t <= ntile; ++t) {
     for (const uint32_t upto = w0 + (uint32_t)t + ring; wreq < upto; ++wreq) {
       const uint32_t slot = wreq % ring, use = wreq / ring;
@@ -354,7 +363,7 @@ __device__ __forceinline__ void wk_stream(const WalkArgs& a, const WalkSm& sm, c
     }
     if (t == ntile) break;
     const uint32_t x = w0 + (uint32_t)t;
-    const int i = t % WK_ROUND;
+    const int i = t % (4 * a.tr);
     if (i == 0 && t > 0) ++rnd;
     if (i < 4 && !wk_drained(a, sm, i, rnd)) return;
     if (!__all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + x % ring, (x / ring) & 1, a, sm.abort))) return;
@@ -399,14 +408,15 @@ __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm,
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = warp & 3, set = warp >> 2;
   const int ntile = (tlen + 127) / 128;
   const float zs = (1.f / a.T) * 1.4426950408889634f;   // exponentials as powers of two
-  float* mine = sm.part + (size_t)warp * WK_REQ * WK_VALS;
+  float* mine = sm.part + (size_t)warp * a.req * WK_VALS;
   constexpr uint32_t SEG = wk_seg(AL), SLOT = wk_slot(AL);
-  const uint32_t ring = smem_u32(sm.stage) + (uint32_t)warp * (WK_SLOTS * SLOT), dbase = smem_u32(desc);
+  const uint32_t ring = smem_u32(sm.stage) + (uint32_t)warp * (uint32_t)(2 * a.pairs) * SLOT, dbase = smem_u32(desc);
   constexpr int CPS = AL ? 4 : 5;                       // 16-byte copies of a segment
   const int seg = lane / CPS, ch = lane - seg * CPS;    // lane's copy of a request: 16 bytes of one segment (tile, row)
   bool alive = true;
-  for (int r0 = 0; r0 < ntile; r0 += WK_ROUND, ++rnd) {
-    const int left = min(ntile - r0, WK_ROUND) - set, ntl = left > 0 ? (left + 3) / 4 : 0;   // the set's tiles: r0 + set + 4 i
+  const int round = 4 * a.tr;
+  for (int r0 = 0; r0 < ntile; r0 += round, ++rnd) {
+    const int left = min(ntile - r0, round) - set, ntl = left > 0 ? (left + 3) / 4 : 0;   // the set's tiles: r0 + set + 4 i
     const int tok = (r0 + set) * 128 + q * 32;                                              // the warp's first token in the first of them; then + 512 i
     int nt = 0;                                                                             // its tiles with any token
 #pragma unroll
@@ -448,7 +458,7 @@ __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm,
       used ^= 1u << slot;
     }
     tc_fence_after();
-    const uint32_t tcol = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(set * WK_REQ);
+    const uint32_t tcol = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(set * a.req);
     uint32_t at = 0u, ahead = 4u * SLOT;   // places of this pair and of the one to be requested
 #pragma unroll 1
     for (int j = 0; j < nreq && alive; j += 2) {
@@ -458,7 +468,7 @@ __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm,
       uint32_t acc[2 * WK_TR];
 #pragma unroll
       for (int i = 0; i < WK_TR; ++i)
-        if (i < nt) asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(acc[2 * i]), "=r"(acc[2 * i + 1]) : "r"(tcol + (uint32_t)(4 * i * WK_REQ + j)) : "memory");
+        if (i < nt) asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(acc[2 * i]), "=r"(acc[2 * i + 1]) : "r"(tcol + (uint32_t)(4 * i * a.req + j)) : "memory");
       float p[2 * WK_TR], qq[2 * WK_TR], c0[2]; int nC[2];
       const int two = j + 1 < nreq ? 1 : 0;
       const uint32_t dj = dbase + (uint32_t)j * (uint32_t)sizeof(RedDesc);
@@ -561,6 +571,119 @@ __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm,
   }
 }
 
+// The same for ranges of up to four tiles (a set has one: V to 75,776 on 148 SMs) and aligned rows: four requests at a time, whose copies are one
+// instruction of the warp.  (Pairs: 104 us of verification for the chain of 100 requests at V = 64,000.)
+__device__ __forceinline__ void wk_epilogue4(const WalkArgs& a, const WalkSm& sm, const int nreq, const int ncol, const int t0, const int tlen,
+                                             const uint32_t tmem_base, uint32_t& used, uint32_t& rnd, const bool first_pass, const RedDesc* desc) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = warp & 3, set = warp >> 2;
+  const int ntile = (tlen + 127) / 128, tok = set * 128 + q * 32;
+  const float zs = (1.f / a.T) * 1.4426950408889634f;   // exponentials as powers of two
+  float* mine = sm.part + (size_t)warp * a.req * WK_VALS;
+  constexpr uint32_t GROUP = 8u * 64u;                  // four requests' two segments
+  const uint32_t ring = smem_u32(sm.stage) + (uint32_t)warp * (WK_SLOTS * (uint32_t)wk_slot(true)), dbase = smem_u32(desc);
+  const int ch = lane & 3, mine4 = lane >> 3;           // lane's copy: 16 bytes of the target or base segment of one of the four
+  const bool has = set < ntile, any = has && tok < tlen, act = any && tok + 8 * ch < tlen, tail = any && tok + 32 > tlen;
+  const uint64_t off = 2ull * (uint64_t)(uint32_t)(t0 + tok) + 16u * (uint32_t)ch;
+  const uint32_t from = dbase + (uint32_t)mine4 * (uint32_t)sizeof(RedDesc) + (uint32_t)((lane >> 2) & 1) * 8u, to = ring + (uint32_t)(lane >> 2) * 64u + (uint32_t)ch * 16u;
+  bool alive = true;
+  auto stage = [&](int j, uint32_t at) {
+    if (act && j + mine4 < nreq) {
+      uint64_t row;
+      asm volatile("ld.shared.u64 %0, [%1];" : "=l"(row) : "r"(from + (uint32_t)j * (uint32_t)sizeof(RedDesc)));
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + at), "l"(row + off) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  stage(0, 0u);
+  stage(4, GROUP);
+  if (q == 0 && !a.ring) {
+    alive = wk_drained(a, sm, set, rnd);
+    if (has && alive && first_pass && a.use_tma) alive = __all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + set, 0, a, sm.abort));
+    if (has && alive) wk_mma(a, sm, ncol, (uint32_t)set, (uint32_t)set, tmem_base);
+  }
+  if (has) {
+    if (alive) alive = __all_sync(0xFFFFFFFFu, wk_wait(sm.t_full + set, (used >> set) & 1u, a, sm.abort));
+    used ^= 1u << set;
+  }
+  tc_fence_after();
+  const uint32_t tcol = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(set * a.req);
+  uint32_t at = 0u, ahead = 2u * GROUP;
+#pragma unroll 1
+  for (int j = 0; j < nreq && alive; j += 4) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
+    stage(j + 8, ahead);
+    uint32_t acc[4] = {0u, 0u, 0u, 0u};
+    if (any) asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(acc[0]), "=r"(acc[1]), "=r"(acc[2]), "=r"(acc[3]) : "r"(tcol + (uint32_t)j) : "memory");
+    const int n = min(4, nreq - j);
+    const uint32_t dj = dbase + (uint32_t)j * (uint32_t)sizeof(RedDesc);
+    float p[4], qq[4], zoff[4], qoff[4], c0[4]; int nC[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      int b;
+      const uint32_t dh = dj + (uint32_t)(h < n ? h : 0) * (uint32_t)sizeof(RedDesc);   // (the first stands in for those that are not there)
+      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=f"(zoff[h]), "=f"(qoff[h]), "=r"(b), "=r"(nC[h]) : "r"(dh + 16u));
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(c0[h]) : "r"(dh + 32u));
+    }
+    tmem_ld_wait();
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      p[h] = qq[h] = 0.f;
+      if (any && h < n) {
+        uint32_t z, u;
+        const uint32_t zr = ring + at + (uint32_t)h * 128u + (uint32_t)lane * 2u;
+        asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(z) : "r"(zr));
+        asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(u) : "r"(zr + 64u));
+        p[h] = ex2_approx(fmaf(__uint_as_float(z << 16), zs, zoff[h]));
+        qq[h] = ex2_approx(fmaf(__uint_as_float(acc[h]) + __uint_as_float(u << 16), zs, qoff[h]));
+        if (tail && tok + lane >= tlen) { p[h] = 0.f; qq[h] = 0.f; }
+      }
+    }
+    at = at == 2u * GROUP ? 0u : at + GROUP;
+    ahead = ahead == 2u * GROUP ? 0u : ahead + GROUP;
+    float* to_part = mine + j * WK_VALS;
+    if (nC[0] == 1 && nC[1] == 1 && nC[2] == 1 && nC[3] == 1) {
+      float x[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) x[h] = fmaxf(fmaf(-c0[h], qq[h], p[h]), 0.f);
+      const float v = wk_fold<4>(x, lane);
+      if ((lane & 7) == 0 && mine4 < n) to_part[mine4 * WK_VALS] = v;
+      continue;
+    }
+#pragma unroll 1
+    for (int h = 0; h < n; ++h, to_part += WK_VALS) {
+      const float ph = h == 0 ? p[0] : (h == 1 ? p[1] : (h == 2 ? p[2] : p[3])), qh = h == 0 ? qq[0] : (h == 1 ? qq[1] : (h == 2 ? qq[2] : qq[3]));
+      const int cols = h == 0 ? nC[0] : (h == 1 ? nC[1] : (h == 2 ? nC[2] : nC[3]));
+      float c[WK_COLS];
+      const uint32_t dc = dj + (uint32_t)h * (uint32_t)sizeof(RedDesc) + 32u;
+      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3]) : "r"(dc));
+      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(c[4]), "=f"(c[5]), "=f"(c[6]), "=f"(c[7]) : "r"(dc + 16u));
+      if (cols == 1 || (cols & WK_GRID)) {
+        float x[WK_COLS];
+        x[0] = fmaxf(fmaf(-c[0], qh, ph), 0.f);
+#pragma unroll
+        for (int k = 1; k < WK_COLS; ++k) x[k] = fabsf(fmaf(-c[k], qh, ph));
+        const float v = wk_fold<WK_COLS>(x, lane);
+        if ((lane & 3) == 0) to_part[lane >> 2] = v;
+      } else {
+        float x[WK_VALS];
+#pragma unroll
+        for (int k = 0; k < WK_COLS; ++k) {
+          const float t = fmaf(-c[k], qh, ph);
+          x[k] = fmaxf(t, 0.f); x[WK_COLS + k] = t > 0.f ? qh : 0.f;
+        }
+        const float v = wk_fold<WK_VALS>(x, lane);
+        if ((lane & 1) == 0) to_part[lane >> 1] = v;
+      }
+    }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(sm.t_empty + set);
+  ++rnd;
+}
+
 // ---- the bonus token of one request whose walk is over, by the CTA that owns it ----------------------------------------------
 __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st, const int b, float* s_dot) {
   __shared__ float s_a[RMAX];
@@ -571,6 +694,7 @@ __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st,
   const int v = st.cur, nf = st.nf;
   const double C = st.C;
   const NodeDesc nd = a.node[cb + v + 1];
+  const uint64_t hv = a.node_hash[cb + v + 1];
   // the range that holds the token: cumulative range sums at C (to first order from the coefficient they were evaluated at),
   // corrected for the tested siblings, which keep the residual they had when tested
   double* s_pt = reinterpret_cast<double*>(s_dot);
@@ -589,7 +713,7 @@ __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st,
   for (int k = tid; k < a.r; k += WK_THREADS) s_a[k] = __bfloat162float(a.A[(size_t)nd.tok * a.r + k]);
   __syncthreads();
   if (warp == 0) {
-    const double u = u01(stream_words(a.seed, b, a.node_hash[cb + v + 1], STREAM_BONUS, 0u).x);
+    const double u = u01(stream_words(a.seed, b, hv, STREAM_BONUS, 0u).x);
     // a lane adds up neighbouring ranges, the warp scans the lanes, the lane with the crossing looks closer
     const double target = u * st.Zj;
     const int per = (a.vt_n + 31) / 32, r0 = min(a.vt_n, lane * per), r1 = min(a.vt_n, r0 + per);
@@ -617,6 +741,10 @@ __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st,
   double carry = 0.0;
   for (int c0 = s_lo; c0 < s_hi; c0 += WK_CHUNK) {
     const int len = min(WK_CHUNK, s_hi - c0);
+    float zv[2] = {0.f, 0.f}, uv[2] = {0.f, 0.f};   // requested before the low-rank part, used after it
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (2 * tid + h < len) { zv[h] = __bfloat162float(zr[c0 + 2 * tid + h]); if (need_q) uv[h] = __bfloat162float(ur[c0 + 2 * tid + h]); }
     // low-rank part of the draft logits, rank in four slices (one when rows are not aligned): loads of eight rows together
     if (need_q) {
       if (vec) {
@@ -669,10 +797,10 @@ __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st,
       if (o < len) {
         double Cw = C;
         for (int f = 0; f < nf; ++f) if (st.fx[f] == w) Cw = st.fC[f];
-        const double p = exp(((double)__bfloat162float(zr[w]) - (double)nd.zmax) / (double)a.T - (double)nd.zlogs);
+        const double p = exp(((double)zv[h] - (double)nd.zmax) / (double)a.T - (double)nd.zlogs);
         double q = 0.0;
         if (Cw != 0.0) {
-          const float lg = __bfloat162float(ur[w]) + ((s_dot[o] + s_dot[WK_CHUNK + o]) + (s_dot[2 * WK_CHUNK + o] + s_dot[3 * WK_CHUNK + o]));
+          const float lg = uv[h] + ((s_dot[o] + s_dot[WK_CHUNK + o]) + (s_dot[2 * WK_CHUNK + o] + s_dot[3 * WK_CHUNK + o]));
           q = exp((double)lg / (double)a.T - lseT);
         }
         rw[h] = fmax(p - Cw * q, 0.0);
@@ -707,11 +835,11 @@ template <bool AL>
 __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_constant__ WalkArgs a, const __grid_constant__ CUtensorMap tmW) {
   extern __shared__ __align__(16) unsigned char raw[];
   __shared__ RedDesc s_desc[WK_REQ];
-  __shared__ int s_tok[WK_REQ], s_par[256], s_cnt[WK_EPI + 1];
+  __shared__ int s_tok[WK_REQ], s_par[256], s_kid[256], s_cnt[WK_EPI + 1];
   __shared__ float2 s_z[257];   // (maximum, log-sum-exp) of a request's rows
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = (int)blockIdx.x, ncta = (int)gridDim.x;
-  const int rp = (a.r + 63) / 64 * 64, t0 = cta * a.vt_TV, tlen = min(a.vt_TV, a.V - t0), ntile = (tlen + 127) / 128;
-  const uint32_t slab = (uint32_t)rp * 128u;
+  const int rp = (a.r + 63) / 64 * 64, rw = (a.r + 15) / 16 * 16, t0 = cta * a.vt_TV, tlen = min(a.vt_TV, a.V - t0), ntile = (tlen + 127) / 128;
+  const uint32_t slab = (uint32_t)rw * 128u;
   unsigned char* base = raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u);
   WalkSm sm;
   sm.Ws = base; sm.Bs = base + a.oB; sm.stage = base + a.oT; sm.part = reinterpret_cast<float*>(base + a.oP);
@@ -740,8 +868,8 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
   if (!a.use_tma) {   // no tensor map, or rows that are not whole 16 bytes: plain loads into the same swizzled places
     const bool vec = (a.V & 7) == 0;
     const unsigned short* Wg = reinterpret_cast<const unsigned short*>(a.W);
-    for (int idx = tid; idx < a.vt_TV / 64 * rp * 8; idx += WK_THREADS) {
-      const int sl = idx / (rp * 8), rem = idx - sl * rp * 8, k = rem >> 3, j = rem & 7, v = t0 + sl * 64 + j * 8;
+    for (int idx = tid; idx < a.vt_TV / 64 * rw * 8; idx += WK_THREADS) {
+      const int sl = idx / (rw * 8), rem = idx - sl * rw * 8, k = rem >> 3, j = rem & 7, v = t0 + sl * 64 + j * 8;
       uint32_t w[4] = {0u, 0u, 0u, 0u};
       if (k < a.r) {
         const unsigned short* src = Wg + (size_t)k * a.V + v;
@@ -753,7 +881,7 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
       *reinterpret_cast<uint4*>(sm.Ws + (size_t)sl * slab + k * 128 + ((j ^ (k & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
-  for (int i = tid; i < rp / 64 * WK_REQ * 8; i += WK_THREADS) reinterpret_cast<uint4*>(sm.Bs)[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = tid; i < rp / 64 * a.req * 8; i += WK_THREADS) reinterpret_cast<uint4*>(sm.Bs)[i] = make_uint4(0u, 0u, 0u, 0u);
   fence_async_smem();
   tc_fence_before();
   __syncthreads();
@@ -763,7 +891,7 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
   pdl_launch_dependents();
 
   const int nown = a.B > cta ? (a.B - cta + ncta - 1) / ncta : 0;   // requests cta, cta + ncta, ...
-  for (int i = 0; i < nown; ++i) wk_setup(a, sm.st[i], cta + i * ncta, s_par, s_z);
+  for (int i = 0; i < nown; ++i) wk_setup(a, sm.st[i], cta + i * ncta, s_par, s_kid, s_z);
   unsigned gen = 0;
   const unsigned nexpect = (unsigned)ncta + (a.lost_arrival ? 1u : 0u);
   bool dead = false, finished = false;
@@ -792,8 +920,8 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
       for (int i = warp; i < nown; i += WK_EPI) wk_advance(a, sm.st[i], cta + i * ncta, lane, step + 1);
     if (!grid_barrier(a.barrier, nexpect, gen, a.wait_limit)) { dead = true; break; }
     int nwk = 0;
-    for (int sb = 0; sb == 0 || sb < nwk; sb += WK_REQ) {
-      // the requests that asked, in order of their numbers: the sb-th to the (sb + WK_REQ - 1)-th of them
+    for (int sb = 0; sb == 0 || sb < nwk; sb += a.req) {
+      // the requests that asked, in order of their numbers: the sb-th to the (sb + req - 1)-th of them
       nwk = 0;
       for (int c0 = 0; c0 < a.B; c0 += WK_EPI * 32) {
         const int b = c0 + tid;
@@ -809,7 +937,7 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
         int off = nwk;
         for (int w = 0; w < WK_EPI; ++w) { if (w < warp) off += s_cnt[w]; nwk += s_cnt[w]; }
         const int at = off + __popc(bal & ((1u << lane) - 1u)) - sb;
-        if (want && at >= 0 && at < WK_REQ) {
+        if (want && at >= 0 && at < a.req) {
           RedDesc d;
           const int64_t zrow = (int64_t)(((uint64_t)r0.y << 32) | r0.x);
           d.z = a.Z + zrow * a.V; d.u = __uint_as_float(r2.x) != 0.f ? a.U + (size_t)(int)r0.z * a.V : d.z;   // (no proposal in the sum: its base row is not touched)
@@ -822,11 +950,11 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
         __syncthreads();
       }
       if (nwk == 0) break;
-      const int nreq = min(WK_REQ, nwk - sb), ncol = (nreq + 15) & ~15;
+      const int nreq = min(a.req, nwk - sb), ncol = (nreq + 15) & ~15;
       // head rows of the requests' nodes: the B operand, K-major with the 128-byte swizzle
       for (int idx = tid; idx < nreq * (a.r / 8); idx += WK_THREADS) {
         const int g = idx / (a.r / 8), ck = idx - g * (a.r / 8);
-        *reinterpret_cast<uint4*>(sm.Bs + (ck >> 3) * (WK_REQ * 128) + g * 128 + (((ck & 7) ^ (g & 7)) << 4)) =
+        *reinterpret_cast<uint4*>(sm.Bs + (ck >> 3) * (a.req * 128) + g * 128 + (((ck & 7) ^ (g & 7)) << 4)) =
             __ldg(reinterpret_cast<const uint4*>(a.A + (size_t)s_tok[g] * a.r + ck * 8));
       }
       // ask L2 for this range of the rows that will be read
@@ -840,8 +968,9 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
-      if (warp < WK_EPI) wk_epilogue<AL>(a, sm, nreq, ncol, t0, tlen, tmem_base, used, rnd, pass == 0u, s_desc);
-      else if (a.ring) wk_stream(a, sm, &tmW, ncol, t0, tlen, pass, wreq, pass * (uint32_t)((ntile + WK_ROUND - 1) / WK_ROUND), tmem_base);
+      if (AL && a.tr == 1) { if (warp < WK_EPI) wk_epilogue4(a, sm, nreq, ncol, t0, tlen, tmem_base, used, rnd, pass == 0u, s_desc); }
+      else if (warp < WK_EPI) wk_epilogue<AL>(a, sm, nreq, ncol, t0, tlen, tmem_base, used, rnd, pass == 0u, s_desc);
+      if (warp == WK_LOAD && a.ring) wk_stream(a, sm, &tmW, ncol, t0, tlen, pass, wreq, pass * (uint32_t)((ntile + 4 * a.tr - 1) / (4 * a.tr)), tmem_base);
       ++pass;
       tc_fence_before();
       __syncthreads();
@@ -853,7 +982,7 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
         if (wk_has(d.nC, val)) {
           float s = 0.f;
 #pragma unroll
-          for (int w = 0; w < WK_EPI; ++w) s += sm.part[w * WK_REQ * WK_VALS + x];
+          for (int w = 0; w < WK_EPI; ++w) s += sm.part[w * a.req * WK_VALS + x];
           a.part[((size_t)d.b * WK_VALS + val) * a.vt_n + cta] = s;
         }
       }
@@ -892,27 +1021,40 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
 // Host side
 // ------------------------------------------------------------------------------------------------
 // Shared-memory plan: the range of W resident where it fits, else a ring of 128-token blocks (that needs the tensor map).
+// Requests a pass takes and tiles a set holds: 64 requests where a range has eight tiles at most (the columns of eight tiles are all of tensor
+// memory), else 32 and three tiles; fewer where the batch has fewer, so that W stays resident in more of shared memory.  (32 for all: the
+// chain of 100 requests at V = 64,000 took 104 us to verify instead of 85 before several coefficients; room for 32 always: one request at
+// V = 200,008 streamed W and took 48 us instead of 41.)
 bool walk_plan(const ts_ctx* ctx, int B, bool tma, WalkPlan* out) {
   const ts_config& c = ctx->cfg;
-  const size_t rp = (size_t)(c.r + 63) / 64 * 64, slab = rp * 128;
-  const size_t head = rp / 64 * WK_REQ * 128, stage = (size_t)WK_EPI * WK_SLOTS * wk_slot(c.V % 8 == 0), part = (size_t)WK_EPI * WK_REQ * WK_VALS * 4;
-  const size_t fixed = head + stage + part + 64 * 8 + (size_t)((B + ctx->vt_n - 1) / ctx->vt_n) * sizeof(WalkState) + 1024;
-  const size_t avail = (size_t)ctx->max_smem - 10 * 1024;   // static shared memory
+  const size_t rp = (size_t)(c.r + 63) / 64 * 64, slab = (size_t)(c.r + 15) / 16 * 2048;
+  const int ntile = (ctx->vt_TV + 127) / 128;
+  const size_t avail = (size_t)ctx->max_smem - 11 * 1024;   // static shared memory
   const size_t dot = 4 * WK_CHUNK * sizeof(float);
   WalkPlan p{};
-  size_t w = (size_t)(ctx->vt_TV / 64) * slab;
-  if (w + fixed > avail || ctx->vt_TV / 128 >= 32) {
-    if (!tma) return false;
-    p.ring = (int)((avail - (fixed < avail ? fixed : avail)) / (2 * slab));
-    p.ring = p.ring > 8 ? 8 : p.ring;
-    if (p.ring < 2) return false;
-    w = (size_t)p.ring * 2 * slab;
+  p.req = B <= 16 ? 16 : (B <= 32 || ntile > 8 ? 32 : 64);
+  for (;; p.req = 32) {
+    p.tr = ntile <= 4 ? 1 : (ntile <= 8 ? 2 : 3);
+    const int pairs = B <= 2 ? 1 : (B <= 4 ? 2 : 3);
+    const size_t head = rp / 64 * p.req * 128, stage = (size_t)WK_EPI * (p.tr == 1 && c.V % 8 == 0 ? WK_SLOTS : 2 * pairs) * wk_slot(c.V % 8 == 0), part = (size_t)WK_EPI * p.req * WK_VALS * 4;
+    const size_t fixed = head + stage + part + 64 * 8 + (size_t)((B + ctx->vt_n - 1) / ctx->vt_n) * sizeof(WalkState) + 1024;
+    size_t w = (size_t)(ctx->vt_TV / 64) * slab;
+    p.ring = 0;
+    if (w + fixed > avail || ctx->vt_TV / 128 >= 32) {
+      if (p.req == 64) continue;   // (the room of 32 requests may do)
+      if (!tma) return false;
+      p.ring = (int)((avail - (fixed < avail ? fixed : avail)) / (2 * slab));
+      p.ring = p.ring > 8 ? 8 : p.ring;
+      if (p.ring < 2) return false;
+      w = (size_t)p.ring * 2 * slab;
+    }
+    if (w < dot) w = (dot + 1023) & ~(size_t)1023;
+    if (w + fixed > avail) return false;
+    p.oB = (uint32_t)w; p.oT = (uint32_t)(w + head); p.oP = (uint32_t)(p.oT + stage); p.oS = (uint32_t)(p.oP + part); p.smem = w + fixed;
+    p.pairs = pairs;
+    *out = p;
+    return true;
   }
-  if (w < dot) w = (dot + 1023) & ~(size_t)1023;
-  if (w + fixed > avail) return false;
-  p.oB = (uint32_t)w; p.oT = (uint32_t)(w + head); p.oP = (uint32_t)(p.oT + stage); p.oS = (uint32_t)(p.oP + part); p.smem = w + fixed;
-  *out = p;
-  return true;
 }
 
 size_t walk_ws_bytes(const ts_ctx* ctx, int B) {
@@ -933,7 +1075,7 @@ cudaError_t launch_walk_mma(ts_ctx* ctx, WalkArgs& a, char* ws, const WalkPlan& 
   a.edge = (WalkEdge*)ws; ws += align_up(b * n * sizeof(WalkEdge), 256);
   a.rec = (WalkRec*)ws; ws += align_up(b * sizeof(WalkRec), 256);
   a.part = (float*)ws;
-  a.ring = p.ring; a.oB = p.oB; a.oT = p.oT; a.oP = p.oP; a.oS = p.oS;
+  a.ring = p.ring; a.req = p.req; a.tr = p.tr; a.pairs = p.tr == 1 && a.V % 8 == 0 ? 3 : p.pairs; a.oB = p.oB; a.oT = p.oT; a.oP = p.oP; a.oS = p.oS;
   CUtensorMap tm;
   memset(&tm, 0, sizeof(tm));
   if (a.use_tma) memcpy(&tm, ctx->tmapW, sizeof(tm));
