@@ -1532,7 +1532,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
       // (given parents: of their rows, before anything else)
       if (turn == 0 && (d == -2 || (a.score_P == 0 && d + 2 < a.D))) {
         const int h0 = d >= -1 && ncta - a.B >= ncta / 4 ? a.B : 0;
-        const int piece_len = a.piece_len;
+        const int piece_len = (((a.V + a.npiece - 1) / a.npiece) + 7) & ~7;
         uint2* ut = a.utop + (size_t)(d & 1) * a.B * a.npiece;
         if (cta >= h0)
 #pragma unroll 1
@@ -1540,7 +1540,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
             const int x = i / a.npiece;
             if (d >= 0 && __ldcg(a.req_npar + (d & 1) * a.B + x) <= 0) continue;
             const int row = a.score_P > 0 ? a.p_req[x] * a.D + a.p_depth[x] : x * a.D + d + 2;
-            scout_piece(a, row, i % a.npiece * a.piece_step, piece_len, ut + i, lane);
+            scout_piece(a, row, i % a.npiece, piece_len, ut + i, lane);
           }
       }
       if (d + 1 >= a.D && a.score_P == 0) { over = true; break; }
@@ -1705,9 +1705,6 @@ static void fill_args(ts_ctx* ctx, TreeArgs& a, char* base, const TreeWs& w, boo
   a.wait_limit = ctx->wait_limit; a.lost_arrival = (ctx->test_mode & TS_TEST_LOST_ARRIVAL) ? 1 : 0;
 }
 
-// Where no CTA is without a request, every one sweeps after its owner phase and the sweep is in the way: every fourth piece is enough there
-// (any tokens give valid bounds; chain of 128 requests: 11 us a level for all pieces, 4.5 for a quarter, the scans as long as before).
-constexpr int SAMPLE = 4;
 static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream_t st) {
   // Crowded levels (a request with dozens of parents) need room for them in the tree and CTAs to spare.  Expansion, owners
   // alone / sharing (us): K = 16, flat logits, Nmax 96: 331 / 257 for 1 request, 591 / 520 for 8, 1,916 / 1,918 for 64; Nmax
@@ -1721,8 +1718,6 @@ static cudaError_t launch_tree(ts_ctx* ctx, TreeArgs& a, int prof_id, cudaStream
   const TreePlan& p = ctx->tree;
   const bool ring = p.ring_nW > 0 && a.score_P == 0 && !many && a.B >= TX_RING_MIN && a.B <= a.rowsU && u_tensor_map(ctx, a.Uscan, a.Vs, a.B, a.rowsU, &tmU);
   if (ring) { a.nW = p.ring_nW; a.oX = p.ring_oX; a.oU = p.ring_oU; }
-  a.piece_step = 1; a.piece_len = (((a.V + a.npiece - 1) / a.npiece) + 7) & ~7;
-  if (SAMPLE > 1 && !a.ragged && a.score_P == 0 && ctx->num_sms - a.B < ctx->num_sms / 4 && a.npiece >= 32 * SAMPLE) { a.piece_step = SAMPLE; a.npiece = (a.npiece + SAMPLE - 1) / SAMPLE; }
   cudaError_t e;
   { ProfScope ps(ctx, K_INIT, st); e = launch_kernel(tree_init_kernel, 1, 64, 0, st, true, a.barrier, 8 + 2 * (DMAX + 2)); }
   if (e != cudaSuccess) return e;

@@ -51,7 +51,7 @@ struct TreeArgs {
   float *o_lse0, *o_lseT; int* o_top_tok; float* o_top_logit; int* o_draw_tok; float* o_draw_logit;
   // plan
   int wide_u;            // base-logit rows start on 32 bytes
-  int TV, ntiles, BN, nW, npiece, piece_len, piece_step, w_over, use_tma, no_seed, ragged;   // (swept: every piece_step-th piece of piece_len tokens, npiece of them)
+  int TV, ntiles, BN, nW, npiece, w_over, use_tma, no_seed, ragged;
   int tail_copies;       // the last group of a list may hold its rows in copies
   int rowsU;             // requests a stage of the base-logit ring holds
   uint32_t oL, oW, oX, oU;   // byte offsets of the selection state, the W ring, the fixed part and the base-logit ring

@@ -236,12 +236,3 @@ def test_walks_that_reject_every_sibling(over, T):
 @pytest.mark.parametrize("P", [129, 160, 161, 192, 193])
 def test_last_group_of_a_list(P):
     check_scores("bf16", 2048, 8, 8, P, 0.7)
-
-
-def test_sampled_sweep_for_seed_bounds():
-    """From 112 requests on a large vocabulary's rows are swept for seed tokens in part."""
-    wl = parity.small("serve32", dtype="bf16", V=140008, B=112, Nmax=8, K=4, D=3, r=8)
-    rnd = Round(wl, seed=5)
-    ts = make_gpu(wl, rnd.table, max_batch=rnd.B)
-    st = check_round(ts, make_oracle(wl, rnd.table), rnd, 1.0, round_seed=2, reqs=[0, 57, 111])
-    assert st["nodes"] > 3
