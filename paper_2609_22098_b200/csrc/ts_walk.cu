@@ -475,7 +475,7 @@ __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm,
       float zoff[2], qoff[2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        int b;
+        [[maybe_unused]] int b;
         const uint32_t dh = dj + (uint32_t)(h * two) * (uint32_t)sizeof(RedDesc);   // (a lone request stands in for its partner)
         asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=f"(zoff[h]), "=f"(qoff[h]), "=r"(b), "=r"(nC[h]) : "r"(dh + 16u));
         asm volatile("ld.shared.f32 %0, [%1];" : "=f"(c0[h]) : "r"(dh + 32u));
@@ -620,7 +620,7 @@ __device__ __forceinline__ void wk_epilogue4(const WalkArgs& a, const WalkSm& sm
     float p[4], qq[4], zoff[4], qoff[4], c0[4]; int nC[4];
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-      int b;
+      [[maybe_unused]] int b;
       const uint32_t dh = dj + (uint32_t)(h < n ? h : 0) * (uint32_t)sizeof(RedDesc);   // (the first stands in for those that are not there)
       asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=f"(zoff[h]), "=f"(qoff[h]), "=r"(b), "=r"(nC[h]) : "r"(dh + 16u));
       asm volatile("ld.shared.f32 %0, [%1];" : "=f"(c0[h]) : "r"(dh + 32u));
@@ -1041,7 +1041,7 @@ bool walk_plan(const ts_ctx* ctx, int B, bool tma, WalkPlan* out) {
     size_t w = (size_t)(ctx->vt_TV / 64) * slab;
     p.ring = 0;
     if (w + fixed > avail || ctx->vt_TV / 128 >= 32) {
-      if (p.req == 64) continue;   // (the room of 32 requests may do)
+      if (p.req == 64 && (!tma || avail < fixed + 8 * slab || (size_t)(ctx->vt_TV / 64) * slab + fixed - head / 2 - part / 2 <= avail)) continue;   // (the room of 32 requests may do; else W is streamed once for 64)
       if (!tma) return false;
       p.ring = (int)((avail - (fixed < avail ? fixed : avail)) / (2 * slab));
       p.ring = p.ring > 8 ? 8 : p.ring;
