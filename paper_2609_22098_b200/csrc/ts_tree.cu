@@ -1104,10 +1104,11 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
         if (!live(e)) continue;
         const uint64_t k = skey(key_of(e));
         if (sh8 == 56 || (k >> (sh8 + 8)) == (prefix >> (sh8 + 8))) {
-          // (one addition per bin and warp: the first pass, over sign and exponent, has two or three bins for 1,700 keys)
           const int bin = (int)((k >> sh8) & 255u);
-          const unsigned peers = __match_any_sync(__activemask(), bin);
-          if (lane == __ffs(peers) - 1) atomicAdd(&s.hist[bin], __popc(peers));
+          if (MANY) {   // one addition per bin and warp: the first pass, over sign and exponent, has two or three bins for 1,700 keys
+            const unsigned peers = __match_any_sync(__activemask(), bin);
+            if (lane == __ffs(peers) - 1) atomicAdd(&s.hist[bin], __popc(peers));
+          } else atomicAdd(&s.hist[bin], 1);
         }
       }
       __syncthreads();
@@ -1276,7 +1277,10 @@ __device__ __forceinline__ void tx_owner(const TreeArgs& a, unsigned char* sm, c
 }
 
 // Canonical (BFS) renumbering, outputs and ancestor bitmasks of one request, out of shared memory.
+// (MANY: rounds of the counting loop together, 18 us at 256 nodes without; in the forms for small trees it cost the chain of 128 requests 2 %.)
+template <bool MANY>
 __device__ __forceinline__ void tx_finalize(const TreeArgs& a, unsigned char* sm, const int b, const bool timed_out) {
+  constexpr int UNROLL = MANY ? 4 : 1;
   const OwnerSm s = owner_carve(sm, a);
   const int tid = threadIdx.x, N = a.N;
   const size_t pb = (size_t)b * N;
@@ -1298,9 +1302,9 @@ __device__ __forceinline__ void tx_finalize(const TreeArgs& a, unsigned char* sm
     int cr = 0, pr = 0;
     if (have) {
       const int dx = (s.pv.meta[x] >> 8) & 255; const uint64_t px = s.pv.path[x]; const double kx = s.pv.key[x];
-#pragma unroll 4
+#pragma unroll UNROLL
       for (int t = sub; t < N; t += G) {
-        const int mt = s.pv.meta[t], dt = (mt >> 8) & 255;   // (no branches: the loads of four rounds go out together)
+        const int mt = s.pv.meta[t], dt = (mt >> 8) & 255;   // (no branches: the loads of several rounds go out together)
         const uint64_t pt = s.pv.path[t]; const double kt = s.pv.key[t];
         const bool other = t != x && (mt >> 16) != 0, first = dt < dx || (dt == dx && pt < px);
         cr += other && first ? 1 : 0;
@@ -1577,7 +1581,7 @@ __global__ void __launch_bounds__(TX_THREADS, 1) tree_kernel(const __grid_consta
   __syncthreads();
   const bool late = dead || *reinterpret_cast<volatile int*>(a.err) != 0;
   if (a.score_P == 0) {
-    for (int b = cta; b < a.B; b += ncta) tx_finalize(a, base_sm, b, late);
+    for (int b = cta; b < a.B; b += ncta) tx_finalize<MANY>(a, base_sm, b, late);
   } else if (!MANY && !RING && late) {   // given parents: there is no status array to report it in (in the other instantiations
                                          // the code alone cost the chain of 128 requests 20 us of 726)
     for (int p = cta; p < a.score_P; p += ncta) {
