@@ -552,8 +552,10 @@ __device__ __forceinline__ void tx_drain(const TreeArgs& a, const TxSm& sm, cons
   }
 }
 
-// Copies of the rows in group g: the last group of a list may have few parents (a list of 150: its 22 took as long as the 128
-// before them, 26 us).  Not without room for the copies' candidates (a.tail_copies).
+// Copies of the rows in group g.  The copies decide which chunks of the range a partial sum covers, so a parent's sums may have
+// copies only by what is the same on every run.  Lists of one group: their length.  Given parents also by group (the place in the list is
+// the caller's): the last one may hold few (150 parents: its 22 took as long as the 128 before them, 26 us); not without room for
+// the copies' candidates (a.tail_copies).  An expansion's parents come to the list in the order their owners are done.
 __device__ __forceinline__ int group_replicas(const TreeArgs& a, const int P, const int g) { return g == 0 || a.tail_copies ? mma_replicas(P - g * TX_ROWS) : 1; }
 // where the candidates of parent p start
 __device__ __forceinline__ size_t cand_base(const TreeArgs& a, const int P, const int p) {
@@ -1656,8 +1658,8 @@ bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
 
 // Workspace of one call over `nreq` requests (or given parents) whose lists hold up to `cap` parents.
 struct TreeWs { size_t head, ent[2], slot[2], sums, cnt, top, key, lg, thr, utop, pool, state, caps, rlse, rcand, upad, wpad, total; int cap; };
-// the built-in scratch array has no room for them
-static bool tail_copies(bool expand, int rows) { return expand || rows > 0; }
+// given parents whose last group may be held in copies (the built-in scratch array, rows = 0, has no room for them)
+static bool tail_copies(bool expand, int rows) { return !expand && rows > 0; }
 static TreeWs tree_ws(const ts_ctx* ctx, int nreq, int cap, bool expand, int rows) {
   const ts_config& c = ctx->cfg; const TreePlan& p = ctx->tree;
   TreeWs w{}; size_t at = 0;
@@ -1754,7 +1756,7 @@ cudaError_t tree_expand(ts_ctx* ctx, char* ws, const TreeOut& o, const void* U, 
   TreeArgs a{};
   const TreeWs w = tree_ws(ctx, B, B * c.Nmax > B ? B * c.Nmax : B, true, B * c.D);
   fill_args(ctx, a, ws, w, true, U, A, W, T, seed);
-  a.B = B; a.tail_copies = 1; a.anchor = anchor; a.theta = theta; a.calib = ctx->calib; a.calib_qT = (ctx->ablation & TS_ABLATE_CALIB_QT) ? 1 : 0;
+  a.B = B; a.anchor = anchor; a.theta = theta; a.calib = ctx->calib; a.calib_qT = (ctx->ablation & TS_ABLATE_CALIB_QT) ? 1 : 0;
   a.pool = (unsigned char*)ws + w.pool; a.pool_stride = pool_bytes(c.Nmax);
   int* state = (int*)(ws + w.state);
   a.req_npar = state; a.req_base = state + 2 * (size_t)B; a.req_nscored = state + 3 * (size_t)B; a.root_lseT = (float*)(state + 4 * (size_t)B);

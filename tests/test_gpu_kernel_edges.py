@@ -236,3 +236,25 @@ def test_walks_that_reject_every_sibling(over, T):
 @pytest.mark.parametrize("P", [129, 160, 161, 192, 193])
 def test_last_group_of_a_list(P):
     check_scores("bf16", 2048, 8, 8, P, 0.7)
+
+
+def test_expansions_repeat_to_the_last_bit():
+    """A level's list holds its parents in the order in which their owners are done, another one on every run: no sum may
+    depend on the place.  Lists of 129 to 192 parents, whose second group is short, must be among the levels."""
+    wl = parity.small("wide", V=20008, B=40, Nmax=32, K=8, D=5, r=32, dtype="bf16")
+    rnd = Round(wl, seed=77)
+    ts = make_gpu(wl, rnd.table, max_batch=rnd.B)
+    levels, first = set(), None
+    for scale in (1.0, 1.4, 2.0, 2.8, 4.0):
+        rnd.theta.fill_(0.02 * scale)
+        first = None
+        for _ in range(25):
+            t = to_cpu(ts.expand_tree(rnd.U, rnd.A, rnd.W, rnd.anchor, rnd.theta, 1.0, 5))
+            live = torch.arange(wl.Nmax)[None] < t["n_nodes"][:, None]
+            got = [t[k][live].contiguous().view(torch.int32) for k in ("logS", "q0", "logqT", "logkey")] + [t["tok"][live], t["node_lseT"][:, 1:][live].contiguous().view(torch.int32)]
+            if first is None:
+                first = got
+                scored = live & ~torch.isnan(t["node_lseT"][:, 1:])
+                levels |= {int((scored & (t["depth"] == d)).sum()) for d in range(1, wl.D)}
+            assert all(torch.equal(a, b) for a, b in zip(first, got))
+    assert any(128 < n <= 192 for n in levels), levels
