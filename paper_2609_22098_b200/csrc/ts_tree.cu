@@ -44,7 +44,7 @@ __device__ __forceinline__ void load16_bf16(const __nv_bfloat16* p, const bool w
 struct TxSm {
   unsigned char *As, *Ws, *Us;
   unsigned long long* q;       // [TX_QCAP] queued candidates (QEntry)
-  float* lists;                // [128][list_stride(K)]: topv, topi, keyv, keyi, keyl of every row, sorted (value desc, token asc)
+  float* lists;                // [128][lstride]: topv, topi, keyv, keyi, keyl of every row, sorted (value desc, token asc)
   int* ln;                     // [2][128] entries in use
   volatile float* lthr;        // [2][128] K-th best of the row's own list (-inf until it is full)
   volatile float* best;        // [2][TX_SPLIT][128] best value published by the piece (row, split)
@@ -58,8 +58,8 @@ struct TxSm {
   volatile unsigned* q_head; unsigned* q_tail;
 };
 
-// words between two rows' lists: odd, so that the threads of neighbouring rows read different banks
-__host__ __device__ constexpr int list_stride(int K) { return (5 * K) | 1; }
+// words between two rows' lists: no multiple of four, so that at most two of the threads of neighbouring rows read the same bank
+constexpr int list_stride(int K) { return 5 * K + (K % 4 == 0 ? 1 : 0); }
 constexpr size_t tx_select_bytes(int K) {
   return (size_t)TX_QCAP * 8 + (size_t)TX_ROWS * list_stride(K) * 4 + 2 * TX_ROWS * 4 + 2 * TX_ROWS * 4 + 2 * TX_SPLIT * TX_ROWS * 4 + 3 * TX_SPLIT * TX_ROWS * 4;
 }
@@ -70,7 +70,7 @@ __device__ __forceinline__ TxSm tx_carve(unsigned char* sm, const TreeArgs& a) {
   s.As = sm; s.Ws = sm + a.oW; s.Us = sm + a.oU;
   s.q = reinterpret_cast<unsigned long long*>(sm + a.oL);
   s.lists = reinterpret_cast<float*>(s.q + TX_QCAP);
-  s.ln = reinterpret_cast<int*>(s.lists + (size_t)TX_ROWS * list_stride(a.K));
+  s.ln = reinterpret_cast<int*>(s.lists + (size_t)TX_ROWS * a.lstride);
   s.lthr = reinterpret_cast<float*>(s.ln + 2 * TX_ROWS);
   s.best = s.lthr + 2 * TX_ROWS;
   s.part = const_cast<float*>(s.best) + 2 * TX_SPLIT * TX_ROWS;
@@ -159,7 +159,7 @@ __device__ __forceinline__ void tx_select(const TreeArgs& a, const TxSm& sm, con
   const int prow = R > 1 ? row % per : row, rho = R > 1 ? row / per : 0;
   const int p = g * TX_ROWS + prow;
   const int pid = ((tile * TX_SPLIT + s) * R + rho) % K;
-  float* L = sm.lists + (size_t)row * list_stride(K);
+  float* L = sm.lists + (size_t)row * a.lstride;
   if (kind & 1u) {
     if (lg >= sm.thr[prow] && lg >= sm.lthr[row]) {
       sm.lthr[row] = tx_insert(L, reinterpret_cast<int*>(L) + K, nullptr, sm.ln[row], K, lg, tok, 0.f);
@@ -604,7 +604,7 @@ __device__ __forceinline__ void tx_publish(const TreeArgs& a, const TxSm& sm, co
     return;
   }
   const size_t base = cand_base(a, P, p);
-  const float* L = sm.lists + (size_t)row * list_stride(K) + (role == 2 ? 2 * K : 0);
+  const float* L = sm.lists + (size_t)row * a.lstride + (role == 2 ? 2 * K : 0);
   const float bound = sm.thr[(role == 2 ? TX_ROWS : 0) + prow];
   const int n = sm.ln[(role == 2 ? TX_ROWS : 0) + row];
   int k = 0;
@@ -1635,6 +1635,10 @@ bool tree_plan(const ts_config& c, int num_sms, int max_smem, TreePlan* out) {
     auto total = [&](int nw) { return A + sel + fix + (size_t)nw * w; };
     if (total(nW) > avail) continue;
     while (nW < TX_STAGE_MAX && total(nW + 1) <= avail) ++nW;
+    // An even number of blocks of 128: with an odd one the two issuing warps' slots don't alternate (expansion of 32 requests at
+    // V = 64,000: rank 160, K = 14: 267 us with two, 287 with three; rank 128, K = 2: 123 with four, 127 with five).  Blocks of 64
+    // are too short for two stages (rank 256, V = 151,936: 322 with two, 305 with three).
+    if (BN == 128) nW &= ~1;
     p.BN = BN; p.nW = nW;
     p.oL = (uint32_t)A; p.oW = (uint32_t)(p.oL + sel); p.oX = (uint32_t)(p.oW + (size_t)nW * w);
     // owners work in [A, selection state] and, where that is not enough, in the W ring (which then does not run ahead);
@@ -1698,7 +1702,7 @@ static void fill_args(ts_ctx* ctx, TreeArgs& a, char* base, const TreeWs& w, boo
   a.Vs = p.Vs; a.Uscan = a.ragged ? base + w.upad : U; a.Wscan = a.ragged ? base + w.wpad : W;
   a.wide_u = (p.Vs % 16 == 0 && ((uintptr_t)a.Uscan & 31u) == 0) ? 1 : 0;
   a.TV = p.TV; a.ntiles = p.ntiles; a.BN = p.BN; a.nW = p.nW; a.npiece = p.npiece; a.w_over = p.w_over;
-  a.oL = p.oL; a.oW = p.oW; a.oX = p.oX; a.oU = 0; a.rowsU = p.rowsU;
+  a.lstride = list_stride(c.K); a.oL = p.oL; a.oW = p.oW; a.oX = p.oX; a.oU = 0; a.rowsU = p.rowsU;
   for (uint32_t i = 0; i < 10; ++i) { a.rk[2 * i] = (uint32_t)seed + i * 0x9E3779B9u; a.rk[2 * i + 1] = (uint32_t)(seed >> 32) + i * 0xBB67AE85u; }
   a.no_seed = (ctx->test_mode & TS_TEST_NO_SEED) ? 1 : 0;
   int* head = (int*)(base + w.head);

@@ -53,6 +53,7 @@ struct TreeArgs {
   int wide_u;            // base-logit rows start on 32 bytes
   int TV, ntiles, BN, nW, npiece, w_over, use_tma, no_seed, ragged;
   int tail_copies;       // the last group of a list may hold its rows in copies
+  int lstride;           // words between two rows' lists
   int rowsU;             // requests a stage of the base-logit ring holds
   uint32_t oL, oW, oX, oU;   // byte offsets of the selection state, the W ring, the fixed part and the base-logit ring
   uint32_t rk[20];       // round keys of the sampling generator
