@@ -14,9 +14,9 @@
 // When no request asks any more, every owner draws its requests' bonus tokens by itself: the range from the stored
 // range sums, then the token inside it.  Two barriers a step and none at the start and the end.
 //
-// Measured at 32 requests, V = 151,936, r = 64 (one of them rejects eight siblings): 108 us in five steps, 146 in nine with one
-// coefficient a reduction.  A step: sums and advance 3 to 7 (predictions), barriers 1.1 and 1.5, operands 2, the pass 18 (all requests, grid),
-// 12 and 10 (a few, eight coefficients), 3 (one request, one coefficient).  Set-up 6, bonus draws 12.
+// Measured at 32 requests, V = 151,936, r = 64 (several of them reject eight siblings): 106 us in five steps; with one coefficient a
+// reduction it was nine steps and 146.  A step: sums and advance 3 to 7 (predictions), barriers 1.1 and 1.5, operands 2, the pass 18 (all
+// requests, grid), 12 and 10 (a few, eight coefficients), 3 (one request, one coefficient).  Set-up 6, bonus draws 11.
 #include <math.h>
 #include <string.h>
 
@@ -27,17 +27,17 @@ namespace ts {
 constexpr int WK_EPI = 16;                 // warps that read accumulators: 4 lane quarters x 4 sets of tiles
 constexpr int WK_LOAD = WK_EPI;            // tensor memory; in the streaming form it requests W and issues the MMAs
 constexpr int WK_THREADS = (WK_EPI + 1) * 32;
-constexpr int WK_REQ = 64;                 // requests of one reduction pass (columns of a tile) at most: WalkArgs::req of them, 16, 32 or 64
 constexpr int WK_TR = 3;                   // tiles of a set in tensor memory together at most: WalkArgs::tr of them; a round is four sets' (512 columns)
 constexpr int WK_ROUND = 4 * WK_TR;
 constexpr int WK_VALS = 2 * WK_COLS;       // sums of a request: residual and proposal mass at every coefficient
-constexpr int WK_SLOTS = 6;                // requests whose rows a warp has in flight or in work: three pairs
 constexpr int WK_GRID = 16;                // beside the number of coefficients: all but the first are guesses from the grid
 __host__ __device__ constexpr int wk_seg(bool aligned) { return aligned ? 64 : 80; }   // bytes of a staged segment: 32 tokens that, unaligned, may start anywhere in a 16-byte chunk
-__host__ __device__ constexpr int wk_slot(bool aligned) { return 2 * WK_TR * wk_seg(aligned); }
+constexpr int WK_STATIC = 2048;            // static shared memory at most
 constexpr int WK_CHUNK = 1088;             // tokens of one step of the bonus rescan: 8 tokens x 136 places x 4 slices of the rank
+constexpr size_t WK_DOT = 4 * WK_CHUNK * sizeof(float);   // shared memory of the rescan
 constexpr double WK_TOL = 9.5367431640625e-7;   // 2^-20: a coefficient this close (relative) to an evaluated one counts as evaluated
 
+// A request of a pass.  b: its number; rows that may start anywhere: and where in a 16-byte chunk the two do (bits 28, 24).
 struct __align__(16) RedDesc { const __nv_bfloat16 *z, *u; float zoff, qoff; int b, nC; float C[WK_COLS]; };
 static_assert(sizeof(RedDesc) == 64, "four 16-byte loads");
 
@@ -53,7 +53,7 @@ struct WalkState {
 };
 
 struct WalkSm {
-  unsigned char *Ws, *Bs, *stage; float* part; WalkState* st;
+  unsigned char *Ws, *Bs, *stage; float* part; RedDesc* desc; int* tok; WalkState* st;
   uint64_t *t_full, *t_empty, *w_full, *w_free; uint32_t* tmem; volatile int* abort;
 };
 
@@ -330,25 +330,25 @@ __device__ __forceinline__ void wk_mma(const WalkArgs& a, const WalkSm& sm, cons
   tc_fence_after();
   if (elect_one()) {
     const uint64_t ad = smem_desc(smem_u32(sm.Ws) + 2u * ws * slab, slab, 1024u), bd = smem_desc(smem_u32(sm.Bs), 16u, 1024u);
-    const uint32_t idesc = wk_idesc(ncol), d = tmem_base + slot * (uint32_t)a.req;
+    const uint32_t idesc = wk_idesc(ncol), d = tmem_base + slot * (uint32_t)a.cols;
 #pragma unroll 4
     for (int ks = 0; ks < ksteps; ++ks)
-      mma_bf16(d, ad + (uint64_t)(ks * 128), bd + (uint64_t)((ks >> 2) * (a.req * 8) + (ks & 3) * 2), idesc, ks > 0 ? 1u : 0u);
+      mma_bf16(d, ad + (uint64_t)(ks * 128), bd + (uint64_t)((ks >> 2) * (a.cols * 8) + (ks & 3) * 2), idesc, ks > 0 ? 1u : 0u);
     mma_commit(sm.t_full + slot);
     if (a.ring) mma_commit(sm.w_free + ws);
   }
   __syncwarp();
 }
-// a set's accumulators are free for round `rnd` (counted over all passes) when its four warps are done with the round before
-__device__ __forceinline__ bool wk_drained(const WalkArgs& a, const WalkSm& sm, const int set, const uint32_t rnd) {
-  return rnd == 0u || __all_sync(0xFFFFFFFFu, wk_wait(sm.t_empty + set, (rnd - 1u) & 1u, a, sm.abort));
+// the accumulators are free for round `rnd` (counted over all passes) when all warps are done with the round before
+__device__ __forceinline__ bool wk_drained(const WalkArgs& a, const WalkSm& sm, const uint32_t rnd) {
+  return rnd == 0u || __all_sync(0xFFFFFFFFu, wk_wait(sm.t_empty, (rnd - 1u) & 1u, a, sm.abort));
 }
 // Streaming form, one warp: blocks of 128 tokens of W through the ring, one after the other round the range and on into the next
 // pass (W does not depend on which requests that sums), and the tiles in the same order.  (In order, and by one warp: a wait
 // for a parity tells a slot's turns apart only while the waiter follows every one of them.)
 __device__ __forceinline__ void wk_stream(const WalkArgs& a, const WalkSm& sm, const CUtensorMap* tm, const int ncol, const int t0, const int tlen, const uint32_t pass,
-                                          uint32_t& wreq, uint32_t rnd, const uint32_t tmem_base) {
-  const int ntile = (tlen + 127) / 128;
+                                          uint32_t& wreq, uint32_t& rnd, const uint32_t tmem_base) {
+  const int ntile = (tlen + 127) / 128, round = a.sets * a.tr;
   const uint32_t slab = (uint32_t)((a.r + 15) / 16) * 2048u, ring = (uint32_t)a.ring, w0 = pass * (uint32_t)ntile;
   for (int t = 0; t <= ntile; ++t) {
     for (const uint32_t upto = w0 + (uint32_t)t + ring; wreq < upto; ++wreq) {
@@ -363,12 +363,13 @@ __device__ __forceinline__ void wk_stream(const WalkArgs& a, const WalkSm& sm, c
     }
     if (t == ntile) break;
     const uint32_t x = w0 + (uint32_t)t;
-    const int i = t % (4 * a.tr);
+    const int i = t % round;
     if (i == 0 && t > 0) ++rnd;
-    if (i < 4 && !wk_drained(a, sm, i, rnd)) return;
+    if (i == 0 && !wk_drained(a, sm, rnd)) return;
     if (!__all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + x % ring, (x / ring) & 1, a, sm.abort))) return;
     wk_mma(a, sm, ncol, x % ring, (uint32_t)i, tmem_base);
   }
+  ++rnd;
 }
 
 // Sums of N values over the lanes: halve the values while halving the lanes; lane (32 / N) v ends with value v.
@@ -396,95 +397,94 @@ __device__ __forceinline__ bool wk_has(const int nC, const int val) {
   return val < WK_COLS ? val < cols : (cols > 1 && !(nC & WK_GRID) && val - WK_COLS < cols);
 }
 
-// The scanning warps.  A warp holds the accumulators of 32 tokens in each of up to three tiles and goes through the requests;
-// the two rows of a request come through a ring of 16-byte copies, two pairs ahead (AL: rows start on 16 bytes).  A request's chain
-// of waits, loads and exponentials is some 600 cycles, so two requests go through it together, and what does not depend on the request
-// is worked out before the loop.  A pass of 32 requests and one coefficient: 13.8 us; one request at a time 17, with the copies' addresses
-// and sizes worked out for every one 23; two-byte loads by every token's
-// thread, one group of eight requests ahead, took 18 us for 32 and 32 us for 64.
+// The scanning warps.  A warp holds the accumulators of 32 tokens in each of its set's tiles, up to three, and goes through the requests two
+// at a time: a request's chain of waits, loads and exponentials is some 600 cycles, so two go through it together, and what does not depend on
+// the request is worked out before the loop.  Their rows come through shared memory by 16-byte copies (AL: rows start on 16 bytes),
+// requested when the pair before has been read: one and two pairs further ahead cost 12 to 30 KB each and were no faster, the four warps
+// of a scheduler cover for one another.  One request at a time, with the copies' addresses and sizes worked out for every one, a pass of 32 requests
+// and one coefficient took 23 us instead of 14; two-byte loads by every token's thread 18.
+// A request's several coefficients cost a warp a sum over its lanes each, so the tiles are shared by as few sets of four warps as hold them, and
+// the sets that are left take every second or all but every fourth pair instead; with one pair (two pairs) the tiles go to all sets (two).
 template <bool AL>
 __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm, const int nreq, const int ncol, const int t0, const int tlen,
-                                            const uint32_t tmem_base, uint32_t& used, uint32_t& rnd, const bool first_pass, const RedDesc* desc) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = warp & 3, set = warp >> 2;
+                                            const uint32_t tmem_base, uint32_t& used, uint32_t& rnd, const bool first_pass) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = warp & 3, sets = nreq > 4 ? a.sets : (nreq > 2 ? max(a.sets, 2) : 4), set = (warp >> 2) & (sets - 1), part = (warp >> 2) / sets, nparts = 4 / sets;
   const int ntile = (tlen + 127) / 128;
   const float zs = (1.f / a.T) * 1.4426950408889634f;   // exponentials as powers of two
   float* mine = sm.part + (size_t)warp * a.req * WK_VALS;
-  constexpr uint32_t SEG = wk_seg(AL), SLOT = wk_slot(AL);
-  const uint32_t ring = smem_u32(sm.stage) + (uint32_t)warp * (uint32_t)(2 * a.pairs) * SLOT, dbase = smem_u32(desc);
   constexpr int CPS = AL ? 4 : 5;                       // 16-byte copies of a segment
+  constexpr uint32_t SEG = wk_seg(AL);
+  const uint32_t SLOT = 2u * (uint32_t)a.tr * SEG;      // a request's segments
+  const uint32_t dbase = smem_u32(sm.desc), place = smem_u32(sm.stage) + (uint32_t)warp * 2u * SLOT;
   const int seg = lane / CPS, ch = lane - seg * CPS;    // lane's copy of a request: 16 bytes of one segment (tile, row)
   bool alive = true;
-  const int round = 4 * a.tr;
+  const int round = a.sets * a.tr, step = 128 * sets;   // (a round is the plan's, however many sets share it)
   for (int r0 = 0; r0 < ntile; r0 += round, ++rnd) {
-    const int left = min(ntile - r0, round) - set, ntl = left > 0 ? (left + 3) / 4 : 0;   // the set's tiles: r0 + set + 4 i
-    const int tok = (r0 + set) * 128 + q * 32;                                              // the warp's first token in the first of them; then + 512 i
+    const int left = min(ntile - r0, round) - set, ntl = left > 0 ? (left + sets - 1) / sets : 0;   // the set's tiles: r0 + set + sets i
+    const int tok = (r0 + set) * 128 + q * 32;                                              // the warp's first token in the first of them; then + step i
     int nt = 0;                                                                             // its tiles with any token
 #pragma unroll
-    for (int i = 0; i < WK_TR; ++i) if (i < ntl && tok + 512 * i < tlen) nt = i + 1;
-    const bool tail = nt > 0 && tok + 512 * (nt - 1) + 32 > tlen;                           // (uniform) the last of them is cut short
-    const int o = tok + 512 * (seg >> 1), nv = min(32, tlen - o);
+    for (int i = 0; i < WK_TR; ++i) if (i < ntl && tok + step * i < tlen) nt = i + 1;
+    const bool tail = nt > 0 && tok + step * (nt - 1) + 32 > tlen;                          // (uniform) the last of them is cut short
+    const int o = tok + step * (seg >> 1), nv = min(32, tlen - o);
     const bool act = seg < 2 * nt && (!AL || 8 * ch < nv);
-    const uint64_t off = 2ull * (uint64_t)(uint32_t)(t0 + o) + (AL ? 16u * (uint32_t)ch : 0u);
-    const uint32_t from = dbase + (uint32_t)(seg & 1) * 8u, to = ring + (uint32_t)seg * SEG + (uint32_t)ch * 16u;
-    auto stage = [&](int j, uint32_t at) {   // requests j and j + 1 into the places at `at`
+    const uint64_t off = 2ull * (uint64_t)(uint32_t)(t0 + o) + 16u * (uint32_t)ch;
+    const int bytes = 2 * nv - 16 * ch;                                                     // of the segment from the lane's chunk on
+    const uint32_t from = dbase + (uint32_t)(seg & 1) * 8u, to = place + (uint32_t)seg * SEG + (uint32_t)ch * 16u;
+    auto stage = [&](int j) {   // requests j and j + 1
 #pragma unroll
       for (int h = 0; h < 2; ++h)
         if (act && j + h < nreq) {
           uint64_t row;
           asm volatile("ld.shared.u64 %0, [%1];" : "=l"(row) : "r"(from + (uint32_t)(j + h) * (uint32_t)sizeof(RedDesc)));
-          const uint32_t dst = to + at + (uint32_t)h * SLOT;
+          const uint32_t dst = to + (uint32_t)h * SLOT;
           if (AL) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(row + off) : "memory");
-          else {   // 32 tokens that start anywhere: up to five whole chunks, cut at the last token's end
-            const uint64_t x = row + off, src = (x & ~15ull) + 16u * (uint32_t)ch, end = x + 2u * (uint32_t)nv;
-            const int bytes = src < end ? (end - src < 16 ? (int)(end - src) : 16) : 0;
-            if (bytes) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+          else {   // 32 tokens that start anywhere: up to five whole chunks, cut at the last token's end (segments are whole 64 bytes into the row)
+            const int shift = (int)((uint32_t)row & 15u), n = min(16, bytes + shift);
+            if (n > 0) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(row + off - (uint64_t)shift), "r"(n) : "memory");
           }
         }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    stage(0, 0u);
-    stage(2, 2u * SLOT);
-    if (q == 0 && !a.ring) {
-      if (alive) alive = wk_drained(a, sm, set, rnd);
-      for (int i = 0; i < ntl && alive; ++i) {
-        const int t = r0 + set + 4 * i;
+    stage(2 * part);
+    if (q == 0 && !a.ring) {   // (the parts share a set's tiles)
+      if (alive) alive = wk_drained(a, sm, rnd);
+      for (int i = part; i < ntl && alive; i += nparts) {
+        const int t = r0 + set + sets * i;
         if (first_pass && a.use_tma) alive = __all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + t, 0, a, sm.abort));
-        if (alive) wk_mma(a, sm, ncol, (uint32_t)t, (uint32_t)(set + 4 * i), tmem_base);
+        if (alive) wk_mma(a, sm, ncol, (uint32_t)t, (uint32_t)(set + sets * i), tmem_base);
       }
     }
     for (int i = 0; i < ntl; ++i) {
-      const uint32_t slot = (uint32_t)(set + 4 * i);
+      const uint32_t slot = (uint32_t)(set + sets * i);
       if (alive) alive = __all_sync(0xFFFFFFFFu, wk_wait(sm.t_full + slot, (used >> slot) & 1u, a, sm.abort));
-      used ^= 1u << slot;
     }
+    used ^= (1u << min(ntile - r0, round)) - 1u;
     tc_fence_after();
-    const uint32_t tcol = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(set * a.req);
-    uint32_t at = 0u, ahead = 4u * SLOT;   // places of this pair and of the one to be requested
+    const uint32_t tcol = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(set * a.cols);
 #pragma unroll 1
-    for (int j = 0; j < nreq && alive; j += 2) {
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-      __syncwarp();   // the lanes' copies of this pair are all there, and nobody reads the places the next copies go to
-      stage(j + 4, ahead);
+    for (int j = 2 * part; j < nreq && alive; j += 2 * nparts) {
       uint32_t acc[2 * WK_TR];
 #pragma unroll
       for (int i = 0; i < WK_TR; ++i)
-        if (i < nt) asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(acc[2 * i]), "=r"(acc[2 * i + 1]) : "r"(tcol + (uint32_t)(4 * i * a.req + j)) : "memory");
-      float p[2 * WK_TR], qq[2 * WK_TR], c0[2]; int nC[2];
+        if (i < nt) asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(acc[2 * i]), "=r"(acc[2 * i + 1]) : "r"(tcol + (uint32_t)(sets * i * a.cols + j)) : "memory");
+      float p[2 * WK_TR], qq[2 * WK_TR], c0[2]; int b[2], nC[2];
       const int two = j + 1 < nreq ? 1 : 0;
       const uint32_t dj = dbase + (uint32_t)j * (uint32_t)sizeof(RedDesc);
       float zoff[2], qoff[2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        [[maybe_unused]] int b;
         const uint32_t dh = dj + (uint32_t)(h * two) * (uint32_t)sizeof(RedDesc);   // (a lone request stands in for its partner)
-        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=f"(zoff[h]), "=f"(qoff[h]), "=r"(b), "=r"(nC[h]) : "r"(dh + 16u));
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=f"(zoff[h]), "=f"(qoff[h]), "=r"(b[h]), "=r"(nC[h]) : "r"(dh + 16u));
         asm volatile("ld.shared.f32 %0, [%1];" : "=f"(c0[h]) : "r"(dh + 32u));
       }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncwarp();   // the lanes' copies of this pair are all there
       tmem_ld_wait();
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        uint32_t zr = ring + at + (uint32_t)h * SLOT + (uint32_t)lane * 2u, ur = zr + SEG;
-        if (!AL) { zr += (uint32_t)(uintptr_t)desc[j + h * two].z & 15u; ur += (uint32_t)(uintptr_t)desc[j + h * two].u & 15u; }
+        uint32_t zr = place + (uint32_t)h * SLOT + (uint32_t)lane * 2u, ur = zr + SEG;
+        if (!AL) { zr += (uint32_t)b[h] >> 28; ur += ((uint32_t)b[h] >> 24) & 15u; }
 #pragma unroll
         for (int i = 0; i < WK_TR; ++i) {
           const int e = h * WK_TR + i;
@@ -498,11 +498,11 @@ __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm,
           }
         }
       }
-      at = ahead == 4u * SLOT ? 2u * SLOT : (ahead == 0u ? 4u * SLOT : 0u);
-      ahead = ahead == 4u * SLOT ? 0u : ahead + 2u * SLOT;
+      __syncwarp();   // nobody reads this pair's places any more
+      stage(j + 2 * nparts);
       if (tail) {
 #pragma unroll
-        for (int e = 0; e < 2 * WK_TR; ++e) if (tok + 512 * (e % WK_TR) + lane >= tlen) { p[e] = 0.f; qq[e] = 0.f; }   // (the accumulator may hold anything)
+        for (int e = 0; e < 2 * WK_TR; ++e) if (tok + step * (e % WK_TR) + lane >= tlen) { p[e] = 0.f; qq[e] = 0.f; }   // (the accumulator may hold anything)
       }
       float* to_part = mine + j * WK_VALS;
       if (nC[0] == 1 && nC[1] == 1) {
@@ -567,121 +567,8 @@ __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm,
     asm volatile("cp.async.wait_all;" ::: "memory");
     tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive(sm.t_empty + set);
+    if (lane == 0) mbar_arrive(sm.t_empty);
   }
-}
-
-// The same for ranges of up to four tiles (a set has one: V to 75,776 on 148 SMs) and aligned rows: four requests at a time, whose copies are one
-// instruction of the warp.  (Pairs: 104 us of verification for the chain of 100 requests at V = 64,000.)
-__device__ __forceinline__ void wk_epilogue4(const WalkArgs& a, const WalkSm& sm, const int nreq, const int ncol, const int t0, const int tlen,
-                                             const uint32_t tmem_base, uint32_t& used, uint32_t& rnd, const bool first_pass, const RedDesc* desc) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = warp & 3, set = warp >> 2;
-  const int ntile = (tlen + 127) / 128, tok = set * 128 + q * 32;
-  const float zs = (1.f / a.T) * 1.4426950408889634f;   // exponentials as powers of two
-  float* mine = sm.part + (size_t)warp * a.req * WK_VALS;
-  constexpr uint32_t GROUP = 8u * 64u;                  // four requests' two segments
-  const uint32_t ring = smem_u32(sm.stage) + (uint32_t)warp * (WK_SLOTS * (uint32_t)wk_slot(true)), dbase = smem_u32(desc);
-  const int ch = lane & 3, mine4 = lane >> 3;           // lane's copy: 16 bytes of the target or base segment of one of the four
-  const bool has = set < ntile, any = has && tok < tlen, act = any && tok + 8 * ch < tlen, tail = any && tok + 32 > tlen;
-  const uint64_t off = 2ull * (uint64_t)(uint32_t)(t0 + tok) + 16u * (uint32_t)ch;
-  const uint32_t from = dbase + (uint32_t)mine4 * (uint32_t)sizeof(RedDesc) + (uint32_t)((lane >> 2) & 1) * 8u, to = ring + (uint32_t)(lane >> 2) * 64u + (uint32_t)ch * 16u;
-  bool alive = true;
-  auto stage = [&](int j, uint32_t at) {
-    if (act && j + mine4 < nreq) {
-      uint64_t row;
-      asm volatile("ld.shared.u64 %0, [%1];" : "=l"(row) : "r"(from + (uint32_t)j * (uint32_t)sizeof(RedDesc)));
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + at), "l"(row + off) : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  stage(0, 0u);
-  stage(4, GROUP);
-  if (q == 0 && !a.ring) {
-    alive = wk_drained(a, sm, set, rnd);
-    if (has && alive && first_pass && a.use_tma) alive = __all_sync(0xFFFFFFFFu, wk_wait(sm.w_full + set, 0, a, sm.abort));
-    if (has && alive) wk_mma(a, sm, ncol, (uint32_t)set, (uint32_t)set, tmem_base);
-  }
-  if (has) {
-    if (alive) alive = __all_sync(0xFFFFFFFFu, wk_wait(sm.t_full + set, (used >> set) & 1u, a, sm.abort));
-    used ^= 1u << set;
-  }
-  tc_fence_after();
-  const uint32_t tcol = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(set * a.req);
-  uint32_t at = 0u, ahead = 2u * GROUP;
-#pragma unroll 1
-  for (int j = 0; j < nreq && alive; j += 4) {
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncwarp();
-    stage(j + 8, ahead);
-    uint32_t acc[4] = {0u, 0u, 0u, 0u};
-    if (any) asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(acc[0]), "=r"(acc[1]), "=r"(acc[2]), "=r"(acc[3]) : "r"(tcol + (uint32_t)j) : "memory");
-    const int n = min(4, nreq - j);
-    const uint32_t dj = dbase + (uint32_t)j * (uint32_t)sizeof(RedDesc);
-    float p[4], qq[4], zoff[4], qoff[4], c0[4]; int nC[4];
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      [[maybe_unused]] int b;
-      const uint32_t dh = dj + (uint32_t)(h < n ? h : 0) * (uint32_t)sizeof(RedDesc);   // (the first stands in for those that are not there)
-      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=f"(zoff[h]), "=f"(qoff[h]), "=r"(b), "=r"(nC[h]) : "r"(dh + 16u));
-      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(c0[h]) : "r"(dh + 32u));
-    }
-    tmem_ld_wait();
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      p[h] = qq[h] = 0.f;
-      if (any && h < n) {
-        uint32_t z, u;
-        const uint32_t zr = ring + at + (uint32_t)h * 128u + (uint32_t)lane * 2u;
-        asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(z) : "r"(zr));
-        asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(u) : "r"(zr + 64u));
-        p[h] = ex2_approx(fmaf(__uint_as_float(z << 16), zs, zoff[h]));
-        qq[h] = ex2_approx(fmaf(__uint_as_float(acc[h]) + __uint_as_float(u << 16), zs, qoff[h]));
-        if (tail && tok + lane >= tlen) { p[h] = 0.f; qq[h] = 0.f; }
-      }
-    }
-    at = at == 2u * GROUP ? 0u : at + GROUP;
-    ahead = ahead == 2u * GROUP ? 0u : ahead + GROUP;
-    float* to_part = mine + j * WK_VALS;
-    if (nC[0] == 1 && nC[1] == 1 && nC[2] == 1 && nC[3] == 1) {
-      float x[4];
-#pragma unroll
-      for (int h = 0; h < 4; ++h) x[h] = fmaxf(fmaf(-c0[h], qq[h], p[h]), 0.f);
-      const float v = wk_fold<4>(x, lane);
-      if ((lane & 7) == 0 && mine4 < n) to_part[mine4 * WK_VALS] = v;
-      continue;
-    }
-#pragma unroll 1
-    for (int h = 0; h < n; ++h, to_part += WK_VALS) {
-      const float ph = h == 0 ? p[0] : (h == 1 ? p[1] : (h == 2 ? p[2] : p[3])), qh = h == 0 ? qq[0] : (h == 1 ? qq[1] : (h == 2 ? qq[2] : qq[3]));
-      const int cols = h == 0 ? nC[0] : (h == 1 ? nC[1] : (h == 2 ? nC[2] : nC[3]));
-      float c[WK_COLS];
-      const uint32_t dc = dj + (uint32_t)h * (uint32_t)sizeof(RedDesc) + 32u;
-      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3]) : "r"(dc));
-      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(c[4]), "=f"(c[5]), "=f"(c[6]), "=f"(c[7]) : "r"(dc + 16u));
-      if (cols == 1 || (cols & WK_GRID)) {
-        float x[WK_COLS];
-        x[0] = fmaxf(fmaf(-c[0], qh, ph), 0.f);
-#pragma unroll
-        for (int k = 1; k < WK_COLS; ++k) x[k] = fabsf(fmaf(-c[k], qh, ph));
-        const float v = wk_fold<WK_COLS>(x, lane);
-        if ((lane & 3) == 0) to_part[lane >> 2] = v;
-      } else {
-        float x[WK_VALS];
-#pragma unroll
-        for (int k = 0; k < WK_COLS; ++k) {
-          const float t = fmaf(-c[k], qh, ph);
-          x[k] = fmaxf(t, 0.f); x[WK_COLS + k] = t > 0.f ? qh : 0.f;
-        }
-        const float v = wk_fold<WK_VALS>(x, lane);
-        if ((lane & 1) == 0) to_part[lane >> 1] = v;
-      }
-    }
-  }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  tc_fence_before();
-  __syncwarp();
-  if (lane == 0) mbar_arrive(sm.t_empty + set);
-  ++rnd;
 }
 
 // ---- the bonus token of one request whose walk is over, by the CTA that owns it ----------------------------------------------
@@ -834,9 +721,7 @@ __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st,
 template <bool AL>
 __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_constant__ WalkArgs a, const __grid_constant__ CUtensorMap tmW) {
   extern __shared__ __align__(16) unsigned char raw[];
-  __shared__ RedDesc s_desc[WK_REQ];
-  __shared__ int s_tok[WK_REQ], s_par[256], s_kid[256], s_cnt[WK_EPI + 1];
-  __shared__ float2 s_z[257];   // (maximum, log-sum-exp) of a request's rows
+  __shared__ int s_cnt[WK_EPI + 1];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = (int)blockIdx.x, ncta = (int)gridDim.x;
   const int rp = (a.r + 63) / 64 * 64, rw = (a.r + 15) / 16 * 16, t0 = cta * a.vt_TV, tlen = min(a.vt_TV, a.V - t0), ntile = (tlen + 127) / 128;
   const uint32_t slab = (uint32_t)rw * 128u;
@@ -846,14 +731,14 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + a.oS);
   sm.t_full = bars; sm.t_empty = bars + WK_ROUND; sm.w_full = bars + WK_ROUND + 4; sm.w_free = sm.w_full + 32;
   sm.tmem = reinterpret_cast<uint32_t*>(sm.w_free + 8); sm.abort = reinterpret_cast<volatile int*>(sm.tmem + 1);
-  sm.st = reinterpret_cast<WalkState*>(bars + 64);
+  sm.desc = reinterpret_cast<RedDesc*>(bars + 64); sm.tok = reinterpret_cast<int*>(sm.desc + a.req); sm.st = reinterpret_cast<WalkState*>(sm.tok + a.req);
   if (warp == WK_LOAD) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(sm.tmem)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
     for (int i = 0; i < WK_ROUND; ++i) mbar_init(sm.t_full + i, 1);
-    for (int i = 0; i < 4; ++i) mbar_init(sm.t_empty + i, 4);
+    mbar_init(sm.t_empty, WK_EPI);
     for (int i = 0; i < (a.ring ? a.ring : ntile); ++i) mbar_init(sm.w_full + i, 1);
     for (int i = 0; i < a.ring; ++i) mbar_init(sm.w_free + i, 1);
     *sm.abort = 0;
@@ -881,7 +766,7 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
       *reinterpret_cast<uint4*>(sm.Ws + (size_t)sl * slab + k * 128 + ((j ^ (k & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
-  for (int i = tid; i < rp / 64 * a.req * 8; i += WK_THREADS) reinterpret_cast<uint4*>(sm.Bs)[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = tid; i < rp / 64 * a.cols * 8; i += WK_THREADS) reinterpret_cast<uint4*>(sm.Bs)[i] = make_uint4(0u, 0u, 0u, 0u);
   fence_async_smem();
   tc_fence_before();
   __syncthreads();
@@ -891,7 +776,10 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
   pdl_launch_dependents();
 
   const int nown = a.B > cta ? (a.B - cta + ncta - 1) / ncta : 0;   // requests cta, cta + ncta, ...
-  for (int i = 0; i < nown; ++i) wk_setup(a, sm.st[i], cta + i * ncta, s_par, s_kid, s_z);
+  {   // (parents, tokens, and maximum and log-sum-exp of a request's rows, where the passes put their sums later)
+    float2* z = reinterpret_cast<float2*>(sm.part); int* par = reinterpret_cast<int*>(z + 257);
+    for (int i = 0; i < nown; ++i) wk_setup(a, sm.st[i], cta + i * ncta, par, par + 256, z);
+  }
   unsigned gen = 0;
   const unsigned nexpect = (unsigned)ncta + (a.lost_arrival ? 1u : 0u);
   bool dead = false, finished = false;
@@ -943,9 +831,11 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
           d.z = a.Z + zrow * a.V; d.u = __uint_as_float(r2.x) != 0.f ? a.U + (size_t)(int)r0.z * a.V : d.z;   // (no proposal in the sum: its base row is not touched)
           d.zoff = __uint_as_float(r1.x); d.qoff = __uint_as_float(r2.x) != 0.f ? __uint_as_float(r1.y) : -1e30f;   // (lseT may be NaN where it is not needed)
           d.b = b; d.nC = (int)r4.x;
-          s_desc[at].z = d.z; s_desc[at].u = d.u; s_desc[at].zoff = d.zoff; s_desc[at].qoff = d.qoff; s_desc[at].b = d.b; s_desc[at].nC = d.nC;
-          reinterpret_cast<uint4*>(s_desc[at].C)[0] = r2; reinterpret_cast<uint4*>(s_desc[at].C)[1] = r3;
-          s_tok[at] = (int)r0.w;
+          if (!AL) d.b |= (int)(((uint32_t)(uintptr_t)d.z & 15u) << 28 | ((uint32_t)(uintptr_t)d.u & 15u) << 24);   // (where in a 16-byte chunk the rows start)
+          RedDesc& o = sm.desc[at];
+          o.z = d.z; o.u = d.u; o.zoff = d.zoff; o.qoff = d.qoff; o.b = d.b; o.nC = d.nC;
+          reinterpret_cast<uint4*>(o.C)[0] = r2; reinterpret_cast<uint4*>(o.C)[1] = r3;
+          sm.tok[at] = (int)r0.w;
         }
         __syncthreads();
       }
@@ -954,12 +844,12 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
       // head rows of the requests' nodes: the B operand, K-major with the 128-byte swizzle
       for (int idx = tid; idx < nreq * (a.r / 8); idx += WK_THREADS) {
         const int g = idx / (a.r / 8), ck = idx - g * (a.r / 8);
-        *reinterpret_cast<uint4*>(sm.Bs + (ck >> 3) * (a.req * 128) + g * 128 + (((ck & 7) ^ (g & 7)) << 4)) =
-            __ldg(reinterpret_cast<const uint4*>(a.A + (size_t)s_tok[g] * a.r + ck * 8));
+        *reinterpret_cast<uint4*>(sm.Bs + (ck >> 3) * (a.cols * 128) + g * 128 + (((ck & 7) ^ (g & 7)) << 4)) =
+            __ldg(reinterpret_cast<const uint4*>(a.A + (size_t)sm.tok[g] * a.r + ck * 8));
       }
       // ask L2 for this range of the rows that will be read
       for (int x = warp; x < 2 * nreq; x += WK_THREADS / 32) {
-        const RedDesc& d = s_desc[x >> 1];
+        const RedDesc& d = sm.desc[x >> 1];
         const __nv_bfloat16* src = ((x & 1) ? d.u : d.z) + t0;
         if (!(x & 1) || d.u != d.z)
           for (int l = lane * 64; l < tlen; l += 32 * 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + l));
@@ -968,22 +858,22 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
-      if (AL && a.tr == 1) { if (warp < WK_EPI) wk_epilogue4(a, sm, nreq, ncol, t0, tlen, tmem_base, used, rnd, pass == 0u, s_desc); }
-      else if (warp < WK_EPI) wk_epilogue<AL>(a, sm, nreq, ncol, t0, tlen, tmem_base, used, rnd, pass == 0u, s_desc);
-      if (warp == WK_LOAD && a.ring) wk_stream(a, sm, &tmW, ncol, t0, tlen, pass, wreq, pass * (uint32_t)((ntile + 4 * a.tr - 1) / (4 * a.tr)), tmem_base);
+      if (warp < WK_EPI) wk_epilogue<AL>(a, sm, nreq, ncol, t0, tlen, tmem_base, used, rnd, pass == 0u);
+      if (warp == WK_LOAD && a.ring) wk_stream(a, sm, &tmW, ncol, t0, tlen, pass, wreq, rnd, tmem_base);
       ++pass;
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
       if (*sm.abort) { dead = true; break; }
       for (int x = tid; x < nreq * WK_VALS; x += WK_THREADS) {
-        const RedDesc& d = s_desc[x / WK_VALS];
+        const RedDesc& d = sm.desc[x / WK_VALS];
         const int val = x % WK_VALS;
         if (wk_has(d.nC, val)) {
+          const int sets = nreq > 4 ? a.sets : (nreq > 2 ? max(a.sets, 2) : 4), nw = 4 * sets, w0 = ((x / WK_VALS) >> 1) % (4 / sets) * nw;   // the warps that had the request
           float s = 0.f;
 #pragma unroll
-          for (int w = 0; w < WK_EPI; ++w) s += sm.part[w * a.req * WK_VALS + x];
-          a.part[((size_t)d.b * WK_VALS + val) * a.vt_n + cta] = s;
+          for (int w = 0; w < WK_EPI; ++w) s += w < nw ? sm.part[(w0 + w) * a.req * WK_VALS + x] : 0.f;
+          a.part[((size_t)(d.b & 0xFFFFFF) * WK_VALS + val) * a.vt_n + cta] = s;
         }
       }
       __syncthreads();
@@ -1020,41 +910,60 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
 // ------------------------------------------------------------------------------------------------
 // Host side
 // ------------------------------------------------------------------------------------------------
-// Shared-memory plan: the range of W resident where it fits, else a ring of 128-token blocks (that needs the tensor map).
-// Requests a pass takes and tiles a set holds: 64 requests where a range has eight tiles at most (the columns of eight tiles are all of tensor
-// memory), else 32 and three tiles; fewer where the batch has fewer, so that W stays resident in more of shared memory.  (32 for all: the
-// chain of 100 requests at V = 64,000 took 104 us to verify instead of 85 before several coefficients; room for 32 always: one request at
-// V = 200,008 streamed W and took 48 us instead of 41.)
-bool walk_plan(const ts_ctx* ctx, int B, bool tma, WalkPlan* out) {
+// What a plan takes of shared memory; false: too much, or more accumulators than tensor memory has.
+static bool walk_fit(const ts_ctx* ctx, int B, int req, int sets, int tr, bool stream, WalkPlan* out) {
   const ts_config& c = ctx->cfg;
-  const size_t rp = (size_t)(c.r + 63) / 64 * 64, slab = (size_t)(c.r + 15) / 16 * 2048;
   const int ntile = (ctx->vt_TV + 127) / 128;
-  const size_t avail = (size_t)ctx->max_smem - 11 * 1024;   // static shared memory
-  const size_t dot = 4 * WK_CHUNK * sizeof(float);
   WalkPlan p{};
-  p.req = B <= 16 ? 16 : (B <= 32 || ntile > 8 ? 32 : 64);
-  for (;; p.req = 32) {
-    p.tr = ntile <= 4 ? 1 : (ntile <= 8 ? 2 : 3);
-    const int pairs = B <= 2 ? 1 : (B <= 4 ? 2 : 3);
-    const size_t head = rp / 64 * p.req * 128, stage = (size_t)WK_EPI * (p.tr == 1 && c.V % 8 == 0 ? WK_SLOTS : 2 * pairs) * wk_slot(c.V % 8 == 0), part = (size_t)WK_EPI * p.req * WK_VALS * 4;
-    const size_t fixed = head + stage + part + 64 * 8 + (size_t)((B + ctx->vt_n - 1) / ctx->vt_n) * sizeof(WalkState) + 1024;
-    size_t w = (size_t)(ctx->vt_TV / 64) * slab;
-    p.ring = 0;
-    if (w + fixed > avail || ctx->vt_TV / 128 >= 32) {
-      if (p.req == 64 && (!tma || avail < fixed + 8 * slab || (size_t)(ctx->vt_TV / 64) * slab + fixed - head / 2 - part / 2 <= avail)) continue;   // (the room of 32 requests may do; else W is streamed once for 64)
-      if (!tma) return false;
-      p.ring = (int)((avail - (fixed < avail ? fixed : avail)) / (2 * slab));
-      p.ring = p.ring > 8 ? 8 : p.ring;
-      if (p.ring < 2) return false;
-      w = (size_t)p.ring * 2 * slab;
+  p.req = req; p.cols = req < 16 ? 16 : req; p.tr = tr; p.sets = sets;
+  if (sets * tr * p.cols > 512) return false;
+  const size_t slab = (size_t)(c.r + 15) / 16 * 2048, avail = (size_t)ctx->max_smem - WK_STATIC;
+  const size_t head = (size_t)((c.r + 63) / 64) * p.cols * 128, stage = (size_t)WK_EPI * tr * 4 * wk_seg(c.V % 8 == 0);
+  const size_t part = (size_t)WK_EPI * req * WK_VALS * 4, states = (size_t)((B + ctx->vt_n - 1) / ctx->vt_n) * sizeof(WalkState);
+  const size_t fixed = head + stage + part + 64 * 8 + (size_t)req * (sizeof(RedDesc) + 4) + states + 1024;
+  if (fixed > avail) return false;
+  size_t w = (size_t)(ctx->vt_TV / 64) * slab;
+  const size_t tiles = (size_t)ntile * 2 * slab + 1024;   // (the MMAs of a last tile of 64 tokens read the slab behind it too)
+  if (stream) {
+    p.ring = (int)((avail - fixed) / (2 * slab));
+    p.ring = p.ring > 8 ? 8 : p.ring;
+    if (p.ring < 2) return false;
+    w = (size_t)p.ring * 2 * slab;
+  } else if (ctx->vt_TV / 128 >= 32) return false;   // (barriers)
+  if (w < WK_DOT) w = (WK_DOT + 1023) & ~(size_t)1023;   // (where the bonus draws work)
+  p.smem = w + fixed;
+  if (!stream && p.smem < tiles) p.smem = tiles;
+  if (p.smem > avail) return false;
+  p.oB = (uint32_t)w; p.oT = (uint32_t)(w + head); p.oP = (uint32_t)(p.oT + stage); p.oS = (uint32_t)(p.oP + part);
+  *out = p;
+  return true;
+}
+
+// Shared-memory plan.  (Verification, us, prepared rounds of the given batch; "before": the plan that went from 64 requests to 32 and then gave W up.)
+//   Tiles.  As few sets of warps as hold them: what several coefficients cost is a sum over the lanes per request, set and quarter.
+//     V = 50,257, 128 requests: 190 to 205 (three tiles in one set), 235 to 260 (in three); V = 100,000: 225 to 257, before 265 to 315.
+//   W resident before W streamed, passes of fewer requests (not fewer tiles) where that takes room: V = 200,064, r = 64, 32 requests:
+//     172 and 158 (16 a pass), 214 and 204 (32, a third of the tiles), 192 and 181 (32, streamed).  Eight a pass pay up to 32 requests (V = 230,000: 32:
+//     220 and 214 against 230 and 223 streamed; 48: 295 and 320 against 272 and 315).
+//   Streamed passes take 64 requests only if that costs no round of tiles more: r = 96, V = 151,936, 48 requests: 221 and 234 by 32, 245 and 259 by 64.
+//   Without a tensor map (rows that are not whole 16 bytes) W has to be resident, whatever becomes of the rest: else the walk runs on fused
+//     multiply-adds.  V = 151,643, r = 64, 32 requests: 161 and 166, without a plan 735 and 717; the last size, V = 230,003: 314 and 257.
+bool walk_plan(const ts_ctx* ctx, int B, bool tma, WalkPlan* out) {
+  const int ntile = (ctx->vt_TV + 127) / 128, sets = ntile <= WK_TR ? 1 : (ntile <= 2 * WK_TR ? 2 : 4), full = ntile <= sets * WK_TR ? (ntile + sets - 1) / sets : WK_TR;
+  const int most = B <= 16 ? 16 : (B <= 32 || (ntile + 7) / 8 != (ntile + 11) / 12 ? 32 : 64);
+  auto tiles = [&](int req) { return sets * full * req > 512 ? 512 / (sets * req) : full; };
+  for (int req = most; req >= 8; req /= 2)
+    if ((req > 8 || B <= 32 || !tma) && walk_fit(ctx, B, req, sets, tiles(req), false, out)) return true;
+  if (!tma || B <= 8)
+    for (int n = sets, tr = full;;) {
+      if (n < 4) { n *= 2; tr = (ntile + n - 1) / n; } else --tr;
+      if (tr < 1) break;
+      if (walk_fit(ctx, B, 8, n, tr, false, out)) return true;
     }
-    if (w < dot) w = (dot + 1023) & ~(size_t)1023;
-    if (w + fixed > avail) return false;
-    p.oB = (uint32_t)w; p.oT = (uint32_t)(w + head); p.oP = (uint32_t)(p.oT + stage); p.oS = (uint32_t)(p.oP + part); p.smem = w + fixed;
-    p.pairs = pairs;
-    *out = p;
-    return true;
-  }
+  if (tma)
+    for (int req = most; req >= 8; req /= 2)
+      if (walk_fit(ctx, B, req, sets, tiles(req), true, out)) return true;
+  return false;
 }
 
 size_t walk_ws_bytes(const ts_ctx* ctx, int B) {
@@ -1064,6 +973,12 @@ size_t walk_ws_bytes(const ts_ctx* ctx, int B) {
 }
 
 cudaError_t walk_setup(ts_ctx* ctx) {
+  cudaFuncAttributes fa;
+  for (const void* fn : {(const void*)walk_mma_kernel<true>, (const void*)walk_mma_kernel<false>}) {
+    cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+    if (e == cudaSuccess && fa.sharedSizeBytes > WK_STATIC) e = cudaErrorInvalidConfiguration;   // (the plan counts on no more)
+    if (e != cudaSuccess) return e;
+  }
   const cudaError_t e = allow_all_smem(walk_mma_kernel<true>, ctx->max_smem);
   return e != cudaSuccess ? e : allow_all_smem(walk_mma_kernel<false>, ctx->max_smem);
 }
@@ -1075,7 +990,7 @@ cudaError_t launch_walk_mma(ts_ctx* ctx, WalkArgs& a, char* ws, const WalkPlan& 
   a.edge = (WalkEdge*)ws; ws += align_up(b * n * sizeof(WalkEdge), 256);
   a.rec = (WalkRec*)ws; ws += align_up(b * sizeof(WalkRec), 256);
   a.part = (float*)ws;
-  a.ring = p.ring; a.req = p.req; a.tr = p.tr; a.pairs = p.tr == 1 && a.V % 8 == 0 ? 3 : p.pairs; a.oB = p.oB; a.oT = p.oT; a.oP = p.oP; a.oS = p.oS;
+  a.ring = p.ring; a.req = p.req; a.cols = p.cols; a.tr = p.tr; a.sets = p.sets; a.oB = p.oB; a.oT = p.oT; a.oP = p.oP; a.oS = p.oS;
   CUtensorMap tm;
   memset(&tm, 0, sizeof(tm));
   if (a.use_tma) memcpy(&tm, ctx->tmapW, sizeof(tm));

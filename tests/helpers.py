@@ -72,3 +72,22 @@ def sigmoid(x):
 
 def logit(q):
     return math.log(q) - math.log1p(-q)
+
+
+# (vocabulary, rank, batch) of walks -> is W streamed, requests a pass, sets of warps that share a range's tiles, tiles of a set together
+# (148 SMs): one of every form that the walk's shared-memory plan can take
+WALK_SHAPES = {
+    (4104, 64, 97): (0, 64, 1, 1),      # one tile, passes of 64 and 33
+    (2501, 16, 70): (0, 64, 1, 1),      # ragged rows, passes of 64 and 6
+    (50257, 32, 9): (0, 16, 1, 3),      # three tiles in one set, ragged rows
+    (64008, 32, 20): (0, 32, 2, 2),     # four tiles in two sets
+    (100000, 64, 70): (0, 64, 2, 3),    # six, passes of 64 and 6
+    (128256, 64, 36): (0, 64, 4, 2),    # seven: all of tensor memory
+    (128256, 128, 70): (1, 64, 4, 2),   # the same streamed, passes of 64 and 6
+    (151936, 96, 40): (1, 32, 4, 3),    # nine, streamed, passes of 32 and 8
+    (151643, 64, 24): (0, 32, 4, 3),    # ragged rows
+    (100277, 128, 20): (0, 16, 2, 3),   # ragged rows, passes of 16 and 4
+    (113001, 128, 12): (0, 8, 2, 3),    # ragged rows, passes of 8 and 4
+    (45000, 256, 20): (0, 32, 1, 3),    # an odd number of half tiles at the largest rank
+    (230003, 64, 10): (0, 8, 4, 2),     # thirteen tiles, two rounds, ragged rows, passes of 8 and 2
+}

@@ -6,6 +6,7 @@ import torch
 import oracle
 import test_gpu_parity as parity
 from gpu_harness import Round, check_round, close, make_gpu, make_oracle, to_cpu
+from helpers import WALK_SHAPES
 from paper_2609_22098_b200 import binding
 from paper_2609_22098_b200.binding import TreeSpark
 
@@ -199,7 +200,7 @@ class HardRound(Round):
 
 
 @pytest.mark.parametrize("over,T", [
-    (dict(V=4104, B=33, Nmax=24, K=8, D=3, r=64), 1.0),       # more requests than one pass holds, a partial second one
+    (dict(V=4104, B=33, Nmax=24, K=8, D=3, r=64), 1.0),       # an odd number of requests, one tile for four sets of warps
     (dict(V=3001, B=3, Nmax=40, K=16, D=3, r=16), 0.7),       # sixteen rejections: more coefficients than one reduction evaluates; ragged rows
     (dict(V=3003, B=2, Nmax=8, K=2, D=3, r=8), 1.3),          # two children
     (dict(V=60008, B=2, Nmax=24, K=8, D=3, r=256), 1.0),      # W through the ring
@@ -208,11 +209,15 @@ class HardRound(Round):
 def test_walks_that_reject_every_sibling(over, T):
     """The residual masses after several rejections come from one reduction at guessed coefficients: the walk has to be the
     oracle's, sibling by sibling, and it has to count the sums that it needed."""
+    check_hard_walks(over, T)
+
+
+def check_hard_walks(over, T, reqs=None):
     wl = parity.small("wide", dtype="bf16", **over)
     rnd = HardRound(wl, seed=over["V"])
     rnd.theta.fill_(0.01)
     ts = make_gpu(wl, rnd.table, max_batch=rnd.B)
-    st = check_round(ts, make_oracle(wl, rnd.table), rnd, T, round_seed=4)
+    st = check_round(ts, make_oracle(wl, rnd.table), rnd, T, round_seed=4, reqs=reqs)
     assert st["walks_exempt"] <= 0.1 * st["walks"] + 1
     tree = ts.expand_tree(rnd.U, rnd.A, rnd.W, rnd.anchor, rnd.theta, T, 4)
     Z, off = rnd.target_logits(tree)
@@ -230,6 +235,14 @@ def test_walks_that_reject_every_sibling(over, T):
         want += max(len(kids.get(cur, [])), 1)
         assert int(sums[b]) == want
     assert int(sums.max()) >= wl.K   # the case was reached
+
+
+@pytest.mark.parametrize("V,r,B", list(WALK_SHAPES))
+def test_every_form_of_the_walk_under_hard_targets(V, r, B):
+    """A sample of the requests against the oracle, the ends of every pass among them; the sums of all."""
+    size = WALK_SHAPES[V, r, B][1]
+    ends = {b for k in range(0, B, size) for b in (k, min(k + size, B) - 1)} | {B // 2}
+    check_hard_walks(dict(V=V, r=r, B=B, Nmax=12, K=8, D=3), 0.9, sorted(ends))
 
 
 # several groups of 128 parents whose last is held once, twice or four times over
