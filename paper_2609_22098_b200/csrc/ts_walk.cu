@@ -200,14 +200,14 @@ __device__ __forceinline__ void wk_advance(const WalkArgs& a, WalkState& st, con
         int nC = 1;
         float mine = (float)C;   // lane k: coefficient k
         const int need = kind == 2 ? 1 : m - nf + 1;   // sums that this node can still ask for
-        if (need > 1 && !have) {
+        if (need > 2 && have <= 1) {   // (of two sums the second's coefficient follows from the first)
           nC = WK_COLS | WK_GRID;
           constexpr float places[WK_COLS] = {1.f, 1.2f, 1.45f, 1.75f, 2.15f, 2.7f, 3.6f, 5.5f};
           float g = 1.f;
 #pragma unroll
           for (int k = 1; k < WK_COLS; ++k) g = lane == k ? places[k] : g;
           mine = (float)C * g;
-        } else if (need > 1) {
+        } else if (need > 1 && have > 1) {
           // what does not depend on the sequence, by all lanes at once: lane i's 1 / (1 - proposal mass of the siblings before
           // it), lane k's 1 / (width of interval k)
           double Q = e.qx;
