@@ -36,6 +36,7 @@ constexpr int WK_STATIC = 2048;            // static shared memory at most
 constexpr int WK_CHUNK = 1088;             // tokens of one step of the bonus rescan: 8 tokens x 136 places x 4 slices of the rank
 constexpr size_t WK_DOT = 4 * WK_CHUNK * sizeof(float);   // shared memory of the rescan
 constexpr double WK_TOL = 9.5367431640625e-7;   // 2^-20: a coefficient this close (relative) to an evaluated one counts as evaluated
+constexpr double WK_REL = 6.103515625e-5;       // 2^-14: and the step to it times the proposal mass may be this much of the residual
 
 // A request of a pass.  b: its number; rows that may start anywhere: and where in a 16-byte chunk the two do (bits 28, 24).
 struct __align__(16) RedDesc { const __nv_bfloat16 *z, *u; float zoff, qoff; int b, nC; float C[WK_COLS]; };
@@ -144,9 +145,12 @@ __device__ __forceinline__ void wk_setup(const WalkArgs& a, WalkState& st, const
 // fixed grid (there the sums are of |p - C q|, two instructions a token and coefficient: F = (1 - C + sum |p - C q|) / 2, good
 // enough for guesses); from its values (cubic interpolation of what the node's other tokens give; the children's own terms are known
 // exactly) the rest of the sequence is predicted, evaluated, and where a prediction was within 2^-20 of what its
-// predecessors turn out to give, F there is F and G at the prediction, to first order: the term left out is at most the step times the mass
-// whose ratio p / q lies inside the step, less than the rounding of the exponentials in any case.  Where it was not, the next reduction
-// evaluates the corrected predictions (errors go down quadratically).  A node's eight rejections take three reductions, sixteen take four or five.
+// predecessors turn out to give, F there is F and G at the prediction, to first order.  The term left out is at most the step times the
+// proposal mass whose ratio p / q lies inside the step: some per cent of G where a tie of logits lies there, all of it only where no more than the step
+// times G is left of F.  So the step times G may be 2^-14 of F at most, which keeps the term below the rounding of the
+// exponentials.  (2^-20 costs 32 requests 5 us of 140.  A grid's slopes come from a parabola: its coefficients stand for themselves only, as
+// does one that was evaluated alone.)  Where the prediction was not close enough, the next reduction evaluates the corrected
+// predictions (errors go down quadratically).  A node's eight rejections take three reductions, sixteen take four or five.
 __device__ __forceinline__ double wk_lanes_sum(double x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
@@ -192,7 +196,8 @@ __device__ __forceinline__ void wk_advance(const WalkArgs& a, WalkState& st, con
     if (kind) {   // ---- the sum at passC: from the reduction that just ran, or by another one ----
       const double C = st.passC;
       const int nf = st.nf;
-      const unsigned hit = __ballot_sync(0xFFFFFFFFu, lane < have && ((lane == 0 && fresh) || ((lane == 0 || !grid) && fabs(C - ck) <= WK_TOL * C)));
+      const double off = fabs(C - ck);
+      const unsigned hit = __ballot_sync(0xFFFFFFFFu, lane < have && ((lane == 0 && fresh) || (have > 1 && !grid && off <= WK_TOL * C && off * Gk <= WK_REL * fmax(Fk, 0.0))));
       fresh = false;
       // a child's own term: the residual it had when it was tested, or the one it has
       double own = lane < m ? fmax(e.px - (lane < nf && lane < KMAX ? st.fC[lane] : C) * e.qx, 0.0) : 0.0;
