@@ -353,7 +353,7 @@ __device__ __forceinline__ bool wk_drained(const WalkArgs& a, const WalkSm& sm, 
 // for a parity tells a slot's turns apart only while the waiter follows every one of them.)
 __device__ __forceinline__ void wk_stream(const WalkArgs& a, const WalkSm& sm, const CUtensorMap* tm, const int ncol, const int t0, const int tlen, const uint32_t pass,
                                           uint32_t& wreq, uint32_t& rnd, const uint32_t tmem_base) {
-  const int ntile = (tlen + 127) / 128, round = a.sets * a.tr;
+  const int ntile = (tlen + 127) / 128, round = a.tr << a.lsets;
   const uint32_t slab = (uint32_t)((a.r + 15) / 16) * 2048u, ring = (uint32_t)a.ring, w0 = pass * (uint32_t)ntile;
   for (int t = 0; t <= ntile; ++t) {
     for (const uint32_t upto = w0 + (uint32_t)t + ring; wreq < upto; ++wreq) {
@@ -376,6 +376,9 @@ __device__ __forceinline__ void wk_stream(const WalkArgs& a, const WalkSm& sm, c
   }
   ++rnd;
 }
+
+// Of the four sets of warps, how many (as a power of two) share the tiles: the plan's, or more for one pair of requests or two; the rest share the requests.
+__device__ __forceinline__ int wk_sets(const WalkArgs& a, const int nreq) { return nreq > 4 ? a.lsets : (nreq > 2 ? max(a.lsets, 1) : 2); }
 
 // Sums of N values over the lanes: halve the values while halving the lanes; lane (32 / N) v ends with value v.
 template <int N>
@@ -413,7 +416,7 @@ __device__ __forceinline__ bool wk_has(const int nC, const int val) {
 template <bool AL>
 __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm, const int nreq, const int ncol, const int t0, const int tlen,
                                             const uint32_t tmem_base, uint32_t& used, uint32_t& rnd, const bool first_pass) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = warp & 3, sets = nreq > 4 ? a.sets : (nreq > 2 ? max(a.sets, 2) : 4), set = (warp >> 2) & (sets - 1), part = (warp >> 2) / sets, nparts = 4 / sets;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = warp & 3, ls = wk_sets(a, nreq), sets = 1 << ls, set = (warp >> 2) & (sets - 1), part = warp >> (2 + ls), nparts = 4 >> ls;
   const int ntile = (tlen + 127) / 128;
   const float zs = (1.f / a.T) * 1.4426950408889634f;   // exponentials as powers of two
   float* mine = sm.part + (size_t)warp * a.req * WK_VALS;
@@ -423,9 +426,9 @@ __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm,
   const uint32_t dbase = smem_u32(sm.desc), place = smem_u32(sm.stage) + (uint32_t)warp * 2u * SLOT;
   const int seg = lane / CPS, ch = lane - seg * CPS;    // lane's copy of a request: 16 bytes of one segment (tile, row)
   bool alive = true;
-  const int round = a.sets * a.tr, step = 128 * sets;   // (a round is the plan's, however many sets share it)
+  const int round = a.tr << a.lsets, step = 128 << ls;   // (a round is the plan's, however many sets share it)
   for (int r0 = 0; r0 < ntile; r0 += round, ++rnd) {
-    const int left = min(ntile - r0, round) - set, ntl = left > 0 ? (left + sets - 1) / sets : 0;   // the set's tiles: r0 + set + sets i
+    const int left = min(ntile - r0, round) - set, ntl = left > 0 ? (left + sets - 1) >> ls : 0;   // the set's tiles: r0 + set + sets i
     const int tok = (r0 + set) * 128 + q * 32;                                              // the warp's first token in the first of them; then + step i
     int nt = 0;                                                                             // its tiles with any token
 #pragma unroll
@@ -874,10 +877,11 @@ __global__ void __launch_bounds__(WK_THREADS, 1) walk_mma_kernel(const __grid_co
         const RedDesc& d = sm.desc[x / WK_VALS];
         const int val = x % WK_VALS;
         if (wk_has(d.nC, val)) {
-          const int sets = nreq > 4 ? a.sets : (nreq > 2 ? max(a.sets, 2) : 4), nw = 4 * sets, w0 = ((x / WK_VALS) >> 1) % (4 / sets) * nw;   // the warps that had the request
+          const int ls = wk_sets(a, nreq), nw = 4 << ls, w0 = ((x / (2 * WK_VALS)) & ((4 >> ls) - 1)) << (2 + ls);   // the warps that had the request
+          const float* from = sm.part + (size_t)w0 * (a.req * WK_VALS) + x;
           float s = 0.f;
 #pragma unroll
-          for (int w = 0; w < WK_EPI; ++w) s += w < nw ? sm.part[(w0 + w) * a.req * WK_VALS + x] : 0.f;
+          for (int w = 0; w < WK_EPI; ++w) s += w < nw ? from[w * a.req * WK_VALS] : 0.f;
           a.part[((size_t)(d.b & 0xFFFFFF) * WK_VALS + val) * a.vt_n + cta] = s;
         }
       }
@@ -920,7 +924,7 @@ static bool walk_fit(const ts_ctx* ctx, int B, int req, int sets, int tr, bool s
   const ts_config& c = ctx->cfg;
   const int ntile = (ctx->vt_TV + 127) / 128;
   WalkPlan p{};
-  p.req = req; p.cols = req < 16 ? 16 : req; p.tr = tr; p.sets = sets;
+  p.req = req; p.cols = req < 16 ? 16 : req; p.tr = tr; p.lsets = sets == 4 ? 2 : sets - 1;
   if (sets * tr * p.cols > 512) return false;
   const size_t slab = (size_t)(c.r + 15) / 16 * 2048, avail = (size_t)ctx->max_smem - WK_STATIC;
   const size_t head = (size_t)((c.r + 63) / 64) * p.cols * 128, stage = (size_t)WK_EPI * tr * 4 * wk_seg(c.V % 8 == 0);
@@ -995,7 +999,7 @@ cudaError_t launch_walk_mma(ts_ctx* ctx, WalkArgs& a, char* ws, const WalkPlan& 
   a.edge = (WalkEdge*)ws; ws += align_up(b * n * sizeof(WalkEdge), 256);
   a.rec = (WalkRec*)ws; ws += align_up(b * sizeof(WalkRec), 256);
   a.part = (float*)ws;
-  a.ring = p.ring; a.req = p.req; a.cols = p.cols; a.tr = p.tr; a.sets = p.sets; a.oB = p.oB; a.oT = p.oT; a.oP = p.oP; a.oS = p.oS;
+  a.ring = p.ring; a.req = p.req; a.cols = p.cols; a.tr = p.tr; a.lsets = p.lsets; a.oB = p.oB; a.oT = p.oT; a.oP = p.oP; a.oS = p.oS;
   CUtensorMap tm;
   memset(&tm, 0, sizeof(tm));
   if (a.use_tma) memcpy(&tm, ctx->tmapW, sizeof(tm));

@@ -26,13 +26,13 @@ struct WalkArgs {
   NodeDesc* node; int2* child; WalkEdge* edge; WalkRec* rec;
   float* part;   // [B][2 * WK_COLS][vt_n]: range sums of the residual at every coefficient, then of the proposal where the residual is positive
   unsigned* barrier;
-  int vt_TV, vt_n, max_steps, ring, use_tma, req, cols, tr, sets; uint32_t oB, oT, oP, oS;   // offsets of the head rows, the staged rows, the partial sums and the rest; ring > 0: blocks of 128 tokens of W stream through that many slots
+  int vt_TV, vt_n, max_steps, ring, use_tma, req, cols, tr, lsets; uint32_t oB, oT, oP, oS;   // offsets of the head rows, the staged rows, the partial sums and the rest; ring > 0: blocks of 128 tokens of W stream through that many slots
   uint32_t wait_limit; int lost_arrival;
 };
 
-// A pass: `req` requests on `cols` accumulator columns; `sets` sets of four warps share a range's tiles, up to `tr` of a set in tensor memory together,
-// and 4 / sets parts of them the requests.
-struct WalkPlan { int ring, req, cols, tr, sets; uint32_t oB, oT, oP, oS; size_t smem; };
+// A pass: `req` requests on `cols` accumulator columns; 2^`lsets` sets of four warps share a range's tiles, up to `tr` of a set in tensor memory together,
+// and the parts that makes of all four the requests.
+struct WalkPlan { int ring, req, cols, tr, lsets; uint32_t oB, oT, oP, oS; size_t smem; };
 bool walk_plan(const ts_ctx* ctx, int B, bool tma, WalkPlan* out);
 cudaError_t launch_walk_mma(ts_ctx* ctx, WalkArgs& a, char* ws, const WalkPlan& p, cudaStream_t st);
 

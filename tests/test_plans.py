@@ -53,7 +53,7 @@ int main() {
     c.vt_TV = ((c.cfg.V + SMS - 1) / SMS + 63) / 64 * 64; c.vt_n = (c.cfg.V + c.vt_TV - 1) / c.vt_TV;
     ts::WalkPlan p{};
     const bool ok = ts::walk_plan(&c, B, c.cfg.V % 8 == 0, &p);
-    std::printf("%d %d %d %d %d %d %d %d %d\n", ok ? 1 : 0, p.ring, p.req, p.cols, p.sets, p.tr, (int)p.smem, c.vt_TV, c.vt_n);
+    std::printf("%d %d %d %d %d %d %d %d %d\n", ok ? 1 : 0, p.ring, p.req, p.cols, 1 << p.lsets, p.tr, (int)p.smem, c.vt_TV, c.vt_n);
   }
 }
 """
