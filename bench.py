@@ -161,9 +161,9 @@ def tree_stats(wl, tree, verdict):
     return dict(nodes=int(n.sum()), parents=parents, u_rows=urows, z_rows=int((n + 1).sum()),
                 levels_used=sum(1 for p in per_level if p > 0), parents_per_level=per_level,
                 acc=int(verdict["acc_len"].sum()), walk_rows=int((verdict["acc_len"].long() + 1).sum()),
-                walk_passes=int(((verdict["flags"].long() >> 8) & 0xFFFF).sum()),
-                # a request's reductions follow one another, one grid step each: the longest chain bounds the walk's steps
-                walk_chain=int(((verdict["flags"].long() >> 8) & 0xFFFF).max()))
+                # residual sums that the walks used (one reduction of the walk may give several of a request's)
+                walk_sums=int(((verdict["flags"].long() >> 8) & 0xFFFF).sum()),
+                walk_sums_most=int(((verdict["flags"].long() >> 8) & 0xFFFF).max()))
 
 
 def snapshot(tree, verdict):
@@ -304,9 +304,8 @@ def run_ours(args, rank, world, device):
     bytes_round_min = mean("u_rows") * row_b + w_b + mean("parents") * wl.r * es + mean("walk_rows") * row_b
     peak, peak_src = measured_peak()
     dom = max(kern, key=lambda k: kern[k]["ms_per_round"]) if kern else None
-    # walk: every residual reduction streams one target row and (recomputing the proposal) one base row;
-    # its range of W is staged once per launch
-    bytes_walk = mean("walk_passes") * 2 * row_b + w_b
+    # walk: the target row and (recomputing the proposal) the base row of every visited node once; W once
+    bytes_walk = mean("walk_rows") * 2 * row_b + w_b
     alg = {"score_tile": bytes_score, "expand_persistent": bytes_score, "zrow_stats": bytes_zrows, "verify_walk": bytes_walk}
     # DRAM bytes of the dominant kernel from a committed ncu capture of one round of this workload
     # (per launch: the round's bytes over the round's launches), null where none was captured
@@ -357,7 +356,7 @@ def run_ours(args, rank, world, device):
         "parents_scored_per_s": world * mean("parents") / sec, "nodes_per_s": world * mean("nodes") / sec,
         "detail": {"mean_nodes_per_tree": mean("nodes") / B, "mean_parents_per_round": mean("parents"),
                    "mean_accepted_len": mean("acc") / B, "mean_z_rows": mean("z_rows"),
-                   "mean_walk_reductions": mean("walk_passes"), "mean_longest_walk_chain": mean("walk_chain"),
+                   "mean_walk_sums": mean("walk_sums"), "mean_most_walk_sums_of_a_request": mean("walk_sums_most"),
                    "launches_per_round": launches / max(args.steps, 1),
                    "parents_per_level": used[0]["parents_per_level"], "outputs_reproduced": same},
         "clocks": clocks, "gpu_launches": launches, "kernels": kern,

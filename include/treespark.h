@@ -54,8 +54,9 @@ extern "C" {
 #define TS_DMAX 16       /* largest block depth D */
 #define TS_CALIB_KNOTS 16
 
-/* per-request flag word written by ts_verify_tree: bits 0..7 flags, bits 8..23 the number of
- * vocabulary-wide residual reductions the walk of that request needed (T > 0; a statistic) */
+/* per-request flag word written by ts_verify_tree: bits 0..7 flags, bits 8..23 the number of vocabulary-wide
+ * residual sums that the walk of that request used (T > 0; a statistic.  On the tensor cores one pass over the
+ * vocabulary can give several of them) */
 #define TS_FLAG_ZERO_MASS 64u  /* a residual target lost all mass; the previous residual was kept */
 #define TS_FLAGS_MASK 0xFFu
 
@@ -155,7 +156,8 @@ int32_t ts_score_parents(ts_ctx* ctx, const void* U, const void* A, const void* 
  * What it does instead: the per-tile records the scoring pass writes and the merge pass reads live in
  * one array of TS_STATIC_SCRATCH_BYTES (8 MiB) that is part of the library's device image.  Every GPU
  * that loads the library carries that array until the process ends.  The call makes no cudaMalloc,
- * cudaFree or other allocating call, and the results are the same as ts_score_parents'.
+ * cudaFree or other allocating call, and the results are the same as ts_score_parents' (log-normalisers of
+ * lists of more than 128 parents up to the last place: there is no room to share a short last group's work the same way).
  *
  * Limits and rules:
  *   - The array bounds P.  Every parent needs 2K lines of 128 bytes for its pruning bounds and, on the tensor

@@ -281,7 +281,7 @@ __device__ void advance(const VerifyArgs& a, int b, int lane, int parity, bool c
     if (st.need == 2) {  // the rescan wrote its token
       a.bonus[b] = st.result;
       a.acc_len[b] = st.acc;
-      a.flags[b] |= (uint32_t)min(st.npass, 0xFFFF) << 8;   // bits 8..23: reductions this walk needed
+      a.flags[b] |= (uint32_t)min(st.npass, 0xFFFF) << 8;   // bits 8..23: sums this walk used (a reduction each)
       st.need = 3;
     }
     if (st.need == 5) go_scan = 1;   // closing: draw the bonus token now

@@ -721,7 +721,7 @@ __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st,
     if (o == 0x7FFFFFFF) o = s_last >= 0 ? s_last : s_hi - s_lo - 1;   // rounding pushed the crossing past the range
     a.bonus[b] = s_lo + o;
     a.acc_len[b] = st.acc;
-    a.flags[b] |= (uint32_t)min(st.npass, 0xFFFF) << 8;   // bits 8..23: reductions this walk needed
+    a.flags[b] |= (uint32_t)min(st.npass, 0xFFFF) << 8;   // bits 8..23: sums this walk used
   }
   __syncthreads();
 }
