@@ -50,7 +50,7 @@ struct WalkState {
   float col[WK_COLS];
   double C, Zj, Qused, passC, partsC;      // partsC: the C that the stored range sums were computed for (-1: none)
   double S[WK_VALS];                       // the last reduction's sums
-  int fx[KMAX]; double fC[KMAX], fp[KMAX], fq[KMAX];
+  double fC[KMAX];                         // residual coefficients that the siblings tested so far keep
 };
 
 struct WalkSm {
@@ -305,7 +305,7 @@ __device__ __forceinline__ void wk_advance(const WalkArgs& a, WalkState& st, con
       } else {
         if (lane == 0) {
           const int k = st.nf;
-          st.fx[k] = x; st.fp[k] = px; st.fq[k] = qx; st.fC[k] = C + cj; st.nf = k + 1;
+          st.fC[k] = C + cj; st.nf = k + 1;
           st.Qused = Q + qx; st.j = j + 1; st.passC = C + cj;
         }
         kind = 1;
@@ -583,13 +583,15 @@ __device__ __forceinline__ void wk_epilogue(const WalkArgs& a, const WalkSm& sm,
 __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st, const int b, float* s_dot) {
   __shared__ float s_a[RMAX];
   __shared__ double s_scan[WK_EPI + 1], s_target, s_before;
-  __shared__ int s_tile, s_found, s_last;
+  __shared__ int s_tile, s_found, s_last, s_fx[KMAX];   // the tested siblings: token, target and draft probability
+  __shared__ double s_fp[KMAX], s_fq[KMAX];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const size_t cb = (size_t)b * (a.N + 1);
   const int v = st.cur, nf = st.nf;
   const double C = st.C;
   const NodeDesc nd = a.node[cb + v + 1];
   const uint64_t hv = a.node_hash[cb + v + 1];
+  if (tid < nf) { const WalkEdge e = a.edge[(size_t)b * a.N + st.cfirst + tid]; s_fx[tid] = e.x; s_fp[tid] = e.px; s_fq[tid] = e.qx; }
   // the range that holds the token: cumulative range sums at C (to first order from the coefficient they were evaluated at),
   // corrected for the tested siblings, which keep the residual they had when tested
   double* s_pt = reinterpret_cast<double*>(s_dot);
@@ -597,11 +599,13 @@ __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st,
     const float col = st.col[st.pcol];
     const double Ce = (double)col, Cf = (double)(float)C, step = st.nC > 1 && !(st.nC & WK_GRID) && fabs(Cf - Ce) <= 2.0 * WK_TOL * Cf ? Cf - Ce : 0.0;
     const float* part = a.part + ((size_t)b * WK_VALS + st.pcol) * a.vt_n;
-    for (int t = tid; t < a.vt_n; t += WK_THREADS) {
-      double pt = (double)__ldcg(part + t);
-      if (step != 0.0) pt -= step * (double)__ldcg(part + (size_t)WK_COLS * a.vt_n + t);
+    const int t = tid;   // (a range each: there are no more than SMs)
+    double pt = t < a.vt_n ? (double)__ldcg(part + t) : 0.0;
+    if (step != 0.0 && t < a.vt_n) pt -= step * (double)__ldcg(part + (size_t)WK_COLS * a.vt_n + t);
+    __syncthreads();
+    if (t < a.vt_n) {
       for (int i = 0; i < nf; ++i)
-        if (st.fx[i] >= t * a.vt_TV && st.fx[i] < (t + 1) * a.vt_TV) pt += fmax(st.fp[i] - st.fC[i] * st.fq[i], 0.0) - fmax(st.fp[i] - Ce * st.fq[i], 0.0) + (st.fp[i] > Ce * st.fq[i] ? step * st.fq[i] : 0.0);
+        if (s_fx[i] >= t * a.vt_TV && s_fx[i] < (t + 1) * a.vt_TV) pt += fmax(s_fp[i] - st.fC[i] * s_fq[i], 0.0) - fmax(s_fp[i] - Ce * s_fq[i], 0.0) + (s_fp[i] > Ce * s_fq[i] ? step * s_fq[i] : 0.0);
       s_pt[t] = fmax(pt, 0.0);
     }
   }
@@ -691,7 +695,7 @@ __device__ __forceinline__ void wk_bonus(const WalkArgs& a, const WalkState& st,
       rw[h] = 0.0;
       if (o < len) {
         double Cw = C;
-        for (int f = 0; f < nf; ++f) if (st.fx[f] == w) Cw = st.fC[f];
+        for (int f = 0; f < nf; ++f) if (s_fx[f] == w) Cw = st.fC[f];
         const double p = exp(((double)zv[h] - (double)nd.zmax) / (double)a.T - (double)nd.zlogs);
         double q = 0.0;
         if (Cw != 0.0) {

@@ -79,6 +79,7 @@ def logit(q):
 WALK_SHAPES = {
     (4104, 64, 97): (0, 64, 1, 1),      # one tile, passes of 64 and 33
     (2501, 16, 70): (0, 64, 1, 1),      # ragged rows, passes of 64 and 6
+    (696, 8, 300): (0, 64, 1, 1),       # dozens of requests an owner
     (50257, 32, 9): (0, 16, 1, 3),      # three tiles in one set, ragged rows
     (64008, 32, 20): (0, 32, 2, 2),     # four tiles in two sets
     (100000, 64, 70): (0, 64, 2, 3),    # six, passes of 64 and 6

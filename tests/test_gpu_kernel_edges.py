@@ -241,7 +241,7 @@ def check_hard_walks(over, T, reqs=None):
 def test_every_form_of_the_walk_under_hard_targets(V, r, B):
     """A sample of the requests against the oracle, the ends of every pass among them; the sums of all."""
     size = WALK_SHAPES[V, r, B][1]
-    ends = {b for k in range(0, B, size) for b in (k, min(k + size, B) - 1)} | {B // 2}
+    ends = {b for k in range(0, B, size) for b in (k, min(k + size, B) - 1)} | {B // 2}   # (of every pass of the first step)
     check_hard_walks(dict(V=V, r=r, B=B, Nmax=12, K=8, D=3), 0.9, sorted(ends))
 
 

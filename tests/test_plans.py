@@ -69,7 +69,7 @@ def test_every_walk_whose_weights_fit_has_a_tensor_core_plan(tmp_path):
     """A range of W in shared memory beside one tile of head rows and the walks' state is all that the walk needs at least: a
     plan must be found wherever that much fits (ranks padded to 64, 16 KB of static memory, the state of an owner 360 bytes),
     resident where there is no tensor map (ragged rows)."""
-    grid = [(V, r, B) for V0 in range(1000, 262000, 3000) for V in (V0 // 8 * 8, V0 | 1) for r in (8, 24, 56, 64, 96, 128, 160, 192, 256) for B in (1, 3, 8, 16, 17, 32, 33, 64, 128, 400)]
+    grid = [(V, r, B) for V0 in (*range(100, 4000, 300), *range(4000, 262000, 3000)) for V in (V0 // 8 * 8, V0 | 1) for r in (8, 24, 56, 64, 96, 128, 160, 192, 256) for B in (1, 3, 8, 16, 17, 32, 33, 64, 128, 400, 1500, 4096)]
     missing = []
     for (V, r, B), (ok, ring, req, cols, sets, tr, smem, TV, n) in zip(grid, ask(tmp_path, WALK, grid)):
         slab, ntile = (r + 63) // 64 * 8192, (TV + 127) // 128
