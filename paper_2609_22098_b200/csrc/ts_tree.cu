@@ -13,7 +13,7 @@
 // Before this, a level was three dependent launches (scan with its own set-up, merge of fixed-size records, level
 // step on global-memory state): about 70 us per level at 32 requests, V = 151,936, r = 64, of which the arithmetic
 // needs less than ten.  Now (serve shape: 32 requests, 16 nodes): 12 to 30 us of scan, 11 to 19 us of owner phase and two
-// grid barriers of 1.2 to 2.3 us per level, 196 us for the expansion with its set-up launch (365 with three launches a level).
+// grid barriers of 1.2 to 2.3 us per level, 192 us for the expansion and 6 for its set-up launch (365 with three launches a level).
 //
 // Bounds.  Per parent K slots in global memory, slot j = best value published by the pieces (range, split, replica)
 // whose number is j mod K; pieces hold disjoint tokens, so the minimum over the slots is a lower bound of the K-th
