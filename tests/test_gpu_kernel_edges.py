@@ -212,11 +212,11 @@ def test_walks_that_reject_every_sibling(over, T):
     check_hard_walks(over, T)
 
 
-def check_hard_walks(over, T, reqs=None):
+def check_hard_walks(over, T, reqs=None, mode=0):
     wl = parity.small("wide", dtype="bf16", **over)
     rnd = HardRound(wl, seed=over["V"])
     rnd.theta.fill_(0.01)
-    ts = make_gpu(wl, rnd.table, max_batch=rnd.B)
+    ts = make_gpu(wl, rnd.table, max_batch=rnd.B, test_mode=mode)
     st = check_round(ts, make_oracle(wl, rnd.table), rnd, T, round_seed=4, reqs=reqs)
     assert st["walks_exempt"] <= 0.1 * st["walks"] + 1
     tree = ts.expand_tree(rnd.U, rnd.A, rnd.W, rnd.anchor, rnd.theta, T, 4)
@@ -243,6 +243,11 @@ def test_every_form_of_the_walk_under_hard_targets(V, r, B):
     size = WALK_SHAPES[V, r, B][1]
     ends = {b for k in range(0, B, size) for b in (k, min(k + size, B) - 1)} | {B // 2}   # (of every pass of the first step)
     check_hard_walks(dict(V=V, r=r, B=B, Nmax=12, K=8, D=3), 0.9, sorted(ends))
+
+
+@pytest.mark.parametrize("V,r,B", [(64008, 32, 18), (200008, 64, 20)])   # (the second: passes of 16 and 4 beside a resident range)
+def test_walk_without_a_tensor_map(V, r, B):
+    check_hard_walks(dict(V=V, r=r, B=B, Nmax=12, K=8, D=3), 0.9, [0, B // 2, B - 1], binding.TEST_NO_TMA)
 
 
 # several groups of 128 parents whose last is held once, twice or four times over
